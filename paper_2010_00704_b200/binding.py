@@ -1,4 +1,4 @@
-"""Thin ctypes binding of the C ABI in include/bcnn.h.
+"""Thin binding of the C ABI in include/bcnn.h: the launching calls through a CPython module, the queries through ctypes.
 
 Argument marshalling only: every step of the path runs in the CUDA kernels.  Tensors
 are torch CUDA tensors used purely as device buffers; the functions take their
@@ -33,6 +33,7 @@ OK, ERR_INVALID_ARG, ERR_UNSUPPORTED, ERR_ALIGNMENT, ERR_CUDA, ERR_WORKSPACE, ER
 SELFTEST_TIMEOUT_CODE = 120
 
 _lib = None
+_native = None
 
 
 class BcnnError(RuntimeError):
@@ -43,7 +44,7 @@ class BcnnError(RuntimeError):
 
 def load() -> ctypes.CDLL:
     """Load libbcnn.so (built in-tree by ``build.py``); raises if it is absent."""
-    global _lib
+    global _lib, _native
     if _lib is None:
         if not os.path.exists(LIB_PATH):
             raise ImportError(f"{LIB_PATH} not built: run python -m paper_2010_00704_b200.build")
@@ -81,8 +82,19 @@ def load() -> ctypes.CDLL:
         for name in EXPORTS:
             if name not in ("bcnn_status_string", "bcnn_workspace_bytes", "bcnn_prepared_weights_bytes"):
                 getattr(lib, name).restype = i32
-        _lib = lib
+        try:
+            from . import _native as native
+        except ImportError as e:
+            raise ImportError(f"{_PKG}/_native not built: run python -m paper_2010_00704_b200.build") from e
+        _lib, _native = lib, native
     return _lib
+
+
+def _n():
+    """The launching calls' CPython front (csrc/pymodule.c, built beside the library)."""
+    if _native is None:
+        load()
+    return _native
 
 
 def status_string(status: int) -> str:
@@ -93,12 +105,20 @@ def version() -> int:
     return load().bcnn_version()
 
 
+def _resolve_stream():
+    """The current stream's address straight from torch's C layer: ``torch.cuda.current_stream()`` builds a Stream
+    object, which took 3.3 us of a call's 9."""
+    torch.cuda.init()
+    get_device, get_stream = getattr(torch._C, "_cuda_getDevice", None), getattr(torch._C, "_cuda_getCurrentRawStream", None)
+    if get_device is None or get_stream is None:
+        return lambda: torch.cuda.current_stream().cuda_stream
+    return lambda: get_stream(get_device())
+
+
 def _stream() -> int:
-    return torch.cuda.current_stream().cuda_stream
-
-
-def _p(t) -> int | None:
-    return None if t is None else t.data_ptr()
+    global _stream
+    _stream = _resolve_stream()
+    return _stream()
 
 
 def _check(status: int, what: str):
@@ -112,7 +132,7 @@ def out_hw(H, W, kh, kw, stride, pad):
 
 def bcnn_pack(x: torch.Tensor, bias, out_bits: torch.Tensor, B, H, W, C_in, R=1):
     """x fp32 NHWC device tensor -> packed sign bits written into ``out_bits``."""
-    _check(load().bcnn_pack(_p(x), _p(bias), _p(out_bits), B, H, W, C_in, R, _stream()), "bcnn_pack")
+    _check(_n().pack(x, bias, out_bits, B, H, W, C_in, R, _stream()), "bcnn_pack")
     return out_bits
 
 
@@ -120,28 +140,24 @@ def bcnn_stem_fused(x, bias, w_bits, thr, y_bits, B, H, W, C_in, R, C_out):
     """fp32 NHWC input -> (bias, sign, replication) -> binary 1x1 convolution -> threshold -> packed bits."""
     if thr is None:
         raise BcnnError(-1, "bcnn_stem_fused")
-    _check(load().bcnn_stem_fused(_p(x), _p(bias), _p(w_bits), _p(thr), _p(y_bits), B, H, W, C_in, R, C_out,
-                                  _stream()), "bcnn_stem_fused")
+    _check(_n().stem_fused(x, bias, w_bits, thr, y_bits, B, H, W, C_in, R, C_out, _stream()), "bcnn_stem_fused")
     return y_bits
 
 
 def bcnn_gemm_b1(A_bits, W_bits, C, M, N, K, engine=ENGINE_AUTO):
-    _check(load().bcnn_gemm_b1_engine(engine, _p(A_bits), _p(W_bits), None, _p(C), M, N, K, _stream()),
-           "bcnn_gemm_b1")
+    _check(_n().gemm(A_bits, W_bits, None, C, engine, M, N, K, _stream()), "bcnn_gemm_b1")
     return C
 
 
 def bcnn_gemm_b1_fused(A_bits, W_bits, thr, out_bits, M, N, K, engine=ENGINE_AUTO):
     if thr is None:
         raise BcnnError(-1, "bcnn_gemm_b1_fused")
-    _check(load().bcnn_gemm_b1_engine(engine, _p(A_bits), _p(W_bits), _p(thr), _p(out_bits), M, N, K, _stream()),
-           "bcnn_gemm_b1_fused")
+    _check(_n().gemm(A_bits, W_bits, thr, out_bits, engine, M, N, K, _stream()), "bcnn_gemm_b1_fused")
     return out_bits
 
 
 def bcnn_conv2d_b1(x_bits, w_bits, y, B, H, W, C_in, C_out, kh, kw, stride, pad, engine=ENGINE_AUTO):
-    _check(load().bcnn_conv2d_b1_engine(engine, _p(x_bits), _p(w_bits), None, _p(y), B, H, W, C_in, C_out,
-                                        kh, kw, stride, pad, _stream()), "bcnn_conv2d_b1")
+    _check(_n().conv2d(x_bits, w_bits, None, y, engine, B, H, W, C_in, C_out, kh, kw, stride, pad, _stream()), "bcnn_conv2d_b1")
     return y
 
 
@@ -149,48 +165,45 @@ def bcnn_conv2d_b1_fused(x_bits, w_bits, thr, y_bits, B, H, W, C_in, C_out, kh, 
                          engine=ENGINE_AUTO):
     if thr is None:
         raise BcnnError(-1, "bcnn_conv2d_b1_fused")
-    _check(load().bcnn_conv2d_b1_engine(engine, _p(x_bits), _p(w_bits), _p(thr), _p(y_bits), B, H, W, C_in,
-                                        C_out, kh, kw, stride, pad, _stream()), "bcnn_conv2d_b1_fused")
+    _check(_n().conv2d(x_bits, w_bits, thr, y_bits, engine, B, H, W, C_in, C_out, kh, kw, stride, pad, _stream()), "bcnn_conv2d_b1_fused")
     return y_bits
 
 
 def bcnn_conv2d_b1_module(x_bits, w_bits, bn_scale, bn_shift, identity, prelu_slope, next_bias, y_real, y_bits,
                           B, H, W, C_in, C_out, kh, kw, stride, pad):
     """Binary conv -> batch norm -> + identity (fp16) -> PReLU -> fp16 map and the next module's packed signs."""
-    _check(load().bcnn_conv2d_b1_module(_p(x_bits), _p(w_bits), _p(bn_scale), _p(bn_shift), _p(identity),
-                                        _p(prelu_slope), _p(next_bias), _p(y_real), _p(y_bits), B, H, W, C_in, C_out,
-                                        kh, kw, stride, pad, _stream()), "bcnn_conv2d_b1_module")
+    _check(_n().conv2d_module(x_bits, w_bits, bn_scale, bn_shift, identity, prelu_slope, next_bias, y_real, y_bits, B, H, W,
+                              C_in, C_out, kh, kw, stride, pad, _stream()), "bcnn_conv2d_b1_module")
     return y_real, y_bits
 
 
 def bcnn_conv2d_b1_branches(x_bits, w_bits, bn_scale, bn_shift, pad_dot, identity, prelu_slope, next_bias, y_real, y_bits,
                             B, H, W, C_in, C_out, P, kh=1, kw=1):
     """Module with P parallel binary branches (kh*kw > 1: the P = kh*kw shifted taps of a binary kh x kw convolution)."""
-    _check(load().bcnn_conv2d_b1_branches(_p(x_bits), _p(w_bits), _p(bn_scale), _p(bn_shift), _p(pad_dot), _p(identity),
-                                          _p(prelu_slope), _p(next_bias), _p(y_real), _p(y_bits), B, H, W, C_in, C_out, P,
-                                          kh, kw, _stream()), "bcnn_conv2d_b1_branches")
+    _check(_n().conv2d_branches(x_bits, w_bits, bn_scale, bn_shift, pad_dot, identity, prelu_slope, next_bias, y_real, y_bits,
+                                B, H, W, C_in, C_out, P, kh, kw, _stream()), "bcnn_conv2d_b1_branches")
     return y_real, y_bits
 
 
 def bcnn_dwconv3x3_module(x, w, bn_scale, bn_shift, prelu_slope, next_bias, y_real, y_bits, B, H, W, C_in, R=1, S=1):
     """Real depth-wise 3x3 convolution (stride S, replication R) -> batch norm -> PReLU -> fp16 map (+ next signs)."""
-    _check(load().bcnn_dwconv3x3_module(_p(x), _p(w), _p(bn_scale), _p(bn_shift), _p(prelu_slope), _p(next_bias), _p(y_real),
-                                        _p(y_bits), B, H, W, C_in, R, S, _stream()), "bcnn_dwconv3x3_module")
+    _check(_n().dwconv3x3_module(x, w, bn_scale, bn_shift, prelu_slope, next_bias, y_real, y_bits, B, H, W, C_in, R, S,
+                                 _stream()), "bcnn_dwconv3x3_module")
     return y_real, y_bits
 
 
 def bcnn_avgpool(x, y, B, H, W, C_in, R=1, S=1):
-    _check(load().bcnn_avgpool(_p(x), _p(y), B, H, W, C_in, R, S, _stream()), "bcnn_avgpool")
+    _check(_n().avgpool(x, y, B, H, W, C_in, R, S, _stream()), "bcnn_avgpool")
     return y
 
 
 def bcnn_gap(x, pooled, B, H, W, C):
-    _check(load().bcnn_gap(_p(x), _p(pooled), B, H, W, C, _stream()), "bcnn_gap")
+    _check(_n().gap(x, pooled, B, H, W, C, _stream()), "bcnn_gap")
     return pooled
 
 
 def bcnn_fc(pooled, w, bias, logits, B, C, N):
-    _check(load().bcnn_fc(_p(pooled), _p(w), _p(bias), _p(logits), B, C, N, _stream()), "bcnn_fc")
+    _check(_n().fc(pooled, w, bias, logits, B, C, N, _stream()), "bcnn_fc")
     return logits
 
 
@@ -200,18 +213,17 @@ def bcnn_prepared_weights_bytes(C_out, K) -> int:
 
 def bcnn_prepare_weights(w_bits, prepared, C_out, K):
     """Expand a layer's packed weights once into the caller's buffer ``prepared`` (256-byte aligned)."""
-    _check(load().bcnn_prepare_weights(_p(w_bits), _p(prepared), C_out, K, _stream()), "bcnn_prepare_weights")
+    _check(_n().prepare_weights(w_bits, prepared, C_out, K, _stream()), "bcnn_prepare_weights")
     return prepared
 
 
 def bcnn_conv2d_b1_prepared(x_bits, prepared, thr, out, B, H, W, C_in, C_out, kh, kw, stride, pad):
-    _check(load().bcnn_conv2d_b1_prepared(_p(x_bits), _p(prepared), _p(thr), _p(out), B, H, W, C_in, C_out, kh, kw, stride, pad,
-                                          _stream()), "bcnn_conv2d_b1_prepared")
+    _check(_n().conv2d_prepared(x_bits, prepared, thr, out, B, H, W, C_in, C_out, kh, kw, stride, pad, _stream()), "bcnn_conv2d_b1_prepared")
     return out
 
 
 def bcnn_gemm_b1_prepared(A_bits, prepared, thr, out, M, N, K):
-    _check(load().bcnn_gemm_b1_prepared(_p(A_bits), _p(prepared), _p(thr), _p(out), M, N, K, _stream()), "bcnn_gemm_b1_prepared")
+    _check(_n().gemm_prepared(A_bits, prepared, thr, out, M, N, K, _stream()), "bcnn_gemm_b1_prepared")
     return out
 
 
@@ -223,8 +235,7 @@ def bcnn_conv2d_b1_fused_noalloc(x_bits, w_bits, thr, y_bits, B, H, W, C_in, C_o
     library (4 MiB per GPU); layers whose prepared form is larger raise BCNN_ERR_WORKSPACE."""
     if thr is None:
         raise BcnnError(-1, "bcnn_conv2d_b1_fused_noalloc")
-    _check(load().bcnn_conv2d_b1_fused_noalloc(_p(x_bits), _p(w_bits), _p(thr), _p(y_bits), B, H, W, C_in, C_out, kh, kw,
-                                               stride, pad, _stream()), "bcnn_conv2d_b1_fused_noalloc")
+    _check(_n().conv2d_fused_noalloc(x_bits, w_bits, thr, y_bits, B, H, W, C_in, C_out, kh, kw, stride, pad, _stream()), "bcnn_conv2d_b1_fused_noalloc")
     return y_bits
 
 

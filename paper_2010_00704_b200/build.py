@@ -1,15 +1,17 @@
-"""In-tree build of the CUDA library: nvcc -> paper_2010_00704_b200/libbcnn.so (sm_100a only)."""
+"""In-tree build: nvcc -> libbcnn.so (sm_100a only), then the CPython front of its launching calls -> _native*.so."""
 from __future__ import annotations
 
 import glob
 import os
 import subprocess
 import sys
+import sysconfig
 
 PKG = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(PKG)
 CSRC = os.path.join(PKG, "csrc")
 LIB = os.path.join(PKG, "libbcnn.so")
+NATIVE = os.path.join(PKG, "_native" + sysconfig.get_config_var("EXT_SUFFIX"))
 
 NVCC_FLAGS = [
     "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
@@ -22,15 +24,15 @@ def sources():
 
 
 def _stale() -> bool:
-    if not os.path.exists(LIB):
+    if not os.path.exists(LIB) or not os.path.exists(NATIVE):
         return True
-    deps = sources() + glob.glob(os.path.join(CSRC, "*.cuh")) + [os.path.join(ROOT, "include", "bcnn.h"),
+    deps = sources() + glob.glob(os.path.join(CSRC, "*.cuh")) + [os.path.join(CSRC, "pymodule.c"), os.path.join(ROOT, "include", "bcnn.h"),
                                                                   os.path.abspath(__file__)]
-    return os.path.getmtime(LIB) < max(os.path.getmtime(d) for d in deps)
+    return min(os.path.getmtime(LIB), os.path.getmtime(NATIVE)) < max(os.path.getmtime(d) for d in deps)
 
 
 def build(force: bool = False, verbose: bool = False) -> str:
-    """Compile every .cu under csrc/ into one shared library next to this file."""
+    """Compile every .cu under csrc/ into one shared library next to this file, and pymodule.c against it."""
     if not force and not _stale():
         return LIB
     nvcc = os.environ.get("NVCC", "nvcc")
@@ -49,6 +51,10 @@ def build(force: bool = False, verbose: bool = False) -> str:
     tmp = LIB + f".tmp{os.getpid()}"
     subprocess.run([nvcc, "-shared", "-o", tmp] + objs + ["-lcudart"], check=True)
     os.replace(tmp, LIB)
+    tmp = NATIVE + f".tmp{os.getpid()}"
+    subprocess.run([os.environ.get("CC", "gcc"), "-O2", "-shared", "-fPIC", "-I", sysconfig.get_paths()["include"], "-I", os.path.join(ROOT, "include"),
+                    os.path.join(CSRC, "pymodule.c"), "-o", tmp, "-L", PKG, "-l:libbcnn.so", "-Wl,-rpath,$ORIGIN"], check=True)
+    os.replace(tmp, NATIVE)
     return LIB
 
 
