@@ -4,6 +4,7 @@
 #include <cstdint>
 #include <cuda_runtime.h>
 #include "bcnn.h"
+#include "launch.cuh"
 
 namespace bcnn {
 

@@ -38,6 +38,8 @@ dwconv3x3_module_kernel(const uint16_t *x, const float *w, const float *scale, c
     // 8-channel groups - channels 8g..8g+3 at [2q][g], 8g+4..8g+7 at [2q+1][g] - so that a warp's groups read
     // consecutive 16-byte pieces (one float per lane, or 32-byte pieces per lane, would conflict 8- and 2-way)
     extern __shared__ __align__(16) float dw_smem[];
+    pdl_trigger();
+    pdl_wait();
     const int groups = C / 8;
     const float4 *vec = reinterpret_cast<const float4 *>(dw_smem);
     for (int i = threadIdx.x; i < 13 * C; i += blockDim.x) {
@@ -128,6 +130,8 @@ dwconv3x3_module_kernel(const uint16_t *x, const float *w, const float *scale, c
 __global__ void __launch_bounds__(256)
 avgpool_kernel(const uint16_t *x, uint16_t *y, int B, int H, int W, int C_in, int C, int S)
 {
+    pdl_trigger();
+    pdl_wait();
     const int OH = H / S, OW = W / S, groups = C / 8;
     const long total = (long)B * OH * OW * groups;
     const float inv = 1.0f / (float)(S * S);
@@ -158,6 +162,7 @@ avgpool_kernel(const uint16_t *x, uint16_t *y, int B, int H, int W, int C_in, in
 __global__ void __launch_bounds__(256)
 gap_kernel(const uint16_t *x, float *pooled, int B, int HW, int C)
 {
+    pdl_wait();
     const int groups = C / 8;
     const long total = (long)B * groups;
     for (long i = (long)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (long)gridDim.x * blockDim.x) {
@@ -175,6 +180,7 @@ gap_kernel(const uint16_t *x, float *pooled, int B, int HW, int C)
         dst[0] = make_float4(acc[0] * inv, acc[1] * inv, acc[2] * inv, acc[3] * inv);
         dst[1] = make_float4(acc[4] * inv, acc[5] * inv, acc[6] * inv, acc[7] * inv);
     }
+    pdl_trigger();          // late: blocks of the next kernel that came in beside these ones would end up unevenly spread
 }
 
 // logits[b][n] = sum_c pooled[b][c] * w[n][c] + bias[n].  A CTA takes FC_IMAGES images (their pooled rows in shared
@@ -185,6 +191,7 @@ __global__ void __launch_bounds__(256)
 fc_kernel(const float *pooled, const float *w, const float *bias, float *logits, int B, int C, int N)
 {
     extern __shared__ __align__(16) float fc_smem[];           // [FC_IMAGES][C]
+    pdl_wait();
     const int b0 = blockIdx.x * FC_IMAGES;
     const int nb = min(FC_IMAGES, B - b0);
     for (int i = threadIdx.x; i < FC_IMAGES * C; i += blockDim.x)
@@ -214,13 +221,12 @@ fc_kernel(const float *pooled, const float *w, const float *bias, float *logits,
         if (lane == 3) v = acc[3];
         if (lane < nb) logits[(long)(b0 + lane) * N + n] = v + (bias ? __ldg(bias + n) : 0.f);
     }
+    pdl_trigger();          // late: blocks of the next kernel that came in beside these ones would end up unevenly spread
 }
 
 int grid_for(long total_threads)
 {
-    int dev = 0, sms = 148;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    const int sms = sm_count();
     const long blocks = (total_threads + 255) / 256;
     const long cap = (long)sms * 16;
     return (int)(blocks < cap ? (blocks < 1 ? 1 : blocks) : cap);
@@ -239,40 +245,34 @@ int launch_dwconv3x3_module(const uint16_t *x, const float *w, const float *scal
     if ((long)B * OH * OW >= (1L << 31)) return BCNN_ERR_UNSUPPORTED;         // pixel indices are 32-bit
     const int threads = (256 / groups) * groups;                            // <= 256, a multiple of groups
     const long passes = ((long)B * OH * OW + threads / groups - 1) / (threads / groups);
-    int dev = 0, sms = 148;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    const int sms = sm_count();
     const long cap = (long)sms * 8;
     const unsigned blocks = (unsigned)(passes < cap ? passes : cap);
-    if (cudaFuncSetAttribute(dwconv3x3_module_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024) != cudaSuccess) return BCNN_ERR_CUDA;
-    dwconv3x3_module_kernel<<<blocks, threads, smem, stream>>>(x, w, scale, shift, slope, next_bias, y, y_bits,
-                                                               B, H, W, C_in, C, S, OH, OW);
-    return cudaGetLastError() == cudaSuccess ? BCNN_OK : BCNN_ERR_CUDA;
+    if (!allow_smem((const void *)dwconv3x3_module_kernel, 200 * 1024)) return BCNN_ERR_CUDA;
+    return launch(dwconv3x3_module_kernel, blocks, threads, smem, stream, x, w, scale, shift, slope, next_bias, y, y_bits,
+                  B, H, W, C_in, C, S, OH, OW);
 }
 
 int launch_avgpool(const uint16_t *x, uint16_t *y, int B, int H, int W, int C_in, int R, int S, cudaStream_t stream)
 {
     const int C = C_in * R;
-    avgpool_kernel<<<grid_for((long)B * (H / S) * (W / S) * (C / 8)), 256, 0, stream>>>(x, y, B, H, W, C_in, C, S);
-    return cudaGetLastError() == cudaSuccess ? BCNN_OK : BCNN_ERR_CUDA;
+    return launch(avgpool_kernel, grid_for((long)B * (H / S) * (W / S) * (C / 8)), 256, 0, stream, x, y, B, H, W, C_in, C, S);
 }
 
 int launch_gap(const uint16_t *x, float *pooled, int B, int HW, int C, cudaStream_t stream)
 {
-    gap_kernel<<<grid_for((long)B * (C / 8)), 256, 0, stream>>>(x, pooled, B, HW, C);
-    return cudaGetLastError() == cudaSuccess ? BCNN_OK : BCNN_ERR_CUDA;
+    return launch(gap_kernel, grid_for((long)B * (C / 8)), 256, 0, stream, x, pooled, B, HW, C);
 }
 
 int launch_fc(const float *pooled, const float *w, const float *bias, float *logits, int B, int C, int N, cudaStream_t stream)
 {
     const int smem = FC_IMAGES * C * 4;
     if (smem > 200 * 1024) return BCNN_ERR_UNSUPPORTED;
-    if (cudaFuncSetAttribute(fc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024) != cudaSuccess) return BCNN_ERR_CUDA;
+    if (!allow_smem((const void *)fc_kernel, 200 * 1024)) return BCNN_ERR_CUDA;
     const int images = (B + FC_IMAGES - 1) / FC_IMAGES;
     int ny = 1;                                     // enough CTAs to fill the GPU a few times over
     while (images * ny < 592 && ny * 8 < N) ny *= 2;
-    fc_kernel<<<dim3(images, ny), 256, smem, stream>>>(pooled, w, bias, logits, B, C, N);
-    return cudaGetLastError() == cudaSuccess ? BCNN_OK : BCNN_ERR_CUDA;
+    return launch(fc_kernel, dim3(images, ny), 256, smem, stream, pooled, w, bias, logits, B, C, N);
 }
 
 }  // namespace bcnn

@@ -25,6 +25,7 @@ __global__ void __launch_bounds__(THREADS)
 conv_branches_kernel(const BranchProblem p, const int NS /* channels per slice */, const int tile_rows)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
+    pdl_wait();
     // Per-channel vectors of the slice, each stored as two 16-byte arrays over its 8-channel groups (channels 8g..8g+3
     // at [2q][g], 8g+4..8g+7 at [2q+1][g]) so that a warp's groups read consecutive 16-byte pieces without bank
     // conflicts: vectors q = br * cw + k are the weight words, then per branch scale, shift, pad dot, then slope and
@@ -144,6 +145,7 @@ conv_branches_kernel(const BranchProblem p, const int NS /* channels per slice *
             if (p.y_bits) p.y_bits[e0 >> 3] = (uint8_t)bits;
         }
     }
+    pdl_trigger();          // late: blocks of the next kernel that came in beside these ones would end up unevenly spread
 }
 
 }  // namespace
@@ -158,17 +160,14 @@ int launch_conv_branches(const BranchProblem &p, cudaStream_t stream)
     if (NS * per_channel > MAX_SMEM) return BCNN_ERR_UNSUPPORTED;
     const int slices = (p.C_out + NS - 1) / NS;
     const int smem = (int)(NS * per_channel);
-    int dev = 0, sms = 148;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    const int sms = sm_count();
     const int tile_rows = 8 * (THREADS / (NS / 8));            // eight passes per tile
     const long tiles = (p.M + tile_rows - 1) / tile_rows;
     long gx = (long)sms * 4 / slices;
     if (gx < 1) gx = 1;
     if (gx > tiles) gx = tiles;
-    if (cudaFuncSetAttribute(conv_branches_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, MAX_SMEM) != cudaSuccess) return BCNN_ERR_CUDA;
-    conv_branches_kernel<<<dim3((unsigned)gx, (unsigned)slices), THREADS, smem, stream>>>(p, NS, tile_rows);
-    return cudaGetLastError() == cudaSuccess ? BCNN_OK : BCNN_ERR_CUDA;
+    if (!allow_smem((const void *)conv_branches_kernel, MAX_SMEM)) return BCNN_ERR_CUDA;
+    return launch(conv_branches_kernel, dim3((unsigned)gx, (unsigned)slices), THREADS, smem, stream, p, NS, tile_rows);
 }
 
 }  // namespace bcnn

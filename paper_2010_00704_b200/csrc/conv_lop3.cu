@@ -18,6 +18,8 @@ template <bool FUSED>
 __global__ void __launch_bounds__(256)
 conv_lop3_kernel(const ConvProblem p)
 {
+    pdl_trigger();
+    pdl_wait();
     __shared__ __align__(16) uint32_t As[BM * LDS_STRIDE];
     __shared__ __align__(16) uint32_t Ws[BN * LDS_STRIDE];
 
@@ -144,6 +146,8 @@ template <bool FUSED>
 __global__ void __launch_bounds__(256)
 conv_k32_kernel(const ConvProblem p)
 {
+    pdl_trigger();
+    pdl_wait();
     uint32_t w[32];       // uniform across the grid: weight words and popcount limits
     int lim[32];
 #pragma unroll
@@ -203,17 +207,11 @@ conv_k32_kernel(const ConvProblem p)
 template <bool FUSED>
 int launch_k32(const ConvProblem &p, cudaStream_t stream)
 {
-    int dev = 0, sms = 148, per_sm = 1;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, conv_k32_kernel<FUSED>, 256, 0) != cudaSuccess || per_sm < 1)
-        per_sm = 1;
     const long groups = ((long)p.M + 3) / 4;
     long blocks = (groups + 255) / 256;
-    const long wave = (long)sms * per_sm;                 // one resident wave, grid-stride beyond it
+    const long wave = (long)sm_count() * blocks_per_sm((const void *)conv_k32_kernel<FUSED>, 256, 0);   // one resident wave, grid-stride beyond it
     if (blocks > wave) blocks = wave;
-    conv_k32_kernel<FUSED><<<(unsigned)blocks, 256, 0, stream>>>(p);
-    return cudaGetLastError() == cudaSuccess ? BCNN_OK : BCNN_ERR_CUDA;
+    return launch(conv_k32_kernel<FUSED>, (unsigned)blocks, 256, 0, stream, p);
 }
 
 }  // namespace
@@ -229,11 +227,7 @@ int launch_conv_lop3(const ConvProblem &p, cudaStream_t stream)
     if (conv_lop3_pointwise_k32(p)) return p.thr ? launch_k32<true>(p, stream) : launch_k32<false>(p, stream);
     dim3 grid((unsigned)(((long)p.M + BM - 1) / BM), (p.C_out + BN - 1) / BN);
     if (grid.y > 65535) return BCNN_ERR_UNSUPPORTED;
-    if (p.thr)
-        conv_lop3_kernel<true><<<grid, 256, 0, stream>>>(p);
-    else
-        conv_lop3_kernel<false><<<grid, 256, 0, stream>>>(p);
-    return cudaGetLastError() == cudaSuccess ? BCNN_OK : BCNN_ERR_CUDA;
+    return launch(p.thr ? conv_lop3_kernel<true> : conv_lop3_kernel<false>, grid, 256, 0, stream, p);
 }
 
 }  // namespace bcnn

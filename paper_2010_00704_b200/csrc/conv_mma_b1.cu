@@ -70,6 +70,8 @@ template <int WN, int GW, bool FUSED>
 __global__ void __launch_bounds__(THREADS)
 conv_mma_b1_kernel(const ConvProblem p)
 {
+    pdl_trigger();
+    pdl_wait();
     constexpr int BN = 32 * WN;
     constexpr int WM = 8 / WN;
     constexpr int MI = BM / WM / 16;           // m16 atoms per warp
@@ -274,19 +276,9 @@ int launch_variant(const ConvProblem &p, cudaStream_t stream)
     const int smem = STAGES * (BM + BN) * ROW_BYTES;
     dim3 grid((unsigned)(((long)p.M + BM - 1) / BM), (p.C_out + BN - 1) / BN);
     if (grid.y > 65535) return BCNN_ERR_UNSUPPORTED;
-    cudaError_t e;
-    if (p.thr) {
-        auto k = conv_mma_b1_kernel<WN, GW, true>;
-        e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-        if (e != cudaSuccess) return BCNN_ERR_CUDA;
-        k<<<grid, THREADS, smem, stream>>>(p);
-    } else {
-        auto k = conv_mma_b1_kernel<WN, GW, false>;
-        e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-        if (e != cudaSuccess) return BCNN_ERR_CUDA;
-        k<<<grid, THREADS, smem, stream>>>(p);
-    }
-    return cudaGetLastError() == cudaSuccess ? BCNN_OK : BCNN_ERR_CUDA;
+    void (*k)(const ConvProblem) = p.thr ? conv_mma_b1_kernel<WN, GW, true> : conv_mma_b1_kernel<WN, GW, false>;
+    if (!allow_smem((const void *)k, smem)) return BCNN_ERR_CUDA;
+    return launch(k, grid, THREADS, smem, stream, p);
 }
 
 template <int WN>

@@ -44,6 +44,8 @@ template <int NA, bool FUSED>
 __global__ void __launch_bounds__(THREADS, 2)
 conv_mma_s8_kernel(const ConvProblem p)
 {
+    pdl_trigger();
+    pdl_wait();
     constexpr int BN = 8 * NA;
     extern __shared__ __align__(16) unsigned char smem[];
     uint2 *wfrag = reinterpret_cast<uint2 *>(smem);                 // [kwords][NA][32 lanes]
@@ -252,15 +254,11 @@ template <int NA>
 int launch_na(const ConvProblem &p, cudaStream_t stream)
 {
     const size_t smem = smem_bytes(p, NA);
-    int dev = 0, sms = 148;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    const int sms = sm_count();
     const long nblocks = ((long)p.M + 16 * MA - 1) / (16 * MA);
     void (*k)(const ConvProblem) = p.thr ? conv_mma_s8_kernel<NA, true> : conv_mma_s8_kernel<NA, false>;
-    // a property of the kernel, not of the launch: always the limit, so that captured launches stay valid
-    if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, MAX_SMEM) != cudaSuccess) return BCNN_ERR_CUDA;
-    int per_sm = 1;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, THREADS, smem) != cudaSuccess || per_sm < 1) per_sm = 1;
+    if (!allow_smem((const void *)k, MAX_SMEM)) return BCNN_ERR_CUDA;
+    const int per_sm = blocks_per_sm((const void *)k, THREADS, smem);
     // persistent grid: every resident CTA slot of the chip, split over the N tiles
     const long ny = (p.C_out + 8 * NA - 1) / (8 * NA);
     if (ny > 65535) return BCNN_ERR_UNSUPPORTED;
@@ -270,8 +268,7 @@ int launch_na(const ConvProblem &p, cudaStream_t stream)
     if (gx > cap) gx = cap;
     if (gx < 1) gx = 1;
     dim3 grid((unsigned)gx, (unsigned)ny);
-    k<<<grid, THREADS, smem, stream>>>(p);
-    return cudaGetLastError() == cudaSuccess ? BCNN_OK : BCNN_ERR_CUDA;
+    return launch(k, grid, THREADS, smem, stream, p);
 }
 
 }  // namespace

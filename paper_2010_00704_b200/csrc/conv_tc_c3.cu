@@ -174,6 +174,7 @@ conv_tc_c3_kernel(const ConvProblem p, const C3Geom g, const __grid_constant__ C
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base_smem)), "r"(512u) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
+    pdl_wait();
     // ---- one-off: expanded weights and the constant bytes.  K position e of the MMAs = channel word e / 9, tap e % 9
     // (global weight word tap * CW + channel word) -> stage e / 4, 32-byte piece e % 4; MMA row `row` carries channel ch
     for (int idx = tid; idx < (KT + 1) * BN; idx += C::THREADS) {
@@ -217,6 +218,7 @@ conv_tc_c3_kernel(const ConvProblem p, const C3Geom g, const __grid_constant__ C
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
+    pdl_trigger();
     const uint32_t tmem_base = tmem_base_smem;
     // the constant activation tile: every byte 32
     if (warp >= C::FIRST_PRODUCER_WARP && warp < C::FIRST_PRODUCER_WARP + 4) {
@@ -468,9 +470,7 @@ int launch_c3(const ConvProblem &p0, cudaStream_t stream)
     const C3Geom g = c3_geometry(p);
     const int smem = c3_smem_bytes<CW, BN>(g);
     if (smem > 227 * 1024 - 1024) return BCNN_ERR_UNSUPPORTED;
-    int dev = 0, sms = 148;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    const int sms = sm_count();
     EncodeTiledFn encode = c3_encode_fn();
     if (!encode) return BCNN_ERR_CUDA;
     // the packed input as [B][H][W * CW] 32-bit words; box = wbw words x hb rows of one image; zero fill outside
@@ -485,9 +485,8 @@ int launch_c3(const ConvProblem &p0, cudaStream_t stream)
     const unsigned grid = (unsigned)(g.total_tiles < sms ? g.total_tiles : sms);
     void (*k)(const ConvProblem, const C3Geom, const CUtensorMap) = conv_tc_c3_kernel<CW, BN>;
     const int ask = smem < 120 * 1024 ? 120 * 1024 : smem;          // one CTA per SM (it takes all of tensor memory)
-    if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024 - 1024) != cudaSuccess) return BCNN_ERR_CUDA;
-    k<<<grid, C::THREADS, ask, stream>>>(p, g, xmap);
-    return cudaGetLastError() == cudaSuccess ? BCNN_OK : BCNN_ERR_CUDA;
+    if (!allow_smem((const void *)k, 227 * 1024 - 1024)) return BCNN_ERR_CUDA;
+    return launch(k, grid, C::THREADS, ask, stream, p, g, xmap);
 }
 
 }  // namespace

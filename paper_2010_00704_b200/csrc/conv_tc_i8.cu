@@ -120,9 +120,11 @@ conv_tc_i8_kernel(const ConvProblem p, const int ktab_words)
     }
     const int gwidth = gather_width(p.cw);
     build_unit_table(p, ktab_addr, ktiles * (4 / gwidth), gwidth, tid, C::THREADS);
+    pdl_wait();
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
+    pdl_trigger();
     const uint32_t tmem_base = tmem_base_smem;
 
     if (warp == 0) {
@@ -503,9 +505,7 @@ int launch_bn(const ConvProblem &p0, cudaStream_t stream)
 {
     ConvProblem p = p0;
     p.err = device_error_word();
-    int dev = 0, sms = 148;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    const int sms = sm_count();
     const long m_tiles = ((long)p.M + BM - 1) / BM;
     const long n_tiles = ((long)p.C_out + BN - 1) / BN;
     const long total = m_tiles * n_tiles;
@@ -515,11 +515,8 @@ int launch_bn(const ConvProblem &p0, cudaStream_t stream)
     const int smem = smem_bytes<BN>(ktw, p.mode);
     if (smem > MAX_SMEM) return BCNN_ERR_UNSUPPORTED;
     void (*k)(const ConvProblem, const int) = p.mode == 2 ? conv_tc_i8_kernel<BN, 2> : (p.mode == 1 ? conv_tc_i8_kernel<BN, 1> : conv_tc_i8_kernel<BN, 0>);
-    // the attribute is a property of the kernel, not of the launch: always the limit, so that a captured
-    // launch stays valid whatever later calls with other shapes ask for
-    if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, MAX_SMEM) != cudaSuccess) return BCNN_ERR_CUDA;
-    k<<<grid, Cfg<BN>::THREADS, smem, stream>>>(p, ktw);
-    return cudaGetLastError() == cudaSuccess ? BCNN_OK : BCNN_ERR_CUDA;
+    if (!allow_smem((const void *)k, MAX_SMEM)) return BCNN_ERR_CUDA;
+    return launch(k, grid, Cfg<BN>::THREADS, smem, stream, p, ktw);
 }
 
 }  // namespace
@@ -544,9 +541,7 @@ int launch_conv_tc_i8(const ConvProblem &p, cudaStream_t stream)
     if (p.C_out > 128 && p.kwords >= 24 && p.mode != 2 && !(p.mode == 0 && p.kwords <= 144)) {
         // ... unless the narrower tiles fill the last wave so much better that they win anyway: a 128-wide tile
         // costs about 0.6 of a 256-wide one (measured on the K = 2304 and K = 4608 layers)
-        int dev = 0, sms = 148;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+        const int sms = sm_count();
         const long m_tiles = ((long)p.M + BM - 1) / BM;
         const long waves256 = (m_tiles * ((p.C_out + 255) / 256) + sms - 1) / sms;
         const long waves128 = (m_tiles * ((p.C_out + 127) / 128) + sms - 1) / sms;

@@ -118,6 +118,7 @@ conv_tc_pn_kernel(const ConvProblem p, const PnPlan plan)
         abort_flag_smem = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
+    pdl_wait();
     __syncthreads();
     // The loader warps start now: the first row tiles arrive while the other warps expand the weights (these kernels
     // run for 10 - 40 us; the weights' expansion and the first copy's latency are 1.5 - 2 us each).  The other warps meet
@@ -169,6 +170,7 @@ conv_tc_pn_kernel(const ConvProblem p, const PnPlan plan)
     tc_fence_before();
     sync_workers();
     tc_fence_after();
+    pdl_trigger();
     // the constant activation tile: every byte 32
     if (warp >= FIRST_PRODUCER_WARP && warp < FIRST_PRODUCER_WARP + 4) {
         const uint32_t c8[8] = {0x20202020u, 0x20202020u, 0x20202020u, 0x20202020u, 0x20202020u, 0x20202020u, 0x20202020u, 0x20202020u};
@@ -373,17 +375,14 @@ int launch_pn(const ConvProblem &p0, cudaStream_t stream)
     plan.m_tiles = (p.M - 1) / BM + 1;
     const int smem = 1024 + (plan.rs * KT + 1) * W_TILE_BYTES + NGRP * RD * TILE_BYTES + 128;
     if (smem > 227 * 1024 - 1024) return BCNN_ERR_UNSUPPORTED;
-    int dev = 0, sms = 148;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    const int sms = sm_count();
     int per_group = sms / plan.ng;
     if (per_group > plan.m_tiles) per_group = plan.m_tiles;
     if (per_group < 1) per_group = 1;
     void (*k)(const ConvProblem, const PnPlan) = conv_tc_pn_kernel<UPT, AW>;
     const int ask = smem < 120 * 1024 ? 120 * 1024 : smem;          // one CTA per SM (it takes all of tensor memory)
-    if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024 - 1024) != cudaSuccess) return BCNN_ERR_CUDA;
-    k<<<(unsigned)(per_group * plan.ng), THREADS, ask, stream>>>(p, plan);
-    return cudaGetLastError() == cudaSuccess ? BCNN_OK : BCNN_ERR_CUDA;
+    if (!allow_smem((const void *)k, 227 * 1024 - 1024)) return BCNN_ERR_CUDA;
+    return launch(k, (unsigned)(per_group * plan.ng), THREADS, ask, stream, p, plan);
 }
 
 }  // namespace

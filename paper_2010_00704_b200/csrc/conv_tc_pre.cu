@@ -117,9 +117,11 @@ conv_tc_pre_kernel(const ConvProblem p, const int32_t *cst, const __grid_constan
     }
     const int gwidth = gather_width(p.cw);
     build_unit_table(p, ktab_addr, ktiles * (4 / gwidth), gwidth, tid, C::THREADS);
+    pdl_wait();
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
+    pdl_trigger();
     const uint32_t tmem_base = tmem_base_smem;
 
     if (warp == 0) {
@@ -394,6 +396,8 @@ conv_tc_pre_kernel(const ConvProblem p, const int32_t *cst, const __grid_constan
 __global__ void __launch_bounds__(256)
 prepare_weights_kernel(const uint32_t *w, uint8_t *wexp, int32_t *cst, int N, int kwords, int n_pad, int k_pad)
 {
+    pdl_trigger();
+    pdl_wait();
     const int kw_pad = k_pad / 32;
     const long total = (long)n_pad * kw_pad;
     for (long i = (long)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (long)gridDim.x * blockDim.x) {
@@ -441,9 +445,7 @@ int launch_bn(const ConvProblem &p0, const PreparedWeights &pw, cudaStream_t str
 {
     ConvProblem p = p0;
     p.err = device_error_word();
-    int dev = 0, sms = 148;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    const int sms = sm_count();
     const long m_tiles = ((long)p.M + BM - 1) / BM;
     const long n_tiles = ((long)p.C_out + BN - 1) / BN;
     const long total = m_tiles * n_tiles;
@@ -463,9 +465,8 @@ int launch_bn(const ConvProblem &p0, const PreparedWeights &pw, cudaStream_t str
                CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
         return BCNN_ERR_CUDA;
     void (*k)(const ConvProblem, const int32_t *, const CUtensorMap, const int) = p.mode == 1 ? conv_tc_pre_kernel<BN, 1> : conv_tc_pre_kernel<BN, 0>;
-    if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, MAX_SMEM) != cudaSuccess) return BCNN_ERR_CUDA;
-    k<<<grid, Cfg<BN>::THREADS, smem, stream>>>(p, pw.cst, wmap, ktw);
-    return cudaGetLastError() == cudaSuccess ? BCNN_OK : BCNN_ERR_CUDA;
+    if (!allow_smem((const void *)k, MAX_SMEM)) return BCNN_ERR_CUDA;
+    return launch(k, grid, Cfg<BN>::THREADS, smem, stream, p, pw.cst, wmap, ktw);
 }
 
 }  // namespace
@@ -489,8 +490,7 @@ int launch_prepare_weights(const uint32_t *w, void *prepared, int C_out, int K, 
     int32_t *cst = reinterpret_cast<int32_t *>(wexp + (size_t)pw.n_pad * pw.k_pad);
     const long total = (long)pw.n_pad * (pw.k_pad / 32);
     const int blocks = (int)((total + 255) / 256 < 1184 ? (total + 255) / 256 : 1184);
-    prepare_weights_kernel<<<blocks, 256, 0, stream>>>(w, wexp, cst, C_out, K / 32, pw.n_pad, pw.k_pad);
-    return cudaGetLastError() == cudaSuccess ? BCNN_OK : BCNN_ERR_CUDA;
+    return launch(prepare_weights_kernel, blocks, 256, 0, stream, w, wexp, cst, C_out, K / 32, pw.n_pad, pw.k_pad);
 }
 
 // ---- the variant that allocates nothing -------------------------------------------------------------------------
@@ -557,9 +557,7 @@ int launch_conv_tc_pre(const ConvProblem &p, const void *prepared, cudaStream_t 
     // 256-wide tiles have a single accumulator buffer (their epilogue is not overlapped): worth it when the K loop is
     // long and the narrower tiles do not fill the last wave so much better (as in the streaming engine)
     if (p.C_out > 128 && p.kwords >= 24) {
-        int dev = 0, sms = 148;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+        const int sms = sm_count();
         const long m_tiles = ((long)p.M + BM - 1) / BM;
         const long waves256 = (m_tiles * ((p.C_out + 255) / 256) + sms - 1) / sms;
         const long waves128 = (m_tiles * ((p.C_out + 127) / 128) + sms - 1) / sms;

@@ -152,6 +152,7 @@ conv_tc_pw_kernel(const ConvProblem p)
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base_smem)), "r"(512u) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
+    pdl_wait();
     // ---- one-off: expanded weights and constant bytes; MMA row `row` carries channel 32 * (row / 32) + channel_of_column(row % 32)
     for (int row = tid; row < BN; row += C::THREADS) {
         const int ch = (row & ~31) + channel_of_column(row & 31);
@@ -189,6 +190,7 @@ conv_tc_pw_kernel(const ConvProblem p)
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
+    pdl_trigger();
     const uint32_t tmem_base = tmem_base_smem;
     // the constant activation tile: every byte 32 (one producer group writes its four lane quadrants)
     if (warp >= C::FIRST_PRODUCER_WARP && warp < C::FIRST_PRODUCER_WARP + 4) {
@@ -399,15 +401,12 @@ int launch_pw(const ConvProblem &p0, cudaStream_t stream)
     using C = PwCfg<KW, BN>;
     ConvProblem p = p0;
     p.err = device_error_word();
-    int dev = 0, sms = 148;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    const int sms = sm_count();
     const long n_blocks = ((long)p.M + C::BLOCK_ROWS - 1) / C::BLOCK_ROWS;
     const unsigned grid = (unsigned)(n_blocks < sms ? n_blocks : sms);
     void (*k)(const ConvProblem) = conv_tc_pw_kernel<KW, BN>;
-    if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM_ASK) != cudaSuccess) return BCNN_ERR_CUDA;
-    k<<<grid, C::THREADS, C::SMEM_ASK, stream>>>(p);
-    return cudaGetLastError() == cudaSuccess ? BCNN_OK : BCNN_ERR_CUDA;
+    if (!allow_smem((const void *)k, C::SMEM_ASK)) return BCNN_ERR_CUDA;
+    return launch(k, grid, C::THREADS, C::SMEM_ASK, stream, p);
 }
 
 template <int KW>

@@ -159,7 +159,10 @@ conv_tc_ws_kernel(const ConvProblem p)
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
 
-    // ---- one-off: expand the weight tile, per-channel constants, K-word table
+    const int gw = gather_width(p.cw);
+    build_unit_table(p, ktab_addr, ktiles * (4 / gw), gw, tid, C::THREADS);
+    pdl_wait();
+    // ---- one-off: expand the weight tile, per-channel constants
     for (int idx = tid; idx < ktiles * BN; idx += C::THREADS) {
         const int kt = idx / BN, row = idx - kt * BN;
         const uint32_t row_addr = wexp + (uint32_t)kt * C::W_TILE_BYTES + (uint32_t)row * ROWB;
@@ -188,12 +191,11 @@ conv_tc_ws_kernel(const ConvProblem p)
         cst *= 32;
         asm volatile("st.shared.b32 [%0], %1;" ::"r"(colc_addr + 4u * c), "r"(cst) : "memory");
     }
-    const int gw = gather_width(p.cw);
-    build_unit_table(p, ktab_addr, ktiles * (4 / gw), gw, tid, C::THREADS);
     fence_async_proxy();
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
+    pdl_trigger();
     const uint32_t tmem_base = tmem_base_smem;
 
     if (warp == 0) {
@@ -544,9 +546,7 @@ int launch_ws(const ConvProblem &p0, cudaStream_t stream)
 {
     ConvProblem p = p0;
     p.err = device_error_word();
-    int dev = 0, sms = 148;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    const int sms = sm_count();
     using C = Cfg<BN, G, DUAL, TEAMS>;
     const WsLayout L = ws_layout<BN, G, DUAL, TEAMS>(p.kwords, p.mode);
     const long m_tiles = ((long)p.M + BM - 1) / BM;
@@ -558,11 +558,8 @@ int launch_ws(const ConvProblem &p0, cudaStream_t stream)
     const unsigned grid = (unsigned)(per_slice * n_tiles);
     void (*k)(const ConvProblem) = p.mode == 2 ? conv_tc_ws_kernel<BN, G, DUAL, 2, TEAMS>
                                    : (p.mode == 1 ? conv_tc_ws_kernel<BN, G, DUAL, 1, TEAMS> : conv_tc_ws_kernel<BN, G, DUAL, 0, TEAMS>);
-    // the attribute is a property of the kernel, not of the launch: always the configuration's limit, so
-    // that a captured launch stays valid whatever later calls with other shapes ask for
-    if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, DUAL ? 113 * 1024 : MAX_SMEM - 1024) != cudaSuccess) return BCNN_ERR_CUDA;
-    k<<<grid, C::THREADS, L.smem, stream>>>(p);
-    return cudaGetLastError() == cudaSuccess ? BCNN_OK : BCNN_ERR_CUDA;
+    if (!allow_smem((const void *)k, DUAL ? 113 * 1024 : MAX_SMEM - 1024)) return BCNN_ERR_CUDA;
+    return launch(k, grid, C::THREADS, L.smem, stream, p);
 }
 
 // The expanded weights, the packed-word staging ring and the tables must fit in shared memory

@@ -16,6 +16,8 @@ __global__ void __launch_bounds__(256)
 pack_stream_kernel(const float *__restrict__ x, const float *__restrict__ bias,
                    uint32_t *__restrict__ out, long nwords, int cwords)
 {
+    pdl_trigger();
+    pdl_wait();
     const int lane = threadIdx.x & 31;
     const long warp = (long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
     const long nwarps = (long)gridDim.x * (blockDim.x >> 5);
@@ -53,6 +55,8 @@ __global__ void __launch_bounds__(256)
 pack_general_kernel(const float *__restrict__ x, const float *__restrict__ bias,
                     uint32_t *__restrict__ out, long nwords, int C_in, int cwords)
 {
+    pdl_trigger();
+    pdl_wait();
     const int lane = threadIdx.x & 31;
     const long warp = (long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
     const long nwarps = (long)gridDim.x * (blockDim.x >> 5);
@@ -79,6 +83,8 @@ __global__ void __launch_bounds__(256)
 pack_c4r8_kernel(const float4 *__restrict__ x, const float *__restrict__ bias,
                  uint32_t *__restrict__ out, long npix)
 {
+    pdl_trigger();
+    pdl_wait();
     constexpr int U = 4;                       // pixels in flight per thread
     __shared__ float sb[32];
     __shared__ float sts[4][8];                // sorted thresholds of input i
@@ -176,9 +182,7 @@ int launch_pack(const float *x, const float *bias, uint32_t *out, long npix, int
     const int C = C_in * R;
     const int cwords = C / 32;
     const long nwords = npix * cwords;
-    int dev = 0, sms = 148;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    const int sms = sm_count();
     const int threads = 256;
     if (R == 1 && C_in % 32 == 0) {
         constexpr int UNROLL = 8;
@@ -187,26 +191,20 @@ int launch_pack(const float *x, const float *bias, uint32_t *out, long npix, int
         const long cap = (long)sms * 8;
         if (blocks > cap) blocks = cap;
         if (blocks < 1) blocks = 1;
-        if (bias)
-            pack_stream_kernel<UNROLL, true><<<(int)blocks, threads, 0, stream>>>(x, bias, out, nwords, cwords);
-        else
-            pack_stream_kernel<UNROLL, false><<<(int)blocks, threads, 0, stream>>>(x, bias, out, nwords, cwords);
+        return launch(bias ? pack_stream_kernel<UNROLL, true> : pack_stream_kernel<UNROLL, false>, (unsigned)blocks, threads, 0, stream,
+                      x, bias, out, nwords, cwords);
     } else if (C_in == 4 && R == 8) {
         long blocks = (npix + threads * 4 - 1) / (threads * 4);
-        int per_sm = 4;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, pack_c4r8_kernel, threads, 0) != cudaSuccess || per_sm < 1)
-            per_sm = 4;
-        const long cap = (long)sms * per_sm;       // one wave of resident CTAs, grid-stride inside
+        const long cap = (long)sms * blocks_per_sm((const void *)pack_c4r8_kernel, threads, 0);       // one wave of resident CTAs, grid-stride inside
         if (blocks > cap) blocks = cap;
         if (blocks < 1) blocks = 1;
-        pack_c4r8_kernel<<<(int)blocks, threads, 0, stream>>>(reinterpret_cast<const float4 *>(x), bias, out, npix);
+        return launch(pack_c4r8_kernel, (unsigned)blocks, threads, 0, stream, reinterpret_cast<const float4 *>(x), bias, out, npix);
     } else {
         long blocks = (nwords + 7) / 8;
         const long cap = (long)sms * 8;
         if (blocks > cap) blocks = cap;
-        pack_general_kernel<<<(int)blocks, threads, 0, stream>>>(x, bias, out, nwords, C_in, cwords);
+        return launch(pack_general_kernel, (unsigned)blocks, threads, 0, stream, x, bias, out, nwords, C_in, cwords);
     }
-    return cudaGetLastError() == cudaSuccess ? BCNN_OK : BCNN_ERR_CUDA;
 }
 
 }  // namespace bcnn

@@ -34,6 +34,8 @@ __global__ void __launch_bounds__(128, 1) selftest_wait_timeout_kernel(int *err,
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
+    pdl_trigger();
+    pdl_wait();
     const uint32_t tmem_base = tmem_base_smem;
     if (warp == 1) {
         mbar_wait_warp(smem_u32(&bars[0]), 0, abort_flag, err, BCNN_SELFTEST_TIMEOUT_CODE, polls);
@@ -52,8 +54,7 @@ int launch_selftest_wait_timeout(int polls, cudaStream_t stream)
 {
     int *err = device_error_word();
     if (!err) return BCNN_ERR_CUDA;
-    selftest_wait_timeout_kernel<<<1, 128, 0, stream>>>(err, (uint32_t)polls);
-    return cudaGetLastError() == cudaSuccess ? BCNN_OK : BCNN_ERR_CUDA;
+    return launch(selftest_wait_timeout_kernel, 1, 128, 0, stream, err, (uint32_t)polls);
 }
 
 }  // namespace bcnn

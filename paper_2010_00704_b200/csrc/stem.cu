@@ -31,6 +31,8 @@ __global__ void __launch_bounds__(STEM_THREADS, 1)
 stem_c4r8_k32_kernel(const float4 *__restrict__ x, const float *__restrict__ bias, const uint32_t *__restrict__ w,
                      const int32_t *__restrict__ thr, uint32_t *__restrict__ out, long npix)
 {
+    pdl_trigger();
+    pdl_wait();
     constexpr int U = 4;                        // pixels in flight per thread
     __shared__ float sb[32];
     __shared__ float sts[4][8];                 // sorted thresholds of input i
@@ -161,14 +163,11 @@ stem_c4r8_k32_kernel(const float4 *__restrict__ x, const float *__restrict__ bia
 int launch_stem_c4r8_k32(const float *x, const float *bias, const uint32_t *w, const int32_t *thr, uint32_t *out,
                          long npix, cudaStream_t stream)
 {
-    int dev = 0, sms = 148;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    const int sms = sm_count();
     long blocks = (npix + STEM_THREADS * 4 - 1) / (STEM_THREADS * 4);
     if (blocks > sms) blocks = sms;             // one resident CTA per SM builds the table once, grid-stride inside
     if (blocks < 1) blocks = 1;
-    stem_c4r8_k32_kernel<<<(int)blocks, STEM_THREADS, 0, stream>>>(reinterpret_cast<const float4 *>(x), bias, w, thr, out, npix);
-    return cudaGetLastError() == cudaSuccess ? BCNN_OK : BCNN_ERR_CUDA;
+    return launch(stem_c4r8_k32_kernel, (unsigned)blocks, STEM_THREADS, 0, stream, reinterpret_cast<const float4 *>(x), bias, w, thr, out, npix);
 }
 
 }  // namespace bcnn
