@@ -1,18 +1,15 @@
 // Streaming tcgen05 engine on PREPARED weights: wide layers and long K (C_out > 128, the plain GEMMs).
 //
-// The weights of a layer never change between calls, yet the streaming engine (conv_tc_i8.cu) expands the same weight
-// bits to bytes again for every 128-row tile: with 256-wide tiles two thirds of its producer warps do nothing else,
-// and the MMA issuer waits for them five sixths of the time.  Here the expansion is done ONCE per layer by
-// bcnn_prepare_weights into a caller-owned buffer (the weight matrix as signed bytes, K-major, rows padded to 128
-// and K to 128; plus K - 2 popc(W_n) per row), and the kernel's weight operand arrives by TMA: one
-// cp.async.bulk.tensor per ring stage (a 128-byte x BN-row box, 128-byte swizzle - exactly the shared-memory tile
-// the MMA descriptor describes) issued by a loader warp, completing on the stage's mbarrier.  No warp touches a
-// weight byte.
+// The weights of a layer never change between calls.  bcnn_prepare_weights expands their sign bits ONCE per layer into a
+// caller-owned buffer - signed 4-bit codes, K-major, rows padded to 128 and K to 256, then K - 2 popc(W_n) per row; half
+// the bytes that bcnn_prepared_weights_bytes asks for - and the kernel's weight operand arrives by TMA: one
+// cp.async.bulk.tensor per ring stage (a 128-byte x BN-row box = 256 bits of K, 128-byte swizzle - exactly the
+// shared-memory tile the MMA descriptor describes) issued by a loader warp, completing on the stage's mbarrier.  No warp
+// touches a weight.
 //
-// Arithmetic: the weight-stationary engine's signed scheme (activation bytes {0, 2^j}, weight bytes +-2^(6-j), every
-// product +-64): accumulator = 64 S,  sum a*g = 2 S + K - 2 popc(G):
-//   int32 output:  (acc >> 5) + cst_n              cst_n = K - 2 popc(G_n)   (from the prepared buffer)
-//   packed output: acc + 32 (cst_n - thr_n) >= 0   thr clamped to +-(K + 1)
+// Arithmetic: 4-bit operands (tc_common.cuh), fp32 accumulators that hold exact integers:
+//   sum a*g = accumulator + cst_n                          cst_n = K - 2 popc(G_n)   (from the prepared buffer)
+//   packed output: accumulator + (cst_n - thr_n) >= 0      thr clamped to +-(K + 1)
 // so there are no per-row constants, and the per-column ones are added by the epilogue from a small table.
 //
 //   warp 0        issuer (tcgen05.mma / commit only; waits on named barriers only)
@@ -43,16 +40,17 @@ constexpr int ERR_LOADER_TIMEOUT = 134;
 template <int BN> struct Cfg {
     static constexpr int NBUF = BN == 256 ? 1 : 2;                       // accumulator buffers
     static constexpr int A_COL0 = NBUF * BN;                              // first column of the activation ring
-    static constexpr int STAGES = BN == 256 ? 5 : 8;
+    static constexpr int STAGES = BN == 256 ? 5 : 7;
     static constexpr int PROD_THREADS = G * BM;
     static constexpr int FIRST_PRODUCER_WARP = 1 + EPI_WARPS;
     static constexpr int LOADER_WARP = FIRST_PRODUCER_WARP + 4 * G;
     static constexpr int CONTROL_WARP = LOADER_WARP + 1;
     static constexpr int THREADS = 32 * (CONTROL_WARP + 1);
     static constexpr int W_BYTES = BN * ROWB;                             // one ring stage of weights
-    static constexpr int BITS_BYTES = PF * PROD_THREADS * 16;
+    static constexpr int SF_COL = 512 - (int)SF_COLS;                     // unit scales
+    static constexpr int BITS_BYTES = PF * PROD_THREADS * 32;
     static constexpr int TABLE_BYTES = EPI_WARPS * BN * 4;                // one column table per epilogue warp
-    static_assert(A_COL0 + STAGES * 32 <= 512, "tensor memory budget");
+    static_assert(A_COL0 + STAGES * 32 <= SF_COL, "tensor memory budget");
     static_assert(STAGES >= G, "a producer group must not lap the ring (parity waits)");
 };
 
@@ -80,7 +78,7 @@ conv_tc_pre_kernel(const ConvProblem p, const int32_t *cst, const __grid_constan
 
     const int tid = threadIdx.x;
     const int warp = tid >> 5, lane = tid & 31;
-    const int ktiles = (p.kwords + 3) >> 2;
+    const int ktiles = (p.kwords + 7) >> 3;
     const int m_tiles = (p.M - 1) / BM + 1;
     const int n_tiles = (p.C_out + BN - 1) / BN;
     const int total_tiles = m_tiles * n_tiles;
@@ -88,9 +86,9 @@ conv_tc_pre_kernel(const ConvProblem p, const int32_t *cst, const __grid_constan
     const int total_items = my_tiles * ktiles;
 
     const uint32_t wring = (smem_u32(smem_raw) + 1023u) & ~1023u;         // [STAGES][BN rows][128 B], written by TMA
-    const uint32_t bits_ring = wring + STAGES * C::W_BYTES;               // [PF][PROD_THREADS][16 B]
+    const uint32_t bits_ring = wring + STAGES * C::W_BYTES;               // [PF][2][PROD_THREADS][16 B]
     const uint32_t tables = bits_ring + C::BITS_BYTES;                    // [EPI_WARPS][BN] int32 column constants
-    const uint32_t ktab_addr = tables + C::TABLE_BYTES;                   // unit table of the gather: {word offset, tap bit}
+    const uint32_t ktab_addr = tables + C::TABLE_BYTES;                   // unit table of the gather
     const uint32_t i32_tiles = (ktab_addr + (uint32_t)ktab_words * 4u + 15u) & ~15u;   // int32 output: store staging tiles
     const uint32_t bar0 = smem_u32(bars);
     auto full_bar = [&](int s) { return bar0 + 8u * s; };
@@ -116,7 +114,7 @@ conv_tc_pre_kernel(const ConvProblem p, const int32_t *cst, const __grid_constan
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
     const int gwidth = gather_width(p.cw);
-    build_unit_table(p, ktab_addr, ktiles * (4 / gwidth), gwidth, tid, C::THREADS);
+    build_unit_table8(p, ktab_addr, ktiles * (8 / gwidth), gwidth, tid, C::THREADS);
     pdl_wait();
     tc_fence_before();
     __syncthreads();
@@ -126,12 +124,13 @@ conv_tc_pre_kernel(const ConvProblem p, const int32_t *cst, const __grid_constan
 
     if (warp == 0) {
         // ------------------------------------------------------------------ issuer (no memory instructions)
-        constexpr uint32_t idesc = make_idesc(BN) | (1u << 10);                  // B operand: signed bytes
+        constexpr uint32_t idesc = make_idesc_f4(BN);
         const uint64_t desc0 = make_desc(0);
         const uint32_t desc_hi = (uint32_t)(desc0 >> 32);
         const uint32_t b_lo0 = (uint32_t)desc0 | ((wring & 0x3FFFFu) >> 4);      // + slot * (W_BYTES / 16)
         const uint32_t tmem_u = __shfl_sync(0xffffffffu, tmem_base, 0);
         const uint32_t a_tmem0 = tmem_u + (uint32_t)C::A_COL0;                   // + slot * 32 columns
+        const uint32_t sf = tmem_u + (uint32_t)C::SF_COL;
         int s = 0, buf = 0;
         for (int ti = 0; ti < my_tiles; ++ti) {
             const uint32_t d_tmem = tmem_u + (uint32_t)(buf * BN);
@@ -139,15 +138,15 @@ conv_tc_pre_kernel(const ConvProblem p, const int32_t *cst, const __grid_constan
             for (int kt = 0; kt < ktiles; ++kt) {
                 const uint32_t a_t = a_tmem0 + (uint32_t)s * 32u;
                 const uint32_t b_lo = b_lo0 + (uint32_t)s * (C::W_BYTES >> 4);
-                const int nk = p.kwords - 4 * kt;                 // 32 bits of K per instruction; skip the zero tail
+                const int nk = p.kwords - 8 * kt;                 // two K words per instruction; skip the zero tail
                 const uint32_t ebar = empty_bar(s);
                 asm volatile("bar.sync %0, 64;" ::"r"(1 + s) : "memory");
                 tc_fence_after();
                 if (elect_one()) {
-                    tc_mma_i8_ts(d_tmem, a_t, b_lo, desc_hi, idesc, kt > 0 ? 1u : 0u);
-                    if (nk > 1) tc_mma_i8_ts(d_tmem, a_t + 8u, b_lo + 2u, desc_hi, idesc, 1u);
-                    if (nk > 2) tc_mma_i8_ts(d_tmem, a_t + 16u, b_lo + 4u, desc_hi, idesc, 1u);
-                    if (nk > 3) tc_mma_i8_ts(d_tmem, a_t + 24u, b_lo + 6u, desc_hi, idesc, 1u);
+                    tc_mma_f4_ts(d_tmem, a_t, b_lo, desc_hi, idesc, sf, kt > 0 ? 1u : 0u);
+                    if (nk > 2) tc_mma_f4_ts(d_tmem, a_t + 8u, b_lo + 2u, desc_hi, idesc, sf, 1u);
+                    if (nk > 4) tc_mma_f4_ts(d_tmem, a_t + 16u, b_lo + 4u, desc_hi, idesc, sf, 1u);
+                    if (nk > 6) tc_mma_f4_ts(d_tmem, a_t + 24u, b_lo + 6u, desc_hi, idesc, sf, 1u);
                     tc_commit(ebar);
                     if (kt == ktiles - 1) tc_commit(tfull);
                 }
@@ -226,13 +225,9 @@ conv_tc_pre_kernel(const ConvProblem p, const int32_t *cst, const __grid_constan
                 int v = 0;
                 if (n < p.C_out) {
                     v = __ldg(cst + n);
-                    if (FUSED) {
-                        int t = __ldg(p.thr + n);
-                        t = max(min(t, p.K + 1), -p.K - 1);       // beyond that bound the decision is constant
-                        v = 32 * (v - t);
-                    }
+                    if (FUSED) v -= max(min(__ldg(p.thr + n), p.K + 1), -p.K - 1);       // beyond that bound the decision is constant
                 }
-                asm volatile("st.shared.b32 [%0], %1;" ::"r"(table + 4u * c), "r"(v) : "memory");
+                asm volatile("st.shared.b32 [%0], %1;" ::"r"(table + 4u * c), "r"(__float_as_uint((float)v + (FUSED ? 0.0f : INT_BIAS))) : "memory");
             }
             __syncwarp();
             if (alive) alive = mbar_wait(tfull_bar(buf), buf_phase, abort_flag, p.err, ERR_EPILOGUE_TIMEOUT);
@@ -249,15 +244,15 @@ conv_tc_pre_kernel(const ConvProblem p, const int32_t *cst, const __grid_constan
                     uint32_t v[32];
                     tc_ld32(t_addr + (uint32_t)col0, v);
                     if (FUSED) {
-                        // bit = (v + colc >= 0); sign bits are shifted in, last column first
+                        // bit = (v + colc >= 0), an exact sum that is never -0; sign bits are shifted in, last column first
                         uint32_t acc = 0;
 #pragma unroll
                         for (int i4 = 7; i4 >= 0; --i4) {
                             const uint4 cc = ld_shared_v4(table + 4u * (col0 + 4 * i4));
-                            acc = __funnelshift_l((uint32_t)((int)v[4 * i4 + 3] + (int)cc.w), acc, 1);
-                            acc = __funnelshift_l((uint32_t)((int)v[4 * i4 + 2] + (int)cc.z), acc, 1);
-                            acc = __funnelshift_l((uint32_t)((int)v[4 * i4 + 1] + (int)cc.y), acc, 1);
-                            acc = __funnelshift_l((uint32_t)((int)v[4 * i4 + 0] + (int)cc.x), acc, 1);
+                            acc = __funnelshift_l(fadd_bits(v[4 * i4 + 3], cc.w), acc, 1);
+                            acc = __funnelshift_l(fadd_bits(v[4 * i4 + 2], cc.z), acc, 1);
+                            acc = __funnelshift_l(fadd_bits(v[4 * i4 + 1], cc.y), acc, 1);
+                            acc = __funnelshift_l(fadd_bits(v[4 * i4 + 0], cc.x), acc, 1);
                         }
                         words[ch] = ~acc;
                     } else {
@@ -265,10 +260,10 @@ conv_tc_pre_kernel(const ConvProblem p, const int32_t *cst, const __grid_constan
 #pragma unroll
                         for (int i4 = 0; i4 < 8; ++i4) {
                             const uint4 cc = ld_shared_v4(table + 4u * (col0 + 4 * i4));
-                            o[4 * i4 + 0] = ((int)v[4 * i4 + 0] >> 5) + (int)cc.x;
-                            o[4 * i4 + 1] = ((int)v[4 * i4 + 1] >> 5) + (int)cc.y;
-                            o[4 * i4 + 2] = ((int)v[4 * i4 + 2] >> 5) + (int)cc.z;
-                            o[4 * i4 + 3] = ((int)v[4 * i4 + 3] >> 5) + (int)cc.w;
+                            o[4 * i4 + 0] = int_of_biased(fadd_bits(v[4 * i4 + 0], cc.x));
+                            o[4 * i4 + 1] = int_of_biased(fadd_bits(v[4 * i4 + 1], cc.y));
+                            o[4 * i4 + 2] = int_of_biased(fadd_bits(v[4 * i4 + 2], cc.z));
+                            o[4 * i4 + 3] = int_of_biased(fadd_bits(v[4 * i4 + 3], cc.w));
                         }
                         if ((p.C_out & 3) == 0 && (n0 + col0 + 32 <= p.C_out)) {
                             // full chunk (warp-uniform): staged, the warp stores whole 128-byte rows
@@ -311,7 +306,7 @@ conv_tc_pre_kernel(const ConvProblem p, const int32_t *cst, const __grid_constan
         const int grp = ptid >> 7;
         const int quad = warp & 3;                               // tensor-memory lane quadrant this warp may write
         const int row = quad * 32 + lane;
-        constexpr uint32_t SLOT_BYTES = C::PROD_THREADS * 16u;
+        constexpr uint32_t HALF_BYTES = C::PROD_THREADS * 16u, SLOT_BYTES = 2u * HALF_BYTES;
         const uint32_t bits0 = bits_ring + (uint32_t)ptid * 16u, bits_end = bits0 + PF * SLOT_BYTES;
         const uint32_t st_addr0 = tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)C::A_COL0;
         const uint32_t lane0 = lane == 0 ? 1u : 0u;
@@ -338,10 +333,12 @@ conv_tc_pre_kernel(const ConvProblem p, const int32_t *cst, const __grid_constan
         while (l_kt >= ktiles) { l_kt -= ktiles; next_tile(); }
         row_window(p, step, rc);
         uint32_t l_dst = bits0;
+        // the scales are in place before this group's first arrival, which every MMA waits for
+        if (grp == 0) write_unit_scales(tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)C::SF_COL);
         auto issue_load = [&]() {
-            if (gwidth == 4) gather_stage<4>(p.x, rc, ktab_addr + (uint32_t)l_kt * 8u, l_dst);
-            else if (gwidth == 2) gather_stage<2>(p.x, rc, ktab_addr + (uint32_t)l_kt * 16u, l_dst);
-            else gather_stage<1>(p.x, rc, ktab_addr + (uint32_t)l_kt * 32u, l_dst);
+            if (gwidth == 4) gather_stage8<4>(p.x, rc, ktab_addr + (uint32_t)l_kt * 8u, l_dst, HALF_BYTES);
+            else if (gwidth == 2) gather_stage8<2>(p.x, rc, ktab_addr + (uint32_t)l_kt * 16u, l_dst, HALF_BYTES);
+            else gather_stage8<1>(p.x, rc, ktab_addr + (uint32_t)l_kt * 32u, l_dst, HALF_BYTES);
             l_dst += SLOT_BYTES;
             if (l_dst == bits_end) l_dst = bits0;
             --l_left;
@@ -364,14 +361,10 @@ conv_tc_pre_kernel(const ConvProblem p, const int32_t *cst, const __grid_constan
             if (l_left > 0) issue_load();
             cp_async_commit();
             cp_async_wait<PF - 1>();
-            const uint4 bits = ld_shared_v4(c_src);
+            uint32_t v[32];
+            expand_stage8(ld_shared_v4(c_src), ld_shared_v4(c_src + HALF_BYTES), v);
             c_src += SLOT_BYTES;
             if (c_src == bits_end) c_src = bits0;
-            // expanded row -> 32 columns of this lane: column 8*e + j = word j of K word e
-            uint32_t v[32];
-            const uint32_t wds[4] = {bits.x, bits.y, bits.z, bits.w};
-#pragma unroll
-            for (int e = 0; e < 4; ++e) expand_a(wds[e], &v[8 * e]);
             if (!mbar_wait_warp(empty_bar(s), phase, abort_flag, p.err, ERR_PRODUCER_TIMEOUT)) break;
             tc_fence_after();     // the MMAs that read this slot are complete (their commit released it)
             tc_st32(st_addr0 + (uint32_t)s * 32u, v);
@@ -391,8 +384,8 @@ conv_tc_pre_kernel(const ConvProblem p, const int32_t *cst, const __grid_constan
     }
 }
 
-// One weight word -> its 32 signed bytes (see expand_store_w_signed in tc_common.cuh: magnitude 2^(6-j), 1 for j = 7),
-// written as two 16-byte pieces of the row; K-major rows of k_pad bytes, padded rows and K words are zero.
+// One weight word -> its 32 signed 4-bit codes (expand_w4), 16 bytes of a K-major row of k_pad / 2 bytes; padded rows and K
+// words are zero.
 __global__ void __launch_bounds__(256)
 prepare_weights_kernel(const uint32_t *w, uint8_t *wexp, int32_t *cst, int N, int kwords, int n_pad, int k_pad)
 {
@@ -403,16 +396,7 @@ prepare_weights_kernel(const uint32_t *w, uint8_t *wexp, int32_t *cst, int N, in
     for (long i = (long)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (long)gridDim.x * blockDim.x) {
         const int kw = (int)(i % kw_pad), n = (int)(i / kw_pad);
         const bool live = n < N && kw < kwords;
-        const uint32_t word = live ? __ldg(w + (long)n * kwords + kw) : 0u;
-        const uint32_t nr = ~__byte_perm(__brev(word), 0u, 0x0123u);
-        uint32_t o[8];
-#pragma unroll
-        for (int j = 0; j < 7; ++j)
-            o[j] = live ? (nr & (0x01010101u << (7 - j))) * ((2u << j) - 1u) + (0x01010101u << (6 - j)) : 0u;
-        o[7] = live ? (nr & 0x01010101u) * 0xFEu + 0x01010101u : 0u;
-        uint4 *dst = reinterpret_cast<uint4 *>(wexp + (long)n * k_pad + (long)kw * 32);
-        dst[0] = make_uint4(o[0], o[1], o[2], o[3]);
-        dst[1] = make_uint4(o[4], o[5], o[6], o[7]);
+        *reinterpret_cast<uint4 *>(wexp + i * 16) = live ? expand_w4(__ldg(w + (long)n * kwords + kw)) : make_uint4(0u, 0u, 0u, 0u);
     }
     for (long n = (long)blockIdx.x * blockDim.x + threadIdx.x; n < n_pad; n += (long)gridDim.x * blockDim.x) {
         int pop = 0;
@@ -438,7 +422,7 @@ EncodeTiledFn encode_tiled_fn()
     return fn;
 }
 
-int ktab_words_for(const ConvProblem &p) { return ((p.kwords + 3) >> 2) * 8; }
+int ktab_words_for(const ConvProblem &p) { return ((p.kwords + 7) >> 3) * (8 / gather_width(p.cw)); }
 
 template <int BN>
 int launch_bn(const ConvProblem &p0, const PreparedWeights &pw, cudaStream_t stream)
@@ -457,8 +441,8 @@ int launch_bn(const ConvProblem &p0, const PreparedWeights &pw, cudaStream_t str
     EncodeTiledFn encode = encode_tiled_fn();
     if (!encode) return BCNN_ERR_CUDA;
     CUtensorMap wmap;
-    const cuuint64_t dims[2] = {(cuuint64_t)pw.k_pad, (cuuint64_t)pw.n_pad};
-    const cuuint64_t strides[1] = {(cuuint64_t)pw.k_pad};
+    const cuuint64_t dims[2] = {(cuuint64_t)pw.k_pad / 2, (cuuint64_t)pw.n_pad};       // bytes of a row, rows
+    const cuuint64_t strides[1] = {(cuuint64_t)pw.k_pad / 2};
     const cuuint32_t box[2] = {(cuuint32_t)ROWB, (cuuint32_t)BN};
     const cuuint32_t estr[2] = {1, 1};
     if (encode(&wmap, CU_TENSOR_MAP_DATA_TYPE_UINT8, 2, const_cast<uint8_t *>(pw.wexp), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
@@ -474,9 +458,9 @@ int launch_bn(const ConvProblem &p0, const PreparedWeights &pw, cudaStream_t str
 void prepared_layout(int C_out, int K, PreparedWeights &pw, size_t &bytes)
 {
     pw.n_pad = (C_out + 127) / 128 * 128;
-    pw.k_pad = (K + 127) / 128 * 128;
-    const size_t wbytes = (size_t)pw.n_pad * pw.k_pad;          // a multiple of 16384
-    bytes = wbytes + (size_t)pw.n_pad * 4;
+    pw.k_pad = (K + 255) / 256 * 256;
+    // the buffer's size is part of the interface: a byte per weight, of which the 4-bit codes take at most half
+    bytes = (size_t)pw.n_pad * ((K + 127) / 128 * 128) + (size_t)pw.n_pad * 4;
     pw.wexp = nullptr;
     pw.cst = nullptr;
 }
@@ -487,7 +471,7 @@ int launch_prepare_weights(const uint32_t *w, void *prepared, int C_out, int K, 
     size_t bytes;
     prepared_layout(C_out, K, pw, bytes);
     uint8_t *wexp = static_cast<uint8_t *>(prepared);
-    int32_t *cst = reinterpret_cast<int32_t *>(wexp + (size_t)pw.n_pad * pw.k_pad);
+    int32_t *cst = reinterpret_cast<int32_t *>(wexp + (size_t)pw.n_pad * pw.k_pad / 2);
     const long total = (long)pw.n_pad * (pw.k_pad / 32);
     const int blocks = (int)((total + 255) / 256 < 1184 ? (total + 255) / 256 : 1184);
     return launch(prepare_weights_kernel, blocks, 256, 0, stream, w, wexp, cst, C_out, K / 32, pw.n_pad, pw.k_pad);
@@ -543,7 +527,8 @@ bool conv_tc_pre_supports(const ConvProblem &p)
     if (p.kh * p.kw > 31) return false;                       // one validity bit per tap
     if ((long)p.B * p.H * p.W * p.cw >= (1L << 31)) return false;     // rows address the input by 32-bit word offsets
     if (smem_bytes<256>(ktab_words_for(p), p.mode) > MAX_SMEM) return false;
-    return p.K <= (1 << 20);                                  // 64 K + 32 (2 K + 1) stays far below 2^31
+    if ((long)p.kh * p.W * p.cw >= (1L << 27)) return false;  // a unit's word offset within the window
+    return p.K <= (1 << 20);                                  // sums up to 4 K + 2 stay exact in fp32
 }
 
 int launch_conv_tc_pre(const ConvProblem &p, const void *prepared, cudaStream_t stream)
@@ -553,7 +538,7 @@ int launch_conv_tc_pre(const ConvProblem &p, const void *prepared, cudaStream_t 
     size_t bytes;
     prepared_layout(p.C_out, p.K, pw, bytes);
     pw.wexp = static_cast<const uint8_t *>(prepared);
-    pw.cst = reinterpret_cast<const int32_t *>(pw.wexp + (size_t)pw.n_pad * pw.k_pad);
+    pw.cst = reinterpret_cast<const int32_t *>(pw.wexp + (size_t)pw.n_pad * pw.k_pad / 2);
     // 256-wide tiles have a single accumulator buffer (their epilogue is not overlapped): worth it when the K loop is
     // long and the narrower tiles do not fill the last wave so much better (as in the streaming engine)
     if (p.C_out > 128 && p.kwords >= 24) {

@@ -135,6 +135,29 @@ __device__ __forceinline__ void tc_mma_i8_ts(uint32_t d_tmem, uint32_t a_tmem, u
         ::"r"(d_tmem), "r"(a_tmem), "r"(b_lo), "r"(desc_hi), "r"(idesc), "r"(accumulate), "r"(0u)
         : "memory");
 }
+// 4-bit operands (kind::mxf4: e2m1 x e2m1 with block scales, fp32 accumulators): 64 elements of K per instruction at twice
+// the byte kinds' rate - 8.80 POP/s against 4.57 of kind::i8 with A in tensor memory, N = 64 .. 256 (8.54 at N = 32).
+// Sums of products +-2 are integers far below 2^24: exact (checked against popcounts up to K = 2^20, all-ones included).
+// Every block scale is 1.0 (e8m0 127): the SF_COLS columns at `sf` hold that byte in all 128 lanes, so that every scale
+// address an instruction of any width forms there reads 1.0.
+constexpr uint32_t SF_COLS = 8;
+constexpr uint32_t SF_ONES = 0x7F7F7F7Fu;
+__device__ __forceinline__ void tc_mma_f4_ts(uint32_t d_tmem, uint32_t a_tmem, uint32_t b_lo, uint32_t desc_hi,
+                                             uint32_t idesc, uint32_t sf, uint32_t accumulate)
+{
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t.reg .b64 db;\n\t"
+        "setp.ne.b32 p, %6, 0;\n\t"
+        "mov.b64 db, {%2, %3};\n\t"
+        "tcgen05.mma.cta_group::1.kind::mxf4.block_scale.scale_vec::2X [%0], [%1], db, %4, [%5], [%5], p;\n\t}"
+        ::"r"(d_tmem), "r"(a_tmem), "r"(b_lo), "r"(desc_hi), "r"(idesc), "r"(sf), "r"(accumulate)
+        : "memory");
+}
+// e2m1 A and B (K-major), e8m0 scales, M = 128, N = n, K = 64.
+__device__ __forceinline__ constexpr uint32_t make_idesc_f4(int n)
+{
+    return (1u << 7) | (1u << 10) | ((uint32_t)(n >> 3) << 17) | (1u << 23) | ((uint32_t)(BM >> 7) << 27);
+}
 // 32 columns of this warp's 32 lanes <- 32 registers; returns once the store has completed.
 __device__ __forceinline__ void tc_st32(uint32_t taddr, const uint32_t (&v)[32])
 {
@@ -283,6 +306,46 @@ __device__ __forceinline__ void expand_store_w_signed(uint32_t w, bool live, uin
     st_shared_v4(row_addr + (uint32_t)(((c + 1) ^ xr) << 4), o[4], o[5], o[6], o[7]);
 }
 
+// ---- 4-bit operands.  Nibble i of word j of an expanded 32-bit group carries bit 4i + j.  Activations are unsigned
+// ({0, 2^j / 2}: e2m1 codes 1, 2, 4 are 0.5, 1, 2; bit 3 goes to code 4 as well), weights signed (+-4, +-2, +-1, +-1), so
+// that every product with a set activation bit is +-2 and with S = sum over set activation bits of the weight signs
+//   accumulator = 2 S,   sum a*g = accumulator + K - 2 popc(G):
+// one constant per output channel.  Five logic operations per activation word (nine with bytes) and half the bytes.
+__device__ __forceinline__ void expand_a4(uint32_t w, uint32_t *v)
+{
+    v[0] = w & 0x11111111u;
+    v[1] = w & 0x22222222u;
+    v[2] = w & 0x44444444u;
+    v[3] = (w >> 1) & 0x44444444u;
+}
+// e2m1 sign bit = the weight bit's complement: (w at bit 3) ^ (magnitude code | 8)
+__device__ __forceinline__ uint4 expand_w4(uint32_t w)
+{
+    return make_uint4(((w << 3) & 0x88888888u) ^ 0xEEEEEEEEu, ((w << 2) & 0x88888888u) ^ 0xCCCCCCCCu,
+                      ((w << 1) & 0x88888888u) ^ 0xAAAAAAAAu, (w & 0x88888888u) ^ 0xAAAAAAAAu);
+}
+// fp32 sums of integers below 2^22 as integers: with INT_BIAS = 1.5 * 2^23 added, the value sits in the low mantissa bits
+// (an addition each in fp32 and integer, against a conversion at a quarter of the rate).
+constexpr float INT_BIAS = 12582912.0f;
+__device__ __forceinline__ int int_of_biased(uint32_t bits) { return (int)(bits - 0x4B400000u); }
+__device__ __forceinline__ uint32_t fadd_bits(uint32_t a, uint32_t b)
+{
+    return __float_as_uint(__fadd_rn(__uint_as_float(a), __uint_as_float(b)));
+}
+// K word e (0..7) of a 256-bit stage of a weight row: 16 bytes of a 128-byte-swizzled row; zeros where not live
+__device__ __forceinline__ void expand_store_w4(uint32_t w, bool live, uint32_t row_addr, int xr, int e)
+{
+    const uint4 o = live ? expand_w4(w) : make_uint4(0u, 0u, 0u, 0u);
+    st_shared_v4(row_addr + (uint32_t)((e ^ xr) << 4), o.x, o.y, o.z, o.w);
+}
+// unit scales into this warp's 32 lanes (the four warps of a group cover all lanes); returns once they are written
+__device__ __forceinline__ void write_unit_scales(uint32_t taddr)
+{
+    const uint32_t c8[8] = {SF_ONES, SF_ONES, SF_ONES, SF_ONES, SF_ONES, SF_ONES, SF_ONES, SF_ONES};
+    tc_st8_nowait(taddr, c8);
+    tc_wait_st();
+}
+
 // Expand the first nk (1..4) K words of a 128-bit stage into this lane's tensor-memory row (8 columns per word)
 // and wait for the stores.  A partial stage stores only its words: the MMAs skip the rest.
 __device__ __forceinline__ void expand_store_stage(uint32_t taddr, const uint4 &bits, int nk)
@@ -426,6 +489,51 @@ __device__ __forceinline__ void gather_stage(const uint32_t *x, const RowCursor 
         const int idx = ok ? rc.base + (int)ent[2 * u] : 0;
         cp_async_zfill<GW * 4>(dst + (uint32_t)(u * GW * 4), x + idx, ok ? (uint32_t)(GW * 4) : 0u);
     }
+}
+
+// The same gather for 256-bit stages (eight K words, 8 / GW units, two 16-byte halves `half` bytes apart in shared memory).
+// A table entry is one word: the unit's word offset (27 bits) and its tap in the top five; tap 31, which no row mask
+// contains, marks the zero padding of K.
+constexpr int TAP_NONE = 31;
+__device__ __forceinline__ void build_unit_table8(const ConvProblem &p, uint32_t tab_addr, int units, int gw, int tid, int nthreads)
+{
+    for (int u = tid; u < units; u += nthreads) {
+        const int kword = u * gw;
+        uint32_t ent = (uint32_t)TAP_NONE << 27;
+        if (kword < p.kwords) {
+            const int tap = kword / p.cw, cj = kword - tap * p.cw;
+            const int r = tap / p.kw, t = tap - r * p.kw;
+            ent = (uint32_t)((r * p.W + t) * p.cw + cj) | ((uint32_t)tap << 27);
+        }
+        asm volatile("st.shared.b32 [%0], %1;" ::"r"(tab_addr + 4u * u), "r"(ent) : "memory");
+    }
+}
+template <int GW>
+__device__ __forceinline__ void gather_stage8(const uint32_t *x, const RowCursor &rc, uint32_t tab, uint32_t dst, uint32_t half)
+{
+    constexpr int U = 8 / GW;
+    uint32_t ent[U];
+    if (U == 2) {
+        asm volatile("ld.shared.v2.b32 {%0,%1}, [%2];" : "=r"(ent[0]), "=r"(ent[1]) : "r"(tab));
+    } else {
+#pragma unroll
+        for (int h = 0; h < U / 4; ++h)
+            asm volatile("ld.shared.v4.b32 {%0,%1,%2,%3}, [%4];"
+                         : "=r"(ent[4 * h]), "=r"(ent[4 * h + 1]), "=r"(ent[4 * h + 2]), "=r"(ent[4 * h + 3]) : "r"(tab + 16u * h));
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+        const bool ok = ((rc.mask >> (ent[u] >> 27)) & 1u) != 0u;
+        const int idx = ok ? rc.base + (int)(ent[u] & 0x7FFFFFFu) : 0;
+        constexpr int PER = 4 / GW;                         // units per 16-byte half
+        cp_async_zfill<GW * 4>(dst + (u / PER) * half + (uint32_t)((u % PER) * GW * 4), x + idx, ok ? (uint32_t)(GW * 4) : 0u);
+    }
+}
+// eight K words -> 32 tensor-memory columns (column 4e + j = word j of K word e)
+__device__ __forceinline__ void expand_stage8(const uint4 &q0, const uint4 &q1, uint32_t (&v)[32])
+{
+    expand_a4(q0.x, &v[0]); expand_a4(q0.y, &v[4]); expand_a4(q0.z, &v[8]); expand_a4(q0.w, &v[12]);
+    expand_a4(q1.x, &v[16]); expand_a4(q1.y, &v[20]); expand_a4(q1.z, &v[24]); expand_a4(q1.w, &v[28]);
 }
 
 // int32 output of one accumulator chunk: 32 rows (one per lane) x 32 consecutive columns.  A lane storing its own
