@@ -1,8 +1,6 @@
-// Streaming tcgen05 engine of the binary implicit GEMM (kind::i8): wide layers (C_out >= 256),
-// long K, and the plain GEMMs.  Arithmetic as in the other tensor-core engines: sign bits are
-// expanded to bytes on chip (activations {0, 2^j}, weights {0, 2^(7-j)}; byte 4j+i of a 32-bit
-// group carries bit j+8i), every product of two set bits is 128, accumulators are int32 in
-// tensor memory and   sum a*g = K - 2*popc(A) - 2*popc(G) + 4*popc(A and G).
+// Streaming tcgen05 engine of the binary implicit GEMM: wide layers (C_out > 128), long K, and the plain GEMMs, on
+// weights that are expanded as they arrive.  Arithmetic: 4-bit operands (tc_common.cuh), fp32 accumulators that hold exact
+// integers,  sum a*g = accumulator + K - 2 popc(G):  one constant per output channel, nothing per row.
 //
 // Persistent, warp-specialised; each CTA walks a static list of 128 x BN tiles.
 //   warp 0          issuer: tcgen05.mma / commit only, waits on named barriers only (a memory
@@ -11,13 +9,13 @@
 //   G = 2 producer groups, each 4 activation warps + BN/32 weight warps, one thread per tile
 //                   row; the groups take the ring's stages alternately so that one group gathers
 //                   while the other expands.  Packed words are staged with cp.async (16 bytes per
-//                   row and stage, zero-fill out of range).
+//                   row half and stage, zero-fill out of range).
 //                     activation rows -> TENSOR memory (tcgen05.st, 32 columns per stage): the
 //                       MMA takes A from tensor memory, so shared memory carries only weights
 //                     weight rows     -> shared memory, 128-byte-swizzled K-major tiles
 //   last warp       control: does the issuer's mbarrier waits and releases it stage by stage
-// Tensor memory (512 columns): BN = 256: one accumulator + 5 ring stages; BN = 128: two
-// accumulators + 8 ring stages.  Row / column popcounts are taken from the words as they are
+// A ring stage is 256 bits of K.  Tensor memory (512 columns): BN = 256: one accumulator + 4 ring stages; BN = 128: two
+// accumulators + 7 ring stages, and the unit scales.  Column popcounts are taken from the words as they are
 // expanded; each group leaves its partial constants for a tile in shared-memory slots.
 // Every mbarrier wait is bounded and reports through the device error word.
 #include "tc_common.cuh"
@@ -40,7 +38,7 @@ constexpr int ERR_EPILOGUE_TIMEOUT = 103;
 template <int BN> struct Cfg {
     static constexpr int NBUF = BN == 256 ? 1 : 2;                       // accumulator buffers
     static constexpr int A_COL0 = NBUF * BN;                              // first column of the activation ring
-    static constexpr int STAGES = BN == 256 ? 5 : 8;
+    static constexpr int STAGES = BN == 256 ? 4 : 7;
     static constexpr int GROUP_WARPS = 4 + BN / 32;
     static constexpr int GROUP_THREADS = 32 * GROUP_WARPS;
     static constexpr int PROD_THREADS = G * GROUP_THREADS;
@@ -48,11 +46,13 @@ template <int BN> struct Cfg {
     static constexpr int CONTROL_WARP = FIRST_PRODUCER_WARP + G * GROUP_WARPS;
     static constexpr int THREADS = 32 * (CONTROL_WARP + 1);
     static constexpr int W_BYTES = BN * ROWB;                             // one ring stage of weights
-    static constexpr int BITS_BYTES = PF * PROD_THREADS * 16;
+    static constexpr int SF_COL = 512 - (int)SF_COLS;                     // unit scales
+    static constexpr int BITS_BYTES = PF * PROD_THREADS * 32;
     static constexpr int SLOTS = STAGES + NBUF + 2;                       // per-tile constant slots
-    static constexpr int SLOT_INTS = G * (BM + BN);
+    static constexpr int SLOT_INTS = G * BN;
     static constexpr int CONST_BYTES = SLOTS * SLOT_INTS * 4;
-    static_assert(A_COL0 + STAGES * 32 <= 512, "tensor memory budget");
+    static constexpr int TABLE_BYTES = EPI_WARPS * BN * 4;                // column constants as fp32, one table per epilogue warp
+    static_assert(A_COL0 + STAGES * 32 <= SF_COL, "tensor memory budget");
     static_assert(STAGES >= G, "a producer group must not lap the ring (parity waits)");
 };
 
@@ -62,7 +62,7 @@ __host__ __device__ inline int smem_bytes(int ktab_words, int mode = 1)
     using C = Cfg<BN>;
     // module epilogue: + the identity staging ring; int32 output of the 128-wide tiles: + the store staging tiles
     // (both only used where they fit: 128-wide tiles)
-    return 1024 + C::STAGES * C::W_BYTES + C::BITS_BYTES + C::CONST_BYTES + ktab_words * 4 +
+    return 1024 + C::STAGES * C::W_BYTES + C::BITS_BYTES + C::CONST_BYTES + C::TABLE_BYTES + ktab_words * 4 +
            (mode == 2 ? ID_RING_BYTES + 16 : 0) + (mode == 0 && BN == 128 ? EPI_WARPS * I32_TILE_BYTES + 16 : 0);
 }
 
@@ -83,7 +83,7 @@ conv_tc_i8_kernel(const ConvProblem p, const int ktab_words)
 
     const int tid = threadIdx.x;
     const int warp = tid >> 5, lane = tid & 31;
-    const int ktiles = (p.kwords + 3) >> 2;
+    const int ktiles = (p.kwords + 7) >> 3;
     const int m_tiles = (p.M - 1) / BM + 1;                  // M >= 1; no overflow for M close to 2^31
     const int n_tiles = (p.C_out + BN - 1) / BN;
     const int total_tiles = m_tiles * n_tiles;
@@ -91,9 +91,10 @@ conv_tc_i8_kernel(const ConvProblem p, const int ktab_words)
     const int total_items = my_tiles * ktiles;
 
     const uint32_t wring = (smem_u32(smem_raw) + 1023u) & ~1023u;         // [STAGES][BN rows][128 B]
-    const uint32_t bits_ring = wring + STAGES * C::W_BYTES;               // [PF][PROD_THREADS][16 B]
-    const uint32_t consts = bits_ring + C::BITS_BYTES;                    // [SLOTS][G][BM + BN] int32
-    const uint32_t ktab_addr = consts + C::CONST_BYTES;                   // unit table of the gather: {word offset, tap bit}
+    const uint32_t bits_ring = wring + STAGES * C::W_BYTES;               // [PF][2][PROD_THREADS][16 B]
+    const uint32_t consts = bits_ring + C::BITS_BYTES;                    // [SLOTS][G][BN] int32
+    const uint32_t tables = consts + C::CONST_BYTES;                      // [EPI_WARPS][BN] fp32
+    const uint32_t ktab_addr = tables + C::TABLE_BYTES;                   // unit table of the gather
     const uint32_t idring = (ktab_addr + (uint32_t)ktab_words * 4u + 15u) & ~15u;   // module epilogue only: [ID_SLOTS][BM rows][80 B]
     const uint32_t bar0 = smem_u32(bars);
     auto full_bar = [&](int s) { return bar0 + 8u * s; };
@@ -119,7 +120,7 @@ conv_tc_i8_kernel(const ConvProblem p, const int ktab_words)
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
     const int gwidth = gather_width(p.cw);
-    build_unit_table(p, ktab_addr, ktiles * (4 / gwidth), gwidth, tid, C::THREADS);
+    build_unit_table8(p, ktab_addr, ktiles * (8 / gwidth), gwidth, tid, C::THREADS);
     pdl_wait();
     tc_fence_before();
     __syncthreads();
@@ -129,12 +130,13 @@ conv_tc_i8_kernel(const ConvProblem p, const int ktab_words)
 
     if (warp == 0) {
         // ------------------------------------------------------------------ issuer (no memory instructions)
-        constexpr uint32_t idesc = make_idesc(BN);
+        constexpr uint32_t idesc = make_idesc_f4(BN);
         const uint64_t desc0 = make_desc(0);
         const uint32_t desc_hi = (uint32_t)(desc0 >> 32);
         const uint32_t b_lo0 = (uint32_t)desc0 | ((wring & 0x3FFFFu) >> 4);      // + slot * (W_BYTES / 16)
         const uint32_t tmem_u = __shfl_sync(0xffffffffu, tmem_base, 0);             // warp-uniform copy for the issuer
         const uint32_t a_tmem0 = tmem_u + (uint32_t)C::A_COL0;                   // + slot * 32 columns
+        const uint32_t sf = tmem_u + (uint32_t)C::SF_COL;
         int s = 0, buf = 0;
         for (int ti = 0; ti < my_tiles; ++ti) {
             const uint32_t d_tmem = tmem_u + (uint32_t)(buf * BN);
@@ -142,16 +144,16 @@ conv_tc_i8_kernel(const ConvProblem p, const int ktab_words)
             for (int kt = 0; kt < ktiles; ++kt) {
                 const uint32_t a_t = a_tmem0 + (uint32_t)s * 32u;
                 const uint32_t b_lo = b_lo0 + (uint32_t)s * (C::W_BYTES >> 4);
-                const int nk = p.kwords - 4 * kt;                 // 32 bits of K per instruction; skip the zero tail
+                const int nk = p.kwords - 8 * kt;                 // two K words per instruction; skip the zero tail
                 const uint32_t ebar = empty_bar(s);
                 asm volatile("bar.sync %0, 64;" ::"r"(1 + s) : "memory");
                 tc_fence_after();
-                // per 32 bytes of K: 8 tensor-memory columns of A, +2 (16-byte units) in the B descriptor
+                // per instruction: 8 tensor-memory columns of A, +2 (16-byte units) in the B descriptor
                 if (elect_one()) {
-                    tc_mma_i8_ts(d_tmem, a_t, b_lo, desc_hi, idesc, kt > 0 ? 1u : 0u);
-                    if (nk > 1) tc_mma_i8_ts(d_tmem, a_t + 8u, b_lo + 2u, desc_hi, idesc, 1u);
-                    if (nk > 2) tc_mma_i8_ts(d_tmem, a_t + 16u, b_lo + 4u, desc_hi, idesc, 1u);
-                    if (nk > 3) tc_mma_i8_ts(d_tmem, a_t + 24u, b_lo + 6u, desc_hi, idesc, 1u);
+                    tc_mma_f4_ts(d_tmem, a_t, b_lo, desc_hi, idesc, sf, kt > 0 ? 1u : 0u);
+                    if (nk > 2) tc_mma_f4_ts(d_tmem, a_t + 8u, b_lo + 2u, desc_hi, idesc, sf, 1u);
+                    if (nk > 4) tc_mma_f4_ts(d_tmem, a_t + 16u, b_lo + 4u, desc_hi, idesc, sf, 1u);
+                    if (nk > 6) tc_mma_f4_ts(d_tmem, a_t + 24u, b_lo + 6u, desc_hi, idesc, sf, 1u);
                     tc_commit(ebar);
                     if (kt == ktiles - 1) tc_commit(tfull);
                 }
@@ -221,17 +223,21 @@ conv_tc_i8_kernel(const ConvProblem p, const int ktab_words)
             const int first_group = (ti * ktiles) & 1;
             const bool two = ktiles >= 2;
             const uint32_t slot = consts + (uint32_t)((ti % SLOTS) * C::SLOT_INTS * 4);
-            const uint32_t part0 = slot + (uint32_t)(first_group * (BM + BN) * 4);
-            const uint32_t part1 = slot + (uint32_t)((first_group ^ 1) * (BM + BN) * 4);
+            const uint32_t part0 = slot + (uint32_t)(first_group * BN * 4);
+            const uint32_t part1 = slot + (uint32_t)((first_group ^ 1) * BN * 4);
             if (alive) alive = mbar_wait(tfull_bar(buf), buf_phase, abort_flag, p.err, ERR_EPILOGUE_TIMEOUT);
             alive = __all_sync(0xffffffffu, alive && !*abort_flag);
             if (!alive) break;
             tc_fence_after();
-            int rowc, rowc1 = 0;
-            asm volatile("ld.shared.b32 %0, [%1];" : "=r"(rowc) : "r"(part0 + 4u * erow) : "memory");
-            if (two) asm volatile("ld.shared.b32 %0, [%1];" : "=r"(rowc1) : "r"(part1 + 4u * erow) : "memory");
-            rowc += rowc1;
-            const uint32_t c0_addr = part0 + 4u * BM, c1_addr = part1 + 4u * BM;
+            // the groups' partial constants -> this warp's table of fp32 addends (int32 output: + INT_BIAS, see tc_common.cuh)
+            const uint32_t table = tables + (uint32_t)(quad * BN * 4);
+            for (int c = lane; c < BN; c += 32) {
+                int v0, v1 = 0;
+                asm volatile("ld.shared.b32 %0, [%1];" : "=r"(v0) : "r"(part0 + 4u * c) : "memory");
+                if (two) asm volatile("ld.shared.b32 %0, [%1];" : "=r"(v1) : "r"(part1 + 4u * c) : "memory");
+                asm volatile("st.shared.b32 [%0], %1;" ::"r"(table + 4u * c), "r"(__float_as_uint((float)(v0 + v1) + (MODE == 0 ? INT_BIAS : 0.0f))) : "memory");
+            }
+            __syncwarp();
             const uint32_t t_addr = tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)(buf * BN);
             uint32_t words[BN / 32];
 #pragma unroll
@@ -242,34 +248,26 @@ conv_tc_i8_kernel(const ConvProblem p, const int ktab_words)
                     uint32_t v[32];
                     tc_ld32(t_addr + (uint32_t)col0, v);
                     if (FUSED) {
-                        // bit = (v + rowc + colc >= 0); sign bits are shifted in, last column first
+                        // bit = (v + colc >= 0), an exact sum that is never -0; sign bits are shifted in, last column first
                         uint32_t acc = 0;
 #pragma unroll
                         for (int i4 = 7; i4 >= 0; --i4) {
-                            uint4 cc = ld_shared_v4(c0_addr + 4u * (col0 + 4 * i4));
-                            if (two) {
-                                const uint4 c2 = ld_shared_v4(c1_addr + 4u * (col0 + 4 * i4));
-                                cc.x += c2.x; cc.y += c2.y; cc.z += c2.z; cc.w += c2.w;
-                            }
-                            acc = __funnelshift_l((uint32_t)((int)v[4 * i4 + 3] + rowc + (int)cc.w), acc, 1);
-                            acc = __funnelshift_l((uint32_t)((int)v[4 * i4 + 2] + rowc + (int)cc.z), acc, 1);
-                            acc = __funnelshift_l((uint32_t)((int)v[4 * i4 + 1] + rowc + (int)cc.y), acc, 1);
-                            acc = __funnelshift_l((uint32_t)((int)v[4 * i4 + 0] + rowc + (int)cc.x), acc, 1);
+                            const uint4 cc = ld_shared_v4(table + 4u * (col0 + 4 * i4));
+                            acc = __funnelshift_l(fadd_bits(v[4 * i4 + 3], cc.w), acc, 1);
+                            acc = __funnelshift_l(fadd_bits(v[4 * i4 + 2], cc.z), acc, 1);
+                            acc = __funnelshift_l(fadd_bits(v[4 * i4 + 1], cc.y), acc, 1);
+                            acc = __funnelshift_l(fadd_bits(v[4 * i4 + 0], cc.x), acc, 1);
                         }
                         words[ch] = ~acc;
                     } else if (MODULE) {
-                        int dot[32];
+                        float dot[32];
 #pragma unroll
                         for (int i4 = 0; i4 < 8; ++i4) {
-                            uint4 cc = ld_shared_v4(c0_addr + 4u * (col0 + 4 * i4));
-                            if (two) {
-                                const uint4 c2 = ld_shared_v4(c1_addr + 4u * (col0 + 4 * i4));
-                                cc.x += c2.x; cc.y += c2.y; cc.z += c2.z; cc.w += c2.w;
-                            }
-                            dot[4 * i4 + 0] = (int)(v[4 * i4 + 0] >> 5) + rowc + (int)cc.x;
-                            dot[4 * i4 + 1] = (int)(v[4 * i4 + 1] >> 5) + rowc + (int)cc.y;
-                            dot[4 * i4 + 2] = (int)(v[4 * i4 + 2] >> 5) + rowc + (int)cc.z;
-                            dot[4 * i4 + 3] = (int)(v[4 * i4 + 3] >> 5) + rowc + (int)cc.w;
+                            const uint4 cc = ld_shared_v4(table + 4u * (col0 + 4 * i4));
+                            dot[4 * i4 + 0] = __uint_as_float(fadd_bits(v[4 * i4 + 0], cc.x));
+                            dot[4 * i4 + 1] = __uint_as_float(fadd_bits(v[4 * i4 + 1], cc.y));
+                            dot[4 * i4 + 2] = __uint_as_float(fadd_bits(v[4 * i4 + 2], cc.z));
+                            dot[4 * i4 + 3] = __uint_as_float(fadd_bits(v[4 * i4 + 3], cc.w));
                         }
                         prefetch_next();
                         cp_async_wait<ID_AHEAD>();                    // this chunk's copy has landed
@@ -280,15 +278,11 @@ conv_tc_i8_kernel(const ConvProblem p, const int ktab_words)
                         int o[32];
 #pragma unroll
                         for (int i4 = 0; i4 < 8; ++i4) {
-                            uint4 cc = ld_shared_v4(c0_addr + 4u * (col0 + 4 * i4));
-                            if (two) {
-                                const uint4 c2 = ld_shared_v4(c1_addr + 4u * (col0 + 4 * i4));
-                                cc.x += c2.x; cc.y += c2.y; cc.z += c2.z; cc.w += c2.w;
-                            }
-                            o[4 * i4 + 0] = (int)(v[4 * i4 + 0] >> 5) + rowc + (int)cc.x;
-                            o[4 * i4 + 1] = (int)(v[4 * i4 + 1] >> 5) + rowc + (int)cc.y;
-                            o[4 * i4 + 2] = (int)(v[4 * i4 + 2] >> 5) + rowc + (int)cc.z;
-                            o[4 * i4 + 3] = (int)(v[4 * i4 + 3] >> 5) + rowc + (int)cc.w;
+                            const uint4 cc = ld_shared_v4(table + 4u * (col0 + 4 * i4));
+                            o[4 * i4 + 0] = int_of_biased(fadd_bits(v[4 * i4 + 0], cc.x));
+                            o[4 * i4 + 1] = int_of_biased(fadd_bits(v[4 * i4 + 1], cc.y));
+                            o[4 * i4 + 2] = int_of_biased(fadd_bits(v[4 * i4 + 2], cc.z));
+                            o[4 * i4 + 3] = int_of_biased(fadd_bits(v[4 * i4 + 3], cc.w));
                         }
                         const long row0 = (long)em - lane;
                         store_int32_block(static_cast<int32_t *>(p.out) + row0 * p.C_out + n0 + col0, p.C_out, o, i32_tile, row0, p.M, lane);
@@ -297,16 +291,12 @@ conv_tc_i8_kernel(const ConvProblem p, const int ktab_words)
                         const bool vec = (p.C_out & 3) == 0 && (n0 + col0 + 32 <= p.C_out);
 #pragma unroll
                         for (int i4 = 0; i4 < 8; ++i4) {
-                            uint4 cc = ld_shared_v4(c0_addr + 4u * (col0 + 4 * i4));
-                            if (two) {
-                                const uint4 c2 = ld_shared_v4(c1_addr + 4u * (col0 + 4 * i4));
-                                cc.x += c2.x; cc.y += c2.y; cc.z += c2.z; cc.w += c2.w;
-                            }
+                            const uint4 cc = ld_shared_v4(table + 4u * (col0 + 4 * i4));
                             int4 o;
-                            o.x = (int)(v[4 * i4 + 0] >> 5) + rowc + (int)cc.x;
-                            o.y = (int)(v[4 * i4 + 1] >> 5) + rowc + (int)cc.y;
-                            o.z = (int)(v[4 * i4 + 2] >> 5) + rowc + (int)cc.z;
-                            o.w = (int)(v[4 * i4 + 3] >> 5) + rowc + (int)cc.w;
+                            o.x = int_of_biased(fadd_bits(v[4 * i4 + 0], cc.x));
+                            o.y = int_of_biased(fadd_bits(v[4 * i4 + 1], cc.y));
+                            o.z = int_of_biased(fadd_bits(v[4 * i4 + 2], cc.z));
+                            o.w = int_of_biased(fadd_bits(v[4 * i4 + 3], cc.w));
                             if (vec) {
                                 *reinterpret_cast<int4 *>(dst + 4 * i4) = o;
                             } else {
@@ -351,8 +341,7 @@ conv_tc_i8_kernel(const ConvProblem p, const int ktab_words)
         const int quad = warp & 3;
         const int row = is_a ? quad * 32 + lane : (wi - 4) * 32 + lane;   // row of the A or of the W tile
         const int ptid = tid - 32 * C::FIRST_PRODUCER_WARP;
-        const int crow = is_a ? row : BM + row;                  // index into a constants part
-        constexpr uint32_t SLOT_BYTES = C::PROD_THREADS * 16u;
+        constexpr uint32_t HALF_BYTES = C::PROD_THREADS * 16u, SLOT_BYTES = 2u * HALF_BYTES;
         const uint32_t bits0 = bits_ring + (uint32_t)ptid * 16u, bits_end = bits0 + PF * SLOT_BYTES;
         const uint32_t st_addr0 = tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)C::A_COL0;
         const uint32_t lane0 = lane == 0 ? 1u : 0u;
@@ -397,17 +386,22 @@ conv_tc_i8_kernel(const ConvProblem p, const int ktab_words)
         uint32_t l_dst = bits0;
         auto issue_load = [&]() {
             if (is_a) {
-                if (gwidth == 4) gather_stage<4>(p.x, rc, ktab_addr + (uint32_t)l_kt * 8u, l_dst);
-                else if (gwidth == 2) gather_stage<2>(p.x, rc, ktab_addr + (uint32_t)l_kt * 16u, l_dst);
-                else gather_stage<1>(p.x, rc, ktab_addr + (uint32_t)l_kt * 32u, l_dst);
+                if (gwidth == 4) gather_stage8<4>(p.x, rc, ktab_addr + (uint32_t)l_kt * 8u, l_dst, HALF_BYTES);
+                else if (gwidth == 2) gather_stage8<2>(p.x, rc, ktab_addr + (uint32_t)l_kt * 16u, l_dst, HALF_BYTES);
+                else gather_stage8<1>(p.x, rc, ktab_addr + (uint32_t)l_kt * 32u, l_dst, HALF_BYTES);
             } else if (w16) {
-                cp_async_zfill<16>(l_dst, wok ? wrow + l_kt * 4 : p.w, wok ? 16u : 0u);
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    const int kword = l_kt * 8 + 4 * h;
+                    const bool ok = wok && kword < p.kwords;
+                    cp_async_zfill<16>(l_dst + h * HALF_BYTES, ok ? wrow + kword : p.w, ok ? 16u : 0u);
+                }
             } else {
 #pragma unroll
-                for (int e = 0; e < 4; ++e) {
-                    const int kword = l_kt * 4 + e;
+                for (int e = 0; e < 8; ++e) {
+                    const int kword = l_kt * 8 + e;
                     const bool ok = wok && kword < p.kwords;
-                    cp_async_zfill<4>(l_dst + 4u * e, ok ? wrow + kword : p.w, ok ? 4u : 0u);
+                    cp_async_zfill<4>(l_dst + (e >> 2) * HALF_BYTES + 4u * (e & 3), ok ? wrow + kword : p.w, ok ? 4u : 0u);
                 }
             }
             l_dst += SLOT_BYTES;
@@ -426,6 +420,8 @@ conv_tc_i8_kernel(const ConvProblem p, const int ktab_words)
             cp_async_commit();
         }
 
+        // the scales are in place before this group's first arrival, which every MMA waits for
+        if (grp == 0 && is_a) write_unit_scales(tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)C::SF_COL);
         // ---- expand cursor
         uint32_t c_src = bits0;
         int c_ti = 0, c_kt = grp, pop = 0;
@@ -436,47 +432,46 @@ conv_tc_i8_kernel(const ConvProblem p, const int ktab_words)
             if (l_left > 0) issue_load();
             cp_async_commit();
             cp_async_wait<PF - 1>();
-            const uint4 bits = ld_shared_v4(c_src);
+            const uint4 q0 = ld_shared_v4(c_src), q1 = ld_shared_v4(c_src + HALF_BYTES);
             c_src += SLOT_BYTES;
             if (c_src == bits_end) c_src = bits0;
             while (c_kt >= ktiles) { c_kt -= ktiles; ++c_ti; }
-            if (!mbar_wait_warp(empty_bar(s), phase, abort_flag, p.err, ERR_PRODUCER_TIMEOUT)) break;
-            pop += __popc(bits.x) + __popc(bits.y) + __popc(bits.z) + __popc(bits.w);
-            if (c_kt + G >= ktiles) {
-                // this group's last stage of the tile: leave its partial constants for the epilogue.
-                //   fused: bit = acc - 64*pa - 32*(thr - K + 2*pg) >= 0      int32: (acc >> 5) - 2*pa + K - 2*pg
-                // the term that does not depend on the popcounts goes with the group of the tile's first stage
-                const bool first_group = ((c_ti * ktiles) & 1) == grp;
-                int cst = FUSED ? -64 * pop : -2 * pop;
-                if (!is_a && first_group) {
-                    const int tile = (int)blockIdx.x + c_ti * (int)gridDim.x;
-                    const int n = (tile / m_tiles) * BN + row;
-                    // (a threshold beyond +-(K + 1) decides like that bound; clamping keeps the constant inside int32)
-                    const int thr_n = max(min((FUSED && n < p.C_out) ? __ldg(p.thr + n) : 0, p.K + 1), -p.K - 1);
-                    cst += FUSED ? -32 * (thr_n - p.K) : p.K;
-                }
-                const uint32_t part = consts + (uint32_t)(((c_ti % SLOTS) * C::SLOT_INTS + grp * (BM + BN) + crow) * 4);
-                asm volatile("st.shared.b32 [%0], %1;" ::"r"(part), "r"(cst) : "memory");
-                pop = 0;
-            }
             if (is_a) {
+                uint32_t v[32];               // column 4e + j = word j of K word e
+                expand_stage8(q0, q1, v);
+                if (!mbar_wait_warp(empty_bar(s), phase, abort_flag, p.err, ERR_PRODUCER_TIMEOUT)) break;
                 tc_fence_after();     // the MMAs that read this slot are complete (their commit released it)
-                // expanded row -> 32 columns of this lane: column 8*e + j = word j of K word e (bytes 0 or 2^j)
-                uint32_t v[32];
-                const uint32_t wds[4] = {bits.x, bits.y, bits.z, bits.w};
-#pragma unroll
-                for (int e = 0; e < 4; ++e)
-#pragma unroll
-                    for (int j = 0; j < 8; ++j) v[8 * e + j] = wds[e] & (0x01010101u << j);
                 tc_st32(st_addr0 + (uint32_t)s * 32u, v);
                 tc_fence_before();
             } else {
+                if (!mbar_wait_warp(empty_bar(s), phase, abort_flag, p.err, ERR_PRODUCER_TIMEOUT)) break;
                 const uint32_t row_addr = wring + (uint32_t)s * C::W_BYTES + (uint32_t)row * ROWB;
                 const int xr = row & 7;
-                expand_store_w(bits.x, row_addr, xr, 0);
-                expand_store_w(bits.y, row_addr, xr, 2);
-                expand_store_w(bits.z, row_addr, xr, 4);
-                expand_store_w(bits.w, row_addr, xr, 6);
+                // rows and K words beyond the problem have no set bit here, and the codes of their -1 weights meet either
+                // activations of clear bits or accumulator columns that nobody reads
+                const uint32_t wds[8] = {q0.x, q0.y, q0.z, q0.w, q1.x, q1.y, q1.z, q1.w};
+#pragma unroll
+                for (int e = 0; e < 8; ++e) {
+                    expand_store_w4(wds[e], true, row_addr, xr, e);
+                    pop += __popc(wds[e]);
+                }
+                if (c_kt + G >= ktiles) {
+                    // this group's last stage of the tile: leave its partial constants for the epilogue.
+                    //   K - 2 pg, packed output: - thr; the term that does not depend on the popcounts goes with the group
+                    // of the tile's first stage
+                    const bool first_group = ((c_ti * ktiles) & 1) == grp;
+                    int cst = -2 * pop;
+                    if (first_group) {
+                        const int tile = (int)blockIdx.x + c_ti * (int)gridDim.x;
+                        const int n = (tile / m_tiles) * BN + row;
+                        cst += p.K;
+                        // (a threshold beyond +-(K + 1) decides like that bound)
+                        if (FUSED) cst -= max(min(n < p.C_out ? __ldg(p.thr + n) : 0, p.K + 1), -p.K - 1);
+                    }
+                    const uint32_t part = consts + (uint32_t)(((c_ti % SLOTS) * C::SLOT_INTS + grp * BN + row) * 4);
+                    asm volatile("st.shared.b32 [%0], %1;" ::"r"(part), "r"(cst) : "memory");
+                    pop = 0;
+                }
                 fence_async_proxy();  // generic-proxy stores -> visible to the MMA (async proxy)
             }
             __syncwarp();
@@ -495,10 +490,7 @@ conv_tc_i8_kernel(const ConvProblem p, const int ktab_words)
     }
 }
 
-int ktab_words_for(const ConvProblem &p)
-{
-    return ((p.kwords + 3) >> 2) * 8;        // at most four units of two words per 128-bit stage
-}
+int ktab_words_for(const ConvProblem &p) { return (((p.kwords + 7) >> 3) * (8 / gather_width(p.cw)) + 3) & ~3; }
 
 template <int BN>
 int launch_bn(const ConvProblem &p0, cudaStream_t stream)
@@ -527,8 +519,8 @@ bool conv_tc_i8_supports(const ConvProblem &p)
     if (p.kh * p.kw > 31) return false;                       // one validity bit per tap
     if ((long)p.B * p.H * p.W * p.cw >= (1L << 31)) return false;     // rows address the input by 32-bit word offsets
     if (smem_bytes<256>(ktab_words_for(p)) > MAX_SMEM) return false;   // the K-word table of the gather must fit
-    // the epilogue constants (about 3K << 5) must stay below 2^31
-    return p.K <= (1 << 20);
+    if ((long)p.kh * p.W * p.cw >= (1L << 27)) return false;  // a unit's word offset within the window
+    return p.K <= (1 << 20);                                  // sums up to 4 K + 2 stay exact in fp32
 }
 
 int launch_conv_tc_i8(const ConvProblem &p, cudaStream_t stream)

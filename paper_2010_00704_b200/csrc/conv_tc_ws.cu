@@ -2,17 +2,15 @@
 // 128 output channels fit in shared memory.  Wider layers run as slices of 128 (or 64) output channels: a CTA
 // keeps one slice's weights, so the activations are expanded once per slice.
 //
-// Arithmetic.  Sign bits are expanded to bytes on chip; byte 4j+i of a 32-bit group carries bit j+8i.
-//   activations (unsigned bytes): 0 where the bit is clear, else 2^j (j <= 6) or 64 (j = 7)
-//   weights     (signed bytes):   +-2^(6-j) (j <= 6) or +-1 (j = 7), sign = the weight's sign
-// Every product with a set activation bit is +-64, accumulators are int32 in tensor memory, and with
-// S = sum over set activation bits of the weight signs (acc = 64 S):
-//   sum a*g = 2 S + K - 2 popc(G)          (a, g in {-1,+1})
+// Arithmetic.  4-bit operands (tc_common.cuh): every product with a set activation bit is +-2, accumulators are fp32 in
+// tensor memory and hold exact integers, and with S = sum over set activation bits of the weight signs (acc = 2 S):
+//   sum a*g = acc + K - 2 popc(G)          (a, g in {-1,+1})
 // so the epilogue needs one constant per output channel and nothing per row - and not even an addition: the
-// accumulator buffers START from that constant (scaled by 32; the threshold folded in for the packed output).  The
-// epilogue team writes the constants into its buffers once, and again right after reading a tile out of one; every
-// MMA accumulates.  The packed output is then the complement of the accumulators' sign bits.
-// Differences to conv_tc_i8.cu, all aimed at short tiles (a 128 x 32 x 32 tile is one MMA instruction):
+// accumulator buffers START from that constant (the threshold folded in for the packed output, and half a unit added, so
+// that no sum is zero and its sign bit alone decides).  The epilogue team writes the constants into its buffers once, and
+// again right after reading a tile out of one; every MMA accumulates.  The packed output is the complement of the
+// accumulators' sign bits.
+// Differences to conv_tc_i8.cu, all aimed at short tiles (a 128 x 32 x 64 tile is one MMA instruction):
 //   * the CTA expands its weight tile ONCE into shared memory and keeps it for all its
 //     output tiles; only activations stream through the ring;
 //   * the activation ring lives in TENSOR memory, not shared memory: producers write expanded rows
@@ -52,24 +50,26 @@ template <int BN, int G, bool DUAL, int TEAMS = 1> struct Cfg {
     static constexpr int FIRST_PRODUCER_THREAD = 32 * (1 + EPI_WARPS * TEAMS);
     static constexpr int PROD_THREADS = G * BM;
     // Tensor memory (512 columns): NBUF accumulator buffers of BN columns, then the activation ring,
-    // one stage = 128 rows x 128 expanded bytes = 32 columns.
+    // one stage = 128 rows x 256 bits of K expanded to 128 bytes = 32 columns.
     static constexpr int TMEM_COLS = DUAL ? 256 : 512;
     static constexpr int NBUF = DUAL ? (BN == 128 ? 1 : 2) : (BN == 32 ? 4 : (BN == 64 ? 3 : 2));
     static constexpr int CONTROL_WARP = (FIRST_PRODUCER_THREAD + PROD_THREADS) / 32;
     static constexpr int THREADS = FIRST_PRODUCER_THREAD + PROD_THREADS + 32;
     static constexpr int A_COL0 = NBUF * BN;
-    static constexpr int STAGES = (TMEM_COLS - A_COL0) / 32 > 8 ? 8 : (TMEM_COLS - A_COL0) / 32;
+    static constexpr int SF_COL = TMEM_COLS - (int)SF_COLS;      // unit scales
+    static constexpr int STAGES = (SF_COL - A_COL0) / 32 > 8 ? 8 : (SF_COL - A_COL0) / 32;
     static constexpr int CTAS_PER_SM = DUAL ? 2 : 1;
     // registers are granted in blocks of 8 per thread: bound the pair of CTAs to 64 registers per thread
     static constexpr int BOUND_THREADS = DUAL ? 512 : THREADS;
-    static_assert(A_COL0 + STAGES * 32 <= TMEM_COLS, "tensor memory budget");
+    static_assert(A_COL0 + STAGES * 32 <= SF_COL, "tensor memory budget");
     static_assert(STAGES >= G, "a producer group must not lap the ring (parity waits)");
     static constexpr int W_TILE_BYTES = BN * ROWB;           // one K stage of the expanded weights
-    static constexpr int BITS_BYTES = PF * PROD_THREADS * 16;
+    static constexpr int HALF_BYTES = PROD_THREADS * 16;     // four K words of every producer thread
 };
 
 struct WsLayout {
-    int ktiles;       // 128-bit K stages
+    int ktiles;       // 256-bit K stages
+    int halves;       // 16-byte halves staged per producer thread and ring slot
     int row_kt;       // > 0: producers work tile by tile (all row_kt stages of a row at once), see the producers
     int bits_bytes;   // staging ring of the packed words
     int smem;         // dynamic shared memory in bytes
@@ -80,13 +80,14 @@ __host__ __device__ inline WsLayout ws_layout(int kwords, int mode)
 {
     using C = Cfg<BN, G, DUAL, TEAMS>;
     WsLayout l;
-    l.ktiles = (kwords + 3) >> 2;
+    l.ktiles = (kwords + 7) >> 3;
     // Short K: a producer group takes whole tiles in turn instead of single stages, so the per-tile work
     // (row coordinates, tap mask, bookkeeping) is done once per row and tile.  A group then runs up to
     // (G - 1) * ktiles + 1 ring slots ahead of the slot it waits for; the parity waits need the ring
     // to be at least that deep.
-    l.row_kt = (l.ktiles <= 3 && C::STAGES >= (G - 1) * l.ktiles + 1) ? l.ktiles : 0;
-    l.bits_bytes = C::BITS_BYTES * (l.row_kt ? l.row_kt : 1);
+    l.row_kt = (l.ktiles <= 2 && C::STAGES >= (G - 1) * l.ktiles + 1) ? l.ktiles : 0;
+    l.halves = l.row_kt ? (kwords + 3) >> 2 : 2;
+    l.bits_bytes = PF * C::HALF_BYTES * l.halves;
     l.smem = 1024 + l.ktiles * C::W_TILE_BYTES + l.bits_bytes + BN * 4 + l.ktiles * 32;
     if (mode == 2) l.smem += TEAMS * ID_RING_BYTES + 16;      // identity staging rings of the module epilogue
     if (mode == 0) l.smem += TEAMS * EPI_WARPS * I32_TILE_BYTES + 16;   // store staging tiles of the int32 epilogue
@@ -131,9 +132,9 @@ conv_tc_ws_kernel(const ConvProblem p)
 
     // shared-memory map (all 1024-byte aligned where the MMA reads)
     const uint32_t wexp = (smem_u32(smem_raw) + 1023u) & ~1023u;          // [ktiles][BN rows][128 B]
-    const uint32_t bits_ring = wexp + (uint32_t)ktiles * C::W_TILE_BYTES; // [PF][PROD_THREADS][16 B]
+    const uint32_t bits_ring = wexp + (uint32_t)ktiles * C::W_TILE_BYTES; // [PF][halves][PROD_THREADS][16 B]
     const uint32_t colc_addr = bits_ring + (uint32_t)L.bits_bytes;                 // [BN] int32
-    const uint32_t ktab_addr = colc_addr + BN * 4;                        // unit table: [ktiles * 4 / gw] x {word offset, tap bit}
+    const uint32_t ktab_addr = colc_addr + BN * 4;                        // unit table of the gather: [ktiles * 8 / gw]
     const uint32_t idring = (ktab_addr + (uint32_t)ktiles * 32u + 15u) & ~15u;   // module epilogue only: [ID_SLOTS][BM rows][80 B]
     const uint32_t bar0 = smem_u32(bars);
     auto full_bar = [&](int s) { return bar0 + 8u * s; };
@@ -160,36 +161,34 @@ conv_tc_ws_kernel(const ConvProblem p)
     }
 
     const int gw = gather_width(p.cw);
-    build_unit_table(p, ktab_addr, ktiles * (4 / gw), gw, tid, C::THREADS);
+    build_unit_table8(p, ktab_addr, ktiles * (8 / gw), gw, tid, C::THREADS);
+    for (int c = tid; c < BN; c += C::THREADS) asm volatile("st.shared.b32 [%0], %1;" ::"r"(colc_addr + 4u * c), "r"(0) : "memory");
     pdl_wait();
-    // ---- one-off: expand the weight tile, per-channel constants
-    for (int idx = tid; idx < ktiles * BN; idx += C::THREADS) {
-        const int kt = idx / BN, row = idx - kt * BN;
-        const uint32_t row_addr = wexp + (uint32_t)kt * C::W_TILE_BYTES + (uint32_t)row * ROWB;
+    __syncthreads();
+    // ---- one-off: expand the weight tile, count every row's set bits.  Eight lanes take the eight K words of one stage of
+    // one row: coalesced loads, 128-byte rows stored without bank conflicts.
+    // WU words of a thread are requested together (the expansion is otherwise one L2 latency per word).
+    constexpr int WU = 8;
+    const int wtotal = ktiles * BN * 8;                      // a multiple of 32: a warp's lanes stay together
+    for (int i0 = tid; i0 < wtotal; i0 += WU * C::THREADS) {
+        uint32_t w[WU];
 #pragma unroll
-        for (int e = 0; e < 4; ++e) {
-            const int kword = kt * 4 + e;
-            const bool live = kword < p.kwords && row < cn;              // rows / K words beyond the problem: zero bytes
-            const uint32_t w = live ? __ldg(p.w + (long)(n0 + row) * p.kwords + kword) : 0u;
-            expand_store_w_signed(w, live, row_addr, row & 7, 2 * e);
+        for (int u = 0; u < WU; ++u) {
+            const int idx = i0 + u * C::THREADS, row = (idx >> 3) / ktiles, kword = ((idx >> 3) - row * ktiles) * 8 + (idx & 7);
+            w[u] = idx < wtotal && kword < p.kwords && row < cn ? __ldg(p.w + (long)(n0 + row) * p.kwords + kword) : 0u;
         }
-    }
-    for (int c = tid; c < BN; c += C::THREADS) {
-        int pop = 0;
-        if (c < cn)
-            for (int kw = 0; kw < p.kwords; ++kw) pop += __popc(__ldg(p.w + (long)(n0 + c) * p.kwords + kw));
-        // The accumulators start from a per-channel constant instead of zero (the epilogue writes it back after
-        // reading a buffer, every MMA accumulates), so with acc = 64 * S + cst:
-        //   int32: acc >> 5 with cst = 32 * (K - 2*pop)        fused: acc >= 0 with cst = 32 * (K - 2*pop - thr)
-        // (a threshold beyond +-(K + 1) decides like that bound; clamping keeps the constant inside int32)
-        int cst = p.K - 2 * pop;
-        if (FUSED) {
-            int t = c < cn ? __ldg(p.thr + n0 + c) : 0;
-            t = max(min(t, p.K + 1), -p.K - 1);
-            cst -= t;
+#pragma unroll
+        for (int u = 0; u < WU; ++u) {
+            const int idx = i0 + u * C::THREADS, row = (idx >> 3) / ktiles, kt = (idx >> 3) - row * ktiles, e = idx & 7;
+            if (idx >= wtotal) break;
+            const bool live = kt * 8 + e < p.kwords && row < cn;           // rows / K words beyond the problem: zeros
+            expand_store_w4(w[u], live, wexp + (uint32_t)kt * C::W_TILE_BYTES + (uint32_t)row * ROWB, row & 7, e);
+            int pop = __popc(w[u]);
+            pop += __shfl_xor_sync(0xffffffffu, pop, 1);
+            pop += __shfl_xor_sync(0xffffffffu, pop, 2);
+            pop += __shfl_xor_sync(0xffffffffu, pop, 4);
+            if (e == 0) asm volatile("red.shared.add.u32 [%0], %1;" ::"r"(colc_addr + 4u * row), "r"(pop) : "memory");
         }
-        cst *= 32;
-        asm volatile("st.shared.b32 [%0], %1;" ::"r"(colc_addr + 4u * c), "r"(cst) : "memory");
     }
     fence_async_proxy();
     tc_fence_before();
@@ -206,11 +205,12 @@ conv_tc_ws_kernel(const ConvProblem p)
         // stage at a time through named barrier 1 + slot.  There is one issuer on purpose: the
         // producers' parity waits rely on the ring being consumed in order (a second issuer working on
         // the next tile lets a late slot fall two phases behind a waiting producer).
-        constexpr uint32_t idesc = make_idesc(BN) | (1u << 10);                  // B operand: signed bytes
+        constexpr uint32_t idesc = make_idesc_f4(BN);
         const uint64_t desc0 = make_desc(0);
         const uint32_t desc_hi = (uint32_t)(desc0 >> 32);
         const uint32_t tmem_u = __shfl_sync(0xffffffffu, tmem_base, 0);             // warp-uniform copy for the issuer
         const uint32_t a_tmem0 = tmem_u + (uint32_t)C::A_COL0;                   // + slot * 32 columns
+        const uint32_t sf = tmem_u + (uint32_t)C::SF_COL;
         const uint32_t b_lo0 = (uint32_t)desc0 | ((wexp & 0x3FFFFu) >> 4);       // + kt * (W_TILE_BYTES / 16)
         int s = 0, buf = 0;
         for (int ti = 0; ti < my_tiles; ++ti) {
@@ -219,16 +219,16 @@ conv_tc_ws_kernel(const ConvProblem p)
             for (int kt = 0; kt < ktiles; ++kt) {
                 const uint32_t a_t = a_tmem0 + (uint32_t)s * 32u;
                 const uint32_t b_lo = b_lo0 + (uint32_t)kt * (C::W_TILE_BYTES >> 4);
-                const int nk = p.kwords - 4 * kt;                 // 32 bits of K per instruction; skip the zero tail
+                const int nk = p.kwords - 8 * kt;                 // two K words per instruction; skip the zero tail
                 const uint32_t ebar = empty_bar(s);
                 asm volatile("bar.sync %0, 64;" ::"r"(1 + s) : "memory");
                 tc_fence_after();
-                // per 32 bytes of K: 8 tensor-memory columns of A, +2 (16-byte units) in the B descriptor
+                // per instruction: 8 tensor-memory columns of A, +2 (16-byte units) in the B descriptor
                 if (elect_one()) {
-                    tc_mma_i8_ts(d_tmem, a_t, b_lo, desc_hi, idesc, 1u);      // always accumulates: the buffer holds the constants
-                    if (nk > 1) tc_mma_i8_ts(d_tmem, a_t + 8u, b_lo + 2u, desc_hi, idesc, 1u);
-                    if (nk > 2) tc_mma_i8_ts(d_tmem, a_t + 16u, b_lo + 4u, desc_hi, idesc, 1u);
-                    if (nk > 3) tc_mma_i8_ts(d_tmem, a_t + 24u, b_lo + 6u, desc_hi, idesc, 1u);
+                    tc_mma_f4_ts(d_tmem, a_t, b_lo, desc_hi, idesc, sf, 1u);      // always accumulates: the buffer holds the constants
+                    if (nk > 2) tc_mma_f4_ts(d_tmem, a_t + 8u, b_lo + 2u, desc_hi, idesc, sf, 1u);
+                    if (nk > 4) tc_mma_f4_ts(d_tmem, a_t + 16u, b_lo + 4u, desc_hi, idesc, sf, 1u);
+                    if (nk > 6) tc_mma_f4_ts(d_tmem, a_t + 24u, b_lo + 6u, desc_hi, idesc, sf, 1u);
                     tc_commit(ebar);
                     if (kt == ktiles - 1) tc_commit(tfull);
                 }
@@ -283,6 +283,19 @@ conv_tc_ws_kernel(const ConvProblem p)
         };
         if (MODULE)
             for (int a = 0; a < ID_AHEAD; ++a) prefetch_next();
+        // the rows' bit counts -> the accumulators' start values:  int32, module: K - 2 popc    packed: K - 2 popc - thr + 1/2
+        // (a threshold beyond +-(K + 1) decides like that bound)
+        for (int c = tid - 32; c < BN; c += 32 * EPI_WARPS * TEAMS) {
+            int pop;
+            asm volatile("ld.shared.b32 %0, [%1];" : "=r"(pop) : "r"(colc_addr + 4u * c) : "memory");
+            float cst = (float)(p.K - 2 * pop);
+            if (FUSED) {
+                const int t = c < cn ? __ldg(p.thr + n0 + c) : 0;
+                cst = (float)(p.K - 2 * pop - max(min(t, p.K + 1), -p.K - 1)) + 0.5f;
+            }
+            asm volatile("st.shared.b32 [%0], %1;" ::"r"(colc_addr + 4u * c), "r"(__float_as_uint(cst)) : "memory");
+        }
+        asm volatile("bar.sync 9, %0;" ::"n"(32 * EPI_WARPS * TEAMS) : "memory");
         // write the per-channel constants into 32 accumulator columns of this warp's rows (8 columns at a time:
         // the values are the same for every row)
         auto write_consts = [&](uint32_t t_chunk, int col0) {
@@ -330,9 +343,9 @@ conv_tc_ws_kernel(const ConvProblem p)
                         for (int i = 31; i >= 0; --i) acc = __funnelshift_l(v[i], acc, 1);
                         words[ch] = ~acc;
                     } else if (MODULE) {
-                        int dot[32];
+                        float dot[32];
 #pragma unroll
-                        for (int i = 0; i < 32; ++i) dot[i] = (int)v[i] >> 5;
+                        for (int i = 0; i < 32; ++i) dot[i] = __uint_as_float(v[i]);
                         prefetch_next();
                         cp_async_wait<ID_AHEAD>();                    // this chunk's copy has landed
                         words[ch] = module_chunk(p, dot, id_warp + (uint32_t)cur_slot * (BM * ID_ROW_BYTES), (long)em - lane, n0 + col0, lane);
@@ -341,7 +354,7 @@ conv_tc_ws_kernel(const ConvProblem p)
                         // full chunk (warp-uniform): staged, the warp stores whole 128-byte rows
                         int o[32];
 #pragma unroll
-                        for (int i = 0; i < 32; ++i) o[i] = (int)v[i] >> 5;
+                        for (int i = 0; i < 32; ++i) o[i] = int_of_biased(fadd_bits(v[i], __float_as_uint(INT_BIAS)));
                         const long row0 = (long)em - lane;
                         store_int32_block(static_cast<int32_t *>(p.out) + row0 * p.C_out + n0 + col0, p.C_out, o, i32_tile, row0, p.M, lane);
                     } else if (em < p.M) {
@@ -350,10 +363,10 @@ conv_tc_ws_kernel(const ConvProblem p)
 #pragma unroll
                         for (int i4 = 0; i4 < 8; ++i4) {
                             int4 o;
-                            o.x = (int)v[4 * i4 + 0] >> 5;
-                            o.y = (int)v[4 * i4 + 1] >> 5;
-                            o.z = (int)v[4 * i4 + 2] >> 5;
-                            o.w = (int)v[4 * i4 + 3] >> 5;
+                            o.x = int_of_biased(fadd_bits(v[4 * i4 + 0], __float_as_uint(INT_BIAS)));
+                            o.y = int_of_biased(fadd_bits(v[4 * i4 + 1], __float_as_uint(INT_BIAS)));
+                            o.z = int_of_biased(fadd_bits(v[4 * i4 + 2], __float_as_uint(INT_BIAS)));
+                            o.w = int_of_biased(fadd_bits(v[4 * i4 + 3], __float_as_uint(INT_BIAS)));
                             if (vec) {
                                 *reinterpret_cast<int4 *>(dst + 4 * i4) = o;
                             } else {
@@ -389,21 +402,24 @@ conv_tc_ws_kernel(const ConvProblem p)
     } else {
         // ------------------------------------------------------------------ producers
         // Group g takes items g, g + G, ... of the CTA's flattened (tile, stage) list.  Per item a
-        // thread copies its row's 128 bits of K into its staging slot (PF items ahead), then expands
+        // thread copies its row's 256 bits of K into its staging slot (PF items ahead), then expands
         // the oldest staged item into the ring slot of tensor memory.
         const int ptid = tid - C::FIRST_PRODUCER_THREAD;
         const int grp = ptid >> 7;                               // group = 4 consecutive warps
         const int quad = warp & 3;                               // tensor-memory lane quadrant this warp may write
         const int row = quad * 32 + lane;                        // the four warps of a group cover rows 0..127
-        constexpr uint32_t SLOT_BYTES = C::PROD_THREADS * 16u;
+        constexpr uint32_t HALF_BYTES = C::HALF_BYTES;
+        const uint32_t SLOT_BYTES = (uint32_t)L.halves * HALF_BYTES;
         const uint32_t bits0 = bits_ring + (uint32_t)ptid * 16u, bits_end = bits0 + PF * SLOT_BYTES;
         const uint32_t st_addr0 = tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)C::A_COL0;
         const uint32_t lane0 = lane == 0 ? 1u : 0u;
         const TileStep step = make_tile_step(p, (uint32_t)(BM * mstride));
+        // the scales are in place before this group's first arrival, which every MMA waits for
+        if (grp == 0) write_unit_scales(tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)C::SF_COL);
 
         auto produce = [&](auto gw_tag) {
             constexpr int GW = decltype(gw_tag)::value;
-            constexpr uint32_t TAB_STAGE = (4 / GW) * 8u;        // table bytes per stage
+            constexpr uint32_t TAB_STAGE = (8 / GW) * 4u;        // table bytes per stage
             // ---- load cursor
             RowCursor rc;
             rc.m = (uint32_t)mb * BM + (uint32_t)row;
@@ -414,7 +430,7 @@ conv_tc_ws_kernel(const ConvProblem p)
             row_window(p, step, rc);
             uint32_t l_dst = bits0;
             auto issue = [&]() {
-                gather_stage<GW>(p.x, rc, ktab_addr + (uint32_t)l_kt * TAB_STAGE, l_dst);
+                gather_stage8<GW>(p.x, rc, ktab_addr + (uint32_t)l_kt * TAB_STAGE, l_dst, HALF_BYTES);
                 l_dst += SLOT_BYTES;
                 if (l_dst == bits_end) l_dst = bits0;
                 --l_left;
@@ -438,16 +454,12 @@ conv_tc_ws_kernel(const ConvProblem p)
                 if (l_left > 0) issue();
                 cp_async_commit();
                 cp_async_wait<PF - 1>();
-                const uint4 bits = ld_shared_v4(c_src);
+                uint32_t v[32];               // column 4e + j = word j of K word e
+                expand_stage8(ld_shared_v4(c_src), ld_shared_v4(c_src + HALF_BYTES), v);
                 c_src += SLOT_BYTES;
                 if (c_src == bits_end) c_src = bits0;
                 if (!mbar_wait_warp(empty_bar(s), phase, abort_flag, p.err, ERR_PRODUCER_TIMEOUT)) break;
                 tc_fence_after();     // the MMAs that read this slot are complete (their commit released it)
-                // expanded row -> 32 columns of this lane: column 8*e + j = word j of K word e (bytes 0 or 2^j, 64 for j = 7)
-                uint32_t v[32];
-                const uint32_t wds[4] = {bits.x, bits.y, bits.z, bits.w};
-#pragma unroll
-                for (int e = 0; e < 4; ++e) expand_a(wds[e], &v[8 * e]);
                 tc_st32(st_addr0 + (uint32_t)s * 32u, v);
                 tc_fence_before();
                 __syncwarp();
@@ -462,10 +474,10 @@ conv_tc_ws_kernel(const ConvProblem p)
         auto produce_rows = [&](auto gw_tag, auto kt_tag) {
             constexpr int GW = decltype(gw_tag)::value;
             constexpr int KT = decltype(kt_tag)::value;
-            constexpr uint32_t TAB_STAGE = (4 / GW) * 8u;
-            constexpr uint32_t TSLOT_BYTES = SLOT_BYTES * KT;     // one staged tile: [KT][PROD_THREADS][16 B]
+            constexpr uint32_t TAB_STAGE = (8 / GW) * 4u;
+            const uint32_t TSLOT_BYTES = SLOT_BYTES;              // one staged tile: [halves][PROD_THREADS][16 B]
             const uint32_t tend = bits0 + PF * TSLOT_BYTES;
-            const int nk_last = p.kwords - 4 * (KT - 1);          // K words of the row's last stage (1..4)
+            const int nk_last = p.kwords - 8 * (KT - 1);          // K words of the row's last stage (1..8)
             const TileStep gstep = make_tile_step(p, (uint32_t)(BM * mstride * G));
             RowCursor rc;
             rc.m = (uint32_t)(mb + grp * mstride) * BM + (uint32_t)row;
@@ -476,8 +488,8 @@ conv_tc_ws_kernel(const ConvProblem p)
             auto issue = [&]() {
 #pragma unroll
                 for (int kt = 0; kt < KT; ++kt)
-                    gather_stage<GW>(p.x, rc, ktab_addr + (uint32_t)kt * TAB_STAGE, l_dst + (uint32_t)kt * SLOT_BYTES,
-                                     kt < KT - 1 ? 4 : (nk_last + GW - 1) / GW);
+                    gather_stage8<GW>(p.x, rc, ktab_addr + (uint32_t)kt * TAB_STAGE, l_dst + (uint32_t)(2 * kt) * HALF_BYTES, HALF_BYTES,
+                                      kt < KT - 1 ? 8 : ((nk_last + 3) & ~3) / GW);        // whole halves: what K lacks is zero-filled
                 l_dst += TSLOT_BYTES;
                 if (l_dst == tend) l_dst = bits0;
                 --l_left;
@@ -501,11 +513,11 @@ conv_tc_ws_kernel(const ConvProblem p)
                 bool alive = true;
 #pragma unroll
                 for (int kt = 0; kt < KT; ++kt) {
-                    const uint4 bits = ld_shared_v4(c_src + (uint32_t)kt * SLOT_BYTES);
                     if (alive && !mbar_wait_warp(empty_bar(s), phase, abort_flag, p.err, ERR_PRODUCER_TIMEOUT)) alive = false;
                     if (alive) {
                         tc_fence_after();
-                        expand_store_stage(st_addr0 + (uint32_t)s * 32u, bits, kt < KT - 1 ? 4 : nk_last);
+                        expand_store_stage8(st_addr0 + (uint32_t)s * 32u, c_src + (uint32_t)(2 * kt) * HALF_BYTES, HALF_BYTES, kt < KT - 1 ? 8 : nk_last);
+                        tc_wait_st();
                         tc_fence_before();
                         __syncwarp();
                         mbar_arrive_pred(full_bar(s), lane0);
@@ -522,8 +534,7 @@ conv_tc_ws_kernel(const ConvProblem p)
         };
         auto rows_by_kt = [&](auto gw_tag) {
             if (L.row_kt == 1) produce_rows(gw_tag, IntC<1>{});
-            else if (L.row_kt == 2) produce_rows(gw_tag, IntC<2>{});
-            else produce_rows(gw_tag, IntC<3>{});
+            else produce_rows(gw_tag, IntC<2>{});
         };
         if (L.row_kt) {
             if (gw == 4) rows_by_kt(IntC<4>{});
@@ -577,7 +588,7 @@ bool conv_tc_ws_supports(const ConvProblem &p)
     if (p.mode != 0 && (p.C_out % 32 != 0)) return false;
     if (p.kh * p.kw > 31 || p.K > (1 << 16)) return false;
     // rows address the input by 32-bit word offsets
-    if ((long)p.B * p.H * p.W * p.cw >= (1L << 31)) return false;
+    if ((long)p.B * p.H * p.W * p.cw >= (1L << 31) || (long)p.kh * p.W * p.cw >= (1L << 27)) return false;
     if (p.C_out <= 32) return fits<32, 4, false>(p);
     if (p.C_out <= 64) return fits<64, 4, false>(p);
     if (fits<128, 4, false>(p) || fits<128, 2, false>(p)) return p.C_out <= 128 * 64;

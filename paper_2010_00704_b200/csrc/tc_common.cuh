@@ -187,7 +187,18 @@ __device__ __forceinline__ void tc_st32_nowait(uint32_t taddr, const uint32_t (&
           "r"(v[24]), "r"(v[25]), "r"(v[26]), "r"(v[27]), "r"(v[28]), "r"(v[29]), "r"(v[30]), "r"(v[31])
         : "memory");
 }
-// 8 columns (one K word) of this warp's 32 lanes <- 8 registers.
+// 16 columns of this warp's 32 lanes <- 16 registers.
+__device__ __forceinline__ void tc_st16_nowait(uint32_t taddr, const uint32_t (&v)[16])
+{
+    asm volatile(
+        "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], "
+        "{%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16};"
+        ::"r"(taddr),
+          "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7]),
+          "r"(v[8]), "r"(v[9]), "r"(v[10]), "r"(v[11]), "r"(v[12]), "r"(v[13]), "r"(v[14]), "r"(v[15])
+        : "memory");
+}
+// 8 columns of this warp's 32 lanes <- 8 registers.
 __device__ __forceinline__ void tc_st8_nowait(uint32_t taddr, const uint32_t (&v)[8])
 {
     asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};"
@@ -508,8 +519,9 @@ __device__ __forceinline__ void build_unit_table8(const ConvProblem &p, uint32_t
         asm volatile("st.shared.b32 [%0], %1;" ::"r"(tab_addr + 4u * u), "r"(ent) : "memory");
     }
 }
+// Only the first `nunits` units are copied (warp-uniform; what lies beyond K's last word needs no copy when nobody reads it).
 template <int GW>
-__device__ __forceinline__ void gather_stage8(const uint32_t *x, const RowCursor &rc, uint32_t tab, uint32_t dst, uint32_t half)
+__device__ __forceinline__ void gather_stage8(const uint32_t *x, const RowCursor &rc, uint32_t tab, uint32_t dst, uint32_t half, int nunits = 8)
 {
     constexpr int U = 8 / GW;
     uint32_t ent[U];
@@ -523,6 +535,7 @@ __device__ __forceinline__ void gather_stage8(const uint32_t *x, const RowCursor
     }
 #pragma unroll
     for (int u = 0; u < U; ++u) {
+        if (u >= nunits) break;
         const bool ok = ((rc.mask >> (ent[u] >> 27)) & 1u) != 0u;
         const int idx = ok ? rc.base + (int)(ent[u] & 0x7FFFFFFu) : 0;
         constexpr int PER = 4 / GW;                         // units per 16-byte half
@@ -534,6 +547,20 @@ __device__ __forceinline__ void expand_stage8(const uint4 &q0, const uint4 &q1, 
 {
     expand_a4(q0.x, &v[0]); expand_a4(q0.y, &v[4]); expand_a4(q0.z, &v[8]); expand_a4(q0.w, &v[12]);
     expand_a4(q1.x, &v[16]); expand_a4(q1.y, &v[20]); expand_a4(q1.z, &v[24]); expand_a4(q1.w, &v[28]);
+}
+// the first nk (1..8) words of a stage; a stage of at most four words has one 16-byte half and 16 columns
+__device__ __forceinline__ void expand_store_stage8(uint32_t taddr, uint32_t src, uint32_t half, int nk)
+{
+    const uint4 q0 = ld_shared_v4(src);
+    if (nk > 4) {                                           // warp-uniform
+        uint32_t v[32];
+        expand_stage8(q0, ld_shared_v4(src + half), v);
+        tc_st32_nowait(taddr, v);
+    } else {
+        uint32_t v[16];
+        expand_a4(q0.x, &v[0]); expand_a4(q0.y, &v[4]); expand_a4(q0.z, &v[8]); expand_a4(q0.w, &v[12]);
+        tc_st16_nowait(taddr, v);
+    }
 }
 
 // int32 output of one accumulator chunk: 32 rows (one per lane) x 32 consecutive columns.  A lane storing its own
@@ -602,7 +629,7 @@ __device__ __forceinline__ void module_prefetch(const ConvProblem &p, uint32_t w
 // the 32 sign bits of the lane's row (bit i = channel n0 + i).  The channel count is a multiple of 32, so every
 // 8-channel group is 16-byte aligned.  All 32 lanes must call it.
 template <bool HAS_ID, bool HAS_NB>
-__device__ __forceinline__ uint32_t module_chunk_t(const ConvProblem &p, const int (&dot)[32], uint32_t slot_addr, int n0)
+__device__ __forceinline__ uint32_t module_chunk_t(const ConvProblem &p, const float (&dot)[32], uint32_t slot_addr, int n0)
 {
     uint32_t bits = 0;
 #pragma unroll
@@ -628,7 +655,7 @@ __device__ __forceinline__ uint32_t module_chunk_t(const ConvProblem &p, const i
                 float r[2];
 #pragma unroll
                 for (int e = 0; e < 2; ++e) {
-                    float t = __fmul_rn(__int2float_rn(dot[c + e]), scs[2 * q + e]);
+                    float t = __fmul_rn(dot[c + e], scs[2 * q + e]);       // dot: an exact integer
                     t = __fadd_rn(t, shs[2 * q + e]);
                     const float u = HAS_ID ? __fadd_rn(t, e ? idf.y : idf.x) : t;
                     r[e] = (u >= 0.0f) ? u : __fmul_rn(sls[2 * q + e], u);
@@ -644,7 +671,7 @@ __device__ __forceinline__ uint32_t module_chunk_t(const ConvProblem &p, const i
     }
     return bits;
 }
-__device__ __forceinline__ uint32_t module_chunk(const ConvProblem &p, const int (&dot)[32], uint32_t warp_slot,
+__device__ __forceinline__ uint32_t module_chunk(const ConvProblem &p, const float (&dot)[32], uint32_t warp_slot,
                                                  long row0, int n0, int lane)
 {
     const uint32_t slot_addr = warp_slot + (uint32_t)(lane * ID_ROW_BYTES);
