@@ -235,7 +235,7 @@ conv_tc_i8_kernel(const ConvProblem p, const int ktab_words)
                 int v0, v1 = 0;
                 asm volatile("ld.shared.b32 %0, [%1];" : "=r"(v0) : "r"(part0 + 4u * c) : "memory");
                 if (two) asm volatile("ld.shared.b32 %0, [%1];" : "=r"(v1) : "r"(part1 + 4u * c) : "memory");
-                asm volatile("st.shared.b32 [%0], %1;" ::"r"(table + 4u * c), "r"(__float_as_uint((float)(v0 + v1) + (MODE == 0 ? INT_BIAS : 0.0f))) : "memory");
+                asm volatile("st.shared.b32 [%0], %1;" ::"r"(table + 4u * c), "r"(table_entry<MODE>(v0 + v1)) : "memory");
             }
             __syncwarp();
             const uint32_t t_addr = tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)(buf * BN);
@@ -248,17 +248,7 @@ conv_tc_i8_kernel(const ConvProblem p, const int ktab_words)
                     uint32_t v[32];
                     tc_ld32(t_addr + (uint32_t)col0, v);
                     if (FUSED) {
-                        // bit = (v + colc >= 0), an exact sum that is never -0; sign bits are shifted in, last column first
-                        uint32_t acc = 0;
-#pragma unroll
-                        for (int i4 = 7; i4 >= 0; --i4) {
-                            const uint4 cc = ld_shared_v4(table + 4u * (col0 + 4 * i4));
-                            acc = __funnelshift_l(fadd_bits(v[4 * i4 + 3], cc.w), acc, 1);
-                            acc = __funnelshift_l(fadd_bits(v[4 * i4 + 2], cc.z), acc, 1);
-                            acc = __funnelshift_l(fadd_bits(v[4 * i4 + 1], cc.y), acc, 1);
-                            acc = __funnelshift_l(fadd_bits(v[4 * i4 + 0], cc.x), acc, 1);
-                        }
-                        words[ch] = ~acc;
+                        words[ch] = threshold_word(v, table + 4u * col0);
                     } else if (MODULE) {
                         float dot[32];
 #pragma unroll
@@ -276,35 +266,22 @@ conv_tc_i8_kernel(const ConvProblem p, const int ktab_words)
                     } else if (BN == 128 && (p.C_out & 3) == 0 && (n0 + col0 + 32 <= p.C_out)) {
                         // full chunk (warp-uniform): staged, the warp stores whole 128-byte rows
                         int o[32];
-#pragma unroll
-                        for (int i4 = 0; i4 < 8; ++i4) {
-                            const uint4 cc = ld_shared_v4(table + 4u * (col0 + 4 * i4));
-                            o[4 * i4 + 0] = int_of_biased(fadd_bits(v[4 * i4 + 0], cc.x));
-                            o[4 * i4 + 1] = int_of_biased(fadd_bits(v[4 * i4 + 1], cc.y));
-                            o[4 * i4 + 2] = int_of_biased(fadd_bits(v[4 * i4 + 2], cc.z));
-                            o[4 * i4 + 3] = int_of_biased(fadd_bits(v[4 * i4 + 3], cc.w));
-                        }
+                        biased_ints(v, table + 4u * col0, o);
                         const long row0 = (long)em - lane;
                         store_int32_block(static_cast<int32_t *>(p.out) + row0 * p.C_out + n0 + col0, p.C_out, o, i32_tile, row0, p.M, lane);
                     } else if (em < p.M) {
                         int32_t *dst = static_cast<int32_t *>(p.out) + (long)em * p.C_out + n0 + col0;
                         const bool vec = (p.C_out & 3) == 0 && (n0 + col0 + 32 <= p.C_out);
+                        int o[32];
+                        biased_ints(v, table + 4u * col0, o);
 #pragma unroll
                         for (int i4 = 0; i4 < 8; ++i4) {
-                            const uint4 cc = ld_shared_v4(table + 4u * (col0 + 4 * i4));
-                            int4 o;
-                            o.x = int_of_biased(fadd_bits(v[4 * i4 + 0], cc.x));
-                            o.y = int_of_biased(fadd_bits(v[4 * i4 + 1], cc.y));
-                            o.z = int_of_biased(fadd_bits(v[4 * i4 + 2], cc.z));
-                            o.w = int_of_biased(fadd_bits(v[4 * i4 + 3], cc.w));
                             if (vec) {
-                                *reinterpret_cast<int4 *>(dst + 4 * i4) = o;
+                                *reinterpret_cast<int4 *>(dst + 4 * i4) = make_int4(o[4 * i4], o[4 * i4 + 1], o[4 * i4 + 2], o[4 * i4 + 3]);
                             } else {
-                                const int n = n0 + col0 + 4 * i4;
-                                if (n < p.C_out) dst[4 * i4] = o.x;
-                                if (n + 1 < p.C_out) dst[4 * i4 + 1] = o.y;
-                                if (n + 2 < p.C_out) dst[4 * i4 + 2] = o.z;
-                                if (n + 3 < p.C_out) dst[4 * i4 + 3] = o.w;
+#pragma unroll
+                                for (int i = 0; i < 4; ++i)
+                                    if (n0 + col0 + 4 * i4 + i < p.C_out) dst[4 * i4 + i] = o[4 * i4 + i];
                             }
                         }
                     }

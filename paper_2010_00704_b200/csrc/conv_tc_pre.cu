@@ -227,7 +227,7 @@ conv_tc_pre_kernel(const ConvProblem p, const int32_t *cst, const __grid_constan
                     v = __ldg(cst + n);
                     if (FUSED) v -= max(min(__ldg(p.thr + n), p.K + 1), -p.K - 1);       // beyond that bound the decision is constant
                 }
-                asm volatile("st.shared.b32 [%0], %1;" ::"r"(table + 4u * c), "r"(__float_as_uint((float)v + (FUSED ? 0.0f : INT_BIAS))) : "memory");
+                asm volatile("st.shared.b32 [%0], %1;" ::"r"(table + 4u * c), "r"(table_entry<MODE>(v)) : "memory");
             }
             __syncwarp();
             if (alive) alive = mbar_wait(tfull_bar(buf), buf_phase, abort_flag, p.err, ERR_EPILOGUE_TIMEOUT);
@@ -244,27 +244,10 @@ conv_tc_pre_kernel(const ConvProblem p, const int32_t *cst, const __grid_constan
                     uint32_t v[32];
                     tc_ld32(t_addr + (uint32_t)col0, v);
                     if (FUSED) {
-                        // bit = (v + colc >= 0), an exact sum that is never -0; sign bits are shifted in, last column first
-                        uint32_t acc = 0;
-#pragma unroll
-                        for (int i4 = 7; i4 >= 0; --i4) {
-                            const uint4 cc = ld_shared_v4(table + 4u * (col0 + 4 * i4));
-                            acc = __funnelshift_l(fadd_bits(v[4 * i4 + 3], cc.w), acc, 1);
-                            acc = __funnelshift_l(fadd_bits(v[4 * i4 + 2], cc.z), acc, 1);
-                            acc = __funnelshift_l(fadd_bits(v[4 * i4 + 1], cc.y), acc, 1);
-                            acc = __funnelshift_l(fadd_bits(v[4 * i4 + 0], cc.x), acc, 1);
-                        }
-                        words[ch] = ~acc;
+                        words[ch] = threshold_word(v, table + 4u * col0);
                     } else {
                         int o[32];
-#pragma unroll
-                        for (int i4 = 0; i4 < 8; ++i4) {
-                            const uint4 cc = ld_shared_v4(table + 4u * (col0 + 4 * i4));
-                            o[4 * i4 + 0] = int_of_biased(fadd_bits(v[4 * i4 + 0], cc.x));
-                            o[4 * i4 + 1] = int_of_biased(fadd_bits(v[4 * i4 + 1], cc.y));
-                            o[4 * i4 + 2] = int_of_biased(fadd_bits(v[4 * i4 + 2], cc.z));
-                            o[4 * i4 + 3] = int_of_biased(fadd_bits(v[4 * i4 + 3], cc.w));
-                        }
+                        biased_ints(v, table + 4u * col0, o);
                         if ((p.C_out & 3) == 0 && (n0 + col0 + 32 <= p.C_out)) {
                             // full chunk (warp-uniform): staged, the warp stores whole 128-byte rows
                             const long row0 = (long)em - lane;

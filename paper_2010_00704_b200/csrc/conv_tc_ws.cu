@@ -5,11 +5,7 @@
 // Arithmetic.  4-bit operands (tc_common.cuh): every product with a set activation bit is +-2, accumulators are fp32 in
 // tensor memory and hold exact integers, and with S = sum over set activation bits of the weight signs (acc = 2 S):
 //   sum a*g = acc + K - 2 popc(G)          (a, g in {-1,+1})
-// so the epilogue needs one constant per output channel and nothing per row - and not even an addition: the
-// accumulator buffers START from that constant (the threshold folded in for the packed output, and half a unit added, so
-// that no sum is zero and its sign bit alone decides).  The epilogue team writes the constants into its buffers once, and
-// again right after reading a tile out of one; every MMA accumulates.  The packed output is the complement of the
-// accumulators' sign bits.
+// so the epilogue needs one constant per output channel, from a table in shared memory, and nothing per row.
 // Differences to conv_tc_i8.cu, all aimed at short tiles (a 128 x 32 x 64 tile is one MMA instruction):
 //   * the CTA expands its weight tile ONCE into shared memory and keeps it for all its
 //     output tiles; only activations stream through the ring;
@@ -225,7 +221,7 @@ conv_tc_ws_kernel(const ConvProblem p)
                 tc_fence_after();
                 // per instruction: 8 tensor-memory columns of A, +2 (16-byte units) in the B descriptor
                 if (elect_one()) {
-                    tc_mma_f4_ts(d_tmem, a_t, b_lo, desc_hi, idesc, sf, 1u);      // always accumulates: the buffer holds the constants
+                    tc_mma_f4_ts(d_tmem, a_t, b_lo, desc_hi, idesc, sf, kt > 0 ? 1u : 0u);
                     if (nk > 2) tc_mma_f4_ts(d_tmem, a_t + 8u, b_lo + 2u, desc_hi, idesc, sf, 1u);
                     if (nk > 4) tc_mma_f4_ts(d_tmem, a_t + 16u, b_lo + 4u, desc_hi, idesc, sf, 1u);
                     if (nk > 6) tc_mma_f4_ts(d_tmem, a_t + 24u, b_lo + 6u, desc_hi, idesc, sf, 1u);
@@ -245,7 +241,7 @@ conv_tc_ws_kernel(const ConvProblem p)
         // After a time-out the remaining stages are released without waiting so that the issuer,
         // whose barrier wait has no time limit, always terminates; the error word tells the host.
         int s = 0, buf = 0;
-        uint32_t ring_phase = 0, buf_phase = 0;      // every accumulator buffer is handed over by its epilogue team, first after initialising it
+        uint32_t ring_phase = 0, buf_phase = 1;      // first use of every accumulator buffer: free
         bool alive = true;
         for (int ti = 0; ti < my_tiles; ++ti) {
             if (lane == 0 && alive) alive = mbar_wait(tempty_bar(buf), buf_phase, abort_flag, p.err, ERR_MMA_TIMEOUT);
@@ -283,40 +279,16 @@ conv_tc_ws_kernel(const ConvProblem p)
         };
         if (MODULE)
             for (int a = 0; a < ID_AHEAD; ++a) prefetch_next();
-        // the rows' bit counts -> the accumulators' start values:  int32, module: K - 2 popc    packed: K - 2 popc - thr + 1/2
+        // the rows' bit counts -> the epilogue's column constants: K - 2 popc, for the packed output - thr
         // (a threshold beyond +-(K + 1) decides like that bound)
         for (int c = tid - 32; c < BN; c += 32 * EPI_WARPS * TEAMS) {
             int pop;
             asm volatile("ld.shared.b32 %0, [%1];" : "=r"(pop) : "r"(colc_addr + 4u * c) : "memory");
-            float cst = (float)(p.K - 2 * pop);
-            if (FUSED) {
-                const int t = c < cn ? __ldg(p.thr + n0 + c) : 0;
-                cst = (float)(p.K - 2 * pop - max(min(t, p.K + 1), -p.K - 1)) + 0.5f;
-            }
-            asm volatile("st.shared.b32 [%0], %1;" ::"r"(colc_addr + 4u * c), "r"(__float_as_uint(cst)) : "memory");
+            int cst = p.K - 2 * pop;
+            if (FUSED) cst -= max(min(c < cn ? __ldg(p.thr + n0 + c) : 0, p.K + 1), -p.K - 1);
+            asm volatile("st.shared.b32 [%0], %1;" ::"r"(colc_addr + 4u * c), "r"(table_entry<MODE>(cst)) : "memory");
         }
         asm volatile("bar.sync 9, %0;" ::"n"(32 * EPI_WARPS * TEAMS) : "memory");
-        // write the per-channel constants into 32 accumulator columns of this warp's rows (8 columns at a time:
-        // the values are the same for every row)
-        auto write_consts = [&](uint32_t t_chunk, int col0) {
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                const uint4 a = ld_shared_v4(colc_addr + 4u * (col0 + 8 * q)), b = ld_shared_v4(colc_addr + 4u * (col0 + 8 * q + 4));
-                const uint32_t c8[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
-                tc_st8_nowait(t_chunk + 8u * q, c8);
-            }
-        };
-        // the team's accumulator buffers start out holding the constants
-        for (int b = team; b < NBUF; b += TEAMS) {
-            const uint32_t tb = tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)(b * BN);
-#pragma unroll
-            for (int ch = 0; ch < BN / 32; ++ch)
-                if (ch * 32 < cn) write_consts(tb + (uint32_t)(ch * 32), ch * 32);
-            tc_wait_st();
-            tc_fence_before();
-            __syncwarp();
-            if (lane == 0) mbar_arrive(tempty_bar(b));
-        }
         for (int ti = team; ti < my_tiles; ti += TEAMS) {
             const int buf = ti % NBUF;                            // tiles use the accumulator buffers in turn
             const uint32_t buf_phase = (uint32_t)(ti / NBUF) & 1u;
@@ -335,17 +307,18 @@ conv_tc_ws_kernel(const ConvProblem p)
                 if (col0 < cn) {                                      // warp-uniform
                     uint32_t v[32];
                     tc_ld32(t_addr + (uint32_t)col0, v);
-                    write_consts(t_addr + (uint32_t)col0, col0);      // the buffer's next tile starts from the constants again
                     if (FUSED) {
-                        // bit = (v >= 0): the sign bits are shifted in, last column first
-                        uint32_t acc = 0;
-#pragma unroll
-                        for (int i = 31; i >= 0; --i) acc = __funnelshift_l(v[i], acc, 1);
-                        words[ch] = ~acc;
+                        words[ch] = threshold_word(v, colc_addr + 4u * col0);
                     } else if (MODULE) {
                         float dot[32];
 #pragma unroll
-                        for (int i = 0; i < 32; ++i) dot[i] = __uint_as_float(v[i]);
+                        for (int i4 = 0; i4 < 8; ++i4) {
+                            const uint4 c = ld_shared_v4(colc_addr + 4u * (col0 + 4 * i4));
+                            dot[4 * i4] = __uint_as_float(fadd_bits(v[4 * i4], c.x));
+                            dot[4 * i4 + 1] = __uint_as_float(fadd_bits(v[4 * i4 + 1], c.y));
+                            dot[4 * i4 + 2] = __uint_as_float(fadd_bits(v[4 * i4 + 2], c.z));
+                            dot[4 * i4 + 3] = __uint_as_float(fadd_bits(v[4 * i4 + 3], c.w));
+                        }
                         prefetch_next();
                         cp_async_wait<ID_AHEAD>();                    // this chunk's copy has landed
                         words[ch] = module_chunk(p, dot, id_warp + (uint32_t)cur_slot * (BM * ID_ROW_BYTES), (long)em - lane, n0 + col0, lane);
@@ -353,34 +326,27 @@ conv_tc_ws_kernel(const ConvProblem p)
                     } else if ((p.C_out & 3) == 0 && (n0 + col0 + 32 <= p.C_out)) {
                         // full chunk (warp-uniform): staged, the warp stores whole 128-byte rows
                         int o[32];
-#pragma unroll
-                        for (int i = 0; i < 32; ++i) o[i] = int_of_biased(fadd_bits(v[i], __float_as_uint(INT_BIAS)));
+                        biased_ints(v, colc_addr + 4u * col0, o);
                         const long row0 = (long)em - lane;
                         store_int32_block(static_cast<int32_t *>(p.out) + row0 * p.C_out + n0 + col0, p.C_out, o, i32_tile, row0, p.M, lane);
                     } else if (em < p.M) {
                         int32_t *dst = static_cast<int32_t *>(p.out) + (long)em * p.C_out + n0 + col0;
                         const bool vec = (p.C_out & 3) == 0 && (n0 + col0 + 32 <= p.C_out);
+                        int o[32];
+                        biased_ints(v, colc_addr + 4u * col0, o);
 #pragma unroll
                         for (int i4 = 0; i4 < 8; ++i4) {
-                            int4 o;
-                            o.x = int_of_biased(fadd_bits(v[4 * i4 + 0], __float_as_uint(INT_BIAS)));
-                            o.y = int_of_biased(fadd_bits(v[4 * i4 + 1], __float_as_uint(INT_BIAS)));
-                            o.z = int_of_biased(fadd_bits(v[4 * i4 + 2], __float_as_uint(INT_BIAS)));
-                            o.w = int_of_biased(fadd_bits(v[4 * i4 + 3], __float_as_uint(INT_BIAS)));
                             if (vec) {
-                                *reinterpret_cast<int4 *>(dst + 4 * i4) = o;
+                                *reinterpret_cast<int4 *>(dst + 4 * i4) = make_int4(o[4 * i4], o[4 * i4 + 1], o[4 * i4 + 2], o[4 * i4 + 3]);
                             } else {
-                                const int n = n0 + col0 + 4 * i4;
-                                if (n < p.C_out) dst[4 * i4] = o.x;
-                                if (n + 1 < p.C_out) dst[4 * i4 + 1] = o.y;
-                                if (n + 2 < p.C_out) dst[4 * i4 + 2] = o.z;
-                                if (n + 3 < p.C_out) dst[4 * i4 + 3] = o.w;
+#pragma unroll
+                                for (int i = 0; i < 4; ++i)
+                                    if (n0 + col0 + 4 * i4 + i < p.C_out) dst[4 * i4 + i] = o[4 * i4 + i];
                             }
                         }
                     }
                 }
             }
-            tc_wait_st();                     // the constants are back in the buffer
             tc_fence_before();
             __syncwarp();
             if (lane == 0) mbar_arrive(tempty_bar(buf));
@@ -611,8 +577,8 @@ int launch_conv_tc_ws(const ConvProblem &p, cudaStream_t stream)
     if (p.C_out <= 32) return fits<32, 2, true>(p) ? launch_ws<32, 2, true>(p, stream) : launch_ws<32, 4, false>(p, stream);
     if (p.C_out <= 64) return fits<64, 2, true>(p) ? launch_ws<64, 2, true>(p, stream) : launch_ws<64, 4, false>(p, stream);
     // C_out > 128: slices of 128 (or 64) output channels, each CTA keeps one slice's weights
+    if (fits<128, 4, false, 2>(p)) return launch_ws<128, 4, false, 2>(p, stream);
     if (fits<128, 2, true>(p)) return launch_ws<128, 2, true>(p, stream);
-    if (fits<128, 4, false>(p)) return launch_ws<128, 4, false>(p, stream);
     if (fits<128, 2, false>(p)) return launch_ws<128, 2, false>(p, stream);     // long K: fewer producer groups, smaller staging ring
     return fits<64, 2, true>(p) ? launch_ws<64, 2, true>(p, stream) : launch_ws<64, 4, false>(p, stream);
 }

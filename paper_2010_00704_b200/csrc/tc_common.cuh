@@ -343,6 +343,44 @@ __device__ __forceinline__ uint32_t fadd_bits(uint32_t a, uint32_t b)
 {
     return __float_as_uint(__fadd_rn(__uint_as_float(a), __uint_as_float(b)));
 }
+// Output word of 32 accumulator columns: bit = (v + c >= 0) for exact integers v and c, with 2 c + 1 of column i at
+// table + 4 i.  2 (v + c) + 1 is an odd integer, so saturated to [0, 1] it is the bit; two chains of 16 Horner steps collect
+// the bits as fp32 integers below 2^16.  All of it runs on the fp32 pipe at full rate - an addition and a shift per column
+// would take two slots of the logic pipe, which the activations' expansion needs.
+__device__ __forceinline__ uint32_t threshold_word(const uint32_t (&v)[32], uint32_t table)
+{
+    float lo = 0.0f, hi = 0.0f;
+#pragma unroll
+    for (int i4 = 3; i4 >= 0; --i4) {
+        const uint4 a = ld_shared_v4(table + 16u * i4), b = ld_shared_v4(table + 64u + 16u * i4);
+        const uint32_t ca[4] = {a.x, a.y, a.z, a.w}, cb[4] = {b.x, b.y, b.z, b.w};
+#pragma unroll
+        for (int i = 3; i >= 0; --i) {
+            lo = fmaf(lo, 2.0f, __saturatef(fmaf(__uint_as_float(v[4 * i4 + i]), 2.0f, __uint_as_float(ca[i]))));
+            hi = fmaf(hi, 2.0f, __saturatef(fmaf(__uint_as_float(v[16 + 4 * i4 + i]), 2.0f, __uint_as_float(cb[i]))));
+        }
+    }
+    // integers below 2^16 in the low mantissa bits of 2^23 + x
+    return __byte_perm(__float_as_uint(lo + 8388608.0f), __float_as_uint(hi + 8388608.0f), 0x5410);
+}
+// ... and 32 exact integers v + c, with c + INT_BIAS of column i at table + 4 i.
+__device__ __forceinline__ void biased_ints(const uint32_t (&v)[32], uint32_t table, int (&o)[32])
+{
+#pragma unroll
+    for (int i4 = 0; i4 < 8; ++i4) {
+        const uint4 c = ld_shared_v4(table + 16u * i4);
+        o[4 * i4] = int_of_biased(fadd_bits(v[4 * i4], c.x));
+        o[4 * i4 + 1] = int_of_biased(fadd_bits(v[4 * i4 + 1], c.y));
+        o[4 * i4 + 2] = int_of_biased(fadd_bits(v[4 * i4 + 2], c.z));
+        o[4 * i4 + 3] = int_of_biased(fadd_bits(v[4 * i4 + 3], c.w));
+    }
+}
+// What an epilogue's column table holds for the constant c (MODE 0: int32, 1: packed, 2: module).
+template <int MODE> __device__ __forceinline__ uint32_t table_entry(int c)
+{
+    return __float_as_uint(MODE == 0 ? (float)c + INT_BIAS : (MODE == 1 ? (float)(2 * c + 1) : (float)c));
+}
+
 // K word e (0..7) of a 256-bit stage of a weight row: 16 bytes of a 128-byte-swizzled row; zeros where not live
 __device__ __forceinline__ void expand_store_w4(uint32_t w, bool live, uint32_t row_addr, int xr, int e)
 {
