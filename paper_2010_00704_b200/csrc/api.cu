@@ -470,6 +470,7 @@ const char *bcnn_status_string(int status)
     case 154: return "device wait timed out: wide pointwise tcgen05 engine, epilogue waiting for an accumulator";
     case 155: return "device wait timed out: wide pointwise tcgen05 engine, producer waiting for an activation unit's previous MMAs";
     case 156: return "device wait timed out: wide pointwise tcgen05 engine, issuer waiting for an accumulator";
+    case 161: return "device wait timed out: depth-wise module, a tile's input did not arrive";
     case BCNN_SELFTEST_TIMEOUT_CODE: return "device wait timed out: self-test (expected)";
     default: return status > 0 ? "device-side error code" : "unknown status";
     }

@@ -5,7 +5,8 @@
 // traffic of the fp16 NHWC maps: a thread handles 8 consecutive channels (16 bytes) of one output pixel, arithmetic in
 // fp32.  The depth-wise module can also emit the next binary module's sign bits (bias + sign of the stored value), so
 // that the map is not read again by a pack pass.
-#include "bcnn_common.cuh"
+#include "tc_common.cuh"
+#include "tensor_map.cuh"
 #include <cuda_fp16.h>
 
 namespace bcnn {
@@ -23,6 +24,212 @@ __device__ __forceinline__ void unpack8(const uint4 &v, float (&f)[8])
     }
 }
 
+// ---- depth-wise 3x3, stride 1 or 2 --------------------------------------------------------------------------------
+// Bound by the fp16 maps' traffic once everything else is out of the way.  A CTA owns CB channels (32 or 64) and walks
+// tiles of 8 x TW output pixels; a tile's input halo arrives by one tiled TMA copy (4D box, out-of-image = zero fill = the
+// padding) into one of two buffers, the next tile's while this one is computed.  A thread owns four channels - weights and
+// per-channel values in registers for the CTA's life - and slides along a strip of L = TW / 2 pixels of two output rows:
+// every input column is read and converted once for both rows (4 or 5 8-byte shared loads at immediate offsets).  Per output
+// value: nine multiply-adds in the fixed order (r, t), two at a time (f32x2: the same two IEEE operations, half the issue
+// slots).  The kernel before this one kept one output pixel per thread and read 13 per-channel vectors from shared memory
+// for each - 26 16-byte shared loads per 16 bytes of output, 0.7 TB/s at stride 1 (maps read + written once).
+struct F4 { unsigned long long lo, hi; };                  // four fp32 values as two f32x2 pairs
+
+__device__ __forceinline__ unsigned long long pack2(float a, float b)
+{
+    unsigned long long r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+    return r;
+}
+__device__ __forceinline__ void unpack2(unsigned long long v, float &a, float &b) { asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v)); }
+__device__ __forceinline__ unsigned long long fma2(unsigned long long a, unsigned long long b, unsigned long long c)
+{
+    unsigned long long d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+    return d;
+}
+__device__ __forceinline__ F4 to_f4(const uint2 &v)
+{
+    const float2 a = __half22float2(*reinterpret_cast<const __half2 *>(&v.x)), b = __half22float2(*reinterpret_cast<const __half2 *>(&v.y));
+    return {pack2(a.x, a.y), pack2(b.x, b.y)};
+}
+
+constexpr int DW_TH = 8, DW_NR = 2, DW_STRIPS = DW_TH;        // strips of a tile: TH / NR row pairs x two segments
+constexpr int ERR_DW_TIMEOUT = 161;
+
+// S: stride; TW: output columns of a tile; CB: channels of a CTA
+template <int S, int TW, int CB> struct DwCfg {
+    static constexpr int L = TW / 2;
+    static constexpr int HB = (DW_TH - 1) * S + 3, WB = (TW - 1) * S + 3;      // halo: rows, pixels
+    static constexpr int G = CB / 4, THREADS = DW_STRIPS * G;
+    static constexpr int BYTES = HB * WB * CB * 2, BUF = (BYTES + 127) / 128 * 128;     // a copy's bytes; buffers on 128-byte boundaries
+    static constexpr int SMEM = 2 * BUF + 128;
+};
+
+template <int S, int TW, int CB, bool BITS>
+__global__ void __launch_bounds__(DwCfg<S, TW, CB>::THREADS, 512 / DwCfg<S, TW, CB>::THREADS)
+dw_tile_kernel(const __grid_constant__ CUtensorMap xmap, const float *w, const float *scale, const float *shift, const float *slope,
+               const float *next_bias, uint16_t *y, uint8_t *y_bits, int C_in, int C, int OH, int OW,
+               unsigned tiles_x, unsigned tiles_y, unsigned tiles, unsigned cblocks, int *err)
+{
+    using D = DwCfg<S, TW, CB>;
+    constexpr int ROWS = (DW_NR - 1) * S + 3;                  // input rows of a strip: 4 or 5
+    extern __shared__ unsigned char dw_raw[];
+    __shared__ __align__(8) unsigned long long full[2];
+    __shared__ int abort_flag;
+    const unsigned tid = threadIdx.x, cb = blockIdx.x % cblocks, step = gridDim.x / cblocks;
+    const uint32_t buf0 = (tc::smem_u32(dw_raw) + 127u) & ~127u, bar0 = tc::smem_u32(full);
+    if (tid == 0) {
+        tc::mbar_init(bar0, 1);
+        tc::mbar_init(bar0 + 8, 1);
+        abort_flag = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    __syncthreads();
+    const unsigned g = tid % D::G, st = tid / D::G;
+    const int c0 = (int)cb * CB + 4 * (int)g;                  // first output channel; it reads channel c mod C_in
+    const bool have = c0 < C;
+    const int rp = (int)(st >> 1), sg = (int)(st & 1);
+    pdl_wait();
+    auto tile_at = [&](unsigned t, unsigned &b, int &oh0, int &ow0) {
+        const unsigned per = tiles_x * tiles_y;
+        b = t / per;
+        const unsigned rem = t - b * per, ty = rem / tiles_x;
+        oh0 = (int)ty * DW_TH;
+        ow0 = (int)(rem - ty * tiles_x) * TW;
+    };
+    auto issue = [&](unsigned t, unsigned which) {              // one thread
+        unsigned b;
+        int oh0, ow0;
+        tile_at(t, b, oh0, ow0);
+        const uint32_t bar = bar0 + 8u * which;
+        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"((uint32_t)D::BYTES) : "memory");
+        asm volatile("cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, %5}], [%6];"
+                     ::"r"(buf0 + which * (uint32_t)D::BUF), "l"(reinterpret_cast<uint64_t>(&xmap)), "r"((int)(cb * CB) % C_in), "r"(ow0 * S - 1),
+                       "r"(oh0 * S - 1), "r"((int)b), "r"(bar) : "memory");
+    };
+    const unsigned first = blockIdx.x / cblocks;
+    if (tid == 0) {
+        if (first < tiles) issue(first, 0);
+        if (first + step < tiles) issue(first + step, 1);
+    }
+    // weights of the four channels: 36 consecutive floats [c][9]
+    F4 wt[9], sc, sh;
+    float sl[4], nb[4];
+    {
+        float f[36];
+        const int cw = have ? c0 : 0;
+#pragma unroll
+        for (int i = 0; i < 9; ++i) {
+            const float4 v = __ldg(reinterpret_cast<const float4 *>(w + (long)cw * 9) + i);
+            f[4 * i] = v.x; f[4 * i + 1] = v.y; f[4 * i + 2] = v.z; f[4 * i + 3] = v.w;
+        }
+#pragma unroll
+        for (int i = 0; i < 9; ++i) wt[i] = {pack2(f[i], f[9 + i]), pack2(f[18 + i], f[27 + i])};
+        const float4 a = __ldg(reinterpret_cast<const float4 *>(scale + cw)), d = __ldg(reinterpret_cast<const float4 *>(shift + cw));
+        const float4 e = __ldg(reinterpret_cast<const float4 *>(slope + cw));
+        const float4 n = BITS && next_bias ? __ldg(reinterpret_cast<const float4 *>(next_bias + cw)) : make_float4(0.f, 0.f, 0.f, 0.f);
+        sc = {pack2(a.x, a.y), pack2(a.z, a.w)};
+        sh = {pack2(d.x, d.y), pack2(d.z, d.w)};
+        sl[0] = e.x; sl[1] = e.y; sl[2] = e.z; sl[3] = e.w;
+        nb[0] = n.x; nb[1] = n.y; nb[2] = n.z; nb[3] = n.w;
+    }
+    const uint32_t my_off = (uint32_t)((2 * rp * S * D::WB + sg * D::L * S) * CB * 2) + 8u * g;
+    unsigned n = 0;
+    bool ok = true;
+    for (unsigned t = first; t < tiles; t += step, ++n) {
+        ok = tc::mbar_wait(bar0 + 8u * (n & 1u), (n >> 1) & 1u, &abort_flag, err, ERR_DW_TIMEOUT);
+        if (__syncthreads_or(!ok)) break;
+        unsigned b;
+        int oh0, ow0;
+        tile_at(t, b, oh0, ow0);
+        const int oh = oh0 + DW_NR * rp, ow1 = ow0 + sg * D::L;
+        const uint32_t src = buf0 + (n & 1u) * (uint32_t)D::BUF + my_off;
+        uint16_t *yp = y + (((long)b * OH + oh) * OW + ow1) * C + c0;
+        const bool row_ok[DW_NR] = {have && oh < OH, have && oh + 1 < OH};
+        auto column = [&](int col, F4 (&c)[ROWS]) {             // column `col` of the strip's window
+#pragma unroll
+            for (int r = 0; r < ROWS; ++r) {
+                uint2 v;
+                asm volatile("ld.shared.v2.b32 {%0,%1}, [%2];" : "=r"(v.x), "=r"(v.y) : "r"(src + (uint32_t)((r * D::WB + col) * CB * 2)));
+                c[r] = to_f4(v);
+            }
+        };
+        F4 win[3][ROWS];
+        column(0, win[0]);
+        if (S == 1) column(1, win[1]);
+#pragma unroll
+        for (int i = 0; i < D::L; ++i) {
+            const int ia = S == 1 ? i % 3 : (2 * i) % 3, im = S == 1 ? (i + 1) % 3 : (2 * i + 1) % 3, iz = S == 1 ? (i + 2) % 3 : (2 * i + 2) % 3;
+            if (S == 2) column(2 * i + 1, win[im]);
+            column(S * i + 2, win[iz]);
+#pragma unroll
+            for (int q = 0; q < DW_NR; ++q) {
+                F4 acc = {0ull, 0ull};
+#pragma unroll
+                for (int r = 0; r < 3; ++r) {
+                    acc.lo = fma2(win[ia][q * S + r].lo, wt[3 * r].lo, acc.lo); acc.hi = fma2(win[ia][q * S + r].hi, wt[3 * r].hi, acc.hi);
+                    acc.lo = fma2(win[im][q * S + r].lo, wt[3 * r + 1].lo, acc.lo); acc.hi = fma2(win[im][q * S + r].hi, wt[3 * r + 1].hi, acc.hi);
+                    acc.lo = fma2(win[iz][q * S + r].lo, wt[3 * r + 2].lo, acc.lo); acc.hi = fma2(win[iz][q * S + r].hi, wt[3 * r + 2].hi, acc.hi);
+                }
+                acc.lo = fma2(acc.lo, sc.lo, sh.lo);
+                acc.hi = fma2(acc.hi, sc.hi, sh.hi);
+                float v[4];
+                unpack2(acc.lo, v[0], v[1]);
+                unpack2(acc.hi, v[2], v[3]);
+#pragma unroll
+                for (int k = 0; k < 4; ++k) v[k] = v[k] >= 0.f ? v[k] : sl[k] * v[k];
+                const __half2 h0 = __floats2half2_rn(v[0], v[1]), h1 = __floats2half2_rn(v[2], v[3]);
+                const bool live = row_ok[q] && ow1 + i < OW;
+                uint16_t *dst = yp + (long)q * OW * C;
+                if (live) *reinterpret_cast<uint2 *>(dst) = make_uint2(*reinterpret_cast<const uint32_t *>(&h0), *reinterpret_cast<const uint32_t *>(&h1));
+                if (BITS) {
+                    const float2 f0 = __half22float2(h0), f1 = __half22float2(h1);
+                    uint32_t bits = (__fadd_rn(f0.x, nb[0]) >= 0.f ? 1u : 0u) | (__fadd_rn(f0.y, nb[1]) >= 0.f ? 2u : 0u) |
+                                    (__fadd_rn(f1.x, nb[2]) >= 0.f ? 4u : 0u) | (__fadd_rn(f1.y, nb[3]) >= 0.f ? 8u : 0u);
+                    bits |= __shfl_down_sync(0xffffffffu, bits, 1) << 4;      // an even lane and its neighbour are one byte
+                    if (live && (g & 1u) == 0) y_bits[(dst - y) >> 3] = (uint8_t)bits;
+                }
+            }
+            yp += C;
+        }
+        __syncthreads();                                        // the buffer has been read
+        if (tid == 0 && t + 2 * step < tiles) issue(t + 2 * step, n & 1u);
+    }
+    // after a time-out: copies still in flight must land before the CTA's shared memory goes away
+    if (!ok || abort_flag) {
+        for (unsigned k = 0; k < 2; ++k)
+            if (first + (n + k) * step < tiles) tc::mbar_wait(bar0 + 8u * ((n + k) & 1u), ((n + k) >> 1) & 1u, &abort_flag, nullptr, 0);
+    }
+    pdl_trigger();
+}
+
+template <int S, int TW, int CB>
+int launch_dw_tile(const uint16_t *x, const float *w, const float *scale, const float *shift, const float *slope, const float *next_bias,
+                   uint16_t *y, uint8_t *y_bits, int B, int H, int W, int C_in, int C, int OH, int OW, cudaStream_t stream)
+{
+    using D = DwCfg<S, TW, CB>;
+    EncodeTiledFn encode = encode_tiled_fn();
+    if (!encode) return BCNN_ERR_CUDA;
+    CUtensorMap xmap;
+    const cuuint64_t dims[4] = {(cuuint64_t)C_in, (cuuint64_t)W, (cuuint64_t)H, (cuuint64_t)B};
+    const cuuint64_t strides[3] = {(cuuint64_t)C_in * 2, (cuuint64_t)W * C_in * 2, (cuuint64_t)H * W * C_in * 2};
+    const cuuint32_t box[4] = {CB, D::WB, D::HB, 1}, estr[4] = {1, 1, 1, 1};
+    if (encode(&xmap, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 4, const_cast<uint16_t *>(x), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+               CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+        return BCNN_ERR_CUDA;
+    auto k = y_bits ? dw_tile_kernel<S, TW, CB, true> : dw_tile_kernel<S, TW, CB, false>;
+    if (!allow_smem((const void *)k, D::SMEM)) return BCNN_ERR_CUDA;
+    const unsigned tx = (unsigned)(OW + TW - 1) / TW, ty = (unsigned)(OH + DW_TH - 1) / DW_TH, tiles = tx * ty * (unsigned)B;
+    const unsigned cblocks = (unsigned)(C + CB - 1) / CB;
+    // resident blocks, the same number for every channel block and the same number of tiles (+-1) for each
+    unsigned per = (unsigned)sm_count() * (unsigned)blocks_per_sm((const void *)k, D::THREADS, D::SMEM) / cblocks;
+    if (per < 1) per = 1;
+    if (per > tiles) per = tiles;
+    return launch(k, per * cblocks, D::THREADS, D::SMEM, stream, xmap, w, scale, shift, slope, next_bias, y, y_bits, C_in, C, OH, OW, tx, ty, tiles, cblocks, device_error_word());
+}
+
+// Any stride and channel count (the tiles above take strides 1 and 2 and channel blocks that replication does not split): one output pixel x 8 channels per thread.
 // x fp16 [B][H][W][C_in] -> y fp16 [B][OH][OW][C], C = R * C_in; w fp32 [C][3][3].
 // The block's thread count is a multiple of the 8-channel groups, so a thread keeps its group; weights (tap-major, so
 // that a warp's groups read consecutive 32-byte pieces) and per-channel values sit in shared memory.  A block walks a
@@ -127,34 +334,76 @@ dwconv3x3_module_kernel(const uint16_t *x, const float *w, const float *scale, c
     }
 }
 
+// S x S / S average pooling with replication, bound by the maps' traffic.  A thread takes 8 channels of AP output pixels
+// (AP * S * S 16-byte loads in flight), reads every input value once and writes its R copies (channel c reads c mod C_in).
+// SS: the stride where it is known to the compiler (1, 2), else 0.
+constexpr int AP = 4;
+template <int SS>
 __global__ void __launch_bounds__(256)
-avgpool_kernel(const uint16_t *x, uint16_t *y, int B, int H, int W, int C_in, int C, int S)
+avgpool_kernel(const uint16_t *x, uint16_t *y, unsigned items, int H, int W, int C_in, int R, int S_any)
 {
     pdl_trigger();
-    pdl_wait();
-    const int OH = H / S, OW = W / S, groups = C / 8;
-    const long total = (long)B * OH * OW * groups;
+    const int S = SS ? SS : S_any;
+    const unsigned OW = (unsigned)(W / S), OH = (unsigned)(H / S), groups = (unsigned)C_in / 8;
+    const long C = (long)C_in * R;
     const float inv = 1.0f / (float)(S * S);
-    for (long i = (long)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (long)gridDim.x * blockDim.x) {
-        const int g = (int)(i % groups);
-        const long pix = i / groups;
-        const int ow = (int)(pix % OW), oh = (int)((pix / OW) % OH), b = (int)(pix / ((long)OW * OH));
-        const int c0 = 8 * g, ci0 = c0 % C_in;
-        float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-        for (int r = 0; r < S; ++r)
-            for (int t = 0; t < S; ++t) {
-                float xv[8];
-                unpack8(__ldg(reinterpret_cast<const uint4 *>(x + (((long)b * H + oh * S + r) * W + ow * S + t) * C_in + ci0)), xv);
+    pdl_wait();
+    const unsigned stride = gridDim.x * 256u, first = blockIdx.x * 256u + threadIdx.x;
+    // AP items, `stride` apart, at a time: item = (output pixel, group of 8 channels)
+    for (unsigned i0 = first; i0 < items; i0 += AP * stride) {
+        float acc[AP][8];
+        long src[AP], dst[AP];
+        bool ok[AP];
 #pragma unroll
-                for (int c = 0; c < 8; ++c) acc[c] += xv[c];
-            }
-        uint32_t o[4];
+        for (int u = 0; u < AP; ++u) {
+            const unsigned i = i0 + u * stride;
+            ok[u] = i < items && i >= i0;
+            const unsigned pix = i / groups, g = i - pix * groups;
+            const unsigned row = pix / OW, ow = pix - row * OW, b = row / OH, oh = row - b * OH;
+            src[u] = (((long)b * H + (long)oh * S) * W + (long)ow * S) * C_in + 8 * g;
+            dst[u] = (long)pix * C + 8 * g;
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            const __half2 y2 = __floats2half2_rn(acc[2 * q] * inv, acc[2 * q + 1] * inv);
-            o[q] = *reinterpret_cast<const uint32_t *>(&y2);
+            for (int c = 0; c < 8; ++c) acc[u][c] = 0.f;
         }
-        *reinterpret_cast<uint4 *>(y + pix * C + c0) = make_uint4(o[0], o[1], o[2], o[3]);
+        if (SS) {
+            uint4 v[AP][SS ? SS * SS : 1];
+#pragma unroll
+            for (int u = 0; u < AP; ++u)
+#pragma unroll
+                for (int q = 0; q < SS * SS; ++q)
+                    v[u][q] = ok[u] ? __ldg(reinterpret_cast<const uint4 *>(x + src[u] + ((long)(q / (SS ? SS : 1)) * W + q % (SS ? SS : 1)) * C_in)) : make_uint4(0u, 0u, 0u, 0u);
+#pragma unroll
+            for (int u = 0; u < AP; ++u)
+#pragma unroll
+                for (int q = 0; q < SS * SS; ++q) {
+                    float xv[8];
+                    unpack8(v[u][q], xv);
+#pragma unroll
+                    for (int c = 0; c < 8; ++c) acc[u][c] += xv[c];
+                }
+        } else {
+            for (int r = 0; r < S; ++r)
+                for (int t = 0; t < S; ++t)
+#pragma unroll
+                    for (int u = 0; u < AP; ++u)
+                        if (ok[u]) {
+                            float xv[8];
+                            unpack8(__ldg(reinterpret_cast<const uint4 *>(x + src[u] + ((long)r * W + t) * C_in)), xv);
+#pragma unroll
+                            for (int c = 0; c < 8; ++c) acc[u][c] += xv[c];
+                        }
+        }
+#pragma unroll
+        for (int u = 0; u < AP; ++u) {
+            uint32_t o[4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const __half2 y2 = __floats2half2_rn(acc[u][2 * q] * inv, acc[u][2 * q + 1] * inv);
+                o[q] = *reinterpret_cast<const uint32_t *>(&y2);
+            }
+            if (ok[u])
+                for (int k = 0; k < R; ++k) *reinterpret_cast<uint4 *>(y + dst[u] + (long)k * C_in) = make_uint4(o[0], o[1], o[2], o[3]);
+        }
     }
 }
 
@@ -243,6 +492,18 @@ int launch_dwconv3x3_module(const uint16_t *x, const float *w, const float *scal
     const int smem = 13 * C * 4;
     if (groups > 256 || smem > 200 * 1024) return BCNN_ERR_UNSUPPORTED;      // more than 2048 channels
     if ((long)B * OH * OW >= (1L << 31)) return BCNN_ERR_UNSUPPORTED;         // pixel indices are 32-bit
+    // tiles of 8 x 16 output pixels at stride 1 (8 x 8 where that covers the row with less waste, and at stride 2: the halo is
+    // 17 x 17 pixels); 64 channels, or 32 where 64 do not divide the input's channels
+    const int CB = C_in % 64 == 0 ? 64 : 32;
+    if (S <= 2 && (R == 1 || C_in % CB == 0) && (long)B * ((OH + 7) / 8) * ((OW + 7) / 8) < (1L << 30)) {
+        const bool narrow = S == 2 || (OW + 7) / 8 * 8 < (OW + 15) / 16 * 16;
+        if (S == 1 && narrow) return CB == 64 ? launch_dw_tile<1, 8, 64>(x, w, scale, shift, slope, next_bias, y, y_bits, B, H, W, C_in, C, OH, OW, stream)
+                                              : launch_dw_tile<1, 8, 32>(x, w, scale, shift, slope, next_bias, y, y_bits, B, H, W, C_in, C, OH, OW, stream);
+        if (S == 1) return CB == 64 ? launch_dw_tile<1, 16, 64>(x, w, scale, shift, slope, next_bias, y, y_bits, B, H, W, C_in, C, OH, OW, stream)
+                                    : launch_dw_tile<1, 16, 32>(x, w, scale, shift, slope, next_bias, y, y_bits, B, H, W, C_in, C, OH, OW, stream);
+        return CB == 64 ? launch_dw_tile<2, 8, 64>(x, w, scale, shift, slope, next_bias, y, y_bits, B, H, W, C_in, C, OH, OW, stream)
+                        : launch_dw_tile<2, 8, 32>(x, w, scale, shift, slope, next_bias, y, y_bits, B, H, W, C_in, C, OH, OW, stream);
+    }
     const int threads = (256 / groups) * groups;                            // <= 256, a multiple of groups
     const long passes = ((long)B * OH * OW + threads / groups - 1) / (threads / groups);
     const int sms = sm_count();
@@ -255,8 +516,19 @@ int launch_dwconv3x3_module(const uint16_t *x, const float *w, const float *scal
 
 int launch_avgpool(const uint16_t *x, uint16_t *y, int B, int H, int W, int C_in, int R, int S, cudaStream_t stream)
 {
-    const int C = C_in * R;
-    return launch(avgpool_kernel, grid_for((long)B * (H / S) * (W / S) * (C / 8)), 256, 0, stream, x, y, B, H, W, C_in, C, S);
+    const long items = (long)B * (H / S) * (W / S) * (C_in / 8);
+    if (items >= (1L << 31)) {                       // item numbers are 32-bit: whole images per launch
+        const int part = (int)(((1L << 31) - 1) / (items / B));
+        if (part < 1) return BCNN_ERR_UNSUPPORTED;
+        for (int b = 0; b < B; b += part) {
+            const int st = launch_avgpool(x + (long)b * H * W * C_in, y + (long)b * (H / S) * (W / S) * C_in * R, B - b < part ? B - b : part, H, W, C_in, R, S, stream);
+            if (st != BCNN_OK) return st;
+        }
+        return BCNN_OK;
+    }
+    void (*k)(const uint16_t *, uint16_t *, unsigned, int, int, int, int, int) = S == 1 ? avgpool_kernel<1> : (S == 2 ? avgpool_kernel<2> : avgpool_kernel<0>);
+    const long blocks = (items + 256 * AP - 1) / (256 * AP), cap = (long)sm_count() * blocks_per_sm((const void *)k, 256, 0);
+    return launch(k, (unsigned)(blocks < cap ? blocks : cap), 256, 0, stream, x, y, (unsigned)items, H, W, C_in, R, S);
 }
 
 int launch_gap(const uint16_t *x, float *pooled, int B, int HW, int C, cudaStream_t stream)

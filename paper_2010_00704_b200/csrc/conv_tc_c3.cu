@@ -39,7 +39,7 @@
 // and, NB being a multiple of NACC, tile n + 8 needs the accumulator of tile n back from the epilogue.
 // Every mbarrier wait is bounded and reports through the device error word.
 #include "tc_slot.cuh"
-#include <cuda.h>
+#include "tensor_map.cuh"
 
 namespace bcnn {
 
@@ -445,22 +445,6 @@ conv_tc_c3_kernel(const ConvProblem p, const C3Geom g, const __grid_constant__ C
     }
 }
 
-typedef CUresult (*EncodeTiledFn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *, const cuuint64_t *, const cuuint64_t *,
-                                  const cuuint32_t *, const cuuint32_t *, CUtensorMapInterleave, CUtensorMapSwizzle,
-                                  CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-
-EncodeTiledFn c3_encode_fn()
-{
-    static EncodeTiledFn fn = nullptr;
-    if (!fn) {
-        void *ptr = nullptr;
-        cudaDriverEntryPointQueryResult qres;
-        if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &ptr, cudaEnableDefault, &qres) == cudaSuccess && qres == cudaDriverEntryPointSuccess)
-            fn = reinterpret_cast<EncodeTiledFn>(ptr);
-    }
-    return fn;
-}
-
 template <int CW, int BN>
 int launch_c3(const ConvProblem &p0, cudaStream_t stream)
 {
@@ -471,7 +455,7 @@ int launch_c3(const ConvProblem &p0, cudaStream_t stream)
     const int smem = c3_smem_bytes<CW, BN>(g);
     if (smem > 227 * 1024 - 1024) return BCNN_ERR_UNSUPPORTED;
     const int sms = sm_count();
-    EncodeTiledFn encode = c3_encode_fn();
+    EncodeTiledFn encode = encode_tiled_fn();
     if (!encode) return BCNN_ERR_CUDA;
     // the packed input as [B][H][W * CW] 32-bit words; box = wbw words x hb rows of one image; zero fill outside
     CUtensorMap xmap;

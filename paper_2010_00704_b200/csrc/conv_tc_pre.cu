@@ -19,7 +19,7 @@
 //   control warp  the issuer's mbarrier waits
 // Every mbarrier wait is bounded and reports through the device error word.
 #include "tc_common.cuh"
-#include <cuda.h>
+#include "tensor_map.cuh"
 
 namespace bcnn {
 
@@ -387,22 +387,6 @@ prepare_weights_kernel(const uint32_t *w, uint8_t *wexp, int32_t *cst, int N, in
             for (int kw = 0; kw < kwords; ++kw) pop += __popc(__ldg(w + n * kwords + kw));
         cst[n] = n < N ? kwords * 32 - 2 * pop : 0;
     }
-}
-
-typedef CUresult (*EncodeTiledFn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *, const cuuint64_t *, const cuuint64_t *,
-                                  const cuuint32_t *, const cuuint32_t *, CUtensorMapInterleave, CUtensorMapSwizzle,
-                                  CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-
-EncodeTiledFn encode_tiled_fn()
-{
-    static EncodeTiledFn fn = nullptr;
-    if (!fn) {
-        void *ptr = nullptr;
-        cudaDriverEntryPointQueryResult qres;
-        if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &ptr, cudaEnableDefault, &qres) == cudaSuccess && qres == cudaDriverEntryPointSuccess)
-            fn = reinterpret_cast<EncodeTiledFn>(ptr);
-    }
-    return fn;
 }
 
 int ktab_words_for(const ConvProblem &p) { return ((p.kwords + 7) >> 3) * (8 / gather_width(p.cw)); }

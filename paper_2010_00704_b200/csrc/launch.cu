@@ -1,5 +1,6 @@
 // Per-process caches behind launch.cuh.
 #include "launch.cuh"
+#include "tensor_map.cuh"
 
 namespace bcnn {
 
@@ -46,6 +47,20 @@ int current_device()
 uint64_t kernel_key(const void *kernel, int dev) { return ((uint64_t)reinterpret_cast<uintptr_t>(kernel) << 6) | (uint64_t)(dev & 63); }
 
 }  // namespace
+
+EncodeTiledFn encode_tiled_fn()
+{
+    static std::atomic<EncodeTiledFn> fn{nullptr};
+    EncodeTiledFn f = fn.load(std::memory_order_relaxed);
+    if (!f) {
+        void *ptr = nullptr;
+        cudaDriverEntryPointQueryResult qres;
+        if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &ptr, cudaEnableDefault, &qres) == cudaSuccess && qres == cudaDriverEntryPointSuccess)
+            f = reinterpret_cast<EncodeTiledFn>(ptr);
+        fn.store(f, std::memory_order_relaxed);
+    }
+    return f;
+}
 
 int sm_count()
 {
