@@ -19,8 +19,6 @@ int *device_error_word()
     return cache[dev];
 }
 
-namespace {
-
 // (mul, shift) of exact_div for the divisor d >= 1
 void exact_div_params(uint32_t d, uint32_t &mul, uint32_t &shift)
 {
@@ -30,6 +28,8 @@ void exact_div_params(uint32_t d, uint32_t &mul, uint32_t &shift)
     mul = (uint32_t)(((1ULL << 32) * ((1ULL << s) - d)) / d + 1);
     shift = s;
 }
+
+namespace {
 
 inline bool aligned16(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
@@ -225,8 +225,10 @@ int bcnn_conv2d_b1_module(const void *x_bits, const void *w_bits, const float *b
     p.identity = static_cast<const uint16_t *>(identity);
     p.y_real = static_cast<uint16_t *>(y_real);
     p.out = y_bits;
-    // the two tcgen05 engines carry this epilogue; it is bound by the epilogue warps, of which the weight-stationary
-    // engine has twice as many per SM whenever two of its CTAs fit (wider layers run as 128-channel slices)
+    // pointwise layers (the paper's only binary convolution) have an engine of their own; the two general tcgen05 engines
+    // carry the same epilogue for every other shape
+    const int mod = launch_conv_tc_mod(p, static_cast<cudaStream_t>(stream));
+    if (mod != BCNN_ERR_UNSUPPORTED) return mod;
     if (conv_tc_ws_supports(p)) return launch_conv_tc_ws(p, static_cast<cudaStream_t>(stream));
     return launch_conv_tc_i8(p, static_cast<cudaStream_t>(stream));
 }
@@ -256,6 +258,9 @@ int bcnn_conv2d_b1_branches(const void *x_bits, const void *w_bits, const float 
     p.cw = C_in / 32;
     p.M = (long)B * H * W;
     if (p.M >= (1L << 40)) return BCNN_ERR_UNSUPPORTED;
+    // on the tensor cores where the branches' accumulators and one slice of their weights fit (13 branches), else on the CUDA cores
+    const int mod = launch_branches_tc_mod(p, static_cast<cudaStream_t>(stream));
+    if (mod != BCNN_ERR_UNSUPPORTED) return mod;
     return launch_conv_branches(p, static_cast<cudaStream_t>(stream));
 }
 
@@ -471,6 +476,12 @@ const char *bcnn_status_string(int status)
     case 155: return "device wait timed out: wide pointwise tcgen05 engine, producer waiting for an activation unit's previous MMAs";
     case 156: return "device wait timed out: wide pointwise tcgen05 engine, issuer waiting for an accumulator";
     case 161: return "device wait timed out: depth-wise module, a tile's input did not arrive";
+    case 171: return "device wait timed out: module engine, producer waiting for a free ring slot";
+    case 172: return "device wait timed out: module engine, issuer waiting for a full slot or a free accumulator";
+    case 173: return "device wait timed out: module engine, epilogue waiting for an accumulator";
+    case 174: return "device wait timed out: module engine, epilogue waiting for an identity tile or a free staging tile";
+    case 175: return "device wait timed out: module engine, loader waiting for a free staging tile";
+    case 176: return "device wait timed out: module engine, store warp waiting for an output tile";
     case BCNN_SELFTEST_TIMEOUT_CODE: return "device wait timed out: self-test (expected)";
     default: return status > 0 ? "device-side error code" : "unknown status";
     }

@@ -114,6 +114,9 @@ bool conv_tc_pre_supports(const ConvProblem &p);
 int launch_conv_tc_pre_static(const ConvProblem &p, cudaStream_t stream);   // prepared weights in the library's static array
 size_t static_prepared_capacity();
 bool conv_tc_i8_supports(const ConvProblem &p);
+int launch_conv_tc_mod(const ConvProblem &p, cudaStream_t stream);
+int launch_branches_tc_mod(const BranchProblem &b, cudaStream_t stream);
+void exact_div_params(uint32_t d, uint32_t &mul, uint32_t &shift);   // (mul, shift) of exact_div for the divisor d >= 1
 int launch_selftest_wait_timeout(int polls, cudaStream_t stream);
 int launch_conv_branches(const BranchProblem &p, cudaStream_t stream);
 int launch_dwconv3x3_module(const uint16_t *x, const float *w, const float *scale, const float *shift, const float *slope,

@@ -6,67 +6,86 @@
 
 namespace bcnn {
 
-// Streaming path, no replication, C_in % 32 == 0: the tensor is a flat array of
-// fp32 values and every aligned group of 32 values becomes one output word.  Lane l of
-// a warp reads value l of a group (one coalesced 128-byte request per group) and the
-// warp vote assembles the word, bit l = lane l = channel l of the group (LSB first).
-// UNROLL groups are in flight per warp to cover HBM latency.
-template <int UNROLL, bool HAS_BIAS>
+// Streaming path, no replication, C_in % 32 == 0: the tensor is a flat array of fp32 values and every aligned group of 32
+// becomes one output word.  A thread takes four consecutive values (one 16-byte load) and leaves a nibble; eight lanes make a
+// word, a warp stores four.  PACK_U loads are in flight per thread, `stride` quads apart.  FIXED: the stride is a multiple of
+// the C_in / 4 quads of a pixel, so a thread keeps its four biases in registers; else one 32-bit remainder per load (the
+// 64-bit remainder per 32 values of the kernel before this one held 28x28x256 at batch 128 to 2.2 TB/s).
+constexpr int PACK_U = 4;
+template <bool FIXED>
 __global__ void __launch_bounds__(256)
-pack_stream_kernel(const float *__restrict__ x, const float *__restrict__ bias,
-                   uint32_t *__restrict__ out, long nwords, int cwords)
+pack_stream_kernel(const float4 *__restrict__ x, const float4 *__restrict__ bias, uint32_t *__restrict__ out, long quads, unsigned q)
 {
     pdl_trigger();
+    const long stride = (long)gridDim.x * 256, first = (long)blockIdx.x * 256 + threadIdx.x;
+    const unsigned lane = threadIdx.x & 31u;
     pdl_wait();
-    const int lane = threadIdx.x & 31;
-    const long warp = (long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    const long nwarps = (long)gridDim.x * (blockDim.x >> 5);
-    for (long w0 = warp * UNROLL; w0 < nwords; w0 += nwarps * UNROLL) {
-        float v[UNROLL];
+    float4 b = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (FIXED && bias) b = __ldg(bias + (unsigned)(first % q));
+    for (long i0 = first; i0 - lane < quads; i0 += PACK_U * stride) {           // warp-uniform: quads is a multiple of 8
+        float4 v[PACK_U];
 #pragma unroll
-        for (int u = 0; u < UNROLL; ++u) {
-            const long wi = w0 + u;
-            v[u] = (wi < nwords) ? __ldcs(x + wi * 32 + lane) : -1.0f;
+        for (int u = 0; u < PACK_U; ++u) {
+            const long i = i0 + u * stride;
+            v[u] = i < quads ? __ldcs(x + i) : make_float4(0.f, 0.f, 0.f, 0.f);
         }
-        uint32_t word[UNROLL];
 #pragma unroll
-        for (int u = 0; u < UNROLL; ++u) {
-            float s = v[u];
-            if (HAS_BIAS) {
-                const long wi = w0 + u;
-                const int cword = (int)(wi % cwords);
-                s = __fadd_rn(s, __ldg(bias + cword * 32 + lane));
-            }
-            word[u] = __ballot_sync(0xffffffffu, s >= 0.0f);
+        for (int u = 0; u < PACK_U; ++u) {
+            const long i = i0 + u * stride;
+            if (!FIXED) b = i < quads ? __ldg(bias + (unsigned)((unsigned long)i < (1ul << 32) ? (unsigned)i % q : i % q)) : b;
+            // without a bias b is zero: x + 0 >= 0 decides like x >= 0 (NaN and -0 included)
+            uint32_t w = (__fadd_rn(v[u].x, b.x) >= 0.f ? 1u : 0u) | (__fadd_rn(v[u].y, b.y) >= 0.f ? 2u : 0u) |
+                         (__fadd_rn(v[u].z, b.z) >= 0.f ? 4u : 0u) | (__fadd_rn(v[u].w, b.w) >= 0.f ? 8u : 0u);
+            w <<= 4 * (lane & 7u);
+            w |= __shfl_xor_sync(0xffffffffu, w, 1);
+            w |= __shfl_xor_sync(0xffffffffu, w, 2);
+            w |= __shfl_xor_sync(0xffffffffu, w, 4);
+            if ((lane & 7u) == 0 && i < quads) __stcs(out + (i >> 3), w);
         }
-        // lane u stores word u: one contiguous UNROLL*4-byte segment per warp
-        uint32_t mine = 0;
-#pragma unroll
-        for (int u = 0; u < UNROLL; ++u)
-            if (lane == u) mine = word[u];
-        if (lane < UNROLL && w0 + lane < nwords) out[w0 + lane] = mine;
     }
 }
 
-// General path: any C_in and replication factor R with R*C_in % 32 == 0.  One warp
-// per output word; lane l evaluates channel c = 32*word + l, which reads input channel
-// c mod C_in of the same pixel.
+// General path: any C_in and replication factor R with R*C_in % 32 == 0.  A warp takes PACK_P pixels at a time (as many loads
+// in flight) and walks their words; lane l evaluates channel c = 32*word + l, which reads input channel c mod C_in.  NV: where
+// a lane meets only NV different input channels (C_in a divisor of 32: 1; 64: 2; 128: 4) they are read once per pixel, else
+// (NV = 0) once per word.
+constexpr int PACK_P = 8;
+template <int NV>
 __global__ void __launch_bounds__(256)
-pack_general_kernel(const float *__restrict__ x, const float *__restrict__ bias,
-                    uint32_t *__restrict__ out, long nwords, int C_in, int cwords)
+pack_general_kernel(const float *__restrict__ x, const float *__restrict__ bias, uint32_t *__restrict__ out, long npix, int C_in, int cwords)
 {
     pdl_trigger();
-    pdl_wait();
     const int lane = threadIdx.x & 31;
-    const long warp = (long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    const long nwarps = (long)gridDim.x * (blockDim.x >> 5);
-    for (long wi = warp; wi < nwords; wi += nwarps) {
-        const long pix = wi / cwords;
-        const int c = (int)(wi - pix * cwords) * 32 + lane;
-        float s = __ldg(x + pix * C_in + (c % C_in));
-        if (bias) s = __fadd_rn(s, __ldg(bias + c));
-        const uint32_t word = __ballot_sync(0xffffffffu, s >= 0.0f);
-        if (lane == 0) out[wi] = word;
+    const long warp = (long)blockIdx.x * 8 + (threadIdx.x >> 5), nwarps = (long)gridDim.x * 8;
+    const int adv = 32 % C_in;
+    pdl_wait();
+    for (long p0 = warp * PACK_P; p0 < npix; p0 += nwarps * PACK_P) {
+        int ci = lane % C_in;
+        float v[NV ? NV : 1][PACK_P];
+        auto load = [&](float (&d)[PACK_P], int c) {
+#pragma unroll
+            for (int u = 0; u < PACK_P; ++u) d[u] = p0 + u < npix ? __ldg(x + (p0 + u) * C_in + c) : -1.f;
+        };
+        if (NV)
+#pragma unroll
+            for (int k = 0; k < NV; ++k) load(v[k], ci + 32 * k);
+        for (int w0 = 0; w0 < cwords; w0 += NV ? NV : 1) {      // cwords is a multiple of NV
+#pragma unroll
+            for (int k = 0; k < (NV ? NV : 1); ++k) {
+                const int w = w0 + k;
+                if (!NV) load(v[0], ci);
+                const float b = bias ? __ldg(bias + 32 * w + lane) : 0.f;
+                uint32_t mine = 0;
+#pragma unroll
+                for (int u = 0; u < PACK_P; ++u) {
+                    const uint32_t word = __ballot_sync(0xffffffffu, __fadd_rn(v[k][u], b) >= 0.f);
+                    if (lane == u) mine = word;
+                }
+                if (lane < PACK_P && p0 + lane < npix) out[(p0 + lane) * cwords + w] = mine;
+            }
+            ci += adv;
+            if (ci >= C_in) ci -= C_in;
+        }
     }
 }
 
@@ -185,14 +204,18 @@ int launch_pack(const float *x, const float *bias, uint32_t *out, long npix, int
     const int sms = sm_count();
     const int threads = 256;
     if (R == 1 && C_in % 32 == 0) {
-        constexpr int UNROLL = 8;
-        const long warps_needed = (nwords + UNROLL - 1) / UNROLL;
-        long blocks = (warps_needed + 7) / 8;
+        const long quads = nwords * 8;
+        const unsigned q = (unsigned)C_in / 4;
+        long blocks = (quads + threads * PACK_U - 1) / (threads * PACK_U);
         const long cap = (long)sms * 8;
         if (blocks > cap) blocks = cap;
-        if (blocks < 1) blocks = 1;
-        return launch(bias ? pack_stream_kernel<UNROLL, true> : pack_stream_kernel<UNROLL, false>, (unsigned)blocks, threads, 0, stream,
-                      x, bias, out, nwords, cwords);
+        // blocks such that a pass is a whole number of pixels
+        unsigned m = q;                                  // q / gcd(q, 256)
+        for (int i = 0; i < 8 && m % 2 == 0; ++i) m /= 2;
+        const bool fixed = !bias || (long)m <= blocks;
+        if (bias && fixed) blocks -= blocks % m;
+        return launch(fixed ? pack_stream_kernel<true> : pack_stream_kernel<false>, (unsigned)blocks, threads, 0, stream,
+                      reinterpret_cast<const float4 *>(x), reinterpret_cast<const float4 *>(bias), out, quads, q);
     } else if (C_in == 4 && R == 8) {
         long blocks = (npix + threads * 4 - 1) / (threads * 4);
         const long cap = (long)sms * blocks_per_sm((const void *)pack_c4r8_kernel, threads, 0);       // one wave of resident CTAs, grid-stride inside
@@ -200,10 +223,11 @@ int launch_pack(const float *x, const float *bias, uint32_t *out, long npix, int
         if (blocks < 1) blocks = 1;
         return launch(pack_c4r8_kernel, (unsigned)blocks, threads, 0, stream, reinterpret_cast<const float4 *>(x), bias, out, npix);
     } else {
-        long blocks = (nwords + 7) / 8;
+        long blocks = (npix + 8 * PACK_P - 1) / (8 * PACK_P);
         const long cap = (long)sms * 8;
         if (blocks > cap) blocks = cap;
-        return launch(pack_general_kernel, (unsigned)blocks, threads, 0, stream, x, bias, out, nwords, C_in, cwords);
+        auto k = 32 % C_in == 0 ? pack_general_kernel<1> : (C_in == 64 ? pack_general_kernel<2> : (C_in == 128 ? pack_general_kernel<4> : pack_general_kernel<0>));
+        return launch(k, (unsigned)blocks, threads, 0, stream, x, bias, out, npix, C_in, cwords);
     }
 }
 
