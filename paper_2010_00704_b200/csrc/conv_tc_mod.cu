@@ -31,7 +31,7 @@ constexpr int ERR_MOD_PRODUCER = 171, ERR_MOD_ISSUER = 172, ERR_MOD_EPILOGUE = 1
 constexpr int G = 2;                      // producer groups of four warps
 constexpr int PF = 3;                     // packed-word stages in flight per producer thread
 constexpr int TEAMS = 2, NS = 3;          // epilogue teams of four warps; staging tiles per team
-constexpr int ISSUER = 0, LOADER = 1, STORER = 2, FIRST_PRODUCER = 4, FIRST_EPILOGUE = FIRST_PRODUCER + 4 * G;
+constexpr int ISSUER = 0, LOADER = 1, STORER = 2 /* + team */, FIRST_PRODUCER = 4, FIRST_EPILOGUE = FIRST_PRODUCER + 4 * G;
 constexpr int THREADS = 32 * (FIRST_EPILOGUE + 4 * TEAMS);
 constexpr int PROD_THREADS = G * BM;
 constexpr int HALF_BYTES = PROD_THREADS * 16, SLOT_BYTES = 2 * HALF_BYTES;
@@ -99,7 +99,7 @@ conv_tc_mod_kernel(const ModPlan L, const __grid_constant__ CUtensorMap idmap, c
 {
     constexpr int TILE_BYTES = BM * BN * 2, ROW_BYTES = BN * 2, W_STAGE = BN * ROWB;
     extern __shared__ unsigned char smem_raw[];
-    __shared__ __align__(8) unsigned long long bars[2 * MAX_STAGES + 4 + 3 * TEAMS * NS];
+    __shared__ __align__(8) unsigned long long bars[2 * MAX_STAGES + 4 + 3 * TEAMS * NS + 1];
     __shared__ uint32_t tmem_base_smem;
     __shared__ int abort_flag_smem;
 
@@ -122,6 +122,7 @@ conv_tc_mod_kernel(const ModPlan L, const __grid_constant__ CUtensorMap idmap, c
     auto id_full = [&](int t, int s) { return bar0 + 8u * (2 * MAX_STAGES + 4 + t * NS + s); };
     auto slot_free = [&](int t, int s) { return bar0 + 8u * (2 * MAX_STAGES + 4 + TEAMS * NS + t * NS + s); };
     auto out_full = [&](int t, int s) { return bar0 + 8u * (2 * MAX_STAGES + 4 + 2 * TEAMS * NS + t * NS + s); };
+    const uint32_t ready_bar = bar0 + 8u * (2 * MAX_STAGES + 4 + 3 * TEAMS * NS);      // the resident weights are expanded
     volatile int *abort_flag = &abort_flag_smem;
 
     if (tid == 0) {
@@ -138,6 +139,7 @@ conv_tc_mod_kernel(const ModPlan L, const __grid_constant__ CUtensorMap idmap, c
                 mbar_init(out_full(t, s), 4);
             }
         }
+        mbar_init(ready_bar, 4 * TEAMS);
         abort_flag_smem = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
@@ -157,58 +159,11 @@ conv_tc_mod_kernel(const ModPlan L, const __grid_constant__ CUtensorMap idmap, c
     }
     const int npop = rs * P * BN;
     for (int i = tid; i < npop; i += THREADS) asm volatile("st.shared.b32 [%0], %1;" ::"r"(pops + 4u * i), "r"(0) : "memory");
-    pdl_wait();
-    __syncthreads();
-    // ---- one-off: the resident slices' weights and their bit counts, eight words in flight per thread
-    {
-        constexpr int WU = 8;
-        const int total = rs * kst * BN * 8;
-        for (int i0 = tid; i0 < total; i0 += WU * THREADS) {
-            uint32_t w[WU];
-            bool live[WU];
-            int pop_at[WU];
-            uint32_t dst[WU];
-#pragma unroll
-            for (int u = 0; u < WU; ++u) {
-                const int i = i0 + u * THREADS, e = i & 7, rk = i >> 3, row_s = rk / kst, kt = rk - row_s * kst;     // row_s = slice * BN + row
-                const int sl = row_s / BN, row = row_s % BN, ch = (cg * L.rs + sl) * BN + row;
-                const int kw = kt * 8 + e, br = kw / L.kwp, j = kw - br * L.kwp;
-                live[u] = i < total && br < P && j < L.bcw && ch < p.C_out;
-                w[u] = live[u] ? __ldg(p.w + ((long)br * p.C_out + ch) * L.bcw + j) : 0u;
-                pop_at[u] = (sl * P + br) * BN + row;
-                dst[u] = base + (uint32_t)((sl * kst + kt) * W_STAGE + row * ROWB + ((e ^ (row & 7)) << 4));
-            }
-#pragma unroll
-            for (int u = 0; u < WU; ++u) {
-                if (i0 + u * THREADS >= total) break;
-                const uint4 o = live[u] ? expand_w4(w[u]) : make_uint4(0u, 0u, 0u, 0u);
-                st_shared_v4(dst[u], o.x, o.y, o.z, o.w);
-                if (live[u]) asm volatile("red.shared.add.u32 [%0], %1;" ::"r"(pops + 4u * pop_at[u]), "r"(__popc(w[u])) : "memory");
-            }
-        }
-    }
-    __syncthreads();
-    for (int i = tid; i < rs * BN; i += THREADS) {
-        const int sl = i / BN, c = i % BN, ch = (cg * L.rs + sl) * BN + c;
-        const bool have = ch < p.C_out;
-        const uint32_t ent = table + (uint32_t)(i >> 1) * pair_bytes(P) + 4u * (i & 1);
-        for (int br = 0; br < P; ++br) {
-            int pop;
-            asm volatile("ld.shared.b32 %0, [%1];" : "=r"(pop) : "r"(pops + 4u * ((sl * P + br) * BN + c)) : "memory");
-            const long at = (long)br * p.C_out + ch;
-            const float v[4] = {have ? __ldg(L.scale + at) : 0.f, have ? __ldg(L.shift + at) : 0.f, (float)(32 * L.bcw - 2 * pop),
-                                SHIFTED && have && L.pad_dot ? (float)__ldg(L.pad_dot + at) : 0.f};
-#pragma unroll
-            for (int k = 0; k < 4; ++k) asm volatile("st.shared.b32 [%0], %1;" ::"r"(ent + 32u * br + 8u * k), "r"(__float_as_uint(v[k])) : "memory");
-        }
-        asm volatile("st.shared.b32 [%0], %1;" ::"r"(ent + 32u * P), "r"(__float_as_uint(have ? __ldg(p.slope + ch) : 0.f)) : "memory");
-        asm volatile("st.shared.b32 [%0], %1;" ::"r"(ent + 32u * P + 8u), "r"(__float_as_uint(have && p.next_bias ? __ldg(p.next_bias + ch) : 0.f)) : "memory");
-    }
-    fence_async_proxy();
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
     pdl_trigger();
+    pdl_wait();
     const uint32_t tmem_base = tmem_base_smem;
 
     // part n = (row tile n / rs, slice n % rs); team n % 2, its n / 2-th part, staging tile (n / 2) % NS
@@ -223,7 +178,8 @@ conv_tc_mod_kernel(const ModPlan L, const __grid_constant__ CUtensorMap idmap, c
         const uint32_t tmem_u = __shfl_sync(0xffffffffu, tmem_base, 0);
         const uint32_t sf = tmem_u + (uint32_t)SF_COL, a_col0 = tmem_u + (uint32_t)(L.nbuf * P * BN);
         const int per_branch = L.kwp >> 1, granules = P * per_branch;      // two-word MMAs of a branch, of a row
-        bool ok = true;
+        bool ok = mbar_wait_warp(ready_bar, 0, abort_flag, p.err, ERR_MOD_ISSUER);
+        tc_fence_after();
         for (int n = 0; n < parts && ok; ++n) {
             const int tile = n / rs, s = n - tile * rs;
             if (n >= L.nbuf) {
@@ -273,18 +229,19 @@ conv_tc_mod_kernel(const ModPlan L, const __grid_constant__ CUtensorMap idmap, c
                 for (int n = issued > TEAMS * NS ? issued - TEAMS * NS : 0; n < issued; ++n)
                     mbar_wait_warp(id_full(n & 1, (n >> 1) % NS), (uint32_t)((n >> 1) / NS) & 1u, abort_flag, nullptr, 0);
         }
-    } else if (warp == STORER) {
-        // ------------------------------------------------------------------ output tiles
-        for (int n = 0; n < parts; ++n) {
-            const int team = n & 1, m = n >> 1, s = m % NS;
+    } else if (warp < FIRST_PRODUCER) {
+        // ------------------------------------------------------------------ output tiles of team warp - STORER
+        const int team = warp - STORER;
+        for (int n = team; n < parts; n += TEAMS) {
+            const int m = n >> 1, s = m % NS;
             if (!mbar_wait_warp(out_full(team, s), (uint32_t)(m / NS) & 1u, abort_flag, p.err, ERR_MOD_STORE)) break;
             if (lane == 0) {
                 asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.tile.bulk_group [%0, {%1, %2}], [%3];"
                              ::"l"(reinterpret_cast<uint64_t>(&ymap)), "r"(part_ch(n)), "r"(part_row(n)), "r"(staging + (uint32_t)((team * NS + s) * TILE_BYTES)) : "memory");
                 asm volatile("cp.async.bulk.commit_group;" ::: "memory");
-                if (n > 0) {                                                // the store before this one has read its tile
+                if (m > 0) {                                                // the store before this one has read its tile
                     asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory");
-                    mbar_arrive(slot_free((n - 1) & 1, ((n - 1) >> 1) % NS));
+                    mbar_arrive(slot_free(team, (m - 1) % NS));
                 }
             }
             __syncwarp();
@@ -293,6 +250,63 @@ conv_tc_mod_kernel(const ModPlan L, const __grid_constant__ CUtensorMap idmap, c
         __syncwarp();
     } else if (warp >= FIRST_EPILOGUE) {
         // ------------------------------------------------------------------ epilogue
+        // ---- one-off, while the first rows and identity tiles arrive: the resident slices' weights (the issuer waits for them)
+        // with their bit counts, then the table.  Eight words are in flight per thread, and a channel's parameters before them.
+        constexpr int ETHREADS = 128 * TEAMS;
+        const int etid = tid - 32 * FIRST_EPILOGUE;
+        {
+            constexpr int WU = 8;
+            const int total = rs * kst * BN * 8;
+            for (int i0 = etid; i0 < total; i0 += WU * ETHREADS) {
+                uint32_t w[WU];
+                bool live[WU];
+                int pop_at[WU];
+                uint32_t dst[WU];
+#pragma unroll
+                for (int u = 0; u < WU; ++u) {
+                    const int i = i0 + u * ETHREADS, e = i & 7, rk = i >> 3, row_s = rk / kst, kt = rk - row_s * kst;     // row_s = slice * BN + row
+                    const int sl = row_s / BN, row = row_s % BN, ch = (cg * L.rs + sl) * BN + row;
+                    const int kw = kt * 8 + e, br = kw / L.kwp, j = kw - br * L.kwp;
+                    live[u] = i < total && br < P && j < L.bcw && ch < p.C_out;
+                    w[u] = live[u] ? __ldg(p.w + ((long)br * p.C_out + ch) * L.bcw + j) : 0u;
+                    pop_at[u] = (sl * P + br) * BN + row;
+                    dst[u] = base + (uint32_t)((sl * kst + kt) * W_STAGE + row * ROWB + ((e ^ (row & 7)) << 4));
+                }
+#pragma unroll
+                for (int u = 0; u < WU; ++u) {
+                    if (i0 + u * ETHREADS >= total) break;
+                    const uint4 o = live[u] ? expand_w4(w[u]) : make_uint4(0u, 0u, 0u, 0u);
+                    st_shared_v4(dst[u], o.x, o.y, o.z, o.w);
+                    if (live[u]) asm volatile("red.shared.add.u32 [%0], %1;" ::"r"(pops + 4u * pop_at[u]), "r"(__popc(w[u])) : "memory");
+                }
+            }
+        }
+        fence_async_proxy();
+        asm volatile("bar.sync 1, %0;" ::"n"(ETHREADS) : "memory");
+        if (lane == 0) mbar_arrive(ready_bar);
+        for (int i = etid; i < rs * P * BN; i += ETHREADS) {                // (slice, branch, channel)
+            const int c = i % BN, sb = i / BN, br = sb % P, sl = sb / P, ch = (cg * L.rs + sl) * BN + c;
+            const bool have = ch < p.C_out;
+            const long at = (long)br * p.C_out + ch;
+            const float sc = have ? __ldg(L.scale + at) : 0.f, sh = have ? __ldg(L.shift + at) : 0.f;
+            const float pd = SHIFTED && have && L.pad_dot ? (float)__ldg(L.pad_dot + at) : 0.f;
+            float slope = 0.f, nb = 0.f;
+            if (br == 0 && have) {
+                slope = __ldg(p.slope + ch);
+                nb = p.next_bias ? __ldg(p.next_bias + ch) : 0.f;
+            }
+            int pop;
+            asm volatile("ld.shared.b32 %0, [%1];" : "=r"(pop) : "r"(pops + 4u * i) : "memory");
+            const uint32_t ent = table + (uint32_t)((sl * BN + c) >> 1) * pair_bytes(P) + 4u * (c & 1);
+            const float v[4] = {sc, sh, (float)(32 * L.bcw - 2 * pop), pd};
+#pragma unroll
+            for (int k = 0; k < 4; ++k) asm volatile("st.shared.b32 [%0], %1;" ::"r"(ent + 32u * br + 8u * k), "r"(__float_as_uint(v[k])) : "memory");
+            if (br == 0) {
+                asm volatile("st.shared.b32 [%0], %1;" ::"r"(ent + 32u * P), "r"(__float_as_uint(slope)) : "memory");
+                asm volatile("st.shared.b32 [%0], %1;" ::"r"(ent + 32u * P + 8u), "r"(__float_as_uint(nb)) : "memory");
+            }
+        }
+        asm volatile("bar.sync 1, %0;" ::"n"(ETHREADS) : "memory");
         const int team = (warp - FIRST_EPILOGUE) >> 2, quad = warp & 3, row = quad * 32 + lane;
         const uint32_t t_lane = tmem_base + ((uint32_t)(quad * 32) << 16);
         const int owords = p.C_out >> 5;
@@ -472,7 +486,7 @@ bool make_plan(ModPlan &L, int &smem)
     for (int rs = 1; rs <= L.slices && rs <= 16; ++rs) {
         if (rs > 1 && L.kst > L.stages) break;               // the row tile's stages stay in the ring for all its parts
         const long pops = (long)rs * L.P * BN * 4, table = (long)rs * (BN / 2) * pair_bytes(L.P);
-        const long bytes = 1024 + rs * slice_bytes + (pops > staging ? pops : staging) + (long)PF * SLOT_BYTES + table + 4L * L.units + 64;
+        const long bytes = 1024 + rs * slice_bytes + staging + pops + (long)PF * SLOT_BYTES + table + 4L * L.units + 64;
         if (bytes > MAX_SMEM) break;
         const int ng = (L.slices + rs - 1) / rs, per = sms / ng;
         if (per < 1) continue;
@@ -483,8 +497,8 @@ bool make_plan(ModPlan &L, int &smem)
         L.rs = rs;
         L.ng = ng;
         L.off_stage = (uint32_t)(rs * slice_bytes);
-        L.off_pop = L.off_stage;                             // (the counts are read before the first copy is issued)
-        L.off_bits = L.off_stage + (uint32_t)((pops > staging ? pops : staging) + 127) / 128 * 128;
+        L.off_pop = L.off_stage + (uint32_t)staging;
+        L.off_bits = L.off_pop + (uint32_t)pops;
         L.off_table = L.off_bits + (uint32_t)PF * SLOT_BYTES;
         L.off_tab = (L.off_table + (uint32_t)table + 15u) & ~15u;
         smem = (int)bytes;
@@ -525,7 +539,7 @@ int launch_mod(ModPlan &L, bool shifted, cudaStream_t stream)
     if ((long)q.B * q.H * q.W * q.cw >= (1L << 31) || (long)q.kh * q.W * q.cw >= (1L << 27) || 32L * L.bcw > (1 << 16)) return BCNN_ERR_UNSUPPORTED;
     L.m_tiles = (q.M - 1) / BM + 1;
     int smem = 0;
-    if (L.P <= 3 && make_plan<64>(L, smem)) {
+    if (L.P <= 3 && q.C_out > 32 && make_plan<64>(L, smem)) {
         if (shifted) return launch_plan<64, 0, true>(L, smem, stream);
         if (L.P == 1) return launch_plan<64, 1, false>(L, smem, stream);
         if (L.P == 2) return launch_plan<64, 2, false>(L, smem, stream);
