@@ -11,32 +11,28 @@
 //     copy's first word must be 16-byte aligned, so the box starts up to three pixels left of the halo (XOFF);
 //   * a producer thread (= one output pixel) reads its nine pixels' words from the halo tile at compile-time offsets,
 //     expands them and stores them to tensor memory: per K word one shared-memory load and the eight logic operations.
-// Arithmetic as in the pointwise engine (conv_tc_pw.cu): unsigned activation bytes {0, 2^j} against signed weight bytes,
-// every product +-64, the per-channel constant written by a first MMA against a constant activation tile.
+// Arithmetic: 4-bit operands (tc_common.cuh), fp32 accumulators that hold exact integers, the per-channel constants written by
+// a first MMA so that the epilogue needs 16 bits and a sign (tc_slot.cuh).
 //
 // One commit per tile.  Tensor memory holds NACC accumulators and a ring of NUNIT activation UNITS: the nine taps of
-// 32 input channels of one tile (72 columns).  A tile is one unit for C_in = 32 and two for C_in = 64 (K order: channel
-// word, then tap).  An issuer warp walks tiles in order: it waits until the tile's units are full and its accumulator
-// free, issues the tile's MMAs and ONE commit on the tile's "done" barrier, which the epilogue (accumulator ready) and
-// the producers (units free again) wait on: with the producers ahead the MMAs of consecutive tiles queue back to back.
+// 32 input channels of one tile, 40 columns (ten words of K: two per MMA, the tenth meets zero weights).  A tile is one unit
+// for C_in = 32 and two for C_in = 64 (K order: channel word, then tap).  Two issuer warps take alternate tiles (an issuer's
+// waits, its 5 or 10 instructions and its commit take about as long as a tile's MMAs run): wait until the tile's units are
+// full and its accumulator free, issue the tile's MMAs and ONE commit on the tile's "done" barrier, which the epilogue
+// (accumulator ready) and the producers (units free again) wait on.
 // Four producer groups of four warps fill ONE unit of every tile they take:
-//   * C_in = 64 (tiles of 640+ tensor-pipe cycles, one issuer): groups 2 j and 2 j + 1 fill the two units of the tiles
-//     n = j (mod 2).  The ring holds five (six) units = two and a half (three) tiles, so a tile's first unit reuses
-//     columns that were free one tile earlier than those of its second unit: only half of a tile's stores have to fit
-//     into the time of one tile's MMAs;
-//   * C_in = 32 (tiles of 160 - 320 tensor-pipe cycles, bound by instruction issue): group j fills the tiles
-//     n = j (mod 4), and two issuer warps take alternate tiles (one issuer's waits and commit would be the bound); the
-//     ring then has an even number of units, so that a unit's next user belongs to the same issuer.
+//   * C_in = 64: groups 2 j and 2 j + 1 fill the two units of the tiles n = j (mod 2);
+//   * C_in = 32: group j fills the tiles n = j (mod 4).
 // Two loader warps and two epilogue groups take alternate tiles.
-// The "done" barriers form a ring of NB = 8 (tile n -> barrier n % 8), a multiple of NACC and more than the tiles in
-// flight.  K = 288: |accumulator| <= 32 (2 K + 1) < 2^15, so the epilogue reads packed 16-bit halves and gathers sign
-// bits with byte permutes; K = 576: 32-bit accumulators, sign bits shifted in.
+// The "done" barriers form a ring of NB = 16 (tile n -> barrier n % 16), a multiple of NACC and more than the tiles in
+// flight.
 // A parity wait on an mbarrier is only right while the waiter starts waiting for completion k after completion k - 1 and
-// before completion k + 1.  Tile n's "done" is completion n / 8 of its barrier; its waiters are the epilogue of tile n
-// and the producers of the tiles (at most four ahead) that reuse its units.  Every one of them has seen an earlier tile
-// of the same issuer done within the last eight (an issuer's tiles complete in order), and tile n + 8 cannot be issued
-// before they are through: its issuer first issues the reusing tiles (the same issuer), which need those units filled,
-// and, NB being a multiple of NACC, tile n + 8 needs the accumulator of tile n back from the epilogue.
+// before completion k + 1.  Tile m's "done" is completion m / NB of its barrier; its waiters are the epilogue of tile m and
+// the producers of tile m + D, D = NUNIT / CW <= NB / 2, which reuse its units.  A producer group's tiles are an even number
+// apart, so its wait before this one was for an earlier tile of the same issuer, and an issuer's tiles complete in order:
+// completion k - 1 has happened.  Tile m + NB cannot be done before the waiter is through: the fills of the tiles from
+// m + 2 D on need tile m + D (or a later one of its issuer) done, hence filled; NB being a multiple of NACC, it also needs the
+// accumulator of tile m back from the epilogue.
 // Every mbarrier wait is bounded and reports through the device error word.
 #include "tc_slot.cuh"
 #include "tensor_map.cuh"
@@ -58,33 +54,27 @@ constexpr int TH = 8, TW = 16;            // output tile (TH * TW = 128 = tensor
 constexpr int NGRP = 2;                   // loader / epilogue groups (alternate tiles)
 constexpr int NPG = 4;                    // producer groups of four warps
 constexpr int RD = 6;                     // halo tiles in a loader's ring
-constexpr int CONST_COLS = 8;
-constexpr int TAPS = 9;
-constexpr int U_COLS = 8 * TAPS;          // columns of a unit
-constexpr int NB = 8;                     // ring of "tile done" barriers
-constexpr int NAF = 4;                    // ring of "tile full" barriers (at most four tiles are being filled)
-constexpr int MAX_NUNIT = 6, MAX_NACC = 4;
+constexpr int TAPS = 9, UWORDS = 10;      // K words of a unit: the nine taps and a zero
+constexpr int U_COLS = 4 * UWORDS;        // columns of a unit
+constexpr int NB = 16;                    // ring of "tile done" barriers
+constexpr int NAF = 8;                    // ring of "tile full" barriers (at most eight tiles are being filled)
+constexpr int MAX_NUNIT = 8, MAX_NACC = 4;
 
 // CW: words per input pixel (1, 2) = units per tile; BN: accumulator columns per tile (32, 64, 128 >= C_out).
 template <int CW, int BN> struct C3Cfg {
     static constexpr int KW = TAPS * CW;                    // words of K per row
-    static constexpr int KT = (KW + 3) / 4;                 // 128-byte stages of the expanded weights
+    static constexpr int KT = (UWORDS * CW + 7) / 8;        // 256-bit stages of the expanded weights
     // 128 output channels run as two halves of 64 against the same activation units: the accumulator of one half is
-    // read by its epilogue group while the other half's MMAs run (one 128-column accumulator would leave room for
-    // neither a second one nor enough units)
+    // read by its epilogue group while the other half's MMAs run
     static constexpr int NH = BN == 128 ? 2 : 1;            // halves
     static constexpr int AW = BN / NH;                      // accumulator columns
-    static constexpr int NACC = NH == 2 ? 2 : (CW == 1 && BN == 32 ? 4 : 2);   // accumulators (NH == 2: one per half)
-    static constexpr int NISS = CW == 2 || NH == 2 ? 1 : 2; // issuer warps
-    static constexpr bool PACK16 = CW == 1;
-    static constexpr int NU0 = (512 - CONST_COLS - NACC * AW) / U_COLS;
-    static constexpr int NU1 = NU0 > MAX_NUNIT ? MAX_NUNIT : NU0;
-    static constexpr int NUNIT = CW == 1 ? (NU1 > 4 ? 4 : NU1 / 2 * 2) : NU1;   // 4 (C_in 32); 6, 5, 5 (C_in 64)
+    static constexpr int NACC = NH == 2 ? 2 : 4;            // accumulators (NH == 2: one per half)
+    static constexpr int NISS = NH == 2 ? 1 : 2;            // issuer warps
+    static constexpr int NU0 = (CB_COL - NACC * AW) / U_COLS;
+    static constexpr int NUNIT = NU0 >= MAX_NUNIT ? MAX_NUNIT : NU0 / CW * CW;   // 8 (32 columns), 6 (64), 8 (128)
     static constexpr int A_COL0 = NACC * AW;
-    static constexpr int C_COL = A_COL0 + NUNIT * U_COLS;   // the constant activation tile
-    static_assert(C_COL + CONST_COLS <= 512, "tensor memory budget");
-    static_assert(NUNIT >= 2 * CW && (NUNIT + CW - 1) / CW <= NAF && NB % NACC == 0 && NACC <= MAX_NACC && NACC % NISS == 0 &&
-                  (NISS == 1 || NUNIT % NISS == 0), "barrier rings");
+    static_assert(A_COL0 + NUNIT * U_COLS <= CB_COL, "tensor memory budget");
+    static_assert(NUNIT >= 2 * CW && NUNIT / CW <= NAF && 2 * (NUNIT / CW) <= NB && NB % NACC == 0 && NACC <= MAX_NACC && NACC % NISS == 0, "barrier rings");
     // warps: 0 (and 1) issuers, 2 and 3 loaders, then the producer groups, then the epilogue groups (groups start at
     // multiples of four: warp % 4 is the tensor-memory lane quadrant of a warp)
     static constexpr int FIRST_LOADER_WARP = 2;
@@ -123,7 +113,7 @@ template <int CW, int BN>
 int c3_smem_bytes(const C3Geom &g)
 {
     using C = C3Cfg<CW, BN>;
-    return 1024 + (C::KT + 1) * C::W_TILE_BYTES + NGRP * RD * g.stage_bytes + 128;
+    return 1024 + (C::KT + 1) * C::W_TILE_BYTES + (BN * 4 + 127) / 128 * 128 + NGRP * RD * g.stage_bytes + 128;
 }
 
 template <int CW, int BN>
@@ -131,7 +121,7 @@ __global__ void __launch_bounds__(C3Cfg<CW, BN>::THREADS, 1)
 conv_tc_c3_kernel(const ConvProblem p, const C3Geom g, const __grid_constant__ CUtensorMap xmap)
 {
     using C = C3Cfg<CW, BN>;
-    constexpr int KW = C::KW, KT = C::KT, NACC = C::NACC, NUNIT = C::NUNIT, NH = C::NH, AW = C::AW;
+    constexpr int KT = C::KT, NACC = C::NACC, NUNIT = C::NUNIT, NH = C::NH, AW = C::AW;
     constexpr int NBARS = 2 * NGRP * RD + NAF + NB + MAX_NACC;
 
     extern __shared__ unsigned char smem_raw[];
@@ -149,8 +139,9 @@ conv_tc_c3_kernel(const ConvProblem p, const C3Geom g, const __grid_constant__ C
     const int cn = min(BN, p.C_out);
 
     const uint32_t wexp = (smem_u32(smem_raw) + 1023u) & ~1023u;          // [KT][BN rows][128 B] expanded weights
-    const uint32_t cexp = wexp + KT * C::W_TILE_BYTES;                    // [BN rows][128 B] constant bytes (first 32 of a row)
-    const uint32_t ring = cexp + C::W_TILE_BYTES;                         // [NGRP][RD] halo tiles
+    const uint32_t cexp = wexp + KT * C::W_TILE_BYTES;                    // [BN rows][128 B] constant rows (first 32 bytes)
+    const uint32_t pops = cexp + C::W_TILE_BYTES;                         // [BN] bit counts
+    const uint32_t ring = pops + (BN * 4 + 127) / 128 * 128;              // [NGRP][RD] halo tiles
     const uint32_t bar0 = smem_u32(bars);
     auto load_full = [&](int gr, int s) { return bar0 + 8u * (gr * RD + s); };
     auto load_empty = [&](int gr, int s) { return bar0 + 8u * (NGRP * RD + gr * RD + s); };
@@ -174,82 +165,72 @@ conv_tc_c3_kernel(const ConvProblem p, const C3Geom g, const __grid_constant__ C
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base_smem)), "r"(512u) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
+    for (int c = tid; c < BN; c += C::THREADS) asm volatile("st.shared.b32 [%0], %1;" ::"r"(pops + 4u * c), "r"(0) : "memory");
     pdl_wait();
-    // ---- one-off: expanded weights and the constant bytes.  K position e of the MMAs = channel word e / 9, tap e % 9
-    // (global weight word tap * CW + channel word) -> stage e / 4, 32-byte piece e % 4; MMA row `row` carries channel ch
-    for (int idx = tid; idx < (KT + 1) * BN; idx += C::THREADS) {
-        const int kt = idx / BN, row = idx - kt * BN;
-        const int ch = C::PACK16 ? (row & ~31) + channel_of_column(row & 31) : row;
-        const bool have = ch < cn;
-        const int xr = row & 7;
-        if (kt < KT) {
-            const uint32_t row_addr = wexp + (uint32_t)kt * C::W_TILE_BYTES + (uint32_t)row * ROWB;
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                const int kpos = kt * 4 + e;
-                const bool live = kpos < KW && have;
-                const uint32_t w = live ? __ldg(p.w + (long)ch * KW + (kpos % TAPS) * CW + kpos / TAPS) : 0u;
-                expand_store_w_signed(w, live, row_addr, xr, 2 * e);
-            }
-        } else {
-            // cst = 32 * c, c = K - 2 popc(G) - thr (thr clamped to +-(K + 1)); the constant activation tile's bytes are
-            // all 32, so the row's 32 signed bytes add up to c: c / 32 everywhere, one more unit of c's sign in |c % 32|
-            int pop = 0;
-            if (have)
-                for (int e = 0; e < KW; ++e) pop += __popc(__ldg(p.w + (long)ch * KW + e));
-            int t = have ? __ldg(p.thr + ch) : 0;
-            t = max(min(t, p.K + 1), -p.K - 1);
-            const int c = have ? p.K - 2 * pop - t : 0;
-            const int base = c / 32, rem = c - 32 * base, unit = rem < 0 ? -1 : 1, nrem = rem < 0 ? -rem : rem;
-            uint32_t cw[8];
-#pragma unroll
-            for (int q = 0; q < 8; ++q) {
-                uint32_t word = 0;
-#pragma unroll
-                for (int b = 0; b < 4; ++b) word |= (uint32_t)((base + ((4 * q + b) < nrem ? unit : 0)) & 0xFF) << (8 * b);
-                cw[q] = word;
-            }
-            const uint32_t crow = cexp + (uint32_t)row * ROWB;
-            st_shared_v4(crow + (uint32_t)((0 ^ xr) << 4), cw[0], cw[1], cw[2], cw[3]);
-            st_shared_v4(crow + (uint32_t)((1 ^ xr) << 4), cw[4], cw[5], cw[6], cw[7]);
-        }
+    __syncthreads();
+    // ---- one-off: expanded weights and the channels' bit counts.  K position e of the MMAs = channel word e / 10, tap e % 10
+    // (global weight word tap * CW + channel word) -> stage e / 8, 16-byte piece e % 8; MMA row `row` carries channel ch
+    for (int idx = tid; idx < KT * 8 * BN; idx += C::THREADS) {
+        const int e = idx % (KT * 8), row = idx / (KT * 8), tap = e % UWORDS, cword = e / UWORDS;
+        const int ch = (row & ~31) + channel_of_column(row & 31);
+        const bool live = tap < TAPS && cword < CW && ch < cn;
+        const uint32_t w = live ? __ldg(p.w + (long)ch * C::KW + tap * CW + cword) : 0u;
+        expand_store_w4(w, live, wexp + (uint32_t)(e >> 3) * C::W_TILE_BYTES + (uint32_t)row * ROWB, row & 7, e & 7);
+        if (live) asm volatile("red.shared.add.u32 [%0], %1;" ::"r"(pops + 4u * row), "r"(__popc(w)) : "memory");
     }
-    fence_async_proxy();
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
     pdl_trigger();
     const uint32_t tmem_base = tmem_base_smem;
-    // the constant activation tile: every byte 32
-    if (warp >= C::FIRST_PRODUCER_WARP && warp < C::FIRST_PRODUCER_WARP + 4) {
-        const uint32_t c8[8] = {0x20202020u, 0x20202020u, 0x20202020u, 0x20202020u, 0x20202020u, 0x20202020u, 0x20202020u, 0x20202020u};
-        tc_st8_nowait(tmem_base + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)C::C_COL, c8);
-        tc_wait_st();
+    // constants K - 2 popc - thr (thr clamped to +-(K + 1))
+    for (int row = tid; row < BN; row += C::THREADS) {
+        const int ch = (row & ~31) + channel_of_column(row & 31);
+        int pop;
+        asm volatile("ld.shared.b32 %0, [%1];" : "=r"(pop) : "r"(pops + 4u * row) : "memory");
+        const int t = ch < cn ? __ldg(p.thr + ch) : 0;
+        store_const_row(p.K - 2 * pop - max(min(t, p.K + 1), -p.K - 1), cexp + (uint32_t)row * ROWB, row & 7);
     }
+    if (warp >= C::FIRST_PRODUCER_WARP && warp < C::FIRST_PRODUCER_WARP + 4) write_const_block(tmem_base + ((uint32_t)((warp & 3) * 32) << 16));
+    fence_async_proxy();
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
 
-    // tile index -> image and the tile's first output pixel
-    auto tile_origin = [&](int tile, int &b, int &oh0, int &ow0) {
-        const unsigned per_img = (unsigned)(g.tiles_x * g.tiles_y);
-        b = (int)((unsigned)tile / per_img);
-        const unsigned rem = (unsigned)tile - (unsigned)b * per_img;
-        const unsigned ty = rem / (unsigned)g.tiles_x;
-        oh0 = (int)ty * TH;
-        ow0 = (int)(rem - ty * (unsigned)g.tiles_x) * TW;
+    // A role's tiles are a fixed number of tiles apart: image and tile coordinates follow by carries (two divisions per tile
+    // were a third of an epilogue warp's time).
+    struct TileCursor {
+        int b, ty, tx, db, dty, dtx;
     };
-    auto tile_of = [&](int n) { return (int)blockIdx.x + n * (int)gridDim.x; };
+    auto cursor = [&](int n0, int nstep) {
+        const unsigned per_img = (unsigned)(g.tiles_x * g.tiles_y), t = blockIdx.x + (unsigned)n0 * gridDim.x, st = (unsigned)nstep * gridDim.x;
+        TileCursor c;
+        c.b = (int)(t / per_img);
+        const unsigned rem = t - (unsigned)c.b * per_img;
+        c.ty = (int)(rem / (unsigned)g.tiles_x);
+        c.tx = (int)(rem - (unsigned)c.ty * (unsigned)g.tiles_x);
+        c.db = (int)(st / per_img);
+        const unsigned srem = st - (unsigned)c.db * per_img;
+        c.dty = (int)(srem / (unsigned)g.tiles_x);
+        c.dtx = (int)(srem - (unsigned)c.dty * (unsigned)g.tiles_x);
+        return c;
+    };
+    auto advance = [&](TileCursor &c) {
+        c.tx += c.dtx;
+        if (c.tx >= g.tiles_x) { c.tx -= g.tiles_x; ++c.ty; }
+        c.ty += c.dty;
+        if (c.ty >= g.tiles_y) { c.ty -= g.tiles_y; ++c.b; }
+        c.b += c.db;
+    };
 
     if (warp < C::NISS) {
         // ------------------------------------------------------------------ MMA issuer of tiles n = warp (mod NISS), in order
-        constexpr uint32_t idesc = make_idesc(AW) | (1u << 10);                  // B operand: signed bytes
+        constexpr uint32_t idesc = make_idesc_f4(AW);
         constexpr uint32_t HALF_DESC = (uint32_t)(AW * ROWB) >> 4;               // weight rows of the second half
         const uint64_t desc0 = make_desc(wexp);
         const uint32_t desc_hi = (uint32_t)(desc0 >> 32), b_lo = (uint32_t)desc0;
-        const uint32_t c_lo = (uint32_t)make_desc(cexp);
         const uint32_t tmem_u = __shfl_sync(0xffffffffu, tmem_base, 0);
-        const uint32_t c_t = tmem_u + (uint32_t)C::C_COL;
+        const uint32_t sf = tmem_u + (uint32_t)CB_COL, c_lo = (uint32_t)make_desc(cexp);
         bool ok = true;
         for (int n = warp; n < my_tiles && ok; n += C::NISS) {
             if (!pw_wait(a_full(n % NAF), (uint32_t)(n / NAF) & 1u, abort_flag, p.err, ERR_C3_ISSUER_TIMEOUT)) break;
@@ -265,15 +246,15 @@ conv_tc_c3_kernel(const ConvProblem p, const C3Geom g, const __grid_constant__ C
                 tc_fence_after();
                 if (elect_one()) {
                     const uint32_t d_t = tmem_u + (uint32_t)(acc * AW);
-                    tc_mma_i8_ts(d_t, c_t, c_lo + hf * HALF_DESC, desc_hi, idesc, 0u);   // accumulator = the per-channel constants
+                    tc_mma_const(d_t, tmem_u, c_lo + hf * HALF_DESC, desc_hi, idesc);
 #pragma unroll
                     for (int h = 0; h < CW; ++h) {
                         const uint32_t a_t = tmem_u + (uint32_t)(C::A_COL0 + ((n * CW + h) % NUNIT) * U_COLS);
 #pragma unroll
-                        for (int t = 0; t < TAPS; ++t) {
-                            const int e = h * TAPS + t;
-                            tc_mma_i8_ts(d_t, a_t + 8u * t, b_lo + hf * HALF_DESC + (uint32_t)((e >> 2) * (C::W_TILE_BYTES >> 4) + 2 * (e & 3)),
-                                         desc_hi, idesc, 1u);
+                        for (int t = 0; t < UWORDS / 2; ++t) {
+                            const int e = h * UWORDS + 2 * t;
+                            tc_mma_f4_ts(d_t, a_t + 8u * t, b_lo + hf * HALF_DESC + (uint32_t)((e >> 3) * (C::W_TILE_BYTES >> 4) + (e & 7)),
+                                         desc_hi, idesc, sf, 1u);
                         }
                     }
                     tc_commit(tile_done((n * NH + hf) % NB));
@@ -289,17 +270,16 @@ conv_tc_c3_kernel(const ConvProblem p, const C3Geom g, const __grid_constant__ C
         int stage = 0;
         uint32_t phase = 1;                       // first pass through the ring: the stages are free
         int issued = 0;
-        for (int n = grp; n < my_tiles; n += NGRP) {
+        TileCursor tc = cursor(grp, NGRP);
+        for (int n = grp; n < my_tiles; n += NGRP, advance(tc)) {
             if (!pw_wait<256>(load_empty(grp, stage), phase, abort_flag, p.err, ERR_C3_LOADER_TIMEOUT)) break;
             if (lane == 0) {
                 const uint32_t dst = ring + (uint32_t)(grp * RD + stage) * (uint32_t)g.stage_bytes;
-                int b, oh0, ow0;
-                tile_origin(tile_of(n), b, oh0, ow0);
-                const int x = (ow0 * g.stride - p.pad - g.xoff) * CW;        // words; a multiple of 4 by construction
-                const int y = oh0 * g.stride - p.pad;
+                const int x = (tc.tx * TW * g.stride - p.pad - g.xoff) * CW;     // words; a multiple of 4 by construction
+                const int y = tc.ty * TH * g.stride - p.pad;
                 asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(load_full(grp, stage)), "r"((uint32_t)(g.hb * g.wbw * 4)) : "memory");
                 asm volatile("cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];"
-                             ::"r"(dst), "l"(reinterpret_cast<uint64_t>(&xmap)), "r"(x), "r"(y), "r"(b), "r"(load_full(grp, stage)) : "memory");
+                             ::"r"(dst), "l"(reinterpret_cast<uint64_t>(&xmap)), "r"(x), "r"(y), "r"(tc.b), "r"(load_full(grp, stage)) : "memory");
             }
             __syncwarp();
             ++issued;
@@ -319,63 +299,37 @@ conv_tc_c3_kernel(const ConvProblem p, const C3Geom g, const __grid_constant__ C
         const uint32_t t_lane = tmem_base + ((uint32_t)(quad * 32) << 16);
         const int owords = p.C_out >> 5;
         // NH == 1: the group takes alternate tiles; NH == 2: the group takes its half (64 channels) of every tile
-        for (int n = NH == 2 ? 0 : grp; n < my_tiles; n += NH == 2 ? 1 : NGRP) {
+        TileCursor tc = cursor(NH == 2 ? 0 : grp, NH == 2 ? 1 : NGRP);
+        for (int n = NH == 2 ? 0 : grp; n < my_tiles; n += NH == 2 ? 1 : NGRP, advance(tc)) {
             const int acc = NH == 2 ? grp : n % NACC;
             const int d = NH == 2 ? 2 * n + grp : n;                              // the tile's (half's) "done" number
             const int ch0 = NH == 2 ? 2 * grp : 0;                                // first output word of this accumulator
             if (!pw_wait<C::NISS == 1 ? 64 : 128>(tile_done(d % NB), (uint32_t)(d / NB) & 1u, abort_flag, p.err, ERR_C3_EPILOGUE_TIMEOUT)) break;
             tc_fence_after();
             uint32_t words[AW / 32];
-            if constexpr (C::PACK16) {
-                constexpr int NR = AW == 32 ? 16 : 32;                       // registers per load
-                constexpr int NL = AW == 32 ? 1 : AW / 64;                   // loads
-                uint32_t rr[NL][NR];
-                if constexpr (AW == 32) {
-                    tc_ld32_pack16(t_lane + (uint32_t)(acc * AW), rr[0]);
-                } else {
-#pragma unroll
-                    for (int h = 0; h < NL; ++h) tc_ld64_pack16(t_lane + (uint32_t)(acc * AW + h * 64), rr[h]);
-                }
+            if constexpr (AW == 32) {
+                uint32_t v[16];
+                tc_ld32_pack16(t_lane + (uint32_t)(acc * AW), v);
                 tc_wait_ld();
-#pragma unroll
-                for (int h = 0; h < NL; ++h) pin_regs(rr[h]);
+                pin_regs(v);
                 tc_fence_before();
                 __syncwarp();
                 if (lane == 0) mbar_arrive(acc_free(acc));
-                if constexpr (AW == 32) {
-                    words[0] = sign_word(rr[0]);
-                } else {
-#pragma unroll
-                    for (int h = 0; h < NL; ++h) {
-                        words[2 * h] = sign_word(rr[h]);
-                        words[2 * h + 1] = sign_word(rr[h] + 16);
-                    }
-                }
+                words[0] = sign_word(v);
             } else {
-#pragma unroll
-                for (int ch = 0; ch < AW / 32; ++ch) {
-                    uint32_t v[32];
-                    tc_ld32(t_lane + (uint32_t)(acc * AW + ch * 32), v);
-                    if (ch == AW / 32 - 1) {                              // the accumulator's last columns are in registers
-                        tc_fence_before();
-                        __syncwarp();
-                        if (lane == 0) mbar_arrive(acc_free(acc));
-                    }
-                    // bit i = (v[i] >= 0): sign bits shifted in, last column first; two chains of 16
-                    uint32_t hi = 0, lo = 0;
-#pragma unroll
-                    for (int i = 15; i >= 0; --i) {
-                        hi = __funnelshift_l(v[16 + i], hi, 1);
-                        lo = __funnelshift_l(v[i], lo, 1);
-                    }
-                    words[ch] = ~__byte_perm(lo, hi, 0x5410);
-                }
+                uint32_t v[32];
+                tc_ld64_pack16(t_lane + (uint32_t)(acc * AW), v);
+                tc_wait_ld();
+                pin_regs(v);
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(acc_free(acc));
+                words[0] = sign_word(v);
+                words[1] = sign_word(v + 16);
             }
-            int b, oh0, ow0;
-            tile_origin(tile_of(n), b, oh0, ow0);
-            const int oh = oh0 + (r >> 4), ow = ow0 + (r & 15);
+            const int oh = tc.ty * TH + (r >> 4), ow = tc.tx * TW + (r & 15);
             if (oh < p.OH && ow < p.OW) {
-                uint32_t *dst = static_cast<uint32_t *>(p.out) + (((long)b * p.OH + oh) * p.OW + ow) * owords + ch0;
+                uint32_t *dst = static_cast<uint32_t *>(p.out) + (long)(((unsigned)tc.b * p.OH + oh) * p.OW + ow) * owords + ch0;
                 if (AW == 64 && (owords & 1) == 0) {                  // (an even word count keeps the pair 8-byte aligned)
                     *reinterpret_cast<uint2 *>(dst) = make_uint2(words[0], words[1 % (AW / 32)]);
                 } else {
@@ -409,10 +363,11 @@ conv_tc_c3_kernel(const ConvProblem p, const C3Geom g, const __grid_constant__ C
                 asm volatile("ld.shared.b32 %0, [%1];" : "=r"(wds[tap]) : "r"(src + (uint32_t)(tap / 3) * row_pitch + (uint32_t)((tap % 3) * CW * 4)) : "memory");
             __syncwarp();
             mbar_arrive_pred(load_empty(lg, stage), lane0);        // the stage may be refilled
-            // the first four words are expanded before the wait for the unit
-            uint32_t v[32];
+            // expanded before the wait for the unit (the unit's tenth word is not written: its weights are zero)
+            uint32_t v[32], v4[4];
 #pragma unroll
-            for (int e = 0; e < 4; ++e) expand_a(wds[e], &v[8 * e]);
+            for (int e = 0; e < 8; ++e) expand_a4(wds[e], &v[4 * e]);
+            expand_a4(wds[8], v4);
             // the MMAs of the tile that used this ring position last have read it (nothing to wait for the first time round)
             const int u = n * CW + h;
             if (u >= NUNIT) {
@@ -422,15 +377,7 @@ conv_tc_c3_kernel(const ConvProblem p, const C3Geom g, const __grid_constant__ C
             tc_fence_after();
             const uint32_t taddr = t_lane + (uint32_t)((u % NUNIT) * U_COLS);
             tc_st32_nowait(taddr, v);
-            {
-                uint32_t v4[32];
-#pragma unroll
-                for (int e = 0; e < 4; ++e) expand_a(wds[4 + e], &v4[8 * e]);
-                tc_st32_nowait(taddr + 32u, v4);
-                uint32_t v8[8];
-                expand_a(wds[8], v8);
-                tc_st8_nowait(taddr + 64u, v8);
-            }
+            tc_st4_nowait(taddr + 32u, v4);
             tc_wait_st();
             tc_fence_before();
             __syncwarp();
