@@ -3,10 +3,8 @@
 // memory, not by the tensor pipe: the binary 1x1 convolution is the only binary operator of the paper's own network
 // (Section 4.2.1; Table 1), at resolutions up to 224 x 224.
 //
-// Arithmetic as in the weight-stationary engine (conv_tc_ws.cu): sign bits expanded to bytes on chip, unsigned
-// activation bytes {0, 2^j} against signed weight bytes +-2^(6-j), int32 accumulators in tensor memory, and with
-// S = sum over set activation bits of the weight signs:  sum a*g = 2 S + K - 2 popc(G),  accumulator = 64 S + cst,
-// cst = 32 (K - 2 popc(G) - threshold), output bit = (accumulator >= 0).
+// Arithmetic: 4-bit operands (tc_common.cuh), fp32 accumulators that hold exact integers, the per-channel constants
+// K - 2 popc(G) - threshold written by a first MMA so that the epilogue needs 16 bits and a sign (tc_slot.cuh).
 //
 // What differs is everything around the MMAs; a row of the patch matrix is simply KW consecutive words of x.
 //   * Work is cut into CHUNKS of T tiles (T * 128 rows) and BLOCKS of G consecutive chunks; a CTA takes whole
@@ -23,15 +21,12 @@
 //     do its own mbarrier waits.  (An issuer that waits right behind its own MMAs stalls until they drain: with one
 //     issuer for all slots that was about 700 cycles per chunk and the whole kernel's bound; two buffers per slot
 //     fed by one issuer stall the same way on the second commit.)
-//   * The per-channel constant is the accumulator's starting value, and an MMA writes it: the first MMA of a tile
-//     (not accumulating) multiplies a constant activation tile (every byte 32, written once) with 32 signed bytes
-//     per channel that add up to cst / 32.  Nobody ever stores constants into tensor memory, so the epilogue only
-//     reads.
-//   * The epilogue loads accumulators as packed 16-bit halves (tcgen05.ld .pack::16b: |accumulator| < 2^15 for
-//     K <= 128), two columns per register, and gathers sign bits with byte permutes in sign-replication mode: one
-//     PRMT + one LOP3 per four columns instead of one shift per column.  Bit s of byte B of an output word then
-//     comes from accumulator column 2s (B = 0), 2s + 1 (B = 1), 16 + 2s (B = 2), 17 + 2s (B = 3) of its 32-column
-//     block; the weight rows are laid out in that order (channel_of_column), which costs nothing.
+//   * The per-channel constant is the accumulator's starting value and an MMA writes it: nobody ever stores constants into
+//     tensor memory, so the epilogue only reads.
+//   * The epilogue loads accumulators as packed 16-bit halves, two columns per register, and gathers sign bits with byte
+//     permutes in sign-replication mode: one PRMT + one LOP3 per four columns instead of one shift per column.  Bit s of
+//     byte B of an output word then comes from accumulator column 2s (B = 0), 2s + 1 (B = 1), 16 + 2s (B = 2), 17 + 2s
+//     (B = 3) of its 32-column block; the weight rows are laid out in that order (channel_of_column), which costs nothing.
 // Parity waits on an mbarrier are only right while the waiter starts waiting for completion k after completion k - 1
 // and before completion k + 1; binding every role of a slot to that slot, and giving every slot the same number of
 // chunks in every block (G is a multiple of NSLOT), gives every waiter each completion of its barriers in turn.
@@ -55,11 +50,11 @@ constexpr int ERR_PW_ACC_TIMEOUT = 126;          // issuer: the slot's accumulat
 constexpr int MAX_BLOCKS = 16;            // stages of the shared-memory ring (one block each)
 constexpr int RING_BYTES = 96 * 1024;
 constexpr int BLOCK_BYTES_TARGET = 12 * 1024;
-constexpr int CONST_COLS = 8;             // the constant activation tile: 32 bytes per row
 
 // tiles (accumulator + expanded activations) that fit in tensor memory beside the constant tile, cut into three slots
 // where that leaves whole tiles (3, 6..12 tiles), else two (4, 5 tiles)
-__host__ __device__ constexpr int pw_tiles(int kw, int bn) { return (512 - CONST_COLS) / (bn + 8 * kw); }
+__host__ __device__ constexpr int pw_words(int kw) { return (kw + 1) & ~1; }      // two K words per MMA
+__host__ __device__ constexpr int pw_tiles(int kw, int bn) { return CB_COL / (bn + 4 * pw_words(kw)); }
 __host__ __device__ constexpr int pw_nslot(int kw, int bn) { return (pw_tiles(kw, bn) >= 6 || pw_tiles(kw, bn) == 3) ? 3 : 2; }
 __host__ __device__ constexpr int pw_t(int kw, int bn)
 {
@@ -72,9 +67,8 @@ template <int KW, int BN> struct PwCfg {
     static constexpr int NSLOT = pw_nslot(KW, BN);
     static constexpr int TILES = NSLOT * T;
     static constexpr int A_COL0 = TILES * BN;               // accumulators first, then the expanded activation tiles
-    static constexpr int A_COLS = 8 * KW;
-    static constexpr int C_COL = A_COL0 + TILES * A_COLS;   // the constant activation tile
-    static_assert(C_COL + CONST_COLS <= 512, "tensor memory budget");
+    static constexpr int A_COLS = 4 * pw_words(KW);
+    static_assert(A_COL0 + TILES * A_COLS <= CB_COL, "tensor memory budget");
     static_assert(T >= 1 && T <= 4 && NSLOT >= 2 && NSLOT <= 3, "slot shape");
     static constexpr int CHUNK_ROWS = T * BM;
     static constexpr int CHUNK_BYTES = CHUNK_ROWS * KW * 4;
@@ -92,7 +86,7 @@ template <int KW, int BN> struct PwCfg {
     static constexpr int FIRST_EPILOGUE_WARP = 4 + 4 * NSLOT;
     static constexpr int WARPS = 4 + 8 * NSLOT;
     static constexpr int THREADS = 32 * WARPS;
-    static constexpr int W_BYTES = BN * ROWB;               // expanded weights: [BN rows][128 B], 32 * KW bytes used per row
+    static constexpr int W_BYTES = BN * ROWB;               // expanded weights: [BN rows][128 B], 16 bytes per K word used
     static constexpr int SMEM = 1024 + 2 * W_BYTES + NBLK * BLOCK_BYTES + 64;
     static constexpr int SMEM_ASK = SMEM < 120 * 1024 ? 120 * 1024 : SMEM;     // one CTA per SM (it takes all of tensor memory)
 };
@@ -125,7 +119,7 @@ conv_tc_pw_kernel(const ConvProblem p)
     const int cn = min(BN, p.C_out);
 
     const uint32_t wexp = (smem_u32(smem_raw) + 1023u) & ~1023u;          // [BN rows][128 B] expanded weights
-    const uint32_t cexp = wexp + C::W_BYTES;                              // [BN rows][128 B] constant bytes (first 32 of a row)
+    const uint32_t cexp = wexp + C::W_BYTES;                              // [BN rows][128 B] constant rows (first 32 bytes)
     const uint32_t ring = cexp + C::W_BYTES;                              // [NBLK][BLOCK_ROWS][KW words]
     const uint32_t bar0 = smem_u32(bars);
     auto load_full = [&](int s) { return bar0 + 8u * s; };
@@ -153,38 +147,22 @@ conv_tc_pw_kernel(const ConvProblem p)
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
     pdl_wait();
-    // ---- one-off: expanded weights and constant bytes; MMA row `row` carries channel 32 * (row / 32) + channel_of_column(row % 32)
+    // ---- one-off: expanded weights and constant rows; MMA row `row` carries channel 32 * (row / 32) + channel_of_column(row % 32)
     for (int row = tid; row < BN; row += C::THREADS) {
         const int ch = (row & ~31) + channel_of_column(row & 31);
         const bool have = ch < cn;
         const uint32_t row_addr = wexp + (uint32_t)row * ROWB;
         int pop = 0;
 #pragma unroll
-        for (int e = 0; e < 4; ++e) {
+        for (int e = 0; e < pw_words(KW); ++e) {
             const bool live = e < KW && have;
             const uint32_t w = live ? __ldg(p.w + (long)ch * KW + e) : 0u;
             pop += __popc(w);
-            expand_store_w_signed(w, live, row_addr, row & 7, 2 * e);
+            expand_store_w4(w, live, row_addr, row & 7, e);
         }
-        // cst = 32 * c, c = K - 2 popc(G) - thr with thr clamped to +-(K + 1) (beyond that bound the decision is
-        // constant); the constant tile's bytes are all 32, so the row's 32 signed bytes must add up to c:
-        // c / 32 everywhere and one more unit of c's sign in the first |c % 32| of them
-        int t = have ? __ldg(p.thr + ch) : 0;
-        t = max(min(t, p.K + 1), -p.K - 1);
-        const int c = have ? p.K - 2 * pop - t : 0;
-        const int base = c / 32, rem = c - 32 * base, unit = rem < 0 ? -1 : 1, nrem = rem < 0 ? -rem : rem;
-        uint32_t cw[8];
-#pragma unroll
-        for (int q = 0; q < 8; ++q) {
-            uint32_t word = 0;
-#pragma unroll
-            for (int b = 0; b < 4; ++b) word |= (uint32_t)((base + ((4 * q + b) < nrem ? unit : 0)) & 0xFF) << (8 * b);
-            cw[q] = word;
-        }
-        const uint32_t crow = cexp + (uint32_t)row * ROWB;
-        const int xr = row & 7;
-        st_shared_v4(crow + (uint32_t)((0 ^ xr) << 4), cw[0], cw[1], cw[2], cw[3]);
-        st_shared_v4(crow + (uint32_t)((1 ^ xr) << 4), cw[4], cw[5], cw[6], cw[7]);
+        // thr clamped to +-(K + 1): beyond that bound the decision is constant
+        const int t = have ? __ldg(p.thr + ch) : 0;
+        store_const_row(have ? p.K - 2 * pop - max(min(t, p.K + 1), -p.K - 1) : 0, cexp + (uint32_t)row * ROWB, row & 7);
     }
     fence_async_proxy();
     tc_fence_before();
@@ -192,12 +170,7 @@ conv_tc_pw_kernel(const ConvProblem p)
     tc_fence_after();
     pdl_trigger();
     const uint32_t tmem_base = tmem_base_smem;
-    // the constant activation tile: every byte 32 (one producer group writes its four lane quadrants)
-    if (warp >= C::FIRST_PRODUCER_WARP && warp < C::FIRST_PRODUCER_WARP + 4) {
-        const uint32_t c8[8] = {0x20202020u, 0x20202020u, 0x20202020u, 0x20202020u, 0x20202020u, 0x20202020u, 0x20202020u, 0x20202020u};
-        tc_st8_nowait(tmem_base + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)C::C_COL, c8);
-        tc_wait_st();
-    }
+    if (warp >= C::FIRST_PRODUCER_WARP && warp < C::FIRST_PRODUCER_WARP + 4) write_const_block(tmem_base + ((uint32_t)((warp & 3) * 32) << 16));
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -205,12 +178,12 @@ conv_tc_pw_kernel(const ConvProblem p)
     if (warp < NSLOT) {
         // ------------------------------------------------------------------ MMA issuer of slot `warp`
         const int slot = warp;
-        constexpr uint32_t idesc = make_idesc(BN) | (1u << 10);                  // B operand: signed bytes
+        constexpr uint32_t idesc = make_idesc_f4(BN);
         const uint64_t desc0 = make_desc(wexp);
         const uint32_t desc_hi = (uint32_t)(desc0 >> 32), b_lo = (uint32_t)desc0;
         const uint32_t c_lo = (uint32_t)make_desc(cexp);
         const uint32_t tmem_u = __shfl_sync(0xffffffffu, tmem_base, 0);
-        const uint32_t c_t = tmem_u + (uint32_t)C::C_COL;
+        const uint32_t sf = tmem_u + (uint32_t)CB_COL;
         uint32_t phase = 0;
         for (int j = slot; j < my_chunks; j += NSLOT) {
             // the epilogue has read the slot's previous accumulators (nothing to wait for the first time round)
@@ -222,10 +195,10 @@ conv_tc_pw_kernel(const ConvProblem p)
                 for (int t = 0; t < T; ++t) {
                     const uint32_t d_t = tmem_u + (uint32_t)((slot * T + t) * BN);
                     const uint32_t a_t = tmem_u + (uint32_t)(C::A_COL0 + (slot * T + t) * C::A_COLS);
-                    tc_mma_i8_ts(d_t, c_t, c_lo, desc_hi, idesc, 0u);            // accumulator = the per-channel constants
+                    tc_mma_const(d_t, tmem_u, c_lo, desc_hi, idesc);             // accumulator = the per-channel constants
 #pragma unroll
-                    for (int e = 0; e < KW; ++e)
-                        tc_mma_i8_ts(d_t, a_t + 8u * e, b_lo + 2u * e, desc_hi, idesc, 1u);
+                    for (int e = 0; e < pw_words(KW) / 2; ++e)
+                        tc_mma_f4_ts(d_t, a_t + 8u * e, b_lo + 2u * e, desc_hi, idesc, sf, 1u);
                 }
                 tc_commit(mma_done(slot));
             }
@@ -359,26 +332,21 @@ conv_tc_pw_kernel(const ConvProblem p)
             __syncwarp();
             mbar_arrive_pred(load_empty(stage), lane0);           // (the stage may be refilled once all its chunks have been read)
             // expanded rows in registers first; only the stores wait for the slot
-            uint32_t v[T][8 * KW];
+            uint32_t v[T][4 * KW];
 #pragma unroll
             for (int t = 0; t < T; ++t)
 #pragma unroll
-                for (int e = 0; e < KW; ++e) expand_a(wds[t][e], &v[t][8 * e]);
+                for (int e = 0; e < KW; ++e) expand_a4(wds[t][e], &v[t][4 * e]);
             // the MMAs of the slot's previous chunk have read its activation columns
             if (j >= NSLOT && !pw_wait(mma_done(slot), phase ^ 1u, abort_flag, p.err, ERR_PW_SLOT_TIMEOUT)) break;
             tc_fence_after();
 #pragma unroll
             for (int t = 0; t < T; ++t) {
                 const uint32_t taddr = t_lane + (uint32_t)(t * C::A_COLS);
-                if constexpr (KW == 4) {
-                    tc_st32_nowait(taddr, v[t]);
-                } else {
-#pragma unroll
-                    for (int e = 0; e < KW; ++e) {
-                        const uint32_t (&v8)[8] = *reinterpret_cast<const uint32_t (*)[8]>(&v[t][8 * e]);
-                        tc_st8_nowait(taddr + 8u * e, v8);
-                    }
-                }
+                // (the second word of an odd K's last pair is not written: its weights are zero)
+                if constexpr (KW == 4) tc_st16_nowait(taddr, v[t]);
+                if constexpr (KW == 2 || KW == 3) tc_st8_nowait(taddr, reinterpret_cast<const uint32_t (&)[8]>(v[t][0]));
+                if constexpr (KW == 1 || KW == 3) tc_st4_nowait(taddr + (KW - 1) * 4u, reinterpret_cast<const uint32_t (&)[4]>(v[t][4 * (KW - 1)]));
             }
             tc_wait_st();
             tc_fence_before();
