@@ -263,12 +263,11 @@ conv_tc_i8_kernel(const ConvProblem p, const int ktab_words)
                         cp_async_wait<ID_AHEAD>();                    // this chunk's copy has landed
                         words[ch] = module_chunk(p, dot, id_warp + (uint32_t)cur_slot * (BM * ID_ROW_BYTES), (long)em - lane, n0 + col0, lane);
                         if (++cur_slot == ID_SLOTS) cur_slot = 0;
-                    } else if (BN == 128 && (p.C_out & 3) == 0 && (n0 + col0 + 32 <= p.C_out)) {
-                        // full chunk (warp-uniform): staged, the warp stores whole 128-byte rows
+                    } else if constexpr (BN == 128) {
                         int o[32];
                         biased_ints(v, table + 4u * col0, o);
                         const long row0 = (long)em - lane;
-                        store_int32_block(static_cast<int32_t *>(p.out) + row0 * p.C_out + n0 + col0, p.C_out, o, i32_tile, row0, p.M, lane);
+                        store_int32_block(static_cast<int32_t *>(p.out) + row0 * p.C_out + n0 + col0, p.C_out, o, i32_tile, row0, p.M, lane, p.C_out - n0 - col0);
                     } else if (em < p.M) {
                         int32_t *dst = static_cast<int32_t *>(p.out) + (long)em * p.C_out + n0 + col0;
                         const bool vec = (p.C_out & 3) == 0 && (n0 + col0 + 32 <= p.C_out);

@@ -27,8 +27,6 @@ namespace {
 
 using namespace tc;
 
-constexpr int EPI_WARPS = 4;
-constexpr int G = 2;                      // activation producer groups
 constexpr int PF = 3;                     // packed-word stages in flight per producer thread
 constexpr int MAX_SMEM = 227 * 1024 - 512;
 
@@ -37,42 +35,46 @@ constexpr int ERR_MMA_TIMEOUT = 132;
 constexpr int ERR_EPILOGUE_TIMEOUT = 133;
 constexpr int ERR_LOADER_TIMEOUT = 134;
 
-template <int BN> struct Cfg {
-    static constexpr int NBUF = BN == 256 ? 1 : 2;                       // accumulator buffers
+// BN: output channels of a tile; MODE: 0 int32, 1 packed output; G: activation producer groups of four warps; TEAMS: epilogue
+// teams of four warps, each with its share of a tile's columns
+template <int BN, int MODE, int G, int TEAMS> struct Cfg {
+    static constexpr int EPI_WARPS = 4 * TEAMS;
+    static constexpr int NBUF = BN == 256 ? 1 : (BN == 128 ? 2 : 4);     // accumulator buffers
     static constexpr int A_COL0 = NBUF * BN;                              // first column of the activation ring
-    static constexpr int STAGES = BN == 256 ? 5 : 7;
+    static constexpr int STAGES = BN == 256 ? (MODE == 0 ? 4 : 5) : 7;
     static constexpr int PROD_THREADS = G * BM;
     static constexpr int FIRST_PRODUCER_WARP = 1 + EPI_WARPS;
     static constexpr int LOADER_WARP = FIRST_PRODUCER_WARP + 4 * G;
     static constexpr int CONTROL_WARP = LOADER_WARP + 1;
     static constexpr int THREADS = 32 * (CONTROL_WARP + 1);
+    static constexpr int EC = BN / TEAMS;                                 // columns of a team
     static constexpr int W_BYTES = BN * ROWB;                             // one ring stage of weights
     static constexpr int SF_COL = 512 - (int)SF_COLS;                     // unit scales
     static constexpr int BITS_BYTES = PF * PROD_THREADS * 32;
-    static constexpr int TABLE_BYTES = EPI_WARPS * BN * 4;                // one column table per epilogue warp
+    static constexpr int TABLE_BYTES = EPI_WARPS * EC * 4;                // one column table per epilogue warp
     static_assert(A_COL0 + STAGES * 32 <= SF_COL, "tensor memory budget");
     static_assert(STAGES >= G, "a producer group must not lap the ring (parity waits)");
 };
 
-template <int BN>
+template <typename C>
 __host__ __device__ inline int smem_bytes(int ktab_words, int mode)
 {
-    using C = Cfg<BN>;
     return 1024 + C::STAGES * C::W_BYTES + C::BITS_BYTES + C::TABLE_BYTES + ktab_words * 4 + 16 +
-           (mode == 0 ? EPI_WARPS * I32_TILE_BYTES + 16 : 0);
+           (mode == 0 ? C::EPI_WARPS * I32_TILE_BYTES + 16 : 0);
 }
 
-template <int BN, int MODE>
-__global__ void __launch_bounds__(Cfg<BN>::THREADS, 1)
+template <int BN, int MODE, int G, int TEAMS>
+__global__ void __launch_bounds__(Cfg<BN, MODE, G, TEAMS>::THREADS, 1)
 conv_tc_pre_kernel(const ConvProblem p, const int32_t *cst, const __grid_constant__ CUtensorMap wmap, const int ktab_words)
 {
-    using C = Cfg<BN>;
+    using C = Cfg<BN, MODE, G, TEAMS>;
+    constexpr int EPI_WARPS = C::EPI_WARPS, EC = C::EC;
     constexpr bool FUSED = MODE == 1;
     constexpr int NBUF = C::NBUF;
     constexpr int STAGES = C::STAGES;
 
     extern __shared__ unsigned char smem_raw[];
-    __shared__ __align__(8) unsigned long long bars[2 * 8 + 2 * 2];
+    __shared__ __align__(8) unsigned long long bars[2 * 8 + 2 * 4];
     __shared__ uint32_t tmem_base_smem;
     __shared__ int abort_flag_smem;
 
@@ -87,14 +89,14 @@ conv_tc_pre_kernel(const ConvProblem p, const int32_t *cst, const __grid_constan
 
     const uint32_t wring = (smem_u32(smem_raw) + 1023u) & ~1023u;         // [STAGES][BN rows][128 B], written by TMA
     const uint32_t bits_ring = wring + STAGES * C::W_BYTES;               // [PF][2][PROD_THREADS][16 B]
-    const uint32_t tables = bits_ring + C::BITS_BYTES;                    // [EPI_WARPS][BN] int32 column constants
+    const uint32_t tables = bits_ring + C::BITS_BYTES;                    // [EPI_WARPS][EC] column constants
     const uint32_t ktab_addr = tables + C::TABLE_BYTES;                   // unit table of the gather
     const uint32_t i32_tiles = (ktab_addr + (uint32_t)ktab_words * 4u + 15u) & ~15u;   // int32 output: store staging tiles
     const uint32_t bar0 = smem_u32(bars);
     auto full_bar = [&](int s) { return bar0 + 8u * s; };
     auto empty_bar = [&](int s) { return bar0 + 8u * (8 + s); };
     auto tfull_bar = [&](int b) { return bar0 + 8u * (16 + b); };
-    auto tempty_bar = [&](int b) { return bar0 + 8u * (18 + b); };
+    auto tempty_bar = [&](int b) { return bar0 + 8u * (20 + b); };
     volatile int *abort_flag = &abort_flag_smem;
 
     if (tid == 0) {
@@ -102,7 +104,7 @@ conv_tc_pre_kernel(const ConvProblem p, const int32_t *cst, const __grid_constan
             mbar_init(full_bar(s), 4 + 1);           // the four activation warps of the stage's group + the loader's arrive (+ its bytes)
             mbar_init(empty_bar(s), 1);
         }
-        for (int b = 0; b < 2; ++b) {
+        for (int b = 0; b < 4; ++b) {
             mbar_init(tfull_bar(b), 1);
             mbar_init(tempty_bar(b), EPI_WARPS);
         }
@@ -115,11 +117,12 @@ conv_tc_pre_kernel(const ConvProblem p, const int32_t *cst, const __grid_constan
     }
     const int gwidth = gather_width(p.cw);
     build_unit_table8(p, ktab_addr, ktiles * (8 / gwidth), gwidth, tid, C::THREADS);
-    pdl_wait();
+    if (tid == 32 * C::LOADER_WARP) asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&wmap)) : "memory");
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
     pdl_trigger();
+    pdl_wait();
     const uint32_t tmem_base = tmem_base_smem;
 
     if (warp == 0) {
@@ -207,20 +210,20 @@ conv_tc_pre_kernel(const ConvProblem p, const int32_t *cst, const __grid_constan
     } else if (warp <= EPI_WARPS) {
         // ------------------------------------------------------------------ epilogue
         const int quad = warp & 3;                 // tensor-memory lane quadrant this warp may read
-        const int erow = quad * 32 + lane;
-        const uint32_t i32_tile = i32_tiles + (uint32_t)quad * I32_TILE_BYTES;
+        const int erow = quad * 32 + lane, team = (warp - 1) >> 2;
+        const uint32_t i32_tile = i32_tiles + (uint32_t)(warp - 1) * I32_TILE_BYTES;
         bool alive = true;
         int buf = 0;
         uint32_t buf_phase = 0;
         for (int ti = 0; ti < my_tiles; ++ti) {
             const int tile = (int)blockIdx.x + ti * (int)gridDim.x;
             const int n_tile = tile / m_tiles, m_tile = tile - n_tile * m_tiles;
-            const int m0 = m_tile * BM, n0 = n_tile * BN;
+            const int m0 = m_tile * BM, n0 = n_tile * BN + team * EC;       // this team's columns
             const int em = m0 + erow;
             // this tile's column constants, built while its MMAs run; every warp keeps its own table, so the four
             // warps need no barrier among themselves
-            const uint32_t table = tables + (uint32_t)(quad * BN * 4);
-            for (int c = lane; c < BN; c += 32) {
+            const uint32_t table = tables + (uint32_t)((warp - 1) * EC * 4);
+            for (int c = lane; c < EC; c += 32) {
                 const int n = n0 + c;
                 int v = 0;
                 if (n < p.C_out) {
@@ -234,10 +237,10 @@ conv_tc_pre_kernel(const ConvProblem p, const int32_t *cst, const __grid_constan
             alive = __all_sync(0xffffffffu, alive && !*abort_flag);
             if (!alive) break;
             tc_fence_after();
-            const uint32_t t_addr = tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)(buf * BN);
-            uint32_t words[BN / 32];
+            const uint32_t t_addr = tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)(buf * BN + team * EC);
+            uint32_t words[EC / 32];
 #pragma unroll
-            for (int ch = 0; ch < BN / 32; ++ch) {
+            for (int ch = 0; ch < EC / 32; ++ch) {
                 const int col0 = ch * 32;
                 words[ch] = 0;
                 if (n0 + col0 < p.C_out) {             // warp-uniform
@@ -248,16 +251,8 @@ conv_tc_pre_kernel(const ConvProblem p, const int32_t *cst, const __grid_constan
                     } else {
                         int o[32];
                         biased_ints(v, table + 4u * col0, o);
-                        if ((p.C_out & 3) == 0 && (n0 + col0 + 32 <= p.C_out)) {
-                            // full chunk (warp-uniform): staged, the warp stores whole 128-byte rows
-                            const long row0 = (long)em - lane;
-                            store_int32_block(static_cast<int32_t *>(p.out) + row0 * p.C_out + n0 + col0, p.C_out, o, i32_tile, row0, p.M, lane);
-                        } else if (em < p.M) {
-                            int32_t *dst = static_cast<int32_t *>(p.out) + (long)em * p.C_out + n0 + col0;
-#pragma unroll
-                            for (int i = 0; i < 32; ++i)
-                                if (n0 + col0 + i < p.C_out) dst[i] = o[i];
-                        }
+                        const long row0 = (long)em - lane;
+                        store_int32_block(static_cast<int32_t *>(p.out) + row0 * p.C_out + n0 + col0, p.C_out, o, i32_tile, row0, p.M, lane, p.C_out - n0 - col0);
                     }
                 }
             }
@@ -269,14 +264,17 @@ conv_tc_pre_kernel(const ConvProblem p, const int32_t *cst, const __grid_constan
             if (FUSED && em < p.M) {
                 const int owords = p.C_out >> 5;
                 uint32_t *dst = static_cast<uint32_t *>(p.out) + (long)em * owords + (n0 >> 5);
-                if ((owords & 3) == 0 && n0 + BN <= p.C_out) {
+                if (EC >= 128 && (owords & 3) == 0 && n0 + EC <= p.C_out) {
 #pragma unroll
-                    for (int c4 = 0; c4 < BN / 128; ++c4)
+                    for (int c4 = 0; c4 < EC / 128; ++c4)
                         *reinterpret_cast<uint4 *>(dst + 4 * c4) =
                             make_uint4(words[4 * c4], words[4 * c4 + 1], words[4 * c4 + 2], words[4 * c4 + 3]);
+                } else if (EC >= 64 && (owords & 1) == 0 && n0 + EC <= p.C_out) {
+#pragma unroll
+                    for (int c2 = 0; c2 < EC / 64; ++c2) *reinterpret_cast<uint2 *>(dst + 2 * c2) = make_uint2(words[2 * c2], words[2 * c2 + 1]);
                 } else {
 #pragma unroll
-                    for (int ch = 0; ch < BN / 32; ++ch)
+                    for (int ch = 0; ch < EC / 32; ++ch)
                         if (n0 + ch * 32 < p.C_out) dst[ch] = words[ch];
                 }
             }
@@ -391,9 +389,10 @@ prepare_weights_kernel(const uint32_t *w, uint8_t *wexp, int32_t *cst, int N, in
 
 int ktab_words_for(const ConvProblem &p) { return ((p.kwords + 7) >> 3) * (8 / gather_width(p.cw)); }
 
-template <int BN>
+template <int BN, int MODE, int G, int TEAMS>
 int launch_bn(const ConvProblem &p0, const PreparedWeights &pw, cudaStream_t stream)
 {
+    using C = Cfg<BN, MODE, G, TEAMS>;
     ConvProblem p = p0;
     p.err = device_error_word();
     const int sms = sm_count();
@@ -403,7 +402,7 @@ int launch_bn(const ConvProblem &p0, const PreparedWeights &pw, cudaStream_t str
     if (total >= (1L << 31)) return BCNN_ERR_UNSUPPORTED;
     const unsigned grid = (unsigned)(total < sms ? total : sms);
     const int ktw = ktab_words_for(p);
-    const int smem = smem_bytes<BN>(ktw, p.mode);
+    const int smem = smem_bytes<C>(ktw, MODE);
     if (smem > MAX_SMEM) return BCNN_ERR_UNSUPPORTED;
     EncodeTiledFn encode = encode_tiled_fn();
     if (!encode) return BCNN_ERR_CUDA;
@@ -415,9 +414,9 @@ int launch_bn(const ConvProblem &p0, const PreparedWeights &pw, cudaStream_t str
     if (encode(&wmap, CU_TENSOR_MAP_DATA_TYPE_UINT8, 2, const_cast<uint8_t *>(pw.wexp), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
                CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
         return BCNN_ERR_CUDA;
-    void (*k)(const ConvProblem, const int32_t *, const CUtensorMap, const int) = p.mode == 1 ? conv_tc_pre_kernel<BN, 1> : conv_tc_pre_kernel<BN, 0>;
+    auto k = conv_tc_pre_kernel<BN, MODE, G, TEAMS>;
     if (!allow_smem((const void *)k, MAX_SMEM)) return BCNN_ERR_CUDA;
-    return launch(k, grid, Cfg<BN>::THREADS, smem, stream, p, pw.cst, wmap, ktw);
+    return launch(k, grid, C::THREADS, smem, stream, p, pw.cst, wmap, ktw);
 }
 
 }  // namespace
@@ -493,7 +492,7 @@ bool conv_tc_pre_supports(const ConvProblem &p)
     if (p.mode == 1 && (p.C_out % 32 != 0)) return false;
     if (p.kh * p.kw > 31) return false;                       // one validity bit per tap
     if ((long)p.B * p.H * p.W * p.cw >= (1L << 31)) return false;     // rows address the input by 32-bit word offsets
-    if (smem_bytes<256>(ktab_words_for(p), p.mode) > MAX_SMEM) return false;
+    if (smem_bytes<Cfg<256, 1, 2, 2>>(ktab_words_for(p), 1) > MAX_SMEM) return false;
     if ((long)p.kh * p.W * p.cw >= (1L << 27)) return false;  // a unit's word offset within the window
     return p.K <= (1 << 20);                                  // sums up to 4 K + 2 stay exact in fp32
 }
@@ -506,16 +505,22 @@ int launch_conv_tc_pre(const ConvProblem &p, const void *prepared, cudaStream_t 
     prepared_layout(p.C_out, p.K, pw, bytes);
     pw.wexp = static_cast<const uint8_t *>(prepared);
     pw.cst = reinterpret_cast<const int32_t *>(pw.wexp + (size_t)pw.n_pad * pw.k_pad / 2);
-    // 256-wide tiles have a single accumulator buffer (their epilogue is not overlapped): worth it when the K loop is
-    // long and the narrower tiles do not fill the last wave so much better (as in the streaming engine)
-    if (p.C_out > 128 && p.kwords >= 24) {
-        const int sms = sm_count();
-        const long m_tiles = ((long)p.M + BM - 1) / BM;
-        const long waves256 = (m_tiles * ((p.C_out + 255) / 256) + sms - 1) / sms;
-        const long waves128 = (m_tiles * ((p.C_out + 127) / 128) + sms - 1) / sms;
-        if (10 * waves256 <= 6 * waves128) return launch_bn<256>(p, pw, stream);
-    }
-    return launch_bn<128>(p, pw, stream);
+    // Tile width: 256 (two epilogue teams, one accumulator: the epilogue is not overlapped), 128 or 64.  Narrow tiles spread a
+    // small layer over more multiprocessors and shorten its epilogue, but every tile expands its activation rows again.
+    // Estimated time in ns, fitted to layers and products on B200 (28 shapes, within 10 %): a start, a term per tile column
+    // of the longest CTA and one per 256-bit stage.
+    //   3x3 256 -> 256, M = 50176: 16.0 (256), 16.7 (128), 25.5 (64) us;  M = 196: 6.9, 5.6, 5.2;  512 -> 512, M = 12544: 16.9, 15.9, 25.5
+    const int sms = sm_count();
+    const long m_tiles = ((long)p.M + BM - 1) / BM, kt = (p.kwords + 7) / 8;
+    auto cost = [&](int bn, long start, long wave, long stage) {
+        const long waves = (m_tiles * ((p.C_out + bn - 1) / bn) + sms - 1) / sms;
+        return start + waves * (wave + kt * stage);
+    };
+    const bool packed = p.mode == 1;
+    const long c256 = cost(256, 3200, packed ? 1660 : 4300, 288), c128 = cost(128, 3500, packed ? 600 : 2200, 185), c64 = cost(64, 3100, packed ? 530 : 1150, 167);
+    if (c64 <= c128 && c64 <= c256) return packed ? launch_bn<64, 1, 2, 1>(p, pw, stream) : launch_bn<64, 0, 2, 1>(p, pw, stream);
+    if (c128 <= c256) return packed ? launch_bn<128, 1, 2, 1>(p, pw, stream) : launch_bn<128, 0, 3, 2>(p, pw, stream);
+    return packed ? launch_bn<256, 1, 2, 2>(p, pw, stream) : launch_bn<256, 0, 2, 2>(p, pw, stream);
 }
 
 }  // namespace bcnn

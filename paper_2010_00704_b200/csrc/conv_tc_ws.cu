@@ -323,27 +323,11 @@ conv_tc_ws_kernel(const ConvProblem p)
                         cp_async_wait<ID_AHEAD>();                    // this chunk's copy has landed
                         words[ch] = module_chunk(p, dot, id_warp + (uint32_t)cur_slot * (BM * ID_ROW_BYTES), (long)em - lane, n0 + col0, lane);
                         if (++cur_slot == ID_SLOTS) cur_slot = 0;
-                    } else if ((p.C_out & 3) == 0 && (n0 + col0 + 32 <= p.C_out)) {
-                        // full chunk (warp-uniform): staged, the warp stores whole 128-byte rows
+                    } else {
                         int o[32];
                         biased_ints(v, colc_addr + 4u * col0, o);
                         const long row0 = (long)em - lane;
-                        store_int32_block(static_cast<int32_t *>(p.out) + row0 * p.C_out + n0 + col0, p.C_out, o, i32_tile, row0, p.M, lane);
-                    } else if (em < p.M) {
-                        int32_t *dst = static_cast<int32_t *>(p.out) + (long)em * p.C_out + n0 + col0;
-                        const bool vec = (p.C_out & 3) == 0 && (n0 + col0 + 32 <= p.C_out);
-                        int o[32];
-                        biased_ints(v, colc_addr + 4u * col0, o);
-#pragma unroll
-                        for (int i4 = 0; i4 < 8; ++i4) {
-                            if (vec) {
-                                *reinterpret_cast<int4 *>(dst + 4 * i4) = make_int4(o[4 * i4], o[4 * i4 + 1], o[4 * i4 + 2], o[4 * i4 + 3]);
-                            } else {
-#pragma unroll
-                                for (int i = 0; i < 4; ++i)
-                                    if (n0 + col0 + 4 * i4 + i < p.C_out) dst[4 * i4 + i] = o[4 * i4 + i];
-                            }
-                        }
+                        store_int32_block(static_cast<int32_t *>(p.out) + row0 * p.C_out + n0 + col0, p.C_out, o, i32_tile, row0, p.M, lane, cn - col0);
                     }
                 }
             }

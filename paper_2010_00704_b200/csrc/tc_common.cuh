@@ -606,26 +606,37 @@ __device__ __forceinline__ void expand_store_stage8(uint32_t taddr, uint32_t src
     }
 }
 
-// int32 output of one accumulator chunk: 32 rows (one per lane) x 32 consecutive columns.  A lane storing its own
-// row touches 32 rows x 16 bytes per instruction; staged through shared memory the warp stores 4 rows x 128
-// contiguous bytes per instruction instead.  `warp_tile`: I32_TILE_BYTES of shared memory owned by this warp;
-// `dst0` points at (row0, first column), `ldc` is the row pitch in elements (a multiple of 4, 16-byte aligned rows).
-// All 32 lanes must call it.
+// int32 output of one accumulator chunk: 32 rows (one per lane) x 32 consecutive columns, of which the first `ncols` exist.
+// A lane storing its own row touches 32 rows per instruction; staged through shared memory the warp stores contiguous pieces
+// of rows instead: four whole 128-byte rows per instruction where rows are 16-byte aligned, else one row of 32 integers
+// (13208 x 473, K = 704: 40 -> 12 us).  `warp_tile`: I32_TILE_BYTES of shared memory owned by this warp; `dst0` points at (row0, first
+// column), `ldc` is the row pitch in elements.  All 32 lanes must call it.
 constexpr int I32_ROW_BYTES = 144;                         // 128 + 16: conflict-free both ways
 constexpr int I32_TILE_BYTES = 32 * I32_ROW_BYTES;
 __device__ __forceinline__ void store_int32_block(int32_t *dst0, long ldc, const int (&o)[32], uint32_t warp_tile,
-                                                  long row0, long M, int lane)
+                                                  long row0, long M, int lane, int ncols)
 {
     const uint32_t mine = warp_tile + (uint32_t)(lane * I32_ROW_BYTES);
 #pragma unroll
     for (int i4 = 0; i4 < 8; ++i4)
         st_shared_v4(mine + 16u * i4, (uint32_t)o[4 * i4], (uint32_t)o[4 * i4 + 1], (uint32_t)o[4 * i4 + 2], (uint32_t)o[4 * i4 + 3]);
     __syncwarp();
+    if ((ldc & 3) == 0 && ncols >= 32) {                   // warp-uniform; the output is 16-byte aligned and chunks start at multiples of 32
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {
-        const int r = (lane >> 3) + 4 * i;
-        const uint4 v = ld_shared_v4(warp_tile + (uint32_t)(r * I32_ROW_BYTES + (lane & 7) * 16));
-        if (row0 + r < M) *reinterpret_cast<uint4 *>(dst0 + (long)r * ldc + 4 * (lane & 7)) = v;
+        for (int i = 0; i < 8; ++i) {
+            const int r = (lane >> 3) + 4 * i;
+            const uint4 v = ld_shared_v4(warp_tile + (uint32_t)(r * I32_ROW_BYTES + (lane & 7) * 16));
+            if (row0 + r < M) *reinterpret_cast<uint4 *>(dst0 + (long)r * ldc + 4 * (lane & 7)) = v;
+        }
+    } else {
+        const int rows = (int)min(32L, M - row0);
+        int32_t *dst = dst0 + lane;
+#pragma unroll 8
+        for (int r = 0; r < 32; ++r, dst += ldc) {
+            int v;
+            asm volatile("ld.shared.b32 %0, [%1];" : "=r"(v) : "r"(warp_tile + (uint32_t)(r * I32_ROW_BYTES + 4 * lane)) : "memory");
+            if (r < rows && lane < ncols) *dst = v;
+        }
     }
     __syncwarp();
 }
