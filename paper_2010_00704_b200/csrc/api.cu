@@ -76,9 +76,9 @@ int make_conv_problem(ConvProblem &p, const void *x, const void *w, const int32_
 // Measured on B200 (bench.py --mode sweep):
 //   * pointwise layers (1x1, stride 1, no padding; GEMMs) with K <= 128 and C_out <= 128, packed output: pointwise
 //     tcgen05 engine (memory-bound shapes: rows bulk-copied in chunks, one hand-over per chunk);
-//   * pointwise layers with K = 256 or 512 and 128, 256 or 512 output channels, packed output: wide pointwise tcgen05
-//     engine (a row tile expanded once for all resident weight slices; 1.2 - 2x the weight-stationary engine);
-//   * 3x3 layers (stride 1 or 2) on 32 or 64 input channels with C_out <= 64, packed output, whose 8 x 16 output tiles
+//   * pointwise layers with K = 128, 256 or 512 and a multiple of 128 output channels, packed output: wide pointwise tcgen05
+//     engine (a row tile expanded once for all resident weight slices; 1.5 - 3x the weight-stationary engine);
+//   * 3x3 layers (stride 1 or 2) on 32 or 64 input channels with C_out <= 128, packed output, whose 8 x 16 output tiles
 //     are at least three quarters full: halo-tile tcgen05 engine (input tiles by tiled TMA copies);
 //   * C_out >= 256, or weights too large to keep expanded in shared memory: streaming tcgen05 engine;
 //   * 1x1 layer with C_in = 32 and C_out <= 32 (one XOR + popcount per output): CUDA-core pointwise kernel;
@@ -90,7 +90,7 @@ int auto_engine(const ConvProblem &p)
 {
     if (conv_tc_pw_supports(p)) return BCNN_ENGINE_TC_PW;
     if (conv_tc_pn_supports(p)) return BCNN_ENGINE_TC_PN;
-    if (p.C_out <= 64 && conv_tc_c3_supports(p)) {
+    if (conv_tc_c3_supports(p)) {
         const long covered = (long)((p.OH + 7) / 8 * 8) * ((p.OW + 15) / 16 * 16);
         if (4L * p.OH * p.OW >= 3L * covered) return BCNN_ENGINE_TC_C3;
     }
@@ -387,10 +387,17 @@ int bcnn_prepared_preferred(int B, int H, int W, int C_in, int C_out, int kh, in
     const int st = make_conv_problem(p, dummy, dummy, fused ? static_cast<const int32_t *>(dummy) : nullptr, dummy,
                                      B, H, W, C_in, C_out, kh, kw, stride, pad, fused != 0);
     if (st != BCNN_OK) return 0;
-    // measured (bench.py --mode sweep): streaming prepared weights wins wherever AUTO would run the streaming engine
-    // (wide layers, long K) and on every K >= 2048; the weight-stationary and pointwise engines keep the short-K layers
+    // Measured: streaming prepared weights wins wherever AUTO would expand them on every call - the streaming engine always,
+    // the weight-stationary one except on many rows of a short K, where its expansion is spread thin (56x56 64 -> 128 /2 at
+    // batch 256, M = 200704, K = 576: 16.1 against 18.2 us; K = 1152: 19.7 against 19.0; M = 784: 6.5 against 4.0).  The pointwise
+    // and halo-tile engines keep their layers.
     if (!conv_tc_pre_supports(p)) return 0;
-    return (auto_engine(p) == BCNN_ENGINE_TC_I8 || p.K >= 2048) ? 1 : 0;
+    switch (auto_engine(p)) {
+    case BCNN_ENGINE_TC_PW: case BCNN_ENGINE_TC_PN: case BCNN_ENGINE_TC_C3: return 0;
+    case BCNN_ENGINE_TC_WS: return p.K >= 1024 || p.M < 98304 ? 1 : 0;
+    case BCNN_ENGINE_LOP3: return conv_lop3_pointwise_k32(p) ? 0 : 1;
+    default: return 1;
+    }
 }
 
 int bcnn_auto_engine(int B, int H, int W, int C_in, int C_out, int kh, int kw, int stride, int pad, int fused)

@@ -1,5 +1,5 @@
-// Wide pointwise engine: binary 1x1 convolutions (stride 1, no padding) and plain GEMMs with K = 256 or 512 bits and
-// 128, 256 or 512 output channels, packed output - the deeper binary 1x1 convolutions of the paper's network (Section
+// Wide pointwise engine: binary 1x1 convolutions (stride 1, no padding) and plain GEMMs with K = 128, 256 or 512 bits
+// and a multiple of 128 output channels, packed output - the deeper binary 1x1 convolutions of the paper's network (Section
 // 4.2.1; Table 1: 256 and 512 channels at 56 x 56 ... 14 x 14).  A 128-row tile of such a layer is only 8 or 16 words of
 // K per row and a few hundred tensor-pipe cycles per 128 output channels: the engines that cut the output channels
 // into slices and walk the rows once per slice expand every activation row once per slice and pay a pipeline's
@@ -10,8 +10,8 @@
 // group walks all row tiles).
 //   * A row tile is a contiguous block of x (128 rows x K / 8 bytes): one bulk asynchronous copy (cp.async.bulk) per tile
 //     into a ring in shared memory, two loader warps taking alternate tiles.
-//   * Tensor memory: two accumulators and a ring of activation UNITS of eight K words (32 columns); a tile is one unit
-//     (K = 256) or two (K = 512, filled by two producer groups).  Four producer groups of four warps (thread = row: two
+//   * Tensor memory: two accumulators and a ring of activation UNITS of eight K words (32 columns; four words for K = 128); a
+//     tile is one unit, or two for K = 512 (filled by two producer groups).  Four producer groups of four warps (thread = row: two
 //     16-byte shared-memory loads, 40 logic operations, one tensor-memory store).
 //   * A tile's output channels are cut into PARTS of 128 (one slice each).  Two issuer warps walk the tiles in order and take
 //     alternate parts, each with its own accumulator and epilogue group: per part an issuer waits for its accumulator, issues
@@ -46,10 +46,9 @@ constexpr int ERR_PN_ACC_TIMEOUT = 156;          // issuer: an accumulator was n
 constexpr int NGRP = 2;                   // loader / epilogue groups
 constexpr int NPG = 4;                    // producer groups of four warps
 constexpr int RD = 4;                     // row tiles in a loader's ring
-constexpr int UWORDS = 8;                 // K words per unit
-constexpr int U_COLS = 4 * UWORDS;
 constexpr int BN = 128;                   // output channels per weight slice (rows of a weight tile)
 constexpr int NB = 64, NAF = 8;
+constexpr int MAX_TILES = 7;              // row tiles in the ring of units
 constexpr int NISS = 2;                   // issuer warps (parts alternate)
 constexpr int MAX_NACC = 4;
 constexpr int FIRST_LOADER_WARP = 2, FIRST_PRODUCER_WARP = 4, FIRST_EPILOGUE_WARP = 4 + 4 * NPG;
@@ -63,18 +62,18 @@ struct PnPlan {
     int m_tiles;
 };
 
-// UPT: units per tile = K / 256
-template <int UPT>
+// UPT: units per tile; UWORDS: K words per unit (8; 4 for K = 128)
+template <int UPT, int UWORDS>
 __global__ void __launch_bounds__(THREADS, 1)
 conv_tc_pn_kernel(const ConvProblem p, const PnPlan plan)
 {
-    constexpr int KWORDS = UWORDS * UPT, KT = KWORDS / 8;
+    constexpr int KWORDS = UWORDS * UPT, KT = (KWORDS + 7) / 8, U_COLS = 4 * UWORDS;
     constexpr int TILE_BYTES = BM * KWORDS * 4;
     constexpr int NBARS = 2 * NGRP * RD + NAF + NB + MAX_NACC;
-    // an accumulator per issuer / epilogue group; seven units beside them: seven tiles (K = 256) or three (K = 512)
-    constexpr int NACC = 2, NUNIT = (CB_COL - NACC * BN) / U_COLS / UPT * UPT;
+    // an accumulator per issuer / epilogue group; beside them seven tiles (three for K = 512)
+    constexpr int NACC = 2, NU0 = (CB_COL - NACC * BN) / U_COLS / UPT * UPT, NUNIT = NU0 < MAX_TILES ? NU0 : MAX_TILES;
     constexpr int A_COL0 = NACC * BN;
-    static_assert(NUNIT / UPT <= NAF, "ring of tile-full barriers");
+    static_assert(NUNIT / UPT <= MAX_TILES && MAX_TILES < NAF, "ring of tile-full barriers");
 
     extern __shared__ unsigned char smem_raw[];
     __shared__ __align__(8) unsigned long long bars[NBARS];
@@ -148,8 +147,8 @@ conv_tc_pn_kernel(const ConvProblem p, const PnPlan plan)
             int pop = __popc(w[u]);
             pop += __shfl_xor_sync(0xffffffffu, pop, 1);
             pop += __shfl_xor_sync(0xffffffffu, pop, 2);
-            pop += __shfl_xor_sync(0xffffffffu, pop, 4);
-            if ((e & 7) == 0) asm volatile("red.shared.add.u32 [%0], %1;" ::"r"(pops + 4u * rw), "r"(pop) : "memory");
+            if (KWORDS >= 8) pop += __shfl_xor_sync(0xffffffffu, pop, 4);
+            if (KWORDS >= 8 ? (e & 7) == 0 : (e & 3) == 0) asm volatile("red.shared.add.u32 [%0], %1;" ::"r"(pops + 4u * rw), "r"(pop) : "memory");
         }
     }
     tc_fence_before();
@@ -287,11 +286,13 @@ conv_tc_pn_kernel(const ConvProblem p, const PnPlan plan)
             const int lg = n & 1, stage = (n >> 1) % RD;
             if (!pw_wait<64>(load_full(lg, stage), (uint32_t)((n >> 1) / RD) & 1u, abort_flag, p.err, ERR_PN_PRODUCER_TIMEOUT)) break;
             const uint32_t src = ring + (uint32_t)(lg * RD + stage) * TILE_BYTES + my_off;
-            const uint4 q0 = ld_shared_v4(src), q1 = ld_shared_v4(src + 16u);
+            const uint4 q0 = ld_shared_v4(src);
+            uint4 q1 = q0;
+            if (UWORDS == 8) q1 = ld_shared_v4(src + 16u);
             __syncwarp();
             mbar_arrive_pred(load_empty(lg, stage), lane0);        // the stage may be refilled
             uint32_t v[32];                       // expanded before the wait for the unit
-            expand_stage8(q0, q1, v);
+            expand_stage8(q0, q1, v);             // (four words: the second half is dropped)
             // the MMAs of the tile that used this ring position last have read it (nothing to wait for the first time round)
             const int u = n * UPT + h;
             if (u >= NUNIT) {
@@ -301,7 +302,8 @@ conv_tc_pn_kernel(const ConvProblem p, const PnPlan plan)
             }
             tc_fence_after();
             const uint32_t taddr = t_lane + (uint32_t)((u % NUNIT) * U_COLS);
-            tc_st32_nowait(taddr, v);
+            if constexpr (UWORDS == 8) tc_st32_nowait(taddr, v);
+            else tc_st16_nowait(taddr, reinterpret_cast<const uint32_t (&)[16]>(v[0]));
             tc_wait_st();
             tc_fence_before();
             __syncwarp();
@@ -320,12 +322,12 @@ conv_tc_pn_kernel(const ConvProblem p, const PnPlan plan)
 // but every group expands all the rows; two share a row tile's expansion.  Two win once a CTA would walk more than a dozen row
 // tiles with one (256 x 256 at M = 802816: 39 -> 28 us, at 200704: 13.4 -> 11.3; 512 x 512 at M = 200704: 28.4 -> 23.9, at 50176:
 // 11.0 -> 11.5); four never do (one issuer pair cannot use them).
-int pn_resident_slices(int slices, int m_tiles, int sms) { return slices > 1 && (long)m_tiles * slices > 12L * sms ? 2 : 1; }
+int pn_resident_slices(int slices, int m_tiles, int sms) { return slices % 2 == 0 && (long)m_tiles * slices > 12L * sms ? 2 : 1; }
 
-template <int UPT>
+template <int UPT, int UWORDS>
 int launch_pn(const ConvProblem &p0, cudaStream_t stream)
 {
-    constexpr int KWORDS = UWORDS * UPT, KT = KWORDS / 8, TILE_BYTES = BM * KWORDS * 4;
+    constexpr int KWORDS = UWORDS * UPT, KT = (KWORDS + 7) / 8, TILE_BYTES = BM * KWORDS * 4;
     ConvProblem p = p0;
     p.err = device_error_word();
     PnPlan plan;
@@ -339,7 +341,7 @@ int launch_pn(const ConvProblem &p0, cudaStream_t stream)
     int per_group = sms / plan.ng;
     if (per_group > plan.m_tiles) per_group = plan.m_tiles;
     if (per_group < 1) per_group = 1;
-    void (*k)(const ConvProblem, const PnPlan) = conv_tc_pn_kernel<UPT>;
+    void (*k)(const ConvProblem, const PnPlan) = conv_tc_pn_kernel<UPT, UWORDS>;
     const int ask = smem < 120 * 1024 ? 120 * 1024 : smem;          // one CTA per SM (it takes all of tensor memory)
     if (!allow_smem((const void *)k, 227 * 1024 - 1024)) return BCNN_ERR_CUDA;
     return launch(k, (unsigned)(per_group * plan.ng), THREADS, ask, stream, p, plan);
@@ -351,14 +353,14 @@ bool conv_tc_pn_supports(const ConvProblem &p)
 {
     if (p.mode != 1) return false;                               // packed output only
     if (!(p.kh == 1 && p.kw == 1 && p.stride == 1 && p.pad == 0)) return false;
-    if (p.kwords != 8 && p.kwords != 16) return false;           // K = 256 or 512
-    return p.C_out == 128 || p.C_out == 256 || p.C_out == 512;
+    if (p.kwords != 4 && p.kwords != 8 && p.kwords != 16) return false;      // K = 128, 256 or 512
+    return p.C_out % BN == 0 && p.C_out <= 16 * BN;
 }
 
 int launch_conv_tc_pn(const ConvProblem &p, cudaStream_t stream)
 {
     if (!conv_tc_pn_supports(p)) return BCNN_ERR_UNSUPPORTED;
-    return p.kwords == 8 ? launch_pn<1>(p, stream) : launch_pn<2>(p, stream);
+    return p.kwords == 4 ? launch_pn<1, 4>(p, stream) : (p.kwords == 8 ? launch_pn<1, 8>(p, stream) : launch_pn<2, 8>(p, stream));
 }
 
 }  // namespace bcnn

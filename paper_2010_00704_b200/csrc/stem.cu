@@ -16,6 +16,8 @@
 // carries 127 - theta_n, theta_n = floor((32 - thr_n) / 2) clamped to [-1, 32], so that bit 7 of field n
 // is set exactly when mismatches > theta_n, i.e. when the output bit is 0.
 //
+// The table pays for itself only when a CTA has many pixels: up to PLAIN_PIXELS per multiprocessor the plain per-channel path
+// runs, spread over all of them (one 224 x 224 image: 7.6 -> @@ us).
 // With a NaN or infinite bias the thermometer argument fails (inf - inf = NaN -> -1): the plain
 // per-channel path runs instead (32 fp32 adds + compares, 32 popcounts per pixel).
 #include "bcnn_common.cuh"
@@ -25,11 +27,12 @@ namespace bcnn {
 namespace {
 
 constexpr int STEM_THREADS = 1024;
+constexpr long PLAIN_PIXELS = 1024;        // per multiprocessor
 constexpr int STEM_LEVELS = 9 * 9 * 9 * 9;
 
 __global__ void __launch_bounds__(STEM_THREADS, 1)
 stem_c4r8_k32_kernel(const float4 *__restrict__ x, const float *__restrict__ bias, const uint32_t *__restrict__ w,
-                     const int32_t *__restrict__ thr, uint32_t *__restrict__ out, long npix)
+                     const int32_t *__restrict__ thr, uint32_t *__restrict__ out, long npix, const bool plain)
 {
     pdl_trigger();
     pdl_wait();
@@ -60,7 +63,7 @@ stem_c4r8_k32_kernel(const float4 *__restrict__ x, const float *__restrict__ bia
     __syncthreads();
     const long stride = (long)gridDim.x * blockDim.x;
 
-    if (!all_finite) {
+    if (!all_finite || plain) {
         // plain path: every sign channel evaluated as written, then 32 XOR + popcount
         for (long p = (long)blockIdx.x * blockDim.x + tid; p < npix; p += stride) {
             const float4 v = __ldcs(x + p);
@@ -164,10 +167,11 @@ int launch_stem_c4r8_k32(const float *x, const float *bias, const uint32_t *w, c
                          long npix, cudaStream_t stream)
 {
     const int sms = sm_count();
-    long blocks = (npix + STEM_THREADS * 4 - 1) / (STEM_THREADS * 4);
-    if (blocks > sms) blocks = sms;             // one resident CTA per SM builds the table once, grid-stride inside
+    const bool plain = npix <= sms * PLAIN_PIXELS;
+    long blocks = plain ? (npix + 255) / 256 : (npix + STEM_THREADS * 4 - 1) / (STEM_THREADS * 4);
+    if (!plain && blocks > sms) blocks = sms;   // one resident CTA per SM builds the table once, grid-stride inside
     if (blocks < 1) blocks = 1;
-    return launch(stem_c4r8_k32_kernel, (unsigned)blocks, STEM_THREADS, 0, stream, reinterpret_cast<const float4 *>(x), bias, w, thr, out, npix);
+    return launch(stem_c4r8_k32_kernel, (unsigned)blocks, plain ? 256 : STEM_THREADS, 0, stream, reinterpret_cast<const float4 *>(x), bias, w, thr, out, npix, plain);
 }
 
 }  // namespace bcnn
