@@ -85,9 +85,13 @@ int make_conv_problem(ConvProblem &p, const void *x, const void *w, const int32_
 //   * C_out <= 128 with K >= 64, and wider layers with K <= 1152 and M >= 32768 (in 128-channel slices):
 //     weight-stationary tcgen05 engine;
 //   * other K = 32 layers: register-fed warp-level int8 engine;
-//   * the single-bit mma.sync and CUDA-core engines never win and serve as fallbacks.
+//   * CUDA-core engine: the smallest calls with K <= 256;
+//   * the single-bit mma.sync engine never wins and serves as a fallback.
 int auto_engine(const ConvProblem &p)
 {
+    // a call whose work is a wave of 64 x 64 tiles of up to 256 bits is over before a tensor-core engine has its weights expanded
+    // (1x1 64 -> 64 at M = 3136: 3.4 against 4.2 us, 256 -> 256 at M = 196: 3.4 against 4.4)
+    if (p.K <= 256 && ((p.M + 63L) / 64) * ((p.C_out + 63) / 64) <= sm_count()) return BCNN_ENGINE_LOP3;
     if (conv_tc_pw_supports(p)) return BCNN_ENGINE_TC_PW;
     if (conv_tc_pn_supports(p)) return BCNN_ENGINE_TC_PN;
     if (conv_tc_c3_supports(p)) {
@@ -390,12 +394,14 @@ int bcnn_prepared_preferred(int B, int H, int W, int C_in, int C_out, int kh, in
     // Measured: streaming prepared weights wins wherever AUTO would expand them on every call - the streaming engine always,
     // the weight-stationary one except on many rows of a short K, where its expansion is spread thin (56x56 64 -> 128 /2 at
     // batch 256, M = 200704, K = 576: 16.1 against 18.2 us; K = 1152: 19.7 against 19.0; M = 784: 6.5 against 4.0).  The pointwise
-    // and halo-tile engines keep their layers.
+    // and halo-tile engines keep their layers, except the smallest: they expand their weights at the start.
     if (!conv_tc_pre_supports(p)) return 0;
     switch (auto_engine(p)) {
-    case BCNN_ENGINE_TC_PW: case BCNN_ENGINE_TC_PN: case BCNN_ENGINE_TC_C3: return 0;
+    case BCNN_ENGINE_TC_PW: case BCNN_ENGINE_TC_PN: case BCNN_ENGINE_TC_C3:
+        // 1x1 512 -> 512: 5.0 against 3.7 us at M = 49, 6.5 against 8.3 at 12544; 3x3 64 -> 64: 4.4 against 4.0 at 3136
+        return p.M <= 4096 && ((p.M + 127) / 128) * ((p.C_out + 63) / 64) <= sm_count() ? 1 : 0;
     case BCNN_ENGINE_TC_WS: return p.K >= 1024 || p.M < 98304 ? 1 : 0;
-    case BCNN_ENGINE_LOP3: return conv_lop3_pointwise_k32(p) ? 0 : 1;
+    case BCNN_ENGINE_LOP3: return p.K <= 64 ? 0 : 1;
     default: return 1;
     }
 }

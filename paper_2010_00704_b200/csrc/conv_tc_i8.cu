@@ -63,7 +63,7 @@ __host__ __device__ inline int smem_bytes(int ktab_words, int mode = 1)
     // module epilogue: + the identity staging ring; int32 output of the 128-wide tiles: + the store staging tiles
     // (both only used where they fit: 128-wide tiles)
     return 1024 + C::STAGES * C::W_BYTES + C::BITS_BYTES + C::CONST_BYTES + C::TABLE_BYTES + ktab_words * 4 +
-           (mode == 2 ? ID_RING_BYTES + 16 : 0) + (mode == 0 && BN == 128 ? EPI_WARPS * I32_TILE_BYTES + 16 : 0);
+           (mode == 2 ? ID_RING_BYTES + 16 : 0) + (mode == 0 && BN <= 128 ? EPI_WARPS * I32_TILE_BYTES + 16 : 0);
 }
 
 template <int BN, int MODE>
@@ -121,11 +121,11 @@ conv_tc_i8_kernel(const ConvProblem p, const int ktab_words)
     }
     const int gwidth = gather_width(p.cw);
     build_unit_table8(p, ktab_addr, ktiles * (8 / gwidth), gwidth, tid, C::THREADS);
-    pdl_wait();
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
     pdl_trigger();
+    pdl_wait();
     const uint32_t tmem_base = tmem_base_smem;
 
     if (warp == 0) {
@@ -263,7 +263,7 @@ conv_tc_i8_kernel(const ConvProblem p, const int ktab_words)
                         cp_async_wait<ID_AHEAD>();                    // this chunk's copy has landed
                         words[ch] = module_chunk(p, dot, id_warp + (uint32_t)cur_slot * (BM * ID_ROW_BYTES), (long)em - lane, n0 + col0, lane);
                         if (++cur_slot == ID_SLOTS) cur_slot = 0;
-                    } else if constexpr (BN == 128) {
+                    } else if constexpr (BN <= 128) {
                         int o[32];
                         biased_ints(v, table + 4u * col0, o);
                         const long row0 = (long)em - lane;
@@ -294,7 +294,7 @@ conv_tc_i8_kernel(const ConvProblem p, const int ktab_words)
             if ((FUSED || (MODULE && p.out != nullptr)) && em < p.M) {
                 const int owords = p.C_out >> 5;
                 uint32_t *dst = static_cast<uint32_t *>(p.out) + (long)em * owords + (n0 >> 5);
-                if ((owords & 3) == 0 && n0 + BN <= p.C_out) {
+                if (BN >= 128 && (owords & 3) == 0 && n0 + BN <= p.C_out) {
 #pragma unroll
                     for (int c4 = 0; c4 < BN / 128; ++c4)
                         *reinterpret_cast<uint4 *>(dst + 4 * c4) =
@@ -513,9 +513,14 @@ int launch_conv_tc_i8(const ConvProblem &p, cudaStream_t stream)
         const long m_tiles = ((long)p.M + BM - 1) / BM;
         const long waves256 = (m_tiles * ((p.C_out + 255) / 256) + sms - 1) / sms;
         const long waves128 = (m_tiles * ((p.C_out + 127) / 128) + sms - 1) / sms;
-        if (10 * waves256 <= 6 * waves128) return launch_bn<256>(p, stream);
-        return launch_bn<128>(p, stream);
+        if (waves256 > 1 && 10 * waves256 <= 6 * waves128) return launch_bn<256>(p, stream);
     }
+    // small problems: 64-wide tiles on twice the multiprocessors, with a shorter epilogue.  A tile column costs about 0.42 us per
+    // 256-bit stage at 128 and 0.33 at 64, the start 0.5 us less (1024 x 1024 x 4608: 12.3 -> 10.2 us, 20 x 64 x 960: 5.3 -> 4.7)
+    const int sms = sm_count();
+    const long m_tiles = ((long)p.M + BM - 1) / BM, kt = (p.kwords + 7) / 8;
+    const long w64 = (m_tiles * ((p.C_out + 63) / 64) + sms - 1) / sms, w128 = (m_tiles * ((p.C_out + 127) / 128) + sms - 1) / sms;
+    if (p.mode != 2 && w64 * kt * 330 < w128 * kt * 420 + 500) return launch_bn<64>(p, stream);
     return launch_bn<128>(p, stream);
 }
 

@@ -17,7 +17,8 @@
 // is set exactly when mismatches > theta_n, i.e. when the output bit is 0.
 //
 // The table pays for itself only when a CTA has many pixels: up to PLAIN_PIXELS per multiprocessor the plain per-channel path
-// runs, spread over all of them (one 224 x 224 image: 7.6 -> @@ us).
+// runs in a kernel of its own, spread over all of them (one 224 x 224 image:
+// 7.6 -> 2.8 us; four images: 7.9 -> 5.9 us; eight: 8.2 with the table, 10 without).
 // With a NaN or infinite bias the thermometer argument fails (inf - inf = NaN -> -1): the plain
 // per-channel path runs instead (32 fp32 adds + compares, 32 popcounts per pixel).
 #include "bcnn_common.cuh"
@@ -27,12 +28,54 @@ namespace bcnn {
 namespace {
 
 constexpr int STEM_THREADS = 1024;
-constexpr long PLAIN_PIXELS = 1024;        // per multiprocessor
+constexpr long PLAIN_PIXELS = 1792;        // per multiprocessor
 constexpr int STEM_LEVELS = 9 * 9 * 9 * 9;
+
+// One pixel, every sign channel evaluated as written, then 32 XOR + popcount.
+__device__ __forceinline__ uint32_t stem_pixel(const float4 &v, const float *sb, const uint32_t *sw, const int *stheta)
+{
+    const float f[4] = {v.x, v.y, v.z, v.w};
+    uint32_t word = 0;
+#pragma unroll
+    for (int c = 0; c < 32; ++c) {
+        const float s = __fadd_rn(f[c & 3], sb[c]);
+        word |= (s >= 0.0f ? 1u : 0u) << c;
+    }
+    uint32_t o = 0;
+#pragma unroll 8
+    for (int n = 0; n < 32; ++n) o |= (__popc(word ^ sw[n]) <= stheta[n] ? 1u : 0u) << n;
+    return o;
+}
+// out bit n = (32 - 2*mism >= thr)  <=>  mism <= floor((32 - thr) / 2)
+__device__ __forceinline__ int stem_theta(int thr)
+{
+    const long long th = (32LL - (long long)thr) >> 1;
+    return (int)(th < -1 ? -1 : (th > 32 ? 32 : th));
+}
+
+__global__ void __launch_bounds__(256)
+stem_plain_kernel(const float4 *__restrict__ x, const float *__restrict__ bias, const uint32_t *__restrict__ w,
+                  const int32_t *__restrict__ thr, uint32_t *__restrict__ out, long npix)
+{
+    __shared__ float sb[32];
+    __shared__ uint32_t sw[32];
+    __shared__ int stheta[32];
+    pdl_trigger();
+    const long p = (long)blockIdx.x * 256 + threadIdx.x;
+    pdl_wait();
+    const float4 v = p < npix ? __ldcs(x + p) : make_float4(0.f, 0.f, 0.f, 0.f);
+    if (threadIdx.x < 32) {
+        sb[threadIdx.x] = bias ? bias[threadIdx.x] : 0.0f;
+        sw[threadIdx.x] = w[threadIdx.x];
+        stheta[threadIdx.x] = stem_theta(thr[threadIdx.x]);
+    }
+    __syncthreads();
+    if (p < npix) __stcs(out + p, stem_pixel(v, sb, sw, stheta));
+}
 
 __global__ void __launch_bounds__(STEM_THREADS, 1)
 stem_c4r8_k32_kernel(const float4 *__restrict__ x, const float *__restrict__ bias, const uint32_t *__restrict__ w,
-                     const int32_t *__restrict__ thr, uint32_t *__restrict__ out, long npix, const bool plain)
+                     const int32_t *__restrict__ thr, uint32_t *__restrict__ out, long npix)
 {
     pdl_trigger();
     pdl_wait();
@@ -55,29 +98,14 @@ stem_c4r8_k32_kernel(const float4 *__restrict__ x, const float *__restrict__ bia
         sb[tid] = b;
         if (!(fabsf(b) <= 3.402823466e38f)) all_finite = 0;      // NaN or infinity
         sw[tid] = w[tid];
-        // out bit n = (32 - 2*mism >= thr)  <=>  mism <= floor((32 - thr) / 2)
-        long long th = (32LL - (long long)thr[tid]) >> 1;
-        th = th < -1 ? -1 : (th > 32 ? 32 : th);
-        stheta[tid] = (int)th;
+        stheta[tid] = stem_theta(thr[tid]);
     }
     __syncthreads();
     const long stride = (long)gridDim.x * blockDim.x;
 
-    if (!all_finite || plain) {
-        // plain path: every sign channel evaluated as written, then 32 XOR + popcount
+    if (!all_finite) {
         for (long p = (long)blockIdx.x * blockDim.x + tid; p < npix; p += stride) {
-            const float4 v = __ldcs(x + p);
-            const float f[4] = {v.x, v.y, v.z, v.w};
-            uint32_t word = 0;
-#pragma unroll
-            for (int c = 0; c < 32; ++c) {
-                const float s = __fadd_rn(f[c & 3], sb[c]);
-                word |= (s >= 0.0f ? 1u : 0u) << c;
-            }
-            uint32_t o = 0;
-#pragma unroll 8
-            for (int n = 0; n < 32; ++n) o |= (__popc(word ^ sw[n]) <= stheta[n] ? 1u : 0u) << n;
-            __stcs(out + p, o);
+            __stcs(out + p, stem_pixel(__ldcs(x + p), sb, sw, stheta));
         }
         return;
     }
@@ -167,11 +195,11 @@ int launch_stem_c4r8_k32(const float *x, const float *bias, const uint32_t *w, c
                          long npix, cudaStream_t stream)
 {
     const int sms = sm_count();
-    const bool plain = npix <= sms * PLAIN_PIXELS;
-    long blocks = plain ? (npix + 255) / 256 : (npix + STEM_THREADS * 4 - 1) / (STEM_THREADS * 4);
-    if (!plain && blocks > sms) blocks = sms;   // one resident CTA per SM builds the table once, grid-stride inside
-    if (blocks < 1) blocks = 1;
-    return launch(stem_c4r8_k32_kernel, (unsigned)blocks, plain ? 256 : STEM_THREADS, 0, stream, reinterpret_cast<const float4 *>(x), bias, w, thr, out, npix, plain);
+    if (npix <= sms * PLAIN_PIXELS)
+        return launch(stem_plain_kernel, (unsigned)((npix + 255) / 256), 256, 0, stream, reinterpret_cast<const float4 *>(x), bias, w, thr, out, npix);
+    long blocks = (npix + STEM_THREADS * 4 - 1) / (STEM_THREADS * 4);
+    if (blocks > sms) blocks = sms;             // one resident CTA per SM builds the table once, grid-stride inside
+    return launch(stem_c4r8_k32_kernel, (unsigned)blocks, STEM_THREADS, 0, stream, reinterpret_cast<const float4 *>(x), bias, w, thr, out, npix);
 }
 
 }  // namespace bcnn
