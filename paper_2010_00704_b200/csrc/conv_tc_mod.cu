@@ -7,8 +7,11 @@
 //   * identity tiles arrive and output tiles leave by tiled TMA copies of 128 rows x BN channels through a ring of NS tiles per
 //     epilogue team in shared memory (swizzled: one 16-byte access per lane and row without bank conflicts); a loader warp and a
 //     store warp issue them (an issue costs its warp some 500 cycles), the epilogue turns a tile in place;
-//   * per-channel values lie in shared memory as pairs of channels, read as 16-byte broadcasts; the arithmetic runs on pairs
-//     (f32x2: the same IEEE operations, half the issue slots);
+//   * per-channel values lie in shared memory as pairs of channels, read as 16-byte broadcasts - four cycles of the shared-memory
+//     pipe each, the epilogue's scarcest resource: one per branch {scale, shift} and one {slope, next bias}.  The constant
+//     K - 2 popc of a dot product is not among them, an MMA against a constant tile puts it into the accumulator
+//     (tc_slot.cuh);
+//   * the arithmetic runs on pairs (f32x2: the same IEEE operations, half the issue slots);
 //   * two epilogue teams take alternate PARTS (128 rows x BN channels).
 // The binary products are cheap beside that: a CTA keeps RS slices of BN channels' expanded weights in shared memory, expands
 // a row tile once (256-bit stages in a ring in tensor memory, as in conv_tc_ws.cu) and multiplies it against every resident
@@ -17,7 +20,7 @@
 // Arithmetic (bit-exact against the oracle): t_p = dot_p * scale_p + shift_p, summed in branch order, + identity, PReLU,
 // fp16, sign of (stored value + next bias): one fp32 operation per step, no contraction.
 // Every mbarrier wait is bounded and reports through the device error word.
-#include "tc_common.cuh"
+#include "tc_slot.cuh"
 #include "tensor_map.cuh"
 
 namespace bcnn {
@@ -35,8 +38,7 @@ constexpr int ISSUER = 0, LOADER = 1, STORER = 2 /* + team */, FIRST_PRODUCER = 
 constexpr int THREADS = 32 * (FIRST_EPILOGUE + 4 * TEAMS);
 constexpr int PROD_THREADS = G * BM;
 constexpr int HALF_BYTES = PROD_THREADS * 16, SLOT_BYTES = 2 * HALF_BYTES;
-constexpr int SF_COL = 512 - (int)SF_COLS;
-constexpr int MAX_STAGES = 11;
+constexpr int MAX_STAGES = 11, MAX_NBUF = 4;
 constexpr int MAX_SMEM = 226 * 1024;
 
 struct ModPlan {
@@ -50,11 +52,13 @@ struct ModPlan {
     int rs, ng, slices;       // resident slices, CTA groups, slices of BN channels
     int m_tiles;
     int units, gw;            // gather units of a row
-    uint32_t off_bits, off_stage, off_table, off_pop, off_tab;      // shared-memory offsets from the 1024-byte aligned base (weights first)
+    uint32_t off_bits, off_stage, off_table, off_pad, off_pop, off_tab, off_const;      // shared-memory offsets from the 1024-byte aligned base (weights first)
 };
 
-// per-channel-pair table of a slice: P entries of 32 bytes {scale, shift, cst, pad_dot} x 2, then 16 bytes {slope, next bias} x 2
-__host__ __device__ inline uint32_t pair_bytes(int P) { return 32u * (uint32_t)P + 16u; }
+// per-channel-pair table of a slice: P entries of 16 bytes {scale, shift} x 2, then 16 bytes {slope, next bias} x 2
+__host__ __device__ inline uint32_t pair_bytes(int P) { return 16u * (uint32_t)P + 16u; }
+// constant tiles: four 32-byte rows of (slice, branch) pairs side by side
+__host__ __device__ inline int const_tiles(int rs, int P) { return (rs * P + 3) / 4; }
 
 __device__ __forceinline__ unsigned long long add2(unsigned long long a, unsigned long long b)
 {
@@ -81,15 +85,15 @@ __device__ __forceinline__ unsigned long long mul2(unsigned long long a, unsigne
     const float2 x = floats2(a), y = floats2(b);
     return bits2(__float_as_uint(__fmul_rn(x.x, y.x)), __float_as_uint(__fmul_rn(x.y, y.y)));
 }
-__device__ __forceinline__ void tc_ld16(uint32_t taddr, uint32_t (&v)[16])
+__device__ __forceinline__ void tc_ld8_nowait(uint32_t taddr, uint32_t (&v)[8])
 {
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
-        "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];\n\t"
-        "tcgen05.wait::ld.sync.aligned;"
-        : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
-          "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
-        : "r"(taddr) : "memory");
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+                 : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7])
+                 : "r"(taddr) : "memory");
+}
+__device__ __forceinline__ void pin_regs8(uint32_t (&v)[8])
+{
+    asm volatile("" : "+r"(v[0]), "+r"(v[1]), "+r"(v[2]), "+r"(v[3]), "+r"(v[4]), "+r"(v[5]), "+r"(v[6]), "+r"(v[7]) :: "memory");
 }
 
 // BN: channels of a part (64, 32); PP: branches where known to the compiler (1, 2), else 0; SHIFTED: taps with a row mask
@@ -99,7 +103,7 @@ conv_tc_mod_kernel(const ModPlan L, const __grid_constant__ CUtensorMap idmap, c
 {
     constexpr int TILE_BYTES = BM * BN * 2, ROW_BYTES = BN * 2, W_STAGE = BN * ROWB;
     extern __shared__ unsigned char smem_raw[];
-    __shared__ __align__(8) unsigned long long bars[2 * MAX_STAGES + 4 + 3 * TEAMS * NS + 1];
+    __shared__ __align__(8) unsigned long long bars[2 * MAX_STAGES + 2 * MAX_NBUF + 3 * TEAMS * NS + 1];
     __shared__ uint32_t tmem_base_smem;
     __shared__ int abort_flag_smem;
 
@@ -113,16 +117,16 @@ conv_tc_mod_kernel(const ModPlan L, const __grid_constant__ CUtensorMap idmap, c
     const int parts = my_tiles * rs;
     const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;         // [rs][kst][BN rows][128 B] weights, then the rest
     const uint32_t bits_ring = base + L.off_bits, staging = base + L.off_stage, table = base + L.off_table, pops = base + L.off_pop;
-    const uint32_t tab = base + L.off_tab;
+    const uint32_t tab = base + L.off_tab, pads = base + L.off_pad, cexp = base + L.off_const;
     const uint32_t bar0 = smem_u32(bars);
     auto full_bar = [&](int s) { return bar0 + 8u * s; };
     auto empty_bar = [&](int s) { return bar0 + 8u * (MAX_STAGES + s); };
-    auto tfull_bar = [&](int t) { return bar0 + 8u * (2 * MAX_STAGES + t); };
-    auto tempty_bar = [&](int t) { return bar0 + 8u * (2 * MAX_STAGES + 2 + t); };
-    auto id_full = [&](int t, int s) { return bar0 + 8u * (2 * MAX_STAGES + 4 + t * NS + s); };
-    auto slot_free = [&](int t, int s) { return bar0 + 8u * (2 * MAX_STAGES + 4 + TEAMS * NS + t * NS + s); };
-    auto out_full = [&](int t, int s) { return bar0 + 8u * (2 * MAX_STAGES + 4 + 2 * TEAMS * NS + t * NS + s); };
-    const uint32_t ready_bar = bar0 + 8u * (2 * MAX_STAGES + 4 + 3 * TEAMS * NS);      // the resident weights are expanded
+    auto tfull_bar = [&](int b) { return bar0 + 8u * (2 * MAX_STAGES + b); };
+    auto tempty_bar = [&](int b) { return bar0 + 8u * (2 * MAX_STAGES + MAX_NBUF + b); };
+    auto id_full = [&](int t, int s) { return bar0 + 8u * (2 * MAX_STAGES + 2 * MAX_NBUF + t * NS + s); };
+    auto slot_free = [&](int t, int s) { return bar0 + 8u * (2 * MAX_STAGES + 2 * MAX_NBUF + TEAMS * NS + t * NS + s); };
+    auto out_full = [&](int t, int s) { return bar0 + 8u * (2 * MAX_STAGES + 2 * MAX_NBUF + 2 * TEAMS * NS + t * NS + s); };
+    const uint32_t ready_bar = bar0 + 8u * (2 * MAX_STAGES + 2 * MAX_NBUF + 3 * TEAMS * NS);      // the resident weights are expanded
     volatile int *abort_flag = &abort_flag_smem;
 
     if (tid == 0) {
@@ -130,9 +134,11 @@ conv_tc_mod_kernel(const ModPlan L, const __grid_constant__ CUtensorMap idmap, c
             mbar_init(full_bar(s), 4);
             mbar_init(empty_bar(s), 1);
         }
+        for (int b = 0; b < MAX_NBUF; ++b) {
+            mbar_init(tfull_bar(b), 1);
+            mbar_init(tempty_bar(b), 4);
+        }
         for (int t = 0; t < TEAMS; ++t) {
-            mbar_init(tfull_bar(t), 1);
-            mbar_init(tempty_bar(t), 4);
             for (int s = 0; s < NS; ++s) {
                 mbar_init(id_full(t, s), 1);
                 mbar_init(slot_free(t, s), 1);
@@ -176,39 +182,46 @@ conv_tc_mod_kernel(const ModPlan L, const __grid_constant__ CUtensorMap idmap, c
         const uint64_t desc0 = make_desc(base);
         const uint32_t desc_hi = (uint32_t)(desc0 >> 32), b_lo0 = (uint32_t)desc0;
         const uint32_t tmem_u = __shfl_sync(0xffffffffu, tmem_base, 0);
-        const uint32_t sf = tmem_u + (uint32_t)SF_COL, a_col0 = tmem_u + (uint32_t)(L.nbuf * P * BN);
+        const uint32_t sf = tmem_u + (uint32_t)CB_COL, c_lo0 = (uint32_t)make_desc(cexp), a_col0 = tmem_u + (uint32_t)(L.nbuf * P * BN);
         const int per_branch = L.kwp >> 1, granules = P * per_branch;      // two-word MMAs of a branch, of a row
-        bool ok = mbar_wait_warp(ready_bar, 0, abort_flag, p.err, ERR_MOD_ISSUER);
-        tc_fence_after();
-        for (int n = 0; n < parts && ok; ++n) {
-            const int tile = n / rs, s = n - tile * rs;
-            if (n >= L.nbuf) {
-                const int m = n - L.nbuf;                                  // the part whose accumulators these were
-                if (!mbar_wait_warp(tempty_bar(m & 1), (uint32_t)(m >> 1) & 1u, abort_flag, p.err, ERR_MOD_ISSUER)) break;
-            }
-            const uint32_t d0 = tmem_u + (uint32_t)((n % L.nbuf) * P * BN);
-            int br = 0, j = 0;                                             // branch and MMA within it
-            for (int k = 0; k < kst; ++k) {
-                const int item = tile * kst + k, slot = item % stages;
-                if (s == 0) {
-                    ok = mbar_wait_warp(full_bar(slot), (uint32_t)(item / stages) & 1u, abort_flag, p.err, ERR_MOD_ISSUER);
-                    if (!ok) break;
-                }
-                tc_fence_after();
-                const uint32_t a_t = a_col0 + (uint32_t)slot * 32u, b_lo = b_lo0 + (uint32_t)((s * kst + k) * (W_STAGE >> 4));
-                const int here = min(4, granules - 4 * k);
-                const bool lead = elect_one();
-                for (int g4 = 0; g4 < here; ++g4) {
-                    if (lead) tc_mma_f4_ts(d0 + (uint32_t)(br * BN), a_t + 8u * g4, b_lo + 2u * g4, desc_hi, idesc, sf, j > 0 ? 1u : 0u);
-                    if (++j == per_branch) { j = 0; ++br; }
-                }
-                if (lead) {
+        // (the elected lane runs the whole loop: a vote and a reconvergence per instruction cost more than the instruction)
+        if (elect_one()) {
+            bool ok = mbar_wait(ready_bar, 0, abort_flag, p.err, ERR_MOD_ISSUER);
+            int s = 0, buf = 0, slot0 = 0;                      // part = (row tile, slice s); its buffer; the tile's first item and ring slot
+            uint32_t buf_phase = 1, ring_phase0 = 0;                       // first use of every accumulator buffer: free
+            for (int n = 0; n < parts && ok; ++n) {
+                ok = mbar_wait(tempty_bar(buf), buf_phase, abort_flag, p.err, ERR_MOD_ISSUER);
+                if (!ok) break;
+                const uint32_t d0 = tmem_u + (uint32_t)(buf * P * BN);
+                int br = 0, j = 0, slot = slot0;                           // branch and MMA within it
+                uint32_t ring_phase = ring_phase0;
+                for (int k = 0; k < kst; ++k) {
+                    if (s == 0) {
+                        ok = mbar_wait(full_bar(slot), ring_phase, abort_flag, p.err, ERR_MOD_ISSUER);
+                        if (!ok) break;
+                    }
+                    tc_fence_after();
+                    const uint32_t a_t = a_col0 + (uint32_t)slot * 32u, b_lo = b_lo0 + (uint32_t)((s * kst + k) * (W_STAGE >> 4));
+                    const int here = min(4, granules - 4 * k);
+                    for (int g4 = 0; g4 < here; ++g4) {
+                        const uint32_t d = d0 + (uint32_t)(br * BN);
+                        if (j == 0) {                                      // the branch's constants
+                            const int ct = s * P + br;
+                            tc_mma_const(d, tmem_u, c_lo0 + (uint32_t)((ct >> 2) * (W_STAGE >> 4) + 2 * (ct & 3)), desc_hi, idesc);
+                        }
+                        tc_mma_f4_ts(d, a_t + 8u * g4, b_lo + 2u * g4, desc_hi, idesc, sf, 1u);
+                        if (++j == per_branch) { j = 0; ++br; }
+                    }
                     if (s == rs - 1) tc_commit(empty_bar(slot));           // the row tile's last part: the stage may be refilled
-                    if (k == kst - 1) tc_commit(tfull_bar(n & 1));
+                    if (++slot == stages) { slot = 0; ring_phase ^= 1u; }
                 }
-                __syncwarp();
+                if (!ok) break;
+                tc_commit(tfull_bar(buf));
+                if (++buf == L.nbuf) { buf = 0; buf_phase ^= 1u; }
+                if (++s == rs) { s = 0; slot0 = slot; ring_phase0 = ring_phase; }
             }
         }
+        __syncwarp();
     } else if (warp == LOADER) {
         // ------------------------------------------------------------------ identity tiles
         if (HAS_ID) {
@@ -281,9 +294,7 @@ conv_tc_mod_kernel(const ModPlan L, const __grid_constant__ CUtensorMap idmap, c
                 }
             }
         }
-        fence_async_proxy();
         asm volatile("bar.sync 1, %0;" ::"n"(ETHREADS) : "memory");
-        if (lane == 0) mbar_arrive(ready_bar);
         for (int i = etid; i < rs * P * BN; i += ETHREADS) {                // (slice, branch, channel)
             const int c = i % BN, sb = i / BN, br = sb % P, sl = sb / P, ch = (cg * L.rs + sl) * BN + c;
             const bool have = ch < p.C_out;
@@ -297,19 +308,25 @@ conv_tc_mod_kernel(const ModPlan L, const __grid_constant__ CUtensorMap idmap, c
             }
             int pop;
             asm volatile("ld.shared.b32 %0, [%1];" : "=r"(pop) : "r"(pops + 4u * i) : "memory");
-            const uint32_t ent = table + (uint32_t)((sl * BN + c) >> 1) * pair_bytes(P) + 4u * (c & 1);
-            const float v[4] = {sc, sh, (float)(32 * L.bcw - 2 * pop), pd};
-#pragma unroll
-            for (int k = 0; k < 4; ++k) asm volatile("st.shared.b32 [%0], %1;" ::"r"(ent + 32u * br + 8u * k), "r"(__float_as_uint(v[k])) : "memory");
+            const uint32_t pair = (uint32_t)((sl * BN + c) >> 1), odd = 4u * (c & 1), ent = table + pair * pair_bytes(P) + odd;
+            const int ct = sl * P + br;
+            store_const_row<false>(32 * L.bcw - 2 * pop, cexp + (uint32_t)((ct >> 2) * W_STAGE + c * ROWB), (c & 7) ^ (2 * (ct & 3)));
+            asm volatile("st.shared.b32 [%0], %1;" ::"r"(ent + 16u * br), "r"(__float_as_uint(sc)) : "memory");
+            asm volatile("st.shared.b32 [%0], %1;" ::"r"(ent + 16u * br + 8u), "r"(__float_as_uint(sh)) : "memory");
+            if (SHIFTED) asm volatile("st.shared.b32 [%0], %1;" ::"r"(pads + (pair * P + br) * 8u + odd), "r"(__float_as_uint(pd)) : "memory");
             if (br == 0) {
-                asm volatile("st.shared.b32 [%0], %1;" ::"r"(ent + 32u * P), "r"(__float_as_uint(slope)) : "memory");
-                asm volatile("st.shared.b32 [%0], %1;" ::"r"(ent + 32u * P + 8u), "r"(__float_as_uint(nb)) : "memory");
+                asm volatile("st.shared.b32 [%0], %1;" ::"r"(ent + 16u * P), "r"(__float_as_uint(slope)) : "memory");
+                asm volatile("st.shared.b32 [%0], %1;" ::"r"(ent + 16u * P + 8u), "r"(__float_as_uint(nb)) : "memory");
             }
         }
+        fence_async_proxy();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(ready_bar);
         asm volatile("bar.sync 1, %0;" ::"n"(ETHREADS) : "memory");
         const int team = (warp - FIRST_EPILOGUE) >> 2, quad = warp & 3, row = quad * 32 + lane;
         const uint32_t t_lane = tmem_base + ((uint32_t)(quad * 32) << 16);
         const int owords = p.C_out >> 5;
+        const bool want_bits = p.out != nullptr;
         const TileStep ts = make_tile_step(p, 0);
         bool ok = true;
         for (int n = team; n < parts; n += TEAMS) {
@@ -326,67 +343,79 @@ conv_tc_mod_kernel(const ModPlan L, const __grid_constant__ CUtensorMap idmap, c
                 row_window(p, ts, rc);
                 inside = rc.mask;
             }
-            if (!mbar_wait_warp(tfull_bar(team), (uint32_t)m & 1u, abort_flag, p.err, ERR_MOD_EPILOGUE)) break;
+            if (!mbar_wait_warp(tfull_bar(n % L.nbuf), (uint32_t)(n / L.nbuf) & 1u, abort_flag, p.err, ERR_MOD_EPILOGUE)) break;
             tc_fence_after();
             const uint32_t acc = t_lane + (uint32_t)((n % L.nbuf) * P * BN);
             const uint32_t tile = staging + (uint32_t)((team * NS + s) * TILE_BYTES) + (uint32_t)(row * ROW_BYTES);
             const uint32_t sw = BN == 64 ? (uint32_t)(row & 7) : (uint32_t)((row >> 1) & 3);
-            const uint32_t tb = table + (uint32_t)((n % rs) * (BN / 2)) * pair_bytes(P);
+            const uint32_t tb = table + (uint32_t)((n % rs) * (BN / 2)) * pair_bytes(P), pb = pads + (uint32_t)((n % rs) * (BN / 2) * P) * 8u;
             uint32_t words[BN / 32];
+            // (8 channels, branch) at a time; the next piece's accumulators are on their way while one is worked on (a load and
+            // its wait in turn were a third of a part's time)
+            uint32_t nv[8];
+            tc_ld8_nowait(acc, nv);
 #pragma unroll
-            for (int c16 = 0; c16 < BN / 16; ++c16) {
-                unsigned long long t[8];
+            for (int c8 = 0; c8 < BN / 8; ++c8) {
+                unsigned long long t[4];
 #pragma unroll
                 for (int br = 0; br < (PP ? PP : 1); ++br) {
                     int b = br;
                     do {
-                        uint32_t v[16];
-                        tc_ld16(acc + (uint32_t)(b * BN + c16 * 16), v);
+                        tc_wait_ld();
+                        pin_regs8(nv);
+                        unsigned long long dot[4];
 #pragma unroll
-                        for (int j = 0; j < 8; ++j) {
-                            const uint32_t ent = tb + (uint32_t)(c16 * 8 + j) * pair_bytes(P) + 32u * b;
-                            const uint4 ss = ld_shared_v4(ent), cd = ld_shared_v4(ent + 16u);
-                            unsigned long long dot = add2(bits2(v[2 * j], v[2 * j + 1]), bits2(cd.x, cd.y));
-                            if (SHIFTED && !((inside >> b) & 1u)) dot = bits2(cd.z, cd.w);
-                            const unsigned long long tp = add2(mul2(dot, bits2(ss.x, ss.y)), bits2(ss.z, ss.w));
+                        for (int j = 0; j < 4; ++j) dot[j] = bits2(nv[2 * j], nv[2 * j + 1]);
+                        const bool last_branch = b == P - 1;
+                        if (c8 < BN / 8 - 1 || !last_branch) {
+                            tc_ld8_nowait(acc + (uint32_t)(last_branch ? (c8 + 1) * 8 : (b + 1) * BN + c8 * 8), nv);
+                        } else {                                            // the accumulators are in registers
+                            tc_fence_before();
+                            __syncwarp();
+                            if (lane == 0) mbar_arrive(tempty_bar(n % L.nbuf));
+                        }
+#pragma unroll
+                        for (int j = 0; j < 4; ++j) {
+                            const uint4 ss = ld_shared_v4(tb + (uint32_t)(c8 * 4 + j) * pair_bytes(P) + 16u * b);
+                            if (SHIFTED && !((inside >> b) & 1u))
+                                asm volatile("ld.shared.b64 %0, [%1];" : "=l"(dot[j]) : "r"(pb + (uint32_t)((c8 * 4 + j) * P + b) * 8u) : "memory");
+                            const unsigned long long tp = add2(mul2(dot[j], bits2(ss.x, ss.y)), bits2(ss.z, ss.w));
                             t[j] = b == 0 ? tp : add2(t[j], tp);
                         }
                     } while (!PP && ++b < P);
                 }
-                if (c16 == BN / 16 - 1) {                                   // the accumulators are in registers
-                    tc_fence_before();
-                    __syncwarp();
-                    if (lane == 0) mbar_arrive(tempty_bar(team));
+                const uint32_t at = tile + (((uint32_t)c8 ^ sw) << 4);
+                uint32_t idw[4] = {0u, 0u, 0u, 0u}, ow[4], bits = 0;
+                if (HAS_ID) {
+                    const uint4 q = ld_shared_v4(at);
+                    idw[0] = q.x; idw[1] = q.y; idw[2] = q.z; idw[3] = q.w;
                 }
-                uint32_t bits = 0;
+                float2 yf[4];
+                uint4 sn[4];
 #pragma unroll
-                for (int h = 0; h < 2; ++h) {                               // 8 channels = 16 bytes of the maps
-                    const uint32_t at = tile + (((uint32_t)(2 * c16 + h) ^ sw) << 4);
-                    uint32_t idw[4] = {0u, 0u, 0u, 0u}, ow[4];
+                for (int j = 0; j < 4; ++j) {
+                    sn[j] = ld_shared_v4(tb + (uint32_t)(c8 * 4 + j) * pair_bytes(P) + 16u * P);               // slope, next bias
+                    unsigned long long u = t[j];
                     if (HAS_ID) {
-                        const uint4 q = ld_shared_v4(at);
-                        idw[0] = q.x; idw[1] = q.y; idw[2] = q.z; idw[3] = q.w;
+                        const float2 f = __half22float2(*reinterpret_cast<const __half2 *>(&idw[j]));
+                        u = add2(u, bits2(__float_as_uint(f.x), __float_as_uint(f.y)));
                     }
+                    const float2 uf = floats2(u), wf = floats2(mul2(bits2(sn[j].x, sn[j].y), u));
+                    const __half2 y2 = __floats2half2_rn(uf.x >= 0.f ? uf.x : wf.x, uf.y >= 0.f ? uf.y : wf.y);
+                    ow[j] = *reinterpret_cast<const uint32_t *>(&y2);
+                    yf[j] = __half22float2(y2);
+                }
+                st_shared_v4(at, ow[0], ow[1], ow[2], ow[3]);
+                if (want_bits) {
 #pragma unroll
                     for (int j = 0; j < 4; ++j) {
-                        const uint4 sn = ld_shared_v4(tb + (uint32_t)(c16 * 8 + 4 * h + j) * pair_bytes(P) + 32u * P);      // slope, next bias
-                        unsigned long long u = t[4 * h + j];
-                        if (HAS_ID) {
-                            const float2 f = __half22float2(*reinterpret_cast<const __half2 *>(&idw[j]));
-                            u = add2(u, bits2(__float_as_uint(f.x), __float_as_uint(f.y)));
-                        }
-                        const float2 uf = floats2(u), wf = floats2(mul2(bits2(sn.x, sn.y), u));
-                        const __half2 y2 = __floats2half2_rn(uf.x >= 0.f ? uf.x : wf.x, uf.y >= 0.f ? uf.y : wf.y);
-                        ow[j] = *reinterpret_cast<const uint32_t *>(&y2);
-                        const float2 yf = __half22float2(y2);
-                        const float2 v = floats2(add2(bits2(__float_as_uint(yf.x), __float_as_uint(yf.y)), bits2(sn.z, sn.w)));
-                        bits |= (v.x >= 0.f ? 1u : 0u) << (8 * h + 2 * j);
-                        bits |= (v.y >= 0.f ? 1u : 0u) << (8 * h + 2 * j + 1);
+                        const float2 v = floats2(add2(bits2(__float_as_uint(yf[j].x), __float_as_uint(yf[j].y)), bits2(sn[j].z, sn[j].w)));
+                        bits |= (v.x >= 0.f ? 1u : 0u) << (2 * j);
+                        bits |= (v.y >= 0.f ? 1u : 0u) << (2 * j + 1);
                     }
-                    st_shared_v4(at, ow[0], ow[1], ow[2], ow[3]);
                 }
-                if (c16 & 1) words[c16 >> 1] |= bits << 16;
-                else words[c16 >> 1] = bits;
+                if (c8 & 3) words[c8 >> 2] |= bits << (8 * (c8 & 3));
+                else words[c8 >> 2] = bits;
             }
             fence_async_proxy();                                            // the tile's generic stores -> the copy engine
             __syncwarp();
@@ -411,7 +440,7 @@ conv_tc_mod_kernel(const ModPlan L, const __grid_constant__ CUtensorMap idmap, c
         const uint32_t lane0 = lane == 0 ? 1u : 0u;
         const int total = my_tiles * kst;
         const TileStep ts = make_tile_step(p, (uint32_t)(BM * step));
-        if (grp == 0) write_unit_scales(lane_base + (uint32_t)SF_COL);
+        if (grp == 0) write_const_block(lane_base);
         RowCursor rc;
         rc.m = (uint32_t)idx * BM + (uint32_t)row;
         row_locate(p, rc);
@@ -470,12 +499,15 @@ conv_tc_mod_kernel(const ModPlan L, const __grid_constant__ CUtensorMap idmap, c
 
 // The plan for BN-channel slices, or false where the layer does not fit.
 template <int BN>
-bool make_plan(ModPlan &L, int &smem)
+bool make_plan(ModPlan &L, bool shifted, int &smem)
 {
     const ConvProblem &q = L.q;
     L.kst = (L.P * L.kwp + 7) / 8;
-    L.nbuf = 2 * L.P * BN + 32 * G <= SF_COL ? 2 : 1;
-    const int stages = (SF_COL - L.nbuf * L.P * BN) / 32;
+    // as many accumulator buffers as leave ring slots for a row tile and the next one's start (at least one per producer group)
+    const int want = L.kst + 1 < 3 ? 3 : (L.kst + 1 > 8 ? 8 : L.kst + 1);
+    L.nbuf = MAX_NBUF;
+    while (L.nbuf > 1 && (CB_COL - L.nbuf * L.P * BN) / 32 < (L.nbuf > 2 ? want : G)) --L.nbuf;
+    const int stages = (CB_COL - L.nbuf * L.P * BN) / 32;
     if (stages < G) return false;
     L.stages = stages < MAX_STAGES ? stages : MAX_STAGES;
     L.slices = (q.C_out + BN - 1) / BN;
@@ -486,7 +518,8 @@ bool make_plan(ModPlan &L, int &smem)
     for (int rs = 1; rs <= L.slices && rs <= 16; ++rs) {
         if (rs > 1 && L.kst > L.stages) break;               // the row tile's stages stay in the ring for all its parts
         const long pops = (long)rs * L.P * BN * 4, table = (long)rs * (BN / 2) * pair_bytes(L.P);
-        const long bytes = 1024 + rs * slice_bytes + staging + pops + (long)PF * SLOT_BYTES + table + 4L * L.units + 64;
+        const long pad = shifted ? (long)rs * (BN / 2) * L.P * 8 : 0, consts = (long)const_tiles(rs, L.P) * BN * ROWB;
+        const long bytes = 1024 + rs * slice_bytes + consts + pad + staging + pops + (long)PF * SLOT_BYTES + table + 4L * L.units + 64;
         if (bytes > MAX_SMEM) break;
         const int ng = (L.slices + rs - 1) / rs, per = sms / ng;
         if (per < 1) continue;
@@ -496,11 +529,13 @@ bool make_plan(ModPlan &L, int &smem)
         best = cost;
         L.rs = rs;
         L.ng = ng;
-        L.off_stage = (uint32_t)(rs * slice_bytes);
+        L.off_const = (uint32_t)(rs * slice_bytes);
+        L.off_stage = L.off_const + (uint32_t)consts;
         L.off_pop = L.off_stage + (uint32_t)staging;
         L.off_bits = L.off_pop + (uint32_t)pops;
         L.off_table = L.off_bits + (uint32_t)PF * SLOT_BYTES;
-        L.off_tab = (L.off_table + (uint32_t)table + 15u) & ~15u;
+        L.off_pad = L.off_table + (uint32_t)table;
+        L.off_tab = (L.off_pad + (uint32_t)pad + 15u) & ~15u;
         smem = (int)bytes;
     }
     return best >= 0;
@@ -536,16 +571,16 @@ int launch_mod(ModPlan &L, bool shifted, cudaStream_t stream)
     L.gw = L.bcw % 4 == 0 ? 4 : (L.bcw % 2 == 0 ? 2 : 1);
     q.err = device_error_word();
     if (L.P > 13 || q.C_out % 32 != 0 || q.M < 1) return BCNN_ERR_UNSUPPORTED;
-    if ((long)q.B * q.H * q.W * q.cw >= (1L << 31) || (long)q.kh * q.W * q.cw >= (1L << 27) || 32L * L.bcw > (1 << 16)) return BCNN_ERR_UNSUPPORTED;
+    if ((long)q.B * q.H * q.W * q.cw >= (1L << 31) || (long)q.kh * q.W * q.cw >= (1L << 27) || 32L * L.bcw > CONST_MAX) return BCNN_ERR_UNSUPPORTED;
     L.m_tiles = (q.M - 1) / BM + 1;
     int smem = 0;
-    if (L.P <= 3 && q.C_out > 32 && make_plan<64>(L, smem)) {
+    if (L.P <= 3 && q.C_out > 32 && make_plan<64>(L, shifted, smem)) {
         if (shifted) return launch_plan<64, 0, true>(L, smem, stream);
         if (L.P == 1) return launch_plan<64, 1, false>(L, smem, stream);
         if (L.P == 2) return launch_plan<64, 2, false>(L, smem, stream);
         return launch_plan<64, 0, false>(L, smem, stream);
     }
-    if (make_plan<32>(L, smem)) return shifted ? launch_plan<32, 0, true>(L, smem, stream) : launch_plan<32, 0, false>(L, smem, stream);
+    if (make_plan<32>(L, shifted, smem)) return shifted ? launch_plan<32, 0, true>(L, smem, stream) : launch_plan<32, 0, false>(L, smem, stream);
     return BCNN_ERR_UNSUPPORTED;
 }
 

@@ -104,6 +104,8 @@ __device__ __forceinline__ void write_const_block(uint32_t t_lane)
 }
 // first 32 bytes of row `row` of a constant weight tile (128-byte swizzled rows): 16 * digit for up to 28 elements - six as
 // often as it fits (96), then what is left down to below 8 - and 2 * digit for two more
+// (BIAS = false: the first block is zero, the MMA writes c alone)
+template <bool BIAS = true>
 __device__ __forceinline__ void store_const_row(int c, uint32_t row_addr, int xr)
 {
     const uint32_t a = (uint32_t)(c < 0 ? -c : c), neg = c < 0 ? 0x88888888u : 0u;
@@ -123,7 +125,7 @@ __device__ __forceinline__ void store_const_row(int c, uint32_t row_addr, int xr
         if (q == 3) w |= (c3 << 16) | (c4 << 20);
         o[q] = w ^ neg;
     }
-    st_shared_v4(row_addr + (uint32_t)((0 ^ xr) << 4), 0x7u, 0u, 0u, 0u);
+    st_shared_v4(row_addr + (uint32_t)((0 ^ xr) << 4), BIAS ? 0x7u : 0u, 0u, 0u, 0u);
     st_shared_v4(row_addr + (uint32_t)((1 ^ xr) << 4), o[0], o[1], o[2], o[3]);
 }
 // the constant MMA: accumulator = BIAS + c
