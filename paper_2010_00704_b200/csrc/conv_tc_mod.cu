@@ -19,6 +19,9 @@
 // is padded to an even number of words: two words per MMA.
 // Arithmetic (bit-exact against the oracle): t_p = dot_p * scale_p + shift_p, summed in branch order, + identity, PReLU,
 // fp16, sign of (stored value + next bias): one fp32 operation per step, no contraction.
+// "Part full" barriers form a ring of MAX_NBUF, not of the accumulator buffers in use: a parity wait for part n is right once
+// part n - MAX_NBUF is done, and the team has seen part n - TEAMS done (with one buffer and two teams the second team's first
+// wait would pass on the barrier's empty history).
 // Every mbarrier wait is bounded and reports through the device error word.
 #include "tc_slot.cuh"
 #include "tensor_map.cuh"
@@ -34,7 +37,7 @@ constexpr int ERR_MOD_PRODUCER = 171, ERR_MOD_ISSUER = 172, ERR_MOD_EPILOGUE = 1
 constexpr int G = 2;                      // producer groups of four warps
 constexpr int PF = 3;                     // packed-word stages in flight per producer thread
 constexpr int TEAMS = 2, NS = 3;          // epilogue teams of four warps; staging tiles per team
-constexpr int ISSUER = 0, LOADER = 1, STORER = 2 /* + team */, FIRST_PRODUCER = 4, FIRST_EPILOGUE = FIRST_PRODUCER + 4 * G;
+constexpr int ISSUER = 0, LOADER = 1, STORER = 2 /* + team */, FIRST_PRODUCER = STORER + TEAMS, FIRST_EPILOGUE = FIRST_PRODUCER + 4 * G;
 constexpr int THREADS = 32 * (FIRST_EPILOGUE + 4 * TEAMS);
 constexpr int PROD_THREADS = G * BM;
 constexpr int HALF_BYTES = PROD_THREADS * 16, SLOT_BYTES = 2 * HALF_BYTES;
@@ -121,6 +124,7 @@ conv_tc_mod_kernel(const ModPlan L, const __grid_constant__ CUtensorMap idmap, c
     const uint32_t bar0 = smem_u32(bars);
     auto full_bar = [&](int s) { return bar0 + 8u * s; };
     auto empty_bar = [&](int s) { return bar0 + 8u * (MAX_STAGES + s); };
+    static_assert(MAX_NBUF >= TEAMS, "ring of part-full barriers");
     auto tfull_bar = [&](int b) { return bar0 + 8u * (2 * MAX_STAGES + b); };
     auto tempty_bar = [&](int b) { return bar0 + 8u * (2 * MAX_STAGES + MAX_NBUF + b); };
     auto id_full = [&](int t, int s) { return bar0 + 8u * (2 * MAX_STAGES + 2 * MAX_NBUF + t * NS + s); };
@@ -172,7 +176,7 @@ conv_tc_mod_kernel(const ModPlan L, const __grid_constant__ CUtensorMap idmap, c
     pdl_wait();
     const uint32_t tmem_base = tmem_base_smem;
 
-    // part n = (row tile n / rs, slice n % rs); team n % 2, its n / 2-th part, staging tile (n / 2) % NS
+    // part n = (row tile n / rs, slice n % rs); team n % TEAMS, its m = n / TEAMS-th part, staging tile m % NS
     auto part_row = [&](int n) { return (idx + (n / rs) * step) * BM; };
     auto part_ch = [&](int n) { return (cg * L.rs + n % rs) * BN; };
 
@@ -216,7 +220,7 @@ conv_tc_mod_kernel(const ModPlan L, const __grid_constant__ CUtensorMap idmap, c
                     if (++slot == stages) { slot = 0; ring_phase ^= 1u; }
                 }
                 if (!ok) break;
-                tc_commit(tfull_bar(buf));
+                tc_commit(tfull_bar(n % MAX_NBUF));
                 if (++buf == L.nbuf) { buf = 0; buf_phase ^= 1u; }
                 if (++s == rs) { s = 0; slot0 = slot; ring_phase0 = ring_phase; }
             }
@@ -227,7 +231,7 @@ conv_tc_mod_kernel(const ModPlan L, const __grid_constant__ CUtensorMap idmap, c
         if (HAS_ID) {
             int issued = 0;
             for (int n = 0; n < parts; ++n, ++issued) {
-                const int team = n & 1, m = n >> 1, s = m % NS, lap = m / NS;
+                const int team = n % TEAMS, m = n / TEAMS, s = m % NS, lap = m / NS;
                 if (lap > 0 && !mbar_wait_warp(slot_free(team, s), (uint32_t)(lap - 1) & 1u, abort_flag, p.err, ERR_MOD_LOADER)) break;
                 if (lane == 0) {
                     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(id_full(team, s)), "r"((uint32_t)TILE_BYTES) : "memory");
@@ -240,13 +244,13 @@ conv_tc_mod_kernel(const ModPlan L, const __grid_constant__ CUtensorMap idmap, c
             // after a time-out elsewhere: copies still in flight must land before the CTA's shared memory goes away
             if (*abort_flag)
                 for (int n = issued > TEAMS * NS ? issued - TEAMS * NS : 0; n < issued; ++n)
-                    mbar_wait_warp(id_full(n & 1, (n >> 1) % NS), (uint32_t)((n >> 1) / NS) & 1u, abort_flag, nullptr, 0);
+                    mbar_wait_warp(id_full(n % TEAMS, (n / TEAMS) % NS), (uint32_t)(n / TEAMS / NS) & 1u, abort_flag, nullptr, 0);
         }
     } else if (warp < FIRST_PRODUCER) {
         // ------------------------------------------------------------------ output tiles of team warp - STORER
         const int team = warp - STORER;
         for (int n = team; n < parts; n += TEAMS) {
-            const int m = n >> 1, s = m % NS;
+            const int m = n / TEAMS, s = m % NS;
             if (!mbar_wait_warp(out_full(team, s), (uint32_t)(m / NS) & 1u, abort_flag, p.err, ERR_MOD_STORE)) break;
             if (lane == 0) {
                 asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.tile.bulk_group [%0, {%1, %2}], [%3];"
@@ -267,6 +271,21 @@ conv_tc_mod_kernel(const ModPlan L, const __grid_constant__ CUtensorMap idmap, c
         // with their bit counts, then the table.  Eight words are in flight per thread, and a channel's parameters before them.
         constexpr int ETHREADS = 128 * TEAMS;
         const int etid = tid - 32 * FIRST_EPILOGUE;
+        // parameters of a (slice, branch, channel) triple
+        struct Params { float sc, sh, pd, slope, nb; };
+        auto load_params = [&](int i) {
+            const int c = i % BN, sb = i / BN, br = sb % P, ch = (cg * L.rs + sb / P) * BN + c;
+            const bool have = i < rs * P * BN && ch < p.C_out;
+            const long at = (long)br * p.C_out + ch;
+            Params q;
+            q.sc = have ? __ldg(L.scale + at) : 0.f;
+            q.sh = have ? __ldg(L.shift + at) : 0.f;
+            q.pd = SHIFTED && have && L.pad_dot ? (float)__ldg(L.pad_dot + at) : 0.f;
+            q.slope = br == 0 && have ? __ldg(p.slope + ch) : 0.f;
+            q.nb = br == 0 && have && p.next_bias ? __ldg(p.next_bias + ch) : 0.f;
+            return q;
+        };
+        Params q = load_params(etid);
         {
             constexpr int WU = 8;
             const int total = rs * kst * BN * 8;
@@ -296,27 +315,19 @@ conv_tc_mod_kernel(const ModPlan L, const __grid_constant__ CUtensorMap idmap, c
         }
         asm volatile("bar.sync 1, %0;" ::"n"(ETHREADS) : "memory");
         for (int i = etid; i < rs * P * BN; i += ETHREADS) {                // (slice, branch, channel)
-            const int c = i % BN, sb = i / BN, br = sb % P, sl = sb / P, ch = (cg * L.rs + sl) * BN + c;
-            const bool have = ch < p.C_out;
-            const long at = (long)br * p.C_out + ch;
-            const float sc = have ? __ldg(L.scale + at) : 0.f, sh = have ? __ldg(L.shift + at) : 0.f;
-            const float pd = SHIFTED && have && L.pad_dot ? (float)__ldg(L.pad_dot + at) : 0.f;
-            float slope = 0.f, nb = 0.f;
-            if (br == 0 && have) {
-                slope = __ldg(p.slope + ch);
-                nb = p.next_bias ? __ldg(p.next_bias + ch) : 0.f;
-            }
+            const int c = i % BN, sb = i / BN, br = sb % P, sl = sb / P;
+            if (i != etid) q = load_params(i);
             int pop;
             asm volatile("ld.shared.b32 %0, [%1];" : "=r"(pop) : "r"(pops + 4u * i) : "memory");
             const uint32_t pair = (uint32_t)((sl * BN + c) >> 1), odd = 4u * (c & 1), ent = table + pair * pair_bytes(P) + odd;
             const int ct = sl * P + br;
             store_const_row<false>(32 * L.bcw - 2 * pop, cexp + (uint32_t)((ct >> 2) * W_STAGE + c * ROWB), (c & 7) ^ (2 * (ct & 3)));
-            asm volatile("st.shared.b32 [%0], %1;" ::"r"(ent + 16u * br), "r"(__float_as_uint(sc)) : "memory");
-            asm volatile("st.shared.b32 [%0], %1;" ::"r"(ent + 16u * br + 8u), "r"(__float_as_uint(sh)) : "memory");
-            if (SHIFTED) asm volatile("st.shared.b32 [%0], %1;" ::"r"(pads + (pair * P + br) * 8u + odd), "r"(__float_as_uint(pd)) : "memory");
+            asm volatile("st.shared.b32 [%0], %1;" ::"r"(ent + 16u * br), "r"(__float_as_uint(q.sc)) : "memory");
+            asm volatile("st.shared.b32 [%0], %1;" ::"r"(ent + 16u * br + 8u), "r"(__float_as_uint(q.sh)) : "memory");
+            if (SHIFTED) asm volatile("st.shared.b32 [%0], %1;" ::"r"(pads + (pair * P + br) * 8u + odd), "r"(__float_as_uint(q.pd)) : "memory");
             if (br == 0) {
-                asm volatile("st.shared.b32 [%0], %1;" ::"r"(ent + 16u * P), "r"(__float_as_uint(slope)) : "memory");
-                asm volatile("st.shared.b32 [%0], %1;" ::"r"(ent + 16u * P + 8u), "r"(__float_as_uint(nb)) : "memory");
+                asm volatile("st.shared.b32 [%0], %1;" ::"r"(ent + 16u * P), "r"(__float_as_uint(q.slope)) : "memory");
+                asm volatile("st.shared.b32 [%0], %1;" ::"r"(ent + 16u * P + 8u), "r"(__float_as_uint(q.nb)) : "memory");
             }
         }
         fence_async_proxy();
@@ -330,7 +341,7 @@ conv_tc_mod_kernel(const ModPlan L, const __grid_constant__ CUtensorMap idmap, c
         const TileStep ts = make_tile_step(p, 0);
         bool ok = true;
         for (int n = team; n < parts; n += TEAMS) {
-            const int m = n >> 1, s = m % NS, lap = m / NS;
+            const int m = n / TEAMS, s = m % NS, lap = m / NS;
             const int em = part_row(n) + row, ch0 = part_ch(n);
             if (HAS_ID) ok = mbar_wait_warp(id_full(team, s), (uint32_t)lap & 1u, abort_flag, p.err, ERR_MOD_IDENTITY);
             else if (lap > 0) ok = mbar_wait_warp(slot_free(team, s), (uint32_t)(lap - 1) & 1u, abort_flag, p.err, ERR_MOD_IDENTITY);
@@ -343,7 +354,7 @@ conv_tc_mod_kernel(const ModPlan L, const __grid_constant__ CUtensorMap idmap, c
                 row_window(p, ts, rc);
                 inside = rc.mask;
             }
-            if (!mbar_wait_warp(tfull_bar(n % L.nbuf), (uint32_t)(n / L.nbuf) & 1u, abort_flag, p.err, ERR_MOD_EPILOGUE)) break;
+            if (!mbar_wait_warp(tfull_bar(n % MAX_NBUF), (uint32_t)(n / MAX_NBUF) & 1u, abort_flag, p.err, ERR_MOD_EPILOGUE)) break;
             tc_fence_after();
             const uint32_t acc = t_lane + (uint32_t)((n % L.nbuf) * P * BN);
             const uint32_t tile = staging + (uint32_t)((team * NS + s) * TILE_BYTES) + (uint32_t)(row * ROW_BYTES);
@@ -574,13 +585,19 @@ int launch_mod(ModPlan &L, bool shifted, cudaStream_t stream)
     if ((long)q.B * q.H * q.W * q.cw >= (1L << 31) || (long)q.kh * q.W * q.cw >= (1L << 27) || 32L * L.bcw > CONST_MAX) return BCNN_ERR_UNSUPPORTED;
     L.m_tiles = (q.M - 1) / BM + 1;
     int smem = 0;
-    if (L.P <= 3 && q.C_out > 32 && make_plan<64>(L, shifted, smem)) {
+    // 64-channel parts; 32 where that leaves a multiprocessor less than two parts (a part is 2 us of latency per 64 channels)
+    if (L.P <= 3 && q.C_out > 32 && (long)L.m_tiles * ((q.C_out + 63) / 64) > sm_count() && make_plan<64>(L, shifted, smem)) {
         if (shifted) return launch_plan<64, 0, true>(L, smem, stream);
         if (L.P == 1) return launch_plan<64, 1, false>(L, smem, stream);
         if (L.P == 2) return launch_plan<64, 2, false>(L, smem, stream);
         return launch_plan<64, 0, false>(L, smem, stream);
     }
-    if (make_plan<32>(L, shifted, smem)) return shifted ? launch_plan<32, 0, true>(L, smem, stream) : launch_plan<32, 0, false>(L, smem, stream);
+    if (make_plan<32>(L, shifted, smem)) {
+        if (shifted) return launch_plan<32, 0, true>(L, smem, stream);
+        if (L.P == 1) return launch_plan<32, 1, false>(L, smem, stream);
+        if (L.P == 2) return launch_plan<32, 2, false>(L, smem, stream);
+        return launch_plan<32, 0, false>(L, smem, stream);
+    }
     return BCNN_ERR_UNSUPPORTED;
 }
 

@@ -2,7 +2,13 @@
 other GPU tests."""
 import pytest
 
-from test_gpu_block import bk, test_avgpool as check_avgpool, test_dwconv3x3_module as check_dwconv   # noqa: F401 (bk: a fixture)
+import numpy as np
+import torch
+
+from paper_2010_00704_b200 import synth
+from test_gpu_block import bk, dev, test_avgpool as check_avgpool, test_dwconv3x3_module as check_dwconv   # noqa: F401 (bk: a fixture)
+from test_gpu_block import test_fxf_as_shifted_branches as check_shifted, test_parallel_branches as check_branches   # noqa: F401
+from test_gpu_parity import run_conv
 
 pytestmark = pytest.mark.gpu
 
@@ -18,3 +24,113 @@ def test_dwconv_tiles(bk, oracle, shape):
 @pytest.mark.parametrize("shape", [(1, 1, 1, 8, 1, 1), (3, 14, 10, 24, 3, 2), (2, 12, 12, 8, 2, 4), (70, 28, 28, 64, 1, 2)])
 def test_avgpool_items(bk, oracle, shape):
     check_avgpool(bk, oracle, shape)
+
+
+# several parts per block: one accumulator buffer (nine taps), three (two branches), four (one branch); 32- and 64-channel parts,
+# a row tile that does not fit the ring (K = 13 * 512), the CUDA-core kernel behind the engine's limit (14 branches)
+@pytest.mark.parametrize("shape", [(20, 40, 40, 64, 64, 2), (20, 40, 40, 32, 96, 4), (26, 40, 40, 96, 64, 1), (1, 17, 19, 512, 64, 13), (1, 9, 15, 64, 32, 14)])
+def test_branches_many_parts(bk, oracle, shape):
+    check_branches(bk, oracle, shape, "full")
+
+
+@pytest.mark.parametrize("shape", [(16, 40, 40, 32, 64, 3), (2, 30, 31, 224, 96, 3)])
+def test_shifted_branches_many_parts(bk, oracle, shape):
+    check_shifted(bk, oracle, shape, "paper")
+
+
+# packing: pixels that are no whole number of passes (bias in registers or by remainder), NaN and -0, the replicated widths
+@pytest.mark.parametrize("shape", [(3, 7, 5, 32, 1), (2, 11, 13, 96, 1), (1, 9, 7, 1056, 1), (40, 28, 28, 160, 1), (2, 5, 9, 8, 4), (2, 9, 5, 64, 2), (1, 7, 9, 128, 3),
+                                   (1, 5, 7, 96, 2), (1, 3, 4, 48, 4)])
+def test_pack_shapes(bk, oracle, shape):
+    B, H, W, C, R = shape
+    rng = np.random.default_rng(9500 + sum(shape))
+    x, bias = synth.real_input(rng, (B, H, W, C)), synth.real_input(rng, (C * R,))
+    x.reshape(-1)[::7], x.reshape(-1)[::11] = -0.0, np.nan
+    for b in (bias, None):
+        out = torch.empty(B * H * W * C * R // 8, dtype=torch.uint8, device="cuda")
+        bk.bcnn_pack(dev(x), None if b is None else dev(b), out, B, H, W, C, R)
+        torch.cuda.synchronize()
+        want = oracle.binarize(x, b if b is not None else np.zeros(C * R, np.float32), R)
+        assert np.array_equal(synth.unpack_bits(out.cpu().numpy().reshape(B, H, W, C * R // 8)), want)
+
+
+# tiled fp32 product (many images) and one warp per output (few), ragged in every direction
+@pytest.mark.parametrize("shape", [(300, 200, 1000), (97, 36, 3000), (3, 2048, 100), (1, 8, 1)])
+def test_fc_shapes(bk, oracle, shape):
+    B, C, N = shape
+    rng = np.random.default_rng(9600 + sum(shape))
+    x, w, bias = (rng.standard_normal(s).astype(np.float32) for s in ((B, C), (N, C), (N,)))
+    out = torch.empty(B * N, dtype=torch.float32, device="cuda")
+    for b in (bias, None):
+        bk.bcnn_fc(dev(x), dev(w), None if b is None else dev(b), out, B, C, N)
+        torch.cuda.synchronize()
+        ref = x.astype(np.float64) @ w.astype(np.float64).T + (0 if b is None else b)
+        mag = np.abs(x.astype(np.float64)) @ np.abs(w.astype(np.float64)).T + np.abs(bias)
+        assert np.all(np.abs(out.cpu().numpy().reshape(B, N) - ref) <= (C + 76) * 2.0 ** -24 * mag)
+
+
+# pooling in pixel slices: fewer pixels than slices, channels that are no whole block
+@pytest.mark.parametrize("shape", [(2, 1, 1, 8), (3, 5, 7, 264), (1, 14, 14, 2048), (5, 3, 3, 24)])
+def test_gap_shapes(bk, oracle, shape):
+    B, H, W, C = shape
+    x = np.random.default_rng(9700 + sum(shape)).standard_normal(shape).astype(np.float16)
+    out = torch.empty(B * C, dtype=torch.float32, device="cuda")
+    bk.bcnn_gap(dev(x.view(np.uint8).reshape(-1)), out, B, H, W, C)
+    torch.cuda.synchronize()
+    mag = np.abs(x.astype(np.float64)).mean(axis=(1, 2))
+    assert np.all(np.abs(out.cpu().numpy().reshape(B, C) - oracle.gap(x)) <= (H * W + 15) * 2.0 ** -24 * mag + 1e-30)
+
+
+# B, H, W, C_in, C_out, k, stride, pad: wide pointwise engine with one and two resident slices (the latter from a dozen row tiles per
+# block on), K = 128, 256, 512; halo-tile engine with two and three tiles in flight and 128 channels
+@pytest.mark.parametrize("engine,shape", [("tc_pn", (1, 60, 70, 128, 128, 1, 1, 0)), ("tc_pn", (2, 352, 360, 128, 256, 1, 1, 0)), ("tc_pn", (1, 20, 21, 256, 384, 1, 1, 0)),
+                                          ("tc_pn", (1, 15, 9, 512, 1024, 1, 1, 0)), ("tc_c3", (9, 64, 64, 64, 64, 3, 1, 1)), ("tc_c3", (9, 64, 64, 32, 128, 3, 1, 1)),
+                                          ("tc_c3", (5, 64, 64, 64, 128, 3, 2, 1)), ("tc_i8", (1, 700, 1, 1152, 96, 1, 1, 0)), ("lop3", (1, 9, 11, 96, 70, 1, 1, 0))])
+def test_engine_edges(bk, oracle, engine, shape):
+    B, H, W, Ci, Co, k, stride, pad = shape
+    rng = np.random.default_rng(9800 + sum(shape))
+    x, w = synth.pm1(rng, (B, H, W, Ci)), synth.pm1(rng, (Co, k, k, Ci))
+    if H * W > 100000:                                  # the packed checker's sums on a sample of rows
+        thr = synth.thresholds(rng, Ci, Co)
+        got = run_conv(bk, x, w, thr, stride, pad, engine)
+        rows = rng.integers(0, H * W, 400)
+        want = oracle.threshold(x.reshape(-1, Ci)[rows].astype(np.int32) @ w.reshape(Co, Ci).astype(np.int32).T, thr)
+        assert np.array_equal(np.asarray(got).reshape(-1, Co)[rows], want)
+        return
+    acc = oracle.conv2d(x, w, stride, pad)
+    thr = synth.thresholds(rng, k * k * Ci, Co) if Co % 32 == 0 else None
+    want = acc if thr is None else oracle.threshold(acc, thr)
+    assert np.array_equal(run_conv(bk, x, w, thr, stride, pad, engine), want)
+
+
+# prepared weights: tiles 256, 128 and 64 wide by the estimate, int32 rows of any width
+@pytest.mark.parametrize("M,N,K,fused", [(40000, 256, 2304, True), (12544, 512, 1184, True), (3000, 128, 800, True), (700, 473, 704, False), (20000, 257, 512, False), (5000, 1000, 2400, False)])
+def test_prepared_widths(bk, oracle, M, N, K, fused):
+    rng = np.random.default_rng(M + N + K)
+    A, W = synth.random_bits(rng, (M, K // 8)), synth.random_bits(rng, (N, K // 8))
+    thr = synth.thresholds(rng, K, N) if fused else None
+    prep = torch.empty(bk.bcnn_prepared_weights_bytes(N, K), dtype=torch.uint8, device="cuda")
+    bk.bcnn_prepare_weights(dev(W), prep, N, K)
+    out = torch.empty(M * N // 8 if fused else M * N * 4, dtype=torch.uint8, device="cuda")
+    bk.bcnn_gemm_b1_prepared(dev(A), prep, None if thr is None else dev(thr), out, M, N, K)
+    torch.cuda.synchronize()
+    acc = synth.unpack_bits(A).astype(np.float32) @ synth.unpack_bits(W).astype(np.float32).T       # exact: |sums| < 2^24
+    if fused:
+        assert np.array_equal(synth.unpack_bits(out.cpu().numpy().reshape(M, N // 8)), np.where(acc >= thr, 1, -1))
+    else:
+        assert np.array_equal(out.cpu().numpy().view(np.int32).reshape(M, N), acc.astype(np.int32))
+    assert bk.bcnn_device_error() == 0
+
+
+# the stem's plain kernel and its table, on both sides of the line between them (148 * 1792 pixels)
+@pytest.mark.parametrize("shape", [(1, 9, 7), (1, 448, 592), (1, 450, 592)])
+def test_stem_sizes(bk, oracle, shape):
+    B, H, W = shape
+    rng = np.random.default_rng(9900 + sum(shape))
+    x, bias, w = synth.real_input(rng, (B, H, W, 4)), synth.real_input(rng, (32,)), synth.pm1(rng, (32, 1, 1, 32))
+    thr = synth.thresholds(rng, 32, 32)
+    out = torch.empty(B * H * W * 4, dtype=torch.uint8, device="cuda")
+    bk.bcnn_stem_fused(dev(x), dev(bias), dev(synth.pack_bits(w)), dev(thr), out, B, H, W, 4, 8, 32)
+    torch.cuda.synchronize()
+    want = oracle.threshold(oracle.conv2d(oracle.binarize(x, bias, 8), w, 1, 0), thr)
+    assert np.array_equal(synth.unpack_bits(out.cpu().numpy().reshape(B, H, W, 4)), want)
