@@ -80,11 +80,11 @@ int make_conv_problem(ConvProblem &p, const void *x, const void *w, const int32_
 //     engine (a row tile expanded once for all resident weight slices; 1.5 - 3x the weight-stationary engine);
 //   * 3x3 layers (stride 1 or 2) on 32 or 64 input channels with C_out <= 128, packed output, whose 8 x 16 output tiles
 //     are at least three quarters full: halo-tile tcgen05 engine (input tiles by tiled TMA copies);
-//   * C_out >= 256, or weights too large to keep expanded in shared memory: streaming tcgen05 engine;
 //   * 1x1 layer with C_in = 32 and C_out <= 32 (one XOR + popcount per output): CUDA-core pointwise kernel;
-//   * C_out <= 128 with K >= 64, and wider layers with K <= 1152 and M >= 32768 (in 128-channel slices):
-//     weight-stationary tcgen05 engine;
+//   * many rows of C_out <= 128 with K >= 64, or of wider layers with K <= 2304 (in 128-channel slices): weight-stationary
+//     tcgen05 engine;
 //   * other K = 32 layers: register-fed warp-level int8 engine;
+//   * everything else: streaming tcgen05 engine;
 //   * CUDA-core engine: the smallest calls with K <= 256;
 //   * the single-bit mma.sync engine never wins and serves as a fallback.
 int auto_engine(const ConvProblem &p)
@@ -99,10 +99,19 @@ int auto_engine(const ConvProblem &p)
         if (4L * p.OH * p.OW >= 3L * covered) return BCNN_ENGINE_TC_C3;
     }
     if (conv_lop3_pointwise_k32(p)) return BCNN_ENGINE_LOP3;
-    if (p.C_out <= 128 && p.K >= 64 && conv_tc_ws_supports(p)) return BCNN_ENGINE_TC_WS;
-    // wider layers in slices of 128 output channels: ahead of the streaming engine while K is short and there are
-    // enough rows to share one slice's weights among many CTAs (K = 2304 ties, K = 512 at M = 12544 loses)
-    if (p.C_out > 128 && p.K <= 1152 && p.M >= 32768 && conv_tc_ws_supports(p)) return BCNN_ENGINE_TC_WS;
+    // Up to 128 output channels: the weight-stationary engine, unless its CTAs would expand all the weights for less than two
+    // waves of 64-wide tiles of the streaming engine (3x3 128 -> 128: 7.6 against 5.0 us at M = 784, 8.3 against 7.0 at 12544;
+    // 1x1 256 -> 64 at M = 81000: 7.5 against 12.1)
+    const long waves64 = (((p.M + 127L) / 128) * ((p.C_out + 63) / 64) + sm_count() - 1) / sm_count();
+    const bool small = conv_tc_i8_supports(p) && (waves64 <= 1 || (waves64 <= 2 && p.K >= 1024));
+    if (p.C_out <= 128 && p.K >= 64) {
+        if (small) return BCNN_ENGINE_TC_I8;
+        if (conv_tc_ws_supports(p)) return BCNN_ENGINE_TC_WS;
+    }
+    // wider layers in slices of 128 output channels: ahead of the streaming engine while the weights fit and there are enough row
+    // tiles to share one slice's weights (4096 x 4096 x 2304 int32: 33.3 against 38.8 us, 3x3 256 -> 256 at M = 50176: 20.8
+    // against 27.3; 1024 x 1024 x 512: 7.9 against 5.5)
+    if (p.C_out > 128 && p.K <= 2304 && ((p.M + 127L) / 128) * ((p.C_out + 127) / 128) >= 2L * sm_count() && conv_tc_ws_supports(p)) return BCNN_ENGINE_TC_WS;
     if (p.C_out <= 64 && conv_mma_s8_supports(p)) return BCNN_ENGINE_MMA_S8;
     if (conv_tc_i8_supports(p)) return BCNN_ENGINE_TC_I8;
     if (conv_mma_b1_supports(p)) return BCNN_ENGINE_MMA_B1;
@@ -394,11 +403,15 @@ int bcnn_prepared_preferred(int B, int H, int W, int C_in, int C_out, int kh, in
     // Measured: streaming prepared weights wins wherever AUTO would expand them on every call - the streaming engine always,
     // the weight-stationary one except on many rows of a short K, where its expansion is spread thin (56x56 64 -> 128 /2 at
     // batch 256, M = 200704, K = 576: 16.1 against 18.2 us; K = 1152: 19.7 against 19.0; M = 784: 6.5 against 4.0).  The pointwise
-    // and halo-tile engines keep their layers, except the smallest: they expand their weights at the start.
+    // and halo-tile engines keep their layers, all but the smallest with many weights: they expand those at the start.
     if (!conv_tc_pre_supports(p)) return 0;
     switch (auto_engine(p)) {
-    case BCNN_ENGINE_TC_PW: case BCNN_ENGINE_TC_PN: case BCNN_ENGINE_TC_C3:
-        // 1x1 512 -> 512: 5.0 against 3.7 us at M = 49, 6.5 against 8.3 at 12544; 3x3 64 -> 64: 4.4 against 4.0 at 3136
+    case BCNN_ENGINE_TC_C3:
+        if (p.C_out <= 64) return 0;
+        [[fallthrough]];
+    case BCNN_ENGINE_TC_PW: case BCNN_ENGINE_TC_PN:
+        // 3x3 64 -> 128 /2: 5.0 against 4.0 us at M = 784, 15.4 against 18.2 at 200704; 1x1 512 -> 512: 5.0 against 3.7 us at M = 49,
+        // 6.5 against 8.3 at 12544; 128 -> 128: 3.9 against 3.3 at 784
         return p.M <= 4096 && ((p.M + 127) / 128) * ((p.C_out + 63) / 64) <= sm_count() ? 1 : 0;
     case BCNN_ENGINE_TC_WS: return p.K >= 1024 || p.M < 98304 ? 1 : 0;
     case BCNN_ENGINE_LOP3: return p.K <= 64 ? 0 : 1;

@@ -166,36 +166,55 @@ conv_tc_c3_kernel(const ConvProblem p, const C3Geom g, const __grid_constant__ C
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
     for (int c = tid; c < BN; c += C::THREADS) asm volatile("st.shared.b32 [%0], %1;" ::"r"(pops + 4u * c), "r"(0) : "memory");
-    pdl_wait();
-    __syncthreads();
-    // ---- one-off: expanded weights and the channels' bit counts.  K position e of the MMAs = channel word e / 10, tap e % 10
-    // (global weight word tap * CW + channel word) -> stage e / 8, 16-byte piece e % 8; MMA row `row` carries channel ch
-    for (int idx = tid; idx < KT * 8 * BN; idx += C::THREADS) {
-        const int e = idx % (KT * 8), row = idx / (KT * 8), tap = e % UWORDS, cword = e / UWORDS;
-        const int ch = (row & ~31) + channel_of_column(row & 31);
-        const bool live = tap < TAPS && cword < CW && ch < cn;
-        const uint32_t w = live ? __ldg(p.w + (long)ch * C::KW + tap * CW + cword) : 0u;
-        expand_store_w4(w, live, wexp + (uint32_t)(e >> 3) * C::W_TILE_BYTES + (uint32_t)row * ROWB, row & 7, e & 7);
-        if (live) asm volatile("red.shared.add.u32 [%0], %1;" ::"r"(pops + 4u * row), "r"(__popc(w)) : "memory");
-    }
+    if (tid == 64) asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&xmap)) : "memory");
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
     pdl_trigger();
+    pdl_wait();
+    // The loader warps start now: the first halo tiles arrive while the other warps expand the weights (0.5 us of a small layer's
+    // 4).  The other warps meet at a named barrier of their own; everybody meets again at the end.
+    const bool is_loader = warp >= C::FIRST_LOADER_WARP && warp < C::FIRST_PRODUCER_WARP;
     const uint32_t tmem_base = tmem_base_smem;
-    // constants K - 2 popc - thr (thr clamped to +-(K + 1))
-    for (int row = tid; row < BN; row += C::THREADS) {
-        const int ch = (row & ~31) + channel_of_column(row & 31);
-        int pop;
-        asm volatile("ld.shared.b32 %0, [%1];" : "=r"(pop) : "r"(pops + 4u * row) : "memory");
-        const int t = ch < cn ? __ldg(p.thr + ch) : 0;
-        store_const_row(p.K - 2 * pop - max(min(t, p.K + 1), -p.K - 1), cexp + (uint32_t)row * ROWB, row & 7);
+    if (!is_loader) {
+        constexpr int NW = C::THREADS - 64, WTOTAL = KT * 8 * BN, WU = (WTOTAL + NW - 1) / NW;       // (threads 64 .. 127 are the loaders)
+        const int wt = tid < 64 ? tid : tid - 64;
+        auto sync_workers = [&]() { asm volatile("bar.sync 1, %0;" ::"n"(NW) : "memory"); };
+        // ---- one-off: expanded weights and the channels' bit counts.  K position e of the MMAs = channel word e / 10, tap e % 10
+        // (global weight word tap * CW + channel word) -> stage e / 8, 16-byte piece e % 8; MMA row `row` carries channel ch.
+        // All of a thread's words, and its threshold, are requested before the first is used.
+        const int my_ch = (wt & ~31) + channel_of_column(wt & 31);
+        const int thr = wt < BN && my_ch < cn ? __ldg(p.thr + my_ch) : 0;
+        uint32_t w[WU];
+#pragma unroll
+        for (int u = 0; u < WU; ++u) {
+            const int idx = wt + u * NW, e = idx % (KT * 8), row = idx / (KT * 8), tap = e % UWORDS, cword = e / UWORDS;
+            const int ch = (row & ~31) + channel_of_column(row & 31);
+            w[u] = idx < WTOTAL && tap < TAPS && cword < CW && ch < cn ? __ldg(p.w + (long)ch * C::KW + tap * CW + cword) : 0u;
+        }
+#pragma unroll
+        for (int u = 0; u < WU; ++u) {
+            const int idx = wt + u * NW, e = idx % (KT * 8), row = idx / (KT * 8), tap = e % UWORDS, cword = e / UWORDS;
+            const int ch = (row & ~31) + channel_of_column(row & 31);
+            if (idx >= WTOTAL) break;
+            const bool live = tap < TAPS && cword < CW && ch < cn;
+            expand_store_w4(w[u], live, wexp + (uint32_t)(e >> 3) * C::W_TILE_BYTES + (uint32_t)row * ROWB, row & 7, e & 7);
+            if (live) asm volatile("red.shared.add.u32 [%0], %1;" ::"r"(pops + 4u * row), "r"(__popc(w[u])) : "memory");
+        }
+        if (warp >= C::FIRST_PRODUCER_WARP && warp < C::FIRST_PRODUCER_WARP + 4) write_const_block(tmem_base + ((uint32_t)((warp & 3) * 32) << 16));
+        tc_fence_before();
+        sync_workers();
+        tc_fence_after();
+        if (wt < BN) {                  // constants K - 2 popc - thr (thr clamped to +-(K + 1))
+            int pop;
+            asm volatile("ld.shared.b32 %0, [%1];" : "=r"(pop) : "r"(pops + 4u * wt) : "memory");
+            store_const_row(p.K - 2 * pop - max(min(thr, p.K + 1), -p.K - 1), cexp + (uint32_t)wt * ROWB, wt & 7);
+        }
+        fence_async_proxy();
+        tc_fence_before();
+        sync_workers();
+        tc_fence_after();
     }
-    if (warp >= C::FIRST_PRODUCER_WARP && warp < C::FIRST_PRODUCER_WARP + 4) write_const_block(tmem_base + ((uint32_t)((warp & 3) * 32) << 16));
-    fence_async_proxy();
-    tc_fence_before();
-    __syncthreads();
-    tc_fence_after();
 
     // A role's tiles are a fixed number of tiles apart: image and tile coordinates follow by carries (two divisions per tile
     // were a third of an epilogue warp's time).

@@ -111,8 +111,8 @@ conv_tc_pn_kernel(const ConvProblem p, const PnPlan plan)
         abort_flag_smem = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    pdl_wait();
     __syncthreads();
+    pdl_wait();
     // The loader warps start now: the first row tiles arrive while the other warps expand the weights (these kernels
     // run for 10 - 40 us; the weights' expansion and the first copy's latency are 1.5 - 2 us each).  The other warps meet
     // at a named barrier of their own; everybody meets again at the end.

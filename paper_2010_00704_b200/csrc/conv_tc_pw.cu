@@ -146,34 +146,38 @@ conv_tc_pw_kernel(const ConvProblem p)
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base_smem)), "r"(512u) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
-    pdl_wait();
-    // ---- one-off: expanded weights and constant rows; MMA row `row` carries channel 32 * (row / 32) + channel_of_column(row % 32)
-    for (int row = tid; row < BN; row += C::THREADS) {
-        const int ch = (row & ~31) + channel_of_column(row & 31);
-        const bool have = ch < cn;
-        const uint32_t row_addr = wexp + (uint32_t)row * ROWB;
-        int pop = 0;
-#pragma unroll
-        for (int e = 0; e < pw_words(KW); ++e) {
-            const bool live = e < KW && have;
-            const uint32_t w = live ? __ldg(p.w + (long)ch * KW + e) : 0u;
-            pop += __popc(w);
-            expand_store_w4(w, live, row_addr, row & 7, e);
-        }
-        // thr clamped to +-(K + 1): beyond that bound the decision is constant
-        const int t = have ? __ldg(p.thr + ch) : 0;
-        store_const_row(have ? p.K - 2 * pop - max(min(t, p.K + 1), -p.K - 1) : 0, cexp + (uint32_t)row * ROWB, row & 7);
-    }
-    fence_async_proxy();
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
     pdl_trigger();
+    pdl_wait();
+    // The loader warp starts now: the first rows arrive while the other warps expand the weights.  The other warps meet at a named
+    // barrier of their own; everybody meets again at the end.
     const uint32_t tmem_base = tmem_base_smem;
-    if (warp >= C::FIRST_PRODUCER_WARP && warp < C::FIRST_PRODUCER_WARP + 4) write_const_block(tmem_base + ((uint32_t)((warp & 3) * 32) << 16));
-    tc_fence_before();
-    __syncthreads();
-    tc_fence_after();
+    if (warp != C::LOADER_WARP) {
+        // ---- one-off: expanded weights and constant rows; MMA row `row` carries channel 32 * (row / 32) + channel_of_column(row % 32)
+        for (int row = tid - 32 * C::FIRST_PRODUCER_WARP; row >= 0 && row < BN; row += C::THREADS) {
+            const int ch = (row & ~31) + channel_of_column(row & 31);
+            const bool have = ch < cn;
+            const uint32_t row_addr = wexp + (uint32_t)row * ROWB;
+            // thr clamped to +-(K + 1): beyond that bound the decision is constant
+            const int t = have ? __ldg(p.thr + ch) : 0;
+            int pop = 0;
+#pragma unroll
+            for (int e = 0; e < pw_words(KW); ++e) {
+                const bool live = e < KW && have;
+                const uint32_t w = live ? __ldg(p.w + (long)ch * KW + e) : 0u;
+                pop += __popc(w);
+                expand_store_w4(w, live, row_addr, row & 7, e);
+            }
+            store_const_row(have ? p.K - 2 * pop - max(min(t, p.K + 1), -p.K - 1) : 0, cexp + (uint32_t)row * ROWB, row & 7);
+        }
+        if (warp >= C::FIRST_EPILOGUE_WARP && warp < C::FIRST_EPILOGUE_WARP + 4) write_const_block(tmem_base + ((uint32_t)((warp & 3) * 32) << 16));
+        fence_async_proxy();
+        tc_fence_before();
+        asm volatile("bar.sync 1, %0;" ::"n"(C::THREADS - 32) : "memory");
+        tc_fence_after();
+    }
 
     if (warp < NSLOT) {
         // ------------------------------------------------------------------ MMA issuer of slot `warp`
