@@ -245,10 +245,10 @@ def run_probes():
     out = {}
     ms, macs, derr = dbl(0), dbl(0), i32(0)
     for n in (256, 128, 64, 32):
-        st = lib.probe_tcgen05_i8(n, 4000 * (256 // n), ctypes.byref(ms), ctypes.byref(macs), ctypes.byref(derr))
+        st = lib.probe_tcgen05_f4(n, 4000 * (256 // n), ctypes.byref(ms), ctypes.byref(macs), ctypes.byref(derr))
         if st != 0 or derr.value != 0:
             raise SystemExit(f"tcgen05 probe failed: status {st}, device error {derr.value}")
-        out[f"tcgen05_i8_n{n}"] = 2 * macs.value / (ms.value / 1e3) / 1e12
+        out[f"tcgen05_mxf4_n{n}"] = 2 * macs.value / (ms.value / 1e3) / 1e12
     for mode, name in ((0, "mma_sync_b1_and_popc"), (1, "mma_sync_b1_xor_popc"), (2, "mma_sync_s8")):
         st = lib.probe_mma_sync(mode, 2000 if mode < 2 else 20000, ctypes.byref(ms), ctypes.byref(macs))
         if st != 0:
@@ -510,27 +510,27 @@ def run_gpu(args):
             dist.destroy_process_group()
         return 0
 
-    # Tensor peak: the tcgen05.mma kind::i8 rate measured in this process by the tensor-memory-resident probe
-    # (N = 256 instructions back to back).  Beside it, 2 x the measured bf16 GEMM peaks (the nominal 2:1 ratio of
-    # the dense 8-bit and 16-bit pipes): burst for launches timed alone at the maximum clock, sustained for a warm,
+    # Tensor peak: the tcgen05.mma kind::mxf4 rate measured in this process by the tensor-memory-resident probe
+    # (N = 256 instructions back to back).  Beside it, 4 x the measured bf16 GEMM peaks (the nominal 4:1 ratio of
+    # the dense 4-bit and 16-bit pipes): burst for launches timed alone at the maximum clock, sustained for a warm,
     # power-limited GPU.  Which of the two applies to the per-launch times is decided by the clocks sampled
     # while those launches ran.
-    tensor_peak = probes["tcgen05_i8_n256"]
-    peak_alt = {"2x_bf16_burst": 2.0 * peaks["bf16_tflops"], "2x_bf16_sustained": 2.0 * peaks["bf16_tflops_sustained"]}
+    tensor_peak = probes["tcgen05_mxf4_n256"]
+    peak_alt = {"4x_bf16_burst": 4.0 * peaks["bf16_tflops"], "4x_bf16_sustained": 4.0 * peaks["bf16_tflops_sustained"]}
     def regime_of(c):
         if not c or not c.get("sm_mhz") or not c.get("sm_max_mhz"):
             return "unknown"
         return "burst" if c["sm_mhz"] >= 0.95 * c["sm_max_mhz"] else "sustained"
     regime = regime_of(clocks_k)
-    alt_key = "2x_bf16_sustained" if regime == "sustained" else "2x_bf16_burst"
+    alt_key = "4x_bf16_sustained" if regime == "sustained" else "4x_bf16_burst"
     engines = [chain.engine_name(i) for i in range(nl)]   # "stem": the first layer runs inside the stem kernel (slot 0 of per_ms)
-    kernel_of = {"tc_i8": "conv_tc_i8_kernel (tcgen05 kind::i8)", "mma_s8": "conv_mma_s8_kernel (mma.sync u8)",
+    kernel_of = {"tc_i8": "conv_tc_i8_kernel (tcgen05 kind::mxf4)", "mma_s8": "conv_mma_s8_kernel (mma.sync u8)",
                  "mma_b1": "conv_mma_b1_kernel (mma.sync b1)",
-                 "tc_ws": "conv_tc_ws_kernel (tcgen05 kind::i8, weights resident in shared memory)",
-                 "tc_pw": "conv_tc_pw_kernel (tcgen05 kind::i8, pointwise layers, bulk-copied rows)",
-                 "tc_pre": "conv_tc_pre_kernel (tcgen05 kind::i8, prepared weights streamed by TMA)",
-                 "tc_c3": "conv_tc_c3_kernel (tcgen05 kind::i8, 3x3 layers on 32/64 channels, halo tiles by TMA)",
-                 "tc_pn": "conv_tc_pn_kernel (tcgen05 kind::i8, pointwise layers with K = 256 / 512, resident weight slices)",
+                 "tc_ws": "conv_tc_ws_kernel (tcgen05 kind::mxf4, weights resident in shared memory)",
+                 "tc_pw": "conv_tc_pw_kernel (tcgen05 kind::mxf4, pointwise layers, bulk-copied rows)",
+                 "tc_pre": "conv_tc_pre_kernel (tcgen05 kind::mxf4, prepared weights streamed by TMA)",
+                 "tc_c3": "conv_tc_c3_kernel (tcgen05 kind::mxf4, 3x3 layers on 32/64 channels, halo tiles by TMA)",
+                 "tc_pn": "conv_tc_pn_kernel (tcgen05 kind::mxf4, pointwise layers with K = 128 / 256 / 512, resident weight slices)",
                  "lop3": "conv_k32_kernel (CUDA-core xor + popc)"}
     lay_ms = [float(per_ms[0]) if engines[i] == "stem" else float(per_ms[i + 1]) for i in range(nl)]
     per_layer = []
@@ -567,8 +567,8 @@ def run_gpu(args):
     roofline = {
         "kernel": groups[0]["kernel"], "launch": f"{lt.name}: M={lt.M(B)} N={lt.C_out} K={lt.K}",
         "bound": "tensor", "achieved": top_tops, "peak": tensor_peak, "unit": "TOP/s", "frac": top_tops / tensor_peak,
-        "peak_source": "tcgen05.mma kind::i8 (M=128, N=256, K=32, A in tensor memory) issued back to back, measured in this "
-                       f"process by bench_probes.cu; peak_alt = 2 x the {peaks['source']} bf16 GEMM peaks (MEASURED_PEAKS.json), "
+        "peak_source": "tcgen05.mma kind::mxf4 (M=128, N=256, K=64, A in tensor memory) issued back to back, measured in this "
+                       f"process by bench_probes.cu; peak_alt = 4 x the {peaks['source']} bf16 GEMM peaks (MEASURED_PEAKS.json), "
                        f"of {peaks['source']}",
         "peak_alt": peak_alt, "frac_alt": {k: top_tops / v for k, v in peak_alt.items()},
         "regime": regime, "frac_of_regime_peak": top_tops / peak_alt[alt_key],

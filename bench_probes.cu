@@ -1,9 +1,8 @@
 // Instruction-throughput probes of the inner-product choices on sm_100a, used by bench.py for the roofline
 // denominators.  No global-memory traffic inside the timed kernels:
 //   * mma.sync .b1 (and.popc / xor.popc), mma.sync .s8 m16n8k32 and CUDA-core xor + popc: register-resident;
-//   * tcgen05.mma kind::i8: A operand resident in tensor memory, B in shared memory, int32 accumulators in tensor
-//     memory; one thread per SM issues M = 128, K = 32 instructions of width N back to back (N = 256 runs at the
-//     pipe's rate, narrower instructions show the issue-bound regime).
+//   * tcgen05.mma kind::mxf4 (4-bit operands, unit block scales): A operand resident in tensor memory, B in shared memory,
+//     fp32 accumulators in tensor memory; one thread per SM issues M = 128, K = 64 instructions of width N back to back.
 // Built on demand into bench_probes.so (nvcc -shared, sm_100a) and called through ctypes; every function runs its
 // kernel three times and writes the best time in milliseconds.
 #include <cstdint>
@@ -67,11 +66,11 @@ __global__ void __launch_bounds__(256) k_popc(int iters, int *out, uint32_t seed
 }
 
 // One CTA per SM (the shared-memory request keeps a second one out).  Thread 0 of warp 0 issues `iters` groups of
-// four MMAs (128 bits of K) into one accumulator, A from tensor memory, then one commit; warp 1 waits for it with
+// four MMAs (256 elements of K) into one accumulator, A from tensor memory, then one commit; warp 1 waits for it with
 // the library's bounded wait.  The operands' contents do not matter (the weight tile is zeroed, the activation
-// columns are whatever tensor memory holds): integer MMAs take the same time on any data.
+// columns are whatever tensor memory holds).
 template <int N>
-__global__ void __launch_bounds__(128, 1) k_tcgen05_i8(int iters, int *err)
+__global__ void __launch_bounds__(128, 1) k_tcgen05_f4(int iters, int *err)
 {
     extern __shared__ unsigned char smem_raw[];
     __shared__ __align__(8) unsigned long long bar;
@@ -94,17 +93,21 @@ __global__ void __launch_bounds__(128, 1) k_tcgen05_i8(int iters, int *err)
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem_base = tmem_base_smem;
+    write_unit_scales(tmem_base + 288u + ((uint32_t)(warp * 32) << 16));
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
     if (warp == 0) {
-        constexpr uint32_t idesc = make_idesc(N);
+        constexpr uint32_t idesc = make_idesc_f4(N);
         const uint64_t desc0 = make_desc(wtile);
         const uint32_t desc_hi = (uint32_t)(desc0 >> 32), b_lo = (uint32_t)desc0;
-        const uint32_t a_t = tmem_base + 256u;                              // 32 columns of A behind the accumulator
+        const uint32_t a_t = tmem_base + 256u, sf = tmem_base + 288u;       // 32 columns of A behind the accumulator, then the scales
         if (elect_one()) {
             for (int it = 0; it < iters; ++it) {
-                tc_mma_i8_ts(tmem_base, a_t, b_lo, desc_hi, idesc, 1u);
-                tc_mma_i8_ts(tmem_base, a_t + 8u, b_lo + 2u, desc_hi, idesc, 1u);
-                tc_mma_i8_ts(tmem_base, a_t + 16u, b_lo + 4u, desc_hi, idesc, 1u);
-                tc_mma_i8_ts(tmem_base, a_t + 24u, b_lo + 6u, desc_hi, idesc, 1u);
+                tc_mma_f4_ts(tmem_base, a_t, b_lo, desc_hi, idesc, sf, 1u);
+                tc_mma_f4_ts(tmem_base, a_t + 8u, b_lo + 2u, desc_hi, idesc, sf, 1u);
+                tc_mma_f4_ts(tmem_base, a_t + 16u, b_lo + 4u, desc_hi, idesc, sf, 1u);
+                tc_mma_f4_ts(tmem_base, a_t + 24u, b_lo + 6u, desc_hi, idesc, sf, 1u);
             }
             tc_commit(smem_u32(&bar));
         }
@@ -181,7 +184,7 @@ int probe_popc(int iters, double *ms, double *macs)
 }
 
 // n in {32, 64, 128, 256}: width of the instruction.  *dev_err receives the error word of the bounded wait (0 = fine).
-int probe_tcgen05_i8(int n, int iters, double *ms, double *macs, int *dev_err)
+int probe_tcgen05_f4(int n, int iters, double *ms, double *macs, int *dev_err)
 {
     if (iters <= 0 || !ms || !macs || !dev_err) return -1;
     if (n != 32 && n != 64 && n != 128 && n != 256) return -1;
@@ -190,13 +193,13 @@ int probe_tcgen05_i8(int n, int iters, double *ms, double *macs, int *dev_err)
     if (cudaMalloc(&err, 4) != cudaSuccess) return -4;
     cudaMemset(err, 0, 4);
     const int smem = 160 * 1024;                  // more than half an SM: one CTA per SM
-    void (*k)(int, int *) = n == 32 ? k_tcgen05_i8<32> : (n == 64 ? k_tcgen05_i8<64> : (n == 128 ? k_tcgen05_i8<128> : k_tcgen05_i8<256>));
+    void (*k)(int, int *) = n == 32 ? k_tcgen05_f4<32> : (n == 64 ? k_tcgen05_f4<64> : (n == 128 ? k_tcgen05_f4<128> : k_tcgen05_f4<256>));
     int st = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) == cudaSuccess ? 0 : -4;
     if (st == 0) st = best_of_three([&] { k<<<sms, 128, smem>>>(iters, err); }, ms);
     *dev_err = 0;
     if (st == 0 && cudaMemcpy(dev_err, err, 4, cudaMemcpyDeviceToHost) != cudaSuccess) st = -4;
     cudaFree(err);
-    *macs = (double)sms * iters * 4.0 * 128.0 * n * 32.0;
+    *macs = (double)sms * iters * 4.0 * 128.0 * n * 64.0;
     return st;
 }
 

@@ -56,17 +56,18 @@ typedef enum bcnn_engine {
     BCNN_ENGINE_AUTO = 0,
     BCNN_ENGINE_LOP3 = 1,   /* CUDA cores: XOR + popcount                              */
     BCNN_ENGINE_MMA_B1 = 2, /* warp-level mma.sync m16n8k256 .b1 AND + popcount         */
-    BCNN_ENGINE_TC_I8 = 3,  /* sign bits expanded to bytes in shared memory, tcgen05 kind::i8, TMEM accumulators */
+    BCNN_ENGINE_TC_I8 = 3,  /* tcgen05 on sign bits expanded to 4-bit codes; activations and raw weights streamed and expanded
+                               tile by tile */
     BCNN_ENGINE_MMA_S8 = 4, /* sign bits expanded to bytes in registers, warp-level mma.sync 8-bit (narrow layers) */
-    BCNN_ENGINE_TC_WS = 5,  /* tcgen05 kind::i8 with the expanded weight tile resident in shared memory (C_out <= 128) */
-    BCNN_ENGINE_TC_PW = 6,  /* tcgen05 kind::i8 for pointwise layers (1x1, stride 1, no padding; GEMMs) with K <= 128 and
+    BCNN_ENGINE_TC_WS = 5,  /* tcgen05 on 4-bit codes with the expanded weights of 128 output channels resident in shared memory */
+    BCNN_ENGINE_TC_PW = 6,  /* tcgen05 on 4-bit codes for pointwise layers (1x1, stride 1, no padding; GEMMs) with K <= 128 and
                                C_out <= 128, packed output: rows bulk-copied in chunks, one hand-over per chunk */
-    BCNN_ENGINE_TC_C3 = 7,  /* tcgen05 kind::i8 for 3x3 layers (stride 1 or 2, padding 0 or 1) on 32 or 64 input channels
-                               with C_out <= 128 and W * C_in a multiple of 128, packed output: the input halo of an
+    BCNN_ENGINE_TC_C3 = 7,  /* tcgen05 on 4-bit codes for 3x3 layers (stride 1 or 2, padding 0 or 1) on 32 or 64 input
+                               channels with C_out <= 128 and W * C_in a multiple of 128, packed output: the input halo of an
                                8 x 16 tile of output pixels arrives by one tiled TMA copy, padding is the copy's zero fill */
-    BCNN_ENGINE_TC_PN = 8   /* tcgen05 kind::i8 for pointwise layers (1x1, stride 1, no padding; GEMMs) with K = 256 or 512 and
-                               128, 256 or 512 output channels, packed output: a row tile is expanded once and multiplied
-                               against all the weight slices a CTA keeps in shared memory */
+    BCNN_ENGINE_TC_PN = 8   /* tcgen05 on 4-bit codes for pointwise layers (1x1, stride 1, no padding; GEMMs) with K = 128, 256
+                               or 512 and a multiple of 128 output channels up to 2048, packed output: a row tile is expanded
+                               once and multiplied against all the weight slices a CTA keeps in shared memory */
 } bcnn_engine;
 
 /*
@@ -226,10 +227,10 @@ int bcnn_gemm_b1_engine(int engine, const void *A_bits, const void *W_bits, cons
                         void *out, int64_t M, int N, int K, void *stream);
 
 /*
- * Prepared weights.  A layer's weights do not change between calls; expanding their sign bits to the signed bytes the
+ * Prepared weights.  A layer's weights do not change between calls; expanding their sign bits to the 4-bit codes the
  * tensor cores multiply is done once, into a buffer the CALLER owns (the library never allocates), and the *_prepared
  * calls then stream that buffer by TMA instead of expanding the weight bits again for every tile of every call.
- * Worth it for wide layers and long K (C_out > 128: bcnn_prepared_preferred tells); results are bit-identical to the
+ * Worth it for wide layers, long K and small layers (bcnn_prepared_preferred tells); results are bit-identical to the
  * plain calls.
  *   bcnn_prepared_weights_bytes(C_out, K)   size of the buffer for C_out rows of K = kh*kw*C_in bits (0 if invalid)
  *   bcnn_prepare_weights(w_bits, prepared, C_out, K, stream)   w_bits as in bcnn_conv2d_b1; prepared: device, 256-byte

@@ -57,12 +57,6 @@ __device__ __forceinline__ uint32_t exact_div(uint32_t n, uint32_t mul, uint32_t
     return (t + ((n - t) >> 1)) >> (shift - 1);
 }
 
-// n / d through a precomputed multiplier (exact while n * d < 2^32); magic == 0 encodes d == 1.
-__device__ __forceinline__ int fast_div(int n, uint32_t magic)
-{
-    return magic ? (int)__umulhi((uint32_t)n, magic) : n;
-}
-
 // Row m of the implicit patch matrix -> (image, top-left input coordinate).
 struct RowCoord {
     int b, ih0, iw0;

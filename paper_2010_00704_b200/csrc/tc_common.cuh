@@ -1,6 +1,6 @@
 // Device helpers shared by the tcgen05 engines: mbarrier waits with a bound and back-off,
 // tcgen05 instruction wrappers (MMA from shared / tensor memory, commit, ld, st, fences),
-// cp.async staging, shared-memory descriptors and the bit -> byte expansions.
+// cp.async staging, shared-memory descriptors and the expansions of sign bits to 4-bit codes.
 #pragma once
 #include "bcnn_common.cuh"
 #include <cuda_fp16.h>
@@ -9,7 +9,7 @@ namespace bcnn {
 namespace tc {
 
 constexpr int BM = 128;                   // rows of an output tile = tensor-memory lanes
-constexpr int ROWB = 128;                 // bytes of one expanded row per stage (= 128 bits of K)
+constexpr int ROWB = 128;                 // bytes of one expanded row per stage (= 256 elements of K)
 constexpr uint32_t WAIT_LIMIT = 1u << 17; // polls before a wait gives up
 // upper bound (ns) for which one try_wait may suspend the thread
 constexpr uint32_t SUSPEND_HINT_NS = 20000;
@@ -79,61 +79,11 @@ __device__ __forceinline__ void tc_commit(uint32_t bar)
 {
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
 }
-__device__ __forceinline__ void tc_mma_i8(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc, uint32_t accumulate)
-{
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::i8 [%0], %1, %2, %3, {%5, %6, %7, %8}, p;\n\t}"
-        ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate), "r"(0u), "r"(0u), "r"(0u), "r"(0u)
-        : "memory");
-}
-// Predicated forms for the issuer warp: every lane executes the same straight-line code and
-// only the elected lane's predicate is true, so there is no branch to reconverge from.  The
-// descriptors are passed as (low word, high word); only the low word (start address) varies.
-__device__ __forceinline__ void tc_mma_i8_pred(uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo, uint32_t desc_hi,
-                                               uint32_t idesc, uint32_t accumulate, uint32_t pred)
-{
-    asm volatile(
-        "{\n\t.reg .pred p, q;\n\t.reg .b64 da, db;\n\t"
-        "setp.ne.b32 p, %5, 0;\n\t"
-        "setp.ne.b32 q, %6, 0;\n\t"
-        "mov.b64 da, {%1, %3};\n\t"
-        "mov.b64 db, {%2, %3};\n\t"
-        "@q tcgen05.mma.cta_group::1.kind::i8 [%0], da, db, %4, {%7, %7, %7, %7}, p;\n\t}"
-        ::"r"(d_tmem), "r"(a_lo), "r"(b_lo), "r"(desc_hi), "r"(idesc), "r"(accumulate), "r"(pred), "r"(0u)
-        : "memory");
-}
-// A operand from tensor memory (128 lanes x 8 columns = 128 rows x 32 bytes of K), B from shared memory.
-__device__ __forceinline__ void tc_mma_i8_ts_pred(uint32_t d_tmem, uint32_t a_tmem, uint32_t b_lo, uint32_t desc_hi,
-                                                  uint32_t idesc, uint32_t accumulate, uint32_t pred)
-{
-    asm volatile(
-        "{\n\t.reg .pred p, q;\n\t.reg .b64 db;\n\t"
-        "setp.ne.b32 p, %5, 0;\n\t"
-        "setp.ne.b32 q, %6, 0;\n\t"
-        "mov.b64 db, {%2, %3};\n\t"
-        "@q tcgen05.mma.cta_group::1.kind::i8 [%0], [%1], db, %4, {%7, %7, %7, %7}, p;\n\t}"
-        ::"r"(d_tmem), "r"(a_tmem), "r"(b_lo), "r"(desc_hi), "r"(idesc), "r"(accumulate), "r"(pred), "r"(0u)
-        : "memory");
-}
-// Single-thread forms (the caller has already elected one lane).
 __device__ __forceinline__ bool elect_one()
 {
     uint32_t pred = 0;
     asm volatile("{\n\t.reg .b32 rx;\n\t.reg .pred px;\n\telect.sync rx|px, 0xffffffff;\n\tselp.u32 %0, 1, 0, px;\n\t}" : "=r"(pred));
     return pred != 0;
-}
-__device__ __forceinline__ void tc_mma_i8_ts(uint32_t d_tmem, uint32_t a_tmem, uint32_t b_lo, uint32_t desc_hi,
-                                             uint32_t idesc, uint32_t accumulate)
-{
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t.reg .b64 db;\n\t"
-        "setp.ne.b32 p, %5, 0;\n\t"
-        "mov.b64 db, {%2, %3};\n\t"
-        "tcgen05.mma.cta_group::1.kind::i8 [%0], [%1], db, %4, {%6, %6, %6, %6}, p;\n\t}"
-        ::"r"(d_tmem), "r"(a_tmem), "r"(b_lo), "r"(desc_hi), "r"(idesc), "r"(accumulate), "r"(0u)
-        : "memory");
 }
 // 4-bit operands (kind::mxf4: e2m1 x e2m1 with block scales, fp32 accumulators): 64 elements of K per instruction at twice
 // the byte kinds' rate - 8.80 POP/s against 4.57 of kind::i8 with A in tensor memory, N = 64 .. 256 (8.54 at N = 32).
@@ -211,13 +161,6 @@ __device__ __forceinline__ void tc_st4_nowait(uint32_t taddr, const uint32_t (&v
                  ::"r"(taddr), "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]) : "memory");
 }
 __device__ __forceinline__ void tc_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
-__device__ __forceinline__ void tc_commit_pred(uint32_t bar, uint32_t pred)
-{
-    asm volatile(
-        "{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %1, 0;\n\t"
-        "@q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}"
-        ::"r"(bar), "r"(pred) : "memory");
-}
 
 // 32 accumulator columns of this warp's 32 rows.  The load and its completion wait are one asm
 // statement so that no use of the destination registers can be scheduled between them.
@@ -234,13 +177,6 @@ __device__ __forceinline__ void tc_ld32(uint32_t taddr, uint32_t (&v)[32])
           "=r"(v[24]), "=r"(v[25]), "=r"(v[26]), "=r"(v[27]), "=r"(v[28]), "=r"(v[29]), "=r"(v[30]), "=r"(v[31])
         : "r"(taddr) : "memory");
 }
-__device__ __forceinline__ uint32_t tc_ld1(uint32_t taddr)
-{
-    uint32_t v;
-    asm volatile("tcgen05.ld.sync.aligned.32x32b.x1.b32 {%0}, [%1];\n\ttcgen05.wait::ld.sync.aligned;"
-                 : "=r"(v) : "r"(taddr) : "memory");
-    return v;
-}
 
 // K-major tile, 128-byte rows, 128-byte swizzle, 8-row groups 1024 bytes apart, descriptor version 1.
 __device__ __forceinline__ uint64_t make_desc(uint32_t saddr)
@@ -248,11 +184,6 @@ __device__ __forceinline__ uint64_t make_desc(uint32_t saddr)
     const uint32_t lo = ((saddr & 0x3FFFFu) >> 4) | (1u << 16);
     const uint32_t hi = (1024u >> 4) | (1u << 14) | (2u << 29);
     return (static_cast<uint64_t>(hi) << 32) | lo;
-}
-// unsigned 8-bit A and B (K-major), int32 accumulate, M = 128, N = n.
-__device__ __forceinline__ constexpr uint32_t make_idesc(int n)
-{
-    return (2u << 4) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(BM >> 4) << 24);
 }
 __device__ __forceinline__ void st_shared_v4(uint32_t addr, uint32_t a, uint32_t b, uint32_t c, uint32_t d)
 {
@@ -269,64 +200,16 @@ __device__ __forceinline__ void cp_async16(uint32_t dst, const void *src, bool v
     const int n = valid ? 16 : 0;
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(n) : "memory");
 }
-__device__ __forceinline__ void cp_async4(uint32_t dst, const void *src, bool valid)
-{
-    const int n = valid ? 4 : 0;
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(dst), "l"(src), "r"(n) : "memory");
-}
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 template <int N>
 __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
-
-__device__ __forceinline__ void expand_store_a(uint32_t w, uint32_t row_addr, int xr, int c)
-{
-    st_shared_v4(row_addr + (uint32_t)(((c) ^ xr) << 4),
-                 w & 0x01010101u, w & 0x02020202u, w & 0x04040404u, w & 0x08080808u);
-    st_shared_v4(row_addr + (uint32_t)(((c + 1) ^ xr) << 4),
-                 w & 0x10101010u, w & 0x20202020u, w & 0x40404040u, w & 0x80808080u);
-}
-// Weights take the value 2^(7-j) where the activation byte is 2^j: reverse the bits of each byte once
-// (bit j+8i -> bit (7-j)+8i), after which every output word is again a single AND.
-__device__ __forceinline__ void expand_store_w(uint32_t w, uint32_t row_addr, int xr, int c)
-{
-    const uint32_t r = __byte_perm(__brev(w), 0u, 0x0123u);
-    st_shared_v4(row_addr + (uint32_t)(((c) ^ xr) << 4),
-                 r & 0x80808080u, r & 0x40404040u, r & 0x20202020u, r & 0x10101010u);
-    st_shared_v4(row_addr + (uint32_t)(((c + 1) ^ xr) << 4),
-                 r & 0x08080808u, r & 0x04040404u, r & 0x02020202u, r & 0x01010101u);
-}
-
-// Activation word -> 8 words for the signed-weight scheme: word j holds bits j, j+8, j+16, j+24 as bytes
-// 2^j for j <= 6; bit 7 goes to 64 as well (its weight magnitude is 1 where bit 6's is 1 too, see below).
-__device__ __forceinline__ void expand_a(uint32_t w, uint32_t *v)
-{
-#pragma unroll
-    for (int j = 0; j < 7; ++j) v[j] = w & (0x01010101u << j);
-    v[7] = (w >> 1) & 0x40404040u;
-}
-// Weight word -> signed bytes matching expand_a: magnitude 2^(6-j) for j <= 6 and 1 for j = 7, sign = the weight's
-// sign (bit set: +), so that every product with a set activation byte is +-64.  `live` false writes zeros.
-// The bits of each byte are reversed once (bit j -> bit 7-j) and inverted; in word j the flag "weight is -" then
-// sits at bit 7-j of every byte, exactly the lowest bit of the two's-complement pattern of -2^(6-j) above the
-// magnitude bit: flag * (2^(j+1) - 1) sets bits 7-j..7, adding the magnitude bit 6-j completes the byte (no
-// carries between bytes: every byte stays below 256).  Word 7 (magnitude 1): flag at bit 0, * 0xFE, + 1.
-__device__ __forceinline__ void expand_store_w_signed(uint32_t w, bool live, uint32_t row_addr, int xr, int c)
-{
-    const uint32_t nr = ~__byte_perm(__brev(w), 0u, 0x0123u);
-    uint32_t o[8];
-#pragma unroll
-    for (int j = 0; j < 7; ++j)
-        o[j] = live ? (nr & (0x01010101u << (7 - j))) * ((2u << j) - 1u) + (0x01010101u << (6 - j)) : 0u;
-    o[7] = live ? (nr & 0x01010101u) * 0xFEu + 0x01010101u : 0u;
-    st_shared_v4(row_addr + (uint32_t)(((c) ^ xr) << 4), o[0], o[1], o[2], o[3]);
-    st_shared_v4(row_addr + (uint32_t)(((c + 1) ^ xr) << 4), o[4], o[5], o[6], o[7]);
-}
 
 // ---- 4-bit operands.  Nibble i of word j of an expanded 32-bit group carries bit 4i + j.  Activations are unsigned
 // ({0, 2^j / 2}: e2m1 codes 1, 2, 4 are 0.5, 1, 2; bit 3 goes to code 4 as well), weights signed (+-4, +-2, +-1, +-1), so
 // that every product with a set activation bit is +-2 and with S = sum over set activation bits of the weight signs
 //   accumulator = 2 S,   sum a*g = accumulator + K - 2 popc(G):
-// one constant per output channel.  Five logic operations per activation word (nine with bytes) and half the bytes.
+// one constant per output channel.  Five logic operations per
+// activation word.
 __device__ __forceinline__ void expand_a4(uint32_t w, uint32_t *v)
 {
     v[0] = w & 0x11111111u;
@@ -400,52 +283,14 @@ __device__ __forceinline__ void write_unit_scales(uint32_t taddr)
     tc_wait_st();
 }
 
-// Expand the first nk (1..4) K words of a 128-bit stage into this lane's tensor-memory row (8 columns per word)
-// and wait for the stores.  A partial stage stores only its words: the MMAs skip the rest.
-__device__ __forceinline__ void expand_store_stage(uint32_t taddr, const uint4 &bits, int nk)
-{
-    const uint32_t wds[4] = {bits.x, bits.y, bits.z, bits.w};
-    if (nk >= 4) {
-        uint32_t v[32];
-#pragma unroll
-        for (int e = 0; e < 4; ++e) expand_a(wds[e], &v[8 * e]);
-        tc_st32_nowait(taddr, v);
-    } else {
-#pragma unroll
-        for (int e = 0; e < 3; ++e)
-            if (e < nk) {                                   // warp-uniform
-                uint32_t v[8];
-                expand_a(wds[e], v);
-                tc_st8_nowait(taddr + 8u * e, v);
-            }
-    }
-    tc_wait_st();
-}
-
 // ---- implicit-im2col gather -----------------------------------------------------------------------
 // K is cut into units of GW words that never straddle a tap: GW = 4 (one 16-byte copy) when a pixel
 // is a multiple of four words, 2 when it is even, else 1.  The unit table holds, per unit, the word
-// offset from the row's top-left input pixel and the tap's bit (0 for the zero padding of K beyond
-// kwords); a row carries the word offset of its top-left input pixel and the mask of its taps that
+// offset from the row's top-left input pixel and its tap; a row carries the word offset of its top-left input pixel and the mask of its taps that
 // fall inside the image, so one unit costs a mask test, an add and a copy with zero fill.
 __host__ __device__ __forceinline__ int gather_width(int cw) { return (cw & 3) == 0 ? 4 : ((cw & 1) == 0 ? 2 : 1); }
 
 template <int V> struct IntC { static constexpr int value = V; };
-
-__device__ __forceinline__ void build_unit_table(const ConvProblem &p, uint32_t tab_addr, int units, int gw, int tid, int nthreads)
-{
-    for (int u = tid; u < units; u += nthreads) {
-        const int kword = u * gw;
-        uint32_t off = 0, bit = 0;
-        if (kword < p.kwords) {
-            const int tap = kword / p.cw, cj = kword - tap * p.cw;
-            const int r = tap / p.kw, t = tap - r * p.kw;
-            off = (uint32_t)((r * p.W + t) * p.cw + cj);
-            bit = 1u << tap;
-        }
-        asm volatile("st.shared.v2.b32 [%0], {%1,%2};" ::"r"(tab_addr + 8u * u), "r"(off), "r"(bit) : "memory");
-    }
-}
 
 // Advance of a CTA from one of its row tiles to the next: a constant number of rows, split once into
 // whole images, output rows and output columns, so that a row's coordinates follow by carries.
@@ -520,32 +365,7 @@ __device__ __forceinline__ void cp_async_zfill(uint32_t dst, const void *src, ui
     else
         asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(dst), "l"(src), "r"(nbytes) : "memory");
 }
-// One 128-bit stage (4 / GW units, table entries at `tab`) of the row `rc` -> 16 bytes at `dst`.  Only the
-// first `nunits` units are copied (warp-uniform; the zero tail of K beyond the last word needs no copy when
-// nobody reads it).
-template <int GW>
-__device__ __forceinline__ void gather_stage(const uint32_t *x, const RowCursor &rc, uint32_t tab, uint32_t dst, int nunits = 4)
-{
-    constexpr int U = 4 / GW;
-    uint32_t ent[2 * U];
-    if (U == 1) {
-        asm volatile("ld.shared.v2.b32 {%0,%1}, [%2];" : "=r"(ent[0]), "=r"(ent[1]) : "r"(tab));
-    } else {
-#pragma unroll
-        for (int h = 0; h < U / 2; ++h)
-            asm volatile("ld.shared.v4.b32 {%0,%1,%2,%3}, [%4];"
-                         : "=r"(ent[4 * h]), "=r"(ent[4 * h + 1]), "=r"(ent[4 * h + 2]), "=r"(ent[4 * h + 3]) : "r"(tab + 16u * h));
-    }
-#pragma unroll
-    for (int u = 0; u < U; ++u) {
-        if (u >= nunits) break;
-        const bool ok = (rc.mask & ent[2 * u + 1]) != 0u;
-        const int idx = ok ? rc.base + (int)ent[2 * u] : 0;
-        cp_async_zfill<GW * 4>(dst + (uint32_t)(u * GW * 4), x + idx, ok ? (uint32_t)(GW * 4) : 0u);
-    }
-}
-
-// The same gather for 256-bit stages (eight K words, 8 / GW units, two 16-byte halves `half` bytes apart in shared memory).
+// Stages are 256 bits of K: eight words, 8 / GW units, two 16-byte halves `half` bytes apart in shared memory.
 // A table entry is one word: the unit's word offset (27 bits) and its tap in the top five; tap 31, which no row mask
 // contains, marks the zero padding of K.
 constexpr int TAP_NONE = 31;
