@@ -17,7 +17,9 @@
 // One commit per tile.  Tensor memory holds NACC accumulators and a ring of NUNIT activation UNITS: the nine taps of
 // 32 input channels of one tile, 40 columns (ten words of K: two per MMA, the tenth meets zero weights).  A tile is one unit
 // for C_in = 32 and two for C_in = 64 (K order: channel word, then tap).  Two issuer warps take alternate tiles (an issuer's
-// waits, its 5 or 10 instructions and its commit take about as long as a tile's MMAs run): wait until the tile's units are
+// waits, its 5 or 10 instructions and its commit take about as long as a tile's MMAs run; 128 output channels: a half of every
+// tile each, 3x3 64 -> 128 /2 at M = 200704 15.2 us with one issuer, 14.2 with two; four issuers on alternate tiles gain
+// nothing): wait until the tile's units are
 // full and its accumulator free, issue the tile's MMAs and ONE commit on the tile's "done" barrier, which the epilogue
 // (accumulator ready) and the producers (units free again) wait on.
 // Four producer groups of four warps fill ONE unit of every tile they take:
@@ -64,23 +66,23 @@ constexpr int MAX_NUNIT = 8, MAX_NACC = 4;
 template <int CW, int BN> struct C3Cfg {
     static constexpr int KW = TAPS * CW;                    // words of K per row
     static constexpr int KT = (UWORDS * CW + 7) / 8;        // 256-bit stages of the expanded weights
-    // 128 output channels run as two halves of 64 against the same activation units: the accumulator of one half is
-    // read by its epilogue group while the other half's MMAs run
+    // 128 output channels run as two halves of 64 against the same activation units, each with its accumulator, issuer and
+    // epilogue group; the units are free again when both halves are done
     static constexpr int NH = BN == 128 ? 2 : 1;            // halves
     static constexpr int AW = BN / NH;                      // accumulator columns
     static constexpr int NACC = NH == 2 ? 2 : 4;            // accumulators (NH == 2: one per half)
-    static constexpr int NISS = NH == 2 ? 1 : 2;            // issuer warps
+    static constexpr int NISS = 2;                          // issuer warps: alternate tiles, or a half each
     static constexpr int NU0 = (CB_COL - NACC * AW) / U_COLS;
     static constexpr int NUNIT = NU0 >= MAX_NUNIT ? MAX_NUNIT : NU0 / CW * CW;   // 8 (32 columns), 6 (64), 8 (128)
     static constexpr int A_COL0 = NACC * AW;
     static_assert(A_COL0 + NUNIT * U_COLS <= CB_COL, "tensor memory budget");
     static_assert(NUNIT >= 2 * CW && NUNIT / CW <= NAF && 2 * (NUNIT / CW) <= NB && NB % NACC == 0 && NACC <= MAX_NACC && NACC % NISS == 0, "barrier rings");
-    // warps: 0 (and 1) issuers, 2 and 3 loaders, then the producer groups, then the epilogue groups (groups start at
-    // multiples of four: warp % 4 is the tensor-memory lane quadrant of a warp)
-    static constexpr int FIRST_LOADER_WARP = 2;
-    static constexpr int FIRST_PRODUCER_WARP = 4;
-    static constexpr int FIRST_EPILOGUE_WARP = 4 + 4 * NPG;
-    static constexpr int WARPS = 4 + 4 * NPG + 4 * NGRP;
+    // warps: issuers, two loaders, then the producer groups, then the epilogue groups (warp % 4 is the tensor-memory lane
+    // quadrant of a warp: any four consecutive warps cover all of them)
+    static constexpr int FIRST_LOADER_WARP = NISS;
+    static constexpr int FIRST_PRODUCER_WARP = FIRST_LOADER_WARP + NGRP;
+    static constexpr int FIRST_EPILOGUE_WARP = FIRST_PRODUCER_WARP + 4 * NPG;
+    static constexpr int WARPS = FIRST_EPILOGUE_WARP + 4 * NGRP;
     static constexpr int THREADS = 32 * WARPS;
     static constexpr int W_TILE_BYTES = BN * ROWB;
 };
@@ -166,7 +168,7 @@ conv_tc_c3_kernel(const ConvProblem p, const C3Geom g, const __grid_constant__ C
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
     for (int c = tid; c < BN; c += C::THREADS) asm volatile("st.shared.b32 [%0], %1;" ::"r"(pops + 4u * c), "r"(0) : "memory");
-    if (tid == 64) asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&xmap)) : "memory");
+    if (tid == 32 * C::FIRST_LOADER_WARP) asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&xmap)) : "memory");
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -177,8 +179,8 @@ conv_tc_c3_kernel(const ConvProblem p, const C3Geom g, const __grid_constant__ C
     const bool is_loader = warp >= C::FIRST_LOADER_WARP && warp < C::FIRST_PRODUCER_WARP;
     const uint32_t tmem_base = tmem_base_smem;
     if (!is_loader) {
-        constexpr int NW = C::THREADS - 64, WTOTAL = KT * 8 * BN, WU = (WTOTAL + NW - 1) / NW;       // (threads 64 .. 127 are the loaders)
-        const int wt = tid < 64 ? tid : tid - 64;
+        constexpr int NW = C::THREADS - 64, WTOTAL = KT * 8 * BN, WU = (WTOTAL + NW - 1) / NW;
+        const int wt = tid < 32 * C::FIRST_LOADER_WARP ? tid : tid - 64;       // (the loaders are 64 threads)
         auto sync_workers = [&]() { asm volatile("bar.sync 1, %0;" ::"n"(NW) : "memory"); };
         // ---- one-off: expanded weights and the channels' bit counts.  K position e of the MMAs = channel word e / 10, tap e % 10
         // (global weight word tap * CW + channel word) -> stage e / 8, 16-byte piece e % 8; MMA row `row` carries channel ch.
@@ -243,48 +245,42 @@ conv_tc_c3_kernel(const ConvProblem p, const C3Geom g, const __grid_constant__ C
     };
 
     if (warp < C::NISS) {
-        // ------------------------------------------------------------------ MMA issuer of tiles n = warp (mod NISS), in order
+        // ------------------------------------------------------------------ MMA issuer of tiles n = warp (mod NISS), or of
+        // half `warp` of every tile, in order
         constexpr uint32_t idesc = make_idesc_f4(AW);
         constexpr uint32_t HALF_DESC = (uint32_t)(AW * ROWB) >> 4;               // weight rows of the second half
         const uint64_t desc0 = make_desc(wexp);
         const uint32_t desc_hi = (uint32_t)(desc0 >> 32), b_lo = (uint32_t)desc0;
         const uint32_t tmem_u = __shfl_sync(0xffffffffu, tmem_base, 0);
         const uint32_t sf = tmem_u + (uint32_t)CB_COL, c_lo = (uint32_t)make_desc(cexp);
-        bool ok = true;
-        for (int n = warp; n < my_tiles && ok; n += C::NISS) {
+        const uint32_t hf = NH == 2 ? __shfl_sync(0xffffffffu, (uint32_t)warp, 0) : 0u;
+        const uint32_t w_lo = b_lo + hf * HALF_DESC;
+        for (int n = NH == 2 ? 0 : warp; n < my_tiles; n += NH == 2 ? 1 : C::NISS) {
             if (!pw_wait(a_full(n % NAF), (uint32_t)(n / NAF) & 1u, abort_flag, p.err, ERR_C3_ISSUER_TIMEOUT)) break;
+            // the epilogue has read the accumulator's previous tile
+            const int acc = NH == 2 ? (int)hf : n % NACC;
+            const int prev = NH == 2 ? n - 1 : n / NACC - 1;                 // completion of acc_free to wait for
+            if (prev >= 0 && !pw_wait(acc_free(acc), (uint32_t)prev & 1u, abort_flag, p.err, ERR_C3_ACC_TIMEOUT)) break;
+            tc_fence_after();
+            if (elect_one()) {
+                const uint32_t d_t = tmem_u + (uint32_t)(acc * AW);
+                tc_mma_const(d_t, tmem_u, c_lo + hf * HALF_DESC, desc_hi, idesc);
 #pragma unroll
-            for (int hf = 0; hf < NH; ++hf) {
-                // the epilogue has read the accumulator's previous tile
-                const int acc = NH == 2 ? hf : n % NACC;
-                const int prev = NH == 2 ? n - 1 : n / NACC - 1;                 // completion of acc_free to wait for
-                if (prev >= 0) {
-                    ok = pw_wait(acc_free(acc), (uint32_t)prev & 1u, abort_flag, p.err, ERR_C3_ACC_TIMEOUT);
-                    if (!ok) break;
-                }
-                tc_fence_after();
-                if (elect_one()) {
-                    const uint32_t d_t = tmem_u + (uint32_t)(acc * AW);
-                    tc_mma_const(d_t, tmem_u, c_lo + hf * HALF_DESC, desc_hi, idesc);
+                for (int h = 0; h < CW; ++h) {
+                    const uint32_t a_t = tmem_u + (uint32_t)(C::A_COL0 + ((n * CW + h) % NUNIT) * U_COLS);
 #pragma unroll
-                    for (int h = 0; h < CW; ++h) {
-                        const uint32_t a_t = tmem_u + (uint32_t)(C::A_COL0 + ((n * CW + h) % NUNIT) * U_COLS);
-#pragma unroll
-                        for (int t = 0; t < UWORDS / 2; ++t) {
-                            const int e = h * UWORDS + 2 * t;
-                            tc_mma_f4_ts(d_t, a_t + 8u * t, b_lo + hf * HALF_DESC + (uint32_t)((e >> 3) * (C::W_TILE_BYTES >> 4) + (e & 7)),
-                                         desc_hi, idesc, sf, 1u);
-                        }
+                    for (int t = 0; t < UWORDS / 2; ++t) {
+                        const int e = h * UWORDS + 2 * t;
+                        tc_mma_f4_ts(d_t, a_t + 8u * t, w_lo + (uint32_t)((e >> 3) * (C::W_TILE_BYTES >> 4) + (e & 7)),
+                                     desc_hi, idesc, sf, 1u);
                     }
-                    tc_commit(tile_done((n * NH + hf) % NB));
                 }
-                __syncwarp();
+                tc_commit(tile_done((n * NH + (int)hf) % NB));
             }
+            __syncwarp();
         }
-    } else if (warp < C::FIRST_LOADER_WARP) {
-        // (idle)
     } else if (warp < C::FIRST_PRODUCER_WARP) {
-        // ------------------------------------------------------------------ loader of group warp - 2: one halo tile per TMA copy
+        // ------------------------------------------------------------------ loader of a group: one halo tile per TMA copy
         const int grp = warp - C::FIRST_LOADER_WARP;
         int stage = 0;
         uint32_t phase = 1;                       // first pass through the ring: the stages are free
@@ -323,7 +319,7 @@ conv_tc_c3_kernel(const ConvProblem p, const C3Geom g, const __grid_constant__ C
             const int acc = NH == 2 ? grp : n % NACC;
             const int d = NH == 2 ? 2 * n + grp : n;                              // the tile's (half's) "done" number
             const int ch0 = NH == 2 ? 2 * grp : 0;                                // first output word of this accumulator
-            if (!pw_wait<C::NISS == 1 ? 64 : 128>(tile_done(d % NB), (uint32_t)(d / NB) & 1u, abort_flag, p.err, ERR_C3_EPILOGUE_TIMEOUT)) break;
+            if (!pw_wait<NH == 2 ? 64 : 128>(tile_done(d % NB), (uint32_t)(d / NB) & 1u, abort_flag, p.err, ERR_C3_EPILOGUE_TIMEOUT)) break;
             tc_fence_after();
             uint32_t words[AW / 32];
             if constexpr (AW == 32) {
@@ -390,8 +386,9 @@ conv_tc_c3_kernel(const ConvProblem p, const C3Geom g, const __grid_constant__ C
             // the MMAs of the tile that used this ring position last have read it (nothing to wait for the first time round)
             const int u = n * CW + h;
             if (u >= NUNIT) {
-                const int dm = (u - NUNIT) / CW * NH + NH - 1;                    // that tile's last "done" number
+                const int dm = (u - NUNIT) / CW * NH;                             // that tile's first "done" number
                 if (!pw_wait<64>(tile_done(dm % NB), (uint32_t)(dm / NB) & 1u, abort_flag, p.err, ERR_C3_UNIT_TIMEOUT)) break;
+                if (NH == 2 && !pw_wait<64>(tile_done((dm + 1) % NB), (uint32_t)((dm + 1) / NB) & 1u, abort_flag, p.err, ERR_C3_UNIT_TIMEOUT)) break;
             }
             tc_fence_after();
             const uint32_t taddr = t_lane + (uint32_t)((u % NUNIT) * U_COLS);
