@@ -122,13 +122,17 @@ def test_prepared_widths(bk, oracle, M, N, K, fused):
     assert bk.bcnn_device_error() == 0
 
 
-# the stem's plain kernel and its table, on both sides of the line between them (148 * 1792 pixels)
-@pytest.mark.parametrize("shape", [(1, 9, 7), (1, 448, 592), (1, 450, 592)])
-def test_stem_sizes(bk, oracle, shape):
+# the stem's plain kernel and its table, on both sides of the line between them (148 * 2304 pixels), and with the ring of
+# chunks used more than once (148 * 5 * 1984 pixels), a bias for the per-channel path included
+@pytest.mark.parametrize("shape,inf", [((1, 9, 7), False), ((1, 576, 592), False), ((1, 577, 592), True), ((1, 579, 591), False), ((1, 1100, 1351), False),
+                                       ((1, 1100, 1351), True)])
+def test_stem_sizes(bk, oracle, shape, inf):
     B, H, W = shape
     rng = np.random.default_rng(9900 + sum(shape))
     x, bias, w = synth.real_input(rng, (B, H, W, 4)), synth.real_input(rng, (32,)), synth.pm1(rng, (32, 1, 1, 32))
     thr = synth.thresholds(rng, 32, 32)
+    if inf:
+        bias[5], bias[9] = np.inf, -np.inf
     out = torch.empty(B * H * W * 4, dtype=torch.uint8, device="cuda")
     bk.bcnn_stem_fused(dev(x), dev(bias), dev(synth.pack_bits(w)), dev(thr), out, B, H, W, 4, 8, 32)
     torch.cuda.synchronize()
