@@ -289,8 +289,6 @@ conv_tc_pn_kernel(const ConvProblem p, const PnPlan plan)
             const uint4 q0 = ld_shared_v4(src);
             uint4 q1 = q0;
             if (UWORDS == 8) q1 = ld_shared_v4(src + 16u);
-            __syncwarp();
-            mbar_arrive_pred(load_empty(lg, stage), lane0);        // the stage may be refilled
             uint32_t v[32];                       // expanded before the wait for the unit
             expand_stage8(q0, q1, v);             // (four words: the second half is dropped)
             // the MMAs of the tile that used this ring position last have read it (nothing to wait for the first time round)
@@ -302,6 +300,10 @@ conv_tc_pn_kernel(const ConvProblem p, const PnPlan plan)
             }
             tc_fence_after();
             const uint32_t taddr = t_lane + (uint32_t)((u % NUNIT) * U_COLS);
+            // the stage may be refilled: its words are in registers by now, expanded (handing it back right behind the loads
+            // let a refill that hit L2 overtake them, on a CTA's first tiles: a few rows wrong in one launch of fifteen)
+            __syncwarp();
+            mbar_arrive_pred(load_empty(lg, stage), lane0);
             if constexpr (UWORDS == 8) tc_st32_nowait(taddr, v);
             else tc_st16_nowait(taddr, reinterpret_cast<const uint32_t (&)[16]>(v[0]));
             tc_wait_st();
