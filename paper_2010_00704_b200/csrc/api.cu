@@ -89,10 +89,11 @@ int make_conv_problem(ConvProblem &p, const void *x, const void *w, const int32_
 //   * the single-bit mma.sync engine never wins and serves as a fallback.
 int auto_engine(const ConvProblem &p)
 {
-    // a call whose work is a wave of 64 x 64 tiles of up to 256 bits is over before a tensor-core engine has its weights expanded
-    // (1x1 64 -> 64 at M = 3136: 3.4 against 4.2 us, 256 -> 256 at M = 196: 3.4 against 4.4)
-    if (p.K <= 256 && ((p.M + 63L) / 64) * ((p.C_out + 63) / 64) <= sm_count()) return BCNN_ENGINE_LOP3;
+    // at every size, the smallest included: 2.4 .. 2.9 us up to M = 12544, against 3.0 .. 5.9 of the CUDA-core engine
     if (conv_tc_pw_supports(p)) return BCNN_ENGINE_TC_PW;
+    // another call whose work is half a wave of 64 x 64 tiles of up to 256 bits is over before a tensor-core engine has its
+    // weights expanded (1x1 256 -> 256 at M = 196: 3.3 against 4.2 us; 256 -> 128 at M = 3136: 5.3 against 4.2)
+    if (p.K <= 256 && ((p.M + 63L) / 64) * ((p.C_out + 63) / 64) <= sm_count() / 2) return BCNN_ENGINE_LOP3;
     if (conv_tc_pn_supports(p)) return BCNN_ENGINE_TC_PN;
     if (conv_tc_c3_supports(p)) {
         const long covered = (long)((p.OH + 7) / 8 * 8) * ((p.OW + 15) / 16 * 16);
@@ -402,17 +403,19 @@ int bcnn_prepared_preferred(int B, int H, int W, int C_in, int C_out, int kh, in
     if (st != BCNN_OK) return 0;
     // Measured: streaming prepared weights wins wherever AUTO would expand them on every call - the streaming engine always,
     // the weight-stationary one except on many rows of a short K, where its expansion is spread thin (56x56 64 -> 128 /2 at
-    // batch 256, M = 200704, K = 576: 16.1 against 18.2 us; K = 1152: 19.7 against 19.0; M = 784: 6.5 against 4.0).  The pointwise
-    // and halo-tile engines keep their layers, all but the smallest with many weights: they expand those at the start.
+    // batch 256, M = 200704, K = 576: 16.1 against 18.2 us; K = 1152: 19.7 against 19.0; M = 784: 6.5 against 4.0).  The wide
+    // pointwise and halo-tile engines keep their layers, all but the smallest with many weights: they expand those at the start.
     if (!conv_tc_pre_supports(p)) return 0;
     switch (auto_engine(p)) {
+    case BCNN_ENGINE_TC_PW: return 0;           // 2.4 .. 2.9 against 2.9 .. 4.1 us up to M = 12544
     case BCNN_ENGINE_TC_C3:
         if (p.C_out <= 64) return 0;
         [[fallthrough]];
-    case BCNN_ENGINE_TC_PW: case BCNN_ENGINE_TC_PN:
+    case BCNN_ENGINE_TC_PN:
         // 3x3 64 -> 128 /2: 5.0 against 4.0 us at M = 784, 15.4 against 18.2 at 200704; 1x1 512 -> 512: 5.0 against 3.7 us at M = 49,
-        // 6.5 against 8.3 at 12544; 128 -> 128: 3.9 against 3.3 at 784
-        return p.M <= 4096 && ((p.M + 127) / 128) * ((p.C_out + 63) / 64) <= sm_count() ? 1 : 0;
+        // 6.5 against 8.3 at 12544
+        // (1x1 512 -> 128 at M = 12544: 5.2 against 4.4, 256 -> 256: 5.0 against 5.7)
+        return ((p.M + 127L) / 128) * ((p.C_out + 63) / 64) <= sm_count() * 3 / 2 ? 1 : 0;
     case BCNN_ENGINE_TC_WS: return p.K >= 1024 || p.M < 98304 ? 1 : 0;
     case BCNN_ENGINE_LOP3: return p.K <= 64 ? 0 : 1;
     default: return 1;

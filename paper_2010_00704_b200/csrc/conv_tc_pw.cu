@@ -72,11 +72,10 @@ template <int KW, int BN> struct PwCfg {
     static_assert(T >= 1 && T <= 4 && NSLOT >= 2 && NSLOT <= 3, "slot shape");
     static constexpr int CHUNK_ROWS = T * BM;
     static constexpr int CHUNK_BYTES = CHUNK_ROWS * KW * 4;
-    // chunks per block: a multiple of the slots (every slot has the same share of every block), about 12 KB
+    // chunks per block at most: a multiple of the slots (every slot has the same share of every block), about 12 KB
     static constexpr int G0 = BLOCK_BYTES_TARGET / (NSLOT * CHUNK_BYTES);
-    static constexpr int G = NSLOT * (G0 < 1 ? 1 : G0);
-    static constexpr int BLOCK_ROWS = G * CHUNK_ROWS;
-    static constexpr int BLOCK_BYTES = G * CHUNK_BYTES;
+    static constexpr int MAX_G = NSLOT * (G0 < 1 ? 1 : G0);
+    static constexpr int BLOCK_BYTES = MAX_G * CHUNK_BYTES;
     static constexpr int NBLK = RING_BYTES / BLOCK_BYTES > MAX_BLOCKS ? MAX_BLOCKS : RING_BYTES / BLOCK_BYTES;
     static_assert(NBLK >= 4, "ring depth");
     // warps: 0..NSLOT-1 issuers (one per slot), 3 loader, then per slot four producer warps, then per slot four
@@ -93,10 +92,10 @@ template <int KW, int BN> struct PwCfg {
 
 template <int KW, int BN>
 __global__ void __launch_bounds__(PwCfg<KW, BN>::THREADS, 1)
-conv_tc_pw_kernel(const ConvProblem p)
+conv_tc_pw_kernel(const ConvProblem p, const int G /* chunks per block */, const int n_blocks)
 {
     using C = PwCfg<KW, BN>;
-    constexpr int T = C::T, NSLOT = C::NSLOT, G = C::G, NBLK = C::NBLK;
+    constexpr int T = C::T, NSLOT = C::NSLOT, NBLK = C::NBLK;
 
     extern __shared__ unsigned char smem_raw[];
     __shared__ __align__(8) unsigned long long bars[2 * MAX_BLOCKS + 3 * 3];
@@ -107,15 +106,18 @@ conv_tc_pw_kernel(const ConvProblem p)
     const int warp = tid >> 5, lane = tid & 31;
     // this CTA's blocks: blockIdx.x, blockIdx.x + gridDim.x, ...; its j-th chunk (chunk j % G of its block j / G)
     // belongs to slot j % NSLOT.  Only the last block of all can be short; it is the last one of its CTA.
-    const long n_blocks = ((long)p.M + C::BLOCK_ROWS - 1) / C::BLOCK_ROWS;
-    const int my_blocks = (long)blockIdx.x < n_blocks ? (int)((n_blocks - 1 - blockIdx.x) / gridDim.x) + 1 : 0;
+    const int block_rows = G * C::CHUNK_ROWS;
+    const int my_blocks = (int)blockIdx.x < n_blocks ? (int)((unsigned)(n_blocks - 1 - (int)blockIdx.x) / gridDim.x) + 1 : 0;
     int my_chunks = my_blocks * G;
-    if (my_blocks > 0 && (long)blockIdx.x + (long)(my_blocks - 1) * gridDim.x == n_blocks - 1) {
-        const long rows_last = (long)p.M - (n_blocks - 1) * C::BLOCK_ROWS;
-        my_chunks -= G - (int)((rows_last + C::CHUNK_ROWS - 1) / C::CHUNK_ROWS);
+    if (my_blocks > 0 && (int)blockIdx.x + (my_blocks - 1) * (int)gridDim.x == n_blocks - 1) {
+        const int rows_last = (int)((long)p.M - (long)(n_blocks - 1) * block_rows);
+        my_chunks -= G - (rows_last + C::CHUNK_ROWS - 1) / C::CHUNK_ROWS;
     }
-    // first row of this CTA's chunk j
-    auto chunk_row0 = [&](int j) { return ((long)blockIdx.x + (long)(j / G) * gridDim.x) * C::BLOCK_ROWS + (long)(j % G) * C::CHUNK_ROWS; };
+    // a slot's chunks: chunk idx of this CTA's block blk (G is a multiple of NSLOT, or there is one block)
+    auto advance = [&](int &blk, int &idx) {
+        idx += NSLOT;
+        if (idx >= G) { idx -= G; ++blk; }
+    };
     const int cn = min(BN, p.C_out);
 
     const uint32_t wexp = (smem_u32(smem_raw) + 1023u) & ~1023u;          // [BN rows][128 B] expanded weights
@@ -218,8 +220,8 @@ conv_tc_pw_kernel(const ConvProblem p)
         uint32_t phase = 1;                       // first pass through the ring: the stages are free
         int issued = 0;
         for (int b = 0; b < my_blocks; ++b) {
-            const long row0 = ((long)blockIdx.x + (long)b * gridDim.x) * C::BLOCK_ROWS;
-            const long rows = min((long)C::BLOCK_ROWS, (long)p.M - row0);
+            const long row0 = ((long)blockIdx.x + (long)b * gridDim.x) * block_rows;
+            const long rows = min((long)block_rows, (long)p.M - row0);
             const uint32_t bytes = (uint32_t)rows * KW * 4u;
             if (!pw_wait(load_empty(stage), phase, abort_flag, p.err, ERR_PW_LOADER_TIMEOUT)) break;
             const uint32_t dst = ring + (uint32_t)stage * C::BLOCK_BYTES;
@@ -253,8 +255,10 @@ conv_tc_pw_kernel(const ConvProblem p)
         const uint32_t t_lane = tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)(slot * T * BN);
         const int owords = p.C_out >> 5;
         uint32_t phase = 0;
-        for (int j = slot; j < my_chunks; j += NSLOT) {
-            const long row_w = chunk_row0(j) + quad * 32 + lane;                 // this thread's row in tile 0
+        int blk = 0, idx = slot;
+        for (int j = slot; j < my_chunks; j += NSLOT, advance(blk, idx)) {
+            // this thread's row in tile 0
+            const long row_w = ((long)blockIdx.x + (long)blk * gridDim.x) * block_rows + (long)idx * C::CHUNK_ROWS + quad * 32 + lane;
             if (!pw_wait(mma_done(slot), phase, abort_flag, p.err, ERR_PW_EPILOGUE_TIMEOUT)) break;
             tc_fence_after();
             phase ^= 1u;
@@ -314,10 +318,11 @@ conv_tc_pw_kernel(const ConvProblem p)
         const uint32_t t_lane = tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)(C::A_COL0 + slot * T * C::A_COLS);
         const uint32_t lane0 = lane == 0 ? 1u : 0u;
         uint32_t phase = 0;
-        for (int j = slot; j < my_chunks; j += NSLOT) {
-            const int blk = j / G, stage = blk % NBLK;
+        int blk = 0, idx = slot;
+        for (int j = slot; j < my_chunks; j += NSLOT, advance(blk, idx)) {
+            const int stage = blk % NBLK;
             if (!pw_wait(load_full(stage), (uint32_t)(blk / NBLK) & 1u, abort_flag, p.err, ERR_PW_PRODUCER_TIMEOUT)) break;
-            const uint32_t src = ring + (uint32_t)stage * C::BLOCK_BYTES + (uint32_t)(j % G) * C::CHUNK_BYTES + (uint32_t)row * (KW * 4u);
+            const uint32_t src = ring + (uint32_t)stage * C::BLOCK_BYTES + (uint32_t)idx * C::CHUNK_BYTES + (uint32_t)row * (KW * 4u);
             uint32_t wds[T][KW];
 #pragma unroll
             for (int t = 0; t < T; ++t) {
@@ -374,11 +379,17 @@ int launch_pw(const ConvProblem &p0, cudaStream_t stream)
     ConvProblem p = p0;
     p.err = device_error_word();
     const int sms = sm_count();
-    const long n_blocks = ((long)p.M + C::BLOCK_ROWS - 1) / C::BLOCK_ROWS;
+    // Blocks as large as leaves every multiprocessor one; few rows in one block per multiprocessor of any number of chunks (1x1
+    // 32 -> 128 at M = 3136: 6.9 us with blocks of the full size, 2.5
+    // so; 64 -> 64: 3.6 and 2.5)
+    const long chunks = ((long)p.M + C::CHUNK_ROWS - 1) / C::CHUNK_ROWS;
+    const long share = chunks / ((long)sms * C::NSLOT) * C::NSLOT;
+    const int G = chunks <= (long)sms * C::NSLOT ? (int)((chunks + sms - 1) / sms) : (int)(share < C::MAX_G ? share : C::MAX_G);
+    const int n_blocks = (int)((chunks + G - 1) / G);
     const unsigned grid = (unsigned)(n_blocks < sms ? n_blocks : sms);
-    void (*k)(const ConvProblem) = conv_tc_pw_kernel<KW, BN>;
+    void (*k)(const ConvProblem, const int, const int) = conv_tc_pw_kernel<KW, BN>;
     if (!allow_smem((const void *)k, C::SMEM_ASK)) return BCNN_ERR_CUDA;
-    return launch(k, grid, C::THREADS, C::SMEM_ASK, stream, p);
+    return launch(k, grid, C::THREADS, C::SMEM_ASK, stream, p, G, n_blocks);
 }
 
 template <int KW>
