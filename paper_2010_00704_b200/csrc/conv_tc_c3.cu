@@ -376,8 +376,6 @@ conv_tc_c3_kernel(const ConvProblem p, const C3Geom g, const __grid_constant__ C
 #pragma unroll
             for (int tap = 0; tap < TAPS; ++tap)
                 asm volatile("ld.shared.b32 %0, [%1];" : "=r"(wds[tap]) : "r"(src + (uint32_t)(tap / 3) * row_pitch + (uint32_t)((tap % 3) * CW * 4)) : "memory");
-            __syncwarp();
-            mbar_arrive_pred(load_empty(lg, stage), lane0);        // the stage may be refilled
             // expanded before the wait for the unit (the unit's tenth word is not written: its weights are zero)
             uint32_t v[32], v4[4];
 #pragma unroll
@@ -394,6 +392,9 @@ conv_tc_c3_kernel(const ConvProblem p, const C3Geom g, const __grid_constant__ C
             const uint32_t taddr = t_lane + (uint32_t)((u % NUNIT) * U_COLS);
             tc_st32_nowait(taddr, v);
             tc_st4_nowait(taddr + 32u, v4);
+            // the stage may be refilled: its words have left through registers (right behind the loads a refill could overtake them)
+            __syncwarp();
+            mbar_arrive_pred(load_empty(lg, stage), lane0);
             tc_wait_st();
             tc_fence_before();
             __syncwarp();

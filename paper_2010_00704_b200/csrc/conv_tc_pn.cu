@@ -300,12 +300,12 @@ conv_tc_pn_kernel(const ConvProblem p, const PnPlan plan)
             }
             tc_fence_after();
             const uint32_t taddr = t_lane + (uint32_t)((u % NUNIT) * U_COLS);
-            // the stage may be refilled: its words are in registers by now, expanded (handing it back right behind the loads
+            if constexpr (UWORDS == 8) tc_st32_nowait(taddr, v);
+            else tc_st16_nowait(taddr, reinterpret_cast<const uint32_t (&)[16]>(v[0]));
+            // the stage may be refilled: its words have left through registers (handing it back right behind the loads
             // let a refill that hit L2 overtake them, on a CTA's first tiles: a few rows wrong in one launch of fifteen)
             __syncwarp();
             mbar_arrive_pred(load_empty(lg, stage), lane0);
-            if constexpr (UWORDS == 8) tc_st32_nowait(taddr, v);
-            else tc_st16_nowait(taddr, reinterpret_cast<const uint32_t (&)[16]>(v[0]));
             tc_wait_st();
             tc_fence_before();
             __syncwarp();

@@ -338,8 +338,6 @@ conv_tc_pw_kernel(const ConvProblem p, const int G /* chunks per block */, const
                         asm volatile("ld.shared.b32 %0, [%1];" : "=r"(wds[t][e]) : "r"(a + 4u * e) : "memory");
                 }
             }
-            __syncwarp();
-            mbar_arrive_pred(load_empty(stage), lane0);           // (the stage may be refilled once all its chunks have been read)
             // expanded rows in registers first; only the stores wait for the slot
             uint32_t v[T][4 * KW];
 #pragma unroll
@@ -361,6 +359,8 @@ conv_tc_pw_kernel(const ConvProblem p, const int G /* chunks per block */, const
             tc_fence_before();
             __syncwarp();
             mbar_arrive_pred(a_full(slot), lane0);
+            // the stage may be refilled once all its chunks have been read: these words have left through registers
+            mbar_arrive_pred(load_empty(stage), lane0);
             phase ^= 1u;
         }
     }
