@@ -208,14 +208,14 @@ stem_c4r8_k32_kernel(const float4 *__restrict__ x, const float *__restrict__ bia
             for (int u = 0; u < STEM_U; ++u)    // (what lies beyond the last pixel is read and not used)
                 asm volatile("ld.shared.v4.f32 {%0,%1,%2,%3}, [%4];" : "=f"(v[u].x), "=f"(v[u].y), "=f"(v[u].z), "=f"(v[u].w)
                              : "r"(ring + (uint32_t)((stage * STEM_CHUNK + u * STEM_WORKERS + tid) * 16)) : "memory");
-            __syncwarp();
-            mbar_arrive_pred(empty(stage), lane0);
             const long p0 = c * STEM_CHUNK + tid;
 #pragma unroll
             for (int u = 0; u < STEM_U; ++u) {
                 const uint32_t o = pixel(v[u]);
                 if (p0 + u * STEM_WORKERS < npix) __stcs(out + p0 + u * STEM_WORKERS, o);
             }
+            __syncwarp();                       // the words have been used: the stage may be refilled
+            mbar_arrive_pred(empty(stage), lane0);
         }
     };
     if (!all_finite) {
