@@ -20,6 +20,7 @@
 // Every mbarrier wait is bounded and reports through the device error word.
 #include "tc_common.cuh"
 #include "tensor_map.cuh"
+#include <climits>
 
 namespace bcnn {
 
@@ -57,7 +58,7 @@ template <int BN, int MODE, int G, int TEAMS> struct Cfg {
 };
 
 template <typename C>
-__host__ __device__ inline int smem_bytes(int ktab_words, int mode)
+__host__ __device__ constexpr int smem_bytes(int ktab_words, int mode)
 {
     return 1024 + C::STAGES * C::W_BYTES + C::BITS_BYTES + C::TABLE_BYTES + ktab_words * 4 + 16 +
            (mode == 0 ? C::EPI_WARPS * I32_TILE_BYTES + 16 : 0);
@@ -492,7 +493,7 @@ bool conv_tc_pre_supports(const ConvProblem &p)
     if (p.mode == 1 && (p.C_out % 32 != 0)) return false;
     if (p.kh * p.kw > 31) return false;                       // one validity bit per tap
     if ((long)p.B * p.H * p.W * p.cw >= (1L << 31)) return false;     // rows address the input by 32-bit word offsets
-    if (smem_bytes<Cfg<256, 1, 2, 2>>(ktab_words_for(p), 1) > MAX_SMEM) return false;
+    if (smem_bytes<Cfg<256, 1, 2, 2>>(ktab_words_for(p), 1) > MAX_SMEM) return false;      // (the widths below need no more, but for one)
     if ((long)p.kh * p.W * p.cw >= (1L << 27)) return false;  // a unit's word offset within the window
     return p.K <= (1 << 20);                                  // sums up to 4 K + 2 stay exact in fp32
 }
@@ -517,7 +518,13 @@ int launch_conv_tc_pre(const ConvProblem &p, const void *prepared, cudaStream_t 
         return start + waves * (wave + kt * stage);
     };
     const bool packed = p.mode == 1;
-    const long c256 = cost(256, 3200, packed ? 1660 : 4300, 288), c128 = cost(128, 3500, packed ? 600 : 2200, 185), c64 = cost(64, 3100, packed ? 530 : 1150, 167);
+    // What conv_tc_pre_supports vouches for is the packed 256-wide variant's shared memory.  The int32 one needs its store staging
+    // tiles besides: a K beyond 274 176 bits with an odd number of words per pixel, 548 352 with an even one, runs on narrower tiles.
+    static_assert(smem_bytes<Cfg<128, 0, 3, 2>>(0, 0) <= smem_bytes<Cfg<256, 1, 2, 2>>(0, 1) && smem_bytes<Cfg<64, 0, 2, 1>>(0, 0) <= smem_bytes<Cfg<256, 1, 2, 2>>(0, 1) &&
+                  smem_bytes<Cfg<128, 1, 2, 1>>(0, 1) <= smem_bytes<Cfg<256, 1, 2, 2>>(0, 1) && smem_bytes<Cfg<64, 1, 2, 1>>(0, 1) <= smem_bytes<Cfg<256, 1, 2, 2>>(0, 1),
+                  "a supported layer fits the narrower tiles");
+    const bool fits256 = packed || smem_bytes<Cfg<256, 0, 2, 2>>(ktab_words_for(p), 0) <= MAX_SMEM;
+    const long c256 = fits256 ? cost(256, 3200, packed ? 1660 : 4300, 288) : LONG_MAX, c128 = cost(128, 3500, packed ? 600 : 2200, 185), c64 = cost(64, 3100, packed ? 530 : 1150, 167);
     if (c64 <= c128 && c64 <= c256) return packed ? launch_bn<64, 1, 2, 1>(p, pw, stream) : launch_bn<64, 0, 2, 1>(p, pw, stream);
     if (c128 <= c256) return packed ? launch_bn<128, 1, 2, 1>(p, pw, stream) : launch_bn<128, 0, 3, 2>(p, pw, stream);
     return packed ? launch_bn<256, 1, 2, 2>(p, pw, stream) : launch_bn<256, 0, 2, 2>(p, pw, stream);

@@ -68,3 +68,30 @@ def test_argument_validation_needs_no_device():
     assert lib.bcnn_conv2d_b1_engine(99, a, a, None, a, 1, 4, 4, 32, 8, 3, 3, 1, 1, None) == -2
     assert lib.bcnn_selftest_wait_timeout(0, None) == -1
     assert lib.bcnn_selftest_wait_timeout(1 << 20, None) == -1
+
+
+def test_prepared_call_takes_what_it_is_preferred_for():
+    # The gather's table grows with K: near the largest K one of the tile widths no longer fits shared memory, and the call has to
+    # take another.  Rows of an odd, an even and a fourfold number of words around those sizes, both outputs; made-up addresses, so
+    # only where no device could run the call: there it gets as far as the driver (ERR_CUDA) or refuses the shape.
+    import pytest
+    import torch
+    from paper_2010_00704_b200 import build, binding
+    if torch.cuda.is_available():
+        pytest.skip("made-up addresses: only without a device")
+    build.build()
+    lib = binding.load()
+    a = ctypes.c_void_p(4096)
+    seen = set()
+    for unit, lo, hi in ((1, 8000, 10200), (2, 16000, 20400), (4, 31000, 32768)):          # words of K: the limits lie inside
+        for kwords in range(lo, hi + 1, 37 * unit):
+            kwords = kwords // unit * unit + (unit if unit < 4 and (kwords // unit) % 2 == 0 else 0)       # exactly `unit` divides it
+            K = 32 * kwords
+            for M, N in ((1, 64), (700, 256), (4736, 1024), (100000, 512)):
+                for fused in (0, 1):
+                    st = lib.bcnn_gemm_b1_prepared(a, a, a if fused else None, a, M, N, K, None)
+                    preferred = lib.bcnn_prepared_preferred(1, M, 1, K, N, 1, 1, 1, 0, fused)
+                    assert st in (binding.ERR_CUDA, binding.ERR_UNSUPPORTED), (M, N, K, fused)
+                    assert not preferred or st == binding.ERR_CUDA, (M, N, K, fused)
+                    seen.add((fused, st))
+    assert len(seen) == 4                                                                    # both answers, both outputs

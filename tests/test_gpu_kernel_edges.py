@@ -122,6 +122,23 @@ def test_prepared_widths(bk, oracle, M, N, K, fused):
     assert bk.bcnn_device_error() == 0
 
 
+# the longest K: the int32 output's 256-wide tiles fit up to 274 176 bits of an odd number of words, and 37 x 4 of them would
+# be a whole wave; every output row of a sample
+@pytest.mark.parametrize("M,N,K", [(4736, 1024, 274144), (4736, 1024, 274208), (130, 70, 306912)])
+def test_prepared_longest_k(bk, oracle, M, N, K):
+    rng = np.random.default_rng(M + N + K)
+    A, W = synth.random_bits(rng, (M, K // 8)), synth.random_bits(rng, (N, K // 8))
+    assert bk.bcnn_prepared_preferred(1, M, 1, K, N, 1, 1, 1, 0, fused=False)
+    prep = torch.empty(bk.bcnn_prepared_weights_bytes(N, K), dtype=torch.uint8, device="cuda")
+    bk.bcnn_prepare_weights(dev(W), prep, N, K)
+    out = torch.empty(M, N, dtype=torch.int32, device="cuda")
+    bk.bcnn_gemm_b1_prepared(dev(A), prep, None, out, M, N, K)
+    torch.cuda.synchronize()
+    rows = np.array([0, 127, 128, M - 1])
+    assert np.array_equal(out.cpu().numpy()[rows], oracle.gemm(synth.unpack_bits(A[rows]), synth.unpack_bits(W)))
+    assert bk.bcnn_device_error() == 0
+
+
 # the stem's plain kernel and its table, on both sides of the line between them (148 * 2304 pixels), and with the ring of
 # chunks used more than once (148 * 5 * 1984 pixels), a bias for the per-channel path included
 @pytest.mark.parametrize("shape,inf", [((1, 9, 7), False), ((1, 576, 592), False), ((1, 577, 592), True), ((1, 579, 591), False), ((1, 1100, 1351), False),
