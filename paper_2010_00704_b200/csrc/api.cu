@@ -511,6 +511,8 @@ const char *bcnn_status_string(int status)
     case 174: return "device wait timed out: module engine, epilogue waiting for an identity tile or a free staging tile";
     case 175: return "device wait timed out: module engine, loader waiting for a free staging tile";
     case 176: return "device wait timed out: module engine, store warp waiting for an output tile";
+    case 181: return "device wait timed out: fused stem, loader waiting for a free ring stage";
+    case 182: return "device wait timed out: fused stem, worker waiting for a chunk of pixels";
     case BCNN_SELFTEST_TIMEOUT_CODE: return "device wait timed out: self-test (expected)";
     default: return status > 0 ? "device-side error code" : "unknown status";
     }

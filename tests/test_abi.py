@@ -95,3 +95,16 @@ def test_prepared_call_takes_what_it_is_preferred_for():
                     assert not preferred or st == binding.ERR_CUDA, (M, N, K, fused)
                     seen.add((fused, st))
     assert len(seen) == 4                                                                    # both answers, both outputs
+
+
+def test_every_wait_code_has_a_name():
+    # the codes as the kernels define them, each in one place
+    from paper_2010_00704_b200 import build, binding
+    build.build()
+    codes = {}
+    for src in build.sources():
+        for name, code in re.findall(r"\b(ERR_\w+) = (\d{3})\b", open(src).read()):
+            assert codes.setdefault(int(code), (src, name)) == (src, name), code
+    assert len(codes) >= 40 and {101, 131, 161, 171, 181, 182} <= set(codes)
+    for code, where in codes.items():
+        assert "timed out" in binding.status_string(code), where
