@@ -214,7 +214,9 @@ stem_c4r8_k32_kernel(const float4 *__restrict__ x, const float *__restrict__ bia
                 const uint32_t o = pixel(v[u]);
                 if (p0 + u * STEM_WORKERS < npix) __stcs(out + p0 + u * STEM_WORKERS, o);
             }
-            __syncwarp();                       // the words have been used: the stage may be refilled
+            // The stage may be refilled: its words have been used.  (With the arrival right behind the loads a refill can overtake
+            // them: seen in conv_tc_pn.cu, a few rows wrong in one launch of fifteen.)
+            __syncwarp();
             mbar_arrive_pred(empty(stage), lane0);
         }
     };

@@ -155,3 +155,44 @@ def test_stem_sizes(bk, oracle, shape, inf):
     torch.cuda.synchronize()
     want = oracle.threshold(oracle.conv2d(oracle.binarize(x, bias, 8), w, 1, 0), thr)
     assert np.array_equal(synth.unpack_bits(out.cpu().numpy().reshape(B, H, W, 4)), want)
+
+
+# Engines that refill a stage of shared memory by a bulk copy while the CTA works: many row tiles per CTA, the input in L2 (the
+# fastest refill), the call repeated.  A stage handed back too early shows as a few wrong words in some of the launches only (with
+# the arrival right behind the wide pointwise engine's loads one launch of fifteen: 200 pass by luck with probability 1e-6).
+@pytest.mark.parametrize("engine,shape", [("tc_pn", (1, 333 * 128 + 77, 1, 512, 512, 1, 1, 0)), ("tc_pn", (1, 148 * 9 * 128 + 5, 1, 256, 256, 1, 1, 0)),
+                                          ("tc_c3", (16, 128, 128, 64, 64, 3, 1, 1)), ("tc_c3", (8, 160, 176, 32, 64, 3, 2, 1)), ("tc_c3", (16, 128, 128, 64, 128, 3, 2, 1)),
+                                          ("tc_pw", (64, 112, 112, 32, 32, 1, 1, 0)), ("tc_pw", (64, 112, 112, 64, 64, 1, 1, 0)), ("tc_pw", (64, 56, 56, 128, 128, 1, 1, 0))])
+def test_stages_handed_back_in_every_launch(bk, engine, shape):
+    B, H, W, Ci, Co, k, stride, pad = shape
+    rng = np.random.default_rng(9950 + sum(shape))
+    OH, OW = bk.out_hw(H, W, k, k, stride, pad)
+    x, w = dev(synth.random_bits(rng, (B * H * W, Ci // 8))), dev(synth.random_bits(rng, (Co, k * k * Ci // 8)))
+    thr = dev(synth.thresholds(rng, k * k * Ci, Co))
+    ref, out = (torch.empty(B * OH * OW, Co // 8, dtype=torch.uint8, device="cuda") for _ in range(2))
+    bk.bcnn_conv2d_b1_fused(x, w, thr, ref, B, H, W, Ci, Co, k, k, stride, pad, engine=bk.ENGINES["tc_ws"])     # (checked against the oracle elsewhere)
+    wrong = torch.zeros((), dtype=torch.int64, device="cuda")
+    for _ in range(200):
+        out.fill_(0xA5)
+        bk.bcnn_conv2d_b1_fused(x, w, thr, out, B, H, W, Ci, Co, k, k, stride, pad, engine=bk.ENGINES[engine])
+        wrong += (out != ref).any()
+    assert int(wrong) == 0
+    assert bk.bcnn_device_error() == 0
+
+
+# ... and the stem, seventeen chunks a CTA through its ring of five, against the two separate calls
+def test_stem_stages_handed_back_in_every_launch(bk):
+    B, H, W = 100, 224, 224
+    rng = np.random.default_rng(9960)
+    x = torch.randn(B * H * W * 4, device="cuda", generator=torch.Generator(device="cuda").manual_seed(9960))
+    bias, w, thr = dev(synth.real_input(rng, (32,))), dev(synth.random_bits(rng, (32, 4))), dev(synth.thresholds(rng, 32, 32))
+    bits, ref, out = (torch.empty(B * H * W * 4, dtype=torch.uint8, device="cuda") for _ in range(3))
+    bk.bcnn_pack(x, bias, bits, B, H, W, 4, 8)
+    bk.bcnn_conv2d_b1_fused(bits, w, thr, ref, B, H, W, 32, 32, 1, 1, 1, 0, engine=bk.ENGINES["lop3"])
+    wrong = torch.zeros((), dtype=torch.int64, device="cuda")
+    for _ in range(200):
+        out.fill_(0xA5)
+        bk.bcnn_stem_fused(x, bias, w, thr, out, B, H, W, 4, 8, 32)
+        wrong += (out != ref).any()
+    assert int(wrong) == 0
+    assert bk.bcnn_device_error() == 0
