@@ -482,7 +482,11 @@ int launch_bn(const ConvProblem &p0, cudaStream_t stream)
     const int ktw = ktab_words_for(p);
     const int smem = smem_bytes<BN>(ktw, p.mode);
     if (smem > MAX_SMEM) return BCNN_ERR_UNSUPPORTED;
-    void (*k)(const ConvProblem, const int) = p.mode == 2 ? conv_tc_i8_kernel<BN, 2> : (p.mode == 1 ? conv_tc_i8_kernel<BN, 1> : conv_tc_i8_kernel<BN, 0>);
+    void (*k)(const ConvProblem, const int) = p.mode == 1 ? conv_tc_i8_kernel<BN, 1> : conv_tc_i8_kernel<BN, 0>;
+    if (p.mode == 2) {
+        if constexpr (BN == 128) k = conv_tc_i8_kernel<BN, 2>;      // (launch_conv_tc_i8 gives the module no other width)
+        else return BCNN_ERR_UNSUPPORTED;
+    }
     if (!allow_smem((const void *)k, MAX_SMEM)) return BCNN_ERR_CUDA;
     return launch(k, grid, Cfg<BN>::THREADS, smem, stream, p, ktw);
 }

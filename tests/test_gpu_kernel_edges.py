@@ -8,7 +8,7 @@ import torch
 from paper_2010_00704_b200 import synth
 from test_gpu_block import bk, dev, test_avgpool as check_avgpool, test_dwconv3x3_module as check_dwconv   # noqa: F401 (bk: a fixture)
 from test_gpu_block import test_fxf_as_shifted_branches as check_shifted, test_parallel_branches as check_branches   # noqa: F401
-from test_gpu_parity import run_conv
+from test_gpu_parity import run_conv, test_conv_module as check_module   # noqa: F401
 
 pytestmark = pytest.mark.gpu
 
@@ -36,6 +36,15 @@ def test_branches_many_parts(bk, oracle, shape):
 @pytest.mark.parametrize("shape", [(16, 40, 40, 32, 64, 3), (2, 30, 31, 224, 96, 3)])
 def test_shifted_branches_many_parts(bk, oracle, shape):
     check_shifted(bk, oracle, shape, "paper")
+
+
+# the module on the streaming engine: 3 x 3 layers whose resident weights fit beside no producer group (11 stages of 96 channels, 20 of
+# 320); one 128-wide tile column and three with a ragged last one, more row tiles than multiprocessors.  32 channels of that K
+# fit the weight-stationary engine, one block per multiprocessor
+@pytest.mark.parametrize("variant", ["full", "no_identity", "no_bits", "in_place"])
+@pytest.mark.parametrize("shape", [(2, 100, 99, 288, 96, 3, 1, 1), (1, 9, 10, 544, 320, 3, 1, 1), (1, 13, 7, 544, 32, 3, 2, 1)])
+def test_module_long_k(bk, oracle, shape, variant):
+    check_module(bk, oracle, shape, variant)
 
 
 # packing: pixels that are no whole number of passes (bias in registers or by remainder), NaN and -0, the replicated widths
