@@ -33,6 +33,21 @@ def test_branches_many_parts(bk, oracle, shape):
     check_branches(bk, oracle, shape, "full")
 
 
+# the CUDA-core kernel: more branches than the engine has accumulators for, several slices of channels, many row tiles;
+# and a K beyond the engine's constants, where one branch is compared with another kernel's module besides (for a shorter K both
+# calls run on the same engine)
+@pytest.mark.parametrize("variant", ["full", "no_identity", "in_place", "no_bits"])
+@pytest.mark.parametrize("shape", [(2, 7, 9, 32, 320, 20), (3, 60, 61, 32, 32, 14), (1, 9, 11, 2624, 64, 1)])
+def test_branches_cuda_cores(bk, oracle, shape, variant):
+    check_branches(bk, oracle, shape, variant)
+
+
+@pytest.mark.parametrize("reading", ["paper", "zero"])
+@pytest.mark.parametrize("shape", [(2, 9, 13, 32, 64, 5), (1, 5, 33, 96, 32, 5)])
+def test_shifted_branches_cuda_cores(bk, oracle, shape, reading):
+    check_shifted(bk, oracle, shape, reading)
+
+
 @pytest.mark.parametrize("shape", [(16, 40, 40, 32, 64, 3), (2, 30, 31, 224, 96, 3)])
 def test_shifted_branches_many_parts(bk, oracle, shape):
     check_shifted(bk, oracle, shape, "paper")
