@@ -821,7 +821,7 @@ def run_paper1x1(args):
     for l, count in convs:
         ms = float(np.mean([a.elapsed_time(b) for a, b in per[l.name]]))
         shapes.append({"layer": l.name, "count": count, "M": l.M(B), "N": l.C_out, "K": l.K,
-                       "engine": ("branches (CUDA cores)" if branch_call else "tc_ws") if module
+                       "engine": "tc_mod" if module
                        else ("tc_pre" if binding.bcnn_prepared_preferred(B, l.H, l.W, l.C_in, l.C_out, 1, 1, 1, 0)
                              else binding.bcnn_auto_engine(B, l.H, l.W, l.C_in, l.C_out, 1, 1, 1, 0)),
                        "ms_per_launch": ms, "tops": PB * l.ops(B) / (ms / 1e3) / 1e12})

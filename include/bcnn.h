@@ -46,8 +46,8 @@ typedef enum bcnn_status {
     BCNN_ERR_UNSUPPORTED = -2, /* channel count not a multiple of 32, size limits */
     BCNN_ERR_ALIGNMENT = -3,   /* a data pointer is not 16-byte aligned */
     BCNN_ERR_CUDA = -4,        /* the CUDA runtime refused a launch */
-    BCNN_ERR_WORKSPACE = -5,   /* a caller-provided scratch buffer is too small (no call takes one today:
-                                  bcnn_workspace_bytes() is 0 for every shape; the value is reserved) */
+    BCNN_ERR_WORKSPACE = -5,   /* bcnn_conv2d_b1_fused_noalloc: the layer's prepared weights exceed the library's static
+                                  array (no call takes a scratch buffer: bcnn_workspace_bytes() is 0 for every shape) */
     BCNN_ERR_TIMEOUT = -6      /* a bounded device-side wait gave up (see bcnn_device_status) */
 } bcnn_status;
 

@@ -73,20 +73,23 @@ int make_conv_problem(ConvProblem &p, const void *x, const void *w, const int32_
     return BCNN_OK;
 }
 
-// Measured on B200 (bench.py --mode sweep):
+// Which engine, in this order.  Times on B200: single launches with L2 flushed before them (bench.py --mode sweep), or, marked
+// "row", launches in a row.
 //   * pointwise layers (1x1, stride 1, no padding; GEMMs) with K <= 128 and C_out <= 128, packed output: pointwise
-//     tcgen05 engine (memory-bound shapes: rows bulk-copied in chunks, one hand-over per chunk);
+//     tcgen05 engine (memory-bound shapes: rows bulk-copied in chunks, one hand-over per chunk; 64 -> 64 at M = 3211264: 30 us,
+//     weight-stationary 69; 128 -> 128 at M = 802816: 20, wide pointwise 28);
+//   * the smallest calls with K <= 256: CUDA cores;
 //   * pointwise layers with K = 128, 256 or 512 and a multiple of 128 output channels, packed output: wide pointwise tcgen05
-//     engine (a row tile expanded once for all resident weight slices; 1.5 - 3x the weight-stationary engine);
+//     engine (a row tile expanded once for all resident weight slices; 256 -> 256 at M = 802816: 35 us, weight-stationary 74;
+//     512 -> 512 at M = 50176: 16 and 23);
 //   * 3x3 layers (stride 1 or 2) on 32 or 64 input channels with C_out <= 128, packed output, whose 8 x 16 output tiles
 //     are at least three quarters full: halo-tile tcgen05 engine (input tiles by tiled TMA copies);
-//   * 1x1 layer with C_in = 32 and C_out <= 32 (one XOR + popcount per output): CUDA-core pointwise kernel;
+//   * 1x1 layer with C_in = 32 and C_out <= 32, int32 output: one XOR + popcount per output on the CUDA cores;
 //   * many rows of C_out <= 128 with K >= 64, or of wider layers with K <= 2304 (in 128-channel slices): weight-stationary
 //     tcgen05 engine;
-//   * other K = 32 layers: register-fed warp-level int8 engine;
+//   * other layers of C_out <= 64, those with K = 32 (strided, or int32 output): register-fed warp-level int8 engine;
 //   * everything else: streaming tcgen05 engine;
-//   * CUDA-core engine: the smallest calls with K <= 256;
-//   * the single-bit mma.sync engine never wins and serves as a fallback.
+//   * the single-bit mma.sync engine is nowhere the fastest (4096 x 4096 x 9216: 835 us, streaming 106) and serves as a fallback.
 int auto_engine(const ConvProblem &p)
 {
     // at every size, the smallest included: 2.4 .. 2.9 us up to M = 12544, against 3.0 .. 5.9 of the CUDA-core engine
@@ -95,10 +98,14 @@ int auto_engine(const ConvProblem &p)
     // weights expanded (1x1 256 -> 256 at M = 196: 3.3 against 4.2 us; 256 -> 128 at M = 3136: 5.3 against 4.2)
     if (p.K <= 256 && ((p.M + 63L) / 64) * ((p.C_out + 63) / 64) <= sm_count() / 2) return BCNN_ENGINE_LOP3;
     if (conv_tc_pn_supports(p)) return BCNN_ENGINE_TC_PN;
+    // full tiles: 64 -> 64 at 28 x 28, 256 images, row: 8.9 us, weight-stationary 12.9.  A tile that is part empty costs as much as
+    // a full one; the line is on the safe side (20 x 20, half full: 64 -> 128 11.9 and 11.7 us, but 64 -> 64 7.8 and 9.6)
     if (conv_tc_c3_supports(p)) {
         const long covered = (long)((p.OH + 7) / 8 * 8) * ((p.OW + 15) / 16 * 16);
         if (4L * p.OH * p.OW >= 3L * covered) return BCNN_ENGINE_TC_C3;
     }
+    // (int32 output only, row, against the weight-stationary engine: 45 and 25 us at M = 802816, 6.2 and 4.6 at 12544 - the packed
+    // output, for which this line was drawn, runs on the pointwise engine today)
     if (conv_lop3_pointwise_k32(p)) return BCNN_ENGINE_LOP3;
     // Up to 128 output channels: the weight-stationary engine, unless its CTAs would expand all the weights for less than two
     // waves of 64-wide tiles of the streaming engine (3x3 128 -> 128: 7.6 against 5.0 us at M = 784, 8.3 against 7.0 at 12544;
@@ -113,6 +120,8 @@ int auto_engine(const ConvProblem &p)
     // tiles to share one slice's weights (4096 x 4096 x 2304 int32: 33.3 against 38.8 us, 3x3 256 -> 256 at M = 50176: 20.8
     // against 27.3; 1024 x 1024 x 512: 7.9 against 5.5)
     if (p.C_out > 128 && p.K <= 2304 && ((p.M + 127L) / 128) * ((p.C_out + 127) / 128) >= 2L * sm_count() && conv_tc_ws_supports(p)) return BCNN_ENGINE_TC_WS;
+    // K = 32, row: 1x1/2 32 -> 64 packed at M = 50176 5.2 us, streaming 6.4; 32 -> 64 int32 at M = 200704 14.3 and 18.2.  At 128 channels
+    // 8.3 and 7.5 packed, 23.9 and 32.3 int32
     if (p.C_out <= 64 && conv_mma_s8_supports(p)) return BCNN_ENGINE_MMA_S8;
     if (conv_tc_i8_supports(p)) return BCNN_ENGINE_TC_I8;
     if (conv_mma_b1_supports(p)) return BCNN_ENGINE_MMA_B1;
@@ -401,9 +410,10 @@ int bcnn_prepared_preferred(int B, int H, int W, int C_in, int C_out, int kh, in
     const int st = make_conv_problem(p, dummy, dummy, fused ? static_cast<const int32_t *>(dummy) : nullptr, dummy,
                                      B, H, W, C_in, C_out, kh, kw, stride, pad, fused != 0);
     if (st != BCNN_OK) return 0;
-    // Measured: streaming prepared weights wins wherever AUTO would expand them on every call - the streaming engine always,
-    // the weight-stationary one except on many rows of a short K, where its expansion is spread thin (56x56 64 -> 128 /2 at
-    // batch 256, M = 200704, K = 576: 16.1 against 18.2 us; K = 1152: 19.7 against 19.0; M = 784: 6.5 against 4.0).  The wide
+    // Measured: streaming prepared weights wins where AUTO would expand them on every call - the streaming engine always, the
+    // weight-stationary one except on many rows of a short K, where its expansion is spread thin (56x56 64 -> 128 /2 at
+    // batch 256, M = 200704, K = 576: 16.1 against 18.2 us; K = 1152: 19.7 against 19.0; M = 784: 6.5 against 4.0; wide pointwise
+    // layers sit on the other side of the line, 1024 -> 1024 at M = 50176 39 against 49, at 12544 13.5 against 14.8).  The wide
     // pointwise and halo-tile engines keep their layers, all but the smallest with many weights: they expand those at the start.
     if (!conv_tc_pre_supports(p)) return 0;
     switch (auto_engine(p)) {
@@ -417,6 +427,8 @@ int bcnn_prepared_preferred(int B, int H, int W, int C_in, int C_out, int kh, in
         // (1x1 512 -> 128 at M = 12544: 5.2 against 4.4, 256 -> 256: 5.0 against 5.7)
         return ((p.M + 127L) / 128) * ((p.C_out + 63) / 64) <= sm_count() * 3 / 2 ? 1 : 0;
     case BCNN_ENGINE_TC_WS: return p.K >= 1024 || p.M < 98304 ? 1 : 0;
+    // packed, row: 1x1 160 -> 256 at M = 900 5.5 against 4.1 us, 96 -> 256 at M = 196 3.7 against 3.7 (in a graph 3.3 and 3.2); K = 64 at M = 100
+    // 3.5 and 3.6.  int32, in a graph, the other way round: 1x1 128 -> 128 at M = 784 3.3 against 3.8, 96 -> 64 at M = 196 3.1 against 3.5
     case BCNN_ENGINE_LOP3: return p.K <= 64 ? 0 : 1;
     default: return 1;
     }

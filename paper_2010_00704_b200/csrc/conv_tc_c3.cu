@@ -10,7 +10,7 @@
 //     memory.  Out-of-image rows and pixels are the copy's zero fill = the -1 padding: no tap masks anywhere.  The
 //     copy's first word must be 16-byte aligned, so the box starts up to three pixels left of the halo (XOFF);
 //   * a producer thread (= one output pixel) reads its nine pixels' words from the halo tile at compile-time offsets,
-//     expands them and stores them to tensor memory: per K word one shared-memory load and the eight logic operations.
+//     expands them and stores them to tensor memory: per K word one shared-memory load and five logic operations.
 // Arithmetic: 4-bit operands (tc_common.cuh), fp32 accumulators that hold exact integers, the per-channel constants written by
 // a first MMA so that the epilogue needs 16 bits and a sign (tc_slot.cuh).
 //

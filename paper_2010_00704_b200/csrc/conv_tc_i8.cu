@@ -5,7 +5,7 @@
 // Persistent, warp-specialised; each CTA walks a static list of 128 x BN tiles.
 //   warp 0          issuer: tcgen05.mma / commit only, waits on named barriers only (a memory
 //                   instruction after tensor-core instructions would stall it)
-//   warps 1-4       epilogue: tcgen05.ld, threshold + pack (or int32), hand the accumulator back
+//   warps 1-4       epilogue: tcgen05.ld, threshold + pack (or int32, or the module), hand the accumulator back
 //   G = 2 producer groups, each 4 activation warps + BN/32 weight warps, one thread per tile
 //                   row; the groups take the ring's stages alternately so that one group gathers
 //                   while the other expands.  Packed words are staged with cp.async (16 bytes per
@@ -14,8 +14,8 @@
 //                       MMA takes A from tensor memory, so shared memory carries only weights
 //                     weight rows     -> shared memory, 128-byte-swizzled K-major tiles
 //   last warp       control: does the issuer's mbarrier waits and releases it stage by stage
-// A ring stage is 256 bits of K.  Tensor memory (512 columns): BN = 256: one accumulator + 4 ring stages; BN = 128: two
-// accumulators + 7 ring stages, and the unit scales.  Column popcounts are taken from the words as they are
+// A ring stage is 256 bits of K.  Tensor memory (512 columns): BN = 256: one accumulator + 4 ring stages; BN = 128 and 64:
+// two accumulators + 7 ring stages, and the unit scales.  Column popcounts are taken from the words as they are
 // expanded; each group leaves its partial constants for a tile in shared-memory slots.
 // Every mbarrier wait is bounded and reports through the device error word.
 #include "tc_common.cuh"
@@ -60,8 +60,8 @@ template <int BN>
 __host__ __device__ inline int smem_bytes(int ktab_words, int mode = 1)
 {
     using C = Cfg<BN>;
-    // module epilogue: + the identity staging ring; int32 output of the 128-wide tiles: + the store staging tiles
-    // (both only used where they fit: 128-wide tiles)
+    // module epilogue (128-wide tiles only): + the identity staging ring; int32 output of the 128- and 64-wide tiles: + the store
+    // staging tiles (beside 256-wide tiles they do not fit)
     return 1024 + C::STAGES * C::W_BYTES + C::BITS_BYTES + C::CONST_BYTES + C::TABLE_BYTES + ktab_words * 4 +
            (mode == 2 ? ID_RING_BYTES + 16 : 0) + (mode == 0 && BN <= 128 ? EPI_WARPS * I32_TILE_BYTES + 16 : 0);
 }
@@ -506,21 +506,25 @@ bool conv_tc_i8_supports(const ConvProblem &p)
 int launch_conv_tc_i8(const ConvProblem &p, cudaStream_t stream)
 {
     if (!conv_tc_i8_supports(p)) return BCNN_ERR_UNSUPPORTED;
-    // 256-wide tiles have a single accumulator buffer (tensor memory also holds the activation
-    // ring), so their epilogue is not overlapped: worth it only when the K loop is long
-    // (the module epilogue's staging ring only fits beside the 128-wide tiles' weight ring)
-    // (int32 output up to K = 4608: the 128-wide tiles' staged stores, whole 128-byte rows, outweigh their extra expansion)
+    // 256-wide tiles have a single accumulator buffer (tensor memory also holds the activation ring), so their epilogue is not
+    // overlapped: worth it only when the K loop is long.  The module epilogue's staging ring only fits beside the 128-wide tiles'
+    // weight ring.  int32 output up to K = 4608: the 128-wide tiles' staged stores, whole 128-byte rows, outweigh their extra
+    // expansion (4096 x 4096 x 4608: 63.5 against 75.2 us; at 9216 112 against 117, but 16384 x 16384 x 9216 1680 against 1550).
     if (p.C_out > 128 && p.kwords >= 24 && p.mode != 2 && !(p.mode == 0 && p.kwords <= 144)) {
-        // ... unless the narrower tiles fill the last wave so much better that they win anyway: a 128-wide tile
-        // costs about 0.6 of a 256-wide one (measured on the K = 2304 and K = 4608 layers)
+        // ... unless the narrower tiles fill the last wave so much better that they win anyway.  A 128-wide tile costs 0.61 of a
+        // 256-wide one at K = 9216, 0.57 at 4608, 0.51 at 2304 and 0.41 at 768 (16384 x 16384: 1545 : 1284, 807 : 712, 424 : 423 and
+        // 181 : 225 us), so the line is right for the long K: 4096 x 4096 x 9216 102.7 (128) : 97.9, x 4608 56.0 : 56.2, 12544 x 512 x
+        // 4608 29.3 : 31.9; below K = 2304 it is a little early (4096 x 4096 x 768 16.0 : 19.7), and a single wave of 256-wide tiles
+        // would win from K = 4608 on (2048 x 2048: 19.8 : 18.2)
         const int sms = sm_count();
         const long m_tiles = ((long)p.M + BM - 1) / BM;
         const long waves256 = (m_tiles * ((p.C_out + 255) / 256) + sms - 1) / sms;
         const long waves128 = (m_tiles * ((p.C_out + 127) / 128) + sms - 1) / sms;
         if (waves256 > 1 && 10 * waves256 <= 6 * waves128) return launch_bn<256>(p, stream);
     }
-    // small problems: 64-wide tiles on twice the multiprocessors, with a shorter epilogue.  A tile column costs about 0.42 us per
-    // 256-bit stage at 128 and 0.33 at 64, the start 0.5 us less (1024 x 1024 x 4608: 12.3 -> 10.2 us, 20 x 64 x 960: 5.3 -> 4.7)
+    // small problems: 64-wide tiles on twice the multiprocessors, with a shorter epilogue.  A tile column of one wave costs about
+    // 0.42 us per 256-bit stage at 128 and 0.33 at 64, the start 0.5 us less (1024 x 1024 x 4608: 12.3 -> 10.2 us, 20 x 64 x 960:
+    // 5.3 -> 4.7; many waves 0.37 and 0.29 per stage and 0.5 per tile: 16384 x 16384 x 9216 1545 and 2385)
     const int sms = sm_count();
     const long m_tiles = ((long)p.M + BM - 1) / BM, kt = (p.kwords + 7) / 8;
     const long w64 = (m_tiles * ((p.C_out + 63) / 64) + sms - 1) / sms, w128 = (m_tiles * ((p.C_out + 127) / 128) + sms - 1) / sms;

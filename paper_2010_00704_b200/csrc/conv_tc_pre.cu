@@ -1,4 +1,4 @@
-// Streaming tcgen05 engine on PREPARED weights: wide layers and long K (C_out > 128, the plain GEMMs).
+// Streaming tcgen05 engine on PREPARED weights: wide layers, long K, small layers, the plain GEMMs.
 //
 // The weights of a layer never change between calls.  bcnn_prepare_weights expands their sign bits ONCE per layer into a
 // caller-owned buffer - signed 4-bit codes, K-major, rows padded to 128 and K to 256, then K - 2 popc(W_n) per row; half
@@ -13,11 +13,19 @@
 // so there are no per-row constants, and the per-column ones are added by the epilogue from a small table.
 //
 //   warp 0        issuer (tcgen05.mma / commit only; waits on named barriers only)
-//   warps 1-4     epilogue: build the tile's column table, tcgen05.ld, add + sign bits (or int32), store
+//   warps 1-4     epilogue (256-wide and int32 128-wide tiles: 1-8, two teams with half of the columns each): build the tile's
+//                 column table, tcgen05.ld, add + sign bits (or int32), store
 //   G groups of 4 activation warps: implicit-im2col gather (cp.async), expansion, tcgen05.st into the ring in tensor memory
 //   loader warp   weight tiles by TMA into the ring in shared memory
 //   control warp  the issuer's mbarrier waits
 // Every mbarrier wait is bounded and reports through the device error word.
+//
+// What bounds it.  256-wide tiles: the K loop runs at the tensor pipe's rate (16384 x 16384, packed, K = 2304 / 4608 / 9216: 240 / 385 /
+// 670 us, 0.283 us per 256-bit stage and tile, the probe's rate; the expansion is hidden), and with one accumulator buffer the epilogue
+// is not overlapped: 1.8 us per packed and 4.9 us per int32 tile with the pipe idle (842 us at K = 9216).  128- and 64-wide tiles have
+// two and four buffers; they take 185 and 167 ns per stage against 141 and 71 of the pipe, and 0.6 us a packed tile (one epilogue team,
+// which builds its column table anew for every tile).  No unit is saturated there: 3x3 128 -> 128 at M = 200704 has the tensor pipe
+// active 35 % of the time, the logic pipe 36 %, the issue slots 49 %.
 #include "tc_common.cuh"
 #include "tensor_map.cuh"
 #include <climits>

@@ -15,7 +15,7 @@
 //   * Tensor memory is cut into NSLOT slots of T tiles (accumulator + expanded activation tile each).  Every slot is
 //     a pipeline of its own - one issuer warp, one producer group and one epilogue group of four warps - and takes
 //     the chunks slot, slot + NSLOT, ...  Per chunk there is ONE hand-over in each direction: the producers expand
-//     all T tiles (ld.shared, 8 logic operations per word, tcgen05.st) and arrive once; the issuer issues all MMAs
+//     all T tiles (ld.shared, 5 logic operations per word, tcgen05.st) and arrive once; the issuer issues all MMAs
 //     back to back and commits once; the epilogue reads the T accumulators and hands the slot back as soon as
 //     they are in registers.  An issuer only ever waits for MMAs that completed a whole slot cycle ago, so it can
 //     do its own mbarrier waits.  (An issuer that waits right behind its own MMAs stalls until they drain: with one

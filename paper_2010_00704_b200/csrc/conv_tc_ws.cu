@@ -41,7 +41,7 @@ constexpr int ERR_EPILOGUE_TIMEOUT = 113;
 // DUAL: two CTAs share an SM (two independent MMA issuers), each with half of tensor memory.
 // TEAMS: epilogue teams of four warps; team t takes the tiles t, t + TEAMS, ... of the CTA (their accumulator
 // buffers are then a fixed subset, so NBUF is a multiple of TEAMS).  Two teams serve the module epilogue, which is
-// bound by the epilogue warps.
+// bound by the epilogue warps, and the 128-wide slices with one CTA per SM.
 template <int BN, int G, bool DUAL, int TEAMS = 1> struct Cfg {
     static constexpr int FIRST_PRODUCER_THREAD = 32 * (1 + EPI_WARPS * TEAMS);
     static constexpr int PROD_THREADS = G * BM;

@@ -1,4 +1,4 @@
-// Helpers of the slot-pipeline engines (conv_tc_pw.cu, conv_tc_c3.cu): tensor-memory loads that do not wait, the
+// Helpers of the pipelines without a control warp (conv_tc_pw.cu, conv_tc_pn.cu, conv_tc_c3.cu, conv_tc_mod.cu; the waits: stem.cu): tensor-memory loads that do not wait, the
 // register pin that keeps uses behind the wait, the short-sleep bounded mbarrier wait, and the sign-bit gathering
 // from packed 16-bit accumulator halves.
 #pragma once

@@ -97,7 +97,7 @@ def test_parallel_branches(bk, oracle, shape, variant):
     if s is not None:
         assert np.array_equal(s, want_s)
     if P == 1 and variant == "full":
-        # ... and for one branch the tensor-core module call gives the same bits
+        # ... and for one branch the module call gives the same bits (the same kernel up to K = 2560)
         yreal = torch.empty(B * H * W * Co * 2, dtype=torch.uint8, device="cuda")
         ybits = torch.empty(B * H * W * Co // 8, dtype=torch.uint8, device="cuda")
         xb = torch.empty(B * H * W * Ci // 8, dtype=torch.uint8, device="cuda")

@@ -551,13 +551,13 @@ def test_bounded_wait_runs_out_and_is_reported(bk, oracle):
 
 MODULE_SHAPES = [
     # B, H, W, Ci, Co, k, stride, pad
-    (2, 9, 13, 64, 64, 1, 1, 0),       # weight-stationary engine, the paper's 1x1 module shape
+    (2, 9, 13, 64, 64, 1, 1, 0),       # pointwise: the module engine; the paper's 1x1 module shape
     (1, 20, 20, 128, 128, 1, 1, 0),
-    (2, 12, 10, 64, 96, 3, 2, 1),      # 3x3 stride 2, ragged N tile
-    (3, 7, 11, 32, 32, 1, 1, 0),       # one-word K: streaming engine
-    (1, 14, 14, 256, 256, 1, 1, 0),    # streaming engine, 256-wide tile
-    (2, 7, 7, 512, 1024, 1, 1, 0),     # several N tiles
-    (1, 10, 10, 128, 320, 3, 1, 1),    # ragged N tile of the streaming engine, K = 1152
+    (2, 12, 10, 64, 96, 3, 2, 1),      # 3x3 stride 2: the weight-stationary engine; ragged N tile
+    (3, 7, 11, 32, 32, 1, 1, 0),       # one-word K
+    (1, 14, 14, 256, 256, 1, 1, 0),    # eight slices of 32 channels
+    (2, 7, 7, 512, 1024, 1, 1, 0),     # 32 slices, K = 512
+    (1, 10, 10, 128, 320, 3, 1, 1),    # 3x3, 32-channel slices of the weight-stationary engine, K = 1152
 ]
 
 
