@@ -19,7 +19,7 @@
 // Bound by memory (16 bytes per pixel in, 4 out).  A thread that loads its own pixels has nothing in flight while it computes
 // (about 70 instructions a pixel, half of the time), so the pixels arrive by bulk copies into a ring in shared memory: 155 KB
 // in flight per multiprocessor, the first of them while the tables are built.  256 images of 224 x 224: 51.5 us with loads by
-// the threads, 46.3 with the ring, 42.5 (6.05 TB/s; a copy reaches 6.46) with the shorter table build; 16 images 9.6 -> 7.9.
+// the threads, 46.3 with the ring, 42.5 - 43.8 (5.9 - 6.05 TB/s; a copy reaches 6.5) with the shorter table build; 16 images 9.6 -> 7.9.
 //
 // The table pays for itself only when a CTA has many pixels: up to PLAIN_PIXELS per multiprocessor the plain per-channel path
 // runs in a kernel of its own, spread over all of them (one 224 x 224 image 2.5 us against 6.0, four 5.4 against 6.1).
