@@ -410,8 +410,8 @@ int bcnn_prepared_preferred(int B, int H, int W, int C_in, int C_out, int kh, in
     const int st = make_conv_problem(p, dummy, dummy, fused ? static_cast<const int32_t *>(dummy) : nullptr, dummy,
                                      B, H, W, C_in, C_out, kh, kw, stride, pad, fused != 0);
     if (st != BCNN_OK) return 0;
-    // Measured: streaming prepared weights wins where AUTO would expand them on every call - the streaming engine always, the
-    // weight-stationary one except on many rows of a short K, where its expansion is spread thin (56x56 64 -> 128 /2 at
+    // Measured: streaming prepared weights wins where AUTO would expand them on every call - the streaming engine, short K of a
+    // wide packed product apart (16384 x 16384: K = 2304 240 against 434 us, K = 512 227 against 166), the weight-stationary one except on many rows of a short K, where its expansion is spread thin (56x56 64 -> 128 /2 at
     // batch 256, M = 200704, K = 576: 16.1 against 18.2 us; K = 1152: 19.7 against 19.0; M = 784: 6.5 against 4.0; wide pointwise
     // layers sit on the other side of the line, 1024 -> 1024 at M = 50176 39 against 49, at 12544 13.5 against 14.8).  The wide
     // pointwise and halo-tile engines keep their layers, all but the smallest with many weights: they expand those at the start.
