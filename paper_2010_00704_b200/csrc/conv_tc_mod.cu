@@ -7,11 +7,13 @@
 //   * identity tiles arrive and output tiles leave by tiled TMA copies of 128 rows x BN channels through a ring of NS tiles per
 //     epilogue team in shared memory (swizzled: one 16-byte access per lane and row without bank conflicts); a loader warp and a
 //     store warp issue them (an issue costs its warp some 500 cycles), the epilogue turns a tile in place;
-//   * per-channel values lie in shared memory as pairs of channels, read as 16-byte broadcasts - four cycles of the shared-memory
-//     pipe each, the epilogue's scarcest resource: one per branch {scale, shift} and one {slope, next bias}.  The constant
-//     K - 2 popc of a dot product is not among them, an MMA against a constant tile puts it into the accumulator
-//     (tc_slot.cuh);
-//   * the arithmetic runs on pairs (f32x2: the same IEEE operations, half the issue slots);
+//   * accumulators are loaded so that a lane holds a quarter of a part's channels of four rows (16x256b; the weights' rows are
+//     permuted to make them consecutive channels): a channel's values - per branch {scale, shift}, then {slope, sign threshold}, pairs of
+//     channels in 16 bytes - are fetched once for four rows, the four rows are independent chains, and sign bits end in whole
+//     bytes.  With a row per lane a P = 2 part took 3800 cycles of a team, now 2640 (P = 1: 2150, 1780).  The constant K - 2 popc of a
+//     dot product is not among them, an MMA against a constant tile puts it into the accumulator (tc_slot.cuh);
+//   * the arithmetic runs on pairs (f32x2: the same IEEE operations, half the issue slots); PReLU is a compare and a predicated product; the
+//     next sign is one fp16 compare per pair against the smallest fp16 value that passes;
 //   * two epilogue teams take alternate PARTS (128 rows x BN channels).
 // The binary products are cheap beside that: a CTA keeps RS slices of BN channels' expanded weights in shared memory, expands
 // a row tile once (256-bit stages in a ring in tensor memory, as in conv_tc_ws.cu) and multiplies it against every resident
@@ -22,6 +24,10 @@
 // "Part full" barriers form a ring of MAX_NBUF, not of the accumulator buffers in use: a parity wait for part n is right once
 // part n - MAX_NBUF is done, and the team has seen part n - TEAMS done (with one buffer and two teams the second team's first
 // wait would pass on the barrier's empty history).
+// What a launch does once - weights, parameters, constants - is written as small rolled loops with its divisions prepared on the host: an
+// instruction that runs for the first time costs some ten cycles, and unrolled eight times this set-up took 5 us.  In microseconds,
+// before and after: P = 2, 256 channels, M = 50176: 22.0, 17.7; P = 3, 160 channels, M = 96228: 47.7, 31.8; P = 3, 96 channels, M = 10496: 10.1, 7.6;
+// nine taps, 128 channels, M = 12544: 31.1, 19.9; P = 1, 128 channels: M = 1782 4.9, 3.9, M = 153064 18.8, 15.9 (12.3 of the maps' traffic).
 // Every mbarrier wait is bounded and reports through the device error word.
 #include "tc_slot.cuh"
 #include "tensor_map.cuh"
@@ -53,12 +59,15 @@ struct ModPlan {
     int stages;               // ring slots
     int nbuf;                 // accumulator buffers
     int rs, ng, slices;       // resident slices, CTA groups, slices of BN channels
-    int m_tiles;
+    int m_tiles, step;        // row tiles; CTAs of a group
+    uint32_t ng_mul, ng_shift, step_mul, step_shift;      // exact_div by ng and step
+    uint32_t kwp_mul, kwp_shift, row_mul, row_shift;      // ... by kwp and by the gw-word pieces of a branch's weight row
+    TileStep ts;              // from a row tile to the CTA's next
     int units, gw;            // gather units of a row
-    uint32_t off_bits, off_stage, off_table, off_pad, off_pop, off_tab, off_const;      // shared-memory offsets from the 1024-byte aligned base (weights first)
+    uint32_t off_bits, off_stage, off_table, off_pad, off_tab, off_const, off_raw;      // shared-memory offsets from the 1024-byte aligned base (weights first)
 };
 
-// per-channel-pair table of a slice: P entries of 16 bytes {scale, shift} x 2, then 16 bytes {slope, next bias} x 2
+// a pair of channels in the parameter table: P entries of 16 bytes {scale, shift} x 2, then 16 bytes {slope x 2, sign threshold x 2 (fp16), -}
 __host__ __device__ inline uint32_t pair_bytes(int P) { return 16u * (uint32_t)P + 16u; }
 // constant tiles: four 32-byte rows of (slice, branch) pairs side by side
 __host__ __device__ inline int const_tiles(int rs, int P) { return (rs * P + 3) / 4; }
@@ -88,18 +97,51 @@ __device__ __forceinline__ unsigned long long mul2(unsigned long long a, unsigne
     const float2 x = floats2(a), y = floats2(b);
     return bits2(__float_as_uint(__fmul_rn(x.x, y.x)), __float_as_uint(__fmul_rn(x.y, y.y)));
 }
-__device__ __forceinline__ void tc_ld8_nowait(uint32_t taddr, uint32_t (&v)[8])
+// 8 accumulator columns of this warp's 32 rows, lane l = columns 2 (l % 4) and + 1 of rows l / 4 + 8 i in v[2 i], v[2 i + 1]: a
+// lane meets two channels instead of all of them, so a channel's parameters are fetched once for four rows.
+__device__ __forceinline__ void tc_ld8_quads_nowait(uint32_t taddr, uint32_t (&v)[8])
 {
-    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
-                 : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7])
-                 : "r"(taddr) : "memory");
+    asm volatile("tcgen05.ld.sync.aligned.16x256b.x1.b32 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]) : "r"(taddr) : "memory");
+    asm volatile("tcgen05.ld.sync.aligned.16x256b.x1.b32 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]) : "r"(taddr + (16u << 16)) : "memory");
 }
 __device__ __forceinline__ void pin_regs8(uint32_t (&v)[8])
 {
     asm volatile("" : "+r"(v[0]), "+r"(v[1]), "+r"(v[2]), "+r"(v[3]), "+r"(v[4]), "+r"(v[5]), "+r"(v[6]), "+r"(v[7]) :: "memory");
 }
+__device__ __forceinline__ uint32_t ld_shared_b32(uint32_t addr)
+{
+    uint32_t v;
+    asm volatile("ld.shared.b32 %0, [%1];" : "=r"(v) : "r"(addr) : "memory");
+    return v;
+}
+// u >= 0 ? u : slope * u
+__device__ __forceinline__ float prelu(float u, float slope)
+{
+    asm("{\n\t.reg .pred p;\n\tsetp.ge.f32 p, %0, 0f00000000;\n\t@!p mul.rn.f32 %0, %0, %1;\n\t}" : "+f"(u) : "f"(slope));
+    return u;
+}
+// The smallest fp16 y for which y + nb >= 0 in fp32.  A sum of two numbers has the sign of the exact sum (nothing underflows to 0),
+// so for finite nb that is -nb rounded up; a NaN, which no y reaches, where no y will do (y + nb is -infinity or NaN); and
+// the most negative number for nb = +infinity, where only -infinity and NaN give no sum >= 0.
+__device__ __forceinline__ uint16_t sign_threshold(float nb)
+{
+    if (!(nb > -INFINITY)) return 0x7E00u;
+    if (nb == INFINITY) return 0xFBFFu;
+    return __half_as_ushort(__float2half_ru(-nb));
+}
+// Accumulator column of channel c of a part.  Column 8 k + 2 q + o is held by lane 4 r + q of a load, which is to own the BN / 4
+// consecutive channels from q * BN / 4: 16-byte pieces of the identity's and the output's rows, and whole bytes of sign bits.
+template <int BN> __host__ __device__ constexpr int column_of_channel(int c)
+{
+    return ((c >> 1) & (BN / 8 - 1)) * 8 + c / (BN / 4) * 2 + (c & 1);
+}
+template <int BN> __host__ __device__ constexpr int channel_of_column(int n) { return ((n >> 1) & 3) * (BN / 4) + (n >> 3) * 2 + (n & 1); }
+// bytes of a lane's share of the parameter table (16 more than its entries: the four shares lie in different banks)
+template <int BN> __host__ __device__ constexpr uint32_t share_bytes(uint32_t pair) { return (uint32_t)(BN / 8) * pair + 16u; }
 
-// BN: channels of a part (64, 32); PP: branches where known to the compiler (1, 2), else 0; SHIFTED: taps with a row mask
+// BN: channels of a part (64, 32); PP: branches where known to the compiler (1 .. 4, 9), else 0; SHIFTED: taps with a row mask
 template <int BN, int PP, bool SHIFTED, bool HAS_ID>
 __global__ void __launch_bounds__(THREADS, 1)
 conv_tc_mod_kernel(const ModPlan L, const __grid_constant__ CUtensorMap idmap, const __grid_constant__ CUtensorMap ymap)
@@ -114,12 +156,12 @@ conv_tc_mod_kernel(const ModPlan L, const __grid_constant__ CUtensorMap idmap, c
     const int P = PP ? PP : L.P;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int kst = L.kst, stages = L.stages;
-    const int cg = (int)blockIdx.x % L.ng, idx = (int)blockIdx.x / L.ng, step = (int)gridDim.x / L.ng;
+    const int idx = (int)exact_div(blockIdx.x, L.ng_mul, L.ng_shift), cg = (int)blockIdx.x - idx * L.ng, step = L.step;
     const int rs = min(L.rs, L.slices - cg * L.rs);
-    const int my_tiles = idx < L.m_tiles ? (L.m_tiles - 1 - idx) / step + 1 : 0;
+    const int my_tiles = idx < L.m_tiles ? (int)exact_div((uint32_t)(L.m_tiles - 1 - idx), L.step_mul, L.step_shift) + 1 : 0;
     const int parts = my_tiles * rs;
     const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;         // [rs][kst][BN rows][128 B] weights, then the rest
-    const uint32_t bits_ring = base + L.off_bits, staging = base + L.off_stage, table = base + L.off_table, pops = base + L.off_pop;
+    const uint32_t bits_ring = base + L.off_bits, staging = base + L.off_stage, table = base + L.off_table;
     const uint32_t tab = base + L.off_tab, pads = base + L.off_pad, cexp = base + L.off_const;
     const uint32_t bar0 = smem_u32(bars);
     auto full_bar = [&](int s) { return bar0 + 8u * s; };
@@ -133,52 +175,48 @@ conv_tc_mod_kernel(const ModPlan L, const __grid_constant__ CUtensorMap idmap, c
     const uint32_t ready_bar = bar0 + 8u * (2 * MAX_STAGES + 2 * MAX_NBUF + 3 * TEAMS * NS);      // the resident weights are expanded
     volatile int *abort_flag = &abort_flag_smem;
 
-    if (tid == 0) {
-        for (int s = 0; s < MAX_STAGES; ++s) {
-            mbar_init(full_bar(s), 4);
-            mbar_init(empty_bar(s), 1);
-        }
-        for (int b = 0; b < MAX_NBUF; ++b) {
-            mbar_init(tfull_bar(b), 1);
-            mbar_init(tempty_bar(b), 4);
-        }
-        for (int t = 0; t < TEAMS; ++t) {
-            for (int s = 0; s < NS; ++s) {
-                mbar_init(id_full(t, s), 1);
-                mbar_init(slot_free(t, s), 1);
-                mbar_init(out_full(t, s), 4);
-            }
-        }
-        mbar_init(ready_bar, 4 * TEAMS);
-        abort_flag_smem = 0;
+    constexpr int NBARS = sizeof(bars) / 8;
+    if (tid < NBARS) {
+        // a full slot: its four producer warps; a free buffer: a team; an output tile: a team; the weights: all epilogue warps; else one
+        constexpr int T0 = 2 * MAX_STAGES + MAX_NBUF, O0 = 2 * MAX_STAGES + 2 * MAX_NBUF + 2 * TEAMS * NS;
+        const bool team = tid < MAX_STAGES || (tid >= T0 && tid < T0 + MAX_NBUF) || (tid >= O0 && tid < O0 + TEAMS * NS);
+        mbar_init(bar0 + 8u * tid, tid == NBARS - 1 ? 4 * TEAMS : (team ? 4 : 1));
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
+    if (tid == 0) abort_flag_smem = 0;
     if (warp == ISSUER) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base_smem)), "r"(512u) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
     // gather table: unit u = K words u * gw ..; word w belongs to branch w / kwp (its tap when shifted)
+#pragma unroll 1
     for (int u = tid; u < L.units; u += THREADS) {
-        const int w = u * L.gw, br = w / L.kwp, j = w - br * L.kwp;
+        const int w = u * L.gw, br = (int)exact_div((uint32_t)w, L.kwp_mul, L.kwp_shift), j = w - br * L.kwp;
         uint32_t ent = (uint32_t)TAP_NONE << 27;
         if (br < P && j < L.bcw) {
-            const int r = br / p.kw, t = br - r * p.kw;
-            ent = (uint32_t)((SHIFTED ? (r * p.W + t) * p.cw : 0) + br * L.bcw + j) | ((uint32_t)(SHIFTED ? br : 0) << 27);
+            int off = br * L.bcw + j;
+            if (SHIFTED) {
+                const int r = br / p.kw, t = br - r * p.kw;
+                off += (r * p.W + t) * p.cw;
+            }
+            ent = (uint32_t)off | ((uint32_t)(SHIFTED ? br : 0) << 27);
         }
         asm volatile("st.shared.b32 [%0], %1;" ::"r"(tab + 4u * u), "r"(ent) : "memory");
     }
-    const int npop = rs * P * BN;
-    for (int i = tid; i < npop; i += THREADS) asm volatile("st.shared.b32 [%0], %1;" ::"r"(pops + 4u * i), "r"(0) : "memory");
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
     pdl_trigger();
-    pdl_wait();
+    // (each role that touches global memory waits for the previous kernel behind its own set-up: instructions that run for the first
+    // time cost some ten cycles each, which hide in that kernel's tail)
     const uint32_t tmem_base = tmem_base_smem;
 
     // part n = (row tile n / rs, slice n % rs); team n % TEAMS, its m = n / TEAMS-th part, staging tile m % NS
-    auto part_row = [&](int n) { return (idx + (n / rs) * step) * BM; };
-    auto part_ch = [&](int n) { return (cg * L.rs + n % rs) * BN; };
+    struct Part {
+        int row, slice;
+        __device__ __forceinline__ void skip(int n, int rs, int rows) { for (slice += n; slice >= rs; slice -= rs) row += rows; }
+    };
+    const int tile_rows = step * BM, ch_base = cg * L.rs * BN;
 
     if (warp == ISSUER) {
         // ------------------------------------------------------------------ MMA issuer
@@ -229,17 +267,24 @@ conv_tc_mod_kernel(const ModPlan L, const __grid_constant__ CUtensorMap idmap, c
     } else if (warp == LOADER) {
         // ------------------------------------------------------------------ identity tiles
         if (HAS_ID) {
-            int issued = 0;
-            for (int n = 0; n < parts; ++n, ++issued) {
-                const int team = n % TEAMS, m = n / TEAMS, s = m % NS, lap = m / NS;
-                if (lap > 0 && !mbar_wait_warp(slot_free(team, s), (uint32_t)(lap - 1) & 1u, abort_flag, p.err, ERR_MOD_LOADER)) break;
+            int issued = 0, team = 0, s = 0;
+            uint32_t phase = 1;                                             // first lap: tiles are free
+            Part at = {idx * BM, 0};
+            pdl_wait();
+#pragma unroll 1
+            for (int n = 0; n < parts; ++n, ++issued, at.skip(1, rs, tile_rows)) {
+                if (!mbar_wait_warp(slot_free(team, s), phase, abort_flag, p.err, ERR_MOD_LOADER)) break;
                 if (lane == 0) {
                     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(id_full(team, s)), "r"((uint32_t)TILE_BYTES) : "memory");
                     asm volatile("cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
-                                 ::"r"(staging + (uint32_t)((team * NS + s) * TILE_BYTES)), "l"(reinterpret_cast<uint64_t>(&idmap)), "r"(part_ch(n)), "r"(part_row(n)),
+                                 ::"r"(staging + (uint32_t)((team * NS + s) * TILE_BYTES)), "l"(reinterpret_cast<uint64_t>(&idmap)), "r"(ch_base + at.slice * BN), "r"(at.row),
                                    "r"(id_full(team, s)) : "memory");
                 }
                 __syncwarp();
+                if (++team == TEAMS) {
+                    team = 0;
+                    if (++s == NS) { s = 0; phase ^= 1u; }
+                }
             }
             // after a time-out elsewhere: copies still in flight must land before the CTA's shared memory goes away
             if (*abort_flag)
@@ -249,198 +294,253 @@ conv_tc_mod_kernel(const ModPlan L, const __grid_constant__ CUtensorMap idmap, c
     } else if (warp < FIRST_PRODUCER) {
         // ------------------------------------------------------------------ output tiles of team warp - STORER
         const int team = warp - STORER;
-        for (int n = team; n < parts; n += TEAMS) {
-            const int m = n / TEAMS, s = m % NS;
-            if (!mbar_wait_warp(out_full(team, s), (uint32_t)(m / NS) & 1u, abort_flag, p.err, ERR_MOD_STORE)) break;
+        int s = 0, before = -1;
+        uint32_t phase = 0;
+        Part at = {idx * BM, 0};
+        at.skip(team, rs, tile_rows);
+        pdl_wait();
+#pragma unroll 1
+        for (int n = team; n < parts; n += TEAMS, at.skip(TEAMS, rs, tile_rows)) {
+            if (!mbar_wait_warp(out_full(team, s), phase, abort_flag, p.err, ERR_MOD_STORE)) break;
             if (lane == 0) {
                 asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.tile.bulk_group [%0, {%1, %2}], [%3];"
-                             ::"l"(reinterpret_cast<uint64_t>(&ymap)), "r"(part_ch(n)), "r"(part_row(n)), "r"(staging + (uint32_t)((team * NS + s) * TILE_BYTES)) : "memory");
+                             ::"l"(reinterpret_cast<uint64_t>(&ymap)), "r"(ch_base + at.slice * BN), "r"(at.row), "r"(staging + (uint32_t)((team * NS + s) * TILE_BYTES)) : "memory");
                 asm volatile("cp.async.bulk.commit_group;" ::: "memory");
-                if (m > 0) {                                                // the store before this one has read its tile
+                if (before >= 0) {                                          // the store before this one has read its tile
                     asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory");
-                    mbar_arrive(slot_free(team, (m - 1) % NS));
+                    mbar_arrive(slot_free(team, before));
                 }
             }
             __syncwarp();
+            before = s;
+            if (++s == NS) { s = 0; phase ^= 1u; }
         }
         if (lane == 0) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
         __syncwarp();
     } else if (warp >= FIRST_EPILOGUE) {
         // ------------------------------------------------------------------ epilogue
-        // ---- one-off, while the first rows and identity tiles arrive: the resident slices' weights (the issuer waits for them)
-        // with their bit counts, then the table.  Eight words are in flight per thread, and a channel's parameters before them.
+        // ---- one-off, while the first rows and identity tiles arrive: the resident slices' packed weights and parameters come to shared
+        // memory in one go, eight lanes expand a (branch, slice, channel) row and count its bits, then the constants (the issuer
+        // waits for weights and constants).  Rolled loops on purpose: this code runs once, and its instructions come from memory.
+        // (A thread per word with eight loads in flight, an atomic per word and a division per index took 5 us for two branches
+        // of 256 channels, a quarter of the kernel at 50176 rows.)
         constexpr int ETHREADS = 128 * TEAMS;
         const int etid = tid - 32 * FIRST_EPILOGUE;
-        // parameters of a (slice, branch, channel) triple
-        struct Params { float sc, sh, pd, slope, nb; };
-        auto load_params = [&](int i) {
-            const int c = i % BN, sb = i / BN, br = sb % P, ch = (cg * L.rs + sb / P) * BN + c;
-            const bool have = i < rs * P * BN && ch < p.C_out;
-            const long at = (long)br * p.C_out + ch;
-            Params q;
-            q.sc = have ? __ldg(L.scale + at) : 0.f;
-            q.sh = have ? __ldg(L.shift + at) : 0.f;
-            q.pd = SHIFTED && have && L.pad_dot ? (float)__ldg(L.pad_dot + at) : 0.f;
-            q.slope = br == 0 && have ? __ldg(p.slope + ch) : 0.f;
-            q.nb = br == 0 && have && p.next_bias ? __ldg(p.next_bias + ch) : 0.f;
-            return q;
-        };
-        Params q = load_params(etid);
-        {
-            constexpr int WU = 8;
-            const int total = rs * kst * BN * 8;
-            for (int i0 = etid; i0 < total; i0 += WU * ETHREADS) {
-                uint32_t w[WU];
-                bool live[WU];
-                int pop_at[WU];
-                uint32_t dst[WU];
-#pragma unroll
-                for (int u = 0; u < WU; ++u) {
-                    const int i = i0 + u * ETHREADS, e = i & 7, rk = i >> 3, row_s = rk / kst, kt = rk - row_s * kst;     // row_s = slice * BN + row
-                    const int sl = row_s / BN, row = row_s % BN, ch = (cg * L.rs + sl) * BN + row;
-                    const int kw = kt * 8 + e, br = kw / L.kwp, j = kw - br * L.kwp;
-                    live[u] = i < total && br < P && j < L.bcw && ch < p.C_out;
-                    w[u] = live[u] ? __ldg(p.w + ((long)br * p.C_out + ch) * L.bcw + j) : 0u;
-                    pop_at[u] = (sl * P + br) * BN + row;
-                    dst[u] = base + (uint32_t)((sl * kst + kt) * W_STAGE + row * ROWB + ((e ^ (row & 7)) << 4));
-                }
-#pragma unroll
-                for (int u = 0; u < WU; ++u) {
-                    if (i0 + u * ETHREADS >= total) break;
-                    const uint4 o = live[u] ? expand_w4(w[u]) : make_uint4(0u, 0u, 0u, 0u);
-                    st_shared_v4(dst[u], o.x, o.y, o.z, o.w);
-                    if (live[u]) asm volatile("red.shared.add.u32 [%0], %1;" ::"r"(pops + 4u * pop_at[u]), "r"(__popc(w[u])) : "memory");
-                }
+        const int rows1 = rs * BN, rows_w = P * rows1;                      // rows of a branch, of all
+        const int chans = min(rows1, p.C_out - ch_base);                    // the channels that exist
+        const uint32_t pair = pair_bytes(P), share = share_bytes<BN>(pair);
+        const uint32_t raw = base + L.off_raw, raw_par = raw + (uint32_t)(rows_w * L.bcw) * 4u;      // weights; then scale, shift (, pad) by branch, slope, next bias
+        constexpr int PA = SHIFTED ? 3 : 2;
+        pdl_wait();
+#pragma unroll 1
+        for (int br = 0; br < P; ++br) {
+            const long first = (long)br * p.C_out + ch_base;
+            const uint32_t *src = p.w + first * L.bcw;
+            const uint32_t dst = raw + (uint32_t)(br * rows1 * L.bcw) * 4u, dpar = raw_par + (uint32_t)(PA * br * rows1) * 4u;
+#pragma unroll 1
+            for (int i = 4 * etid; i < chans * L.bcw; i += 4 * ETHREADS) cp_async16(dst + 4u * i, src + i, true);
+            if (4 * etid < chans) {
+                cp_async16(dpar + 16u * etid, L.scale + first + 4 * etid, true);
+                cp_async16(dpar + 4u * rows1 + 16u * etid, L.shift + first + 4 * etid, true);
+                if (SHIFTED) cp_async16(dpar + 8u * rows1 + 16u * etid, L.pad_dot ? L.pad_dot + first + 4 * etid : reinterpret_cast<const int32_t *>(L.scale), L.pad_dot != nullptr);
             }
         }
+        const uint32_t raw_slope = raw_par + (uint32_t)(PA * P * rows1) * 4u, raw_nb = raw_slope + 4u * rows1;
+        if (4 * etid < chans) {
+            cp_async16(raw_slope + 16u * etid, p.slope + ch_base + 4 * etid, true);
+            cp_async16(raw_nb + 16u * etid, p.next_bias ? p.next_bias + ch_base + 4 * etid : p.slope, p.next_bias != nullptr);
+        }
+        cp_async_commit();
+        cp_async_wait<0>();
         asm volatile("bar.sync 1, %0;" ::"n"(ETHREADS) : "memory");
-        for (int i = etid; i < rs * P * BN; i += ETHREADS) {                // (slice, branch, channel)
-            const int c = i % BN, sb = i / BN, br = sb % P, sl = sb / P;
-            if (i != etid) q = load_params(i);
-            int pop;
-            asm volatile("ld.shared.b32 %0, [%1];" : "=r"(pop) : "r"(pops + 4u * i) : "memory");
-            const uint32_t pair = (uint32_t)((sl * BN + c) >> 1), odd = 4u * (c & 1), ent = table + pair * pair_bytes(P) + odd;
-            const int ct = sl * P + br;
-            store_const_row<false>(32 * L.bcw - 2 * pop, cexp + (uint32_t)((ct >> 2) * W_STAGE + c * ROWB), (c & 7) ^ (2 * (ct & 3)));
-            asm volatile("st.shared.b32 [%0], %1;" ::"r"(ent + 16u * br), "r"(__float_as_uint(q.sc)) : "memory");
-            asm volatile("st.shared.b32 [%0], %1;" ::"r"(ent + 16u * br + 8u), "r"(__float_as_uint(q.sh)) : "memory");
-            if (SHIFTED) asm volatile("st.shared.b32 [%0], %1;" ::"r"(pads + (pair * P + br) * 8u + odd), "r"(__float_as_uint(q.pd)) : "memory");
-            if (br == 0) {
-                asm volatile("st.shared.b32 [%0], %1;" ::"r"(ent + 16u * P), "r"(__float_as_uint(q.slope)) : "memory");
-                asm volatile("st.shared.b32 [%0], %1;" ::"r"(ent + 16u * P + 8u), "r"(__float_as_uint(q.nb)) : "memory");
+        // A piece is four words of a row where a branch has a multiple of four, else two (the last one half empty if bcw is odd).  Rows
+        // go by accumulator column: neighbouring lanes then write to different places of the swizzle.
+        const int pw = L.gw == 4 ? 4 : 2, per_row = L.kwp / pw, pieces = rows_w * per_row;
+#pragma unroll 1
+        for (int i = etid; i < pieces; i += ETHREADS) {
+            const int r = (int)exact_div((uint32_t)i, L.row_mul, L.row_shift), j = (i - r * per_row) * pw;
+            const int col = r % BN, sb = r / BN, sl = sb / P, br = sb - sl * P;
+            const uint32_t src = raw + (uint32_t)((br * rows1 + sl * BN + channel_of_column<BN>(col)) * L.bcw + j) * 4u;
+            const int kw = br * L.kwp + j;
+            const uint32_t dst = base + (uint32_t)((sl * kst + (kw >> 3)) * W_STAGE + col * ROWB), x = (uint32_t)((kw & 7) ^ (col & 7)) << 4;
+            if (pw == 4) {
+                const uint4 w = ld_shared_v4(src);
+                const uint4 o0 = expand_w4(w.x), o1 = expand_w4(w.y), o2 = expand_w4(w.z), o3 = expand_w4(w.w);
+                st_shared_v4(dst + x, o0.x, o0.y, o0.z, o0.w);
+                st_shared_v4(dst + (x ^ 16u), o1.x, o1.y, o1.z, o1.w);
+                st_shared_v4(dst + (x ^ 32u), o2.x, o2.y, o2.z, o2.w);
+                st_shared_v4(dst + (x ^ 48u), o3.x, o3.y, o3.z, o3.w);
+            } else {
+                const bool two = j + 1 < L.bcw;
+                const uint4 o0 = expand_w4(ld_shared_b32(src)), o1 = two ? expand_w4(ld_shared_b32(src + 4u)) : make_uint4(0u, 0u, 0u, 0u);
+                st_shared_v4(dst + x, o0.x, o0.y, o0.z, o0.w);
+                st_shared_v4(dst + (x ^ 16u), o1.x, o1.y, o1.z, o1.w);
             }
+        }
+#pragma unroll 1
+        for (int r = etid; r < rows1; r += ETHREADS) {
+            const int c = r % BN, sl = r / BN, col = column_of_channel<BN>(c);
+            const uint32_t odd = (uint32_t)(c & 1);
+            const int pi = (sl * 4 + c / (BN / 4)) * (BN / 8) + ((c >> 1) & (BN / 8 - 1));
+            const uint32_t ent = table + (uint32_t)(sl * 4 + c / (BN / 4)) * share + (uint32_t)((c >> 1) & (BN / 8 - 1)) * pair + 4u * odd;
+#pragma unroll 1
+            for (int br = 0; br < P; ++br) {
+                const int ct = sl * P + br;
+                const uint32_t par = raw_par + (uint32_t)(PA * br * rows1 + r) * 4u, wrow = raw + (uint32_t)((br * rows1 + r) * L.bcw) * 4u;
+                int pop = 0;
+                if (pw == 4) {
+#pragma unroll 2
+                    for (int j = 0; j < L.bcw; j += 4) {
+                        const uint4 w = ld_shared_v4(wrow + 4u * j);
+                        pop += __popc(w.x) + __popc(w.y) + __popc(w.z) + __popc(w.w);
+                    }
+                } else {
+#pragma unroll 4
+                    for (int j = 0; j < L.bcw; ++j) pop += __popc(ld_shared_b32(wrow + 4u * j));
+                }
+                asm volatile("st.shared.b32 [%0], %1;" ::"r"(ent + 16u * br), "r"(ld_shared_b32(par)) : "memory");
+                asm volatile("st.shared.b32 [%0], %1;" ::"r"(ent + 16u * br + 8u), "r"(ld_shared_b32(par + 4u * rows1)) : "memory");
+                if (SHIFTED) {
+                    const float pd = (float)(int)ld_shared_b32(par + 8u * rows1);
+                    asm volatile("st.shared.b32 [%0], %1;" ::"r"(pads + (uint32_t)(pi * P + br) * 8u + 4u * odd), "r"(__float_as_uint(pd)) : "memory");
+                }
+                store_const_row<false>(32 * L.bcw - 2 * pop, cexp + (uint32_t)((ct >> 2) * W_STAGE + col * ROWB), (col & 7) ^ (2 * (ct & 3)));
+            }
+            asm volatile("st.shared.b32 [%0], %1;" ::"r"(ent + 16u * P), "r"(ld_shared_b32(raw_slope + 4u * r)) : "memory");
+            const uint16_t th = sign_threshold(__uint_as_float(ld_shared_b32(raw_nb + 4u * r)));
+            asm volatile("st.shared.b16 [%0], %1;" ::"r"(ent + 16u * P + 8u - 2u * odd), "h"(th) : "memory");
         }
         fence_async_proxy();
         __syncwarp();
         if (lane == 0) mbar_arrive(ready_bar);
         asm volatile("bar.sync 1, %0;" ::"n"(ETHREADS) : "memory");
-        const int team = (warp - FIRST_EPILOGUE) >> 2, quad = warp & 3, row = quad * 32 + lane;
+        // Lane 4 r + q works on the BN / 4 consecutive channels q and on the four rows quad * 32 + r + 8 i.
+        const int team = (warp - FIRST_EPILOGUE) >> 2, quad = warp & 3, lq = lane & 3, row = quad * 32 + (lane >> 2);
         const uint32_t t_lane = tmem_base + ((uint32_t)(quad * 32) << 16);
-        const int owords = p.C_out >> 5;
         const bool want_bits = p.out != nullptr;
-        const TileStep ts = make_tile_step(p, 0);
-        bool ok = true;
-        for (int n = team; n < parts; n += TEAMS) {
-            const int m = n / TEAMS, s = m % NS, lap = m / NS;
-            const int em = part_row(n) + row, ch0 = part_ch(n);
-            if (HAS_ID) ok = mbar_wait_warp(id_full(team, s), (uint32_t)lap & 1u, abort_flag, p.err, ERR_MOD_IDENTITY);
-            else if (lap > 0) ok = mbar_wait_warp(slot_free(team, s), (uint32_t)(lap - 1) & 1u, abort_flag, p.err, ERR_MOD_IDENTITY);
+        // rows 8 apart lie at the same place of the swizzle
+        const uint32_t sw = BN == 64 ? (uint32_t)(row & 7) : (uint32_t)((row >> 1) & 3);
+        int s = 0, buf = team % L.nbuf;                                     // staging tile, accumulator buffer
+        uint32_t phase = 0;
+        Part part = {idx * BM, 0};
+        part.skip(team, rs, tile_rows);
+        bool ok;
+#pragma unroll 1
+        for (int n = team; n < parts; n += TEAMS, part.skip(TEAMS, rs, tile_rows)) {
+            const int em = part.row + row, ch0 = ch_base + part.slice * BN;
+            if (HAS_ID) ok = mbar_wait_warp(id_full(team, s), phase, abort_flag, p.err, ERR_MOD_IDENTITY);
+            else ok = mbar_wait_warp(slot_free(team, s), phase ^ 1u, abort_flag, p.err, ERR_MOD_IDENTITY);
             if (!ok) break;
-            uint32_t inside = 0xffffffffu;                                  // taps of this row inside the image
+            uint32_t inside[4] = {0xffffffffu, 0xffffffffu, 0xffffffffu, 0xffffffffu};      // taps of these rows inside the image
             if (SHIFTED) {
-                RowCursor rc;
-                rc.m = (uint32_t)em;
-                row_locate(p, rc);
-                row_window(p, ts, rc);
-                inside = rc.mask;
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    RowCursor rc;
+                    rc.m = (uint32_t)(em + 8 * i);
+                    row_locate(p, rc);
+                    row_window(p, L.ts, rc);
+                    inside[i] = rc.mask;
+                }
             }
             if (!mbar_wait_warp(tfull_bar(n % MAX_NBUF), (uint32_t)(n / MAX_NBUF) & 1u, abort_flag, p.err, ERR_MOD_EPILOGUE)) break;
             tc_fence_after();
-            const uint32_t acc = t_lane + (uint32_t)((n % L.nbuf) * P * BN);
+            const uint32_t acc = t_lane + (uint32_t)(buf * P * BN);
             const uint32_t tile = staging + (uint32_t)((team * NS + s) * TILE_BYTES) + (uint32_t)(row * ROW_BYTES);
-            const uint32_t sw = BN == 64 ? (uint32_t)(row & 7) : (uint32_t)((row >> 1) & 3);
-            const uint32_t tb = table + (uint32_t)((n % rs) * (BN / 2)) * pair_bytes(P), pb = pads + (uint32_t)((n % rs) * (BN / 2) * P) * 8u;
-            uint32_t words[BN / 32];
-            // (8 channels, branch) at a time; the next piece's accumulators are on their way while one is worked on (a load and
-            // its wait in turn were a third of a part's time)
-            uint32_t nv[8];
-            tc_ld8_nowait(acc, nv);
-#pragma unroll
-            for (int c8 = 0; c8 < BN / 8; ++c8) {
-                unsigned long long t[4];
-#pragma unroll
-                for (int br = 0; br < (PP ? PP : 1); ++br) {
-                    int b = br;
-                    do {
-                        tc_wait_ld();
-                        pin_regs8(nv);
-                        unsigned long long dot[4];
-#pragma unroll
-                        for (int j = 0; j < 4; ++j) dot[j] = bits2(nv[2 * j], nv[2 * j + 1]);
-                        const bool last_branch = b == P - 1;
-                        if (c8 < BN / 8 - 1 || !last_branch) {
-                            tc_ld8_nowait(acc + (uint32_t)(last_branch ? (c8 + 1) * 8 : (b + 1) * BN + c8 * 8), nv);
-                        } else {                                            // the accumulators are in registers
-                            tc_fence_before();
-                            __syncwarp();
-                            if (lane == 0) mbar_arrive(tempty_bar(n % L.nbuf));
-                        }
-#pragma unroll
-                        for (int j = 0; j < 4; ++j) {
-                            const uint4 ss = ld_shared_v4(tb + (uint32_t)(c8 * 4 + j) * pair_bytes(P) + 16u * b);
-                            if (SHIFTED && !((inside >> b) & 1u))
-                                asm volatile("ld.shared.b64 %0, [%1];" : "=l"(dot[j]) : "r"(pb + (uint32_t)((c8 * 4 + j) * P + b) * 8u) : "memory");
-                            const unsigned long long tp = add2(mul2(dot[j], bits2(ss.x, ss.y)), bits2(ss.z, ss.w));
-                            t[j] = b == 0 ? tp : add2(t[j], tp);
-                        }
-                    } while (!PP && ++b < P);
-                }
-                const uint32_t at = tile + (((uint32_t)c8 ^ sw) << 4);
-                uint32_t idw[4] = {0u, 0u, 0u, 0u}, ow[4], bits = 0;
+            const int sl = part.slice;
+            const uint32_t tb = table + (uint32_t)(sl * 4 + lq) * share, pb = pads + (uint32_t)((sl * 4 + lq) * (BN / 8) * P) * 8u;
+            // (two channels, branch) of four rows at a time; the next piece's accumulators and parameters are on their way while one is
+            // worked on (a load and its wait in turn were a third of a part's time)
+            uint32_t nv[8], sg[4] = {0u, 0u, 0u, 0u};                       // sg: even channels' bits in the low halves, odd ones' in the high
+            tc_ld8_quads_nowait(acc, nv);
+            uint4 nss = ld_shared_v4(tb);
+#pragma unroll 1
+            for (int k4 = 0; k4 < BN / 8; k4 += 4) {
+                // a 16-byte piece of each row: eight channels
+                const uint32_t at = tile + (((uint32_t)(BN / 32 * lq + k4 / 4) ^ sw) << 4);
+                uint32_t io[4][4], sg4[4] = {0u, 0u, 0u, 0u};
                 if (HAS_ID) {
-                    const uint4 q = ld_shared_v4(at);
-                    idw[0] = q.x; idw[1] = q.y; idw[2] = q.z; idw[3] = q.w;
-                }
-                float2 yf[4];
-                uint4 sn[4];
 #pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    sn[j] = ld_shared_v4(tb + (uint32_t)(c8 * 4 + j) * pair_bytes(P) + 16u * P);               // slope, next bias
-                    unsigned long long u = t[j];
-                    if (HAS_ID) {
-                        const float2 f = __half22float2(*reinterpret_cast<const __half2 *>(&idw[j]));
-                        u = add2(u, bits2(__float_as_uint(f.x), __float_as_uint(f.y)));
-                    }
-                    const float2 uf = floats2(u), wf = floats2(mul2(bits2(sn[j].x, sn[j].y), u));
-                    const __half2 y2 = __floats2half2_rn(uf.x >= 0.f ? uf.x : wf.x, uf.y >= 0.f ? uf.y : wf.y);
-                    ow[j] = *reinterpret_cast<const uint32_t *>(&y2);
-                    yf[j] = __half22float2(y2);
-                }
-                st_shared_v4(at, ow[0], ow[1], ow[2], ow[3]);
-                if (want_bits) {
-#pragma unroll
-                    for (int j = 0; j < 4; ++j) {
-                        const float2 v = floats2(add2(bits2(__float_as_uint(yf[j].x), __float_as_uint(yf[j].y)), bits2(sn[j].z, sn[j].w)));
-                        bits |= (v.x >= 0.f ? 1u : 0u) << (2 * j);
-                        bits |= (v.y >= 0.f ? 1u : 0u) << (2 * j + 1);
+                    for (int i = 0; i < 4; ++i) {
+                        const uint4 q = ld_shared_v4(at + (uint32_t)(8 * i * ROW_BYTES));
+                        io[i][0] = q.x; io[i][1] = q.y; io[i][2] = q.z; io[i][3] = q.w;
                     }
                 }
-                if (c8 & 3) words[c8 >> 2] |= bits << (8 * (c8 & 3));
-                else words[c8 >> 2] = bits;
+#pragma unroll
+                for (int kk = 0; kk < 4; ++kk) {
+                    const int k = k4 + kk;
+                    unsigned long long t[4];
+                    uint4 sn;
+#pragma unroll
+                    for (int br = 0; br < (PP ? PP : 1); ++br) {
+                        int b = br;
+                        do {
+                            const bool last_branch = b == P - 1;
+                            const uint4 ss = nss;                           // two channels' scales and shifts
+                            tc_wait_ld();
+                            pin_regs8(nv);
+                            unsigned long long dot[4];
+#pragma unroll
+                            for (int i = 0; i < 4; ++i) dot[i] = bits2(nv[2 * i], nv[2 * i + 1]);
+                            if (last_branch) sn = ld_shared_v4(tb + (uint32_t)k * pair + 16u * P);     // slopes, sign thresholds
+                            if (k < BN / 8 - 1 || !last_branch) {
+                                tc_ld8_quads_nowait(acc + (uint32_t)(last_branch ? (k + 1) * 8 : (b + 1) * BN + k * 8), nv);
+                                nss = ld_shared_v4(tb + (last_branch ? (uint32_t)(k + 1) * pair : (uint32_t)k * pair + 16u * (b + 1)));
+                            } else {                                        // the accumulators are in registers
+                                tc_fence_before();
+                                __syncwarp();
+                                if (lane == 0) mbar_arrive(tempty_bar(buf));
+                            }
+                            if (SHIFTED) {
+                                unsigned long long pd;
+                                asm volatile("ld.shared.b64 %0, [%1];" : "=l"(pd) : "r"(pb + (uint32_t)(k * P + b) * 8u) : "memory");
+#pragma unroll
+                                for (int i = 0; i < 4; ++i)
+                                    if (!((inside[i] >> b) & 1u)) dot[i] = pd;
+                            }
+#pragma unroll
+                            for (int i = 0; i < 4; ++i) {
+                                const unsigned long long tp = add2(mul2(dot[i], bits2(ss.x, ss.y)), bits2(ss.z, ss.w));
+                                t[i] = b == 0 ? tp : add2(t[i], tp);
+                            }
+                        } while (!PP && ++b < P);
+                    }
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        unsigned long long u = t[i];
+                        if (HAS_ID) {
+                            const float2 f = __half22float2(*reinterpret_cast<const __half2 *>(&io[i][kk]));
+                            u = add2(u, bits2(__float_as_uint(f.x), __float_as_uint(f.y)));
+                        }
+                        const float2 uf = floats2(u);
+                        const __half2 y2 = __floats2half2_rn(prelu(uf.x, __uint_as_float(sn.x)), prelu(uf.y, __uint_as_float(sn.y)));
+                        io[i][kk] = *reinterpret_cast<const uint32_t *>(&y2);
+                        if (want_bits) sg4[i] |= __hge2_mask(y2, *reinterpret_cast<const __half2 *>(&sn.z)) & ((1u << (2 * kk)) | (2u << (16 + 2 * kk)));
+                    }
+                }
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    st_shared_v4(at + (uint32_t)(8 * i * ROW_BYTES), io[i][0], io[i][1], io[i][2], io[i][3]);
+                    sg[i] |= sg4[i] << (2 * k4);
+                }
             }
             fence_async_proxy();                                            // the tile's generic stores -> the copy engine
             __syncwarp();
             if (lane == 0) mbar_arrive(out_full(team, s));
-            if (p.out && em < p.M) {
-                uint32_t *dst = static_cast<uint32_t *>(p.out) + (long)em * owords + (ch0 >> 5);
-                if (BN == 64 && (owords & 1) == 0) {
-                    *reinterpret_cast<uint2 *>(dst) = make_uint2(words[0], words[BN / 32 - 1]);
-                } else {
+            if (want_bits && ch0 + lq * (BN / 4) < p.C_out) {
+                const long pitch = p.C_out >> 3;
+                uint8_t *dst = static_cast<uint8_t *>(p.out) + (long)em * pitch + ((ch0 + lq * (BN / 4)) >> 3);
 #pragma unroll
-                    for (int k = 0; k < BN / 32; ++k)
-                        if ((ch0 >> 5) + k < owords) dst[k] = words[k];
+                for (int i = 0; i < 4; ++i) {
+                    const uint32_t bits = sg[i] | (sg[i] >> 16);
+                    if (em + 8 * i < p.M) {
+                        if (BN == 64) *reinterpret_cast<uint16_t *>(dst + 8 * i * pitch) = (uint16_t)bits;
+                        else dst[8 * i * pitch] = (uint8_t)bits;
+                    }
                 }
             }
+            if (++s == NS) { s = 0; phase ^= 1u; }
+            buf += TEAMS;
+            while (buf >= L.nbuf) buf -= L.nbuf;
         }
     } else if (warp >= FIRST_PRODUCER) {
         // ------------------------------------------------------------------ producers: items grp, grp + G, ... of the (tile, stage) list
@@ -450,7 +550,7 @@ conv_tc_mod_kernel(const ModPlan L, const __grid_constant__ CUtensorMap idmap, c
         const uint32_t st0 = lane_base + (uint32_t)(L.nbuf * P * BN);
         const uint32_t lane0 = lane == 0 ? 1u : 0u;
         const int total = my_tiles * kst;
-        const TileStep ts = make_tile_step(p, (uint32_t)(BM * step));
+        const TileStep &ts = L.ts;
         if (grp == 0) write_const_block(lane_base);
         RowCursor rc;
         rc.m = (uint32_t)idx * BM + (uint32_t)row;
@@ -473,6 +573,7 @@ conv_tc_mod_kernel(const ModPlan L, const __grid_constant__ CUtensorMap idmap, c
                 row_window(p, ts, rc);
             }
         };
+        pdl_wait();
 #pragma unroll 1
         for (int i = 0; i < PF - 1; ++i) {
             if (l_left > 0) issue();
@@ -523,14 +624,17 @@ bool make_plan(ModPlan &L, bool shifted, int &smem)
     L.stages = stages < MAX_STAGES ? stages : MAX_STAGES;
     L.slices = (q.C_out + BN - 1) / BN;
     L.units = L.kst * (8 / L.gw);
+    exact_div_params((uint32_t)L.kwp, L.kwp_mul, L.kwp_shift);
+    exact_div_params((uint32_t)(L.kwp / (L.gw == 4 ? 4 : 2)), L.row_mul, L.row_shift);
     const long slice_bytes = (long)L.kst * BN * ROWB, staging = (long)TEAMS * NS * BM * BN * 2;
     const int sms = sm_count();
     long best = -1;
     for (int rs = 1; rs <= L.slices && rs <= 16; ++rs) {
         if (rs > 1 && L.kst > L.stages) break;               // the row tile's stages stay in the ring for all its parts
-        const long pops = (long)rs * L.P * BN * 4, table = (long)rs * (BN / 2) * pair_bytes(L.P);
+        const long table = (long)rs * 4 * share_bytes<BN>(pair_bytes(L.P));
         const long pad = shifted ? (long)rs * (BN / 2) * L.P * 8 : 0, consts = (long)const_tiles(rs, L.P) * BN * ROWB;
-        const long bytes = 1024 + rs * slice_bytes + consts + pad + staging + pops + (long)PF * SLOT_BYTES + table + 4L * L.units + 64;
+        const long raw = (long)rs * BN * 4 * (L.P * (L.bcw + (shifted ? 3 : 2)) + 2);
+        const long bytes = 1024 + rs * slice_bytes + consts + pad + staging + raw + (long)PF * SLOT_BYTES + table + 4L * L.units + 64;
         if (bytes > MAX_SMEM) break;
         const int ng = (L.slices + rs - 1) / rs, per = sms / ng;
         if (per < 1) continue;
@@ -542,8 +646,8 @@ bool make_plan(ModPlan &L, bool shifted, int &smem)
         L.ng = ng;
         L.off_const = (uint32_t)(rs * slice_bytes);
         L.off_stage = L.off_const + (uint32_t)consts;
-        L.off_pop = L.off_stage + (uint32_t)staging;
-        L.off_bits = L.off_pop + (uint32_t)pops;
+        L.off_raw = L.off_stage + (uint32_t)staging;
+        L.off_bits = L.off_raw + (uint32_t)raw;
         L.off_table = L.off_bits + (uint32_t)PF * SLOT_BYTES;
         L.off_pad = L.off_table + (uint32_t)table;
         L.off_tab = (L.off_pad + (uint32_t)pad + 15u) & ~15u;
@@ -553,7 +657,7 @@ bool make_plan(ModPlan &L, bool shifted, int &smem)
 }
 
 template <int BN, int PP, bool SHIFTED>
-int launch_plan(const ModPlan &L, int smem, cudaStream_t stream)
+int launch_plan(ModPlan &L, int smem, cudaStream_t stream)
 {
     EncodeTiledFn encode = encode_tiled_fn();
     if (!encode) return BCNN_ERR_CUDA;
@@ -571,6 +675,10 @@ int launch_plan(const ModPlan &L, int smem, cudaStream_t stream)
     if (!allow_smem((const void *)k, MAX_SMEM)) return BCNN_ERR_CUDA;
     int per = sm_count() / L.ng;
     if (per > L.m_tiles) per = L.m_tiles;
+    L.step = per;
+    exact_div_params((uint32_t)L.ng, L.ng_mul, L.ng_shift);
+    exact_div_params((uint32_t)per, L.step_mul, L.step_shift);
+    L.ts = make_tile_step(q, (uint32_t)(BM * per));
     if (smem < 120 * 1024) smem = 120 * 1024;                // one CTA per multiprocessor (it takes all of tensor memory)
     return launch(k, (unsigned)(per * L.ng), THREADS, smem, stream, L, map[0], map[1]);
 }
@@ -581,21 +689,22 @@ int launch_mod(ModPlan &L, bool shifted, cudaStream_t stream)
     L.kwp = (L.bcw + 1) & ~1;
     L.gw = L.bcw % 4 == 0 ? 4 : (L.bcw % 2 == 0 ? 2 : 1);
     q.err = device_error_word();
-    if (L.P > 13 || q.C_out % 32 != 0 || q.M < 1) return BCNN_ERR_UNSUPPORTED;
+    if (L.P > 13 || (shifted && L.P != 9) || q.C_out % 32 != 0 || q.M < 1) return BCNN_ERR_UNSUPPORTED;
     if ((long)q.B * q.H * q.W * q.cw >= (1L << 31) || (long)q.kh * q.W * q.cw >= (1L << 27) || 32L * L.bcw > CONST_MAX) return BCNN_ERR_UNSUPPORTED;
     L.m_tiles = (q.M - 1) / BM + 1;
     int smem = 0;
     // 64-channel parts; 32 where that leaves a multiprocessor less than two parts (a part is 2 us of latency per 64 channels)
-    if (L.P <= 3 && q.C_out > 32 && (long)L.m_tiles * ((q.C_out + 63) / 64) > sm_count() && make_plan<64>(L, shifted, smem)) {
-        if (shifted) return launch_plan<64, 0, true>(L, smem, stream);
+    if (L.P <= 3 && !shifted && q.C_out > 32 && (long)L.m_tiles * ((q.C_out + 63) / 64) > sm_count() && make_plan<64>(L, shifted, smem)) {
         if (L.P == 1) return launch_plan<64, 1, false>(L, smem, stream);
         if (L.P == 2) return launch_plan<64, 2, false>(L, smem, stream);
-        return launch_plan<64, 0, false>(L, smem, stream);
+        return launch_plan<64, 3, false>(L, smem, stream);
     }
     if (make_plan<32>(L, shifted, smem)) {
-        if (shifted) return launch_plan<32, 0, true>(L, smem, stream);
+        if (shifted) return launch_plan<32, 9, true>(L, smem, stream);      // odd squares up to 13: 9
         if (L.P == 1) return launch_plan<32, 1, false>(L, smem, stream);
         if (L.P == 2) return launch_plan<32, 2, false>(L, smem, stream);
+        if (L.P == 3) return launch_plan<32, 3, false>(L, smem, stream);
+        if (L.P == 4) return launch_plan<32, 4, false>(L, smem, stream);
         return launch_plan<32, 0, false>(L, smem, stream);
     }
     return BCNN_ERR_UNSUPPORTED;

@@ -300,7 +300,7 @@ struct TileStep {
     uint32_t pat;            // bit r*kw for every kernel row r
     bool pointwise;          // 1x1, stride 1, no padding: row m reads input pixel m, no coordinates needed
 };
-__device__ __forceinline__ TileStep make_tile_step(const ConvProblem &p, uint32_t rows)
+__host__ __device__ __forceinline__ TileStep make_tile_step(const ConvProblem &p, uint32_t rows)
 {
     TileStep s;
     const uint32_t ohw = (uint32_t)(p.OH * p.OW);

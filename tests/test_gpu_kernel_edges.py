@@ -220,3 +220,36 @@ def test_stem_stages_handed_back_in_every_launch(bk):
         wrong += (out != ref).any()
     assert int(wrong) == 0
     assert bk.bcnn_device_error() == 0
+
+
+# the module's sign threshold and PReLU on values where a rounding, a sign of zero, an infinity or a NaN could go the other way: identities
+# and next biases from lists of such values in all combinations, on 32- and 64-channel parts with a half-empty last one
+@pytest.mark.parametrize("has_nb", [True, False])
+@pytest.mark.parametrize("P", [1, 2, 3, 4, 6])
+@pytest.mark.parametrize("shape", [(1, 11, 13, 96), (1, 120, 161, 96)])
+def test_module_special_values(bk, oracle, shape, P, has_nb):
+    B, H, W, C = shape
+    rng = np.random.default_rng(41 + P)
+    inf, nan, tiny = np.inf, np.nan, 2.0 ** -24                                  # tiny: the smallest fp16 number
+    ids = np.array([0.0, -0.0, 1.0, -1.0, tiny, -tiny, 65504.0, -65504.0, inf, -inf, nan, 0.5, -2.0, 1000.0, -1000.0, 6e-5], np.float16)
+    nbs = np.array([0.0, -0.0, 1e-45, -1e-45, tiny, -tiny, 0.7 * tiny, -0.7 * tiny, 1.0, -1.0, 1.0 + 2.0 ** -23, -1.0 - 2.0 ** -23, 65504.0, -65504.0,
+                    65520.0, -65520.0, 1e30, -1e30, inf, -inf, nan, 0.3, -0.3, 2.0], np.float32)
+    slopes = np.array([1.0, 0.25, 0.0, -0.0, -0.5, 2.0, 1e-30, inf, -inf, nan], np.float32)
+    x, w = synth.pm1(rng, (B, H, W, P * 32)), synth.pm1(rng, (P, C, 32))
+    scale = rng.choice(np.array([0.0, 1.0, -1.0, 1e-6, 1e30], np.float32), (P, C), p=[0.6, 0.1, 0.1, 0.1, 0.1])
+    shift = rng.choice(np.array([0.0, -0.0, 1.0, -tiny], np.float32), (P, C))
+    slope, nb = rng.choice(slopes, C), rng.choice(nbs, C)
+    ident = rng.choice(ids, (B, H, W, C))
+    accs = np.stack([oracle.conv2d(np.ascontiguousarray(x[..., 32 * p:32 * p + 32]), w[p].reshape(C, 1, 1, 32), 1, 0) for p in range(P)])
+    want_y, want_s = oracle.conv_module_branches(accs, scale, shift, ident, slope, nb if has_nb else None)
+    y = torch.empty(want_y.size, dtype=torch.float16, device="cuda")
+    bits = torch.empty(want_y.size // 8, dtype=torch.uint8, device="cuda")
+    bk.bcnn_conv2d_b1_branches(dev(synth.pack_bits(x)), dev(synth.pack_bits(w)), dev(scale), dev(shift), None, dev(ident), dev(slope), dev(nb) if has_nb else None,
+                               y, bits, B, H, W, 32, C, P)
+    torch.cuda.synchronize()
+    got = y.cpu().numpy().reshape(want_y.shape)
+    # a NaN's payload is not defined, everything else is
+    assert np.array_equal(np.isnan(got), np.isnan(want_y))
+    assert np.array_equal(np.where(np.isnan(got), 0, got.view(np.uint16)), np.where(np.isnan(want_y), 0, want_y.view(np.uint16)))
+    assert np.array_equal(synth.unpack_bits(bits.cpu().numpy().reshape(B, H, W, C // 8)), want_s)
+    assert bk.bcnn_device_error() == 0
