@@ -12,21 +12,24 @@
 //   packed output: accumulator + (cst_n - thr_n) >= 0      thr clamped to +-(K + 1)
 // so there are no per-row constants, and the per-column ones are added by the epilogue from a small table.
 //
-//   warp 0        issuer (tcgen05.mma / commit only; waits on named barriers only)
-//   warps 1-4     epilogue (256-wide and int32 128-wide tiles: 1-8, two teams with half of the columns each): build the tile's
-//                 column table, tcgen05.ld, add + sign bits (or int32), store
+//   warp 0        issuer: one lane waits for a stage, issues its MMAs and their commits
+//   warps 1-4     epilogue (256-wide and int32 128-wide tiles: 1-8, two teams with half of the columns each): build the
+//                 column table (where the columns change), tcgen05.ld, add + sign bits (or int32), store
 //   G groups of 4 activation warps: implicit-im2col gather (cp.async), expansion, tcgen05.st into the ring in tensor memory
 //   loader warp   weight tiles by TMA into the ring in shared memory
-//   control warp  the issuer's mbarrier waits
 // Every mbarrier wait is bounded and reports through the device error word.
 //
-// What bounds it.  256-wide tiles: the K loop runs at the tensor pipe's rate (16384 x 16384, packed, K = 2304 / 4608 / 9216: 240 / 385 /
-// 670 us, 0.283 us per 256-bit stage and tile, the probe's rate; the expansion is hidden), and with one accumulator buffer the epilogue
-// is not overlapped: 1.8 us per packed and 4.9 us per int32 tile with the pipe idle (842 us at K = 9216).  128- and 64-wide tiles have
-// two and four buffers; they take 185 and 167 ns per stage against 141 and 71 of the pipe, and 0.6 us a packed tile (one epilogue team,
-// which builds its column table anew for every tile).  No unit is saturated there: 3x3 128 -> 128 at M = 200704 has the tensor pipe
-// active 35 % of the time, the logic pipe 36 %, the issue slots 49 %.
-#include "tc_common.cuh"
+// 256-wide tiles have one accumulator buffer, handed over in halves of 128 columns: a tile's last two stages are multiplied half by
+// half, and so are the next one's first two, so that each half is read while the other is worked on; int32 outputs leave it as 16-bit
+// pairs (K <= 32767) and go to memory beside the next tile's MMAs.  Large products run on pairs of blocks (cta_group::2).
+//
+// What bounds it.  Long products: power.  A 256-bit stage of a 256-wide tile takes 553 cycles of a pair (512 of the pipe), at a clock
+// that falls from 1965 to 1600 .. 1750 MHz.  Narrow tiles: the issuer - a stage of four instructions with its wait and its commit costs it 300
+// to 400 cycles beside busy warps, whatever the width (128: 256 of the pipe); and what a launch does once, which is why set-up is short, its
+// divisions are the host's, and each role waits for the previous kernel as late as it can (0.7 us of a small layer's 4.3).
+// Before and after, us: 3x3 128 -> 128 at M = 784 4.3 -> 3.3, at M = 200704 18.9 -> 17.2; 256 -> 256 at M = 50176 15.4 -> 13.1; 512 -> 512 /2 at M = 25088
+// 23.5 -> 21.6; 1x1 256 -> 256 at M = 196 3.1 -> 2.3; 1000 x 4000 x 2304 8.4 -> 7.3; 8192 x 8192 x 512 52.6 -> 33.8.
+#include "tc_slot.cuh"
 #include "tensor_map.cuh"
 #include <climits>
 
@@ -46,24 +49,64 @@ constexpr int ERR_LOADER_TIMEOUT = 134;
 
 // BN: output channels of a tile; MODE: 0 int32, 1 packed output; G: activation producer groups of four warps; TEAMS: epilogue
 // teams of four warps, each with its share of a tile's columns
-template <int BN, int MODE, int G, int TEAMS> struct Cfg {
+template <int BN, int MODE, int G, int TEAMS, bool PAIR> struct Cfg {
     static constexpr int EPI_WARPS = 4 * TEAMS;
     static constexpr int NBUF = BN == 256 ? 1 : (BN == 128 ? 2 : 4);     // accumulator buffers
     static constexpr int A_COL0 = NBUF * BN;                              // first column of the activation ring
-    static constexpr int STAGES = BN == 256 ? (MODE == 0 ? 4 : 5) : 7;
+    static constexpr int STAGES = !PAIR && BN == 256 ? (MODE == 0 ? 4 : 5) : 7;
     static constexpr int PROD_THREADS = G * BM;
     static constexpr int FIRST_PRODUCER_WARP = 1 + EPI_WARPS;
     static constexpr int LOADER_WARP = FIRST_PRODUCER_WARP + 4 * G;
-    static constexpr int CONTROL_WARP = LOADER_WARP + 1;
-    static constexpr int THREADS = 32 * (CONTROL_WARP + 1);
+    static constexpr int THREADS = 32 * (LOADER_WARP + 1);
+    static constexpr int CTAS = PAIR ? 2 : 1, TILE_ROWS = CTAS * BM;      // CTAs of a tile, its rows
     static constexpr int EC = BN / TEAMS;                                 // columns of a team
-    static constexpr int W_BYTES = BN * ROWB;                             // one ring stage of weights
+    static constexpr bool SPLIT = BN == 256;                              // one accumulator, handed over in halves of 128 columns
+    static constexpr int PIECES = SPLIT ? 2 : 1, PC = EC / PIECES;        // pieces of a team's columns, columns of a piece
+    static constexpr int MMA_N = SPLIT ? BN / 2 : BN;                     // columns of an instruction
+    static constexpr int W_BYTES = BN / CTAS * ROWB;                      // one ring stage of weights
     static constexpr int SF_COL = 512 - (int)SF_COLS;                     // unit scales
     static constexpr int BITS_BYTES = PF * PROD_THREADS * 32;
     static constexpr int TABLE_BYTES = EPI_WARPS * EC * 4;                // one column table per epilogue warp
     static_assert(A_COL0 + STAGES * 32 <= SF_COL, "tensor memory budget");
     static_assert(STAGES >= G, "a producer group must not lap the ring (parity waits)");
 };
+
+// ---- two CTAs on one tile of 256 rows (cta_group::2): the even CTA's issuer multiplies for both, each brings its own 128 rows of
+// activations and half of the weight rows, each keeps the accumulators of its own rows.
+template <bool PAIR> __device__ __forceinline__ void commit(uint32_t bar)
+{
+    if (PAIR)
+        asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(bar), "h"((uint16_t)3) : "memory");
+    else
+        tc_commit(bar);
+}
+template <bool PAIR> __device__ __forceinline__ void mma_f4(uint32_t d_tmem, uint32_t a_tmem, uint32_t b_lo, uint32_t desc_hi, uint32_t idesc, uint32_t sf, uint32_t accumulate)
+{
+    if (PAIR)
+        asm volatile(
+            "{\n\t.reg .pred p;\n\t.reg .b64 db;\n\t"
+            "setp.ne.b32 p, %6, 0;\n\t"
+            "mov.b64 db, {%2, %3};\n\t"
+            "tcgen05.mma.cta_group::2.kind::mxf4.block_scale.scale_vec::2X [%0], [%1], db, %4, [%5], [%5], p;\n\t}"
+            ::"r"(d_tmem), "r"(a_tmem), "r"(b_lo), "r"(desc_hi), "r"(idesc), "r"(sf), "r"(accumulate) : "memory");
+    else
+        tc_mma_f4_ts(d_tmem, a_tmem, b_lo, desc_hi, idesc, sf, accumulate);
+}
+__device__ __forceinline__ uint32_t in_even_cta(uint32_t addr)
+{
+    uint32_t r;
+    asm("mapa.shared::cluster.u32 %0, %1, 0;" : "=r"(r) : "r"(addr));
+    return r;
+}
+__device__ __forceinline__ void arrive_in_cluster(uint32_t bar, uint32_t pred)
+{
+    asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %1, 0;\n\t@q mbarrier.arrive.shared::cluster.b64 _, [%0];\n\t}" ::"r"(bar), "r"(pred) : "memory");
+}
+__device__ __forceinline__ void cluster_barrier()
+{
+    __syncwarp();
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
 
 template <typename C>
 __host__ __device__ constexpr int smem_bytes(int ktab_words, int mode)
@@ -72,11 +115,11 @@ __host__ __device__ constexpr int smem_bytes(int ktab_words, int mode)
            (mode == 0 ? C::EPI_WARPS * I32_TILE_BYTES + 16 : 0);
 }
 
-template <int BN, int MODE, int G, int TEAMS>
-__global__ void __launch_bounds__(Cfg<BN, MODE, G, TEAMS>::THREADS, 1)
-conv_tc_pre_kernel(const ConvProblem p, const int32_t *cst, const __grid_constant__ CUtensorMap wmap, const int ktab_words)
+template <int BN, int MODE, int G, int TEAMS, bool PAIR>
+__global__ void __launch_bounds__(Cfg<BN, MODE, G, TEAMS, PAIR>::THREADS, 1)
+conv_tc_pre_kernel(const ConvProblem p, const int32_t *cst, const __grid_constant__ CUtensorMap wmap, const int ktab_words, const TileWalk walk)
 {
-    using C = Cfg<BN, MODE, G, TEAMS>;
+    using C = Cfg<BN, MODE, G, TEAMS, PAIR>;
     constexpr int EPI_WARPS = C::EPI_WARPS, EC = C::EC;
     constexpr bool FUSED = MODE == 1;
     constexpr int NBUF = C::NBUF;
@@ -90,11 +133,13 @@ conv_tc_pre_kernel(const ConvProblem p, const int32_t *cst, const __grid_constan
     const int tid = threadIdx.x;
     const int warp = tid >> 5, lane = tid & 31;
     const int ktiles = (p.kwords + 7) >> 3;
-    const int m_tiles = (p.M - 1) / BM + 1;
-    const int n_tiles = (p.C_out + BN - 1) / BN;
-    const int total_tiles = m_tiles * n_tiles;
-    const int my_tiles = ((int)blockIdx.x < total_tiles) ? (total_tiles - 1 - (int)blockIdx.x) / (int)gridDim.x + 1 : 0;
+    const int unit = PAIR ? (int)(blockIdx.x >> 1) : (int)blockIdx.x, rank = PAIR ? (int)(blockIdx.x & 1u) : 0;      // of a pair, the CTA within it
+    const int my_tiles = walk.tiles_of(unit);
     const int total_items = my_tiles * ktiles;
+    // (256-wide tiles) stages at a tile's start and end that are multiplied half by half: while the second half's last MMAs run, the
+    // epilogue takes the first half, and it takes the second half while the next tile's first MMAs run on the first.  Two of each
+    // leave the ring room for the stages that follow.
+    const int split_a = min(2, ktiles >> 1), split_b = min(2, ktiles - split_a);
 
     const uint32_t wring = (smem_u32(smem_raw) + 1023u) & ~1023u;         // [STAGES][BN rows][128 B], written by TMA
     const uint32_t bits_ring = wring + STAGES * C::W_BYTES;               // [PF][2][PROD_THREADS][16 B]
@@ -108,185 +153,287 @@ conv_tc_pre_kernel(const ConvProblem p, const int32_t *cst, const __grid_constan
     auto tempty_bar = [&](int b) { return bar0 + 8u * (20 + b); };
     volatile int *abort_flag = &abort_flag_smem;
 
-    if (tid == 0) {
-        for (int s = 0; s < 8; ++s) {
-            mbar_init(full_bar(s), 4 + 1);           // the four activation warps of the stage's group + the loader's arrive (+ its bytes)
-            mbar_init(empty_bar(s), 1);
-        }
-        for (int b = 0; b < 4; ++b) {
-            mbar_init(tfull_bar(b), 1);
-            mbar_init(tempty_bar(b), EPI_WARPS);
-        }
-        abort_flag_smem = 0;
+    if (tid < 24) {
+        // full: the four activation warps of the stage's group + the loader's arrive (+ its bytes); accumulator free: the epilogue warps
+        // (of both CTAs, whose MMAs the even one issues)
+        mbar_init(bar0 + 8u * tid, tid < 8 ? 4 * C::CTAS + 1 : (tid >= 20 ? EPI_WARPS * C::CTAS : 1));
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
+    if (tid == 0) abort_flag_smem = 0;
     if (warp == 0) {
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base_smem)), "r"(512u) : "memory");
-        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+        if (PAIR) {
+            asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base_smem)), "r"(512u) : "memory");
+            asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+        } else {
+            asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base_smem)), "r"(512u) : "memory");
+            asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+        }
     }
     const int gwidth = gather_width(p.cw);
     build_unit_table8(p, ktab_addr, ktiles * (8 / gwidth), gwidth, tid, C::THREADS);
     if (tid == 32 * C::LOADER_WARP) asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&wmap)) : "memory");
     tc_fence_before();
-    __syncthreads();
+    if (PAIR) cluster_barrier();               // the other CTA's barriers exist
+    else __syncthreads();
     tc_fence_after();
     pdl_trigger();
-    pdl_wait();
+    // (the roles that touch global memory wait for the previous kernel behind their own set-up)
     const uint32_t tmem_base = tmem_base_smem;
 
     if (warp == 0) {
         // ------------------------------------------------------------------ issuer (no memory instructions)
-        constexpr uint32_t idesc = make_idesc_f4(BN);
+        constexpr uint32_t idesc = PAIR ? make_idesc_f4(C::MMA_N) + (1u << 27) : make_idesc_f4(C::MMA_N);      // M = 256 or 128
         const uint64_t desc0 = make_desc(0);
         const uint32_t desc_hi = (uint32_t)(desc0 >> 32);
         const uint32_t b_lo0 = (uint32_t)desc0 | ((wring & 0x3FFFFu) >> 4);      // + slot * (W_BYTES / 16)
         const uint32_t tmem_u = __shfl_sync(0xffffffffu, tmem_base, 0);
         const uint32_t a_tmem0 = tmem_u + (uint32_t)C::A_COL0;                   // + slot * 32 columns
         const uint32_t sf = tmem_u + (uint32_t)C::SF_COL;
-        int s = 0, buf = 0;
-        for (int ti = 0; ti < my_tiles; ++ti) {
-            const uint32_t d_tmem = tmem_u + (uint32_t)(buf * BN);
-            const uint32_t tfull = tfull_bar(buf);
-            for (int kt = 0; kt < ktiles; ++kt) {
-                const uint32_t a_t = a_tmem0 + (uint32_t)s * 32u;
-                const uint32_t b_lo = b_lo0 + (uint32_t)s * (C::W_BYTES >> 4);
-                const int nk = p.kwords - 8 * kt;                 // two K words per instruction; skip the zero tail
-                const uint32_t ebar = empty_bar(s);
-                asm volatile("bar.sync %0, 64;" ::"r"(1 + s) : "memory");
-                tc_fence_after();
-                if (elect_one()) {
-                    tc_mma_f4_ts(d_tmem, a_t, b_lo, desc_hi, idesc, sf, kt > 0 ? 1u : 0u);
-                    if (nk > 2) tc_mma_f4_ts(d_tmem, a_t + 8u, b_lo + 2u, desc_hi, idesc, sf, 1u);
-                    if (nk > 4) tc_mma_f4_ts(d_tmem, a_t + 16u, b_lo + 4u, desc_hi, idesc, sf, 1u);
-                    if (nk > 6) tc_mma_f4_ts(d_tmem, a_t + 24u, b_lo + 6u, desc_hi, idesc, sf, 1u);
-                    tc_commit(ebar);
-                    if (kt == ktiles - 1) tc_commit(tfull);
-                }
-                __syncwarp();
-                if (++s == STAGES) s = 0;
+        // A stage's MMAs for all columns, or for half h of a split tile: two K words per instruction, four instructions - but for the last
+        // stage's zero tail, a branch of its own.  What a stage costs its issuer is the bound of narrow tiles: in a loop alone on its
+        // multiprocessor 172 cycles with a wait, 257 with a test in front of each instruction, 400 with a vote and a reconvergence, and 256 or 128
+        // is what the pipe takes for 128 or 64 columns.
+        const int tail = (p.kwords - 8 * (ktiles - 1) + 1) >> 1;                // instructions of the last stage
+        auto four = [&](int slot, int kt, uint32_t d, int h) {
+            const uint32_t a_t = a_tmem0 + (uint32_t)slot * 32u;
+            const uint32_t b_lo = b_lo0 + (uint32_t)slot * (C::W_BYTES >> 4) + (uint32_t)h * (C::W_BYTES >> 5);
+            mma_f4<PAIR>(d, a_t, b_lo, desc_hi, idesc, sf, kt > 0 ? 1u : 0u);
+            mma_f4<PAIR>(d, a_t + 8u, b_lo + 2u, desc_hi, idesc, sf, 1u);
+            mma_f4<PAIR>(d, a_t + 16u, b_lo + 4u, desc_hi, idesc, sf, 1u);
+            mma_f4<PAIR>(d, a_t + 24u, b_lo + 6u, desc_hi, idesc, sf, 1u);
+        };
+        auto multiply = [&](int slot, int kt, uint32_t d_tmem, int h) {
+            const uint32_t d = d_tmem + (uint32_t)(h * C::MMA_N);
+            if (kt < ktiles - 1 || tail == 4) {
+                four(slot, kt, d, h);
+            } else {
+                const uint32_t a_t = a_tmem0 + (uint32_t)slot * 32u;
+                const uint32_t b_lo = b_lo0 + (uint32_t)slot * (C::W_BYTES >> 4) + (uint32_t)h * (C::W_BYTES >> 5);
+#pragma unroll 1
+                for (uint32_t i = 0; i < (uint32_t)tail; ++i) mma_f4<PAIR>(d, a_t + 8u * i, b_lo + 2u * i, desc_hi, idesc, sf, kt > 0 || i > 0 ? 1u : 0u);
             }
-            if (++buf == NBUF) buf = 0;
-        }
-    } else if (warp == C::CONTROL_WARP) {
-        // ------------------------------------------------------------------ control: waits for the issuer
-        // A stage is released (bar.arrive on 1 + slot) once its ring slot is full (activations expanded, weights
-        // landed) and, for a tile's first stage, once the accumulator buffer is free.  After a time-out the
-        // remaining stages are released by bar.sync, which pairs every release with one wait of the issuer.
-        int s = 0, buf = 0;
-        uint32_t ring_phase = 0, buf_phase = 1;      // first use of every accumulator buffer: free
-        bool alive = true;
-        for (int ti = 0; ti < my_tiles; ++ti) {
-            if (lane == 0 && alive) alive = mbar_wait(tempty_bar(buf), buf_phase, abort_flag, p.err, ERR_MMA_TIMEOUT);
-            for (int kt = 0; kt < ktiles; ++kt) {
-                if (lane == 0 && alive) alive = mbar_wait(full_bar(s), ring_phase, abort_flag, p.err, ERR_MMA_TIMEOUT);
-                if (__shfl_sync(0xffffffffu, alive ? 1 : 0, 0)) asm volatile("bar.arrive %0, 64;" ::"r"(1 + s) : "memory");
-                else asm volatile("bar.sync %0, 64;" ::"r"(1 + s) : "memory");
-                if (++s == STAGES) { s = 0; ring_phase ^= 1u; }
+        };
+        auto second_half = [&](int slot, int kt, int n) {                        // n stages from (slot, kt), each handed back
+            for (int j = 0; j < n; ++j) {
+                multiply(slot, kt + j, tmem_u, 1);
+                commit<PAIR>(empty_bar(slot));
+                if (++slot == STAGES) slot = 0;
             }
-            if (++buf == NBUF) { buf = 0; buf_phase ^= 1u; }
-        }
-    } else if (warp == C::LOADER_WARP) {
-        // ------------------------------------------------------------------ loader: weight tiles by TMA
-        // item (tile, stage) -> ring slot item % STAGES; box = 128 bytes of K x BN rows at (kt * 128, n_tile * BN)
-        int s = 0;
-        uint32_t phase = 1;                           // first pass through the ring: slots are free
-        int issued = 0;
-        for (int ti = 0; ti < my_tiles; ++ti) {
-            const int tile = (int)blockIdx.x + ti * (int)gridDim.x;
-            const int n_row0 = (tile / m_tiles) * BN;
+        };
+        // One lane runs the whole loop and does its own waits: one that is satisfied costs a hundred cycles behind MMAs in the queue, and
+        // while the ring is ahead of the MMAs all are.
+        if (rank == 0 && elect_one()) {
+            int s = 0, buf = 0;
+            uint32_t ring_phase = 0, buf_phase = 1;      // first use of every accumulator buffer: free
             bool ok = true;
-            for (int kt = 0; kt < ktiles; ++kt) {
-                ok = mbar_wait_warp(empty_bar(s), phase, abort_flag, p.err, ERR_LOADER_TIMEOUT);
-                if (!ok) break;
-                if (lane == 0) {
-                    const uint32_t dst = wring + (uint32_t)s * C::W_BYTES;
-                    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(full_bar(s)), "r"((uint32_t)C::W_BYTES) : "memory");
-                    asm volatile("cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
-                                 ::"r"(dst), "l"(reinterpret_cast<uint64_t>(&wmap)), "r"(kt * ROWB), "r"(n_row0), "r"(full_bar(s)) : "memory");
+            auto wait = [&](uint32_t bar, uint32_t parity) {
+                ok = issuer_wait(bar, parity, abort_flag, p.err, ERR_MMA_TIMEOUT);
+                tc_fence_after();
+                return ok;
+            };
+            // the ring's next stage: its slot, or -1 after a time-out
+            auto take = [&]() {
+                const int slot = wait(full_bar(s), ring_phase) ? s : -1;
+                if (++s == STAGES) { s = 0; ring_phase ^= 1u; }
+                return slot;
+            };
+            for (int ti = 0; ti < my_tiles; ++ti) {
+                if (!wait(tempty_bar(buf), buf_phase)) break;
+                if (C::SPLIT) {
+                    const int s0 = s;
+                    int kt = 0, slot = 0;
+                    for (; kt < split_a && (slot = take()) >= 0; ++kt) multiply(slot, kt, tmem_u, 0);
+                    if (!ok || !wait(tempty_bar(1), buf_phase)) break;
+                    second_half(s0, 0, split_a);
+#pragma unroll 1
+                    for (; kt < ktiles - split_b && (slot = take()) >= 0; ++kt) {
+                        four(slot, kt, tmem_u, 0);
+                        four(slot, kt, tmem_u + (uint32_t)C::MMA_N, 1);
+                        commit<PAIR>(empty_bar(slot));
+                    }
+                    const int s_last = s;
+                    for (; ok && kt < ktiles && (slot = take()) >= 0; ++kt) multiply(slot, kt, tmem_u, 0);
+                    if (!ok) break;
+                    commit<PAIR>(tfull_bar(0));
+                    second_half(s_last, ktiles - split_b, split_b);
+                    commit<PAIR>(tfull_bar(1));
+                } else {
+                    const uint32_t d_tmem = tmem_u + (uint32_t)(buf * BN);
+                    int kt = 0, slot = 0;
+#pragma unroll 1
+                    for (; kt < ktiles - 1 && (slot = take()) >= 0; ++kt) {
+                        four(slot, kt, d_tmem, 0);
+                        commit<PAIR>(empty_bar(slot));
+                    }
+                    if (ok && (slot = take()) >= 0) {
+                        multiply(slot, kt, d_tmem, 0);
+                        commit<PAIR>(empty_bar(slot));
+                    }
+                    if (!ok) break;
+                    commit<PAIR>(tfull_bar(buf));
                 }
-                __syncwarp();
-                ++issued;
-                if (++s == STAGES) { s = 0; phase ^= 1u; }
+                if (++buf == NBUF) { buf = 0; buf_phase ^= 1u; }
             }
-            if (!ok) break;
+        }
+        __syncwarp();
+    } else if (warp >= C::LOADER_WARP) {
+        // ------------------------------------------------------------------ loader: weight tiles by TMA
+        // item (tile, stage) -> ring slot item % STAGES.  A pair: this CTA's 64 rows of every 128 of the tile; the even CTA expects both
+        // CTAs' bytes, and both complete on its barrier.
+        int s = 0, it = 0;
+        uint32_t phase = 1;                           // first pass through the ring: slots are free
+        TilePos at = walk.first(unit);
+        pdl_wait();
+        for (int kt = 0; it < total_items; ++it) {
+            if (!mbar_wait_warp(empty_bar(s), phase, abort_flag, p.err, ERR_LOADER_TIMEOUT)) break;
+            if (lane == 0) {
+                const uint32_t dst = wring + (uint32_t)s * C::W_BYTES;
+                if (rank == 0) asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(full_bar(s)), "r"((uint32_t)(C::CTAS * C::W_BYTES)) : "memory");
+                if (PAIR)
+                    asm volatile("cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes.cta_group::2 [%0], [%1, {%2, %3, %4, %5}], [%6];"
+                                 ::"r"(dst), "l"(reinterpret_cast<uint64_t>(&wmap)), "r"(kt * ROWB), "r"(0), "r"(rank), "r"(at.n * (BN / 128)), "r"(in_even_cta(full_bar(s))) : "memory");
+                else
+                    asm volatile("cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
+                                 ::"r"(dst), "l"(reinterpret_cast<uint64_t>(&wmap)), "r"(kt * ROWB), "r"(at.n * BN), "r"(full_bar(s)) : "memory");
+            }
+            __syncwarp();
+            if (++kt == ktiles) { kt = 0; walk.next(at); }
+            if (++s == STAGES) { s = 0; phase ^= 1u; }
         }
         // after a time-out elsewhere: copies still in flight must land before the CTA's shared memory goes away
-        if (*abort_flag) {
-            const int first = issued > STAGES ? issued - STAGES : 0;
-            for (int it = first; it < issued; ++it)
-                mbar_wait_warp(full_bar(it % STAGES), (uint32_t)(it / STAGES) & 1u, abort_flag, nullptr, 0);
+        if (*abort_flag && rank == 0) {
+            for (int j = it > STAGES ? it - STAGES : 0; j < it; ++j)
+                mbar_wait_warp(full_bar(j % STAGES), (uint32_t)(j / STAGES) & 1u, abort_flag, nullptr, 0);
         }
+        // (the odd CTA's copies complete on the other's barrier: it gives them a millisecond)
+        if (PAIR && *abort_flag && rank != 0)
+            for (int i = 0; i < 1000; ++i) __nanosleep(1000);
     } else if (warp <= EPI_WARPS) {
         // ------------------------------------------------------------------ epilogue
         const int quad = warp & 3;                 // tensor-memory lane quadrant this warp may read
         const int erow = quad * 32 + lane, team = (warp - 1) >> 2;
+        constexpr int PC = C::PC, PIECES = C::PIECES, CH = PC / 32;             // chunks of 32 columns of a piece
         const uint32_t i32_tile = i32_tiles + (uint32_t)(warp - 1) * I32_TILE_BYTES;
+        // column c of this warp's table: piece c / PC, column h * 128 + team * PC + c % PC of the tile (or team * EC + c)
+        const uint32_t table = tables + (uint32_t)((warp - 1) * EC * 4);
+        const bool narrow = p.K <= 32767;          // int32 outputs fit 16 bits
         bool alive = true;
-        int buf = 0;
+        int buf = 0, table_n = -1;
         uint32_t buf_phase = 0;
-        for (int ti = 0; ti < my_tiles; ++ti) {
-            const int tile = (int)blockIdx.x + ti * (int)gridDim.x;
-            const int n_tile = tile / m_tiles, m_tile = tile - n_tile * m_tiles;
-            const int m0 = m_tile * BM, n0 = n_tile * BN + team * EC;       // this team's columns
-            const int em = m0 + erow;
-            // this tile's column constants, built while its MMAs run; every warp keeps its own table, so the four
-            // warps need no barrier among themselves
-            const uint32_t table = tables + (uint32_t)((warp - 1) * EC * 4);
-            for (int c = lane; c < EC; c += 32) {
-                const int n = n0 + c;
-                int v = 0;
-                if (n < p.C_out) {
-                    v = __ldg(cst + n);
-                    if (FUSED) v -= max(min(__ldg(p.thr + n), p.K + 1), -p.K - 1);       // beyond that bound the decision is constant
+        TilePos at = walk.first(unit);
+        const uint32_t tempty0 = PAIR ? in_even_cta(tempty_bar(0)) : tempty_bar(0);
+        pdl_wait();
+        for (int ti = 0; ti < my_tiles; ++ti, walk.next(at)) {
+            const int n_base = at.n * BN + team * PC;                           // first column of this team's first piece
+            const int em = at.m * C::TILE_ROWS + rank * BM + erow;
+            // the column constants, built while the tile's MMAs run, anew only where the columns change; every warp keeps its own table,
+            // so the four warps need no barrier among themselves
+            if (at.n != table_n) {
+                table_n = at.n;
+                __syncwarp();
+#pragma unroll 1
+                for (int c = lane; c < EC; c += 32) {
+                    const int n = n_base + (c / PC) * (BN / 2) + c % PC;
+                    int v = 0;
+                    if (n < p.C_out) {
+                        v = __ldg(cst + n);
+                        if (FUSED) v -= max(min(__ldg(p.thr + n), p.K + 1), -p.K - 1);       // beyond that bound the decision is constant
+                    }
+                    asm volatile("st.shared.b32 [%0], %1;" ::"r"(table + 4u * c), "r"(table_entry<MODE>(v)) : "memory");
                 }
-                asm volatile("st.shared.b32 [%0], %1;" ::"r"(table + 4u * c), "r"(table_entry<MODE>(v)) : "memory");
+                __syncwarp();
             }
-            __syncwarp();
-            if (alive) alive = mbar_wait(tfull_bar(buf), buf_phase, abort_flag, p.err, ERR_EPILOGUE_TIMEOUT);
-            alive = __all_sync(0xffffffffu, alive && !*abort_flag);
-            if (!alive) break;
-            tc_fence_after();
-            const uint32_t t_addr = tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)(buf * BN + team * EC);
-            uint32_t words[EC / 32];
+            const long row0 = (long)em - lane;
+            const int owords = p.C_out >> 5;
+            uint32_t packed[MODE == 0 ? PIECES : 1][CH][16];                    // int32 outputs of a 256-wide tile, two to a register
 #pragma unroll
-            for (int ch = 0; ch < EC / 32; ++ch) {
-                const int col0 = ch * 32;
-                words[ch] = 0;
-                if (n0 + col0 < p.C_out) {             // warp-uniform
-                    uint32_t v[32];
-                    tc_ld32(t_addr + (uint32_t)col0, v);
-                    if (FUSED) {
-                        words[ch] = threshold_word(v, table + 4u * col0);
-                    } else {
+            for (int h = 0; h < PIECES; ++h) {
+                const int n0 = n_base + h * (BN / 2), b = C::SPLIT ? h : buf;
+                if (alive) alive = pw_wait<100>(tfull_bar(b), buf_phase, abort_flag, p.err, ERR_EPILOGUE_TIMEOUT);
+                alive = __all_sync(0xffffffffu, alive && !*abort_flag);
+                if (!alive) break;
+                tc_fence_after();
+                const uint32_t t_addr = tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)(C::SPLIT ? h * (BN / 2) + team * PC : buf * BN + team * EC);
+                // all reads of this accumulator (half) are complete: hand it back
+                auto hand_back = [&]() {
+                    tc_fence_before();
+                    __syncwarp();
+                    if (PAIR) arrive_in_cluster(tempty0 + 8u * b, lane == 0 ? 1u : 0u);
+                    else if (lane == 0) mbar_arrive(tempty0 + 8u * b);
+                };
+                if (FUSED) {
+                    uint32_t words[CH];
+#pragma unroll
+                    for (int c2 = 0; c2 < CH; c2 += 2) {                        // 64 columns in registers at a time
+                        uint32_t v[2][32];
+                        tc_ld32_nowait(t_addr + 32u * c2, v[0]);
+                        tc_ld32_nowait(t_addr + 32u * c2 + 32u, v[1]);
+                        tc_wait_ld();
+                        pin_regs(v[0]);
+                        pin_regs(v[1]);
+                        if (c2 + 2 == CH) hand_back();
+                        threshold_words(v, table + 4u * (h * PC + 32 * c2), words[c2], words[c2 + 1]);
+                    }
+                    if (em < p.M) {
+                        uint32_t *dst = static_cast<uint32_t *>(p.out) + (long)em * owords + (n0 >> 5);
+                        if (PC >= 128 && (owords & 3) == 0 && n0 + PC <= p.C_out) {
+#pragma unroll
+                            for (int c4 = 0; c4 + 3 < CH; c4 += 4) *reinterpret_cast<uint4 *>(dst + c4) = make_uint4(words[c4], words[c4 + 1], words[c4 + 2], words[c4 + 3]);
+                        } else if ((owords & 1) == 0 && n0 + PC <= p.C_out) {
+#pragma unroll
+                            for (int c2 = 0; c2 < CH; c2 += 2) *reinterpret_cast<uint2 *>(dst + c2) = make_uint2(words[c2], words[c2 + 1]);
+                        } else {
+#pragma unroll
+                            for (int ch = 0; ch < CH; ++ch)
+                                if (n0 + ch * 32 < p.C_out) dst[ch] = words[ch];
+                        }
+                    }
+                } else if (C::SPLIT && narrow) {
+                    // out of the accumulator at once, 16 bits each; to memory below, beside the next tile's MMAs
+#pragma unroll
+                    for (int ch = 0; ch < CH; ++ch) {
+                        uint32_t v[32];
                         int o[32];
-                        biased_ints(v, table + 4u * col0, o);
-                        const long row0 = (long)em - lane;
-                        store_int32_block(static_cast<int32_t *>(p.out) + row0 * p.C_out + n0 + col0, p.C_out, o, i32_tile, row0, p.M, lane, p.C_out - n0 - col0);
+                        tc_ld32(t_addr + 32u * ch, v);
+                        if (ch == CH - 1) hand_back();
+                        biased_ints(v, table + 4u * (h * PC + 32 * ch), o);
+#pragma unroll
+                        for (int i = 0; i < 16; ++i) packed[h][ch][i] = __byte_perm((uint32_t)o[2 * i], (uint32_t)o[2 * i + 1], 0x5410);
+                    }
+                } else {
+#pragma unroll 1
+                    for (int ch = 0; ch < CH; ++ch) {
+                        uint32_t v[32];
+                        int o[32];
+                        if (n0 + 32 * ch < p.C_out) {          // warp-uniform
+                            tc_ld32(t_addr + 32u * ch, v);
+                            biased_ints(v, table + 4u * (h * PC + 32 * ch), o);
+                            store_int32_block(static_cast<int32_t *>(p.out) + row0 * p.C_out + n0 + 32 * ch, p.C_out, o, i32_tile, row0, p.M, lane, p.C_out - n0 - 32 * ch);
+                        }
+                    }
+                    hand_back();
+                }
+            }
+            if (!alive) break;
+            if (MODE == 0 && C::SPLIT && narrow) {
+#pragma unroll
+                for (int h = 0; h < PIECES; ++h) {
+#pragma unroll
+                    for (int ch = 0; ch < CH; ++ch) {
+                        const int col0 = n_base + h * (BN / 2) + 32 * ch;
+                        if (col0 < p.C_out) {                  // warp-uniform
+                            int o[32];
+#pragma unroll
+                            for (int i = 0; i < 16; ++i) {
+                                o[2 * i] = (int)(short)(packed[h][ch][i] & 0xffffu);
+                                o[2 * i + 1] = (int)packed[h][ch][i] >> 16;
+                            }
+                            store_int32_block(static_cast<int32_t *>(p.out) + row0 * p.C_out + col0, p.C_out, o, i32_tile, row0, p.M, lane, p.C_out - col0);
+                        }
                     }
                 }
             }
-            // all reads of this accumulator buffer are complete: hand it back
-            tc_fence_before();
-            __syncwarp();
-            if (lane == 0) mbar_arrive(tempty_bar(buf));
             if (++buf == NBUF) { buf = 0; buf_phase ^= 1u; }
-            if (FUSED && em < p.M) {
-                const int owords = p.C_out >> 5;
-                uint32_t *dst = static_cast<uint32_t *>(p.out) + (long)em * owords + (n0 >> 5);
-                if (EC >= 128 && (owords & 3) == 0 && n0 + EC <= p.C_out) {
-#pragma unroll
-                    for (int c4 = 0; c4 < EC / 128; ++c4)
-                        *reinterpret_cast<uint4 *>(dst + 4 * c4) =
-                            make_uint4(words[4 * c4], words[4 * c4 + 1], words[4 * c4 + 2], words[4 * c4 + 3]);
-                } else if (EC >= 64 && (owords & 1) == 0 && n0 + EC <= p.C_out) {
-#pragma unroll
-                    for (int c2 = 0; c2 < EC / 64; ++c2) *reinterpret_cast<uint2 *>(dst + 2 * c2) = make_uint2(words[2 * c2], words[2 * c2 + 1]);
-                } else {
-#pragma unroll
-                    for (int ch = 0; ch < EC / 32; ++ch)
-                        if (n0 + ch * 32 < p.C_out) dst[ch] = words[ch];
-                }
-            }
         }
     } else {
         // ------------------------------------------------------------------ activation producers
@@ -300,24 +447,23 @@ conv_tc_pre_kernel(const ConvProblem p, const int32_t *cst, const __grid_constan
         const uint32_t bits0 = bits_ring + (uint32_t)ptid * 16u, bits_end = bits0 + PF * SLOT_BYTES;
         const uint32_t st_addr0 = tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)C::A_COL0;
         const uint32_t lane0 = lane == 0 ? 1u : 0u;
-        const TileStep step = make_tile_step(p, (uint32_t)BM * gridDim.x);
+        const TileStep &step = walk.step;
 
         int l_kt = grp;
-        int l_left = total_items > grp ? (total_items - grp + G - 1) / G : 0;
-        int l_n = (int)blockIdx.x / m_tiles, l_m = (int)blockIdx.x - l_n * m_tiles;
+        int l_left = total_items > grp ? (int)((unsigned)(total_items - grp + G - 1) / (unsigned)G) : 0;
+        TilePos at = walk.first(unit);
+        const uint32_t full0 = PAIR ? in_even_cta(full_bar(0)) : full_bar(0);
         RowCursor rc;
-        rc.m = (uint32_t)l_m * BM + (uint32_t)row;
+        rc.m = (uint32_t)(at.m * C::TILE_ROWS + rank * BM + row);
         rc.base = 0;
         rc.mask = 0;
         row_locate(p, rc);
-        auto next_tile = [&]() {             // the CTA's next tile: gridDim.x further along (n_tile, m_tile)
-            l_m += (int)gridDim.x;
-            if (l_m < m_tiles) {
-                row_step(p, step, rc);
-            } else {
-                do { l_m -= m_tiles; ++l_n; } while (l_m >= m_tiles);
-                rc.m = (uint32_t)l_m * BM + (uint32_t)row;
+        auto next_tile = [&]() {             // the CTA's next tile
+            if (walk.next(at)) {
+                rc.m = (uint32_t)(at.m * C::TILE_ROWS + rank * BM + row);
                 row_locate(p, rc);
+            } else {
+                row_step(p, step, rc);
             }
         };
         while (l_kt >= ktiles) { l_kt -= ktiles; next_tile(); }
@@ -338,6 +484,7 @@ conv_tc_pre_kernel(const ConvProblem p, const int32_t *cst, const __grid_constan
                 row_window(p, step, rc);
             }
         };
+        pdl_wait();
 #pragma unroll 1
         for (int i = 0; i < PF - 1; ++i) {
             if (l_left > 0) issue_load();
@@ -348,19 +495,22 @@ conv_tc_pre_kernel(const ConvProblem p, const int32_t *cst, const __grid_constan
         uint32_t phase = 1;                   // first pass through the ring: slots are free
 #pragma unroll 1
         for (int it = grp; it < total_items; it += G) {
-            if (l_left > 0) issue_load();
-            cp_async_commit();
-            cp_async_wait<PF - 1>();
+            cp_async_wait<PF - 2>();
             uint32_t v[32];
             expand_stage8(ld_shared_v4(c_src), ld_shared_v4(c_src + HALF_BYTES), v);
             c_src += SLOT_BYTES;
             if (c_src == bits_end) c_src = bits0;
             if (!mbar_wait_warp(empty_bar(s), phase, abort_flag, p.err, ERR_PRODUCER_TIMEOUT)) break;
             tc_fence_after();     // the MMAs that read this slot are complete (their commit released it)
-            tc_st32(st_addr0 + (uint32_t)s * 32u, v);
+            tc_st32_nowait(st_addr0 + (uint32_t)s * 32u, v);
+            // the next copies are issued while the store completes
+            if (l_left > 0) issue_load();
+            cp_async_commit();
+            tc_wait_st();
             tc_fence_before();
             __syncwarp();
-            mbar_arrive_pred(full_bar(s), lane0);
+            if (PAIR) arrive_in_cluster(full0 + 8u * s, lane0);
+            else mbar_arrive_pred(full0 + 8u * s, lane0);
             s += G;
             if (s >= STAGES) { s -= STAGES; phase ^= 1u; }
         }
@@ -368,9 +518,11 @@ conv_tc_pre_kernel(const ConvProblem p, const int32_t *cst, const __grid_constan
     }
 
     tc_fence_before();
-    __syncthreads();
+    if (PAIR) cluster_barrier();               // nothing of the other CTA's refers to this one's memory any more
+    else __syncthreads();
     if (warp == 0) {
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(512u) : "memory");
+        if (PAIR) asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(512u) : "memory");
+        else asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(512u) : "memory");
     }
 }
 
@@ -398,34 +550,36 @@ prepare_weights_kernel(const uint32_t *w, uint8_t *wexp, int32_t *cst, int N, in
 
 int ktab_words_for(const ConvProblem &p) { return ((p.kwords + 7) >> 3) * (8 / gather_width(p.cw)); }
 
-template <int BN, int MODE, int G, int TEAMS>
+template <int BN, int MODE, int G, int TEAMS, bool PAIR>
 int launch_bn(const ConvProblem &p0, const PreparedWeights &pw, cudaStream_t stream)
 {
-    using C = Cfg<BN, MODE, G, TEAMS>;
+    using C = Cfg<BN, MODE, G, TEAMS, PAIR>;
     ConvProblem p = p0;
     p.err = device_error_word();
-    const int sms = sm_count();
-    const long m_tiles = ((long)p.M + BM - 1) / BM;
+    const long units = sm_count() / C::CTAS;
+    const long m_tiles = ((long)p.M + C::TILE_ROWS - 1) / C::TILE_ROWS;
     const long n_tiles = ((long)p.C_out + BN - 1) / BN;
     const long total = m_tiles * n_tiles;
     if (total >= (1L << 31)) return BCNN_ERR_UNSUPPORTED;
-    const unsigned grid = (unsigned)(total < sms ? total : sms);
+    const int grid = (int)(total < units ? total : units);
     const int ktw = ktab_words_for(p);
     const int smem = smem_bytes<C>(ktw, MODE);
     if (smem > MAX_SMEM) return BCNN_ERR_UNSUPPORTED;
     EncodeTiledFn encode = encode_tiled_fn();
     if (!encode) return BCNN_ERR_CUDA;
     CUtensorMap wmap;
-    const cuuint64_t dims[2] = {(cuuint64_t)pw.k_pad / 2, (cuuint64_t)pw.n_pad};       // bytes of a row, rows
-    const cuuint64_t strides[1] = {(cuuint64_t)pw.k_pad / 2};
-    const cuuint32_t box[2] = {(cuuint32_t)ROWB, (cuuint32_t)BN};
-    const cuuint32_t estr[2] = {1, 1};
-    if (encode(&wmap, CU_TENSOR_MAP_DATA_TYPE_UINT8, 2, const_cast<uint8_t *>(pw.wexp), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+    // rows of k_pad / 2 bytes; for a pair as (128 rows, half of them, row)
+    const cuuint64_t pitch = (cuuint64_t)pw.k_pad / 2;
+    const cuuint64_t dims[4] = {pitch, PAIR ? 64u : (cuuint64_t)pw.n_pad, 2, (cuuint64_t)pw.n_pad / 128};
+    const cuuint64_t strides[3] = {pitch, 64 * pitch, 128 * pitch};
+    const cuuint32_t box[4] = {(cuuint32_t)ROWB, PAIR ? 64u : (cuuint32_t)BN, 1, PAIR ? (cuuint32_t)BN / 128 : 1};
+    const cuuint32_t estr[4] = {1, 1, 1, 1};
+    if (encode(&wmap, CU_TENSOR_MAP_DATA_TYPE_UINT8, PAIR ? 4 : 2, const_cast<uint8_t *>(pw.wexp), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
                CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
         return BCNN_ERR_CUDA;
-    auto k = conv_tc_pre_kernel<BN, MODE, G, TEAMS>;
+    auto k = conv_tc_pre_kernel<BN, MODE, G, TEAMS, PAIR>;
     if (!allow_smem((const void *)k, MAX_SMEM)) return BCNN_ERR_CUDA;
-    return launch(k, grid, C::THREADS, smem, stream, p, pw.cst, wmap, ktw);
+    return launch<C::CTAS>(k, (unsigned)(grid * C::CTAS), C::THREADS, smem, stream, p, pw.cst, wmap, ktw, make_tile_walk(p, C::TILE_ROWS, (int)m_tiles, (int)total, grid));
 }
 
 }  // namespace
@@ -501,7 +655,7 @@ bool conv_tc_pre_supports(const ConvProblem &p)
     if (p.mode == 1 && (p.C_out % 32 != 0)) return false;
     if (p.kh * p.kw > 31) return false;                       // one validity bit per tap
     if ((long)p.B * p.H * p.W * p.cw >= (1L << 31)) return false;     // rows address the input by 32-bit word offsets
-    if (smem_bytes<Cfg<256, 1, 2, 2>>(ktab_words_for(p), 1) > MAX_SMEM) return false;      // (the widths below need no more, but for one)
+    if (smem_bytes<Cfg<256, 1, 2, 2, false>>(ktab_words_for(p), 1) > MAX_SMEM) return false;      // (the widths below need no more, but for one)
     if ((long)p.kh * p.W * p.cw >= (1L << 27)) return false;  // a unit's word offset within the window
     return p.K <= (1 << 20);                                  // sums up to 4 K + 2 stay exact in fp32
 }
@@ -514,28 +668,49 @@ int launch_conv_tc_pre(const ConvProblem &p, const void *prepared, cudaStream_t 
     prepared_layout(p.C_out, p.K, pw, bytes);
     pw.wexp = static_cast<const uint8_t *>(prepared);
     pw.cst = reinterpret_cast<const int32_t *>(pw.wexp + (size_t)pw.n_pad * pw.k_pad / 2);
-    // Tile width: 256 (two epilogue teams, one accumulator: the epilogue is not overlapped), 128 or 64.  Narrow tiles spread a
-    // small layer over more multiprocessors and shorten its epilogue, but every tile expands its activation rows again.
-    // Estimated time in ns, fitted to layers and products on B200 (28 shapes, within 10 %): a start, a term per tile column
-    // of the longest CTA and one per 256-bit stage.
-    //   3x3 256 -> 256, M = 50176: 16.0 (256), 16.7 (128), 25.5 (64) us;  M = 196: 6.9, 5.6, 5.2;  512 -> 512, M = 12544: 16.9, 15.9, 25.5
+    // Tile width: 256, 128 or 64 columns.  Narrow tiles spread a small layer over more multiprocessors and shorten its epilogue, but
+    // every tile expands its activation rows again.  Estimated time in ns, fitted to 40 layers and products per output on B200 (the choice is
+    // within 6 % of the best width on all but two): a start, a term per tile column of the longest CTA, one per 256-bit stage - longer
+    // where the gather goes by single or paired words - and one for the tiles that compete for memory at the start.
+    //   packed, us at 64 / 128 / 256: 3x3 256 -> 256 at M = 50176 25.3, 15.5, 13.2; M = 196 4.0, 4.3, 5.6; 512 -> 512 at M = 12544 26.4, 15.2, 14.8;
+    //   3x3 128 -> 128 at M = 6272 3.9, 3.6, 4.7; int32: 256 -> 256 at M = 50176 28.4, 21.3, 22.0; 1000 x 4000 x 2304 12.4, 9.6, 10.7
     const int sms = sm_count();
     const long m_tiles = ((long)p.M + BM - 1) / BM, kt = (p.kwords + 7) / 8;
+    const bool wide_gather = gather_width(p.cw) == 4;
+    auto waves_of = [&](int bn) { return (m_tiles * ((p.C_out + bn - 1) / bn) + sms - 1) / sms; };
     auto cost = [&](int bn, long start, long wave, long stage) {
-        const long waves = (m_tiles * ((p.C_out + bn - 1) / bn) + sms - 1) / sms;
-        return start + waves * (wave + kt * stage);
+        const long tiles = m_tiles * ((p.C_out + bn - 1) / bn);
+        return start + waves_of(bn) * (wave + kt * stage) + 7 * (tiles < sms ? tiles : sms);
     };
     const bool packed = p.mode == 1;
     // What conv_tc_pre_supports vouches for is the packed 256-wide variant's shared memory.  The int32 one needs its store staging
     // tiles besides: a K beyond 274 176 bits with an odd number of words per pixel, 548 352 with an even one, runs on narrower tiles.
-    static_assert(smem_bytes<Cfg<128, 0, 3, 2>>(0, 0) <= smem_bytes<Cfg<256, 1, 2, 2>>(0, 1) && smem_bytes<Cfg<64, 0, 2, 1>>(0, 0) <= smem_bytes<Cfg<256, 1, 2, 2>>(0, 1) &&
-                  smem_bytes<Cfg<128, 1, 2, 1>>(0, 1) <= smem_bytes<Cfg<256, 1, 2, 2>>(0, 1) && smem_bytes<Cfg<64, 1, 2, 1>>(0, 1) <= smem_bytes<Cfg<256, 1, 2, 2>>(0, 1),
+    static_assert(smem_bytes<Cfg<128, 0, 3, 2, false>>(0, 0) <= smem_bytes<Cfg<256, 1, 2, 2, false>>(0, 1) && smem_bytes<Cfg<64, 0, 2, 1, false>>(0, 0) <= smem_bytes<Cfg<256, 1, 2, 2, false>>(0, 1) &&
+                  smem_bytes<Cfg<128, 1, 2, 1, false>>(0, 1) <= smem_bytes<Cfg<256, 1, 2, 2, false>>(0, 1) && smem_bytes<Cfg<64, 1, 2, 1, false>>(0, 1) <= smem_bytes<Cfg<256, 1, 2, 2, false>>(0, 1),
                   "a supported layer fits the narrower tiles");
-    const bool fits256 = packed || smem_bytes<Cfg<256, 0, 2, 2>>(ktab_words_for(p), 0) <= MAX_SMEM;
-    const long c256 = fits256 ? cost(256, 3200, packed ? 1660 : 4300, 288) : LONG_MAX, c128 = cost(128, 3500, packed ? 600 : 2200, 185), c64 = cost(64, 3100, packed ? 530 : 1150, 167);
-    if (c64 <= c128 && c64 <= c256) return packed ? launch_bn<64, 1, 2, 1>(p, pw, stream) : launch_bn<64, 0, 2, 1>(p, pw, stream);
-    if (c128 <= c256) return packed ? launch_bn<128, 1, 2, 1>(p, pw, stream) : launch_bn<128, 0, 3, 2>(p, pw, stream);
-    return packed ? launch_bn<256, 1, 2, 2>(p, pw, stream) : launch_bn<256, 0, 2, 2>(p, pw, stream);
+    static_assert(smem_bytes<Cfg<256, 0, 2, 2, true>>(0, 0) <= smem_bytes<Cfg<256, 0, 2, 2, false>>(0, 0) && smem_bytes<Cfg<256, 1, 2, 2, true>>(0, 1) <= smem_bytes<Cfg<256, 1, 2, 2, false>>(0, 1),
+                  "and the tile of two blocks");
+    const bool fits256 = packed || smem_bytes<Cfg<256, 0, 2, 2, false>>(ktab_words_for(p), 0) <= MAX_SMEM;
+    long c256 = LONG_MAX, c128, c64;
+    if (packed) {
+        c64 = cost(64, 2150, 160, wide_gather ? 212 : 330);
+        c128 = cost(128, 2300, 320, wide_gather ? 210 : 350);
+        // (the first tile column: nothing of it waits for an epilogue; a short K waits for every epilogue)
+        const long stage = wide_gather ? 283 : 350, rest = 910 + kt * stage;
+        c256 = cost(256, 3000 + kt * stage, 0, 0) + (waves_of(256) - 1) * (rest > 2200 ? rest : 2200);
+    } else {
+        c64 = cost(64, 2450, 270, wide_gather ? 212 : 330);
+        c128 = cost(128, 3000, 700, wide_gather ? 225 : 340);
+        if (fits256) c256 = cost(256, 3500, 4300, wide_gather ? 270 : 340);
+    }
+    if (c64 < c128 && c64 <= c256) return packed ? launch_bn<64, 1, 2, 1, false>(p, pw, stream) : launch_bn<64, 0, 2, 1, false>(p, pw, stream);
+    if (c128 <= c256) return packed ? launch_bn<128, 1, 2, 1, false>(p, pw, stream) : launch_bn<128, 0, 3, 2, false>(p, pw, stream);
+    // Two multiprocessors on a tile of 256 x 256: half the weight bytes from L2 and into shared memory.  That pays where the tensor pipe is
+    // kept busy for long - what limits such a product is power, the clock falls to 1.6 GHz (seconds of 16384 x 16384 x 9216 in a row: int32
+    // 978 -> 877 us, packed 774 -> 745; 25088 x 512 x 4608 33.1 -> 30.7 and 23.1 -> 22.7; 16384 x 16384 x 2304 packed 231 -> 218) - and costs a hand-over between
+    // the two elsewhere (50176 x 256 x 2304, three waves: 13.2 -> 14.0)
+    if (waves_of(256) >= 8 || (waves_of(256) >= 3 && p.K >= 4096)) return packed ? launch_bn<256, 1, 2, 2, true>(p, pw, stream) : launch_bn<256, 0, 2, 2, true>(p, pw, stream);
+    return packed ? launch_bn<256, 1, 2, 2, false>(p, pw, stream) : launch_bn<256, 0, 2, 2, false>(p, pw, stream);
 }
 
 }  // namespace bcnn

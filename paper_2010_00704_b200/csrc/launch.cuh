@@ -30,21 +30,24 @@ template <typename T> struct Same { using type = T; };
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
-// kernel<<<grid, threads, smem, stream>>>(args...), the arguments converted to the kernel's parameter types.
-template <typename... P>
+// kernel<<<grid, threads, smem, stream>>>(args...), the arguments converted to the kernel's parameter types; in clusters of CLUSTER blocks.
+template <int CLUSTER = 1, typename... P>
 int launch(void (*kernel)(P...), dim3 grid, unsigned threads, size_t smem, cudaStream_t stream, typename Same<P>::type... args)
 {
     void *argv[] = {const_cast<void *>(static_cast<const void *>(&args))...};
-    cudaLaunchAttribute dependent;
-    dependent.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    dependent.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchAttribute attrs[2];
+    attrs[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attrs[0].val.programmaticStreamSerializationAllowed = 1;
+    attrs[1].id = cudaLaunchAttributeClusterDimension;
+    attrs[1].val.clusterDim.x = CLUSTER;
+    attrs[1].val.clusterDim.y = attrs[1].val.clusterDim.z = 1;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
     cfg.blockDim = dim3(threads);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = stream;
-    cfg.attrs = &dependent;
-    cfg.numAttrs = 1;
+    cfg.attrs = attrs;
+    cfg.numAttrs = CLUSTER > 1 ? 2 : 1;
     if (cudaLaunchKernelExC(&cfg, reinterpret_cast<const void *>(kernel), argv) == cudaSuccess) return BCNN_OK;
     (void)cudaGetLastError();                 // a refused launch leaves no error behind for the caller's next check
     return BCNN_ERR_CUDA;

@@ -178,6 +178,20 @@ __device__ __forceinline__ void tc_ld32(uint32_t taddr, uint32_t (&v)[32])
         : "r"(taddr) : "memory");
 }
 
+// Without the wait, for several loads followed by one tc_wait_ld() (and pin_regs on each destination, tc_slot.cuh).
+__device__ __forceinline__ void tc_ld32_nowait(uint32_t taddr, uint32_t (&v)[32])
+{
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
+        "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"
+        "%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
+        : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
+          "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15]),
+          "=r"(v[16]), "=r"(v[17]), "=r"(v[18]), "=r"(v[19]), "=r"(v[20]), "=r"(v[21]), "=r"(v[22]), "=r"(v[23]),
+          "=r"(v[24]), "=r"(v[25]), "=r"(v[26]), "=r"(v[27]), "=r"(v[28]), "=r"(v[29]), "=r"(v[30]), "=r"(v[31])
+        : "r"(taddr) : "memory");
+}
+
 // K-major tile, 128-byte rows, 128-byte swizzle, 8-row groups 1024 bytes apart, descriptor version 1.
 __device__ __forceinline__ uint64_t make_desc(uint32_t saddr)
 {
@@ -251,6 +265,31 @@ __device__ __forceinline__ uint32_t threshold_word(const uint32_t (&v)[32], uint
     // integers below 2^16 in the low mantissa bits of 2^23 + x
     return __byte_perm(__float_as_uint(lo + 8388608.0f), __float_as_uint(hi + 8388608.0f), 0x5410);
 }
+// Two words of 64 consecutive columns at once: four chains instead of two, the next eight columns' constants on their way.
+__device__ __forceinline__ void threshold_words(const uint32_t (&v)[2][32], uint32_t table, uint32_t &w0, uint32_t &w1)
+{
+    float acc[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+    uint4 c[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) c[q] = ld_shared_v4(table + 64u * q + 48u);
+#pragma unroll
+    for (int i4 = 3; i4 >= 0; --i4) {
+        uint32_t cc[4][4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            cc[q][0] = c[q].x; cc[q][1] = c[q].y; cc[q][2] = c[q].z; cc[q][3] = c[q].w;
+            if (i4) c[q] = ld_shared_v4(table + 64u * q + 16u * (i4 - 1));
+        }
+#pragma unroll
+        for (int i = 3; i >= 0; --i) {
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+                acc[q] = fmaf(acc[q], 2.0f, __saturatef(fmaf(__uint_as_float(v[q >> 1][16 * (q & 1) + 4 * i4 + i]), 2.0f, __uint_as_float(cc[q][i]))));
+        }
+    }
+    w0 = __byte_perm(__float_as_uint(acc[0] + 8388608.0f), __float_as_uint(acc[1] + 8388608.0f), 0x5410);
+    w1 = __byte_perm(__float_as_uint(acc[2] + 8388608.0f), __float_as_uint(acc[3] + 8388608.0f), 0x5410);
+}
 // ... and 32 exact integers v + c, with c + INT_BIAS of column i at table + 4 i.
 __device__ __forceinline__ void biased_ints(const uint32_t (&v)[32], uint32_t table, int (&o)[32])
 {
@@ -314,6 +353,44 @@ __host__ __device__ __forceinline__ TileStep make_tile_step(const ConvProblem &p
     s.pointwise = p.kh == 1 && p.kw == 1 && p.stride == 1 && p.pad == 0;
     return s;
 }
+// A persistent CTA's way through the tiles (n, m), m fastest: from tile blockIdx.x in steps of gridDim.x.  All divisions are the
+// host's: an integer division is some twenty instructions, and in code that runs once an instruction costs some ten cycles.
+struct TilePos {
+    int n, m;
+};
+struct TileWalk {
+    int m_tiles, tiles, extra;       // row tiles; every CTA's tiles, and the number of CTAs that have one more
+    int dn, dm;                      // gridDim.x = dn * m_tiles + dm
+    uint32_t mul, shift;             // exact_div by m_tiles
+    TileStep step;                   // of the rows of two consecutive tiles, as long as n does not change
+    __device__ __forceinline__ int tiles_of(int cta) const { return tiles + (cta < extra ? 1 : 0); }
+    __device__ __forceinline__ TilePos first(int cta) const
+    {
+        const int n = (int)exact_div((uint32_t)cta, mul, shift);
+        return {n, cta - n * m_tiles};
+    }
+    // true where the next tile's rows are not `step` behind the last one's
+    __device__ __forceinline__ bool next(TilePos &t) const
+    {
+        t.n += dn;
+        t.m += dm;
+        const bool wrap = t.m >= m_tiles;
+        if (wrap) { t.m -= m_tiles; ++t.n; }
+        return wrap || dn > 0;
+    }
+};
+inline TileWalk make_tile_walk(const ConvProblem &p, int tile_rows, int m_tiles, int total, int grid)
+{
+    TileWalk w;
+    w.m_tiles = m_tiles;
+    w.tiles = total / grid;
+    w.extra = total % grid;
+    w.dn = grid / m_tiles;
+    w.dm = grid % m_tiles;
+    exact_div_params((uint32_t)m_tiles, w.mul, w.shift);
+    w.step = make_tile_step(p, (uint32_t)tile_rows * (uint32_t)grid);
+    return w;
+}
 struct RowCursor {
     uint32_t m;              // row of the implicit patch matrix
     int b, oh, ow;
@@ -375,8 +452,8 @@ __device__ __forceinline__ void build_unit_table8(const ConvProblem &p, uint32_t
         const int kword = u * gw;
         uint32_t ent = (uint32_t)TAP_NONE << 27;
         if (kword < p.kwords) {
-            const int tap = kword / p.cw, cj = kword - tap * p.cw;
-            const int r = tap / p.kw, t = tap - r * p.kw;
+            const int tap = p.cw_magic ? (int)__umulhi((uint32_t)kword, p.cw_magic) : kword, cj = kword - tap * p.cw;
+            const int r = p.kw_magic ? (int)__umulhi((uint32_t)tap, p.kw_magic) : tap, t = tap - r * p.kw;
             ent = (uint32_t)((r * p.W + t) * p.cw + cj) | ((uint32_t)tap << 27);
         }
         asm volatile("st.shared.b32 [%0], %1;" ::"r"(tab_addr + 4u * u), "r"(ent) : "memory");

@@ -80,6 +80,21 @@ __device__ __forceinline__ bool pw_wait(uint32_t bar, uint32_t parity, volatile 
     return __all_sync(0xffffffffu, ok);
 }
 
+// The wait of a lane that issues MMAs: no sleep, nothing but the question while it is answered with no (one lane of one warp asks).
+__device__ __forceinline__ bool issuer_wait(uint32_t bar, uint32_t parity, volatile int *abort_flag, int *err, int code)
+{
+    for (uint32_t it = 0; !mbar_try_wait(bar, parity); ++it) {
+        if ((it & 4095u) != 4095u) continue;
+        if (*abort_flag) return false;
+        if (it > (1u << 25)) {                 // some seconds
+            *abort_flag = 1;
+            if (err) atomicCAS(err, 0, code);
+            return false;
+        }
+    }
+    return true;
+}
+
 // Per-channel constants by an MMA, and sums that fit 16 bits.  A tile's first MMA (not accumulating) multiplies a constant
 // activation tile with a constant row per channel and leaves BIAS + c in the accumulator: the first K block of 32 has one
 // product 4 * 6 at scale 2^16 = BIAS, the second, at scale 4, adds up to the integer c.  BIAS = 1.5 * 2^20 keeps every

@@ -253,3 +253,17 @@ def test_module_special_values(bk, oracle, shape, P, has_nb):
     assert np.array_equal(np.where(np.isnan(got), 0, got.view(np.uint16)), np.where(np.isnan(want_y), 0, want_y.view(np.uint16)))
     assert np.array_equal(synth.unpack_bits(bits.cpu().numpy().reshape(B, H, W, C // 8)), want_s)
     assert bk.bcnn_device_error() == 0
+
+
+# two blocks on a tile of 256 rows x 256 columns: three waves of tiles with a K of 4096 bits and more, and eight with a short one; the
+# last row tile and the last columns part empty, an odd number of 128-column groups, K with a tail of every length in its last stage
+@pytest.mark.parametrize("M,N,K,fused", [(25100, 512, 4608, True), (29000, 480, 4128, True), (14336, 1000, 4192, False), (40000, 1152, 288, True),
+                                         (9500, 1100, 4448, False), (30011, 640, 4352, True), (152000, 256, 96, True)])
+def test_prepared_block_pairs(bk, oracle, M, N, K, fused):
+    test_prepared_widths(bk, oracle, M, N, K, fused)
+
+
+# 256-wide tiles handed over in halves: one to five stages (none, one and two of them split at either end), several tiles per block
+@pytest.mark.parametrize("K", [32, 256, 288, 512, 768, 992, 1056])
+def test_prepared_split_tiles(bk, oracle, K):
+    test_prepared_widths(bk, oracle, 50000, 256, K, True)
