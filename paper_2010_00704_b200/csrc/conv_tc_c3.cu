@@ -35,6 +35,8 @@
 // completion k - 1 has happened.  Tile m + NB cannot be done before the waiter is through: the fills of the tiles from
 // m + 2 D on need tile m + D (or a later one of its issuer) done, hence filled; NB being a multiple of NACC, it also needs the
 // accumulator of tile m back from the epilogue.
+// A launch's set-up - barriers by a thread each, divisions by the host, every role's wait for the previous kernel behind its own
+// set-up - is half a microsecond of a small layer: 3x3 32 -> 64 /2 at M = 3136 3.0 -> 2.8 us, at M = 200704 6.15 -> 5.85; 64 -> 64 at M = 3136 3.6 -> 3.3.
 // Every mbarrier wait is bounded and reports through the device error word.
 #include "tc_slot.cuh"
 #include "tensor_map.cuh"
@@ -53,7 +55,8 @@ constexpr int ERR_C3_UNIT_TIMEOUT = 145;         // producer: the unit's previou
 constexpr int ERR_C3_ACC_TIMEOUT = 146;          // issuer: an accumulator was not handed back
 
 constexpr int TH = 8, TW = 16;            // output tile (TH * TW = 128 = tensor-memory lanes)
-constexpr int NGRP = 2;                   // loader / epilogue groups (alternate tiles)
+constexpr int NGRP = 2;                   // epilogue groups (alternate tiles)
+constexpr int NLD = 2;                    // loader warps (alternate tiles; four with half the ring each: 34.9 -> 36.3 us on the first 3x3/2 layer)
 constexpr int NPG = 4;                    // producer groups of four warps
 constexpr int RD = 6;                     // halo tiles in a loader's ring
 constexpr int TAPS = 9, UWORDS = 10;      // K words of a unit: the nine taps and a zero
@@ -80,7 +83,7 @@ template <int CW, int BN> struct C3Cfg {
     // warps: issuers, two loaders, then the producer groups, then the epilogue groups (warp % 4 is the tensor-memory lane
     // quadrant of a warp: any four consecutive warps cover all of them)
     static constexpr int FIRST_LOADER_WARP = NISS;
-    static constexpr int FIRST_PRODUCER_WARP = FIRST_LOADER_WARP + NGRP;
+    static constexpr int FIRST_PRODUCER_WARP = FIRST_LOADER_WARP + NLD;
     static constexpr int FIRST_EPILOGUE_WARP = FIRST_PRODUCER_WARP + 4 * NPG;
     static constexpr int WARPS = FIRST_EPILOGUE_WARP + 4 * NGRP;
     static constexpr int THREADS = 32 * WARPS;
@@ -93,6 +96,11 @@ struct C3Geom {
     int stage_bytes;         // hb * wbw * 4 rounded up to 128
     int tiles_x, tiles_y;    // tiles per image row / column of tiles
     int total_tiles;
+    int tiles, extra;        // tiles of every CTA; CTAs that have one more
+    uint32_t img_mul, img_shift, row_mul, row_shift;      // exact_div by the tiles of an image and of a row of tiles
+    struct Step {
+        int db, dty, dtx;    // images, rows of tiles and tiles
+    } step[2];               // one and two of the CTA's tiles further
 };
 
 C3Geom c3_geometry(const ConvProblem &p)
@@ -110,12 +118,25 @@ C3Geom c3_geometry(const ConvProblem &p)
     g.total_tiles = p.B * g.tiles_x * g.tiles_y;
     return g;
 }
+// what depends on the grid: the divisions, done here
+void c3_walk(C3Geom &g, unsigned grid)
+{
+    const unsigned per_img = (unsigned)(g.tiles_x * g.tiles_y);
+    g.tiles = (int)((unsigned)g.total_tiles / grid);
+    g.extra = (int)((unsigned)g.total_tiles % grid);
+    exact_div_params(per_img, g.img_mul, g.img_shift);
+    exact_div_params((uint32_t)g.tiles_x, g.row_mul, g.row_shift);
+    for (int i = 0; i < 2; ++i) {
+        const unsigned st = grid << i, rem = st % per_img;
+        g.step[i] = {(int)(st / per_img), (int)(rem / (unsigned)g.tiles_x), (int)(rem % (unsigned)g.tiles_x)};
+    }
+}
 
 template <int CW, int BN>
 int c3_smem_bytes(const C3Geom &g)
 {
     using C = C3Cfg<CW, BN>;
-    return 1024 + (C::KT + 1) * C::W_TILE_BYTES + (BN * 4 + 127) / 128 * 128 + NGRP * RD * g.stage_bytes + 128;
+    return 1024 + (C::KT + 1) * C::W_TILE_BYTES + (BN * 4 + 127) / 128 * 128 + NLD * RD * g.stage_bytes + 128;
 }
 
 template <int CW, int BN>
@@ -124,7 +145,7 @@ conv_tc_c3_kernel(const ConvProblem p, const C3Geom g, const __grid_constant__ C
 {
     using C = C3Cfg<CW, BN>;
     constexpr int KT = C::KT, NACC = C::NACC, NUNIT = C::NUNIT, NH = C::NH, AW = C::AW;
-    constexpr int NBARS = 2 * NGRP * RD + NAF + NB + MAX_NACC;
+    constexpr int NBARS = 2 * NLD * RD + NAF + NB + MAX_NACC;
 
     extern __shared__ unsigned char smem_raw[];
     __shared__ __align__(8) unsigned long long bars[NBARS];
@@ -137,7 +158,7 @@ conv_tc_c3_kernel(const ConvProblem p, const C3Geom g, const __grid_constant__ C
     // accumulator n % NACC, "full" barrier n % NAF, "done" barrier n % NB (two halves: both epilogue groups, accumulator =
     // half, "done" barrier (2 n + half) % NB); its unit h is the CTA's unit number n * CW + h,
     // in ring position (n * CW + h) % NUNIT
-    const int my_tiles = (int)blockIdx.x < g.total_tiles ? (g.total_tiles - 1 - (int)blockIdx.x) / (int)gridDim.x + 1 : 0;
+    const int my_tiles = g.tiles + ((int)blockIdx.x < g.extra ? 1 : 0);
     const int cn = min(BN, p.C_out);
 
     const uint32_t wexp = (smem_u32(smem_raw) + 1023u) & ~1023u;          // [KT][BN rows][128 B] expanded weights
@@ -146,23 +167,20 @@ conv_tc_c3_kernel(const ConvProblem p, const C3Geom g, const __grid_constant__ C
     const uint32_t ring = pops + (BN * 4 + 127) / 128 * 128;              // [NGRP][RD] halo tiles
     const uint32_t bar0 = smem_u32(bars);
     auto load_full = [&](int gr, int s) { return bar0 + 8u * (gr * RD + s); };
-    auto load_empty = [&](int gr, int s) { return bar0 + 8u * (NGRP * RD + gr * RD + s); };
-    auto a_full = [&](int s) { return bar0 + 8u * (2 * NGRP * RD + s); };
-    auto tile_done = [&](int s) { return bar0 + 8u * (2 * NGRP * RD + NAF + s); };
-    auto acc_free = [&](int s) { return bar0 + 8u * (2 * NGRP * RD + NAF + NB + s); };
+    auto load_empty = [&](int gr, int s) { return bar0 + 8u * (NLD * RD + gr * RD + s); };
+    auto a_full = [&](int s) { return bar0 + 8u * (2 * NLD * RD + s); };
+    auto tile_done = [&](int s) { return bar0 + 8u * (2 * NLD * RD + NAF + s); };
+    auto acc_free = [&](int s) { return bar0 + 8u * (2 * NLD * RD + NAF + NB + s); };
     volatile int *abort_flag = &abort_flag_smem;
 
-    if (tid == 0) {
-        for (int s = 0; s < NGRP * RD; ++s) {
-            mbar_init(load_full(0, s), 1);              // the loader's arrive (+ the copy's bytes)
-            mbar_init(load_empty(0, s), 4 * CW);        // the producer warps that read the stage
-        }
-        for (int s = 0; s < NAF; ++s) mbar_init(a_full(s), 4 * CW);     // the producer warps that fill the tile's units
-        for (int s = 0; s < NB; ++s) mbar_init(tile_done(s), 1);        // the issuer's commit
-        for (int s = 0; s < MAX_NACC; ++s) mbar_init(acc_free(s), 4);   // the four epilogue warps of the tile's group
-        abort_flag_smem = 0;
+    if (tid < NBARS) {
+        // a stage loaded: the loader's arrive (+ the copy's bytes); free again: the producer warps that read it; a tile's units full: the
+        // producer warps that fill them; done: the issuer's commit; an accumulator free: the four epilogue warps of the tile's group
+        constexpr int E0 = NLD * RD, F0 = 2 * NLD * RD, D0 = F0 + NAF, A0 = D0 + NB;
+        mbar_init(bar0 + 8u * tid, tid < E0 || (tid >= D0 && tid < A0) ? 1 : (tid >= A0 ? 4 : 4 * CW));
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
+    if (tid == 0) abort_flag_smem = 0;
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base_smem)), "r"(512u) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
@@ -173,19 +191,19 @@ conv_tc_c3_kernel(const ConvProblem p, const C3Geom g, const __grid_constant__ C
     __syncthreads();
     tc_fence_after();
     pdl_trigger();
-    pdl_wait();
     // The loader warps start now: the first halo tiles arrive while the other warps expand the weights (0.5 us of a small layer's
     // 4).  The other warps meet at a named barrier of their own; everybody meets again at the end.
     const bool is_loader = warp >= C::FIRST_LOADER_WARP && warp < C::FIRST_PRODUCER_WARP;
     const uint32_t tmem_base = tmem_base_smem;
     if (!is_loader) {
-        constexpr int NW = C::THREADS - 64, WTOTAL = KT * 8 * BN, WU = (WTOTAL + NW - 1) / NW;
-        const int wt = tid < 32 * C::FIRST_LOADER_WARP ? tid : tid - 64;       // (the loaders are 64 threads)
+        constexpr int NW = C::THREADS - 32 * NLD, WTOTAL = KT * 8 * BN, WU = (WTOTAL + NW - 1) / NW;
+        const int wt = tid < 32 * C::FIRST_LOADER_WARP ? tid : tid - 32 * NLD;
         auto sync_workers = [&]() { asm volatile("bar.sync 1, %0;" ::"n"(NW) : "memory"); };
         // ---- one-off: expanded weights and the channels' bit counts.  K position e of the MMAs = channel word e / 10, tap e % 10
         // (global weight word tap * CW + channel word) -> stage e / 8, 16-byte piece e % 8; MMA row `row` carries channel ch.
         // All of a thread's words, and its threshold, are requested before the first is used.
         const int my_ch = (wt & ~31) + channel_of_column(wt & 31);
+        pdl_wait();
         const int thr = wt < BN && my_ch < cn ? __ldg(p.thr + my_ch) : 0;
         uint32_t w[WU];
 #pragma unroll
@@ -223,17 +241,16 @@ conv_tc_c3_kernel(const ConvProblem p, const C3Geom g, const __grid_constant__ C
     struct TileCursor {
         int b, ty, tx, db, dty, dtx;
     };
-    auto cursor = [&](int n0, int nstep) {
-        const unsigned per_img = (unsigned)(g.tiles_x * g.tiles_y), t = blockIdx.x + (unsigned)n0 * gridDim.x, st = (unsigned)nstep * gridDim.x;
+    auto cursor = [&](int n0, int log_step) {
+        const uint32_t t = blockIdx.x + (uint32_t)n0 * gridDim.x;
         TileCursor c;
-        c.b = (int)(t / per_img);
-        const unsigned rem = t - (unsigned)c.b * per_img;
-        c.ty = (int)(rem / (unsigned)g.tiles_x);
-        c.tx = (int)(rem - (unsigned)c.ty * (unsigned)g.tiles_x);
-        c.db = (int)(st / per_img);
-        const unsigned srem = st - (unsigned)c.db * per_img;
-        c.dty = (int)(srem / (unsigned)g.tiles_x);
-        c.dtx = (int)(srem - (unsigned)c.dty * (unsigned)g.tiles_x);
+        c.b = (int)exact_div(t, g.img_mul, g.img_shift);
+        const uint32_t rem = t - (uint32_t)c.b * (uint32_t)(g.tiles_x * g.tiles_y);
+        c.ty = (int)exact_div(rem, g.row_mul, g.row_shift);
+        c.tx = (int)rem - c.ty * g.tiles_x;
+        c.db = g.step[log_step].db;
+        c.dty = g.step[log_step].dty;
+        c.dtx = g.step[log_step].dtx;
         return c;
     };
     auto advance = [&](TileCursor &c) {
@@ -255,14 +272,14 @@ conv_tc_c3_kernel(const ConvProblem p, const C3Geom g, const __grid_constant__ C
         const uint32_t sf = tmem_u + (uint32_t)CB_COL, c_lo = (uint32_t)make_desc(cexp);
         const uint32_t hf = NH == 2 ? __shfl_sync(0xffffffffu, (uint32_t)warp, 0) : 0u;
         const uint32_t w_lo = b_lo + hf * HALF_DESC;
-        for (int n = NH == 2 ? 0 : warp; n < my_tiles; n += NH == 2 ? 1 : C::NISS) {
-            if (!pw_wait(a_full(n % NAF), (uint32_t)(n / NAF) & 1u, abort_flag, p.err, ERR_C3_ISSUER_TIMEOUT)) break;
-            // the epilogue has read the accumulator's previous tile
-            const int acc = NH == 2 ? (int)hf : n % NACC;
-            const int prev = NH == 2 ? n - 1 : n / NACC - 1;                 // completion of acc_free to wait for
-            if (prev >= 0 && !pw_wait(acc_free(acc), (uint32_t)prev & 1u, abort_flag, p.err, ERR_C3_ACC_TIMEOUT)) break;
-            tc_fence_after();
-            if (elect_one()) {
+        if (elect_one()) {
+            for (int n = NH == 2 ? 0 : warp; n < my_tiles; n += NH == 2 ? 1 : C::NISS) {
+                if (!issuer_wait(a_full(n % NAF), (uint32_t)(n / NAF) & 1u, abort_flag, p.err, ERR_C3_ISSUER_TIMEOUT)) break;
+                // the epilogue has read the accumulator's previous tile
+                const int acc = NH == 2 ? (int)hf : n % NACC;
+                const int prev = NH == 2 ? n - 1 : n / NACC - 1;                 // completion of acc_free to wait for
+                if (prev >= 0 && !issuer_wait(acc_free(acc), (uint32_t)prev & 1u, abort_flag, p.err, ERR_C3_ACC_TIMEOUT)) break;
+                tc_fence_after();
                 const uint32_t d_t = tmem_u + (uint32_t)(acc * AW);
                 tc_mma_const(d_t, tmem_u, c_lo + hf * HALF_DESC, desc_hi, idesc);
 #pragma unroll
@@ -277,16 +294,17 @@ conv_tc_c3_kernel(const ConvProblem p, const C3Geom g, const __grid_constant__ C
                 }
                 tc_commit(tile_done((n * NH + (int)hf) % NB));
             }
-            __syncwarp();
         }
+        __syncwarp();
     } else if (warp < C::FIRST_PRODUCER_WARP) {
         // ------------------------------------------------------------------ loader of a group: one halo tile per TMA copy
         const int grp = warp - C::FIRST_LOADER_WARP;
         int stage = 0;
         uint32_t phase = 1;                       // first pass through the ring: the stages are free
         int issued = 0;
-        TileCursor tc = cursor(grp, NGRP);
-        for (int n = grp; n < my_tiles; n += NGRP, advance(tc)) {
+        TileCursor tc = cursor(grp, 1);
+        pdl_wait();
+        for (int n = grp; n < my_tiles; n += NLD, advance(tc)) {
             if (!pw_wait<256>(load_empty(grp, stage), phase, abort_flag, p.err, ERR_C3_LOADER_TIMEOUT)) break;
             if (lane == 0) {
                 const uint32_t dst = ring + (uint32_t)(grp * RD + stage) * (uint32_t)g.stage_bytes;
@@ -314,7 +332,7 @@ conv_tc_c3_kernel(const ConvProblem p, const C3Geom g, const __grid_constant__ C
         const uint32_t t_lane = tmem_base + ((uint32_t)(quad * 32) << 16);
         const int owords = p.C_out >> 5;
         // NH == 1: the group takes alternate tiles; NH == 2: the group takes its half (64 channels) of every tile
-        TileCursor tc = cursor(NH == 2 ? 0 : grp, NH == 2 ? 1 : NGRP);
+        TileCursor tc = cursor(NH == 2 ? 0 : grp, NH == 2 ? 0 : 1);
         for (int n = NH == 2 ? 0 : grp; n < my_tiles; n += NH == 2 ? 1 : NGRP, advance(tc)) {
             const int acc = NH == 2 ? grp : n % NACC;
             const int d = NH == 2 ? 2 * n + grp : n;                              // the tile's (half's) "done" number
@@ -369,9 +387,9 @@ conv_tc_c3_kernel(const ConvProblem p, const C3Geom g, const __grid_constant__ C
         const uint32_t t_lane = tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)C::A_COL0;
         const uint32_t lane0 = lane == 0 ? 1u : 0u;
         for (int n = n0; n < my_tiles; n += step) {
-            const int lg = n & 1, stage = (n >> 1) % RD;
+            const int lg = n % NLD, stage = (n / NLD) % RD;
             uint32_t wds[TAPS];
-            if (!pw_wait<64>(load_full(lg, stage), (uint32_t)((n >> 1) / RD) & 1u, abort_flag, p.err, ERR_C3_PRODUCER_TIMEOUT)) break;
+            if (!pw_wait<64>(load_full(lg, stage), (uint32_t)(n / NLD / RD) & 1u, abort_flag, p.err, ERR_C3_PRODUCER_TIMEOUT)) break;
             const uint32_t src = ring + (uint32_t)(lg * RD + stage) * (uint32_t)g.stage_bytes + my_off;
 #pragma unroll
             for (int tap = 0; tap < TAPS; ++tap)
@@ -415,7 +433,7 @@ int launch_c3(const ConvProblem &p0, cudaStream_t stream)
     using C = C3Cfg<CW, BN>;
     ConvProblem p = p0;
     p.err = device_error_word();
-    const C3Geom g = c3_geometry(p);
+    C3Geom g = c3_geometry(p);
     const int smem = c3_smem_bytes<CW, BN>(g);
     if (smem > 227 * 1024 - 1024) return BCNN_ERR_UNSUPPORTED;
     const int sms = sm_count();
@@ -431,6 +449,7 @@ int launch_c3(const ConvProblem &p0, cudaStream_t stream)
                CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
         return BCNN_ERR_CUDA;
     const unsigned grid = (unsigned)(g.total_tiles < sms ? g.total_tiles : sms);
+    c3_walk(g, grid);
     void (*k)(const ConvProblem, const C3Geom, const CUtensorMap) = conv_tc_c3_kernel<CW, BN>;
     const int ask = smem < 120 * 1024 ? 120 * 1024 : smem;          // one CTA per SM (it takes all of tensor memory)
     if (!allow_smem((const void *)k, 227 * 1024 - 1024)) return BCNN_ERR_CUDA;
