@@ -448,82 +448,114 @@ gap_kernel(const uint16_t *x, float *pooled, int HW, int C, int GX)
     }
 }
 
-// logits = pooled * w^T + bias as a tiled fp32 product: FT_M images x FT_N outputs per CTA, K in chunks of FT_K through six
-// cp.async stages.  The eight warps take four of a chunk's K values each and every warp owns all of the tile, 8 x 4 outputs
-// per thread; the warps' sums are added through shared memory.  Small tiles, so that two or more CTAs share a multiprocessor: one
-// CTA's warps leave their barrier together and read while nothing multiplies.  The kernel below, which streams every weight
-// row from L2 once per four images, took 53 us for 256 x 1000 x 1024 (7.2 us of the fp32 pipe).
-constexpr int FT_M = 32, FT_N = 32, FT_K = 32, FT_STAGES = 6, FT_THREADS = 256, FT_PITCH = FT_K + 4;
-constexpr int FT_STAGE_FLOATS = (FT_M + FT_N) * FT_PITCH;
-__global__ void __launch_bounds__(FT_THREADS, 2)
-fc_tile_kernel(const float *pooled, const float *w, const float *bias, float *logits, int B, int C, int N)
+// logits = pooled * w^T + bias as a tiled fp32 product: FT_M images x FT_N outputs per CTA, K in chunks of FT_K through FT_STAGES
+// cp.async stages.  The eight warps take four of a chunk's K values each and every warp owns all of the tile, 8 x 8 outputs
+// per thread; the warps' sums are added through shared memory.  SPLIT CTAs (a cluster) share a tile's K where there are too few
+// tiles for the chip, and add their sums through each other's shared memory (64 x 100 x 2048: 12.0 -> 7.3 us, 256 x 10 x 2048 10.5 ->
+// 7.2).  What is left at 256 x 1000 x 1024 (20.7 -> 19.6 us, 7.1 of the fp32 pipe) did not move with 16 x 8 outputs per thread, pairs of
+// multiply-adds, chunks of 64 or a rolled loop.
+constexpr int FT_M = 32, FT_N = 64, FT_K = 32, FT_STAGES = 8, FT_THREADS = 256, FT_PITCH = FT_K + 4;
+constexpr int FT_PIECES = FT_K / 4, FT_ROWS = FT_THREADS / FT_PIECES, FT_KW = FT_K / 8;      // 16-byte pieces of a row, rows loaded at a time, a warp's K values
+constexpr int FT_STAGE_FLOATS = (FT_M + FT_N) * FT_PITCH, FT_SMEM = (FT_STAGES * FT_STAGE_FLOATS + FT_M * FT_N) * 4;
+static_assert(8 * FT_M * FT_N <= FT_STAGES * FT_STAGE_FLOATS, "the warps' sums fit the stages");
+template <int SPLIT>
+__global__ void __launch_bounds__(FT_THREADS, 1)
+fc_tile_kernel(const float *pooled, const float *w, const float *bias, float *logits, int B, int C, int N, int per)
 {
-    extern __shared__ __align__(16) float sm[];                 // [FT_STAGES][FT_STAGE_FLOATS]
+    extern __shared__ __align__(16) float sm[];                 // [FT_STAGES][FT_STAGE_FLOATS], [FT_M][FT_N] sums of this CTA
     const int tid = threadIdx.x, warp = tid >> 5, tm = (tid & 31) >> 3, tn = tid & 7;
-    const int b0 = blockIdx.y * FT_M, n0 = blockIdx.x * FT_N;
-    const int chunks = (C + FT_K - 1) / FT_K;
+    const int rank = (int)blockIdx.x % SPLIT;
+    const int b0 = blockIdx.y * FT_M, n0 = (int)blockIdx.x / SPLIT * FT_N;
+    // `per` chunks of K are this CTA's
+    const int k_end = min(C, (rank + 1) * per * FT_K), k_first = rank * per * FT_K;
+    const int chunks = max(0, (k_end - k_first + FT_K - 1) / FT_K);
     const uint32_t base = tc::smem_u32(sm);
+    const int lrow = tid / FT_PIECES, lk = 4 * (tid % FT_PIECES);
     pdl_wait();
     auto load = [&](int ch) {
         if (ch < chunks) {
-            const uint32_t dst = base + (uint32_t)((ch % FT_STAGES) * FT_STAGE_FLOATS * 4);
+            const int k = k_first + ch * FT_K + lk;
+            const uint32_t dst = base + (uint32_t)(((ch % FT_STAGES) * FT_STAGE_FLOATS + lrow * FT_PITCH + lk) * 4);
 #pragma unroll
-            for (int i = 0; i < (FT_M + FT_N) * (FT_K / 4) / FT_THREADS; ++i) {
-                const int e = tid + FT_THREADS * i, row = e / (FT_K / 4), k = ch * FT_K + 4 * (e % (FT_K / 4));
-                const int gr = row < FT_M ? b0 + row : n0 + row - FT_M;
-                const bool ok = k < C && gr < (row < FT_M ? B : N);
-                const float *src = (row < FT_M ? pooled : w) + (ok ? (long)gr * C + k : 0);
-                tc::cp_async16(dst + (uint32_t)((row * FT_PITCH + 4 * (e % (FT_K / 4))) * 4), src, ok);
+            for (int i = 0; i < (FT_M + FT_N) / FT_ROWS; ++i) {
+                const int row = lrow + FT_ROWS * i, gr = FT_ROWS * i < FT_M ? b0 + row : n0 + row - FT_M;
+                const bool ok = k < k_end && gr < (FT_ROWS * i < FT_M ? B : N);
+                tc::cp_async16(dst + (uint32_t)(FT_ROWS * i * FT_PITCH * 4), (FT_ROWS * i < FT_M ? pooled : w) + (ok ? (long)gr * C + k : 0), ok);
             }
         }
         tc::cp_async_commit();
     };
-    float acc[8][4];
+    float acc[8][8];
 #pragma unroll
     for (int i = 0; i < 8; ++i)
 #pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = 0.f;
-#pragma unroll
+        for (int j = 0; j < 8; ++j) acc[i][j] = 0.f;
+#pragma unroll 1
     for (int ch = 0; ch < FT_STAGES - 1; ++ch) load(ch);
+#pragma unroll 1
     for (int ch = 0; ch < chunks; ++ch) {
         tc::cp_async_wait<FT_STAGES - 2>();
         __syncthreads();                                        // chunk ch has landed; everybody is done reading chunk ch - 1
         load(ch + FT_STAGES - 1);
-        const float *pa = sm + (ch % FT_STAGES) * FT_STAGE_FLOATS + tm * FT_PITCH + 4 * warp;
-        const float *pb = sm + (ch % FT_STAGES) * FT_STAGE_FLOATS + (FT_M + tn) * FT_PITCH + 4 * warp;
-        float4 fa[8], fb[4];
+        const float *pa = sm + (ch % FT_STAGES) * FT_STAGE_FLOATS + tm * FT_PITCH + FT_KW * warp;
+        const float *pb = sm + (ch % FT_STAGES) * FT_STAGE_FLOATS + (FT_M + tn) * FT_PITCH + FT_KW * warp;
 #pragma unroll
-        for (int i = 0; i < 8; ++i) fa[i] = *reinterpret_cast<const float4 *>(pa + 4 * i * FT_PITCH);
+        for (int h = 0; h < FT_KW / 2; ++h) {
+            float2 fa[8];
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            fb[j] = *reinterpret_cast<const float4 *>(pb + 8 * j * FT_PITCH);
+            for (int i = 0; i < 8; ++i) fa[i] = *reinterpret_cast<const float2 *>(pa + 4 * i * FT_PITCH + 2 * h);
 #pragma unroll
-            for (int i = 0; i < 8; ++i) acc[i][j] = fmaf(fa[i].x, fb[j].x, acc[i][j]);
+            for (int j = 0; j < 8; ++j) {
+                const float2 fb = *reinterpret_cast<const float2 *>(pb + 8 * j * FT_PITCH + 2 * h);
 #pragma unroll
-            for (int i = 0; i < 8; ++i) acc[i][j] = fmaf(fa[i].y, fb[j].y, acc[i][j]);
+                for (int i = 0; i < 8; ++i) acc[i][j] = fmaf(fa[i].x, fb.x, acc[i][j]);
 #pragma unroll
-            for (int i = 0; i < 8; ++i) acc[i][j] = fmaf(fa[i].z, fb[j].z, acc[i][j]);
-#pragma unroll
-            for (int i = 0; i < 8; ++i) acc[i][j] = fmaf(fa[i].w, fb[j].w, acc[i][j]);
+                for (int i = 0; i < 8; ++i) acc[i][j] = fmaf(fa[i].y, fb.y, acc[i][j]);
+            }
         }
     }
     pdl_trigger();
     tc::cp_async_wait<0>();
-    // the warps' sums, eight rows of the tile at a time
-    float *red = sm;                                            // [8 warps][8 rows][FT_N]
+    __syncthreads();
+    // the warps' sums; the banks of rows tm, columns tn are 4 x 8 different ones
+    float *red = sm;                                            // [8 warps][FT_M][FT_N]
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        __syncthreads();
+    for (int i = 0; i < 8; ++i)
 #pragma unroll
-        for (int h = 0; h < 2; ++h)
-#pragma unroll
-            for (int j = 0; j < 4; ++j) red[warp * 256 + (4 * h + tm) * 32 + tn + 8 * j] = acc[2 * i + h][j];
-        __syncthreads();
-        const int b = b0 + 8 * i + (tid >> 5), n = n0 + (tid & 31);       // one output per thread
+        for (int j = 0; j < 8; ++j) red[(warp * FT_M + tm + 4 * i) * FT_N + ((tn + 8 * j) ^ (8 * tm))] = acc[i][j];
+    __syncthreads();
+    float *mine = sm + FT_STAGES * FT_STAGE_FLOATS;
+#pragma unroll 1
+    for (int q = 0; q < FT_M * FT_N / FT_THREADS; ++q) {
+        const int e = tid + FT_THREADS * q, row = e / FT_N, col = e % FT_N, at = row * FT_N + (col ^ (8 * (row & 3)));
         float v = 0.f;
 #pragma unroll
-        for (int q = 0; q < 8; ++q) v += red[q * 256 + tid];
-        if (b < B && n < N) logits[(long)b * N + n] = v + (bias ? __ldg(bias + n) : 0.f);
+        for (int wp = 0; wp < 8; ++wp) v += red[wp * FT_M * FT_N + at];
+        if (SPLIT > 1) {
+            mine[e] = v;
+        } else {
+            const int b = b0 + row, n = n0 + col;
+            if (b < B && n < N) logits[(long)b * N + n] = v + (bias ? __ldg(bias + n) : 0.f);
+        }
+    }
+    if (SPLIT > 1) {
+        asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+        for (int e = rank * (FT_M * FT_N / SPLIT) + tid; e < (rank + 1) * (FT_M * FT_N / SPLIT); e += FT_THREADS) {
+            const int b = b0 + e / FT_N, n = n0 + e % FT_N;
+            const uint32_t at = tc::smem_u32(mine + e);
+            float v = 0.f;
+#pragma unroll
+            for (uint32_t r = 0; r < (uint32_t)SPLIT; ++r) {
+                uint32_t there;
+                float t;
+                asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(there) : "r"(at), "r"(r));
+                asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(t) : "r"(there) : "memory");
+                v += t;
+            }
+            if (b < B && n < N) logits[(long)b * N + n] = v + (bias ? __ldg(bias + n) : 0.f);
+        }
+        // the others have read this CTA's sums
+        asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
     }
 }
 
@@ -626,22 +658,44 @@ int launch_avgpool(const uint16_t *x, uint16_t *y, int B, int H, int W, int C_in
 
 int launch_gap(const uint16_t *x, float *pooled, int B, int HW, int C, cudaStream_t stream)
 {
-    int GX = 32;                                     // channel groups of a block: the power of two that fits the channels
-    while (GX > 1 && GX / 2 >= C / 8) GX /= 2;
-    const long blocks = (long)B * ((C / 8 + GX - 1) / GX);
+    // channel groups of a block: the power of two that fits the channels, up to 32; fewer, and more pixels at a time, where that many
+    // leave multiprocessors idle (8 images of 10 x 10 x 192: 4.0 -> 2.4 us, 4 of 9 x 9 x 2048 3.8 -> 2.7, 2 of 14 x 14 x 1600 6.9 -> 2.9;
+    // 200 of 9 x 9 x 264 4.9 with 32, 5.2 with 8)
+    const int groups = C / 8;
+    int GX = 32;
+    while (GX > 1 && GX / 2 >= groups) GX /= 2;
+    while (GX > 8 && (long)B * ((groups + GX - 1) / GX) < sm_count()) GX /= 2;
+    const long blocks = (long)B * ((groups + GX - 1) / GX);
     if (blocks >= (1L << 31)) return BCNN_ERR_UNSUPPORTED;
     return launch(gap_kernel, (unsigned)blocks, 256, 0, stream, x, pooled, HW, C, GX);
 }
 
+template <int SPLIT>
+static int launch_fc_tile(const float *pooled, const float *w, const float *bias, float *logits, int B, int C, int N, int per, long tiles_n, long tiles_b, cudaStream_t stream)
+{
+    auto k = fc_tile_kernel<SPLIT>;
+    if (!allow_smem((const void *)k, FT_SMEM)) return BCNN_ERR_CUDA;
+    return launch<SPLIT>(k, dim3((unsigned)(tiles_n * SPLIT), (unsigned)tiles_b), FT_THREADS, FT_SMEM, stream, pooled, w, bias, logits, B, C, N, per);
+}
+
 int launch_fc(const float *pooled, const float *w, const float *bias, float *logits, int B, int C, int N, cudaStream_t stream)
 {
-    // the kernel below reads ceil(B / 4) N C weights from L2, about a million a microsecond; a wave of 32 x 32 tiles (two a
-    // multiprocessor) takes about C / 94 us: tiles from there on where the one is the longer (64 x 1000, not 16 x 1000)
+    // Tiles, with the K of each split over as many CTAs as make one wave, or the kernel below, which streams every weight row from L2
+    // once per four images and walks it in steps of 512.  Estimates in ns beyond a launch's own, fitted to fifteen heads (images x outputs x
+    // channels; tiles, streamed us): 32 x 1000 x 512 7.9, 9.1; 64 x 100 x 2048 7.3, 11.9; 16 x 1000 x 1024 9.7, 8.5; 25 x 130 x 728 4.5, 4.9
     const long tiles_n = ((long)N + FT_N - 1) / FT_N, tiles_b = ((long)B + FT_M - 1) / FT_M;
-    const long waves = (tiles_n * tiles_b + 2 * sm_count() - 1) / (2 * sm_count());
-    if ((long)((B + 3) / 4) * N > 10600 * waves && tiles_b < 65536)
-        return !allow_smem((const void *)fc_tile_kernel, FT_STAGES * FT_STAGE_FLOATS * 4) ? BCNN_ERR_CUDA :
-            launch(fc_tile_kernel, dim3((unsigned)tiles_n, (unsigned)tiles_b), FT_THREADS, FT_STAGES * FT_STAGE_FLOATS * 4, stream, pooled, w, bias, logits, B, C, N);
+    const int sms = sm_count(), chunks = (C + FT_K - 1) / FT_K;
+    int split = 1;
+    while (split < 8 && split * 2 <= chunks && tiles_n * tiles_b * split * 2 <= sms) split *= 2;
+    const int per = (chunks + split - 1) / split;
+    const long tiled = (tiles_n * tiles_b * split + sms - 1) / sms * (1900 + per * 480L) + (split > 1 ? 700 : 0) + (long)N * C * 3 / 1000;
+    const long streamed = (long)((B + 3) / 4) * N * C / 1000 + 3L * C;
+    if (tiled < streamed && tiles_b < 65536 && tiles_n < (1L << 27)) {
+        if (split == 8) return launch_fc_tile<8>(pooled, w, bias, logits, B, C, N, per, tiles_n, tiles_b, stream);
+        if (split == 4) return launch_fc_tile<4>(pooled, w, bias, logits, B, C, N, per, tiles_n, tiles_b, stream);
+        if (split == 2) return launch_fc_tile<2>(pooled, w, bias, logits, B, C, N, per, tiles_n, tiles_b, stream);
+        return launch_fc_tile<1>(pooled, w, bias, logits, B, C, N, per, tiles_n, tiles_b, stream);
+    }
     const int smem = FC_IMAGES * C * 4;
     if (smem > 200 * 1024) return BCNN_ERR_UNSUPPORTED;
     if (!allow_smem((const void *)fc_kernel, 200 * 1024)) return BCNN_ERR_CUDA;

@@ -267,3 +267,15 @@ def test_prepared_block_pairs(bk, oracle, M, N, K, fused):
 @pytest.mark.parametrize("K", [32, 256, 288, 512, 768, 992, 1056])
 def test_prepared_split_tiles(bk, oracle, K):
     test_prepared_widths(bk, oracle, 50000, 256, K, True)
+
+
+# the tiled product with its K over two, four and eight blocks (the last of them without a chunk), ragged in images, outputs and K
+@pytest.mark.parametrize("shape", [(64, 2048, 100), (97, 1156, 130), (130, 516, 700), (200, 2052, 1000), (300, 264, 65), (61, 1100, 513), (256, 2048, 10)])
+def test_fc_split(bk, oracle, shape):
+    test_fc_shapes(bk, oracle, shape)
+
+
+# pooling by 8 and 16 channel groups of few images
+@pytest.mark.parametrize("shape", [(8, 10, 10, 192), (1, 13, 11, 264), (20, 9, 9, 1600)])
+def test_gap_few_images(bk, oracle, shape):
+    test_gap_shapes(bk, oracle, shape)
