@@ -1,12 +1,13 @@
-// Streaming tcgen05 engine of the binary implicit GEMM: wide layers (C_out > 128), long K, and the plain GEMMs, on
-// weights that are expanded as they arrive.  Arithmetic: 4-bit operands (tc_common.cuh), fp32 accumulators that hold exact
-// integers,  sum a*g = accumulator + K - 2 popc(G):  one constant per output channel, nothing per row.
+// Streaming tcgen05 engine on weights that are expanded as they arrive: the module epilogue of layers that neither the module engine
+// (pointwise) nor the weight-stationary engine takes; the packed and int32 outputs of such weights run on conv_tc_pre.cu.
+// Arithmetic: 4-bit operands (tc_common.cuh), fp32 accumulators that hold exact integers,
+// sum a*g = accumulator + K - 2 popc(G):  one constant per output channel, nothing per row.
 //
 // Persistent, warp-specialised; each CTA walks a static list of 128 x BN tiles.
 //   warp 0          issuer: tcgen05.mma / commit only, waits on named barriers only (a memory
 //                   instruction after tensor-core instructions would stall it)
-//   warps 1-4       epilogue: tcgen05.ld, threshold + pack (or int32, or the module), hand the accumulator back
-//   G = 2 producer groups, each 4 activation warps + BN/32 weight warps, one thread per tile
+//   warps 1-4       epilogue: tcgen05.ld, the module's steps, hand the accumulator back
+//   G = 2 producer groups, each 4 activation warps + 4 weight warps, one thread per tile
 //                   row; the groups take the ring's stages alternately so that one group gathers
 //                   while the other expands.  Packed words are staged with cp.async (16 bytes per
 //                   row half and stage, zero-fill out of range).
@@ -14,8 +15,8 @@
 //                       MMA takes A from tensor memory, so shared memory carries only weights
 //                     weight rows     -> shared memory, 128-byte-swizzled K-major tiles
 //   last warp       control: does the issuer's mbarrier waits and releases it stage by stage
-// A ring stage is 256 bits of K.  Tensor memory (512 columns): BN = 256: one accumulator + 4 ring stages; BN = 128 and 64:
-// two accumulators + 7 ring stages, and the unit scales.  Column popcounts are taken from the words as they are
+// A ring stage is 256 bits of K.  Tensor memory (512 columns): two accumulators of BN = 128 columns, 7 ring stages and the unit
+// scales.  Column popcounts are taken from the words as they are
 // expanded; each group leaves its partial constants for a tile in shared-memory slots.
 // Every mbarrier wait is bounded and reports through the device error word.
 #include "tc_common.cuh"
@@ -30,15 +31,17 @@ constexpr int EPI_WARPS = 4;
 constexpr int G = 2;                      // producer groups
 constexpr int PF = 3;                     // packed-word stages in flight per producer thread
 constexpr int MAX_SMEM = 227 * 1024 - 512; // dynamic shared memory available beside the static part
+constexpr int MAX_KTAB = 1920;            // units of the gather's table that every variant has room for
 
 constexpr int ERR_PRODUCER_TIMEOUT = 101;
 constexpr int ERR_MMA_TIMEOUT = 102;
 constexpr int ERR_EPILOGUE_TIMEOUT = 103;
 
-template <int BN> struct Cfg {
-    static constexpr int NBUF = BN == 256 ? 1 : 2;                       // accumulator buffers
+constexpr int BN = 128;                   // output channels of a tile
+struct Cfg {
+    static constexpr int NBUF = 2;                                        // accumulator buffers
     static constexpr int A_COL0 = NBUF * BN;                              // first column of the activation ring
-    static constexpr int STAGES = BN == 256 ? 4 : 7;
+    static constexpr int STAGES = 7;
     static constexpr int GROUP_WARPS = 4 + BN / 32;
     static constexpr int GROUP_THREADS = 32 * GROUP_WARPS;
     static constexpr int PROD_THREADS = G * GROUP_THREADS;
@@ -56,22 +59,16 @@ template <int BN> struct Cfg {
     static_assert(STAGES >= G, "a producer group must not lap the ring (parity waits)");
 };
 
-template <int BN>
-__host__ __device__ inline int smem_bytes(int ktab_words, int mode = 1)
+int smem_bytes(int ktab_words)
 {
-    using C = Cfg<BN>;
-    // module epilogue (128-wide tiles only): + the identity staging ring; int32 output of the 128- and 64-wide tiles: + the store
-    // staging tiles (beside 256-wide tiles they do not fit)
-    return 1024 + C::STAGES * C::W_BYTES + C::BITS_BYTES + C::CONST_BYTES + C::TABLE_BYTES + ktab_words * 4 +
-           (mode == 2 ? ID_RING_BYTES + 16 : 0) + (mode == 0 && BN <= 128 ? EPI_WARPS * I32_TILE_BYTES + 16 : 0);
+    using C = Cfg;
+    return 1024 + C::STAGES * C::W_BYTES + C::BITS_BYTES + C::CONST_BYTES + C::TABLE_BYTES + ktab_words * 4 + ID_RING_BYTES + 16;
 }
 
-template <int BN, int MODE>
-__global__ void __launch_bounds__(Cfg<BN>::THREADS, 1)
+__global__ void __launch_bounds__(Cfg::THREADS, 1)
 conv_tc_i8_kernel(const ConvProblem p, const int ktab_words)
 {
-    using C = Cfg<BN>;
-    constexpr bool FUSED = MODE == 1, MODULE = MODE == 2;
+    using C = Cfg;
     constexpr int NBUF = C::NBUF;
     constexpr int STAGES = C::STAGES;
     constexpr int SLOTS = C::SLOTS;
@@ -95,7 +92,7 @@ conv_tc_i8_kernel(const ConvProblem p, const int ktab_words)
     const uint32_t consts = bits_ring + C::BITS_BYTES;                    // [SLOTS][G][BN] int32
     const uint32_t tables = consts + C::CONST_BYTES;                      // [EPI_WARPS][BN] fp32
     const uint32_t ktab_addr = tables + C::TABLE_BYTES;                   // unit table of the gather
-    const uint32_t idring = (ktab_addr + (uint32_t)ktab_words * 4u + 15u) & ~15u;   // module epilogue only: [ID_SLOTS][BM rows][80 B]
+    const uint32_t idring = (ktab_addr + (uint32_t)ktab_words * 4u + 15u) & ~15u;   // [ID_SLOTS][BM rows][80 B]
     const uint32_t bar0 = smem_u32(bars);
     auto full_bar = [&](int s) { return bar0 + 8u * s; };
     auto empty_bar = [&](int s) { return bar0 + 8u * (8 + s); };
@@ -190,11 +187,9 @@ conv_tc_i8_kernel(const ConvProblem p, const int ktab_words)
         bool alive = true;
         int buf = 0;
         uint32_t buf_phase = 0;
-        // module epilogue: the identity values of this thread's row are staged ID_AHEAD live chunks ahead (a chunk is
+        // the identity values of this thread's row are staged ID_AHEAD live chunks ahead (a chunk is
         // live when its first channel exists), in ring slot (live chunk number) % ID_SLOTS
         const uint32_t id_warp = idring + (uint32_t)(quad * 32) * ID_ROW_BYTES;   // slot 0, the warp's first row
-        // int32 output, 128-wide tiles: per-warp staging tile behind the (possibly unused) identity ring
-        const uint32_t i32_tile = idring + (uint32_t)quad * I32_TILE_BYTES;     // (shares the place of the module's ring)
         int pf_ti = 0, pf_ch = 0, pf_slot = 0, cur_slot = 0;
         auto prefetch_next = [&]() {
             bool queued = false;
@@ -211,8 +206,7 @@ conv_tc_i8_kernel(const ConvProblem p, const int ktab_words)
             if (!queued) cp_async_commit();
             if (++pf_slot == ID_SLOTS) pf_slot = 0;
         };
-        if (MODULE)
-            for (int a = 0; a < ID_AHEAD; ++a) prefetch_next();
+        for (int a = 0; a < ID_AHEAD; ++a) prefetch_next();
         for (int ti = 0; ti < my_tiles; ++ti) {
             const int tile = (int)blockIdx.x + ti * (int)gridDim.x;
             const int n_tile = tile / m_tiles, m_tile = tile - n_tile * m_tiles;
@@ -229,13 +223,13 @@ conv_tc_i8_kernel(const ConvProblem p, const int ktab_words)
             alive = __all_sync(0xffffffffu, alive && !*abort_flag);
             if (!alive) break;
             tc_fence_after();
-            // the groups' partial constants -> this warp's table of fp32 addends (int32 output: + INT_BIAS, see tc_common.cuh)
+            // the groups' partial constants -> this warp's table of fp32 addends
             const uint32_t table = tables + (uint32_t)(quad * BN * 4);
             for (int c = lane; c < BN; c += 32) {
                 int v0, v1 = 0;
                 asm volatile("ld.shared.b32 %0, [%1];" : "=r"(v0) : "r"(part0 + 4u * c) : "memory");
                 if (two) asm volatile("ld.shared.b32 %0, [%1];" : "=r"(v1) : "r"(part1 + 4u * c) : "memory");
-                asm volatile("st.shared.b32 [%0], %1;" ::"r"(table + 4u * c), "r"(table_entry<MODE>(v0 + v1)) : "memory");
+                asm volatile("st.shared.b32 [%0], %1;" ::"r"(table + 4u * c), "r"(table_entry<2>(v0 + v1)) : "memory");
             }
             __syncwarp();
             const uint32_t t_addr = tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)(buf * BN);
@@ -247,43 +241,19 @@ conv_tc_i8_kernel(const ConvProblem p, const int ktab_words)
                 if (n0 + col0 < p.C_out) {             // warp-uniform
                     uint32_t v[32];
                     tc_ld32(t_addr + (uint32_t)col0, v);
-                    if (FUSED) {
-                        words[ch] = threshold_word(v, table + 4u * col0);
-                    } else if (MODULE) {
-                        float dot[32];
+                    float dot[32];
 #pragma unroll
-                        for (int i4 = 0; i4 < 8; ++i4) {
-                            const uint4 cc = ld_shared_v4(table + 4u * (col0 + 4 * i4));
-                            dot[4 * i4 + 0] = __uint_as_float(fadd_bits(v[4 * i4 + 0], cc.x));
-                            dot[4 * i4 + 1] = __uint_as_float(fadd_bits(v[4 * i4 + 1], cc.y));
-                            dot[4 * i4 + 2] = __uint_as_float(fadd_bits(v[4 * i4 + 2], cc.z));
-                            dot[4 * i4 + 3] = __uint_as_float(fadd_bits(v[4 * i4 + 3], cc.w));
-                        }
-                        prefetch_next();
-                        cp_async_wait<ID_AHEAD>();                    // this chunk's copy has landed
-                        words[ch] = module_chunk(p, dot, id_warp + (uint32_t)cur_slot * (BM * ID_ROW_BYTES), (long)em - lane, n0 + col0, lane);
-                        if (++cur_slot == ID_SLOTS) cur_slot = 0;
-                    } else if constexpr (BN <= 128) {
-                        int o[32];
-                        biased_ints(v, table + 4u * col0, o);
-                        const long row0 = (long)em - lane;
-                        store_int32_block(static_cast<int32_t *>(p.out) + row0 * p.C_out + n0 + col0, p.C_out, o, i32_tile, row0, p.M, lane, p.C_out - n0 - col0);
-                    } else if (em < p.M) {
-                        int32_t *dst = static_cast<int32_t *>(p.out) + (long)em * p.C_out + n0 + col0;
-                        const bool vec = (p.C_out & 3) == 0 && (n0 + col0 + 32 <= p.C_out);
-                        int o[32];
-                        biased_ints(v, table + 4u * col0, o);
-#pragma unroll
-                        for (int i4 = 0; i4 < 8; ++i4) {
-                            if (vec) {
-                                *reinterpret_cast<int4 *>(dst + 4 * i4) = make_int4(o[4 * i4], o[4 * i4 + 1], o[4 * i4 + 2], o[4 * i4 + 3]);
-                            } else {
-#pragma unroll
-                                for (int i = 0; i < 4; ++i)
-                                    if (n0 + col0 + 4 * i4 + i < p.C_out) dst[4 * i4 + i] = o[4 * i4 + i];
-                            }
-                        }
+                    for (int i4 = 0; i4 < 8; ++i4) {
+                        const uint4 cc = ld_shared_v4(table + 4u * (col0 + 4 * i4));
+                        dot[4 * i4 + 0] = __uint_as_float(fadd_bits(v[4 * i4 + 0], cc.x));
+                        dot[4 * i4 + 1] = __uint_as_float(fadd_bits(v[4 * i4 + 1], cc.y));
+                        dot[4 * i4 + 2] = __uint_as_float(fadd_bits(v[4 * i4 + 2], cc.z));
+                        dot[4 * i4 + 3] = __uint_as_float(fadd_bits(v[4 * i4 + 3], cc.w));
                     }
+                    prefetch_next();
+                    cp_async_wait<ID_AHEAD>();                        // this chunk's copy has landed
+                    words[ch] = module_chunk(p, dot, id_warp + (uint32_t)cur_slot * (BM * ID_ROW_BYTES), (long)em - lane, n0 + col0, lane);
+                    if (++cur_slot == ID_SLOTS) cur_slot = 0;
                 }
             }
             // all reads of this accumulator buffer are complete: hand it back
@@ -291,14 +261,11 @@ conv_tc_i8_kernel(const ConvProblem p, const int ktab_words)
             __syncwarp();
             if (lane == 0) mbar_arrive(tempty_bar(buf));
             if (++buf == NBUF) { buf = 0; buf_phase ^= 1u; }
-            if ((FUSED || (MODULE && p.out != nullptr)) && em < p.M) {
+            if (p.out != nullptr && em < p.M) {
                 const int owords = p.C_out >> 5;
                 uint32_t *dst = static_cast<uint32_t *>(p.out) + (long)em * owords + (n0 >> 5);
-                if (BN >= 128 && (owords & 3) == 0 && n0 + BN <= p.C_out) {
-#pragma unroll
-                    for (int c4 = 0; c4 < BN / 128; ++c4)
-                        *reinterpret_cast<uint4 *>(dst + 4 * c4) =
-                            make_uint4(words[4 * c4], words[4 * c4 + 1], words[4 * c4 + 2], words[4 * c4 + 3]);
+                if ((owords & 3) == 0 && n0 + BN <= p.C_out) {
+                    *reinterpret_cast<uint4 *>(dst) = make_uint4(words[0], words[1], words[2], words[3]);
                 } else {
 #pragma unroll
                     for (int ch = 0; ch < BN / 32; ++ch)
@@ -306,7 +273,7 @@ conv_tc_i8_kernel(const ConvProblem p, const int ktab_words)
                 }
             }
         }
-        if (MODULE) cp_async_wait<0>();
+        cp_async_wait<0>();
     } else {
         // ------------------------------------------------------------------ producers
         const int pw = warp - C::FIRST_PRODUCER_WARP;            // producer warp index
@@ -433,17 +400,8 @@ conv_tc_i8_kernel(const ConvProblem p, const int ktab_words)
                 }
                 if (c_kt + G >= ktiles) {
                     // this group's last stage of the tile: leave its partial constants for the epilogue.
-                    //   K - 2 pg, packed output: - thr; the term that does not depend on the popcounts goes with the group
-                    // of the tile's first stage
-                    const bool first_group = ((c_ti * ktiles) & 1) == grp;
-                    int cst = -2 * pop;
-                    if (first_group) {
-                        const int tile = (int)blockIdx.x + c_ti * (int)gridDim.x;
-                        const int n = (tile / m_tiles) * BN + row;
-                        cst += p.K;
-                        // (a threshold beyond +-(K + 1) decides like that bound)
-                        if (FUSED) cst -= max(min(n < p.C_out ? __ldg(p.thr + n) : 0, p.K + 1), -p.K - 1);
-                    }
+                    //   K - 2 pg; the term that does not depend on the popcounts goes with the group of the tile's first stage
+                    const int cst = -2 * pop + (((c_ti * ktiles) & 1) == grp ? p.K : 0);
                     const uint32_t part = consts + (uint32_t)(((c_ti % SLOTS) * C::SLOT_INTS + grp * BN + row) * 4);
                     asm volatile("st.shared.b32 [%0], %1;" ::"r"(part), "r"(cst) : "memory");
                     pop = 0;
@@ -468,8 +426,7 @@ conv_tc_i8_kernel(const ConvProblem p, const int ktab_words)
 
 int ktab_words_for(const ConvProblem &p) { return (((p.kwords + 7) >> 3) * (8 / gather_width(p.cw)) + 3) & ~3; }
 
-template <int BN>
-int launch_bn(const ConvProblem &p0, cudaStream_t stream)
+int launch_module(const ConvProblem &p0, cudaStream_t stream)
 {
     ConvProblem p = p0;
     p.err = device_error_word();
@@ -480,15 +437,10 @@ int launch_bn(const ConvProblem &p0, cudaStream_t stream)
     if (total >= (1L << 31)) return BCNN_ERR_UNSUPPORTED;
     const unsigned grid = (unsigned)(total < sms ? total : sms);
     const int ktw = ktab_words_for(p);
-    const int smem = smem_bytes<BN>(ktw, p.mode);
+    const int smem = smem_bytes(ktw);
     if (smem > MAX_SMEM) return BCNN_ERR_UNSUPPORTED;
-    void (*k)(const ConvProblem, const int) = p.mode == 1 ? conv_tc_i8_kernel<BN, 1> : conv_tc_i8_kernel<BN, 0>;
-    if (p.mode == 2) {
-        if constexpr (BN == 128) k = conv_tc_i8_kernel<BN, 2>;      // (launch_conv_tc_i8 gives the module no other width)
-        else return BCNN_ERR_UNSUPPORTED;
-    }
-    if (!allow_smem((const void *)k, MAX_SMEM)) return BCNN_ERR_CUDA;
-    return launch(k, grid, Cfg<BN>::THREADS, smem, stream, p, ktw);
+    if (!allow_smem((const void *)conv_tc_i8_kernel, MAX_SMEM)) return BCNN_ERR_CUDA;
+    return launch(conv_tc_i8_kernel, grid, Cfg::THREADS, smem, stream, p, ktw);
 }
 
 }  // namespace
@@ -498,7 +450,7 @@ bool conv_tc_i8_supports(const ConvProblem &p)
     if (p.mode != 0 && (p.C_out % 32 != 0)) return false;
     if (p.kh * p.kw > 31) return false;                       // one validity bit per tap
     if ((long)p.B * p.H * p.W * p.cw >= (1L << 31)) return false;     // rows address the input by 32-bit word offsets
-    if (smem_bytes<256>(ktab_words_for(p)) > MAX_SMEM) return false;   // the K-word table of the gather must fit
+    if (ktab_words_for(p) > MAX_KTAB) return false;           // the K-word table of the gather must fit
     if ((long)p.kh * p.W * p.cw >= (1L << 27)) return false;  // a unit's word offset within the window
     return p.K <= (1 << 20);                                  // sums up to 4 K + 2 stay exact in fp32
 }
@@ -506,30 +458,7 @@ bool conv_tc_i8_supports(const ConvProblem &p)
 int launch_conv_tc_i8(const ConvProblem &p, cudaStream_t stream)
 {
     if (!conv_tc_i8_supports(p)) return BCNN_ERR_UNSUPPORTED;
-    // 256-wide tiles have a single accumulator buffer (tensor memory also holds the activation ring), so their epilogue is not
-    // overlapped: worth it only when the K loop is long.  The module epilogue's staging ring only fits beside the 128-wide tiles'
-    // weight ring.  int32 output up to K = 4608: the 128-wide tiles' staged stores, whole 128-byte rows, outweigh their extra
-    // expansion (4096 x 4096 x 4608: 63.5 against 75.2 us; at 9216 112 against 117, but 16384 x 16384 x 9216 1680 against 1550).
-    if (p.C_out > 128 && p.kwords >= 24 && p.mode != 2 && !(p.mode == 0 && p.kwords <= 144)) {
-        // ... unless the narrower tiles fill the last wave so much better that they win anyway.  A 128-wide tile costs 0.61 of a
-        // 256-wide one at K = 9216, 0.57 at 4608, 0.51 at 2304 and 0.41 at 768 (16384 x 16384: 1545 : 1284, 807 : 712, 424 : 423 and
-        // 181 : 225 us), so the line is right for the long K: 4096 x 4096 x 9216 102.7 (128) : 97.9, x 4608 56.0 : 56.2, 12544 x 512 x
-        // 4608 29.3 : 31.9; below K = 2304 it is a little early (4096 x 4096 x 768 16.0 : 19.7), and a single wave of 256-wide tiles
-        // would win from K = 4608 on (2048 x 2048: 19.8 : 18.2)
-        const int sms = sm_count();
-        const long m_tiles = ((long)p.M + BM - 1) / BM;
-        const long waves256 = (m_tiles * ((p.C_out + 255) / 256) + sms - 1) / sms;
-        const long waves128 = (m_tiles * ((p.C_out + 127) / 128) + sms - 1) / sms;
-        if (waves256 > 1 && 10 * waves256 <= 6 * waves128) return launch_bn<256>(p, stream);
-    }
-    // small problems: 64-wide tiles on twice the multiprocessors, with a shorter epilogue.  A tile column of one wave costs about
-    // 0.42 us per 256-bit stage at 128 and 0.33 at 64, the start 0.5 us less (1024 x 1024 x 4608: 12.3 -> 10.2 us, 20 x 64 x 960:
-    // 5.3 -> 4.7; many waves 0.37 and 0.29 per stage and 0.5 per tile: 16384 x 16384 x 9216 1545 and 2385)
-    const int sms = sm_count();
-    const long m_tiles = ((long)p.M + BM - 1) / BM, kt = (p.kwords + 7) / 8;
-    const long w64 = (m_tiles * ((p.C_out + 63) / 64) + sms - 1) / sms, w128 = (m_tiles * ((p.C_out + 127) / 128) + sms - 1) / sms;
-    if (p.mode != 2 && w64 * kt * 330 < w128 * kt * 420 + 500) return launch_bn<64>(p, stream);
-    return launch_bn<128>(p, stream);
+    return p.mode == 2 ? launch_module(p, stream) : launch_conv_tc_raw(p, stream);
 }
 
 }  // namespace bcnn

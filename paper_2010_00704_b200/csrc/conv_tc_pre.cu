@@ -1,4 +1,4 @@
-// Streaming tcgen05 engine on PREPARED weights: wide layers, long K, small layers, the plain GEMMs.
+// Streaming tcgen05 engine: wide layers, long K, small layers, the plain GEMMs, on PREPARED weights and (below) on raw ones.
 //
 // The weights of a layer never change between calls.  bcnn_prepare_weights expands their sign bits ONCE per layer into a
 // caller-owned buffer - signed 4-bit codes, K-major, rows padded to 128 and K to 256, then K - 2 popc(W_n) per row; half
@@ -22,6 +22,11 @@
 // 256-wide tiles have one accumulator buffer, handed over in halves of 128 columns: a tile's last two stages are multiplied half by
 // half, and so are the next one's first two, so that each half is read while the other is worked on; int32 outputs leave it as 16-bit
 // pairs (K <= 32767) and go to memory beside the next tile's MMAs.  Large products run on pairs of blocks (cta_group::2).
+//
+// RAW WEIGHTS (packed bits, new on each call): in each group as many weight warps as 32-row pieces of the CTA's weight tile expand them into
+// the ring, instead of the loader.  A pair of CTAs is what pays there, each expands half of the weight rows: 4096 x 4096 x 4608
+// packed 56 -> 37.8 us (0.48 us a stage against 0.28 of the pipe: the eight warps of a group have 250 issue slots of work per stage and its latencies),
+// 8192 x 8192 x 9216 329 -> 225, and the short set-up: 2070 x 64 x 288 4.3 -> 3.0, 34 x 3712 x 608 5.5 -> 3.5.
 //
 // What bounds it.  Long products: power.  A 256-bit stage of a 256-wide tile takes 553 cycles of a pair (512 of the pipe), at a clock
 // that falls from 1965 to 1600 .. 1750 MHz.  Narrow tiles: the issuer - a stage of four instructions with its wait and its commit costs it 300
@@ -49,16 +54,18 @@ constexpr int ERR_LOADER_TIMEOUT = 134;
 
 // BN: output channels of a tile; MODE: 0 int32, 1 packed output; G: activation producer groups of four warps; TEAMS: epilogue
 // teams of four warps, each with its share of a tile's columns
-template <int BN, int MODE, int G, int TEAMS, bool PAIR> struct Cfg {
+template <int BN, int MODE, int G, int TEAMS, bool PAIR, bool RAW = false> struct Cfg {
     static constexpr int EPI_WARPS = 4 * TEAMS;
     static constexpr int NBUF = BN == 256 ? 1 : (BN == 128 ? 2 : 4);     // accumulator buffers
     static constexpr int A_COL0 = NBUF * BN;                              // first column of the activation ring
     static constexpr int STAGES = !PAIR && BN == 256 ? (MODE == 0 ? 4 : 5) : 7;
-    static constexpr int PROD_THREADS = G * BM;
-    static constexpr int FIRST_PRODUCER_WARP = 1 + EPI_WARPS;
-    static constexpr int LOADER_WARP = FIRST_PRODUCER_WARP + 4 * G;
-    static constexpr int THREADS = 32 * (LOADER_WARP + 1);
     static constexpr int CTAS = PAIR ? 2 : 1, TILE_ROWS = CTAS * BM;      // CTAs of a tile, its rows
+    static constexpr int WW = RAW ? BN / CTAS / 32 : 0;                   // raw weights: a group's weight warps, a row per thread
+    static constexpr int GROUP_WARPS = 4 + WW;
+    static constexpr int PROD_THREADS = G * 32 * GROUP_WARPS;
+    static constexpr int FIRST_PRODUCER_WARP = 1 + EPI_WARPS;
+    static constexpr int LOADER_WARP = FIRST_PRODUCER_WARP + G * GROUP_WARPS;
+    static constexpr int THREADS = 32 * (LOADER_WARP + (RAW ? 0 : 1));
     static constexpr int EC = BN / TEAMS;                                 // columns of a team
     static constexpr bool SPLIT = BN == 256;                              // one accumulator, handed over in halves of 128 columns
     static constexpr int PIECES = SPLIT ? 2 : 1, PC = EC / PIECES;        // pieces of a team's columns, columns of a piece
@@ -67,6 +74,8 @@ template <int BN, int MODE, int G, int TEAMS, bool PAIR> struct Cfg {
     static constexpr int SF_COL = 512 - (int)SF_COLS;                     // unit scales
     static constexpr int BITS_BYTES = PF * PROD_THREADS * 32;
     static constexpr int TABLE_BYTES = EPI_WARPS * EC * 4;                // one column table per epilogue warp
+    static constexpr int SLOTS = STAGES + NBUF + 2;                       // raw weights: tiles whose rows' bit counts are kept
+    static constexpr int POP_BYTES = RAW ? SLOTS * G * BM * 4 : 0;
     static_assert(A_COL0 + STAGES * 32 <= SF_COL, "tensor memory budget");
     static_assert(STAGES >= G, "a producer group must not lap the ring (parity waits)");
 };
@@ -92,6 +101,11 @@ template <bool PAIR> __device__ __forceinline__ void mma_f4(uint32_t d_tmem, uin
     else
         tc_mma_f4_ts(d_tmem, a_tmem, b_lo, desc_hi, idesc, sf, accumulate);
 }
+__device__ __forceinline__ void add_row(uint32_t (&v)[32], float c)
+{
+#pragma unroll
+    for (int i = 0; i < 32; ++i) v[i] = __float_as_uint(__fadd_rn(__uint_as_float(v[i]), c));
+}
 __device__ __forceinline__ uint32_t in_even_cta(uint32_t addr)
 {
     uint32_t r;
@@ -111,15 +125,18 @@ __device__ __forceinline__ void cluster_barrier()
 template <typename C>
 __host__ __device__ constexpr int smem_bytes(int ktab_words, int mode)
 {
-    return 1024 + C::STAGES * C::W_BYTES + C::BITS_BYTES + C::TABLE_BYTES + ktab_words * 4 + 16 +
+    return 1024 + C::STAGES * C::W_BYTES + C::BITS_BYTES + C::TABLE_BYTES + C::POP_BYTES + ktab_words * 4 + 16 +
            (mode == 0 ? C::EPI_WARPS * I32_TILE_BYTES + 16 : 0);
 }
 
-template <int BN, int MODE, int G, int TEAMS, bool PAIR>
-__global__ void __launch_bounds__(Cfg<BN, MODE, G, TEAMS, PAIR>::THREADS, 1)
+// RAW: the weights are packed bits, expanded on the way; then the activations are the signed operand and the weights the unsigned one,
+//   sum a*g = accumulator + K - 2 popc(a):
+// a constant per row, which the warps that expand the row count, and none that the two CTAs of a pair would have to exchange.
+template <int BN, int MODE, int G, int TEAMS, bool PAIR, bool RAW>
+__global__ void __launch_bounds__(Cfg<BN, MODE, G, TEAMS, PAIR, RAW>::THREADS, 1)
 conv_tc_pre_kernel(const ConvProblem p, const int32_t *cst, const __grid_constant__ CUtensorMap wmap, const int ktab_words, const TileWalk walk)
 {
-    using C = Cfg<BN, MODE, G, TEAMS, PAIR>;
+    using C = Cfg<BN, MODE, G, TEAMS, PAIR, RAW>;
     constexpr int EPI_WARPS = C::EPI_WARPS, EC = C::EC;
     constexpr bool FUSED = MODE == 1;
     constexpr int NBUF = C::NBUF;
@@ -144,7 +161,8 @@ conv_tc_pre_kernel(const ConvProblem p, const int32_t *cst, const __grid_constan
     const uint32_t wring = (smem_u32(smem_raw) + 1023u) & ~1023u;         // [STAGES][BN rows][128 B], written by TMA
     const uint32_t bits_ring = wring + STAGES * C::W_BYTES;               // [PF][2][PROD_THREADS][16 B]
     const uint32_t tables = bits_ring + C::BITS_BYTES;                    // [EPI_WARPS][EC] column constants
-    const uint32_t ktab_addr = tables + C::TABLE_BYTES;                   // unit table of the gather
+    const uint32_t pops = tables + C::TABLE_BYTES;                        // [SLOTS][G][BM] bit counts of activation rows
+    const uint32_t ktab_addr = pops + C::POP_BYTES;                       // unit table of the gather
     const uint32_t i32_tiles = (ktab_addr + (uint32_t)ktab_words * 4u + 15u) & ~15u;   // int32 output: store staging tiles
     const uint32_t bar0 = smem_u32(bars);
     auto full_bar = [&](int s) { return bar0 + 8u * s; };
@@ -154,9 +172,9 @@ conv_tc_pre_kernel(const ConvProblem p, const int32_t *cst, const __grid_constan
     volatile int *abort_flag = &abort_flag_smem;
 
     if (tid < 24) {
-        // full: the four activation warps of the stage's group + the loader's arrive (+ its bytes); accumulator free: the epilogue warps
+        // full: the warps of the stage's group + the loader's arrive (+ its bytes); accumulator free: the epilogue warps
         // (of both CTAs, whose MMAs the even one issues)
-        mbar_init(bar0 + 8u * tid, tid < 8 ? 4 * C::CTAS + 1 : (tid >= 20 ? EPI_WARPS * C::CTAS : 1));
+        mbar_init(bar0 + 8u * tid, tid < 8 ? C::GROUP_WARPS * C::CTAS + (RAW ? 0 : 1) : (tid >= 20 ? EPI_WARPS * C::CTAS : 1));
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (tid == 0) abort_flag_smem = 0;
@@ -171,7 +189,7 @@ conv_tc_pre_kernel(const ConvProblem p, const int32_t *cst, const __grid_constan
     }
     const int gwidth = gather_width(p.cw);
     build_unit_table8(p, ktab_addr, ktiles * (8 / gwidth), gwidth, tid, C::THREADS);
-    if (tid == 32 * C::LOADER_WARP) asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&wmap)) : "memory");
+    if (!RAW && tid == 32 * C::LOADER_WARP) asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&wmap)) : "memory");
     tc_fence_before();
     if (PAIR) cluster_barrier();               // the other CTA's barriers exist
     else __syncthreads();
@@ -276,7 +294,7 @@ conv_tc_pre_kernel(const ConvProblem p, const int32_t *cst, const __grid_constan
             }
         }
         __syncwarp();
-    } else if (warp >= C::LOADER_WARP) {
+    } else if (!RAW && warp >= C::LOADER_WARP) {
         // ------------------------------------------------------------------ loader: weight tiles by TMA
         // item (tile, stage) -> ring slot item % STAGES.  A pair: this CTA's 64 rows of every 128 of the tile; the even CTA expects both
         // CTAs' bytes, and both complete on its barrier.
@@ -320,6 +338,23 @@ conv_tc_pre_kernel(const ConvProblem p, const int32_t *cst, const __grid_constan
         bool alive = true;
         int buf = 0, table_n = -1;
         uint32_t buf_phase = 0;
+        const int owords = p.C_out >> 5;
+        auto store_words = [&](const uint32_t (&words)[CH], int em, int n0) {
+            if (em < p.M) {
+                uint32_t *dst = static_cast<uint32_t *>(p.out) + (long)em * owords + (n0 >> 5);
+                if (PC >= 128 && (owords & 3) == 0 && n0 + PC <= p.C_out) {
+    #pragma unroll
+                    for (int c4 = 0; c4 + 3 < CH; c4 += 4) *reinterpret_cast<uint4 *>(dst + c4) = make_uint4(words[c4], words[c4 + 1], words[c4 + 2], words[c4 + 3]);
+                } else if ((owords & 1) == 0 && n0 + PC <= p.C_out) {
+    #pragma unroll
+                    for (int c2 = 0; c2 < CH; c2 += 2) *reinterpret_cast<uint2 *>(dst + c2) = make_uint2(words[c2], words[c2 + 1]);
+                } else {
+    #pragma unroll
+                    for (int ch = 0; ch < CH; ++ch)
+                        if (n0 + ch * 32 < p.C_out) dst[ch] = words[ch];
+                }
+            }
+        };
         TilePos at = walk.first(unit);
         const uint32_t tempty0 = PAIR ? in_even_cta(tempty_bar(0)) : tempty_bar(0);
         pdl_wait();
@@ -336,7 +371,7 @@ conv_tc_pre_kernel(const ConvProblem p, const int32_t *cst, const __grid_constan
                     const int n = n_base + (c / PC) * (BN / 2) + c % PC;
                     int v = 0;
                     if (n < p.C_out) {
-                        v = __ldg(cst + n);
+                        if (!RAW) v = __ldg(cst + n);
                         if (FUSED) v -= max(min(__ldg(p.thr + n), p.K + 1), -p.K - 1);       // beyond that bound the decision is constant
                     }
                     asm volatile("st.shared.b32 [%0], %1;" ::"r"(table + 4u * c), "r"(table_entry<MODE>(v)) : "memory");
@@ -344,7 +379,6 @@ conv_tc_pre_kernel(const ConvProblem p, const int32_t *cst, const __grid_constan
                 __syncwarp();
             }
             const long row0 = (long)em - lane;
-            const int owords = p.C_out >> 5;
             uint32_t packed[MODE == 0 ? PIECES : 1][CH][16];                    // int32 outputs of a 256-wide tile, two to a register
 #pragma unroll
             for (int h = 0; h < PIECES; ++h) {
@@ -361,7 +395,33 @@ conv_tc_pre_kernel(const ConvProblem p, const int32_t *cst, const __grid_constan
                     if (PAIR) arrive_in_cluster(tempty0 + 8u * b, lane == 0 ? 1u : 0u);
                     else if (lane == 0) mbar_arrive(tempty0 + 8u * b);
                 };
-                if (FUSED) {
+                float row_cst = 0.f;
+                if (RAW) {                                                      // the row's constant: the bit counts of the groups that had a stage of the tile
+                    const uint32_t at_pop = pops + (uint32_t)((ti % C::SLOTS) * G * BM + erow) * 4u;
+                    int n_bits = 0;
+#pragma unroll
+                    for (int g = 0; g < G; ++g) {
+                        const int first = (ti * ktiles) % G;
+                        if ((g >= first ? g - first : g - first + G) < ktiles) {
+                            int v;
+                            asm volatile("ld.shared.b32 %0, [%1];" : "=r"(v) : "r"(at_pop + (uint32_t)(g * BM) * 4u) : "memory");
+                            n_bits += v;
+                        }
+                    }
+                    row_cst = (float)(p.K - 2 * n_bits);
+                }
+                if (FUSED && RAW) {
+                    uint32_t words[CH];
+#pragma unroll
+                    for (int ch = 0; ch < CH; ++ch) {
+                        uint32_t v[32];
+                        tc_ld32(t_addr + 32u * ch, v);
+                        if (ch == CH - 1) hand_back();
+                        add_row(v, row_cst);
+                        words[ch] = threshold_word(v, table + 4u * (h * PC + 32 * ch));
+                    }
+                    store_words(words, em, n0);
+                } else if (FUSED) {
                     uint32_t words[CH];
 #pragma unroll
                     for (int c2 = 0; c2 < CH; c2 += 2) {                        // 64 columns in registers at a time
@@ -374,20 +434,7 @@ conv_tc_pre_kernel(const ConvProblem p, const int32_t *cst, const __grid_constan
                         if (c2 + 2 == CH) hand_back();
                         threshold_words(v, table + 4u * (h * PC + 32 * c2), words[c2], words[c2 + 1]);
                     }
-                    if (em < p.M) {
-                        uint32_t *dst = static_cast<uint32_t *>(p.out) + (long)em * owords + (n0 >> 5);
-                        if (PC >= 128 && (owords & 3) == 0 && n0 + PC <= p.C_out) {
-#pragma unroll
-                            for (int c4 = 0; c4 + 3 < CH; c4 += 4) *reinterpret_cast<uint4 *>(dst + c4) = make_uint4(words[c4], words[c4 + 1], words[c4 + 2], words[c4 + 3]);
-                        } else if ((owords & 1) == 0 && n0 + PC <= p.C_out) {
-#pragma unroll
-                            for (int c2 = 0; c2 < CH; c2 += 2) *reinterpret_cast<uint2 *>(dst + c2) = make_uint2(words[c2], words[c2 + 1]);
-                        } else {
-#pragma unroll
-                            for (int ch = 0; ch < CH; ++ch)
-                                if (n0 + ch * 32 < p.C_out) dst[ch] = words[ch];
-                        }
-                    }
+                    store_words(words, em, n0);
                 } else if (C::SPLIT && narrow) {
                     // out of the accumulator at once, 16 bits each; to memory below, beside the next tile's MMAs
 #pragma unroll
@@ -396,6 +443,7 @@ conv_tc_pre_kernel(const ConvProblem p, const int32_t *cst, const __grid_constan
                         int o[32];
                         tc_ld32(t_addr + 32u * ch, v);
                         if (ch == CH - 1) hand_back();
+                        if (RAW) add_row(v, row_cst);
                         biased_ints(v, table + 4u * (h * PC + 32 * ch), o);
 #pragma unroll
                         for (int i = 0; i < 16; ++i) packed[h][ch][i] = __byte_perm((uint32_t)o[2 * i], (uint32_t)o[2 * i + 1], 0x5410);
@@ -407,6 +455,7 @@ conv_tc_pre_kernel(const ConvProblem p, const int32_t *cst, const __grid_constan
                         int o[32];
                         if (n0 + 32 * ch < p.C_out) {          // warp-uniform
                             tc_ld32(t_addr + 32u * ch, v);
+                            if (RAW) add_row(v, row_cst);
                             biased_ints(v, table + 4u * (h * PC + 32 * ch), o);
                             store_int32_block(static_cast<int32_t *>(p.out) + row0 * p.C_out + n0 + 32 * ch, p.C_out, o, i32_tile, row0, p.M, lane, p.C_out - n0 - 32 * ch);
                         }
@@ -439,10 +488,16 @@ conv_tc_pre_kernel(const ConvProblem p, const int32_t *cst, const __grid_constan
         // ------------------------------------------------------------------ activation producers
         // Group g takes items g, g + G, ... of the CTA's flattened (tile, stage) list: a thread copies its row's 128
         // bits of K into its staging slot (PF items ahead), then expands the oldest staged item into the ring slot.
-        const int ptid = tid - 32 * C::FIRST_PRODUCER_WARP;
-        const int grp = ptid >> 7;
+        // (raw weights: the group's other warps do the same with a weight row per thread, into the ring in shared memory)
+        const int ptid = tid - 32 * C::FIRST_PRODUCER_WARP, pwarp = warp - C::FIRST_PRODUCER_WARP;
+        const int grp = pwarp / C::GROUP_WARPS, wi = pwarp - grp * C::GROUP_WARPS;
+        const bool is_w = RAW && wi >= 4;
         const int quad = warp & 3;                               // tensor-memory lane quadrant this warp may write
-        const int row = quad * 32 + lane;
+        const int row = is_w ? (wi - 4) * 32 + lane : quad * 32 + lane;      // of the weight tile, of the activation tile
+        // the weight row's output channel within the tile (a pair: this CTA's 64 of every 128)
+        const int wcol = PAIR ? (row >> 6) * 128 + rank * 64 + (row & 63) : row;
+        const uint32_t *wrow = p.w;
+        bool wok = false;
         constexpr uint32_t HALF_BYTES = C::PROD_THREADS * 16u, SLOT_BYTES = 2u * HALF_BYTES;
         const uint32_t bits0 = bits_ring + (uint32_t)ptid * 16u, bits_end = bits0 + PF * SLOT_BYTES;
         const uint32_t st_addr0 = tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)C::A_COL0;
@@ -457,9 +512,20 @@ conv_tc_pre_kernel(const ConvProblem p, const int32_t *cst, const __grid_constan
         rc.m = (uint32_t)(at.m * C::TILE_ROWS + rank * BM + row);
         rc.base = 0;
         rc.mask = 0;
-        row_locate(p, rc);
+        if (!is_w) row_locate(p, rc);
+        auto tile_ready = [&]() {            // what a tile's stages need of its row
+            if (is_w) {
+                const int n = at.n * BN + wcol;
+                wok = n < p.C_out;
+                wrow = p.w + (long)(wok ? n : 0) * p.kwords;
+            } else {
+                row_window(p, step, rc);
+            }
+        };
         auto next_tile = [&]() {             // the CTA's next tile
-            if (walk.next(at)) {
+            if (is_w) {
+                walk.next(at);
+            } else if (walk.next(at)) {
                 rc.m = (uint32_t)(at.m * C::TILE_ROWS + rank * BM + row);
                 row_locate(p, rc);
             } else {
@@ -467,12 +533,28 @@ conv_tc_pre_kernel(const ConvProblem p, const int32_t *cst, const __grid_constan
             }
         };
         while (l_kt >= ktiles) { l_kt -= ktiles; next_tile(); }
-        row_window(p, step, rc);
+        tile_ready();
         uint32_t l_dst = bits0;
         // the scales are in place before this group's first arrival, which every MMA waits for
-        if (grp == 0) write_unit_scales(tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)C::SF_COL);
+        if (grp == 0 && !is_w) write_unit_scales(tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)C::SF_COL);
         auto issue_load = [&]() {
-            if (gwidth == 4) gather_stage8<4>(p.x, rc, ktab_addr + (uint32_t)l_kt * 8u, l_dst, HALF_BYTES);
+            if (is_w) {
+                if ((p.kwords & 3) == 0) {
+#pragma unroll
+                    for (int q = 0; q < 2; ++q) {
+                        const int kword = l_kt * 8 + 4 * q;
+                        const bool ok = wok && kword < p.kwords;
+                        cp_async_zfill<16>(l_dst + q * HALF_BYTES, ok ? wrow + kword : p.w, ok ? 16u : 0u);
+                    }
+                } else {
+#pragma unroll
+                    for (int e = 0; e < 8; ++e) {
+                        const int kword = l_kt * 8 + e;
+                        const bool ok = wok && kword < p.kwords;
+                        cp_async_zfill<4>(l_dst + (e >> 2) * HALF_BYTES + 4u * (e & 3), ok ? wrow + kword : p.w, ok ? 4u : 0u);
+                    }
+                }
+            } else if (gwidth == 4) gather_stage8<4>(p.x, rc, ktab_addr + (uint32_t)l_kt * 8u, l_dst, HALF_BYTES);
             else if (gwidth == 2) gather_stage8<2>(p.x, rc, ktab_addr + (uint32_t)l_kt * 16u, l_dst, HALF_BYTES);
             else gather_stage8<1>(p.x, rc, ktab_addr + (uint32_t)l_kt * 32u, l_dst, HALF_BYTES);
             l_dst += SLOT_BYTES;
@@ -481,7 +563,7 @@ conv_tc_pre_kernel(const ConvProblem p, const int32_t *cst, const __grid_constan
             l_kt += G;
             if (l_kt >= ktiles) {
                 do { l_kt -= ktiles; next_tile(); } while (l_kt >= ktiles);
-                row_window(p, step, rc);
+                tile_ready();
             }
         };
         pdl_wait();
@@ -493,21 +575,54 @@ conv_tc_pre_kernel(const ConvProblem p, const int32_t *cst, const __grid_constan
         uint32_t c_src = bits0;
         int s = grp;                          // ring slot (G <= STAGES) and its parity
         uint32_t phase = 1;                   // first pass through the ring: slots are free
+        int c_kt = grp, c_ti = 0, n_bits = 0; // raw weights: the stage within its tile, the tile, the row's bits so far
 #pragma unroll 1
         for (int it = grp; it < total_items; it += G) {
             cp_async_wait<PF - 2>();
-            uint32_t v[32];
-            expand_stage8(ld_shared_v4(c_src), ld_shared_v4(c_src + HALF_BYTES), v);
+            const uint4 q0 = ld_shared_v4(c_src), q1 = ld_shared_v4(c_src + HALF_BYTES);
             c_src += SLOT_BYTES;
             if (c_src == bits_end) c_src = bits0;
-            if (!mbar_wait_warp(empty_bar(s), phase, abort_flag, p.err, ERR_PRODUCER_TIMEOUT)) break;
-            tc_fence_after();     // the MMAs that read this slot are complete (their commit released it)
-            tc_st32_nowait(st_addr0 + (uint32_t)s * 32u, v);
-            // the next copies are issued while the store completes
-            if (l_left > 0) issue_load();
-            cp_async_commit();
-            tc_wait_st();
-            tc_fence_before();
+            if (is_w) {
+                if (!mbar_wait_warp(empty_bar(s), phase, abort_flag, p.err, ERR_PRODUCER_TIMEOUT)) break;
+                const uint32_t row_addr = wring + (uint32_t)s * C::W_BYTES + (uint32_t)row * ROWB;
+                const uint32_t wds[8] = {q0.x, q0.y, q0.z, q0.w, q1.x, q1.y, q1.z, q1.w};
+#pragma unroll
+                for (int e = 0; e < 8; ++e) {
+                    uint32_t v[4];
+                    expand_a4(wds[e], v);
+                    st_shared_v4(row_addr + (uint32_t)((e ^ (row & 7)) << 4), v[0], v[1], v[2], v[3]);
+                }
+                if (l_left > 0) issue_load();
+                cp_async_commit();
+                fence_async_proxy();          // generic stores -> the MMAs
+            } else {
+                uint32_t v[32];
+                if (RAW) {
+                    const uint32_t wds[8] = {q0.x, q0.y, q0.z, q0.w, q1.x, q1.y, q1.z, q1.w};
+#pragma unroll
+                    for (int e = 0; e < 8; ++e) {
+                        const uint4 o = expand_w4(wds[e]);
+                        v[4 * e] = o.x; v[4 * e + 1] = o.y; v[4 * e + 2] = o.z; v[4 * e + 3] = o.w;
+                        n_bits += __popc(wds[e]);
+                    }
+                    while (c_kt >= ktiles) { c_kt -= ktiles; ++c_ti; }
+                    if (c_kt + G >= ktiles) { // this group's last stage of the tile
+                        asm volatile("st.shared.b32 [%0], %1;" ::"r"(pops + (uint32_t)(((c_ti % C::SLOTS) * G + grp) * BM + row) * 4u), "r"(n_bits) : "memory");
+                        n_bits = 0;
+                    }
+                    c_kt += G;
+                } else {
+                    expand_stage8(q0, q1, v);
+                }
+                if (!mbar_wait_warp(empty_bar(s), phase, abort_flag, p.err, ERR_PRODUCER_TIMEOUT)) break;
+                tc_fence_after();             // the MMAs that read this slot are complete (their commit released it)
+                tc_st32_nowait(st_addr0 + (uint32_t)s * 32u, v);
+                // the next copies are issued while the store completes
+                if (l_left > 0) issue_load();
+                cp_async_commit();
+                tc_wait_st();
+                tc_fence_before();
+            }
             __syncwarp();
             if (PAIR) arrive_in_cluster(full0 + 8u * s, lane0);
             else mbar_arrive_pred(full0 + 8u * s, lane0);
@@ -550,10 +665,11 @@ prepare_weights_kernel(const uint32_t *w, uint8_t *wexp, int32_t *cst, int N, in
 
 int ktab_words_for(const ConvProblem &p) { return ((p.kwords + 7) >> 3) * (8 / gather_width(p.cw)); }
 
-template <int BN, int MODE, int G, int TEAMS, bool PAIR>
+// pw.wexp == nullptr where the weights are raw (RAW)
+template <int BN, int MODE, int G, int TEAMS, bool PAIR, bool RAW = false>
 int launch_bn(const ConvProblem &p0, const PreparedWeights &pw, cudaStream_t stream)
 {
-    using C = Cfg<BN, MODE, G, TEAMS, PAIR>;
+    using C = Cfg<BN, MODE, G, TEAMS, PAIR, RAW>;
     ConvProblem p = p0;
     p.err = device_error_word();
     const long units = sm_count() / C::CTAS;
@@ -565,19 +681,21 @@ int launch_bn(const ConvProblem &p0, const PreparedWeights &pw, cudaStream_t str
     const int ktw = ktab_words_for(p);
     const int smem = smem_bytes<C>(ktw, MODE);
     if (smem > MAX_SMEM) return BCNN_ERR_UNSUPPORTED;
-    EncodeTiledFn encode = encode_tiled_fn();
-    if (!encode) return BCNN_ERR_CUDA;
-    CUtensorMap wmap;
-    // rows of k_pad / 2 bytes; for a pair as (128 rows, half of them, row)
-    const cuuint64_t pitch = (cuuint64_t)pw.k_pad / 2;
-    const cuuint64_t dims[4] = {pitch, PAIR ? 64u : (cuuint64_t)pw.n_pad, 2, (cuuint64_t)pw.n_pad / 128};
-    const cuuint64_t strides[3] = {pitch, 64 * pitch, 128 * pitch};
-    const cuuint32_t box[4] = {(cuuint32_t)ROWB, PAIR ? 64u : (cuuint32_t)BN, 1, PAIR ? (cuuint32_t)BN / 128 : 1};
-    const cuuint32_t estr[4] = {1, 1, 1, 1};
-    if (encode(&wmap, CU_TENSOR_MAP_DATA_TYPE_UINT8, PAIR ? 4 : 2, const_cast<uint8_t *>(pw.wexp), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-               CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
-        return BCNN_ERR_CUDA;
-    auto k = conv_tc_pre_kernel<BN, MODE, G, TEAMS, PAIR>;
+    CUtensorMap wmap = {};
+    if constexpr (!RAW) {
+        EncodeTiledFn encode = encode_tiled_fn();
+        if (!encode) return BCNN_ERR_CUDA;
+        // rows of k_pad / 2 bytes; for a pair as (128 rows, half of them, row)
+        const cuuint64_t pitch = (cuuint64_t)pw.k_pad / 2;
+        const cuuint64_t dims[4] = {pitch, PAIR ? 64u : (cuuint64_t)pw.n_pad, 2, (cuuint64_t)pw.n_pad / 128};
+        const cuuint64_t strides[3] = {pitch, 64 * pitch, 128 * pitch};
+        const cuuint32_t box[4] = {(cuuint32_t)ROWB, PAIR ? 64u : (cuuint32_t)BN, 1, PAIR ? (cuuint32_t)BN / 128 : 1};
+        const cuuint32_t estr[4] = {1, 1, 1, 1};
+        if (encode(&wmap, CU_TENSOR_MAP_DATA_TYPE_UINT8, PAIR ? 4 : 2, const_cast<uint8_t *>(pw.wexp), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                   CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+            return BCNN_ERR_CUDA;
+    }
+    auto k = conv_tc_pre_kernel<BN, MODE, G, TEAMS, PAIR, RAW>;
     if (!allow_smem((const void *)k, MAX_SMEM)) return BCNN_ERR_CUDA;
     return launch<C::CTAS>(k, (unsigned)(grid * C::CTAS), C::THREADS, smem, stream, p, pw.cst, wmap, ktw, make_tile_walk(p, C::TILE_ROWS, (int)m_tiles, (int)total, grid));
 }
@@ -711,6 +829,28 @@ int launch_conv_tc_pre(const ConvProblem &p, const void *prepared, cudaStream_t 
     // the two elsewhere (50176 x 256 x 2304, three waves: 13.2 -> 14.0)
     if (waves_of(256) >= 8 || (waves_of(256) >= 3 && p.K >= 4096)) return packed ? launch_bn<256, 1, 2, 2, true>(p, pw, stream) : launch_bn<256, 0, 2, 2, true>(p, pw, stream);
     return packed ? launch_bn<256, 1, 2, 2, false>(p, pw, stream) : launch_bn<256, 0, 2, 2, false>(p, pw, stream);
+}
+
+// ---- raw weights: the streaming engine's packed and int32 outputs
+int launch_conv_tc_raw(const ConvProblem &p, cudaStream_t stream)
+{
+    const PreparedWeights none = {};
+    const bool packed = p.mode == 1;
+    // As for prepared weights, fitted to 20 products (packed, us at 64 / 128 / a pair's 256 columns: 4096 x 4096 x 4608 85.6, 53.1, 37.8; 2048 x
+    // 2048 x 4608 26.3, 17.6, 13.6; 300 x 4000 x 9216 25.2, 17.0, 19.6; 1024 x 1024 x 4608 8.7, 10.3, 12.2; 20 x 64 x 960 3.5, 4.3, 5.5; int32: 4096 x 4096 x 4608 89.7, 56.7,
+    // 53.4; 12544 x 512 x 4608 39.9, 27.4, 29.6; 34 x 3712 x 608 4.2, 5.4, 10.5)
+    const int sms = sm_count(), ktw = ktab_words_for(p);
+    const long kt = (p.kwords + 7) / 8;
+    auto cost = [&](int rows, int bn, int units, long start, long wave, long stage) {
+        const long tiles = (((long)p.M + rows - 1) / rows) * ((p.C_out + bn - 1) / bn);
+        return start + (tiles + units - 1) / units * (wave + kt * stage);
+    };
+    const long c64 = cost(BM, 64, sms, 2500, packed ? 450 : 700, 300), c128 = cost(BM, 128, sms, 3000, packed ? 700 : 1200, 360);
+    const bool fits = smem_bytes<Cfg<256, 0, 2, 2, true, true>>(ktw, 0) <= MAX_SMEM;
+    const long c256 = fits ? cost(2 * BM, 256, sms / 2, packed ? 3900 : 6500, packed ? 900 : 4900, 415) : LONG_MAX;
+    if (c64 <= c128 && c64 <= c256) return packed ? launch_bn<64, 1, 2, 1, false, true>(p, none, stream) : launch_bn<64, 0, 2, 1, false, true>(p, none, stream);
+    if (c128 <= c256) return packed ? launch_bn<128, 1, 2, 1, false, true>(p, none, stream) : launch_bn<128, 0, 2, 1, false, true>(p, none, stream);
+    return packed ? launch_bn<256, 1, 2, 2, true, true>(p, none, stream) : launch_bn<256, 0, 2, 2, true, true>(p, none, stream);
 }
 
 }  // namespace bcnn

@@ -279,3 +279,25 @@ def test_fc_split(bk, oracle, shape):
 @pytest.mark.parametrize("shape", [(8, 10, 10, 192), (1, 13, 11, 264), (20, 9, 9, 1600)])
 def test_gap_few_images(bk, oracle, shape):
     test_gap_shapes(bk, oracle, shape)
+
+
+# raw weights on the streaming engine: pairs of blocks (both outputs, K of 32 to 4640 bits with every tail, columns of a half-empty tile, words by
+# 16, 8 and 4 bytes), 128- and 64-wide tiles of one stage and of several, more tiles in flight than a row keeps bit counts for
+@pytest.mark.parametrize("M,N,K,fused", [(4096, 4096, 1184, True), (9000, 1120, 4640, True), (2048, 1000, 4128, False), (20000, 512, 32, True), (20000, 512, 288, True),
+                                         (12544, 512, 2112, True), (8200, 4000, 4608, False), (300, 992, 9216, True), (20, 64, 960, True), (5000, 70, 4000, False), (40000, 192, 256, False)])
+def test_streamed_raw_weights(bk, oracle, M, N, K, fused):
+    rng = np.random.default_rng(M + N + K)
+    A, W = synth.random_bits(rng, (M, K // 8)), synth.random_bits(rng, (N, K // 8))
+    thr = synth.thresholds(rng, K, N) if fused else None
+    out = torch.empty(M * N // 8 if fused else M * N * 4, dtype=torch.uint8, device="cuda")
+    if fused:
+        bk.bcnn_gemm_b1_fused(dev(A), dev(W), dev(thr), out, M, N, K, engine=bk.ENGINES["tc_i8"])
+    else:
+        bk.bcnn_gemm_b1(dev(A), dev(W), out, M, N, K, engine=bk.ENGINES["tc_i8"])
+    torch.cuda.synchronize()
+    acc = synth.unpack_bits(A).astype(np.float32) @ synth.unpack_bits(W).astype(np.float32).T       # exact: |sums| < 2^24
+    if fused:
+        assert np.array_equal(synth.unpack_bits(out.cpu().numpy().reshape(M, N // 8)), np.where(acc >= thr, 1, -1))
+    else:
+        assert np.array_equal(out.cpu().numpy().view(np.int32).reshape(M, N), acc.astype(np.int32))
+    assert bk.bcnn_device_error() == 0
