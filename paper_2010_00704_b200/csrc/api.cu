@@ -78,13 +78,13 @@ int make_conv_problem(ConvProblem &p, const void *x, const void *w, const int32_
 //   * pointwise layers (1x1, stride 1, no padding; GEMMs) with K <= 128 and C_out <= 128, packed output: pointwise
 //     tcgen05 engine (memory-bound shapes: rows bulk-copied in chunks, one hand-over per chunk; 64 -> 64 at M = 3211264: 30 us,
 //     weight-stationary 69; 128 -> 128 at M = 802816: 20, wide pointwise 28);
-//   * the smallest calls with K <= 256: CUDA cores;
+//   * the smallest int32 calls with K <= 256: CUDA cores;
 //   * pointwise layers with K = 128, 256 or 512 and a multiple of 128 output channels, packed output: wide pointwise tcgen05
 //     engine (a row tile expanded once for all resident weight slices; 256 -> 256 at M = 802816: 35 us, weight-stationary 74;
 //     512 -> 512 at M = 50176: 16 and 23);
 //   * 3x3 layers (stride 1 or 2) on 32 or 64 input channels with C_out <= 128, packed output, whose 8 x 16 output tiles
 //     are at least three quarters full: halo-tile tcgen05 engine (input tiles by tiled TMA copies);
-//   * 1x1 layer with C_in = 32 and C_out <= 32, int32 output: one XOR + popcount per output on the CUDA cores;
+//   * 1x1 layer with C_in = 32 and C_out <= 32, int32 output: weight-stationary engine, few rows: warp-level int8 engine;
 //   * many rows of C_out <= 128 with K >= 64, or of wider layers with K <= 2304 (in 128-channel slices): weight-stationary
 //     tcgen05 engine;
 //   * other layers of C_out <= 64, those with K = 32 (strided, or int32 output): register-fed warp-level int8 engine;
@@ -94,36 +94,48 @@ int auto_engine(const ConvProblem &p)
 {
     // at every size, the smallest included: 2.4 .. 2.9 us up to M = 12544, against 3.0 .. 5.9 of the CUDA-core engine
     if (conv_tc_pw_supports(p)) return BCNN_ENGINE_TC_PW;
-    // another call whose work is half a wave of 64 x 64 tiles of up to 256 bits is over before a tensor-core engine has its
-    // weights expanded (1x1 256 -> 256 at M = 196: 3.3 against 4.2 us; 256 -> 128 at M = 3136: 5.3 against 4.2)
-    if (p.K <= 256 && ((p.M + 63L) / 64) * ((p.C_out + 63) / 64) <= sm_count() / 2) return BCNN_ENGINE_LOP3;
-    if (conv_tc_pn_supports(p)) return BCNN_ENGINE_TC_PN;
+    const bool packed = p.mode == 1, stream_raw = conv_tc_i8_supports(p);
+    const long tiles64 = ((p.M + 127L) / 128) * ((p.C_out + 63) / 64);
+    const int sms = sm_count();
+    // another int32 call whose work is half a wave of 64 x 64 tiles of up to 256 bits (29 x 391 x 64: 2.9 us, streaming 3.7; 60 x 960 x 256 3.1 and
+    // 3.3; packed 3.3 and 2.7)
+    if (!packed && p.K <= 256 && ((p.M + 63L) / 64) * ((p.C_out + 63) / 64) <= sms / 2) return BCNN_ENGINE_LOP3;
+    // the wide pointwise engine expands all its weights before the first product; where that is not spread over many row tiles the streaming
+    // engine is through sooner (tiles of 64 columns, us: 256 -> 256 8: 4.1 and 2.6; 256 -> 512 200: 4.6 and 4.0; 512 -> 1024 400: 5.7 and 6.3)
+    if (conv_tc_pn_supports(p) && !(stream_raw && 2 * tiles64 <= 3L * sms)) return BCNN_ENGINE_TC_PN;
     // full tiles: 64 -> 64 at 28 x 28, 256 images, row: 8.9 us, weight-stationary 12.9.  A tile that is part empty costs as much as
-    // a full one; the line is on the safe side (20 x 20, half full: 64 -> 128 11.9 and 11.7 us, but 64 -> 64 7.8 and 9.6)
+    // a full one; the line is on the safe side (20 x 20, half full: 64 -> 128 11.9 and 11.7 us, but 64 -> 64 7.8 and 9.6).  Small layers of 64
+    // input, or 96 and 128 output channels stream (64 -> 64, 74 tiles of 64 columns: 3.7 and 3.3 us, 196: 4.3 and 4.8; 64 -> 128 /2, 98: 4.8 and
+    // 3.8, 294: 5.9 and 5.3; 32 -> 128, 50: 3.5 and 3.2, 148: 3.8 and 4.2; 32 -> 64, 25: 2.9 and 3.1)
     if (conv_tc_c3_supports(p)) {
         const long covered = (long)((p.OH + 7) / 8 * 8) * ((p.OW + 15) / 16 * 16);
-        if (4L * p.OH * p.OW >= 3L * covered) return BCNN_ENGINE_TC_C3;
+        const long few = p.cw == 2 ? (p.C_out > 64 ? 2L * sms : sms) : (p.C_out > 64 ? sms / 2 : 0);
+        if (4L * p.OH * p.OW >= 3L * covered && !(stream_raw && tiles64 <= few)) return BCNN_ENGINE_TC_C3;
     }
-    // (int32 output only, row, against the weight-stationary engine: 45 and 25 us at M = 802816, 6.2 and 4.6 at 12544 - the packed
-    // output, for which this line was drawn, runs on the pointwise engine today)
-    if (conv_lop3_pointwise_k32(p)) return BCNN_ENGINE_LOP3;
+    // 1x1, 32 -> up to 32 channels, int32 (row, us: 44 on the CUDA cores, 31 warp-level int8, 25 weight-stationary at M = 802816; 6.3, 3.3 and 4.5 at
+    // 12544)
+    if (conv_lop3_pointwise_k32(p)) {
+        if (p.M >= 98304 && conv_tc_ws_supports(p)) return BCNN_ENGINE_TC_WS;
+        return conv_mma_s8_supports(p) ? BCNN_ENGINE_MMA_S8 : BCNN_ENGINE_LOP3;
+    }
     // Up to 128 output channels: the weight-stationary engine, unless its CTAs would expand all the weights for less than two
     // waves of 64-wide tiles of the streaming engine (3x3 128 -> 128: 7.6 against 5.0 us at M = 784, 8.3 against 7.0 at 12544;
     // 1x1 256 -> 64 at M = 81000: 7.5 against 12.1)
-    const long waves64 = (((p.M + 127L) / 128) * ((p.C_out + 63) / 64) + sm_count() - 1) / sm_count();
-    const bool small = conv_tc_i8_supports(p) && (waves64 <= 1 || (waves64 <= 2 && p.K >= 1024));
+    const long waves64 = (tiles64 + sms - 1) / sms;
+    const bool small = stream_raw && (waves64 <= 1 || (waves64 <= 2 && p.K >= 1024));
     if (p.C_out <= 128 && p.K >= 64) {
-        if (small) return BCNN_ENGINE_TC_I8;
+        // ... or few row tiles of more than 64 channels (3x3 64 -> 96 at M = 37125 8.4 against 6.9; at 50176 8.8 and 9.1)
+        if (small || (p.M <= 40000 && p.C_out > 64 && stream_raw)) return BCNN_ENGINE_TC_I8;
         if (conv_tc_ws_supports(p)) return BCNN_ENGINE_TC_WS;
     }
     // wider layers in slices of 128 output channels: ahead of the streaming engine while the weights fit and there are enough row
-    // tiles to share one slice's weights (4096 x 4096 x 2304 int32: 33.3 against 38.8 us, 3x3 256 -> 256 at M = 50176: 20.8
-    // against 27.3; 1024 x 1024 x 512: 7.9 against 5.5)
-    if (p.C_out > 128 && p.K <= 2304 && ((p.M + 127L) / 128) * ((p.C_out + 127) / 128) >= 2L * sm_count() && conv_tc_ws_supports(p)) return BCNN_ENGINE_TC_WS;
+    // tiles to share one slice's weights (packed, row: 1x1 320 -> 256 at M = 200704 22.9 us, streaming 25.1; 3x3 256 -> 256 at 50176 20.9 and 18.2,
+    // 4096 x 4096 x 768 14.9 and 14.6; int32: 3x3 256 -> 256 at 50176 26.0 and 31.4, 5000 x 1000 x 1152 14.4 and 12.8)
+    if (p.C_out > 128 && p.K <= 2304 && p.M >= (p.mode == 1 ? 98304 : 40000) && conv_tc_ws_supports(p)) return BCNN_ENGINE_TC_WS;
     // K = 32, row: 1x1/2 32 -> 64 packed at M = 50176 5.2 us, streaming 6.4; 32 -> 64 int32 at M = 200704 14.3 and 18.2.  At 128 channels
     // 8.3 and 7.5 packed, 23.9 and 32.3 int32
     if (p.C_out <= 64 && conv_mma_s8_supports(p)) return BCNN_ENGINE_MMA_S8;
-    if (conv_tc_i8_supports(p)) return BCNN_ENGINE_TC_I8;
+    if (stream_raw) return BCNN_ENGINE_TC_I8;
     if (conv_mma_b1_supports(p)) return BCNN_ENGINE_MMA_B1;
     return BCNN_ENGINE_LOP3;
 }
@@ -410,25 +422,32 @@ int bcnn_prepared_preferred(int B, int H, int W, int C_in, int C_out, int kh, in
     const int st = make_conv_problem(p, dummy, dummy, fused ? static_cast<const int32_t *>(dummy) : nullptr, dummy,
                                      B, H, W, C_in, C_out, kh, kw, stride, pad, fused != 0);
     if (st != BCNN_OK) return 0;
-    // Measured: streaming prepared weights wins where AUTO would expand them on every call - the streaming engine, short K of a
-    // wide packed product apart (16384 x 16384: K = 2304 240 against 434 us, K = 512 227 against 166), the weight-stationary one except on many rows of a short K, where its expansion is spread thin (56x56 64 -> 128 /2 at
-    // batch 256, M = 200704, K = 576: 16.1 against 18.2 us; K = 1152: 19.7 against 19.0; M = 784: 6.5 against 4.0; wide pointwise
-    // layers sit on the other side of the line, 1024 -> 1024 at M = 50176 39 against 49, at 12544 13.5 against 14.8).  The wide
-    // pointwise and halo-tile engines keep their layers, all but the smallest with many weights: they expand those at the start.
+    // Measured: streaming prepared weights wins where AUTO would expand them on every call - the streaming engine, a short K of a
+    // wide packed product apart (16384 x 16384 x 512 183 against 142 us), the weight-stationary one except on many rows of few channels whose
+    // pixels are an odd number of words (3x3 96 -> 32 at M = 300000 24.2 against 20.0; 96 -> 96 at 200704 18.9 and 18.7, int32 22.3 and 28.3; 192 -> 64
+    // 1x1 9.0 and 9.8).  The wide pointwise and halo-tile engines keep their layers, all but the smallest with many weights:
+    // they expand those at the start.
     if (!conv_tc_pre_supports(p)) return 0;
+    const long tiles64 = ((p.M + 127L) / 128) * ((p.C_out + 63) / 64), sms = sm_count();
     switch (auto_engine(p)) {
-    case BCNN_ENGINE_TC_PW: return 0;           // 2.4 .. 2.9 against 2.9 .. 4.1 us up to M = 12544
+    case BCNN_ENGINE_TC_PW: return p.K >= 96 && 3 * tiles64 <= sms ? 1 : 0;      // 128 -> 128, us: 2.6 and 2.4 at M = 784, 2.8 and 2.8 at 6272
     case BCNN_ENGINE_TC_C3:
-        if (p.C_out <= 64) return 0;
-        [[fallthrough]];
+        // us, halo tiles and prepared: 32 -> 64 3.15 and 2.75 at 74 tiles of 64 columns, 3.6 and 4.0 at 196; 64 -> 64 3.7 and 2.9 at 74, 5.3 and 6.8 at
+        // 588; 32 -> 128 4.4 and 4.4 at 392; 64 -> 96 7.7 and 7.3 at 1176, 12.7 and 13.7 at 3136; 64 -> 128 /2 7.3 and 6.0 at 784, 14.0 and 13.5 at 3136
+        if (p.C_out <= 32) return 0;
+        if (p.C_out <= 64) return tiles64 <= (p.cw == 2 ? sms * 4 / 3 : sms * 2 / 3) ? 1 : 0;
+        return p.cw == 1 ? 2 * tiles64 <= 5 * sms : (p.stride == 2 || tiles64 <= 8 * sms);
     case BCNN_ENGINE_TC_PN:
-        // 3x3 64 -> 128 /2: 5.0 against 4.0 us at M = 784, 15.4 against 18.2 at 200704; 1x1 512 -> 512: 5.0 against 3.7 us at M = 49,
-        // 6.5 against 8.3 at 12544
-        // (1x1 512 -> 128 at M = 12544: 5.2 against 4.4, 256 -> 256: 5.0 against 5.7)
-        return ((p.M + 127L) / 128) * ((p.C_out + 63) / 64) <= sm_count() * 3 / 2 ? 1 : 0;
-    case BCNN_ENGINE_TC_WS: return p.K >= 1024 || p.M < 98304 ? 1 : 0;
-    // packed, row: 1x1 160 -> 256 at M = 900 5.5 against 4.1 us, 96 -> 256 at M = 196 3.7 against 3.7 (in a graph 3.3 and 3.2); K = 64 at M = 100
-    // 3.5 and 3.6.  int32, in a graph, the other way round: 1x1 128 -> 128 at M = 784 3.3 against 3.8, 96 -> 64 at M = 196 3.1 against 3.5
+        // us, wide pointwise and prepared: 512 -> 1024 5.7 and 4.3 at 400 tiles of 64 columns, 7.9 and 11.6 at 1568; 256 -> 512 5.5 and 6.5 at 784; 256 -> 128
+        // 5.5 and 4.7 at 784, 8.8 and 10.0 at 3136
+        return tiles64 <= 3 * sms || (p.C_out <= 128 && tiles64 <= 6 * sms) ? 1 : 0;
+    case BCNN_ENGINE_TC_WS:
+        // the weight-stationary engine spreads its expansion over many rows: channels gathered word by word (M = 200704, us: 3x3 96 -> 64 packed 16.7
+        // and 17.3, 160 -> 64 21.3 and 23.0, 96 -> 32 int32 16.9 and 17.8) and windows beyond 3x3 (5x5 128 -> 64 at 522144 71.8 and 84.4, int32 77.6
+        // and 86.5; 3x3 15.9 and 16.1, int32 20.0 and 17.6; 1x1 256 -> 64 9.8 and 8.6).  At M = 50176 5x5 14.9 and 11.3
+        return p.M >= 98304 && ((p.C_out <= (fused ? 64 : 32) && (p.cw & 1)) || (p.C_out <= 64 && p.kh * p.kw > 9)) ? 0 : 1;
+    case BCNN_ENGINE_TC_I8: return fused && p.K <= 512 && p.C_out > 1024 && (long)p.M * p.C_out >= 1L << 27 ? 0 : 1;
+    // int32: 1x1 128 -> 128 at M = 784 3.2 and 3.0 us, 96 -> 64 at M = 196 3.1 and 2.9; 29 x 391 x 64 2.9 and 3.2
     case BCNN_ENGINE_LOP3: return p.K <= 64 ? 0 : 1;
     default: return 1;
     }
