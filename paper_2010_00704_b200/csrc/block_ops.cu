@@ -451,17 +451,19 @@ gap_kernel(const uint16_t *x, float *pooled, int HW, int C, int GX)
 // logits = pooled * w^T + bias as a tiled fp32 product: FT_M images x FT_N outputs per CTA, K in chunks of FT_K through FT_STAGES
 // cp.async stages.  The eight warps take four of a chunk's K values each and every warp owns all of the tile, 8 x 8 outputs
 // per thread; the warps' sums are added through shared memory.  SPLIT CTAs (a cluster) share a tile's K where there are too few
-// tiles for the chip, and add their sums through each other's shared memory (64 x 100 x 2048: 12.0 -> 7.3 us, 256 x 10 x 2048 10.5 ->
-// 7.2).  What is left at 256 x 1000 x 1024 (20.7 -> 19.6 us, 7.1 of the fp32 pipe) did not move with 16 x 8 outputs per thread, pairs of
+// tiles for the chip, and add their sums through each other's shared memory (64 x 100 x 2048: 12.0 -> 5.4 us, 256 x 10 x 2048 10.5 ->
+// 5.2).  32 outputs, two CTAs a multiprocessor, where tiles are few; with 64 a weight goes twice as far (256 x 1000 x 256: 7.4 and 6.7 us).  What is left at 256 x 1000 x 1024 (20.7 -> 19.6 us, 7.1 of the fp32 pipe) did not move with 16 x 8 outputs per thread, pairs of
 // multiply-adds, chunks of 64 or a rolled loop.
-constexpr int FT_M = 32, FT_N = 64, FT_K = 32, FT_STAGES = 8, FT_THREADS = 256, FT_PITCH = FT_K + 4;
+constexpr int FT_M = 32, FT_K = 32, FT_STAGES = 8, FT_THREADS = 256, FT_PITCH = FT_K + 4;
 constexpr int FT_PIECES = FT_K / 4, FT_ROWS = FT_THREADS / FT_PIECES, FT_KW = FT_K / 8;      // 16-byte pieces of a row, rows loaded at a time, a warp's K values
-constexpr int FT_STAGE_FLOATS = (FT_M + FT_N) * FT_PITCH, FT_SMEM = (FT_STAGES * FT_STAGE_FLOATS + FT_M * FT_N) * 4;
-static_assert(8 * FT_M * FT_N <= FT_STAGES * FT_STAGE_FLOATS, "the warps' sums fit the stages");
-template <int SPLIT>
+
+constexpr int ft_smem(int n) { return (FT_STAGES * (FT_M + n) * FT_PITCH + FT_M * n) * 4; }
+template <int SPLIT, int FT_N>
 __global__ void __launch_bounds__(FT_THREADS, 1)
 fc_tile_kernel(const float *pooled, const float *w, const float *bias, float *logits, int B, int C, int N, int per)
 {
+    constexpr int FT_STAGE_FLOATS = (FT_M + FT_N) * FT_PITCH, NJ = FT_N / 8;
+    static_assert(8 * FT_M * FT_N <= FT_STAGES * FT_STAGE_FLOATS, "the warps' sums fit the stages");
     extern __shared__ __align__(16) float sm[];                 // [FT_STAGES][FT_STAGE_FLOATS], [FT_M][FT_N] sums of this CTA
     const int tid = threadIdx.x, warp = tid >> 5, tm = (tid & 31) >> 3, tn = tid & 7;
     const int rank = (int)blockIdx.x % SPLIT;
@@ -485,11 +487,11 @@ fc_tile_kernel(const float *pooled, const float *w, const float *bias, float *lo
         }
         tc::cp_async_commit();
     };
-    float acc[8][8];
+    float acc[8][NJ];
 #pragma unroll
     for (int i = 0; i < 8; ++i)
 #pragma unroll
-        for (int j = 0; j < 8; ++j) acc[i][j] = 0.f;
+        for (int j = 0; j < NJ; ++j) acc[i][j] = 0.f;
 #pragma unroll 1
     for (int ch = 0; ch < FT_STAGES - 1; ++ch) load(ch);
 #pragma unroll 1
@@ -505,7 +507,7 @@ fc_tile_kernel(const float *pooled, const float *w, const float *bias, float *lo
 #pragma unroll
             for (int i = 0; i < 8; ++i) fa[i] = *reinterpret_cast<const float2 *>(pa + 4 * i * FT_PITCH + 2 * h);
 #pragma unroll
-            for (int j = 0; j < 8; ++j) {
+            for (int j = 0; j < NJ; ++j) {
                 const float2 fb = *reinterpret_cast<const float2 *>(pb + 8 * j * FT_PITCH + 2 * h);
 #pragma unroll
                 for (int i = 0; i < 8; ++i) acc[i][j] = fmaf(fa[i].x, fb.x, acc[i][j]);
@@ -522,7 +524,7 @@ fc_tile_kernel(const float *pooled, const float *w, const float *bias, float *lo
 #pragma unroll
     for (int i = 0; i < 8; ++i)
 #pragma unroll
-        for (int j = 0; j < 8; ++j) red[(warp * FT_M + tm + 4 * i) * FT_N + ((tn + 8 * j) ^ (8 * tm))] = acc[i][j];
+        for (int j = 0; j < NJ; ++j) red[(warp * FT_M + tm + 4 * i) * FT_N + ((tn + 8 * j) ^ (8 * tm))] = acc[i][j];
     __syncthreads();
     float *mine = sm + FT_STAGES * FT_STAGE_FLOATS;
 #pragma unroll 1
@@ -670,33 +672,52 @@ int launch_gap(const uint16_t *x, float *pooled, int B, int HW, int C, cudaStrea
     return launch(gap_kernel, (unsigned)blocks, 256, 0, stream, x, pooled, HW, C, GX);
 }
 
-template <int SPLIT>
+template <int SPLIT, int FT_N>
 static int launch_fc_tile(const float *pooled, const float *w, const float *bias, float *logits, int B, int C, int N, int per, long tiles_n, long tiles_b, cudaStream_t stream)
 {
-    auto k = fc_tile_kernel<SPLIT>;
-    if (!allow_smem((const void *)k, FT_SMEM)) return BCNN_ERR_CUDA;
-    return launch<SPLIT>(k, dim3((unsigned)(tiles_n * SPLIT), (unsigned)tiles_b), FT_THREADS, FT_SMEM, stream, pooled, w, bias, logits, B, C, N, per);
+    auto k = fc_tile_kernel<SPLIT, FT_N>;
+    if (!allow_smem((const void *)k, ft_smem(FT_N))) return BCNN_ERR_CUDA;
+    return launch<SPLIT>(k, dim3((unsigned)(tiles_n * SPLIT), (unsigned)tiles_b), FT_THREADS, ft_smem(FT_N), stream, pooled, w, bias, logits, B, C, N, per);
+}
+
+template <int FT_N>
+static int launch_fc_tiles(const float *pooled, const float *w, const float *bias, float *logits, int B, int C, int N, int split, int per, long tiles_n, long tiles_b, cudaStream_t stream)
+{
+    switch (split) {
+    case 8: return launch_fc_tile<8, FT_N>(pooled, w, bias, logits, B, C, N, per, tiles_n, tiles_b, stream);
+    case 4: return launch_fc_tile<4, FT_N>(pooled, w, bias, logits, B, C, N, per, tiles_n, tiles_b, stream);
+    case 2: return launch_fc_tile<2, FT_N>(pooled, w, bias, logits, B, C, N, per, tiles_n, tiles_b, stream);
+    default: return launch_fc_tile<1, FT_N>(pooled, w, bias, logits, B, C, N, per, tiles_n, tiles_b, stream);
+    }
 }
 
 int launch_fc(const float *pooled, const float *w, const float *bias, float *logits, int B, int C, int N, cudaStream_t stream)
 {
-    // Tiles, with the K of each split over as many CTAs as make one wave, or the kernel below, which streams every weight row from L2
-    // once per four images and walks it in steps of 512.  Estimates in ns beyond a launch's own, fitted to fifteen heads (images x outputs x
-    // channels; tiles, streamed us): 32 x 1000 x 512 7.9, 9.1; 64 x 100 x 2048 7.3, 11.9; 16 x 1000 x 1024 9.7, 8.5; 25 x 130 x 728 4.5, 4.9
-    const long tiles_n = ((long)N + FT_N - 1) / FT_N, tiles_b = ((long)B + FT_M - 1) / FT_M;
+    // Tiles of 64 or 32 outputs, with the K of each split over as many CTAs as make one wave, or the kernel below, which walks K in steps of 512 for
+    // four images at a time.  Estimates in ns, fitted to sixteen heads (images x channels x outputs; 32 and 64 wide, streamed us):
+    // 64 x 128 x 1000 3.5, 4.0, 6.2; 32 x 512 x 1000 5.3, 7.8 (clusters of eight do not all fit at once), 9.1; 256 x 256 x 1000 7.4, 6.7, 21.2;
+    // 64 x 2048 x 100 5.4, 7.2, 11.9; 250 x 32 x 2000 5.0, 5.4, 29.3; 19 x 344 x 202 3.3, 4.0, 3.1; 100 x 96 x 50 3.3, 4.1, 2.1
     const int sms = sm_count(), chunks = (C + FT_K - 1) / FT_K;
-    int split = 1;
-    while (split < 8 && split * 2 <= chunks && tiles_n * tiles_b * split * 2 <= sms) split *= 2;
-    const int per = (chunks + split - 1) / split;
-    const long tiled = (tiles_n * tiles_b * split + sms - 1) / sms * (1900 + per * 480L) + (split > 1 ? 700 : 0) + (long)N * C * 3 / 1000;
-    const long streamed = (long)((B + 3) / 4) * N * C / 1000 + 3L * C;
-    if (tiled < streamed && tiles_b < 65536 && tiles_n < (1L << 27)) {
-        if (split == 8) return launch_fc_tile<8>(pooled, w, bias, logits, B, C, N, per, tiles_n, tiles_b, stream);
-        if (split == 4) return launch_fc_tile<4>(pooled, w, bias, logits, B, C, N, per, tiles_n, tiles_b, stream);
-        if (split == 2) return launch_fc_tile<2>(pooled, w, bias, logits, B, C, N, per, tiles_n, tiles_b, stream);
-        return launch_fc_tile<1>(pooled, w, bias, logits, B, C, N, per, tiles_n, tiles_b, stream);
-    }
+    const long tiles_b = ((long)B + FT_M - 1) / FT_M;
+    auto split_of = [&](long tiles) {
+        int split = 1;
+        while (split < 8 && split * 2 <= chunks && tiles * split * 2 <= sms) split *= 2;
+        return split;
+    };
     const int smem = FC_IMAGES * C * 4;
+    const long n32 = ((long)N + 31) / 32, n64 = ((long)N + 63) / 64;
+    // rows of more channels than the kernel below can hold (12800) are taken in large products only
+    if (smem > 200 * 1024 && (long)((B + 3) / 4) * N <= 10600 * ((n32 * tiles_b + 2 * sms - 1) / (2 * sms))) return BCNN_ERR_UNSUPPORTED;
+    const int split32 = split_of(n32 * tiles_b), split64 = split_of(n64 * tiles_b);
+    const int per32 = (chunks + split32 - 1) / split32, per64 = (chunks + split64 - 1) / split64;
+    // a narrow tile has a multiprocessor to itself in the last wave, or shares it with another
+    const long ctas = n32 * tiles_b * split32, shared = ctas / (2 * sms), rest = ctas % (2 * sms);
+    const long narrow = 1000 + (split32 > 1 ? 300 : 0) + (shared + (rest > sms)) * (1700 + per32 * 550L) + (rest > 0 && rest <= sms ? 1400 + per32 * 430L : 0);
+    const long wide = 1000 + (split64 == 8 ? 1500 : split64 > 1 ? 900 : 0) + (n64 * tiles_b * split64 + sms - 1) / sms * (1500 + per64 * 550L);
+    const long streamed = 1700 + 3L * C + (long)((B + 3) / 4) * N * (200 + 7 * C / 10) / 1000;
+    if ((narrow < wide ? narrow : wide) < streamed && tiles_b < 65536 && n32 < (1L << 27))
+        return narrow <= wide ? launch_fc_tiles<32>(pooled, w, bias, logits, B, C, N, split32, per32, n32, tiles_b, stream)
+                              : launch_fc_tiles<64>(pooled, w, bias, logits, B, C, N, split64, per64, n64, tiles_b, stream);
     if (smem > 200 * 1024) return BCNN_ERR_UNSUPPORTED;
     if (!allow_smem((const void *)fc_kernel, 200 * 1024)) return BCNN_ERR_CUDA;
     const int images = (B + FC_IMAGES - 1) / FC_IMAGES;

@@ -269,8 +269,10 @@ def test_prepared_split_tiles(bk, oracle, K):
     test_prepared_widths(bk, oracle, 50000, 256, K, True)
 
 
-# the tiled product with its K over two, four and eight blocks (the last of them without a chunk), ragged in images, outputs and K
-@pytest.mark.parametrize("shape", [(64, 2048, 100), (97, 1156, 130), (130, 516, 700), (200, 2052, 1000), (300, 264, 65), (61, 1100, 513), (256, 2048, 10)])
+# the tiled product with its K over two, four and eight blocks (the last of them without a chunk), ragged in images, outputs and K; tiles of 32 and 64
+# outputs in one wave and in several
+@pytest.mark.parametrize("shape", [(64, 2048, 100), (97, 1156, 130), (130, 516, 700), (200, 2052, 1000), (300, 264, 65), (61, 1100, 513), (256, 2048, 10),
+                                   (64, 160, 500), (250, 36, 2001), (201, 264, 2999), (129, 516, 1001), (255, 128, 4001)])
 def test_fc_split(bk, oracle, shape):
     test_fc_shapes(bk, oracle, shape)
 
