@@ -524,7 +524,7 @@ def run_gpu(args):
     regime = regime_of(clocks_k)
     alt_key = "4x_bf16_sustained" if regime == "sustained" else "4x_bf16_burst"
     engines = [chain.engine_name(i) for i in range(nl)]   # "stem": the first layer runs inside the stem kernel (slot 0 of per_ms)
-    kernel_of = {"tc_i8": "conv_tc_i8_kernel (tcgen05 kind::mxf4)", "mma_s8": "conv_mma_s8_kernel (mma.sync u8)",
+    kernel_of = {"tc_i8": "conv_tc_pre_kernel on raw weights (tcgen05 kind::mxf4)", "mma_s8": "conv_mma_s8_kernel (mma.sync u8)",
                  "mma_b1": "conv_mma_b1_kernel (mma.sync b1)",
                  "tc_ws": "conv_tc_ws_kernel (tcgen05 kind::mxf4, weights resident in shared memory)",
                  "tc_pw": "conv_tc_pw_kernel (tcgen05 kind::mxf4, pointwise layers, bulk-copied rows)",
@@ -560,8 +560,8 @@ def run_gpu(args):
     top = next(i for i in dom_idx if per_ms[i + 1] >= 0.93 * slowest)
     lt = layers[top]
     top_tops = lt.ops(B) / (per_ms[top + 1] / 1e3) / 1e12
-    src_of = {"tc_ws": ["conv_tc_ws.cu", "tc_common.cuh"], "tc_i8": ["conv_tc_i8.cu", "tc_common.cuh"],
-              "tc_pw": ["conv_tc_pw.cu", "tc_slot.cuh", "tc_common.cuh"], "tc_pre": ["conv_tc_pre.cu", "tc_common.cuh"],
+    src_of = {"tc_ws": ["conv_tc_ws.cu", "tc_common.cuh"], "tc_i8": ["conv_tc_pre.cu", "tc_slot.cuh", "tc_common.cuh"],
+              "tc_pw": ["conv_tc_pw.cu", "tc_slot.cuh", "tc_common.cuh"], "tc_pre": ["conv_tc_pre.cu", "tc_slot.cuh", "tc_common.cuh"],
               "tc_c3": ["conv_tc_c3.cu", "tc_slot.cuh", "tc_common.cuh"],
               "tc_pn": ["conv_tc_pn.cu", "tc_slot.cuh", "tc_common.cuh"]}
     roofline = {

@@ -88,8 +88,8 @@ int make_conv_problem(ConvProblem &p, const void *x, const void *w, const int32_
 //   * many rows of C_out <= 128 with K >= 64, or of wider layers with K <= 2304 (in 128-channel slices): weight-stationary
 //     tcgen05 engine;
 //   * other layers of C_out <= 64, those with K = 32 (strided, or int32 output): register-fed warp-level int8 engine;
-//   * everything else: streaming tcgen05 engine;
-//   * the single-bit mma.sync engine is nowhere the fastest (4096 x 4096 x 9216: 835 us, streaming 106) and serves as a fallback.
+//   * everything else, and the smaller layers of the engines above at their lines: streaming tcgen05 engine;
+//   * the single-bit mma.sync engine is nowhere the fastest (4096 x 4096 x 9216: 835 us; streaming takes 38 for half of that K) and serves as a fallback.
 int auto_engine(const ConvProblem &p)
 {
     // at every size, the smallest included: 2.4 .. 2.9 us up to M = 12544, against 3.0 .. 5.9 of the CUDA-core engine
@@ -507,9 +507,9 @@ const char *bcnn_status_string(int status)
     case BCNN_ERR_WORKSPACE: return "workspace too small (the layer's prepared weights exceed the library's static scratch array)";
     case BCNN_ERR_TIMEOUT: return "a bounded device-side wait gave up";
     // device error word: which bounded wait gave up
-    case 101: return "device wait timed out: streaming tcgen05 engine, producer waiting for a free ring slot";
-    case 102: return "device wait timed out: streaming tcgen05 engine, control warp waiting for a full slot or a free accumulator";
-    case 103: return "device wait timed out: streaming tcgen05 engine, epilogue waiting for an accumulator";
+    case 101: return "device wait timed out: streaming tcgen05 engine (module epilogue), producer waiting for a free ring slot";
+    case 102: return "device wait timed out: streaming tcgen05 engine (module epilogue), control warp waiting for a full slot or a free accumulator";
+    case 103: return "device wait timed out: streaming tcgen05 engine (module epilogue), epilogue waiting for an accumulator";
     case 111: return "device wait timed out: weight-stationary tcgen05 engine, producer waiting for a free ring slot";
     case 112: return "device wait timed out: weight-stationary tcgen05 engine, control warp waiting for a full slot or a free accumulator";
     case 113: return "device wait timed out: weight-stationary tcgen05 engine, epilogue waiting for an accumulator";
@@ -517,10 +517,10 @@ const char *bcnn_status_string(int status)
     case 122: return "device wait timed out: pointwise tcgen05 engine, producer waiting for a chunk's rows";
     case 123: return "device wait timed out: pointwise tcgen05 engine, issuer waiting for a slot's expanded rows";
     case 124: return "device wait timed out: pointwise tcgen05 engine, epilogue waiting for a chunk's accumulators";
-    case 131: return "device wait timed out: prepared-weights tcgen05 engine, producer waiting for a free ring slot";
-    case 132: return "device wait timed out: prepared-weights tcgen05 engine, control warp waiting for a full slot or a free accumulator";
-    case 133: return "device wait timed out: prepared-weights tcgen05 engine, epilogue waiting for an accumulator";
-    case 134: return "device wait timed out: prepared-weights tcgen05 engine, loader waiting for a free ring slot";
+    case 131: return "device wait timed out: streaming tcgen05 engine, producer waiting for a free ring slot";
+    case 132: return "device wait timed out: streaming tcgen05 engine, control warp waiting for a full slot or a free accumulator";
+    case 133: return "device wait timed out: streaming tcgen05 engine, epilogue waiting for an accumulator";
+    case 134: return "device wait timed out: streaming tcgen05 engine, loader waiting for a free ring slot";
     case 125: return "device wait timed out: pointwise tcgen05 engine, producer waiting for a slot's previous MMAs";
     case 126: return "device wait timed out: pointwise tcgen05 engine, issuer waiting for a slot's accumulators";
     case 141: return "device wait timed out: 3x3 halo-tile tcgen05 engine, loader waiting for a free ring stage";

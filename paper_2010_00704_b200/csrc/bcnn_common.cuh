@@ -94,7 +94,7 @@ bool conv_tc_c3_supports(const ConvProblem &p);
 int launch_conv_tc_pn(const ConvProblem &p, cudaStream_t stream);
 bool conv_tc_pn_supports(const ConvProblem &p);
 int launch_conv_tc_i8(const ConvProblem &p, cudaStream_t stream);
-int launch_conv_tc_raw(const ConvProblem &p, cudaStream_t stream);      // packed output, what conv_tc_i8_supports vouches for
+int launch_conv_tc_raw(const ConvProblem &p, cudaStream_t stream);      // packed and int32 outputs, what conv_tc_i8_supports vouches for
 // weights expanded once per layer by launch_prepare_weights (conv_tc_pre.cu): [n_pad][k_pad] signed 4-bit codes, then
 // K - 2 popc(W_n) per row
 struct PreparedWeights {

@@ -303,3 +303,26 @@ def test_streamed_raw_weights(bk, oracle, M, N, K, fused):
     else:
         assert np.array_equal(out.cpu().numpy().view(np.int32).reshape(M, N), acc.astype(np.int32))
     assert bk.bcnn_device_error() == 0
+
+
+# ... and convolutions with padding, strides and odd pixel words, against the CUDA-core engine
+@pytest.mark.parametrize("fused", [True, False])
+@pytest.mark.parametrize("shape", [(16, 28, 29, 160, 512, 3, 1, 1), (40, 27, 27, 96, 1024, 3, 2, 1), (8, 30, 30, 256, 992, 5, 1, 2), (30, 15, 14, 512, 640, 1, 2, 0), (2, 9, 9, 64, 96, 3, 1, 1)])
+def test_streamed_raw_convolutions(bk, oracle, shape, fused):
+    B, H, W, C_in, C_out, k, stride, pad = shape
+    rng = np.random.default_rng(C_in + C_out)
+    K = k * k * C_in
+    x, w = dev(synth.random_bits(rng, (B, H, W, C_in // 8))), dev(synth.random_bits(rng, (C_out, K // 8)))
+    thr = dev(synth.thresholds(rng, K, C_out))
+    OH, OW = bk.out_hw(H, W, k, k, stride, pad)
+    res = []
+    for e in ("tc_i8", "lop3"):
+        out = torch.full((B * OH * OW * C_out // 8 * (1 if fused else 32),), 0x5a, dtype=torch.uint8, device="cuda")
+        if fused:
+            bk.bcnn_conv2d_b1_fused(x, w, thr, out, B, H, W, C_in, C_out, k, k, stride, pad, engine=bk.ENGINES[e])
+        else:
+            bk.bcnn_conv2d_b1(x, w, out, B, H, W, C_in, C_out, k, k, stride, pad, engine=bk.ENGINES[e])
+        torch.cuda.synchronize()
+        res.append(out)
+    assert torch.equal(res[0], res[1])
+    assert bk.bcnn_device_error() == 0
