@@ -821,6 +821,9 @@ int launch_conv_tc_pre(const ConvProblem &p, const void *prepared, cudaStream_t 
         c128 = cost(128, 3000, 700, wide_gather ? 225 : 340);
         if (fits256) c256 = cost(256, 3500, 4300, wide_gather ? 270 : 340);
     }
+    // One stage, int32: the stores are the time, and over several waves 64-wide tiles take longer than the estimate has it (us at 64 and
+    // 128: 5301 x 860 x 32, four waves, 9.0 and 7.5; two waves 5.1 and 5.0; one wave, 1000 x 500 x 256, 3.8 and 4.8, 3000 x 300 x 160 4.2 and 4.8)
+    if (!packed && kt == 1 && waves_of(64) > 2) return launch_bn<128, 0, 3, 2, false>(p, pw, stream);
     if (c64 < c128 && c64 <= c256) return packed ? launch_bn<64, 1, 2, 1, false>(p, pw, stream) : launch_bn<64, 0, 2, 1, false>(p, pw, stream);
     if (c128 <= c256) return packed ? launch_bn<128, 1, 2, 1, false>(p, pw, stream) : launch_bn<128, 0, 3, 2, false>(p, pw, stream);
     // Two multiprocessors on a tile of 256 x 256: half the weight bytes from L2 and into shared memory.  That pays where the tensor pipe is

@@ -269,6 +269,12 @@ def test_prepared_split_tiles(bk, oracle, K):
     test_prepared_widths(bk, oracle, 50000, 256, K, True)
 
 
+# int32 products of one stage: two waves of 64-wide tiles at most, and more of them on 128-wide tiles, ragged in rows and columns
+@pytest.mark.parametrize("M,N,K", [(1000, 500, 256), (5301, 860, 32), (6001, 801, 160), (20000, 300, 256)])
+def test_prepared_one_stage_int32(bk, oracle, M, N, K):
+    test_prepared_widths(bk, oracle, M, N, K, False)
+
+
 # the tiled product with its K over two, four and eight blocks (the last of them without a chunk), ragged in images, outputs and K; tiles of 32 and 64
 # outputs in one wave and in several
 @pytest.mark.parametrize("shape", [(64, 2048, 100), (97, 1156, 130), (130, 516, 700), (200, 2052, 1000), (300, 264, 65), (61, 1100, 513), (256, 2048, 10),
