@@ -8,6 +8,7 @@
 #include "tc_common.cuh"
 #include "tensor_map.cuh"
 #include <cuda_fp16.h>
+#include <climits>
 
 namespace bcnn {
 
@@ -714,7 +715,7 @@ int launch_fc(const float *pooled, const float *w, const float *bias, float *log
     const long ctas = n32 * tiles_b * split32, shared = ctas / (2 * sms), rest = ctas % (2 * sms);
     const long narrow = 1000 + (split32 > 1 ? 300 : 0) + (shared + (rest > sms)) * (1700 + per32 * 550L) + (rest > 0 && rest <= sms ? 1400 + per32 * 430L : 0);
     const long wide = 1000 + (split64 == 8 ? 1500 : split64 > 1 ? 900 : 0) + (n64 * tiles_b * split64 + sms - 1) / sms * (1500 + per64 * 550L);
-    const long streamed = 1700 + 3L * C + (long)((B + 3) / 4) * N * (200 + 7 * C / 10) / 1000;
+    const long streamed = smem > 200 * 1024 ? LONG_MAX : 1700 + 3L * C + (long)((B + 3) / 4) * N * (200 + 7 * C / 10) / 1000;      // (rows it cannot hold)
     if ((narrow < wide ? narrow : wide) < streamed && tiles_b < 65536 && n32 < (1L << 27))
         return narrow <= wide ? launch_fc_tiles<32>(pooled, w, bias, logits, B, C, N, split32, per32, n32, tiles_b, stream)
                               : launch_fc_tiles<64>(pooled, w, bias, logits, B, C, N, split64, per64, n64, tiles_b, stream);

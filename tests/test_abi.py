@@ -97,6 +97,23 @@ def test_prepared_call_takes_what_it_is_preferred_for():
     assert len(seen) == 4                                                                    # both answers, both outputs
 
 
+def test_fc_takes_long_rows_in_large_products():
+    # Rows of more than 12800 channels do not fit the kernel that streams the weights: large products of them run in tiles whatever the estimates
+    # say, small ones are refused.  Made-up addresses, so only where no device could run the call.
+    import pytest
+    import torch
+    from paper_2010_00704_b200 import build, binding
+    if torch.cuda.is_available():
+        pytest.skip("made-up addresses: only without a device")
+    build.build()
+    lib, a = binding.load(), ctypes.c_void_p(4096)
+    for B, C, N in ((5, 12808, 5350), (8, 17104, 9000), (16, 32768, 5350), (6, 72108, 8770), (300, 20000, 1000)):
+        assert lib.bcnn_fc(a, a, a, a, B, C, N, None) == binding.ERR_CUDA, (B, C, N)
+    for B, C, N in ((1, 12804, 100), (4, 40000, 10000)):
+        assert lib.bcnn_fc(a, a, a, a, B, C, N, None) == binding.ERR_UNSUPPORTED, (B, C, N)
+    assert lib.bcnn_fc(a, a, a, a, 1, 12800, 100, None) == binding.ERR_CUDA
+
+
 def test_every_wait_code_has_a_name():
     # the codes as the kernels define them, each in one place
     from paper_2010_00704_b200 import build, binding

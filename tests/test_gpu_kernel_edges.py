@@ -283,6 +283,12 @@ def test_fc_split(bk, oracle, shape):
     test_fc_shapes(bk, oracle, shape)
 
 
+# rows longer than the streaming kernel holds, where its estimate would be the smaller
+@pytest.mark.parametrize("shape", [(5, 12808, 5350), (16, 13004, 2700)])
+def test_fc_long_rows(bk, oracle, shape):
+    test_fc_shapes(bk, oracle, shape)
+
+
 # pooling by 8 and 16 channel groups of few images
 @pytest.mark.parametrize("shape", [(8, 10, 10, 192), (1, 13, 11, 264), (20, 9, 9, 1600)])
 def test_gap_few_images(bk, oracle, shape):
