@@ -449,21 +449,26 @@ gap_kernel(const uint16_t *x, float *pooled, int HW, int C, int GX)
     }
 }
 
-// logits = pooled * w^T + bias as a tiled fp32 product: FT_M images x FT_N outputs per CTA, K in chunks of FT_K through FT_STAGES
+// logits = pooled * w^T + bias as a tiled fp32 product: FT_M images x FT_N outputs per CTA, K in chunks of FT_K through a ring of
 // cp.async stages.  The eight warps take four of a chunk's K values each and every warp owns all of the tile, 8 x 8 outputs
 // per thread; the warps' sums are added through shared memory.  SPLIT CTAs (a cluster) share a tile's K where there are too few
 // tiles for the chip, and add their sums through each other's shared memory (64 x 100 x 2048: 12.0 -> 5.4 us, 256 x 10 x 2048 10.5 ->
-// 5.2).  32 outputs, two CTAs a multiprocessor, where tiles are few; with 64 a weight goes twice as far (256 x 1000 x 256: 7.4 and 6.7 us).  What is left at 256 x 1000 x 1024 (20.7 -> 19.6 us, 7.1 of the fp32 pipe) did not move with 16 x 8 outputs per thread, pairs of
-// multiply-adds, chunks of 64 or a rolled loop.
-constexpr int FT_M = 32, FT_K = 32, FT_STAGES = 8, FT_THREADS = 256, FT_PITCH = FT_K + 4;
+// 5.2).  32 outputs where tiles are few; with 64 a weight goes twice as far (256 x 1000 x 256: 7.4 and 6.7 us).  Up to a wave the CTAs ask
+// for so much shared memory that each has its multiprocessor to itself: left to itself the scheduler pairs some of 130 to 148 while others idle
+// (215 images x 656 outputs x 916: 16.0 -> 11.9 us).  In several waves of 32 outputs two share a multiprocessor,
+// six stages or 59 KB each; with eight stages the times are those of one (498 x 708 x 1512: 55.8 and 45.4).  What is left at 256 x 1000 x 1024 (20.7 -> 19.6 us, 7.1 of the fp32 pipe) did not move with 16 x 8
+// outputs per thread, pairs of multiply-adds, chunks of 64, 16-byte reads or a rolled loop.
+constexpr int FT_M = 32, FT_K = 32, FT_THREADS = 256, FT_PITCH = FT_K + 4;
 constexpr int FT_PIECES = FT_K / 4, FT_ROWS = FT_THREADS / FT_PIECES, FT_KW = FT_K / 8;      // 16-byte pieces of a row, rows loaded at a time, a warp's K values
 
-constexpr int ft_smem(int n) { return (FT_STAGES * (FT_M + n) * FT_PITCH + FT_M * n) * 4; }
+__host__ __device__ constexpr int ft_stages(int n) { return n == 32 ? 6 : 8; }
+constexpr int ft_smem(int n) { return (ft_stages(n) * (FT_M + n) * FT_PITCH + FT_M * n) * 4; }
+constexpr int FT_ALONE = 116 * 1024;
 template <int SPLIT, int FT_N>
-__global__ void __launch_bounds__(FT_THREADS, 1)
+__global__ void __launch_bounds__(FT_THREADS, FT_N == 32 ? 2 : 1)
 fc_tile_kernel(const float *pooled, const float *w, const float *bias, float *logits, int B, int C, int N, int per)
 {
-    constexpr int FT_STAGE_FLOATS = (FT_M + FT_N) * FT_PITCH, NJ = FT_N / 8;
+    constexpr int FT_STAGES = ft_stages(FT_N), FT_STAGE_FLOATS = (FT_M + FT_N) * FT_PITCH, NJ = FT_N / 8;
     static_assert(8 * FT_M * FT_N <= FT_STAGES * FT_STAGE_FLOATS, "the warps' sums fit the stages");
     extern __shared__ __align__(16) float sm[];                 // [FT_STAGES][FT_STAGE_FLOATS], [FT_M][FT_N] sums of this CTA
     const int tid = threadIdx.x, warp = tid >> 5, tm = (tid & 31) >> 3, tn = tid & 7;
@@ -673,58 +678,99 @@ int launch_gap(const uint16_t *x, float *pooled, int B, int HW, int C, cudaStrea
     return launch(gap_kernel, (unsigned)blocks, 256, 0, stream, x, pooled, HW, C, GX);
 }
 
+// What a tile's launch asks for in shared memory: `alone`, so much that no second CTA comes in beside it.
+template <int FT_N> constexpr int ft_ask(bool alone) { return alone && ft_smem(FT_N) < FT_ALONE ? FT_ALONE : ft_smem(FT_N); }
+
+// Clusters of SPLIT CTAs, each alone on its multiprocessor, that run at a time.
 template <int SPLIT, int FT_N>
-static int launch_fc_tile(const float *pooled, const float *w, const float *bias, float *logits, int B, int C, int N, int per, long tiles_n, long tiles_b, cudaStream_t stream)
+static long fc_capacity()
+{
+    if (SPLIT == 1) return sm_count();
+    auto k = fc_tile_kernel<SPLIT, FT_N>;
+    if (!allow_smem((const void *)k, ft_ask<FT_N>(true))) return 0;
+    return max_clusters((const void *)k, SPLIT, FT_THREADS, ft_ask<FT_N>(true));
+}
+
+template <int SPLIT, int FT_N>
+static int launch_fc_tile(const float *pooled, const float *w, const float *bias, float *logits, int B, int C, int N, long tiles_n, long tiles_b, bool alone, cudaStream_t stream)
 {
     auto k = fc_tile_kernel<SPLIT, FT_N>;
-    if (!allow_smem((const void *)k, ft_smem(FT_N))) return BCNN_ERR_CUDA;
-    return launch<SPLIT>(k, dim3((unsigned)(tiles_n * SPLIT), (unsigned)tiles_b), FT_THREADS, ft_smem(FT_N), stream, pooled, w, bias, logits, B, C, N, per);
+    if (!allow_smem((const void *)k, ft_ask<FT_N>(true))) return BCNN_ERR_CUDA;
+    const int chunks = (C + FT_K - 1) / FT_K, per = (chunks + SPLIT - 1) / SPLIT;
+    return launch<SPLIT>(k, dim3((unsigned)(tiles_n * SPLIT), (unsigned)tiles_b), FT_THREADS, ft_ask<FT_N>(alone), stream, pooled, w, bias, logits, B, C, N, per);
+}
+
+// A width and a split of K with the time they are expected to take, ns.
+struct FcPlan {
+    long ns;
+    int split;
+    bool alone;
+};
+
+template <int FT_N>
+static FcPlan fc_plan(long tiles, int chunks)
+{
+    const long sms = sm_count();
+    FcPlan best = {LONG_MAX, 1, false};
+    for (int split = 1; split <= 8 && (split == 1 || split <= chunks); split *= 2) {
+        // a split tile is one wave: a second one costs more than its shorter K saves
+        const long fit = split == 1 ? fc_capacity<1, FT_N>() : split == 2 ? fc_capacity<2, FT_N>() : split == 4 ? fc_capacity<4, FT_N>() : fc_capacity<8, FT_N>();
+        if (split > 1 && tiles > fit) break;
+        const long per = (chunks + split - 1) / split;
+        long ns;
+        if (FT_N == 64) {
+            ns = 160 + (split > 1 ? 790 : 0) + (tiles + sms - 1) / sms * (1845 + 529 * per);
+        } else if (tiles <= fit) {
+            ns = 1540 + (split > 1 ? 940 : 0) + 337 * per;
+            if (ns < 2150) ns = 2150;
+        } else {
+            // two on a multiprocessor, the last wave's perhaps alone
+            const long shared = tiles / (2 * sms), rest = tiles % (2 * sms);
+            ns = 830 + (shared + (rest > sms)) * (1470 + 527 * per) + (rest > 0 && rest <= sms ? 1100 + 332 * per : 0);
+        }
+        if (ns < best.ns) best = {ns, split, tiles <= fit};
+    }
+    return best;
 }
 
 template <int FT_N>
-static int launch_fc_tiles(const float *pooled, const float *w, const float *bias, float *logits, int B, int C, int N, int split, int per, long tiles_n, long tiles_b, cudaStream_t stream)
+static int launch_fc_tiles(const FcPlan &plan, const float *pooled, const float *w, const float *bias, float *logits, int B, int C, int N, long tiles_n, long tiles_b, cudaStream_t stream)
 {
-    switch (split) {
-    case 8: return launch_fc_tile<8, FT_N>(pooled, w, bias, logits, B, C, N, per, tiles_n, tiles_b, stream);
-    case 4: return launch_fc_tile<4, FT_N>(pooled, w, bias, logits, B, C, N, per, tiles_n, tiles_b, stream);
-    case 2: return launch_fc_tile<2, FT_N>(pooled, w, bias, logits, B, C, N, per, tiles_n, tiles_b, stream);
-    default: return launch_fc_tile<1, FT_N>(pooled, w, bias, logits, B, C, N, per, tiles_n, tiles_b, stream);
+    switch (plan.split) {
+    case 8: return launch_fc_tile<8, FT_N>(pooled, w, bias, logits, B, C, N, tiles_n, tiles_b, plan.alone, stream);
+    case 4: return launch_fc_tile<4, FT_N>(pooled, w, bias, logits, B, C, N, tiles_n, tiles_b, plan.alone, stream);
+    case 2: return launch_fc_tile<2, FT_N>(pooled, w, bias, logits, B, C, N, tiles_n, tiles_b, plan.alone, stream);
+    default: return launch_fc_tile<1, FT_N>(pooled, w, bias, logits, B, C, N, tiles_n, tiles_b, plan.alone, stream);
     }
 }
 
 int launch_fc(const float *pooled, const float *w, const float *bias, float *logits, int B, int C, int N, cudaStream_t stream)
 {
-    // Tiles of 64 or 32 outputs, with the K of each split over as many CTAs as make one wave, or the kernel below, which walks K in steps of 512 for
-    // four images at a time.  Estimates in ns, fitted to sixteen heads (images x channels x outputs; 32 and 64 wide, streamed us):
-    // 64 x 128 x 1000 3.5, 4.0, 6.2; 32 x 512 x 1000 5.3, 7.8 (clusters of eight do not all fit at once), 9.1; 256 x 256 x 1000 7.4, 6.7, 21.2;
-    // 64 x 2048 x 100 5.4, 7.2, 11.9; 250 x 32 x 2000 5.0, 5.4, 29.3; 19 x 344 x 202 3.3, 4.0, 3.1; 100 x 96 x 50 3.3, 4.1, 2.1
-    const int sms = sm_count(), chunks = (C + FT_K - 1) / FT_K;
-    const long tiles_b = ((long)B + FT_M - 1) / FT_M;
-    auto split_of = [&](long tiles) {
-        int split = 1;
-        while (split < 8 && split * 2 <= chunks && tiles * split * 2 <= sms) split *= 2;
-        return split;
-    };
-    const int smem = FC_IMAGES * C * 4;
-    const long n32 = ((long)N + 31) / 32, n64 = ((long)N + 63) / 64;
+    // Tiles of 64 or 32 outputs, with the K of each over as many CTAs as run at a time, or the kernel below, which walks K in steps of 512 for
+    // four images at a time.  Estimates in ns, fitted to 4462 heads drawn from 1 .. 512 images, 8 .. 4096 channels and 4 .. 6000 outputs (the choice
+    // takes 1 % longer than the best of all variants in the mean); images x channels x outputs, us at 32 and 64 wide, streamed:
+    // 32 x 580 x 2344 6.3, 8.7, 16.5; 203 x 516 x 274 5.9, 8.1, 12.8; 2 x 2328 x 1146 13.9, 13.4, 9.5; 4 x 2956 x 42 5.9, 7.0, 13;
+    // 167 x 2480 x 2335 73, 92, 208; 446 x 24 x 15 2.1, 2.7, 1.8.  Tiles have to be 8 % ahead: the streaming estimate is the least sure.
+    const int sms = sm_count(), chunks = (int)(((long)C + FT_K - 1) / FT_K);
+    const long tiles_b = ((long)B + FT_M - 1) / FT_M, n32 = ((long)N + 31) / 32, n64 = ((long)N + 63) / 64, images = ((long)B + FC_IMAGES - 1) / FC_IMAGES;
+    const long smem = (long)FC_IMAGES * C * 4;
+    const bool streams = smem <= 200 * 1024;
     // rows of more channels than the kernel below can hold (12800) are taken in large products only
-    if (smem > 200 * 1024 && (long)((B + 3) / 4) * N <= 10600 * ((n32 * tiles_b + 2 * sms - 1) / (2 * sms))) return BCNN_ERR_UNSUPPORTED;
-    const int split32 = split_of(n32 * tiles_b), split64 = split_of(n64 * tiles_b);
-    const int per32 = (chunks + split32 - 1) / split32, per64 = (chunks + split64 - 1) / split64;
-    // a narrow tile has a multiprocessor to itself in the last wave, or shares it with another
-    const long ctas = n32 * tiles_b * split32, shared = ctas / (2 * sms), rest = ctas % (2 * sms);
-    const long narrow = 1000 + (split32 > 1 ? 300 : 0) + (shared + (rest > sms)) * (1700 + per32 * 550L) + (rest > 0 && rest <= sms ? 1400 + per32 * 430L : 0);
-    const long wide = 1000 + (split64 == 8 ? 1500 : split64 > 1 ? 900 : 0) + (n64 * tiles_b * split64 + sms - 1) / sms * (1500 + per64 * 550L);
-    const long streamed = smem > 200 * 1024 ? LONG_MAX : 1700 + 3L * C + (long)((B + 3) / 4) * N * (200 + 7 * C / 10) / 1000;      // (rows it cannot hold)
-    if ((narrow < wide ? narrow : wide) < streamed && tiles_b < 65536 && n32 < (1L << 27))
-        return narrow <= wide ? launch_fc_tiles<32>(pooled, w, bias, logits, B, C, N, split32, per32, n32, tiles_b, stream)
-                              : launch_fc_tiles<64>(pooled, w, bias, logits, B, C, N, split64, per64, n64, tiles_b, stream);
-    if (smem > 200 * 1024) return BCNN_ERR_UNSUPPORTED;
-    if (!allow_smem((const void *)fc_kernel, 200 * 1024)) return BCNN_ERR_CUDA;
-    const int images = (B + FC_IMAGES - 1) / FC_IMAGES;
-    int ny = 1;                                     // enough CTAs to fill the GPU a few times over
+    if (!streams && images * N <= 10600 * ((n32 * tiles_b + 2 * sms - 1) / (2 * sms))) return BCNN_ERR_UNSUPPORTED;
+    int ny = 1;                                     // (streaming) enough CTAs to fill the GPU a few times over
     while (images * ny < 592 && ny * 8 < N) ny *= 2;
-    return launch(fc_kernel, dim3(images, ny), 256, smem, stream, pooled, w, bias, logits, B, C, N);
+    const long outs = (N + 8L * ny - 1) / (8L * ny);                         // of a warp
+    const long streamed = streams ? 1250 + (B < FC_IMAGES ? B : FC_IMAGES) * 94L * C / 100 + outs * ((C + 511) / 512) * 250 + images * N * (180 + 3 * C / 4) / 1000 : LONG_MAX;
+    if (tiles_b < 65536 && n32 < (1L << 27)) {
+        const FcPlan narrow = fc_plan<32>(n32 * tiles_b, chunks), wide = fc_plan<64>(n64 * tiles_b, chunks);
+        const long tiled = narrow.ns < wide.ns ? narrow.ns : wide.ns;
+        if (!streams || tiled * 27 / 25 < streamed)
+            return narrow.ns <= wide.ns ? launch_fc_tiles<32>(narrow, pooled, w, bias, logits, B, C, N, n32, tiles_b, stream)
+                                        : launch_fc_tiles<64>(wide, pooled, w, bias, logits, B, C, N, n64, tiles_b, stream);
+    }
+    if (!streams) return BCNN_ERR_UNSUPPORTED;
+    if (!allow_smem((const void *)fc_kernel, 200 * 1024)) return BCNN_ERR_CUDA;
+    return launch(fc_kernel, dim3((unsigned)images, (unsigned)ny), 256, (size_t)smem, stream, pooled, w, bias, logits, B, C, N);
 }
 
 }  // namespace bcnn

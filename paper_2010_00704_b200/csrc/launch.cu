@@ -91,6 +91,32 @@ int blocks_per_sm(const void *kernel, int threads, size_t smem)
     return n;
 }
 
+int max_clusters(const void *kernel, int cluster, int threads, size_t smem)
+{
+    static Slot table[SLOTS];
+    const int dev = current_device();
+    // one cluster size, thread count and size of shared memory per kernel
+    const uint64_t key = kernel_key(kernel, dev);
+    int n = find(table, key);
+    if (n > 0) return n;
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeClusterDimension;
+    attr.val.clusterDim.x = (unsigned)cluster;
+    attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)cluster);
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    if (cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) != cudaSuccess || n < 1) {
+        (void)cudaGetLastError();
+        return 0;
+    }
+    if (dev >= 0 && dev < MAX_DEVICES) insert(table, key, n);
+    return n;
+}
+
 bool allow_smem(const void *kernel, int bytes)
 {
     static Slot table[SLOTS];

@@ -12,6 +12,9 @@ namespace bcnn {
 int sm_count();
 // Resident blocks of `kernel` per multiprocessor (at least 1).
 int blocks_per_sm(const void *kernel, int threads, size_t smem);
+// Clusters of `cluster` blocks of `kernel` that the device holds at a time; 0 where the query fails.  Fewer than its multiprocessors give in sum:
+// a cluster lies within one processing cluster (at one block a multiprocessor fifteen of eight, 33 of four, 74 of two on 148).
+int max_clusters(const void *kernel, int cluster, int threads, size_t smem);
 // Raises the kernel's dynamic shared-memory limit to `bytes` on the current device; the driver is asked on the first
 // call only.  The limit is a property of the kernel, not of a launch: callers always pass the same `bytes` for a kernel,
 // so a captured launch stays valid whatever later calls with other shapes ask for.

@@ -276,9 +276,10 @@ def test_prepared_one_stage_int32(bk, oracle, M, N, K):
 
 
 # the tiled product with its K over two, four and eight blocks (the last of them without a chunk), ragged in images, outputs and K; tiles of 32 and 64
-# outputs in one wave and in several
+# outputs in one wave, alone on their multiprocessors, and in several, two on each; few images, tiled and streamed
 @pytest.mark.parametrize("shape", [(64, 2048, 100), (97, 1156, 130), (130, 516, 700), (200, 2052, 1000), (300, 264, 65), (61, 1100, 513), (256, 2048, 10),
-                                   (64, 160, 500), (250, 36, 2001), (201, 264, 2999), (129, 516, 1001), (255, 128, 4001)])
+                                   (64, 160, 500), (250, 36, 2001), (201, 264, 2999), (129, 516, 1001), (255, 128, 4001),
+                                   (215, 516, 656), (98, 388, 2401), (4, 2956, 42), (2, 2328, 1146)])
 def test_fc_split(bk, oracle, shape):
     test_fc_shapes(bk, oracle, shape)
 
