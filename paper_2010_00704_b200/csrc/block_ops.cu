@@ -668,11 +668,12 @@ int launch_gap(const uint16_t *x, float *pooled, int B, int HW, int C, cudaStrea
 {
     // channel groups of a block: the power of two that fits the channels, up to 32; fewer, and more pixels at a time, where that many
     // leave multiprocessors idle (8 images of 10 x 10 x 192: 4.0 -> 2.4 us, 4 of 9 x 9 x 2048 3.8 -> 2.7, 2 of 14 x 14 x 1600 6.9 -> 2.9;
-    // 200 of 9 x 9 x 264 4.9 with 32, 5.2 with 8)
+    // 200 of 9 x 9 x 264 4.9 with 32, 5.2 with 8).  Not for so few pixels that a slice has no more than three: the slices' sums are added one after
+    // the other (14 images of 2 x 2 x 1112 1.80 -> 2.07 us, 131 of 4 x 4 x 152 2.21 -> 2.50)
     const int groups = C / 8;
     int GX = 32;
     while (GX > 1 && GX / 2 >= groups) GX /= 2;
-    while (GX > 8 && (long)B * ((groups + GX - 1) / GX) < sm_count()) GX /= 2;
+    while (GX > 8 && HW > 3 * (256 / GX) && (long)B * ((groups + GX - 1) / GX) < sm_count()) GX /= 2;
     const long blocks = (long)B * ((groups + GX - 1) / GX);
     if (blocks >= (1L << 31)) return BCNN_ERR_UNSUPPORTED;
     return launch(gap_kernel, (unsigned)blocks, 256, 0, stream, x, pooled, HW, C, GX);

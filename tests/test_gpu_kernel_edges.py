@@ -290,8 +290,8 @@ def test_fc_long_rows(bk, oracle, shape):
     test_fc_shapes(bk, oracle, shape)
 
 
-# pooling by 8 and 16 channel groups of few images
-@pytest.mark.parametrize("shape", [(8, 10, 10, 192), (1, 13, 11, 264), (20, 9, 9, 1600)])
+# pooling by 8 and 16 channel groups of few images, by 32 and 16 where a slice has three pixels at most
+@pytest.mark.parametrize("shape", [(8, 10, 10, 192), (1, 13, 11, 264), (20, 9, 9, 1600), (14, 2, 2, 1112), (3, 4, 6, 520), (3, 5, 5, 520), (2, 6, 8, 136)])
 def test_gap_few_images(bk, oracle, shape):
     test_gap_shapes(bk, oracle, shape)
 
