@@ -277,6 +277,15 @@ int bcnn_conv2d_b1_fused_noalloc(const void *x_bits, const void *w_bits, const i
 int bcnn_auto_engine(int B, int H, int W, int C_in, int C_out, int kh, int kw, int stride, int pad, int fused);
 
 /*
+ * How bcnn_conv2d_b1_branches runs a module of this shape, five values into plan[]: output channels of one part of the
+ * tensor-core module engine (64 or 32; 0: the module runs on the CUDA cores), slices of that many channels whose weights a
+ * block keeps, 256-bit stages of a row, slots of the ring that holds them, and how many staging tiles do not wait for the
+ * weights.  For tests that have to reach a certain path.  No pointers but plan, no launch; a negative bcnn_status for an
+ * invalid shape.
+ */
+int bcnn_branches_plan(int B, int H, int W, int C_in, int C_out, int P, int kh, int kw, int *plan);
+
+/*
  * Scratch memory (global memory beyond the inputs and outputs) a convolution of this shape needs, in bytes
  * (fused != 0: the packed output).  Every kernel of the library works out of its inputs, outputs, shared and
  * tensor memory, so this is 0 for every valid shape and no call takes a workspace argument; an invalid shape

@@ -175,6 +175,32 @@ int gemm_problem(ConvProblem &p, const void *A, const void *Wb, const int32_t *t
     return make_conv_problem(p, A, Wb, thr, out, 1, (int)M, 1, K, N, 1, 1, 1, 0, fused);
 }
 
+int make_branch_problem(BranchProblem &p, const void *x_bits, const void *w_bits, const float *bn_scale, const float *bn_shift,
+                        const int32_t *pad_dot, const void *identity, const float *prelu_slope, const float *next_bias,
+                        void *y_real, void *y_bits, int B, int H, int W, int C_in, int C_out, int P, int kh, int kw)
+{
+    if (!x_bits || !w_bits || !bn_scale || !bn_shift || !prelu_slope || !y_real) return BCNN_ERR_INVALID_ARG;
+    if (B <= 0 || H <= 0 || W <= 0 || C_in <= 0 || C_out <= 0 || P <= 0 || kh <= 0 || kw <= 0) return BCNN_ERR_INVALID_ARG;
+    if (kh * kw > 1 && P != kh * kw) return BCNN_ERR_INVALID_ARG;
+    if (C_in % 32 != 0 || C_out % 32 != 0 || P > 64 || (kh % 2 == 0) || (kw % 2 == 0)) return BCNN_ERR_UNSUPPORTED;
+    if (!aligned16(x_bits) || !aligned16(w_bits) || !aligned16(bn_scale) || !aligned16(bn_shift) || !aligned16(prelu_slope) ||
+        !aligned16(y_real) || (pad_dot && !aligned16(pad_dot)) || (identity && !aligned16(identity)) ||
+        (next_bias && !aligned16(next_bias)) || (y_bits && !aligned16(y_bits)))
+        return BCNN_ERR_ALIGNMENT;
+    p.x = static_cast<const uint32_t *>(x_bits);
+    p.w = static_cast<const uint32_t *>(w_bits);
+    p.bn_scale = bn_scale; p.bn_shift = bn_shift; p.pad_dot = pad_dot;
+    p.identity = static_cast<const uint16_t *>(identity);
+    p.slope = prelu_slope; p.next_bias = next_bias;
+    p.y_real = static_cast<uint16_t *>(y_real);
+    p.y_bits = static_cast<uint8_t *>(y_bits);
+    p.B = B; p.H = H; p.W = W; p.C_in = C_in; p.C_out = C_out; p.P = P; p.kh = kh; p.kw = kw;
+    p.cw = C_in / 32;
+    p.M = (long)B * H * W;
+    if (p.M >= (1L << 40)) return BCNN_ERR_UNSUPPORTED;
+    return BCNN_OK;
+}
+
 }  // namespace
 }  // namespace bcnn
 
@@ -273,30 +299,28 @@ int bcnn_conv2d_b1_branches(const void *x_bits, const void *w_bits, const float 
                             void *y_real, void *y_bits, int B, int H, int W, int C_in, int C_out, int P, int kh, int kw,
                             void *stream)
 {
-    if (!x_bits || !w_bits || !bn_scale || !bn_shift || !prelu_slope || !y_real) return BCNN_ERR_INVALID_ARG;
-    if (B <= 0 || H <= 0 || W <= 0 || C_in <= 0 || C_out <= 0 || P <= 0 || kh <= 0 || kw <= 0) return BCNN_ERR_INVALID_ARG;
-    if (kh * kw > 1 && P != kh * kw) return BCNN_ERR_INVALID_ARG;
-    if (C_in % 32 != 0 || C_out % 32 != 0 || P > 64 || (kh % 2 == 0) || (kw % 2 == 0)) return BCNN_ERR_UNSUPPORTED;
-    if (!aligned16(x_bits) || !aligned16(w_bits) || !aligned16(bn_scale) || !aligned16(bn_shift) || !aligned16(prelu_slope) ||
-        !aligned16(y_real) || (pad_dot && !aligned16(pad_dot)) || (identity && !aligned16(identity)) ||
-        (next_bias && !aligned16(next_bias)) || (y_bits && !aligned16(y_bits)))
-        return BCNN_ERR_ALIGNMENT;
     BranchProblem p;
-    p.x = static_cast<const uint32_t *>(x_bits);
-    p.w = static_cast<const uint32_t *>(w_bits);
-    p.bn_scale = bn_scale; p.bn_shift = bn_shift; p.pad_dot = pad_dot;
-    p.identity = static_cast<const uint16_t *>(identity);
-    p.slope = prelu_slope; p.next_bias = next_bias;
-    p.y_real = static_cast<uint16_t *>(y_real);
-    p.y_bits = static_cast<uint8_t *>(y_bits);
-    p.B = B; p.H = H; p.W = W; p.C_in = C_in; p.C_out = C_out; p.P = P; p.kh = kh; p.kw = kw;
-    p.cw = C_in / 32;
-    p.M = (long)B * H * W;
-    if (p.M >= (1L << 40)) return BCNN_ERR_UNSUPPORTED;
-    // on the tensor cores where the branches' accumulators and one slice of their weights fit (13 branches), else on the CUDA cores
+    const int st = make_branch_problem(p, x_bits, w_bits, bn_scale, bn_shift, pad_dot, identity, prelu_slope, next_bias, y_real, y_bits, B, H, W,
+                                       C_in, C_out, P, kh, kw);
+    if (st != BCNN_OK) return st;
+    // on the tensor cores where the branches' accumulators and one slice of their weights fit (13 branches; bcnn_branches_plan), else on the CUDA cores
     const int mod = launch_branches_tc_mod(p, static_cast<cudaStream_t>(stream));
     if (mod != BCNN_ERR_UNSUPPORTED) return mod;
     return launch_conv_branches(p, static_cast<cudaStream_t>(stream));
+}
+
+int bcnn_branches_plan(int B, int H, int W, int C_in, int C_out, int P, int kh, int kw, int *plan)
+{
+    if (!plan) return BCNN_ERR_INVALID_ARG;
+    BranchProblem p;
+    void *dummy = reinterpret_cast<void *>(uintptr_t(4096));
+    const float *f = static_cast<const float *>(dummy);
+    const int st = make_branch_problem(p, dummy, dummy, f, f, nullptr, dummy, f, f, dummy, dummy, B, H, W, C_in, C_out, P, kh, kw);
+    if (st != BCNN_OK) return st;
+    int v[5];
+    branches_tc_mod_plan(p, v);
+    for (int i = 0; i < 5; ++i) plan[i] = v[i];
+    return BCNN_OK;
 }
 
 int bcnn_dwconv3x3_module(const void *x, const float *w, const float *bn_scale, const float *bn_shift, const float *prelu_slope,

@@ -111,6 +111,7 @@ size_t static_prepared_capacity();
 bool conv_tc_i8_supports(const ConvProblem &p);
 int launch_conv_tc_mod(const ConvProblem &p, cudaStream_t stream);
 int launch_branches_tc_mod(const BranchProblem &b, cudaStream_t stream);
+void branches_tc_mod_plan(const BranchProblem &b, int (&plan)[5]);
 void exact_div_params(uint32_t d, uint32_t &mul, uint32_t &shift);   // (mul, shift) of exact_div for the divisor d >= 1
 int launch_selftest_wait_timeout(int polls, cudaStream_t stream);
 int launch_conv_branches(const BranchProblem &p, cudaStream_t stream);

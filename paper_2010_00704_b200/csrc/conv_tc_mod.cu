@@ -65,6 +65,7 @@ struct ModPlan {
     TileStep ts;              // from a row tile to the CTA's next
     int units, gw;            // gather units of a row
     uint32_t off_bits, off_stage, off_table, off_pad, off_tab, off_const, off_raw;      // shared-memory offsets from the 1024-byte aligned base (weights first)
+    int early_tiles;          // staging tiles ahead of the packed weights, which lie over the others until they are expanded
 };
 
 // a pair of channels in the parameter table: P entries of 16 bytes {scale, shift} x 2, then 16 bytes {slope x 2, sign threshold x 2 (fp16), -}
@@ -217,6 +218,7 @@ conv_tc_mod_kernel(const ModPlan L, const __grid_constant__ CUtensorMap idmap, c
         __device__ __forceinline__ void skip(int n, int rs, int rows) { for (slice += n; slice >= rs; slice -= rs) row += rows; }
     };
     const int tile_rows = step * BM, ch_base = cg * L.rs * BN;
+    auto stage_tile = [&](int t, int s) { return staging + (uint32_t)((s * TEAMS + t) * TILE_BYTES); };      // in the order of their first use
 
     if (warp == ISSUER) {
         // ------------------------------------------------------------------ MMA issuer
@@ -273,11 +275,13 @@ conv_tc_mod_kernel(const ModPlan L, const __grid_constant__ CUtensorMap idmap, c
             pdl_wait();
 #pragma unroll 1
             for (int n = 0; n < parts; ++n, ++issued, at.skip(1, rs, tile_rows)) {
+                // the epilogue's warps are done with the packed weights, which lay here
+                if (n == L.early_tiles && !mbar_wait_warp(ready_bar, 0, abort_flag, p.err, ERR_MOD_LOADER)) break;
                 if (!mbar_wait_warp(slot_free(team, s), phase, abort_flag, p.err, ERR_MOD_LOADER)) break;
                 if (lane == 0) {
                     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(id_full(team, s)), "r"((uint32_t)TILE_BYTES) : "memory");
                     asm volatile("cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
-                                 ::"r"(staging + (uint32_t)((team * NS + s) * TILE_BYTES)), "l"(reinterpret_cast<uint64_t>(&idmap)), "r"(ch_base + at.slice * BN), "r"(at.row),
+                                 ::"r"(stage_tile(team, s)), "l"(reinterpret_cast<uint64_t>(&idmap)), "r"(ch_base + at.slice * BN), "r"(at.row),
                                    "r"(id_full(team, s)) : "memory");
                 }
                 __syncwarp();
@@ -304,7 +308,7 @@ conv_tc_mod_kernel(const ModPlan L, const __grid_constant__ CUtensorMap idmap, c
             if (!mbar_wait_warp(out_full(team, s), phase, abort_flag, p.err, ERR_MOD_STORE)) break;
             if (lane == 0) {
                 asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.tile.bulk_group [%0, {%1, %2}], [%3];"
-                             ::"l"(reinterpret_cast<uint64_t>(&ymap)), "r"(ch_base + at.slice * BN), "r"(at.row), "r"(staging + (uint32_t)((team * NS + s) * TILE_BYTES)) : "memory");
+                             ::"l"(reinterpret_cast<uint64_t>(&ymap)), "r"(ch_base + at.slice * BN), "r"(at.row), "r"(stage_tile(team, s)) : "memory");
                 asm volatile("cp.async.bulk.commit_group;" ::: "memory");
                 if (before >= 0) {                                          // the store before this one has read its tile
                     asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory");
@@ -323,7 +327,9 @@ conv_tc_mod_kernel(const ModPlan L, const __grid_constant__ CUtensorMap idmap, c
         // memory in one go, eight lanes expand a (branch, slice, channel) row and count its bits, then the constants (the issuer
         // waits for weights and constants).  Rolled loops on purpose: this code runs once, and its instructions come from memory.
         // (A thread per word with eight loads in flight, an atomic per word and a division per index took 5 us for two branches
-        // of 256 channels, a quarter of the kernel at 50176 rows.)
+        // of 256 channels, a quarter of the kernel at 50176 rows.)  What comes lies over the staging tiles behind the first ones, which hold nothing
+        // until all of it is expanded: in an area of its own it left P = 2, 256 channels two resident slices instead of four, and P = 8, 1024
+        // channels no room at all.  (Without an identity these same warps are the tiles' first users.)
         constexpr int ETHREADS = 128 * TEAMS;
         const int etid = tid - 32 * FIRST_EPILOGUE;
         const int rows1 = rs * BN, rows_w = P * rows1;                      // rows of a branch, of all
@@ -445,7 +451,7 @@ conv_tc_mod_kernel(const ModPlan L, const __grid_constant__ CUtensorMap idmap, c
             if (!mbar_wait_warp(tfull_bar(n % MAX_NBUF), (uint32_t)(n / MAX_NBUF) & 1u, abort_flag, p.err, ERR_MOD_EPILOGUE)) break;
             tc_fence_after();
             const uint32_t acc = t_lane + (uint32_t)(buf * P * BN);
-            const uint32_t tile = staging + (uint32_t)((team * NS + s) * TILE_BYTES) + (uint32_t)(row * ROW_BYTES);
+            const uint32_t tile = stage_tile(team, s) + (uint32_t)(row * ROW_BYTES);
             const int sl = part.slice;
             const uint32_t tb = table + (uint32_t)(sl * 4 + lq) * share, pb = pads + (uint32_t)((sl * 4 + lq) * (BN / 8) * P) * 8u;
             // (two channels, branch) of four rows at a time; the next piece's accumulators and parameters are on their way while one is
@@ -634,7 +640,15 @@ bool make_plan(ModPlan &L, bool shifted, int &smem)
         const long table = (long)rs * 4 * share_bytes<BN>(pair_bytes(L.P));
         const long pad = shifted ? (long)rs * (BN / 2) * L.P * 8 : 0, consts = (long)const_tiles(rs, L.P) * BN * ROWB;
         const long raw = (long)rs * BN * 4 * (L.P * (L.bcw + (shifted ? 3 : 2)) + 2);
-        const long bytes = 1024 + rs * slice_bytes + consts + pad + staging + raw + (long)PF * SLOT_BYTES + table + 4L * L.units + 64;
+        // the packed weights over the staging tiles but a team's first, or, where that is too much, over all of them: the first identity
+        // tiles then wait too
+        int early = TEAMS;
+        auto bytes_of = [&]() {
+            const long over = (long)early * BM * BN * 2 + raw, area = over > staging ? over : staging;
+            return 1024 + rs * slice_bytes + consts + pad + area + (long)PF * SLOT_BYTES + table + 4L * L.units + 64;
+        };
+        if (bytes_of() > MAX_SMEM) early = 0;
+        const long bytes = bytes_of();
         if (bytes > MAX_SMEM) break;
         const int ng = (L.slices + rs - 1) / rs, per = sms / ng;
         if (per < 1) continue;
@@ -646,8 +660,10 @@ bool make_plan(ModPlan &L, bool shifted, int &smem)
         L.ng = ng;
         L.off_const = (uint32_t)(rs * slice_bytes);
         L.off_stage = L.off_const + (uint32_t)consts;
-        L.off_raw = L.off_stage + (uint32_t)staging;
+        L.early_tiles = early;
+        L.off_raw = L.off_stage + (uint32_t)(early * BM * BN * 2);
         L.off_bits = L.off_raw + (uint32_t)raw;
+        if (L.off_bits < L.off_stage + (uint32_t)staging) L.off_bits = L.off_stage + (uint32_t)staging;
         L.off_table = L.off_bits + (uint32_t)PF * SLOT_BYTES;
         L.off_pad = L.off_table + (uint32_t)table;
         L.off_tab = (L.off_pad + (uint32_t)pad + 15u) & ~15u;
@@ -683,31 +699,39 @@ int launch_plan(ModPlan &L, int smem, cudaStream_t stream)
     return launch(k, (unsigned)(per * L.ng), THREADS, smem, stream, L, map[0], map[1]);
 }
 
-int launch_mod(ModPlan &L, bool shifted, cudaStream_t stream)
+// Channels of a part (64, 32) with the plan for them, or 0 where the layer is not this engine's.
+int plan_mod(ModPlan &L, bool shifted, int &smem)
 {
-    ConvProblem &q = L.q;
+    const ConvProblem &q = L.q;
     L.kwp = (L.bcw + 1) & ~1;
     L.gw = L.bcw % 4 == 0 ? 4 : (L.bcw % 2 == 0 ? 2 : 1);
-    q.err = device_error_word();
-    if (L.P > 13 || (shifted && L.P != 9) || q.C_out % 32 != 0 || q.M < 1) return BCNN_ERR_UNSUPPORTED;
-    if ((long)q.B * q.H * q.W * q.cw >= (1L << 31) || (long)q.kh * q.W * q.cw >= (1L << 27) || 32L * L.bcw > CONST_MAX) return BCNN_ERR_UNSUPPORTED;
+    if (L.P > 13 || (shifted && L.P != 9) || q.C_out % 32 != 0 || q.M < 1) return 0;          // (odd squares up to 13: 9)
+    if ((long)q.B * q.H * q.W * q.cw >= (1L << 31) || (long)q.kh * q.W * q.cw >= (1L << 27) || 32L * L.bcw > CONST_MAX) return 0;
     L.m_tiles = (q.M - 1) / BM + 1;
-    int smem = 0;
     // 64-channel parts; 32 where that leaves a multiprocessor less than two parts (a part is 2 us of latency per 64 channels)
-    if (L.P <= 3 && !shifted && q.C_out > 32 && (long)L.m_tiles * ((q.C_out + 63) / 64) > sm_count() && make_plan<64>(L, shifted, smem)) {
+    if (L.P <= 3 && !shifted && q.C_out > 32 && (long)L.m_tiles * ((q.C_out + 63) / 64) > sm_count() && make_plan<64>(L, shifted, smem)) return 64;
+    return make_plan<32>(L, shifted, smem) ? 32 : 0;
+}
+
+int launch_mod(ModPlan &L, bool shifted, cudaStream_t stream)
+{
+    int smem = 0;
+    const int width = plan_mod(L, shifted, smem);
+    if (width == 0) return BCNN_ERR_UNSUPPORTED;
+    L.q.err = device_error_word();
+    if (width == 64) {
         if (L.P == 1) return launch_plan<64, 1, false>(L, smem, stream);
         if (L.P == 2) return launch_plan<64, 2, false>(L, smem, stream);
         return launch_plan<64, 3, false>(L, smem, stream);
     }
-    if (make_plan<32>(L, shifted, smem)) {
-        if (shifted) return launch_plan<32, 9, true>(L, smem, stream);      // odd squares up to 13: 9
-        if (L.P == 1) return launch_plan<32, 1, false>(L, smem, stream);
-        if (L.P == 2) return launch_plan<32, 2, false>(L, smem, stream);
-        if (L.P == 3) return launch_plan<32, 3, false>(L, smem, stream);
-        if (L.P == 4) return launch_plan<32, 4, false>(L, smem, stream);
-        return launch_plan<32, 0, false>(L, smem, stream);
+    if (shifted) return launch_plan<32, 9, true>(L, smem, stream);
+    switch (L.P) {
+    case 1: return launch_plan<32, 1, false>(L, smem, stream);
+    case 2: return launch_plan<32, 2, false>(L, smem, stream);
+    case 3: return launch_plan<32, 3, false>(L, smem, stream);
+    case 4: return launch_plan<32, 4, false>(L, smem, stream);
+    default: return launch_plan<32, 0, false>(L, smem, stream);
     }
-    return BCNN_ERR_UNSUPPORTED;
 }
 
 }  // namespace
@@ -725,11 +749,12 @@ int launch_conv_tc_mod(const ConvProblem &p, cudaStream_t stream)
     return launch_mod(L, false, stream);
 }
 
-int launch_branches_tc_mod(const BranchProblem &b, cudaStream_t stream)
+// The module engine's view of a branch module; false for a window it does not take.
+static bool branch_plan(const BranchProblem &b, ModPlan &L, bool &shifted)
 {
-    const bool shifted = b.kh * b.kw > 1;
-    if ((shifted && b.kh != b.kw) || b.M >= (1L << 31) || b.H >= (1 << 30) || b.P * (long)b.cw >= (1L << 20)) return BCNN_ERR_UNSUPPORTED;
-    ModPlan L = {};
+    shifted = b.kh * b.kw > 1;
+    if ((shifted && b.kh != b.kw) || b.M >= (1L << 31) || b.H >= (1 << 30) || b.P * (long)b.cw >= (1L << 20)) return false;
+    L = {};
     ConvProblem &q = L.q;
     q.x = b.x; q.w = b.w; q.out = b.y_bits;
     q.B = b.B; q.H = b.H; q.W = b.W; q.C_in = b.C_in; q.C_out = b.C_out;
@@ -742,7 +767,27 @@ int launch_branches_tc_mod(const BranchProblem &b, cudaStream_t stream)
     L.scale = b.bn_scale; L.shift = b.bn_shift; L.pad_dot = b.pad_dot;
     L.P = b.P;
     L.bcw = b.cw;
-    return launch_mod(L, shifted, stream);
+    return true;
+}
+
+int launch_branches_tc_mod(const BranchProblem &b, cudaStream_t stream)
+{
+    ModPlan L;
+    bool shifted;
+    return branch_plan(b, L, shifted) ? launch_mod(L, shifted, stream) : BCNN_ERR_UNSUPPORTED;
+}
+
+// Channels of a part (0: not this engine's), resident slices, stages of a row, ring slots, staging tiles ahead of the packed weights.
+void branches_tc_mod_plan(const BranchProblem &b, int (&plan)[5])
+{
+    ModPlan L;
+    bool shifted;
+    int smem = 0;
+    plan[0] = branch_plan(b, L, shifted) ? plan_mod(L, shifted, smem) : 0;
+    plan[1] = plan[0] ? L.rs : 0;
+    plan[2] = plan[0] ? L.kst : 0;
+    plan[3] = plan[0] ? L.stages : 0;
+    plan[4] = plan[0] ? L.early_tiles : 0;
 }
 
 }  // namespace bcnn

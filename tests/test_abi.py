@@ -114,6 +114,25 @@ def test_fc_takes_long_rows_in_large_products():
     assert lib.bcnn_fc(a, a, a, a, 1, 12800, 100, None) == binding.ERR_CUDA
 
 
+def test_module_engine_takes_wide_branch_modules():
+    # per number of branches a module at the end of the module engine's range: expanded weights of one slice of 32 output channels fill
+    # shared memory beside what has to lie there for as long
+    from paper_2010_00704_b200 import build, binding
+    build.build()
+    for P, widest in ((4, 2304), (5, 1792), (6, 1472), (7, 1280), (8, 1088), (9, 960), (10, 832), (11, 768), (12, 704), (13, 576)):
+        assert binding.bcnn_branches_plan(64, 28, 28, widest, widest, P)[0] == 32, P
+        assert binding.bcnn_branches_plan(64, 28, 28, widest, 32, P)[0] == 32, P
+        assert binding.bcnn_branches_plan(64, 28, 28, 2 * widest, 64, P)[0] == 0, P
+    assert binding.bcnn_branches_plan(64, 28, 28, 896, 896, 9, 3, 3)[0] == 32
+    for C in (1024, 2560):                                                          # K of one branch: up to 2560 by the constants
+        for P in (1, 2, 3):
+            assert binding.bcnn_branches_plan(64, 28, 28, C, C, P)[0] in (32, 64), (P, C)
+    assert binding.bcnn_branches_plan(64, 28, 28, 64, 64, 14)[0] == 0
+    # the weights as they come do not cost resident slices: P = 2, 256 channels keep all four
+    assert binding.bcnn_branches_plan(64, 28, 28, 256, 256, 2)[:2] == (64, 4)
+    assert binding.bcnn_branches_plan(64, 28, 28, 128, 128, 9, 3, 3)[:2] == (32, 4)
+
+
 def test_every_wait_code_has_a_name():
     # the codes as the kernels define them, each in one place
     from paper_2010_00704_b200 import build, binding

@@ -26,10 +26,39 @@ def test_avgpool_items(bk, oracle, shape):
     check_avgpool(bk, oracle, shape)
 
 
-# several parts per block: one accumulator buffer (nine taps), three (two branches), four (one branch); 32- and 64-channel parts,
-# a row tile that does not fit the ring (K = 13 * 512), the CUDA-core kernel behind the engine's limit (14 branches)
-@pytest.mark.parametrize("shape", [(20, 40, 40, 64, 64, 2), (20, 40, 40, 32, 96, 4), (26, 40, 40, 96, 64, 1), (1, 17, 19, 512, 64, 13), (1, 9, 15, 64, 32, 14)])
+# several parts per block: one accumulator buffer (nine taps), three (two branches), four (one branch); 32- and 64-channel parts; the
+# CUDA-core kernel behind the engine's limit (14 branches)
+@pytest.mark.parametrize("shape", [(20, 40, 40, 64, 64, 2), (20, 40, 40, 32, 96, 4), (26, 40, 40, 96, 64, 1), (1, 9, 15, 64, 32, 14)])
 def test_branches_many_parts(bk, oracle, shape):
+    check_branches(bk, oracle, shape, "full")
+
+
+# a row tile with more stages than the ring has slots: every slot refilled several times for one part, one or more row tiles a block
+@pytest.mark.parametrize("variant", ["full", "no_identity"])
+@pytest.mark.parametrize("shape", [(1, 17, 19, 480, 64, 13), (2, 100, 101, 288, 32, 13), (1, 17, 19, 512, 64, 13)])
+def test_branches_longer_than_the_ring(bk, oracle, shape, variant):
+    B, H, W, C_in, C_out, P = shape
+    part, _, row_stages, slots, _ = bk.bcnn_branches_plan(B, H, W, C_in, C_out, P)
+    assert part == 32 and row_stages > slots
+    check_branches(bk, oracle, shape, variant)
+
+
+# the widest modules the engine takes: the packed weights lie over all staging tiles (960 channels) or all but the teams' first (1024)
+# until they are expanded; tiles behind those are used by the same launch
+@pytest.mark.parametrize("variant", ["full", "no_identity", "in_place"])
+@pytest.mark.parametrize("shape,early", [((2, 40, 41, 960, 64, 9), 0), ((1, 30, 31, 1472, 32, 6), 0), ((2, 40, 41, 1024, 64, 8), 2), ((1, 26, 27, 768, 96, 9), 2)])
+def test_branches_widest(bk, oracle, shape, early, variant):
+    B, H, W, C_in, C_out, P = shape
+    assert bk.bcnn_branches_plan(B, H, W, C_in, C_out, P)[::4] == (32, early)
+    check_branches(bk, oracle, shape, variant)
+
+
+# many parts a block with all slices resident, so that the packed weights lie under identity tiles that come right behind them
+@pytest.mark.parametrize("shape", [(40, 28, 28, 256, 256, 2), (8, 28, 28, 96, 512, 4), (8, 28, 28, 64, 256, 5)])
+def test_branches_weights_under_staging_tiles(bk, oracle, shape):
+    B, H, W, C_in, C_out, P = shape
+    part, resident, _, _, early = bk.bcnn_branches_plan(B, H, W, C_in, C_out, P)
+    assert resident >= 3 and early == 2
     check_branches(bk, oracle, shape, "full")
 
 
