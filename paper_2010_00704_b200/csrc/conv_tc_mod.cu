@@ -142,7 +142,7 @@ template <int BN> __host__ __device__ constexpr int channel_of_column(int n) { r
 // bytes of a lane's share of the parameter table (16 more than its entries: the four shares lie in different banks)
 template <int BN> __host__ __device__ constexpr uint32_t share_bytes(uint32_t pair) { return (uint32_t)(BN / 8) * pair + 16u; }
 
-// BN: channels of a part (64, 32); PP: branches where known to the compiler (1 .. 4, 9), else 0; SHIFTED: taps with a row mask
+// BN: channels of a part (64, 32); PP: branches; SHIFTED: taps with a row mask
 template <int BN, int PP, bool SHIFTED, bool HAS_ID>
 __global__ void __launch_bounds__(THREADS, 1)
 conv_tc_mod_kernel(const ModPlan L, const __grid_constant__ CUtensorMap idmap, const __grid_constant__ CUtensorMap ymap)
@@ -154,7 +154,8 @@ conv_tc_mod_kernel(const ModPlan L, const __grid_constant__ CUtensorMap idmap, c
     __shared__ int abort_flag_smem;
 
     const ConvProblem &p = L.q;
-    const int P = PP ? PP : L.P;
+    constexpr int P = PP;
+    constexpr bool ROLLED = SHIFTED || PP >= 11;              // (below: the channel pairs of a piece in a loop)
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int kst = L.kst, stages = L.stages;
     const int idx = (int)exact_div(blockIdx.x, L.ng_mul, L.ng_shift), cg = (int)blockIdx.x - idx * L.ng, step = L.step;
@@ -454,6 +455,9 @@ conv_tc_mod_kernel(const ModPlan L, const __grid_constant__ CUtensorMap idmap, c
             const uint32_t tile = stage_tile(team, s) + (uint32_t)(row * ROW_BYTES);
             const int sl = part.slice;
             const uint32_t tb = table + (uint32_t)(sl * 4 + lq) * share, pb = pads + (uint32_t)((sl * 4 + lq) * (BN / 8) * P) * 8u;
+            // The branches are unrolled (P = 8, 64 channels at M = 50176 25.7 in a loop, 16.8 us), the four pairs of channels of a piece too where that is
+            // little code: with them in a loop nine taps of 128 channels take 45.9 us instead of 54.7, thirteen branches of 64 30.5 instead of
+            // 32.4, but eight of 64 17.6 instead of 16.8.
             // (two channels, branch) of four rows at a time; the next piece's accumulators and parameters are on their way while one is
             // worked on (a load and its wait in turn were a third of a part's time)
             uint32_t nv[8], sg[4] = {0u, 0u, 0u, 0u};                       // sg: even channels' bits in the low halves, odd ones' in the high
@@ -471,56 +475,58 @@ conv_tc_mod_kernel(const ModPlan L, const __grid_constant__ CUtensorMap idmap, c
                         io[i][0] = q.x; io[i][1] = q.y; io[i][2] = q.z; io[i][3] = q.w;
                     }
                 }
-#pragma unroll
+#pragma unroll(ROLLED ? 1 : 4)
                 for (int kk = 0; kk < 4; ++kk) {
                     const int k = k4 + kk;
                     unsigned long long t[4];
                     uint4 sn;
 #pragma unroll
-                    for (int br = 0; br < (PP ? PP : 1); ++br) {
-                        int b = br;
-                        do {
-                            const bool last_branch = b == P - 1;
-                            const uint4 ss = nss;                           // two channels' scales and shifts
-                            tc_wait_ld();
-                            pin_regs8(nv);
-                            unsigned long long dot[4];
+                    for (int b = 0; b < P; ++b) {
+                        const bool last_branch = b == P - 1;
+                        const uint4 ss = nss;                           // two channels' scales and shifts
+                        tc_wait_ld();
+                        pin_regs8(nv);
+                        unsigned long long dot[4];
 #pragma unroll
-                            for (int i = 0; i < 4; ++i) dot[i] = bits2(nv[2 * i], nv[2 * i + 1]);
-                            if (last_branch) sn = ld_shared_v4(tb + (uint32_t)k * pair + 16u * P);     // slopes, sign thresholds
-                            if (k < BN / 8 - 1 || !last_branch) {
-                                tc_ld8_quads_nowait(acc + (uint32_t)(last_branch ? (k + 1) * 8 : (b + 1) * BN + k * 8), nv);
-                                nss = ld_shared_v4(tb + (last_branch ? (uint32_t)(k + 1) * pair : (uint32_t)k * pair + 16u * (b + 1)));
-                            } else {                                        // the accumulators are in registers
-                                tc_fence_before();
-                                __syncwarp();
-                                if (lane == 0) mbar_arrive(tempty_bar(buf));
-                            }
-                            if (SHIFTED) {
-                                unsigned long long pd;
-                                asm volatile("ld.shared.b64 %0, [%1];" : "=l"(pd) : "r"(pb + (uint32_t)(k * P + b) * 8u) : "memory");
+                        for (int i = 0; i < 4; ++i) dot[i] = bits2(nv[2 * i], nv[2 * i + 1]);
+                        if (last_branch) sn = ld_shared_v4(tb + (uint32_t)k * pair + 16u * P);     // slopes, sign thresholds
+                        if (k < BN / 8 - 1 || !last_branch) {
+                            tc_ld8_quads_nowait(acc + (uint32_t)(last_branch ? (k + 1) * 8 : (b + 1) * BN + k * 8), nv);
+                            nss = ld_shared_v4(tb + (last_branch ? (uint32_t)(k + 1) * pair : (uint32_t)k * pair + 16u * (b + 1)));
+                        } else {                                        // the accumulators are in registers
+                            tc_fence_before();
+                            __syncwarp();
+                            if (lane == 0) mbar_arrive(tempty_bar(buf));
+                        }
+                        if (SHIFTED) {
+                            unsigned long long pd;
+                            asm volatile("ld.shared.b64 %0, [%1];" : "=l"(pd) : "r"(pb + (uint32_t)(k * P + b) * 8u) : "memory");
 #pragma unroll
-                                for (int i = 0; i < 4; ++i)
-                                    if (!((inside[i] >> b) & 1u)) dot[i] = pd;
-                            }
+                            for (int i = 0; i < 4; ++i)
+                                if (!((inside[i] >> b) & 1u)) dot[i] = pd;
+                        }
 #pragma unroll
-                            for (int i = 0; i < 4; ++i) {
-                                const unsigned long long tp = add2(mul2(dot[i], bits2(ss.x, ss.y)), bits2(ss.z, ss.w));
-                                t[i] = b == 0 ? tp : add2(t[i], tp);
-                            }
-                        } while (!PP && ++b < P);
+                        for (int i = 0; i < 4; ++i) {
+                            const unsigned long long tp = add2(mul2(dot[i], bits2(ss.x, ss.y)), bits2(ss.z, ss.w));
+                            t[i] = b == 0 ? tp : add2(t[i], tp);
+                        }
                     }
 #pragma unroll
                     for (int i = 0; i < 4; ++i) {
                         unsigned long long u = t[i];
                         if (HAS_ID) {
-                            const float2 f = __half22float2(*reinterpret_cast<const __half2 *>(&io[i][kk]));
+                            const float2 f = __half22float2(*reinterpret_cast<const __half2 *>(&io[i][ROLLED ? 0 : kk]));
                             u = add2(u, bits2(__float_as_uint(f.x), __float_as_uint(f.y)));
                         }
                         const float2 uf = floats2(u);
                         const __half2 y2 = __floats2half2_rn(prelu(uf.x, __uint_as_float(sn.x)), prelu(uf.y, __uint_as_float(sn.y)));
-                        io[i][kk] = *reinterpret_cast<const uint32_t *>(&y2);
-                        if (want_bits) sg4[i] |= __hge2_mask(y2, *reinterpret_cast<const __half2 *>(&sn.z)) & ((1u << (2 * kk)) | (2u << (16 + 2 * kk)));
+                        if (ROLLED) {
+                            io[i][0] = io[i][1];
+                            io[i][1] = io[i][2];
+                            io[i][2] = io[i][3];
+                        }
+                        io[i][ROLLED ? 3 : kk] = *reinterpret_cast<const uint32_t *>(&y2);
+                        if (want_bits) sg4[i] |= __hge2_mask(y2, *reinterpret_cast<const __half2 *>(&sn.z)) & (0x00020001u << (2 * kk));
                     }
                 }
 #pragma unroll
@@ -730,7 +736,15 @@ int launch_mod(ModPlan &L, bool shifted, cudaStream_t stream)
     case 2: return launch_plan<32, 2, false>(L, smem, stream);
     case 3: return launch_plan<32, 3, false>(L, smem, stream);
     case 4: return launch_plan<32, 4, false>(L, smem, stream);
-    default: return launch_plan<32, 0, false>(L, smem, stream);
+    case 5: return launch_plan<32, 5, false>(L, smem, stream);
+    case 6: return launch_plan<32, 6, false>(L, smem, stream);
+    case 7: return launch_plan<32, 7, false>(L, smem, stream);
+    case 8: return launch_plan<32, 8, false>(L, smem, stream);
+    case 9: return launch_plan<32, 9, false>(L, smem, stream);
+    case 10: return launch_plan<32, 10, false>(L, smem, stream);
+    case 11: return launch_plan<32, 11, false>(L, smem, stream);
+    case 12: return launch_plan<32, 12, false>(L, smem, stream);
+    default: return launch_plan<32, 13, false>(L, smem, stream);
     }
 }
 

@@ -43,6 +43,15 @@ def test_branches_longer_than_the_ring(bk, oracle, shape, variant):
     check_branches(bk, oracle, shape, variant)
 
 
+# every number of branches has a kernel of its own; one part a block and several, with and without an identity
+@pytest.mark.parametrize("variant", ["full", "no_identity"])
+@pytest.mark.parametrize("P", [5, 6, 7, 8, 9, 10, 11, 12, 13])
+def test_branches_each_number(bk, oracle, P, variant):
+    for shape in ((1, 13, 17, 32, 64, P), (2, 90, 107, 64, 96, P)):
+        assert bk.bcnn_branches_plan(*shape)[0] == 32
+        check_branches(bk, oracle, shape, variant)
+
+
 # the widest modules the engine takes: the packed weights lie over all staging tiles (960 channels) or all but the teams' first (1024)
 # until they are expanded; tiles behind those are used by the same launch
 @pytest.mark.parametrize("variant", ["full", "no_identity", "in_place"])
@@ -254,7 +263,7 @@ def test_stem_stages_handed_back_in_every_launch(bk):
 # the module's sign threshold and PReLU on values where a rounding, a sign of zero, an infinity or a NaN could go the other way: identities
 # and next biases from lists of such values in all combinations, on 32- and 64-channel parts with a half-empty last one
 @pytest.mark.parametrize("has_nb", [True, False])
-@pytest.mark.parametrize("P", [1, 2, 3, 4, 6])
+@pytest.mark.parametrize("P", [1, 2, 3, 4, 6, 11])
 @pytest.mark.parametrize("shape", [(1, 11, 13, 96), (1, 120, 161, 96)])
 def test_module_special_values(bk, oracle, shape, P, has_nb):
     B, H, W, C = shape
