@@ -56,7 +56,8 @@ constexpr int ERR_C3_ACC_TIMEOUT = 146;          // issuer: an accumulator was n
 
 constexpr int TH = 8, TW = 16;            // output tile (TH * TW = 128 = tensor-memory lanes)
 constexpr int NGRP = 2;                   // epilogue groups (alternate tiles)
-constexpr int NLD = 2;                    // loader warps (alternate tiles; four with half the ring each: 34.9 -> 36.3 us on the first 3x3/2 layer)
+constexpr int NLD = 2;                    // loader warps (alternate tiles: n & 1, n >> 1; four with half the ring each: 34.9 -> 36.3 us on the first 3x3/2 layer)
+static_assert(NLD == 2, "tile n: loader n & 1, its tile n >> 1");
 constexpr int NPG = 4;                    // producer groups of four warps
 constexpr int RD = 6;                     // halo tiles in a loader's ring
 constexpr int TAPS = 9, UWORDS = 10;      // K words of a unit: the nine taps and a zero
@@ -164,7 +165,7 @@ conv_tc_c3_kernel(const ConvProblem p, const C3Geom g, const __grid_constant__ C
     const uint32_t wexp = (smem_u32(smem_raw) + 1023u) & ~1023u;          // [KT][BN rows][128 B] expanded weights
     const uint32_t cexp = wexp + KT * C::W_TILE_BYTES;                    // [BN rows][128 B] constant rows (first 32 bytes)
     const uint32_t pops = cexp + C::W_TILE_BYTES;                         // [BN] bit counts
-    const uint32_t ring = pops + (BN * 4 + 127) / 128 * 128;              // [NGRP][RD] halo tiles
+    const uint32_t ring = pops + (BN * 4 + 127) / 128 * 128;              // [NLD][RD] halo tiles
     const uint32_t bar0 = smem_u32(bars);
     auto load_full = [&](int gr, int s) { return bar0 + 8u * (gr * RD + s); };
     auto load_empty = [&](int gr, int s) { return bar0 + 8u * (NLD * RD + gr * RD + s); };
@@ -272,30 +273,48 @@ conv_tc_c3_kernel(const ConvProblem p, const C3Geom g, const __grid_constant__ C
         const uint32_t sf = tmem_u + (uint32_t)CB_COL, c_lo = (uint32_t)make_desc(cexp);
         const uint32_t hf = NH == 2 ? __shfl_sync(0xffffffffu, (uint32_t)warp, 0) : 0u;
         const uint32_t w_lo = b_lo + hf * HALF_DESC;
-        if (elect_one()) {
-            for (int n = NH == 2 ? 0 : warp; n < my_tiles; n += NH == 2 ? 1 : C::NISS) {
-                if (!issuer_wait(a_full(n % NAF), (uint32_t)(n / NAF) & 1u, abort_flag, p.err, ERR_C3_ISSUER_TIMEOUT)) break;
-                // the epilogue has read the accumulator's previous tile
-                const int acc = NH == 2 ? (int)hf : n % NACC;
-                const int prev = NH == 2 ? n - 1 : n / NACC - 1;                 // completion of acc_free to wait for
-                if (prev >= 0 && !issuer_wait(acc_free(acc), (uint32_t)prev & 1u, abort_flag, p.err, ERR_C3_ACC_TIMEOUT)) break;
-                tc_fence_after();
-                const uint32_t d_t = tmem_u + (uint32_t)(acc * AW);
-                tc_mma_const(d_t, tmem_u, c_lo + hf * HALF_DESC, desc_hi, idesc);
+        auto issue = [&](int n) {
+            const uint32_t d_t = tmem_u + (uint32_t)((NH == 2 ? (int)hf : n % NACC) * AW);
+            tc_mma_const(d_t, tmem_u, c_lo + hf * HALF_DESC, desc_hi, idesc);
 #pragma unroll
-                for (int h = 0; h < CW; ++h) {
-                    const uint32_t a_t = tmem_u + (uint32_t)(C::A_COL0 + ((n * CW + h) % NUNIT) * U_COLS);
+            for (int h = 0; h < CW; ++h) {
+                const uint32_t a_t = tmem_u + (uint32_t)(C::A_COL0 + ((n * CW + h) % NUNIT) * U_COLS);
 #pragma unroll
-                    for (int t = 0; t < UWORDS / 2; ++t) {
-                        const int e = h * UWORDS + 2 * t;
-                        tc_mma_f4_ts(d_t, a_t + 8u * t, w_lo + (uint32_t)((e >> 3) * (C::W_TILE_BYTES >> 4) + (e & 7)),
-                                     desc_hi, idesc, sf, 1u);
-                    }
+                for (int t = 0; t < UWORDS / 2; ++t) {
+                    const int e = h * UWORDS + 2 * t;
+                    tc_mma_f4_ts(d_t, a_t + 8u * t, w_lo + (uint32_t)((e >> 3) * (C::W_TILE_BYTES >> 4) + (e & 7)),
+                                 desc_hi, idesc, sf, 1u);
                 }
-                tc_commit(tile_done((n * NH + (int)hf) % NB));
+            }
+            tc_commit(tile_done((n * NH + (int)hf) % NB));
+        };
+        constexpr int N_STEP = NH == 2 ? 1 : C::NISS;
+        // completion of acc_free to wait for: the epilogue has read the accumulator's previous tile
+        auto previous = [&](int n) { return NH == 2 ? n - 1 : n / NACC - 1; };
+        // One lane runs the loop where a tile is six short instructions, the whole warp, electing a lane per tile, where it is more of them or both
+        // halves wait for one accumulator each (us, one lane and the warp: 32 -> 32 at M = 3211264 34.6 and 36.0; 32 -> 96 at 1130040 30.7 and 28.3;
+        // 32 -> 128 at 1505280 38.4 and 35.8; 64 -> 64 /2 at 493950 16.4 and 15.2)
+        if constexpr (CW == 1 && NH == 1) {
+            if (elect_one()) {
+                for (int n = warp; n < my_tiles; n += N_STEP) {
+                    if (!issuer_wait(a_full(n % NAF), (uint32_t)(n / NAF) & 1u, abort_flag, p.err, ERR_C3_ISSUER_TIMEOUT)) break;
+                    const int prev = previous(n);
+                    if (prev >= 0 && !issuer_wait(acc_free(n % NACC), (uint32_t)prev & 1u, abort_flag, p.err, ERR_C3_ACC_TIMEOUT)) break;
+                    tc_fence_after();
+                    issue(n);
+                }
+            }
+            __syncwarp();
+        } else {
+            for (int n = NH == 2 ? 0 : warp; n < my_tiles; n += N_STEP) {
+                if (!pw_wait(a_full(n % NAF), (uint32_t)(n / NAF) & 1u, abort_flag, p.err, ERR_C3_ISSUER_TIMEOUT)) break;
+                const int prev = previous(n);
+                if (prev >= 0 && !pw_wait(acc_free(NH == 2 ? (int)hf : n % NACC), (uint32_t)prev & 1u, abort_flag, p.err, ERR_C3_ACC_TIMEOUT)) break;
+                tc_fence_after();
+                if (elect_one()) issue(n);
+                __syncwarp();
             }
         }
-        __syncwarp();
     } else if (warp < C::FIRST_PRODUCER_WARP) {
         // ------------------------------------------------------------------ loader of a group: one halo tile per TMA copy
         const int grp = warp - C::FIRST_LOADER_WARP;
@@ -387,9 +406,9 @@ conv_tc_c3_kernel(const ConvProblem p, const C3Geom g, const __grid_constant__ C
         const uint32_t t_lane = tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)C::A_COL0;
         const uint32_t lane0 = lane == 0 ? 1u : 0u;
         for (int n = n0; n < my_tiles; n += step) {
-            const int lg = n % NLD, stage = (n / NLD) % RD;
+            const int lg = n & 1, stage = (n >> 1) % RD;
             uint32_t wds[TAPS];
-            if (!pw_wait<64>(load_full(lg, stage), (uint32_t)(n / NLD / RD) & 1u, abort_flag, p.err, ERR_C3_PRODUCER_TIMEOUT)) break;
+            if (!pw_wait<64>(load_full(lg, stage), (uint32_t)((n >> 1) / RD) & 1u, abort_flag, p.err, ERR_C3_PRODUCER_TIMEOUT)) break;
             const uint32_t src = ring + (uint32_t)(lg * RD + stage) * (uint32_t)g.stage_bytes + my_off;
 #pragma unroll
             for (int tap = 0; tap < TAPS; ++tap)
