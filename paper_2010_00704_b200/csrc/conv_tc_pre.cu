@@ -71,6 +71,10 @@ template <int BN, int MODE, int G, int TEAMS, bool PAIR, bool RAW = false> struc
     static constexpr int PIECES = SPLIT ? 2 : 1, PC = EC / PIECES;        // pieces of a team's columns, columns of a piece
     static constexpr int MMA_N = SPLIT ? BN / 2 : BN;                     // columns of an instruction
     static constexpr int W_BYTES = BN / CTAS * ROWB;                      // one ring stage of weights
+    // a producer's next copies ahead of the wait for its oldest (three stages in flight), or behind its store (two, and the store's latency
+    // hidden).  us, ahead and behind: 128 wide 5x5 160 -> 128 at M = 336336 87.7 and 89.9, 128 -> 128 at 200704 17.1 and 17.2; 256 wide
+    // 256 -> 256 at 50176 13.2 and 13.0
+    static constexpr bool EARLY = BN < 256 && !RAW;
     static constexpr int SF_COL = 512 - (int)SF_COLS;                     // unit scales
     static constexpr int BITS_BYTES = PF * PROD_THREADS * 32;
     static constexpr int TABLE_BYTES = EPI_WARPS * EC * 4;                // one column table per epilogue warp
@@ -300,23 +304,30 @@ conv_tc_pre_kernel(const ConvProblem p, const int32_t *cst, const __grid_constan
         // CTAs' bytes, and both complete on its barrier.
         int s = 0, it = 0;
         uint32_t phase = 1;                           // first pass through the ring: slots are free
+        bool ok = true;
         TilePos at = walk.first(unit);
         pdl_wait();
-        for (int kt = 0; it < total_items; ++it) {
-            if (!mbar_wait_warp(empty_bar(s), phase, abort_flag, p.err, ERR_LOADER_TIMEOUT)) break;
-            if (lane == 0) {
-                const uint32_t dst = wring + (uint32_t)s * C::W_BYTES;
-                if (rank == 0) asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(full_bar(s)), "r"((uint32_t)(C::CTAS * C::W_BYTES)) : "memory");
-                if (PAIR)
-                    asm volatile("cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes.cta_group::2 [%0], [%1, {%2, %3, %4, %5}], [%6];"
-                                 ::"r"(dst), "l"(reinterpret_cast<uint64_t>(&wmap)), "r"(kt * ROWB), "r"(0), "r"(rank), "r"(at.n * (BN / 128)), "r"(in_even_cta(full_bar(s))) : "memory");
-                else
-                    asm volatile("cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
-                                 ::"r"(dst), "l"(reinterpret_cast<uint64_t>(&wmap)), "r"(kt * ROWB), "r"(at.n * BN), "r"(full_bar(s)) : "memory");
+        // (a tile's coordinates outside of its stages: this warp's loop is what bounds long K on narrow tiles - 3x3 768 -> 64 at M = 487500
+        // 158 us with one loop over all items, 140 as it is)
+        for (int ti = 0; ti < my_tiles && ok; ++ti, walk.next(at)) {
+            const int row = at.n * (PAIR ? BN / 128 : BN);
+            for (int kt = 0; kt < ktiles; ++kt) {
+                ok = mbar_wait_warp(empty_bar(s), phase, abort_flag, p.err, ERR_LOADER_TIMEOUT);
+                if (!ok) break;
+                if (lane == 0) {
+                    const uint32_t dst = wring + (uint32_t)s * C::W_BYTES;
+                    if (rank == 0) asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(full_bar(s)), "r"((uint32_t)(C::CTAS * C::W_BYTES)) : "memory");
+                    if (PAIR)
+                        asm volatile("cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes.cta_group::2 [%0], [%1, {%2, %3, %4, %5}], [%6];"
+                                     ::"r"(dst), "l"(reinterpret_cast<uint64_t>(&wmap)), "r"(kt * ROWB), "r"(0), "r"(rank), "r"(row), "r"(in_even_cta(full_bar(s))) : "memory");
+                    else
+                        asm volatile("cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
+                                     ::"r"(dst), "l"(reinterpret_cast<uint64_t>(&wmap)), "r"(kt * ROWB), "r"(row), "r"(full_bar(s)) : "memory");
+                }
+                __syncwarp();
+                ++it;
+                if (++s == STAGES) { s = 0; phase ^= 1u; }
             }
-            __syncwarp();
-            if (++kt == ktiles) { kt = 0; walk.next(at); }
-            if (++s == STAGES) { s = 0; phase ^= 1u; }
         }
         // after a time-out elsewhere: copies still in flight must land before the CTA's shared memory goes away
         if (*abort_flag && rank == 0) {
@@ -578,7 +589,13 @@ conv_tc_pre_kernel(const ConvProblem p, const int32_t *cst, const __grid_constan
         int c_kt = grp, c_ti = 0, n_bits = 0; // raw weights: the stage within its tile, the tile, the row's bits so far
 #pragma unroll 1
         for (int it = grp; it < total_items; it += G) {
-            cp_async_wait<PF - 2>();
+            if (C::EARLY) {
+                if (l_left > 0) issue_load();
+                cp_async_commit();
+                cp_async_wait<PF - 1>();
+            } else {
+                cp_async_wait<PF - 2>();
+            }
             const uint4 q0 = ld_shared_v4(c_src), q1 = ld_shared_v4(c_src + HALF_BYTES);
             c_src += SLOT_BYTES;
             if (c_src == bits_end) c_src = bits0;
@@ -592,8 +609,10 @@ conv_tc_pre_kernel(const ConvProblem p, const int32_t *cst, const __grid_constan
                     expand_a4(wds[e], v);
                     st_shared_v4(row_addr + (uint32_t)((e ^ (row & 7)) << 4), v[0], v[1], v[2], v[3]);
                 }
-                if (l_left > 0) issue_load();
-                cp_async_commit();
+                if (!C::EARLY) {
+                    if (l_left > 0) issue_load();
+                    cp_async_commit();
+                }
                 fence_async_proxy();          // generic stores -> the MMAs
             } else {
                 uint32_t v[32];
@@ -617,9 +636,10 @@ conv_tc_pre_kernel(const ConvProblem p, const int32_t *cst, const __grid_constan
                 if (!mbar_wait_warp(empty_bar(s), phase, abort_flag, p.err, ERR_PRODUCER_TIMEOUT)) break;
                 tc_fence_after();             // the MMAs that read this slot are complete (their commit released it)
                 tc_st32_nowait(st_addr0 + (uint32_t)s * 32u, v);
-                // the next copies are issued while the store completes
-                if (l_left > 0) issue_load();
-                cp_async_commit();
+                if (!C::EARLY) {              // the next copies are issued while the store completes
+                    if (l_left > 0) issue_load();
+                    cp_async_commit();
+                }
                 tc_wait_st();
                 tc_fence_before();
             }
