@@ -53,8 +53,9 @@ constexpr int ERR_EPILOGUE_TIMEOUT = 133;
 constexpr int ERR_LOADER_TIMEOUT = 134;
 
 // BN: output channels of a tile; MODE: 0 int32, 1 packed output; G: activation producer groups of four warps; TEAMS: epilogue
-// teams of four warps, each with its share of a tile's columns
-template <int BN, int MODE, int G, int TEAMS, bool PAIR, bool RAW = false> struct Cfg {
+// teams of four warps, each with its share of a tile's columns; WHOLE: a 256-wide tile handed over in one piece, each team 128
+// consecutive columns, which go to memory one after the other
+template <int BN, int MODE, int G, int TEAMS, bool PAIR, bool RAW = false, bool WHOLE = false> struct Cfg {
     static constexpr int EPI_WARPS = 4 * TEAMS;
     static constexpr int NBUF = BN == 256 ? 1 : (BN == 128 ? 2 : 4);     // accumulator buffers
     static constexpr int A_COL0 = NBUF * BN;                              // first column of the activation ring
@@ -67,7 +68,7 @@ template <int BN, int MODE, int G, int TEAMS, bool PAIR, bool RAW = false> struc
     static constexpr int LOADER_WARP = FIRST_PRODUCER_WARP + G * GROUP_WARPS;
     static constexpr int THREADS = 32 * (LOADER_WARP + (RAW ? 0 : 1));
     static constexpr int EC = BN / TEAMS;                                 // columns of a team
-    static constexpr bool SPLIT = BN == 256;                              // one accumulator, handed over in halves of 128 columns
+    static constexpr bool SPLIT = BN == 256 && !WHOLE;                    // one accumulator, handed over in halves of 128 columns
     static constexpr int PIECES = SPLIT ? 2 : 1, PC = EC / PIECES;        // pieces of a team's columns, columns of a piece
     static constexpr int MMA_N = SPLIT ? BN / 2 : BN;                     // columns of an instruction
     static constexpr int W_BYTES = BN / CTAS * ROWB;                      // one ring stage of weights
@@ -136,11 +137,11 @@ __host__ __device__ constexpr int smem_bytes(int ktab_words, int mode)
 // RAW: the weights are packed bits, expanded on the way; then the activations are the signed operand and the weights the unsigned one,
 //   sum a*g = accumulator + K - 2 popc(a):
 // a constant per row, which the warps that expand the row count, and none that the two CTAs of a pair would have to exchange.
-template <int BN, int MODE, int G, int TEAMS, bool PAIR, bool RAW>
-__global__ void __launch_bounds__(Cfg<BN, MODE, G, TEAMS, PAIR, RAW>::THREADS, 1)
+template <int BN, int MODE, int G, int TEAMS, bool PAIR, bool RAW, bool WHOLE>
+__global__ void __launch_bounds__(Cfg<BN, MODE, G, TEAMS, PAIR, RAW, WHOLE>::THREADS, 1)
 conv_tc_pre_kernel(const ConvProblem p, const int32_t *cst, const __grid_constant__ CUtensorMap wmap, const int ktab_words, const TileWalk walk)
 {
-    using C = Cfg<BN, MODE, G, TEAMS, PAIR, RAW>;
+    using C = Cfg<BN, MODE, G, TEAMS, PAIR, RAW, WHOLE>;
     constexpr int EPI_WARPS = C::EPI_WARPS, EC = C::EC;
     constexpr bool FUSED = MODE == 1;
     constexpr int NBUF = C::NBUF;
@@ -685,11 +686,21 @@ prepare_weights_kernel(const uint32_t *w, uint8_t *wexp, int32_t *cst, int N, in
 
 int ktab_words_for(const ConvProblem &p) { return ((p.kwords + 7) >> 3) * (8 / gather_width(p.cw)); }
 
+// int32 rows that are no whole number of 32-byte sectors: the sectors at the tile columns' borders and at the ends of the rows are written
+// by two tiles.  With a column of tiles finished before the next is begun they leave the second-level cache half written and come back
+// (300000 x 218 x 384: 57 MB read where the operands are 14; 314286 x 364 x 64 191 -> 117 us across the columns, 126000 x 507 x 576 120 -> 74,
+// 150000 x 756 x 128 163 -> 113).  Up to an eighth as many columns as blocks: a grid that is a multiple of them leaves some idle.
+template <int MODE>
+bool walk_across(const ConvProblem &p, long n_tiles, long units)
+{
+    return MODE == 0 && (p.C_out & 7) != 0 && n_tiles > 1 && 8 * n_tiles <= units;
+}
+
 // pw.wexp == nullptr where the weights are raw (RAW)
-template <int BN, int MODE, int G, int TEAMS, bool PAIR, bool RAW = false>
+template <int BN, int MODE, int G, int TEAMS, bool PAIR, bool RAW = false, bool WHOLE = false>
 int launch_bn(const ConvProblem &p0, const PreparedWeights &pw, cudaStream_t stream)
 {
-    using C = Cfg<BN, MODE, G, TEAMS, PAIR, RAW>;
+    using C = Cfg<BN, MODE, G, TEAMS, PAIR, RAW, WHOLE>;
     ConvProblem p = p0;
     p.err = device_error_word();
     const long units = sm_count() / C::CTAS;
@@ -697,7 +708,9 @@ int launch_bn(const ConvProblem &p0, const PreparedWeights &pw, cudaStream_t str
     const long n_tiles = ((long)p.C_out + BN - 1) / BN;
     const long total = m_tiles * n_tiles;
     if (total >= (1L << 31)) return BCNN_ERR_UNSUPPORTED;
-    const int grid = (int)(total < units ? total : units);
+    const bool across = walk_across<MODE>(p, n_tiles, units);
+    const long rows = across ? (m_tiles < units / n_tiles ? m_tiles : units / n_tiles) : 0;
+    const int grid = (int)(across ? rows * n_tiles : total < units ? total : units);
     const int ktw = ktab_words_for(p);
     const int smem = smem_bytes<C>(ktw, MODE);
     if (smem > MAX_SMEM) return BCNN_ERR_UNSUPPORTED;
@@ -715,9 +728,9 @@ int launch_bn(const ConvProblem &p0, const PreparedWeights &pw, cudaStream_t str
                    CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
             return BCNN_ERR_CUDA;
     }
-    auto k = conv_tc_pre_kernel<BN, MODE, G, TEAMS, PAIR, RAW>;
+    auto k = conv_tc_pre_kernel<BN, MODE, G, TEAMS, PAIR, RAW, WHOLE>;
     if (!allow_smem((const void *)k, MAX_SMEM)) return BCNN_ERR_CUDA;
-    return launch<C::CTAS>(k, (unsigned)(grid * C::CTAS), C::THREADS, smem, stream, p, pw.cst, wmap, ktw, make_tile_walk(p, C::TILE_ROWS, (int)m_tiles, (int)total, grid));
+    return launch<C::CTAS>(k, (unsigned)(grid * C::CTAS), C::THREADS, smem, stream, p, pw.cst, wmap, ktw, make_tile_walk(p, C::TILE_ROWS, (int)m_tiles, (int)n_tiles, grid, across));
 }
 
 }  // namespace
@@ -829,6 +842,11 @@ int launch_conv_tc_pre(const ConvProblem &p, const void *prepared, cudaStream_t 
     static_assert(smem_bytes<Cfg<256, 0, 2, 2, true>>(0, 0) <= smem_bytes<Cfg<256, 0, 2, 2, false>>(0, 0) && smem_bytes<Cfg<256, 1, 2, 2, true>>(0, 1) <= smem_bytes<Cfg<256, 1, 2, 2, false>>(0, 1),
                   "and the tile of two blocks");
     const bool fits256 = packed || smem_bytes<Cfg<256, 0, 2, 2, false>>(ktab_words_for(p), 0) <= MAX_SMEM;
+    // One column of tiles, int32 rows of no whole sectors and more of them than the second-level cache holds: whole rows at a time (us, tiles of 128 and
+    // whole: 300000 x 218 x 384 109 and 71, 500000 x 146 x 768 149 and 108, 350000 x 201 x 1152 120 and 104; 300000 x 250 x 384 84 and 84, but in the
+    // cache 100000 x 218 x 384 26.0 and 27.6, and 300000 x 243 x 64, one stage, 83 and 98)
+    if (!packed && fits256 && kt > 1 && p.C_out > 128 && p.C_out <= 256 && (p.C_out & 7) != 0 && (long)p.M * p.C_out >= 1L << 25)
+        return launch_bn<256, 0, 2, 2, false, false, true>(p, pw, stream);
     long c256 = LONG_MAX, c128, c64;
     if (packed) {
         c64 = cost(64, 2150, 160, wide_gather ? 212 : 330);

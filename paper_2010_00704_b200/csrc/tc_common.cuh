@@ -353,21 +353,25 @@ __host__ __device__ __forceinline__ TileStep make_tile_step(const ConvProblem &p
     s.pointwise = p.kh == 1 && p.kw == 1 && p.stride == 1 && p.pad == 0;
     return s;
 }
-// A persistent CTA's way through the tiles (n, m), m fastest: from tile blockIdx.x in steps of gridDim.x.  All divisions are the
-// host's: an integer division is some twenty instructions, and in code that runs once an instruction costs some ten cycles.
+// A persistent CTA's way through the tiles (n, m), m fastest: from tile blockIdx.x in steps of gridDim.x.  Or ACROSS the columns:
+// blocks beside one another take the tile columns of the same rows, a CTA keeps its column (the grid is a multiple of their
+// number).  All divisions are the host's: an integer division is some twenty instructions, and in code that runs once an instruction
+// costs some ten cycles.
 struct TilePos {
     int n, m;
 };
 struct TileWalk {
     int m_tiles, tiles, extra;       // row tiles; every CTA's tiles, and the number of CTAs that have one more
-    int dn, dm;                      // gridDim.x = dn * m_tiles + dm
-    uint32_t mul, shift;             // exact_div by m_tiles
+    int dn, dm;                      // gridDim.x = dn * m_tiles + dm (across: 0, the columns' share of gridDim.x)
+    int d;                           // m_tiles (across: the number of columns)
+    uint32_t mul, shift;             // exact_div by d
+    bool across;
     TileStep step;                   // of the rows of two consecutive tiles, as long as n does not change
     __device__ __forceinline__ int tiles_of(int cta) const { return tiles + (cta < extra ? 1 : 0); }
     __device__ __forceinline__ TilePos first(int cta) const
     {
-        const int n = (int)exact_div((uint32_t)cta, mul, shift);
-        return {n, cta - n * m_tiles};
+        const int q = (int)exact_div((uint32_t)cta, mul, shift), r = cta - q * d;
+        return across ? TilePos{r, q} : TilePos{q, r};
     }
     // true where the next tile's rows are not `step` behind the last one's
     __device__ __forceinline__ bool next(TilePos &t) const
@@ -379,16 +383,19 @@ struct TileWalk {
         return wrap || dn > 0;
     }
 };
-inline TileWalk make_tile_walk(const ConvProblem &p, int tile_rows, int m_tiles, int total, int grid)
+inline TileWalk make_tile_walk(const ConvProblem &p, int tile_rows, int m_tiles, int n_tiles, int grid, bool across)
 {
     TileWalk w;
+    const int total = m_tiles * n_tiles, rows = across ? grid / n_tiles : grid;       // row tiles from one of a CTA's tiles to its next
     w.m_tiles = m_tiles;
-    w.tiles = total / grid;
-    w.extra = total % grid;
-    w.dn = grid / m_tiles;
-    w.dm = grid % m_tiles;
-    exact_div_params((uint32_t)m_tiles, w.mul, w.shift);
-    w.step = make_tile_step(p, (uint32_t)tile_rows * (uint32_t)grid);
+    w.tiles = across ? m_tiles / rows : total / grid;
+    w.extra = across ? m_tiles % rows * n_tiles : total % grid;
+    w.dn = across ? 0 : grid / m_tiles;
+    w.dm = across ? rows : grid % m_tiles;
+    w.d = across ? n_tiles : m_tiles;
+    w.across = across;
+    exact_div_params((uint32_t)w.d, w.mul, w.shift);
+    w.step = make_tile_step(p, (uint32_t)tile_rows * (uint32_t)rows);
     return w;
 }
 struct RowCursor {

@@ -313,6 +313,13 @@ def test_prepared_one_stage_int32(bk, oracle, M, N, K):
     test_prepared_widths(bk, oracle, M, N, K, False)
 
 
+# int32 rows of no whole sectors: tiles across their columns (two, three and eighteen of them, rows left over in the last round of
+# row tiles), and whole rows by 256-wide tiles in one piece, K of one stage, two and several
+@pytest.mark.parametrize("M,N,K", [(40000, 364, 64), (20000, 255, 288), (30100, 397, 1184), (2500, 2300, 96), (300, 1021, 4640), (262200, 131, 256), (150003, 250, 416), (135000, 253, 2336)])
+def test_prepared_ragged_int32_rows(bk, oracle, M, N, K):
+    test_prepared_widths(bk, oracle, M, N, K, False)
+
+
 # the tiled product with its K over two, four and eight blocks (the last of them without a chunk), ragged in images, outputs and K; tiles of 32 and 64
 # outputs in one wave, alone on their multiprocessors, and in several, two on each; few images, tiled and streamed
 @pytest.mark.parametrize("shape", [(64, 2048, 100), (97, 1156, 130), (130, 516, 700), (200, 2052, 1000), (300, 264, 65), (61, 1100, 513), (256, 2048, 10),
