@@ -277,6 +277,14 @@ int bcnn_conv2d_b1_fused_noalloc(const void *x_bits, const void *w_bits, const i
 int bcnn_auto_engine(int B, int H, int W, int C_in, int C_out, int kh, int kw, int stride, int pad, int fused);
 
 /*
+ * How the streaming engine runs a convolution of this shape on prepared weights (prepared != 0) or on packed ones, six values
+ * into plan[]: output channels of a tile, blocks that share one, 1 where its columns are handed over in one piece, whose bits are
+ * counted on the way (0 nobody's, 1 the weights', 2 the activations'), 256-bit stages of K, the most tiles a block runs.  For tests
+ * that have to reach a certain path.  No pointers but plan, no launch; a negative bcnn_status for a shape it does not take.
+ */
+int bcnn_stream_plan(int prepared, int B, int H, int W, int C_in, int C_out, int kh, int kw, int stride, int pad, int fused, int *plan);
+
+/*
  * How bcnn_conv2d_b1_branches runs a module of this shape, five values into plan[]: output channels of one part of the
  * tensor-core module engine (64 or 32; 0: the module runs on the CUDA cores), slices of that many channels whose weights a
  * block keeps, 256-bit stages of a row, slots of the ring that holds them, and how many staging tiles do not wait for the

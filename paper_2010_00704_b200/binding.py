@@ -24,7 +24,7 @@ EXPORTS = (
     "bcnn_conv2d_b1_branches", "bcnn_dwconv3x3_module", "bcnn_avgpool", "bcnn_gap", "bcnn_fc",
     "bcnn_prepared_weights_bytes", "bcnn_prepare_weights", "bcnn_conv2d_b1_prepared", "bcnn_gemm_b1_prepared", "bcnn_prepared_preferred",
     "bcnn_conv2d_b1_fused_noalloc",
-    "bcnn_conv2d_b1_engine", "bcnn_gemm_b1_engine", "bcnn_auto_engine", "bcnn_branches_plan", "bcnn_device_error", "bcnn_device_status",
+    "bcnn_conv2d_b1_engine", "bcnn_gemm_b1_engine", "bcnn_auto_engine", "bcnn_branches_plan", "bcnn_stream_plan", "bcnn_device_error", "bcnn_device_status",
     "bcnn_workspace_bytes", "bcnn_selftest_wait_timeout", "bcnn_status_string", "bcnn_version",
 )
 
@@ -73,6 +73,7 @@ def load() -> ctypes.CDLL:
         lib.bcnn_gemm_b1_engine.argtypes = [i32, vp, vp, vp, vp, i64, i32, i32, vp]
         lib.bcnn_auto_engine.argtypes = [i32] * 10
         lib.bcnn_branches_plan.argtypes = [i32] * 8 + [ctypes.POINTER(i32)]
+        lib.bcnn_stream_plan.argtypes = [i32] * 11 + [ctypes.POINTER(i32)]
         lib.bcnn_device_error.argtypes = []
         lib.bcnn_device_status.argtypes = [ctypes.POINTER(ctypes.c_int)]
         lib.bcnn_workspace_bytes.argtypes = [i32] * 10
@@ -256,6 +257,13 @@ def bcnn_branches_plan(B, H, W, C_in, C_out, P, kh=1, kw=1):
     """(channels of a part, resident slices, stages of a row, ring slots, staging tiles that do not wait); 0 channels: CUDA cores."""
     plan = (ctypes.c_int * 5)()
     _check(load().bcnn_branches_plan(B, H, W, C_in, C_out, P, kh, kw, plan), "bcnn_branches_plan")
+    return tuple(plan)
+
+
+def bcnn_stream_plan(prepared, B, H, W, C_in, C_out, kh, kw, stride, pad, fused=True):
+    """(channels of a tile, blocks on one, in one piece, whose bits are counted, stages of K, most tiles of a block)."""
+    plan = (ctypes.c_int * 6)()
+    _check(load().bcnn_stream_plan(1 if prepared else 0, B, H, W, C_in, C_out, kh, kw, stride, pad, 1 if fused else 0, plan), "bcnn_stream_plan")
     return tuple(plan)
 
 

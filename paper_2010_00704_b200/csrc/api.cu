@@ -488,6 +488,21 @@ int bcnn_auto_engine(int B, int H, int W, int C_in, int C_out, int kh, int kw, i
     return auto_engine(p);
 }
 
+int bcnn_stream_plan(int prepared, int B, int H, int W, int C_in, int C_out, int kh, int kw, int stride, int pad, int fused, int *plan)
+{
+    if (!plan) return BCNN_ERR_INVALID_ARG;
+    ConvProblem p;
+    void *dummy = reinterpret_cast<void *>(uintptr_t(4096));
+    const int st = make_conv_problem(p, dummy, dummy, fused ? static_cast<const int32_t *>(dummy) : nullptr, dummy,
+                                     B, H, W, C_in, C_out, kh, kw, stride, pad, fused != 0);
+    if (st != BCNN_OK) return st;
+    if (!(prepared ? conv_tc_pre_supports(p) : conv_tc_i8_supports(p))) return BCNN_ERR_UNSUPPORTED;
+    int v[6];
+    conv_tc_stream_plan(p, !prepared, v);
+    for (int i = 0; i < 6; ++i) plan[i] = v[i];
+    return BCNN_OK;
+}
+
 int bcnn_device_error(void)
 {
     int v = 0;

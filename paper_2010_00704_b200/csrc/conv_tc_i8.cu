@@ -31,7 +31,6 @@ constexpr int EPI_WARPS = 4;
 constexpr int G = 2;                      // producer groups
 constexpr int PF = 3;                     // packed-word stages in flight per producer thread
 constexpr int MAX_SMEM = 227 * 1024 - 512; // dynamic shared memory available beside the static part
-constexpr int MAX_KTAB = 1920;            // units of the gather's table that every variant has room for
 
 constexpr int ERR_PRODUCER_TIMEOUT = 101;
 constexpr int ERR_MMA_TIMEOUT = 102;
@@ -450,7 +449,7 @@ bool conv_tc_i8_supports(const ConvProblem &p)
     if (p.mode != 0 && (p.C_out % 32 != 0)) return false;
     if (p.kh * p.kw > 31) return false;                       // one validity bit per tap
     if ((long)p.B * p.H * p.W * p.cw >= (1L << 31)) return false;     // rows address the input by 32-bit word offsets
-    if (ktab_words_for(p) > MAX_KTAB) return false;           // the K-word table of the gather must fit
+    if (ktab_words_for(p) > MAX_RAW_KTAB) return false;           // the K-word table of the gather must fit
     if ((long)p.kh * p.W * p.cw >= (1L << 27)) return false;  // a unit's word offset within the window
     return p.K <= (1 << 20);                                  // sums up to 4 K + 2 stay exact in fp32
 }

@@ -52,10 +52,13 @@ constexpr int ERR_MMA_TIMEOUT = 132;
 constexpr int ERR_EPILOGUE_TIMEOUT = 133;
 constexpr int ERR_LOADER_TIMEOUT = 134;
 
+// where the weights are raw: the operand whose bits are signed and counted, hence what the constants belong to
+constexpr int RAW_COLUMNS = 1, RAW_ROWS = 2;
+
 // BN: output channels of a tile; MODE: 0 int32, 1 packed output; G: activation producer groups of four warps; TEAMS: epilogue
 // teams of four warps, each with its share of a tile's columns; WHOLE: a 256-wide tile handed over in one piece, each team 128
 // consecutive columns, which go to memory one after the other
-template <int BN, int MODE, int G, int TEAMS, bool PAIR, bool RAW = false, bool WHOLE = false> struct Cfg {
+template <int BN, int MODE, int G, int TEAMS, bool PAIR, int RAW = 0, bool WHOLE = false> struct Cfg {
     static constexpr int EPI_WARPS = 4 * TEAMS;
     static constexpr int NBUF = BN == 256 ? 1 : (BN == 128 ? 2 : 4);     // accumulator buffers
     static constexpr int A_COL0 = NBUF * BN;                              // first column of the activation ring
@@ -79,8 +82,12 @@ template <int BN, int MODE, int G, int TEAMS, bool PAIR, bool RAW = false, bool 
     static constexpr int SF_COL = 512 - (int)SF_COLS;                     // unit scales
     static constexpr int BITS_BYTES = PF * PROD_THREADS * 32;
     static constexpr int TABLE_BYTES = EPI_WARPS * EC * 4;                // one column table per epilogue warp
-    static constexpr int SLOTS = STAGES + NBUF + 2;                       // raw weights: tiles whose rows' bit counts are kept
-    static constexpr int POP_BYTES = RAW ? SLOTS * G * BM * 4 : 0;
+    // raw weights: tiles whose bit counts are kept - those with an accumulator, those in the ring, and one per group that has counted but
+    // waits for a slot; a count per row of the operand that is signed
+    static constexpr bool SIGNED_A = RAW == RAW_ROWS;
+    static_assert(!PAIR || RAW != RAW_COLUMNS, "a pair's column constants would have to be exchanged");
+    static constexpr int SLOTS = STAGES + NBUF + G, POP_ROWS = SIGNED_A ? BM : BN;
+    static constexpr int POP_BYTES = RAW ? SLOTS * G * POP_ROWS * 4 : 0;
     static_assert(A_COL0 + STAGES * 32 <= SF_COL, "tensor memory budget");
     static_assert(STAGES >= G, "a producer group must not lap the ring (parity waits)");
 };
@@ -134,16 +141,20 @@ __host__ __device__ constexpr int smem_bytes(int ktab_words, int mode)
            (mode == 0 ? C::EPI_WARPS * I32_TILE_BYTES + 16 : 0);
 }
 
-// RAW: the weights are packed bits, expanded on the way; then the activations are the signed operand and the weights the unsigned one,
+// RAW: the weights are packed bits, expanded on the way by warps that count a row's bits as they go.  RAW_COLUMNS: weights signed and activations
+// plain as above, K - 2 popc(W_n) per column.  RAW_ROWS: the other way round,
 //   sum a*g = accumulator + K - 2 popc(a):
-// a constant per row, which the warps that expand the row count, and none that the two CTAs of a pair would have to exchange.
-template <int BN, int MODE, int G, int TEAMS, bool PAIR, bool RAW, bool WHOLE>
+// a constant per row, for pairs of CTAs (which would have to exchange column constants) and where the activation warps have the time.  A signed
+// word is seven operations and its count, a plain one five: us with columns and rows, 3x3/2 2048 -> 32 at M = 162288 184 and 206, 1x1 96 -> 352
+// at 18177 (one stage) 7.7 and 8.8, 300 x 4000 x 9216 on 128-wide tiles 18.6 and 17.0.
+template <int BN, int MODE, int G, int TEAMS, bool PAIR, int RAW, bool WHOLE>
 __global__ void __launch_bounds__(Cfg<BN, MODE, G, TEAMS, PAIR, RAW, WHOLE>::THREADS, 1)
 conv_tc_pre_kernel(const ConvProblem p, const int32_t *cst, const __grid_constant__ CUtensorMap wmap, const int ktab_words, const TileWalk walk)
 {
     using C = Cfg<BN, MODE, G, TEAMS, PAIR, RAW, WHOLE>;
     constexpr int EPI_WARPS = C::EPI_WARPS, EC = C::EC;
-    constexpr bool FUSED = MODE == 1;
+    constexpr bool FUSED = MODE == 1, COLUMN_COUNTS = RAW == RAW_COLUMNS;       // column constants from counts of the weights' bits
+    static_assert(!COLUMN_COUNTS || !C::SPLIT, "one piece: the counts are read once per tile");
     constexpr int NBUF = C::NBUF;
     constexpr int STAGES = C::STAGES;
 
@@ -166,7 +177,7 @@ conv_tc_pre_kernel(const ConvProblem p, const int32_t *cst, const __grid_constan
     const uint32_t wring = (smem_u32(smem_raw) + 1023u) & ~1023u;         // [STAGES][BN rows][128 B], written by TMA
     const uint32_t bits_ring = wring + STAGES * C::W_BYTES;               // [PF][2][PROD_THREADS][16 B]
     const uint32_t tables = bits_ring + C::BITS_BYTES;                    // [EPI_WARPS][EC] column constants
-    const uint32_t pops = tables + C::TABLE_BYTES;                        // [SLOTS][G][BM] bit counts of activation rows
+    const uint32_t pops = tables + C::TABLE_BYTES;                        // [SLOTS][G][POP_ROWS] bit counts
     const uint32_t ktab_addr = pops + C::POP_BYTES;                       // unit table of the gather
     const uint32_t i32_tiles = (ktab_addr + (uint32_t)ktab_words * 4u + 15u) & ~15u;   // int32 output: store staging tiles
     const uint32_t bar0 = smem_u32(bars);
@@ -374,22 +385,48 @@ conv_tc_pre_kernel(const ConvProblem p, const int32_t *cst, const __grid_constan
             const int n_base = at.n * BN + team * PC;                           // first column of this team's first piece
             const int em = at.m * C::TILE_ROWS + rank * BM + erow;
             // the column constants, built while the tile's MMAs run, anew only where the columns change; every warp keeps its own table,
-            // so the four warps need no barrier among themselves
-            if (at.n != table_n) {
+            // so the four warps need no barrier among themselves.  Where the weights' bits are counted on the way the counts come with
+            // the tile: then only what belongs to the thresholds is fetched here.
+            constexpr int PER = EC / 32;
+            int cc[COLUMN_COUNTS ? PER : 1];
+            const bool new_columns = at.n != table_n;
+            if (new_columns) {
                 table_n = at.n;
                 __syncwarp();
-#pragma unroll 1
-                for (int c = lane; c < EC; c += 32) {
+                auto constant = [&](int c) {
                     const int n = n_base + (c / PC) * (BN / 2) + c % PC;
                     int v = 0;
                     if (n < p.C_out) {
                         if (!RAW) v = __ldg(cst + n);
+                        if (COLUMN_COUNTS) v = p.K;
                         if (FUSED) v -= max(min(__ldg(p.thr + n), p.K + 1), -p.K - 1);       // beyond that bound the decision is constant
                     }
-                    asm volatile("st.shared.b32 [%0], %1;" ::"r"(table + 4u * c), "r"(table_entry<MODE>(v)) : "memory");
+                    return v;
+                };
+                if constexpr (COLUMN_COUNTS) {
+#pragma unroll
+                    for (int i = 0; i < PER; ++i) cc[i] = constant(lane + 32 * i);
+                } else {
+#pragma unroll 1
+                    for (int c = lane; c < EC; c += 32) asm volatile("st.shared.b32 [%0], %1;" ::"r"(table + 4u * c), "r"(table_entry<MODE>(constant(c))) : "memory");
                 }
                 __syncwarp();
             }
+            // the bits of row r of the signed operand: the counts of the groups that had a stage of the tile
+            auto counted = [&](int r) {
+                const uint32_t at_pop = pops + (uint32_t)((ti % C::SLOTS) * G * C::POP_ROWS + r) * 4u;
+                const int first = (ti * ktiles) % G;
+                int n_bits = 0;
+#pragma unroll
+                for (int g = 0; g < G; ++g) {
+                    if ((g >= first ? g - first : g - first + G) < ktiles) {
+                        int v;
+                        asm volatile("ld.shared.b32 %0, [%1];" : "=r"(v) : "r"(at_pop + (uint32_t)(g * C::POP_ROWS) * 4u) : "memory");
+                        n_bits += v;
+                    }
+                }
+                return n_bits;
+            };
             const long row0 = (long)em - lane;
             uint32_t packed[MODE == 0 ? PIECES : 1][CH][16];                    // int32 outputs of a 256-wide tile, two to a register
 #pragma unroll
@@ -408,21 +445,14 @@ conv_tc_pre_kernel(const ConvProblem p, const int32_t *cst, const __grid_constan
                     else if (lane == 0) mbar_arrive(tempty0 + 8u * b);
                 };
                 float row_cst = 0.f;
-                if (RAW) {                                                      // the row's constant: the bit counts of the groups that had a stage of the tile
-                    const uint32_t at_pop = pops + (uint32_t)((ti % C::SLOTS) * G * BM + erow) * 4u;
-                    int n_bits = 0;
+                if (C::SIGNED_A) row_cst = (float)(p.K - 2 * counted(erow));
+                if (COLUMN_COUNTS && new_columns) {
 #pragma unroll
-                    for (int g = 0; g < G; ++g) {
-                        const int first = (ti * ktiles) % G;
-                        if ((g >= first ? g - first : g - first + G) < ktiles) {
-                            int v;
-                            asm volatile("ld.shared.b32 %0, [%1];" : "=r"(v) : "r"(at_pop + (uint32_t)(g * BM) * 4u) : "memory");
-                            n_bits += v;
-                        }
-                    }
-                    row_cst = (float)(p.K - 2 * n_bits);
+                    for (int i = 0; i < PER; ++i)
+                        asm volatile("st.shared.b32 [%0], %1;" ::"r"(table + 4u * (lane + 32 * i)), "r"(table_entry<MODE>(cc[i] - 2 * counted(team * EC + lane + 32 * i))) : "memory");
+                    __syncwarp();
                 }
-                if (FUSED && RAW) {
+                if (FUSED && C::SIGNED_A) {
                     uint32_t words[CH];
 #pragma unroll
                     for (int ch = 0; ch < CH; ++ch) {
@@ -455,7 +485,7 @@ conv_tc_pre_kernel(const ConvProblem p, const int32_t *cst, const __grid_constan
                         int o[32];
                         tc_ld32(t_addr + 32u * ch, v);
                         if (ch == CH - 1) hand_back();
-                        if (RAW) add_row(v, row_cst);
+                        if (C::SIGNED_A) add_row(v, row_cst);
                         biased_ints(v, table + 4u * (h * PC + 32 * ch), o);
 #pragma unroll
                         for (int i = 0; i < 16; ++i) packed[h][ch][i] = __byte_perm((uint32_t)o[2 * i], (uint32_t)o[2 * i + 1], 0x5410);
@@ -467,7 +497,7 @@ conv_tc_pre_kernel(const ConvProblem p, const int32_t *cst, const __grid_constan
                         int o[32];
                         if (n0 + 32 * ch < p.C_out) {          // warp-uniform
                             tc_ld32(t_addr + 32u * ch, v);
-                            if (RAW) add_row(v, row_cst);
+                            if (C::SIGNED_A) add_row(v, row_cst);
                             biased_ints(v, table + 4u * (h * PC + 32 * ch), o);
                             store_int32_block(static_cast<int32_t *>(p.out) + row0 * p.C_out + n0 + 32 * ch, p.C_out, o, i32_tile, row0, p.M, lane, p.C_out - n0 - 32 * ch);
                         }
@@ -600,14 +630,31 @@ conv_tc_pre_kernel(const ConvProblem p, const int32_t *cst, const __grid_constan
             const uint4 q0 = ld_shared_v4(c_src), q1 = ld_shared_v4(c_src + HALF_BYTES);
             c_src += SLOT_BYTES;
             if (c_src == bits_end) c_src = bits0;
+            // a signed row's bits, and their count left for the epilogue at the group's last stage of the tile
+            auto count = [&](const uint32_t (&wds)[8]) {
+#pragma unroll
+                for (int e = 0; e < 8; ++e) n_bits += __popc(wds[e]);
+                while (c_kt >= ktiles) { c_kt -= ktiles; ++c_ti; }
+                if (c_kt + G >= ktiles) {
+                    asm volatile("st.shared.b32 [%0], %1;" ::"r"(pops + (uint32_t)(((c_ti % C::SLOTS) * G + grp) * C::POP_ROWS + row) * 4u), "r"(n_bits) : "memory");
+                    n_bits = 0;
+                }
+                c_kt += G;
+            };
             if (is_w) {
+                const uint32_t wds[8] = {q0.x, q0.y, q0.z, q0.w, q1.x, q1.y, q1.z, q1.w};
+                if (COLUMN_COUNTS) count(wds);
                 if (!mbar_wait_warp(empty_bar(s), phase, abort_flag, p.err, ERR_PRODUCER_TIMEOUT)) break;
                 const uint32_t row_addr = wring + (uint32_t)s * C::W_BYTES + (uint32_t)row * ROWB;
-                const uint32_t wds[8] = {q0.x, q0.y, q0.z, q0.w, q1.x, q1.y, q1.z, q1.w};
 #pragma unroll
                 for (int e = 0; e < 8; ++e) {
                     uint32_t v[4];
-                    expand_a4(wds[e], v);
+                    if (COLUMN_COUNTS) {
+                        const uint4 o = expand_w4(wds[e]);
+                        v[0] = o.x; v[1] = o.y; v[2] = o.z; v[3] = o.w;
+                    } else {
+                        expand_a4(wds[e], v);
+                    }
                     st_shared_v4(row_addr + (uint32_t)((e ^ (row & 7)) << 4), v[0], v[1], v[2], v[3]);
                 }
                 if (!C::EARLY) {
@@ -617,20 +664,14 @@ conv_tc_pre_kernel(const ConvProblem p, const int32_t *cst, const __grid_constan
                 fence_async_proxy();          // generic stores -> the MMAs
             } else {
                 uint32_t v[32];
-                if (RAW) {
+                if (C::SIGNED_A) {
                     const uint32_t wds[8] = {q0.x, q0.y, q0.z, q0.w, q1.x, q1.y, q1.z, q1.w};
 #pragma unroll
                     for (int e = 0; e < 8; ++e) {
                         const uint4 o = expand_w4(wds[e]);
                         v[4 * e] = o.x; v[4 * e + 1] = o.y; v[4 * e + 2] = o.z; v[4 * e + 3] = o.w;
-                        n_bits += __popc(wds[e]);
                     }
-                    while (c_kt >= ktiles) { c_kt -= ktiles; ++c_ti; }
-                    if (c_kt + G >= ktiles) { // this group's last stage of the tile
-                        asm volatile("st.shared.b32 [%0], %1;" ::"r"(pops + (uint32_t)(((c_ti % C::SLOTS) * G + grp) * BM + row) * 4u), "r"(n_bits) : "memory");
-                        n_bits = 0;
-                    }
-                    c_kt += G;
+                    count(wds);
                 } else {
                     expand_stage8(q0, q1, v);
                 }
@@ -697,7 +738,7 @@ bool walk_across(const ConvProblem &p, long n_tiles, long units)
 }
 
 // pw.wexp == nullptr where the weights are raw (RAW)
-template <int BN, int MODE, int G, int TEAMS, bool PAIR, bool RAW = false, bool WHOLE = false>
+template <int BN, int MODE, int G, int TEAMS, bool PAIR, int RAW = 0, bool WHOLE = false>
 int launch_bn(const ConvProblem &p0, const PreparedWeights &pw, cudaStream_t stream)
 {
     using C = Cfg<BN, MODE, G, TEAMS, PAIR, RAW, WHOLE>;
@@ -811,14 +852,16 @@ bool conv_tc_pre_supports(const ConvProblem &p)
     return p.K <= (1 << 20);                                  // sums up to 4 K + 2 stay exact in fp32
 }
 
-int launch_conv_tc_pre(const ConvProblem &p, const void *prepared, cudaStream_t stream)
+// How a product is cut up: columns of a tile, two blocks on one, a tile handed over in one piece, the operand whose bits are counted.
+namespace {
+struct StreamPlan {
+    int bn;
+    bool pair, whole;
+    int raw;
+};
+
+StreamPlan prepared_plan(const ConvProblem &p)
 {
-    if (!conv_tc_pre_supports(p)) return BCNN_ERR_UNSUPPORTED;
-    PreparedWeights pw;
-    size_t bytes;
-    prepared_layout(p.C_out, p.K, pw, bytes);
-    pw.wexp = static_cast<const uint8_t *>(prepared);
-    pw.cst = reinterpret_cast<const int32_t *>(pw.wexp + (size_t)pw.n_pad * pw.k_pad / 2);
     // Tile width: 256, 128 or 64 columns.  Narrow tiles spread a small layer over more multiprocessors and shorten its epilogue, but
     // every tile expands its activation rows again.  Estimated time in ns, fitted to 40 layers and products per output on B200 (the choice is
     // within 6 % of the best width on all but two): a start, a term per tile column of the longest CTA, one per 256-bit stage - longer
@@ -846,7 +889,7 @@ int launch_conv_tc_pre(const ConvProblem &p, const void *prepared, cudaStream_t 
     // whole: 300000 x 218 x 384 109 and 71, 500000 x 146 x 768 149 and 108, 350000 x 201 x 1152 120 and 104; 300000 x 250 x 384 84 and 84, but in the
     // cache 100000 x 218 x 384 26.0 and 27.6, and 300000 x 243 x 64, one stage, 83 and 98)
     if (!packed && fits256 && kt > 1 && p.C_out > 128 && p.C_out <= 256 && (p.C_out & 7) != 0 && (long)p.M * p.C_out >= 1L << 25)
-        return launch_bn<256, 0, 2, 2, false, false, true>(p, pw, stream);
+        return {256, false, true, 0};
     long c256 = LONG_MAX, c128, c64;
     if (packed) {
         c64 = cost(64, 2150, 160, wide_gather ? 212 : 330);
@@ -861,21 +904,18 @@ int launch_conv_tc_pre(const ConvProblem &p, const void *prepared, cudaStream_t 
     }
     // One stage, int32: the stores are the time, and over several waves 64-wide tiles take longer than the estimate has it (us at 64 and
     // 128: 5301 x 860 x 32, four waves, 9.0 and 7.5; two waves 5.1 and 5.0; one wave, 1000 x 500 x 256, 3.8 and 4.8, 3000 x 300 x 160 4.2 and 4.8)
-    if (!packed && kt == 1 && waves_of(64) > 2) return launch_bn<128, 0, 3, 2, false>(p, pw, stream);
-    if (c64 < c128 && c64 <= c256) return packed ? launch_bn<64, 1, 2, 1, false>(p, pw, stream) : launch_bn<64, 0, 2, 1, false>(p, pw, stream);
-    if (c128 <= c256) return packed ? launch_bn<128, 1, 2, 1, false>(p, pw, stream) : launch_bn<128, 0, 3, 2, false>(p, pw, stream);
+    if (!packed && kt == 1 && waves_of(64) > 2) return {128, false, false, 0};
+    if (c64 < c128 && c64 <= c256) return {64, false, false, 0};
+    if (c128 <= c256) return {128, false, false, 0};
     // Two multiprocessors on a tile of 256 x 256: half the weight bytes from L2 and into shared memory.  That pays where the tensor pipe is
     // kept busy for long - what limits such a product is power, the clock falls to 1.6 GHz (seconds of 16384 x 16384 x 9216 in a row: int32
     // 978 -> 877 us, packed 774 -> 745; 25088 x 512 x 4608 33.1 -> 30.7 and 23.1 -> 22.7; 16384 x 16384 x 2304 packed 231 -> 218) - and costs a hand-over between
     // the two elsewhere (50176 x 256 x 2304, three waves: 13.2 -> 14.0)
-    if (waves_of(256) >= 8 || (waves_of(256) >= 3 && p.K >= 4096)) return packed ? launch_bn<256, 1, 2, 2, true>(p, pw, stream) : launch_bn<256, 0, 2, 2, true>(p, pw, stream);
-    return packed ? launch_bn<256, 1, 2, 2, false>(p, pw, stream) : launch_bn<256, 0, 2, 2, false>(p, pw, stream);
+    return {256, waves_of(256) >= 8 || (waves_of(256) >= 3 && p.K >= 4096), false, 0};
 }
 
-// ---- raw weights: the streaming engine's packed and int32 outputs
-int launch_conv_tc_raw(const ConvProblem &p, cudaStream_t stream)
+StreamPlan raw_plan(const ConvProblem &p)
 {
-    const PreparedWeights none = {};
     const bool packed = p.mode == 1;
     // As for prepared weights, fitted to 20 products (packed, us at 64 / 128 / a pair's 256 columns: 4096 x 4096 x 4608 85.6, 53.1, 37.8; 2048 x
     // 2048 x 4608 26.3, 17.6, 13.6; 300 x 4000 x 9216 25.2, 17.0, 19.6; 1024 x 1024 x 4608 8.7, 10.3, 12.2; 20 x 64 x 960 3.5, 4.3, 5.5; int32: 4096 x 4096 x 4608 89.7, 56.7,
@@ -887,11 +927,68 @@ int launch_conv_tc_raw(const ConvProblem &p, cudaStream_t stream)
         return start + (tiles + units - 1) / units * (wave + kt * stage);
     };
     const long c64 = cost(BM, 64, sms, 2500, packed ? 450 : 700, 300), c128 = cost(BM, 128, sms, 3000, packed ? 700 : 1200, 360);
-    const bool fits = smem_bytes<Cfg<256, 0, 2, 2, true, true>>(ktw, 0) <= MAX_SMEM;
+    const bool fits = smem_bytes<Cfg<256, 0, 2, 2, true, RAW_ROWS>>(ktw, 0) <= MAX_SMEM;
     const long c256 = fits ? cost(2 * BM, 256, sms / 2, packed ? 3900 : 6500, packed ? 900 : 4900, 415) : LONG_MAX;
-    if (c64 <= c128 && c64 <= c256) return packed ? launch_bn<64, 1, 2, 1, false, true>(p, none, stream) : launch_bn<64, 0, 2, 1, false, true>(p, none, stream);
-    if (c128 <= c256) return packed ? launch_bn<128, 1, 2, 1, false, true>(p, none, stream) : launch_bn<128, 0, 2, 1, false, true>(p, none, stream);
-    return packed ? launch_bn<256, 1, 2, 2, true, true>(p, none, stream) : launch_bn<256, 0, 2, 2, true, true>(p, none, stream);
+    if (c64 <= c128 && c64 <= c256) return {64, false, false, RAW_COLUMNS};
+    if (c128 <= c256) return {128, false, false, kt < 8 ? RAW_COLUMNS : RAW_ROWS};
+    return {256, true, false, RAW_ROWS};
+}
+
+// the kernels for prepared weights and for raw ones
+template <int MODE>
+int launch_plan(const StreamPlan &plan, const ConvProblem &p, const PreparedWeights &pw, cudaStream_t stream)
+{
+    if (plan.raw) {
+        if (plan.bn == 64) return launch_bn<64, MODE, 2, 1, false, RAW_COLUMNS>(p, pw, stream);
+        if (plan.bn == 128) return plan.raw == RAW_COLUMNS ? launch_bn<128, MODE, 2, 1, false, RAW_COLUMNS>(p, pw, stream) : launch_bn<128, MODE, 2, 1, false, RAW_ROWS>(p, pw, stream);
+        return launch_bn<256, MODE, 2, 2, true, RAW_ROWS>(p, pw, stream);
+    }
+    if (plan.bn == 64) return launch_bn<64, MODE, 2, 1, false>(p, pw, stream);
+    if (plan.bn == 128) return launch_bn<128, MODE, MODE == 0 ? 3 : 2, MODE == 0 ? 2 : 1, false>(p, pw, stream);
+    if constexpr (MODE == 0)
+        if (plan.whole) return launch_bn<256, MODE, 2, 2, false, 0, true>(p, pw, stream);
+    return plan.pair ? launch_bn<256, MODE, 2, 2, true>(p, pw, stream) : launch_bn<256, MODE, 2, 2, false>(p, pw, stream);
+}
+
+// the gather's table at its longest fits beside every raw variant
+template <int BN, int G, int TEAMS, bool PAIR, int RAW>
+constexpr bool raw_fits() { return smem_bytes<Cfg<BN, 0, G, TEAMS, PAIR, RAW>>(MAX_RAW_KTAB, 0) <= MAX_SMEM && smem_bytes<Cfg<BN, 1, G, TEAMS, PAIR, RAW>>(MAX_RAW_KTAB, 1) <= MAX_SMEM; }
+static_assert(raw_fits<64, 2, 1, false, RAW_COLUMNS>() && raw_fits<128, 2, 1, false, RAW_COLUMNS>() && raw_fits<128, 2, 1, false, RAW_ROWS>() && raw_fits<256, 2, 2, true, RAW_ROWS>(),
+              "what conv_tc_i8_supports vouches for");
+
+}  // namespace
+
+int launch_conv_tc_pre(const ConvProblem &p, const void *prepared, cudaStream_t stream)
+{
+    if (!conv_tc_pre_supports(p)) return BCNN_ERR_UNSUPPORTED;
+    PreparedWeights pw;
+    size_t bytes;
+    prepared_layout(p.C_out, p.K, pw, bytes);
+    pw.wexp = static_cast<const uint8_t *>(prepared);
+    pw.cst = reinterpret_cast<const int32_t *>(pw.wexp + (size_t)pw.n_pad * pw.k_pad / 2);
+    const StreamPlan plan = prepared_plan(p);
+    return p.mode == 1 ? launch_plan<1>(plan, p, pw, stream) : launch_plan<0>(plan, p, pw, stream);
+}
+
+// ---- raw weights: the streaming engine's packed and int32 outputs
+int launch_conv_tc_raw(const ConvProblem &p, cudaStream_t stream)
+{
+    const StreamPlan plan = raw_plan(p);
+    return p.mode == 1 ? launch_plan<1>(plan, p, PreparedWeights{}, stream) : launch_plan<0>(plan, p, PreparedWeights{}, stream);
+}
+
+// Columns of a tile, blocks on one, 1 where it is handed over whole, the operand whose bits are counted (0: none), 256-bit stages, the most tiles
+// of a block.
+void conv_tc_stream_plan(const ConvProblem &p, bool raw, int (&out)[6])
+{
+    const StreamPlan plan = raw ? raw_plan(p) : prepared_plan(p);
+    const long ctas = plan.pair ? 2 : 1, units = sm_count() / ctas, tiles = ((long)p.M + ctas * BM - 1) / (ctas * BM) * (((long)p.C_out + plan.bn - 1) / plan.bn);
+    out[0] = plan.bn;
+    out[1] = (int)ctas;
+    out[2] = plan.whole ? 1 : 0;
+    out[3] = plan.raw;
+    out[4] = (p.kwords + 7) >> 3;
+    out[5] = (int)((tiles + units - 1) / units);
 }
 
 }  // namespace bcnn
