@@ -85,8 +85,7 @@ int make_conv_problem(ConvProblem &p, const void *x, const void *w, const int32_
 //   * 3x3 layers (stride 1 or 2) on 32 or 64 input channels with C_out <= 128, packed output, whose 8 x 16 output tiles
 //     are at least three quarters full: halo-tile tcgen05 engine (input tiles by tiled TMA copies);
 //   * 1x1 layer with C_in = 32 and C_out <= 32, int32 output: weight-stationary engine, few rows: warp-level int8 engine;
-//   * many rows of C_out <= 128 with K >= 64, or of wider layers with K <= 2304 (in 128-channel slices): weight-stationary
-//     tcgen05 engine;
+//   * many rows of a K whose weights fit shared memory (wider layers in 128-channel slices): weight-stationary tcgen05 engine;
 //   * other layers of C_out <= 64, those with K = 32 (strided, or int32 output): register-fed warp-level int8 engine;
 //   * everything else, and the smaller layers of the engines above at their lines: streaming tcgen05 engine;
 //   * the single-bit mma.sync engine is nowhere the fastest (4096 x 4096 x 9216: 835 us; streaming takes 38 for half of that K) and serves as a fallback.
@@ -118,20 +117,14 @@ int auto_engine(const ConvProblem &p)
         if (p.M >= 98304 && conv_tc_ws_supports(p)) return BCNN_ENGINE_TC_WS;
         return conv_mma_s8_supports(p) ? BCNN_ENGINE_MMA_S8 : BCNN_ENGINE_LOP3;
     }
-    // Up to 128 output channels: the weight-stationary engine, unless its CTAs would expand all the weights for less than two
-    // waves of 64-wide tiles of the streaming engine (3x3 128 -> 128: 7.6 against 5.0 us at M = 784, 8.3 against 7.0 at 12544;
-    // 1x1 256 -> 64 at M = 81000: 7.5 against 12.1)
-    const long waves64 = (tiles64 + sms - 1) / sms;
-    const bool small = stream_raw && (waves64 <= 1 || (waves64 <= 2 && p.K >= 1024));
-    if (p.C_out <= 128 && p.K >= 64) {
-        // ... or few row tiles of more than 64 channels (3x3 64 -> 96 at M = 37125 8.4 against 6.9; at 50176 8.8 and 9.1)
-        if (small || (p.M <= 40000 && p.C_out > 64 && stream_raw)) return BCNN_ENGINE_TC_I8;
-        if (conv_tc_ws_supports(p)) return BCNN_ENGINE_TC_WS;
+    // Weight-stationary or streaming, by their estimates, which err by a tenth: the streaming one where it is 7 % ahead.  (us, weight-stationary and
+    // streaming: 3x3 128 -> 128 at M = 784 7.6 and 4.3, 64 -> 384 at 85116 19.0 and 26.6, 224 -> 608 at 82000 53 and 73, int32 160 -> 2639 at 29592 109 and
+    // 179, 64 -> 770 5x5 at 23814 33 and 50; 1x1 320 -> 256 at 200704 22.9 and 25.1, 256 -> 96 at 117120 10.5 and 15.9.)
+    const bool ws = conv_tc_ws_supports(p);
+    if (ws && (p.K >= 64 || p.C_out > 64)) {
+        if (stream_raw && 107 * conv_tc_stream_estimate(p, true) < 100 * conv_tc_ws_estimate(p)) return BCNN_ENGINE_TC_I8;
+        return BCNN_ENGINE_TC_WS;
     }
-    // wider layers in slices of 128 output channels: ahead of the streaming engine while the weights fit and there are enough row
-    // tiles to share one slice's weights (packed, row: 1x1 320 -> 256 at M = 200704 22.9 us, streaming 25.1; 3x3 256 -> 256 at 50176 20.9 and 18.2,
-    // 4096 x 4096 x 768 14.9 and 14.6; int32: 3x3 256 -> 256 at 50176 26.0 and 31.4, 5000 x 1000 x 1152 14.4 and 12.8)
-    if (p.C_out > 128 && p.K <= 2304 && p.M >= (p.mode == 1 ? 98304 : 40000) && conv_tc_ws_supports(p)) return BCNN_ENGINE_TC_WS;
     // K = 32, row: 1x1/2 32 -> 64 packed at M = 50176 5.2 us, streaming 6.4; 32 -> 64 int32 at M = 200704 14.3 and 18.2.  At 128 channels
     // 8.3 and 7.5 packed, 23.9 and 32.3 int32
     if (p.C_out <= 64 && conv_mma_s8_supports(p)) return BCNN_ENGINE_MMA_S8;
@@ -447,10 +440,8 @@ int bcnn_prepared_preferred(int B, int H, int W, int C_in, int C_out, int kh, in
                                      B, H, W, C_in, C_out, kh, kw, stride, pad, fused != 0);
     if (st != BCNN_OK) return 0;
     // Measured: streaming prepared weights wins where AUTO would expand them on every call - the streaming engine, a short K of a
-    // wide packed product apart (16384 x 16384 x 512 183 against 142 us), the weight-stationary one except on many rows of few channels whose
-    // pixels are an odd number of words (3x3 96 -> 32 at M = 300000 24.2 against 20.0; 96 -> 96 at 200704 18.9 and 18.7, int32 22.3 and 28.3; 192 -> 64
-    // 1x1 9.0 and 9.8).  The wide pointwise and halo-tile engines keep their layers, all but the smallest with many weights:
-    // they expand those at the start.
+    // wide packed product apart (16384 x 16384 x 512 183 against 142 us), the weight-stationary one by their estimates.  The wide pointwise and halo-tile
+    // engines keep their layers, all but the smallest with many weights: they expand those at the start.
     if (!conv_tc_pre_supports(p)) return 0;
     const long tiles64 = ((p.M + 127L) / 128) * ((p.C_out + 63) / 64), sms = sm_count();
     switch (auto_engine(p)) {
@@ -466,10 +457,10 @@ int bcnn_prepared_preferred(int B, int H, int W, int C_in, int C_out, int kh, in
         // 5.5 and 4.7 at 784, 8.8 and 10.0 at 3136
         return tiles64 <= 3 * sms || (p.C_out <= 128 && tiles64 <= 6 * sms) ? 1 : 0;
     case BCNN_ENGINE_TC_WS:
-        // the weight-stationary engine spreads its expansion over many rows: channels gathered word by word (M = 200704, us: 3x3 96 -> 64 packed 16.7
-        // and 17.3, 160 -> 64 21.3 and 23.0, 96 -> 32 int32 16.9 and 17.8) and windows beyond 3x3 (5x5 128 -> 64 at 522144 71.8 and 84.4, int32 77.6
-        // and 86.5; 3x3 15.9 and 16.1, int32 20.0 and 17.6; 1x1 256 -> 64 9.8 and 8.6).  At M = 50176 5x5 14.9 and 11.3
-        return p.M >= 98304 && ((p.C_out <= (fused ? 64 : 32) && (p.cw & 1)) || (p.C_out <= 64 && p.kh * p.kw > 9)) ? 0 : 1;
+        // the weight-stationary engine spreads its expansion over many rows, and fits less beside its weights the longer K is (us, weight-stationary and
+        // prepared: 1x1 64 -> 14, int32, at M = 1223880 37 and 64, 3x3 64 -> 16 at 3683575 163 and 229, 96 -> 128 at 803000 56 and 65, 32 -> 288 5x5 at 487305
+        // 96 and 117; 3x3 256 -> 96 at 194600 29.8 and 25.6, 448 -> 288 at 86184 79 and 57)
+        return p.K >= 1536 || conv_tc_stream_estimate(p, false) < conv_tc_ws_estimate(p) ? 1 : 0;
     case BCNN_ENGINE_TC_I8: return fused && p.K <= 512 && p.C_out > 1024 && (long)p.M * p.C_out >= 1L << 27 ? 0 : 1;
     // int32: 1x1 128 -> 128 at M = 784 3.2 and 3.0 us, 96 -> 64 at M = 196 3.1 and 2.9; 29 x 391 x 64 2.9 and 3.2
     case BCNN_ENGINE_LOP3: return p.K <= 64 ? 0 : 1;

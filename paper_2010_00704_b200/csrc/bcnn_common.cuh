@@ -97,6 +97,8 @@ int launch_conv_tc_i8(const ConvProblem &p, cudaStream_t stream);
 int launch_conv_tc_raw(const ConvProblem &p, cudaStream_t stream);      // packed and int32 outputs, what conv_tc_i8_supports vouches for
 constexpr int MAX_RAW_KTAB = 1920;       // units of the gather's table that every streaming kernel on raw weights has room for
 void conv_tc_stream_plan(const ConvProblem &p, bool raw, int (&plan)[6]);
+long conv_tc_stream_estimate(const ConvProblem &p, bool raw);            // expected time, ns, on raw or prepared weights
+long conv_tc_ws_estimate(const ConvProblem &p);                          // ... of the weight-stationary engine, packed and int32 outputs
 // weights expanded once per layer by launch_prepare_weights (conv_tc_pre.cu): [n_pad][k_pad] signed 4-bit codes, then
 // K - 2 popc(W_n) per row
 struct PreparedWeights {

@@ -730,11 +730,14 @@ int ktab_words_for(const ConvProblem &p) { return ((p.kwords + 7) >> 3) * (8 / g
 // int32 rows that are no whole number of 32-byte sectors: the sectors at the tile columns' borders and at the ends of the rows are written
 // by two tiles.  With a column of tiles finished before the next is begun they leave the second-level cache half written and come back
 // (300000 x 218 x 384: 57 MB read where the operands are 14; 314286 x 364 x 64 191 -> 117 us across the columns, 126000 x 507 x 576 120 -> 74,
-// 150000 x 756 x 128 163 -> 113).  Up to an eighth as many columns as blocks: a grid that is a multiple of them leaves some idle.
-template <int MODE>
-bool walk_across(const ConvProblem &p, long n_tiles, long units)
+// 150000 x 756 x 128 163 -> 113, 30912 x 4305 x 864 250 -> 166).  Not where the output stays in the cache (6157 x 645 x 224 7.8 -> 8.4), where K is long
+// enough to be the time - blocks beside one another then fetch as many weight columns (94316 x 299 x 4320 79 -> 85) - or where the last column is so
+// empty that its blocks idle (178587 x 135 x 96 33 -> 42).  A grid that is a multiple of the columns may leave an eighth of the blocks idle.
+bool walk_across(const ConvProblem &p, int bn, long units)
 {
-    return MODE == 0 && (p.C_out & 7) != 0 && n_tiles > 1 && 8 * n_tiles <= units;
+    const long n_tiles = ((long)p.C_out + bn - 1) / bn;
+    return p.mode == 0 && (p.C_out & 7) != 0 && n_tiles > 1 && n_tiles <= units && 8 * (units % n_tiles) <= units && p.kwords <= 56 &&
+           (long)p.M * p.C_out >= 1L << 25 && 10L * p.C_out >= 7 * n_tiles * bn;
 }
 
 // pw.wexp == nullptr where the weights are raw (RAW)
@@ -749,7 +752,7 @@ int launch_bn(const ConvProblem &p0, const PreparedWeights &pw, cudaStream_t str
     const long n_tiles = ((long)p.C_out + BN - 1) / BN;
     const long total = m_tiles * n_tiles;
     if (total >= (1L << 31)) return BCNN_ERR_UNSUPPORTED;
-    const bool across = walk_across<MODE>(p, n_tiles, units);
+    const bool across = !PAIR && BN > 64 && walk_across(p, BN, units);
     const long rows = across ? (m_tiles < units / n_tiles ? m_tiles : units / n_tiles) : 0;
     const int grid = (int)(across ? rows * n_tiles : total < units ? total : units);
     const int ktw = ktab_words_for(p);
@@ -860,60 +863,94 @@ struct StreamPlan {
     int raw;
 };
 
+// Expected time of a plan, ns: a start, a term per tile of the longest block and one per 256-bit stage of it - by how the gather goes: four, two, one
+// word at a time - and int32 outputs by the million, those beyond 30 million of rows of no whole sectors once more.  Fitted to 3929 drawn layers and
+// products with every variant timed, and 3070 more with int32 rows; within 7 to 12 % (one standard deviation).
+struct Rates {
+    int bn, ctas, packed, raw, across;
+    long start, tile, stage[3], out, ragged;
+};
+constexpr Rates RATES[] = {
+    {64, 1, 1, 0, 0, 1950, 430, {190, 212, 274}, 0, 0},        {128, 1, 1, 0, 0, 2080, 590, {201, 217, 287}, 0, 0},
+    {256, 1, 1, 0, 0, 1930, 1110, {296, 301, 330}, 0, 0},      {256, 2, 1, 0, 0, 2380, 1200, {283, 289, 324}, 0, 0},
+    {64, 1, 0, 0, 0, 2740, 373, {165, 176, 231}, 706, 788},    {128, 1, 0, 0, 0, 3720, 128, {188, 168, 223}, 785, 857},
+    {128, 1, 0, 0, 1, 3340, 1414, {194, 163, 215}, 143, 413},  {256, 1, 0, 0, 0, 3450, 1053, {305, 292, 318}, 635, 726},
+    {256, 1, 0, 0, 1, 2510, 3663, {306, 290, 312}, 101, 330},  {256, 2, 0, 0, 0, 5350, 1409, {240, 226, 265}, 913, 574},
+    {64, 1, 1, RAW_COLUMNS, 0, 2210, 415, {282, 307, 363}, 0, 0}, {128, 1, 1, RAW_COLUMNS, 0, 2330, 594, {388, 460, 519}, 0, 0},
+    {128, 1, 1, RAW_ROWS, 0, 2350, 689, {390, 459, 529}, 0, 0},   {256, 2, 1, RAW_ROWS, 0, 2620, 1275, {405, 498, 557}, 0, 0},
+    {64, 1, 0, RAW_COLUMNS, 0, 2840, 480, {259, 290, 341}, 750, 0}, {128, 1, 0, RAW_COLUMNS, 0, 3250, 330, {340, 416, 467}, 1030, 0},
+    {128, 1, 0, RAW_ROWS, 0, 3220, 298, {354, 429, 500}, 993, 0}, {256, 2, 0, RAW_ROWS, 0, 6080, 1742, {384, 536, 600}, 1248, 0},
+};
+
+long estimate(const ConvProblem &p, const StreamPlan &plan)
+{
+    const int ctas = plan.pair ? 2 : 1, gw = gather_width(p.cw);
+    const long units = sm_count() / ctas, rows = ((long)p.M + ctas * BM - 1) / (ctas * BM), columns = ((long)p.C_out + plan.bn - 1) / plan.bn, kt = (p.kwords + 7) >> 3;
+    const int across = !plan.raw && !plan.pair && plan.bn > 64 && walk_across(p, plan.bn, units) ? 1 : 0;
+    const long tiles = across ? (rows + units / columns - 1) / (units / columns) : (rows * columns + units - 1) / units, outputs = (long)p.M * p.C_out;
+    for (const Rates &r : RATES)
+        if (r.bn == plan.bn && r.ctas == ctas && r.packed == (p.mode == 1) && r.raw == plan.raw && r.across == across)
+            return r.start + tiles * (r.tile + kt * r.stage[gw == 4 ? 0 : gw == 2 ? 1 : 2]) + outputs / 1000 * r.out / 1000 +
+                   ((p.C_out & 7) != 0 && outputs > 30000000 ? (outputs - 30000000) / 1000 * r.ragged / 1000 : 0);
+    return LONG_MAX;
+}
+
 StreamPlan prepared_plan(const ConvProblem &p)
 {
     // Tile width: 256, 128 or 64 columns.  Narrow tiles spread a small layer over more multiprocessors and shorten its epilogue, but
-    // every tile expands its activation rows again.  Estimated time in ns, fitted to 40 layers and products per output on B200 (the choice is
-    // within 6 % of the best width on all but two): a start, a term per tile column of the longest CTA, one per 256-bit stage - longer
-    // where the gather goes by single or paired words - and one for the tiles that compete for memory at the start.
+    // every tile expands its activation rows again.  By the estimates above; the choice takes 0.6 % longer than the best width in the mean where the output
+    // is packed, 2.6 % where it is int32.
     //   packed, us at 64 / 128 / 256: 3x3 256 -> 256 at M = 50176 25.3, 15.5, 13.2; M = 196 4.0, 4.3, 5.6; 512 -> 512 at M = 12544 26.4, 15.2, 14.8;
-    //   3x3 128 -> 128 at M = 6272 3.9, 3.6, 4.7; int32: 256 -> 256 at M = 50176 28.4, 21.3, 22.0; 1000 x 4000 x 2304 12.4, 9.6, 10.7
+    //   3x3 128 -> 128 at M = 6272 3.9, 3.6, 4.7; 1x1 64 -> 3264 at 13320 37.4, 32.0, 22.4; int32: 5x5 128 -> 7216 at M = 572 22.2, 15.0, 11.9; 3x3 384 -> 859
+    //   at 4680 21.2, 11.7, 10.9; 1x1 224 -> 645 at 6157 8.2, 7.8, 6.9; 384 -> 218 at 10000 6.8, 6.7, 7.5
     const int sms = sm_count();
-    const long m_tiles = ((long)p.M + BM - 1) / BM, kt = (p.kwords + 7) / 8;
-    const bool wide_gather = gather_width(p.cw) == 4;
-    auto waves_of = [&](int bn) { return (m_tiles * ((p.C_out + bn - 1) / bn) + sms - 1) / sms; };
-    auto cost = [&](int bn, long start, long wave, long stage) {
-        const long tiles = m_tiles * ((p.C_out + bn - 1) / bn);
-        return start + waves_of(bn) * (wave + kt * stage) + 7 * (tiles < sms ? tiles : sms);
-    };
+    const long m_tiles = ((long)p.M + BM - 1) / BM, kt = (p.kwords + 7) / 8, outputs = (long)p.M * p.C_out;
     const bool packed = p.mode == 1;
-    // What conv_tc_pre_supports vouches for is the packed 256-wide variant's shared memory.  The int32 one needs its store staging
-    // tiles besides: a K beyond 274 176 bits with an odd number of words per pixel, 548 352 with an even one, runs on narrower tiles.
-    static_assert(smem_bytes<Cfg<128, 0, 3, 2, false>>(0, 0) <= smem_bytes<Cfg<256, 1, 2, 2, false>>(0, 1) && smem_bytes<Cfg<64, 0, 2, 1, false>>(0, 0) <= smem_bytes<Cfg<256, 1, 2, 2, false>>(0, 1) &&
-                  smem_bytes<Cfg<128, 1, 2, 1, false>>(0, 1) <= smem_bytes<Cfg<256, 1, 2, 2, false>>(0, 1) && smem_bytes<Cfg<64, 1, 2, 1, false>>(0, 1) <= smem_bytes<Cfg<256, 1, 2, 2, false>>(0, 1),
-                  "a supported layer fits the narrower tiles");
-    static_assert(smem_bytes<Cfg<256, 0, 2, 2, true>>(0, 0) <= smem_bytes<Cfg<256, 0, 2, 2, false>>(0, 0) && smem_bytes<Cfg<256, 1, 2, 2, true>>(0, 1) <= smem_bytes<Cfg<256, 1, 2, 2, false>>(0, 1),
-                  "and the tile of two blocks");
-    const bool fits256 = packed || smem_bytes<Cfg<256, 0, 2, 2, false>>(ktab_words_for(p), 0) <= MAX_SMEM;
-    // One column of tiles, int32 rows of no whole sectors and more of them than the second-level cache holds: whole rows at a time (us, tiles of 128 and
-    // whole: 300000 x 218 x 384 109 and 71, 500000 x 146 x 768 149 and 108, 350000 x 201 x 1152 120 and 104; 300000 x 250 x 384 84 and 84, but in the
-    // cache 100000 x 218 x 384 26.0 and 27.6, and 300000 x 243 x 64, one stage, 83 and 98)
-    if (!packed && fits256 && kt > 1 && p.C_out > 128 && p.C_out <= 256 && (p.C_out & 7) != 0 && (long)p.M * p.C_out >= 1L << 25)
-        return {256, false, true, 0};
-    long c256 = LONG_MAX, c128, c64;
-    if (packed) {
-        c64 = cost(64, 2150, 160, wide_gather ? 212 : 330);
-        c128 = cost(128, 2300, 320, wide_gather ? 210 : 350);
-        // (the first tile column: nothing of it waits for an epilogue; a short K waits for every epilogue)
-        const long stage = wide_gather ? 283 : 350, rest = 910 + kt * stage;
-        c256 = cost(256, 3000 + kt * stage, 0, 0) + (waves_of(256) - 1) * (rest > 2200 ? rest : 2200);
-    } else {
-        c64 = cost(64, 2450, 270, wide_gather ? 212 : 330);
-        c128 = cost(128, 3000, 700, wide_gather ? 225 : 340);
-        if (fits256) c256 = cost(256, 3500, 4300, wide_gather ? 270 : 340);
-    }
-    // One stage, int32: the stores are the time, and over several waves 64-wide tiles take longer than the estimate has it (us at 64 and
-    // 128: 5301 x 860 x 32, four waves, 9.0 and 7.5; two waves 5.1 and 5.0; one wave, 1000 x 500 x 256, 3.8 and 4.8, 3000 x 300 x 160 4.2 and 4.8)
-    if (!packed && kt == 1 && waves_of(64) > 2) return {128, false, false, 0};
-    if (c64 < c128 && c64 <= c256) return {64, false, false, 0};
-    if (c128 <= c256) return {128, false, false, 0};
+    auto tiles_of = [&](int bn) { return m_tiles * (((long)p.C_out + bn - 1) / bn); };
+    auto waves_of = [&](int bn) { return (tiles_of(bn) + sms - 1) / sms; };
+    static_assert(smem_bytes<Cfg<64, 1, 2, 1, false>>(0, 1) <= smem_bytes<Cfg<256, 1, 2, 2, false>>(0, 1) && smem_bytes<Cfg<128, 1, 2, 1, false>>(0, 1) <= smem_bytes<Cfg<256, 1, 2, 2, false>>(0, 1) &&
+                  smem_bytes<Cfg<64, 0, 2, 1, false>>(0, 0) <= smem_bytes<Cfg<256, 1, 2, 2, false>>(0, 1) && smem_bytes<Cfg<128, 0, 3, 2, false>>(0, 0) <= smem_bytes<Cfg<256, 1, 2, 2, false>>(0, 1) &&
+                  smem_bytes<Cfg<256, 1, 2, 2, true>>(0, 1) <= smem_bytes<Cfg<256, 1, 2, 2, false>>(0, 1),
+                  "what conv_tc_pre_supports vouches for is the packed 256-wide variant's shared memory");
+    const StreamPlan narrow = {64, false, false, 0}, medium = {128, false, false, 0};
+    if (p.C_out <= 64) return narrow;                     // (a wide tile would be part empty)
     // Two multiprocessors on a tile of 256 x 256: half the weight bytes from L2 and into shared memory.  That pays where the tensor pipe is
     // kept busy for long - what limits such a product is power, the clock falls to 1.6 GHz (seconds of 16384 x 16384 x 9216 in a row: int32
     // 978 -> 877 us, packed 774 -> 745; 25088 x 512 x 4608 33.1 -> 30.7 and 23.1 -> 22.7; 16384 x 16384 x 2304 packed 231 -> 218) - and costs a hand-over between
     // the two elsewhere (50176 x 256 x 2304, three waves: 13.2 -> 14.0)
-    return {256, waves_of(256) >= 8 || (waves_of(256) >= 3 && p.K >= 4096), false, 0};
+    const bool long_k = waves_of(256) >= 3 && p.K >= 4096;
+    const StreamPlan pair = {256, true, false, 0};
+    if (packed) {
+        // tiles that start at the same time wait for one another's rows: 7 ns each
+        auto cost = [&](const StreamPlan &s) { return estimate(p, s) + 7 * (tiles_of(s.bn) < sms ? tiles_of(s.bn) : sms); };
+        const StreamPlan wide = {256, false, false, 0};
+        const long c64 = cost(narrow), c128 = cost(medium), c256 = p.C_out > 128 ? cost(wide) : LONG_MAX;
+        if (c64 < c128 && c64 <= c256) return narrow;
+        return c128 <= c256 ? medium : waves_of(256) >= 8 || long_k ? pair : wide;
+    }
+    // int32.  A 256-wide tile of one block goes to memory in one piece, whole pieces of 128 columns at a time (0.79 of the time in halves, in the mean over 238
+    // products); in halves only between two blocks, where its stores run beside the next tile's long K.  It needs its store staging tiles besides what
+    // conv_tc_pre_supports vouches for: a K beyond 274 176 bits with an odd number of words per pixel, 548 352 with an even one, runs on narrower tiles.
+    static_assert(smem_bytes<Cfg<256, 0, 2, 2, true>>(0, 0) <= smem_bytes<Cfg<256, 0, 2, 2, false, 0, true>>(0, 0), "and the tile of two blocks");
+    const bool fits256 = p.C_out > 128 && smem_bytes<Cfg<256, 0, 2, 2, false, 0, true>>(ktab_words_for(p), 0) <= MAX_SMEM;
+    const StreamPlan whole = {256, false, true, 0};
+    // Rows of no whole sectors, more of them than the second-level cache holds, in one column of tiles: no neighbour has to fill them (us, tiles of 128 and
+    // whole: 300000 x 218 x 384 109 and 71, 500000 x 146 x 768 149 and 108, 31405 x 138 x 3200 21.0 and 16.4; 300000 x 243 x 64, one stage, 83 and 98; of 64
+    // and 128: 744810 x 90 x 128 172 and 74)
+    if ((p.C_out & 7) != 0 && p.C_out <= 128 && outputs >= 1L << 25) return medium;
+    if ((p.C_out & 7) != 0 && p.C_out <= 256 && fits256 && !long_k &&
+        ((outputs >= 1L << 24 && (kt > 1 || p.C_out < 232)) || (kt >= 10 && outputs >= 1L << 22)))
+        return whole;
+    // One stage: the stores are the time, and over several waves 64-wide tiles of half-full columns take longer than the estimate has it (us at 64 and
+    // 128: 5301 x 860 x 32, four waves, 9.0 and 7.5; 25435 x 120 x 64 6.7 and 6.0)
+    const long c64 = kt == 1 && waves_of(64) > 2 ? LONG_MAX : estimate(p, narrow), c128 = estimate(p, medium);
+    const long c256 = fits256 ? estimate(p, whole) / 20 * 21 : LONG_MAX, c_pair = fits256 && (waves_of(256) >= 8 || long_k) ? estimate(p, pair) : LONG_MAX;
+    if (c64 <= c128 && c64 <= c256 && c64 <= c_pair) return narrow;
+    if (c128 <= c256 && c128 <= c_pair) return medium;
+    return c256 <= c_pair ? whole : pair;
 }
 
+// ---- raw weights: the streaming engine's packed and int32 outputs
 StreamPlan raw_plan(const ConvProblem &p)
 {
     const bool packed = p.mode == 1;
@@ -945,9 +982,7 @@ int launch_plan(const StreamPlan &plan, const ConvProblem &p, const PreparedWeig
     }
     if (plan.bn == 64) return launch_bn<64, MODE, 2, 1, false>(p, pw, stream);
     if (plan.bn == 128) return launch_bn<128, MODE, MODE == 0 ? 3 : 2, MODE == 0 ? 2 : 1, false>(p, pw, stream);
-    if constexpr (MODE == 0)
-        if (plan.whole) return launch_bn<256, MODE, 2, 2, false, 0, true>(p, pw, stream);
-    return plan.pair ? launch_bn<256, MODE, 2, 2, true>(p, pw, stream) : launch_bn<256, MODE, 2, 2, false>(p, pw, stream);
+    return plan.pair ? launch_bn<256, MODE, 2, 2, true>(p, pw, stream) : launch_bn<256, MODE, 2, 2, false, 0, MODE == 0>(p, pw, stream);
 }
 
 // the gather's table at its longest fits beside every raw variant
@@ -976,6 +1011,8 @@ int launch_conv_tc_raw(const ConvProblem &p, cudaStream_t stream)
     const StreamPlan plan = raw_plan(p);
     return p.mode == 1 ? launch_plan<1>(plan, p, PreparedWeights{}, stream) : launch_plan<0>(plan, p, PreparedWeights{}, stream);
 }
+
+long conv_tc_stream_estimate(const ConvProblem &p, bool raw) { return estimate(p, raw ? raw_plan(p) : prepared_plan(p)); }
 
 // Columns of a tile, blocks on one, 1 where it is handed over whole, the operand whose bits are counted (0: none), 256-bit stages, the most tiles
 // of a block.
