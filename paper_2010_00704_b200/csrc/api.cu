@@ -121,13 +121,16 @@ int auto_engine(const ConvProblem &p)
     // streaming: 3x3 128 -> 128 at M = 784 7.6 and 4.3, 64 -> 384 at 85116 19.0 and 26.6, 224 -> 608 at 82000 53 and 73, int32 160 -> 2639 at 29592 109 and
     // 179, 64 -> 770 5x5 at 23814 33 and 50; 1x1 320 -> 256 at 200704 22.9 and 25.1, 256 -> 96 at 117120 10.5 and 15.9.)
     const bool ws = conv_tc_ws_supports(p);
-    if (ws && (p.K >= 64 || p.C_out > 64)) {
+    if (ws && (p.K >= 64 || p.C_out > (packed ? 64 : 32))) {
         if (stream_raw && 107 * conv_tc_stream_estimate(p, true) < 100 * conv_tc_ws_estimate(p)) return BCNN_ENGINE_TC_I8;
         return BCNN_ENGINE_TC_WS;
     }
-    // K = 32, row: 1x1/2 32 -> 64 packed at M = 50176 5.2 us, streaming 6.4; 32 -> 64 int32 at M = 200704 14.3 and 18.2.  At 128 channels
-    // 8.3 and 7.5 packed, 23.9 and 32.3 int32
-    if (p.C_out <= 64 && conv_mma_s8_supports(p)) return BCNN_ENGINE_MMA_S8;
+    // K = 32, strided, or int32 with few channels (us, warp-level int8 and streaming: packed 32 -> 64 /2 at M = 1360 4.5 and 2.9, 19656 4.8 and 4.2, 43560 5.0
+    // and 5.0; int32 32 -> 22 /2 at 7344 5.1 and 3.5, 32 -> 13 at 36288 3.4 and 5.6)
+    if (p.C_out <= 64 && conv_mma_s8_supports(p)) {
+        if (stream_raw && (packed ? p.M < 40000 : p.C_out > 16 && p.M < 20000)) return BCNN_ENGINE_TC_I8;
+        return BCNN_ENGINE_MMA_S8;
+    }
     if (stream_raw) return BCNN_ENGINE_TC_I8;
     if (conv_mma_b1_supports(p)) return BCNN_ENGINE_MMA_B1;
     return BCNN_ENGINE_LOP3;
@@ -457,10 +460,10 @@ int bcnn_prepared_preferred(int B, int H, int W, int C_in, int C_out, int kh, in
         // 5.5 and 4.7 at 784, 8.8 and 10.0 at 3136
         return tiles64 <= 3 * sms || (p.C_out <= 128 && tiles64 <= 6 * sms) ? 1 : 0;
     case BCNN_ENGINE_TC_WS:
-        // the weight-stationary engine spreads its expansion over many rows, and fits less beside its weights the longer K is (us, weight-stationary and
-        // prepared: 1x1 64 -> 14, int32, at M = 1223880 37 and 64, 3x3 64 -> 16 at 3683575 163 and 229, 96 -> 128 at 803000 56 and 65, 32 -> 288 5x5 at 487305
-        // 96 and 117; 3x3 256 -> 96 at 194600 29.8 and 25.6, 448 -> 288 at 86184 79 and 57)
-        return p.K >= 1536 || conv_tc_stream_estimate(p, false) < conv_tc_ws_estimate(p) ? 1 : 0;
+        // the weight-stationary engine spreads its expansion over many rows; beyond 64 channels it fits less beside its weights the longer K is (us, weight-
+        // stationary and prepared: 1x1 64 -> 14, int32, at M = 1223880 37 and 64, 3x3 64 -> 16 at 3683575 163 and 229, 352 -> 32 at 1010880 148 and 200, 96 ->
+        // 128 at 803000 56 and 65, 32 -> 288 5x5 at 487305 96 and 117; 3x3 256 -> 96 at 194600 29.8 and 25.6, 448 -> 288 at 86184 79 and 57)
+        return p.C_out > 64 ? p.K >= 1536 || 100 * conv_tc_stream_estimate(p, false) < 107 * conv_tc_ws_estimate(p) : conv_tc_stream_estimate(p, false) < conv_tc_ws_estimate(p);
     case BCNN_ENGINE_TC_I8: return fused && p.K <= 512 && p.C_out > 1024 && (long)p.M * p.C_out >= 1L << 27 ? 0 : 1;
     // int32: 1x1 128 -> 128 at M = 784 3.2 and 3.0 us, 96 -> 64 at M = 196 3.1 and 2.9; 29 x 391 x 64 2.9 and 3.2
     case BCNN_ENGINE_LOP3: return p.K <= 64 ? 0 : 1;
