@@ -124,6 +124,13 @@ __device__ __forceinline__ uint32_t in_even_cta(uint32_t addr)
     asm("mapa.shared::cluster.u32 %0, %1, 0;" : "=r"(r) : "r"(addr));
     return r;
 }
+// A warp of either CTA to a barrier of the even one, whose issuer starts MMAs behind it.  The arrive releases at block scope only, and that is
+// enough, because nothing but the signal crosses: what it announces is used on the multiprocessor that made it, by that one's tensor
+// core - its activations and its accumulators in its tensor memory, its half of the weights in its shared memory - and each has been completed
+// for that unit before the arrive: stores and reads of tensor memory by tcgen05.wait and fence::before_thread_sync, expanded weights by a
+// fence.proxy.async of every lane that stored, both before the __syncwarp in front of this.  No thread reads the other CTA's memory: its own
+// counts and constants only.  (.release.cluster waits for all of a warp's memory operations, the int32 stores and the gather's copies too, and
+// took twice the time.)
 __device__ __forceinline__ void arrive_in_cluster(uint32_t bar, uint32_t pred)
 {
     asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %1, 0;\n\t@q mbarrier.arrive.shared::cluster.b64 _, [%0];\n\t}" ::"r"(bar), "r"(pred) : "memory");
@@ -174,7 +181,7 @@ conv_tc_pre_kernel(const ConvProblem p, const int32_t *cst, const __grid_constan
     // leave the ring room for the stages that follow.
     const int split_a = min(2, ktiles >> 1), split_b = min(2, ktiles - split_a);
 
-    const uint32_t wring = (smem_u32(smem_raw) + 1023u) & ~1023u;         // [STAGES][BN rows][128 B], written by TMA
+    const uint32_t wring = (smem_u32(smem_raw) + 1023u) & ~1023u;         // [STAGES][BN / CTAS rows][128 B], by TMA or (raw weights) by warps
     const uint32_t bits_ring = wring + STAGES * C::W_BYTES;               // [PF][2][PROD_THREADS][16 B]
     const uint32_t tables = bits_ring + C::BITS_BYTES;                    // [EPI_WARPS][EC] column constants
     const uint32_t pops = tables + C::TABLE_BYTES;                        // [SLOTS][G][POP_ROWS] bit counts
@@ -338,6 +345,14 @@ conv_tc_pre_kernel(const ConvProblem p, const int32_t *cst, const __grid_constan
                 }
                 __syncwarp();
                 ++it;
+                if (++s == STAGES) { s = 0; phase ^= 1u; }
+            }
+        }
+        // The odd CTA: the commits that hand its last slots back come from the other multiprocessor, and its barriers stay until they are in.  (The last
+        // accumulator, which the epilogue waits for, is committed behind them, but on a barrier of its own.)
+        if (PAIR && rank != 0) {
+            for (int i = 0; i < STAGES && ok; ++i) {
+                ok = mbar_wait_warp(empty_bar(s), phase, abort_flag, p.err, ERR_LOADER_TIMEOUT);
                 if (++s == STAGES) { s = 0; phase ^= 1u; }
             }
         }
@@ -618,8 +633,9 @@ conv_tc_pre_kernel(const ConvProblem p, const int32_t *cst, const __grid_constan
         int s = grp;                          // ring slot (G <= STAGES) and its parity
         uint32_t phase = 1;                   // first pass through the ring: slots are free
         int c_kt = grp, c_ti = 0, n_bits = 0; // raw weights: the stage within its tile, the tile, the row's bits so far
+        int it = grp;
 #pragma unroll 1
-        for (int it = grp; it < total_items; it += G) {
+        for (; it < total_items; it += G) {
             if (C::EARLY) {
                 if (l_left > 0) issue_load();
                 cp_async_commit();
@@ -690,6 +706,14 @@ conv_tc_pre_kernel(const ConvProblem p, const int32_t *cst, const __grid_constan
             else mbar_arrive_pred(full0 + 8u * s, lane0);
             s += G;
             if (s >= STAGES) { s -= STAGES; phase ^= 1u; }
+        }
+        if (PAIR && RAW && rank != 0 && wi == 0 && it >= total_items) {      // as the loader above, which raw weights have not: the ring's next pass, but for its work
+#pragma unroll 1
+            for (; it < total_items + STAGES; it += G) {
+                if (!mbar_wait_warp(empty_bar(s), phase, abort_flag, p.err, ERR_PRODUCER_TIMEOUT)) break;
+                s += G;
+                if (s >= STAGES) { s -= STAGES; phase ^= 1u; }
+            }
         }
         cp_async_wait<0>();
     }

@@ -242,6 +242,38 @@ def test_stages_handed_back_in_every_launch(bk, engine, shape):
     assert bk.bcnn_device_error() == 0
 
 
+# ... the streaming engine's hand-overs, prepared and raw: pairs of blocks (whose signals cross from one to the other) of one stage a tile and of
+# many, 256-wide tiles handed over in halves and in one piece, and raw rows' bit counts, whose places a long walk uses again
+@pytest.mark.parametrize("prepared,M,N,K,fused,plan", [(True, 25100, 512, 4608, True, (256, 2, 0, 0)), (True, 76000, 512, 96, True, (256, 2, 0, 0)), (True, 9500, 1500, 8224, False, (256, 2, 0, 0)),
+                                                       (True, 50000, 256, 992, True, (256, 1, 0, 0)), (True, 150003, 250, 416, False, (256, 1, 1, 0)),
+                                                       (False, 60000, 1024, 96, True, (256, 2, 0, 2)), (False, 9000, 1120, 4640, True, (256, 2, 0, 2)), (False, 5000, 500, 8224, False, (256, 2, 0, 2)),
+                                                       (False, 19000, 512, 288, False, (128, 1, 0, 1)), (False, 300000, 64, 288, True, (64, 1, 0, 1))])
+def test_streamed_stages_handed_back_in_every_launch(bk, prepared, M, N, K, fused, plan):
+    assert bk.bcnn_stream_plan(prepared, 1, M, 1, K, N, 1, 1, 1, 0, fused)[:4] == plan
+    rng = np.random.default_rng(M + N + K)
+    x, w, thr = dev(synth.random_bits(rng, (M, K // 8))), dev(synth.random_bits(rng, (N, K // 8))), dev(synth.thresholds(rng, K, N))
+    ref, out = (torch.empty(M * N // 8 if fused else M * N * 4, dtype=torch.uint8, device="cuda") for _ in range(2))
+    if fused:
+        bk.bcnn_gemm_b1_fused(x, w, thr, ref, M, N, K, engine=bk.ENGINES["lop3"])
+    else:
+        bk.bcnn_gemm_b1(x, w, ref, M, N, K, engine=bk.ENGINES["lop3"])
+    prep = torch.empty(bk.bcnn_prepared_weights_bytes(N, K), dtype=torch.uint8, device="cuda")
+    bk.bcnn_prepare_weights(w, prep, N, K)
+    torch.cuda.synchronize()
+    wrong = torch.zeros((), dtype=torch.int64, device="cuda")
+    for _ in range(200):
+        out.fill_(0xA5)
+        if prepared:
+            bk.bcnn_gemm_b1_prepared(x, prep, thr if fused else None, out, M, N, K)
+        elif fused:
+            bk.bcnn_gemm_b1_fused(x, w, thr, out, M, N, K, engine=bk.ENGINES["tc_i8"])
+        else:
+            bk.bcnn_gemm_b1(x, w, out, M, N, K, engine=bk.ENGINES["tc_i8"])
+        wrong += (out != ref).any()
+    assert int(wrong) == 0
+    assert bk.bcnn_device_error() == 0
+
+
 # ... and the stem, seventeen chunks a CTA through its ring of five, against the two separate calls
 def test_stem_stages_handed_back_in_every_launch(bk):
     B, H, W = 100, 224, 224
