@@ -249,7 +249,7 @@ def test_stages_handed_back_in_every_launch(bk, engine, shape):
                                                        (False, 60000, 1024, 96, True, (256, 2, 0, 2)), (False, 9000, 1120, 4640, True, (256, 2, 0, 2)), (False, 5000, 500, 8224, False, (256, 2, 0, 2)),
                                                        (False, 19000, 512, 288, False, (128, 1, 0, 1)), (False, 300000, 64, 288, True, (64, 1, 0, 1))])
 def test_streamed_stages_handed_back_in_every_launch(bk, prepared, M, N, K, fused, plan):
-    assert bk.bcnn_stream_plan(prepared, 1, M, 1, K, N, 1, 1, 1, 0, fused)[:4] == plan
+    assert stream_plan(bk, prepared, M, N, K, fused)[:4] == plan
     rng = np.random.default_rng(M + N + K)
     x, w, thr = dev(synth.random_bits(rng, (M, K // 8))), dev(synth.random_bits(rng, (N, K // 8))), dev(synth.thresholds(rng, K, N))
     ref, out = (torch.empty(M * N // 8 if fused else M * N * 4, dtype=torch.uint8, device="cuda") for _ in range(2))
@@ -325,30 +325,55 @@ def test_module_special_values(bk, oracle, shape, P, has_nb):
     assert bk.bcnn_device_error() == 0
 
 
-# two blocks on a tile of 256 rows x 256 columns: three waves of tiles with a K of 4096 bits and more, and eight with a short one; the
-# last row tile and the last columns part empty, an odd number of 128-column groups, K with a tail of every length in its last stage
+def stream_plan(bk, prepared, M, N, K, fused):
+    """Channels of a tile, blocks on one, 1 where it is handed over in one piece, whose bits are counted (0 none, 1 weights, 2 rows), stages, tiles of a block."""
+    return bk.bcnn_stream_plan(prepared, 1, M, 1, K, N, 1, 1, 1, 0, fused)
+
+
+# two blocks on a tile of 256 rows x 256 columns, packed: three waves of tiles with a K of 4096 bits and more, and nine to eleven with a short
+# one; the last row tile and the last columns part empty, an odd number of 128-column groups, K with a tail of every length in its last
+# stage.  (The two int32 products are whole rows on single blocks.)
 @pytest.mark.parametrize("M,N,K,fused", [(25100, 512, 4608, True), (29000, 480, 4128, True), (14336, 1000, 4192, False), (40000, 1152, 288, True),
                                          (9500, 1100, 4448, False), (30011, 640, 4352, True), (152000, 256, 96, True)])
 def test_prepared_block_pairs(bk, oracle, M, N, K, fused):
+    assert stream_plan(bk, True, M, N, K, fused)[:3] == ((256, 2, 0) if fused else (256, 1, 1))
     test_prepared_widths(bk, oracle, M, N, K, fused)
 
 
-# 256-wide tiles handed over in halves: one to five stages (none, one and two of them split at either end), several tiles per block
+# ... and int32 ones, as 16-bit pairs beside the next tile's MMAs (K <= 32767) and straight out of the accumulator; eleven tiles of nine stages
+@pytest.mark.parametrize("M,N,K,fused", [(9500, 1500, 8224, False), (12300, 900, 10272, False), (9500, 1100, 32800, False), (40000, 1280, 2080, True)])
+def test_prepared_block_pairs_int32(bk, oracle, M, N, K, fused):
+    assert stream_plan(bk, True, M, N, K, fused)[:3] == (256, 2, 0)
+    test_prepared_widths(bk, oracle, M, N, K, fused)
+
+
+# 256-wide tiles handed over in halves: one to five stages (none, one and two of them split at either end), three tiles per block
 @pytest.mark.parametrize("K", [32, 256, 288, 512, 768, 992, 1056])
 def test_prepared_split_tiles(bk, oracle, K):
+    assert stream_plan(bk, True, 50000, 256, K, True) == (256, 1, 0, 0, (K + 255) // 256, 3)
     test_prepared_widths(bk, oracle, 50000, 256, K, True)
 
 
-# int32 products of one stage: two waves of 64-wide tiles at most, and more of them on 128-wide tiles, ragged in rows and columns
-@pytest.mark.parametrize("M,N,K", [(1000, 500, 256), (5301, 860, 32), (6001, 801, 160), (20000, 300, 256)])
+# int32 products of one stage: a wave of 64-wide tiles, and more on 128-wide ones, ragged in rows and columns; up to 64 columns
+# the narrow tile at any number of rows
+@pytest.mark.parametrize("M,N,K", [(1000, 500, 256), (5301, 860, 32), (6001, 801, 160), (20000, 300, 256), (101003, 64, 256), (150000, 40, 32)])
 def test_prepared_one_stage_int32(bk, oracle, M, N, K):
+    assert stream_plan(bk, True, M, N, K, False)[:2] == (64 if M == 1000 or N <= 64 else 128, 1)
     test_prepared_widths(bk, oracle, M, N, K, False)
 
 
-# int32 rows of no whole sectors: tiles across their columns (two, three and eighteen of them, rows left over in the last round of
-# row tiles), and whole rows by 256-wide tiles in one piece, K of one stage, two and several
+# int32 rows of no whole sectors: tiles down their columns where the output stays in the cache, and whole rows by 256-wide tiles in one piece, K of
+# one stage, two and several
 @pytest.mark.parametrize("M,N,K", [(40000, 364, 64), (20000, 255, 288), (30100, 397, 1184), (2500, 2300, 96), (300, 1021, 4640), (262200, 131, 256), (150003, 250, 416), (135000, 253, 2336)])
 def test_prepared_ragged_int32_rows(bk, oracle, M, N, K):
+    test_prepared_widths(bk, oracle, M, N, K, False)
+
+
+# ... and tiles across their columns: outputs of 2^25 values and more, three, eight and 74 columns of tiles, rows left over in the last round of row
+# tiles, K of one stage, two and several
+@pytest.mark.parametrize("M,N,K", [(100003, 364, 64), (100000, 380, 1184), (34000, 1021, 288), (9000, 9393, 96)])
+def test_prepared_tiles_across_columns(bk, oracle, M, N, K):
+    assert stream_plan(bk, True, M, N, K, False)[:4] == (128, 1, 0, 0)
     test_prepared_widths(bk, oracle, M, N, K, False)
 
 
@@ -374,10 +399,18 @@ def test_gap_few_images(bk, oracle, shape):
 
 
 # raw weights on the streaming engine: pairs of blocks (both outputs, K of 32 to 4640 bits with every tail, columns of a half-empty tile, words by
-# 16, 8 and 4 bytes), 128- and 64-wide tiles of one stage and of several, more tiles in flight than a row keeps bit counts for
-@pytest.mark.parametrize("M,N,K,fused", [(4096, 4096, 1184, True), (9000, 1120, 4640, True), (2048, 1000, 4128, False), (20000, 512, 32, True), (20000, 512, 288, True),
-                                         (12544, 512, 2112, True), (8200, 4000, 4608, False), (300, 992, 9216, True), (20, 64, 960, True), (5000, 70, 4000, False), (40000, 192, 256, False)])
-def test_streamed_raw_weights(bk, oracle, M, N, K, fused):
+# 16, 8 and 4 bytes; int32 of more than 16 bits), 128-wide tiles that count their weights' bits or their rows' and 64-wide ones, of one stage and
+# of several, and on each more tiles in a block's walk than bit counts are kept for (10, 11, 13)
+@pytest.mark.parametrize("M,N,K,fused,plan", [(4096, 4096, 1184, True, (256, 2, 0, 2)), (9000, 1120, 4640, True, (256, 2, 0, 2)), (2048, 1000, 4128, False, (128, 1, 0, 2)),
+                                              (20000, 512, 32, True, (256, 2, 0, 2)), (20000, 512, 288, True, (256, 2, 0, 2)), (12544, 512, 2112, True, (256, 2, 0, 2)),
+                                              (8200, 4000, 4608, False, (256, 2, 0, 2)), (300, 992, 9216, True, (64, 1, 0, 1)), (20, 64, 960, True, (64, 1, 0, 1)),
+                                              (5000, 70, 4000, False, (64, 1, 0, 1)), (40000, 192, 256, False, (64, 1, 0, 1)),
+                                              (60000, 1024, 96, True, (256, 2, 0, 2)), (60000, 1024, 288, True, (256, 2, 0, 2)), (5000, 1000, 33056, False, (256, 2, 0, 2)),
+                                              (300000, 64, 32, True, (64, 1, 0, 1)), (270000, 50, 288, False, (64, 1, 0, 1)),
+                                              (2001, 2048, 32, True, (128, 1, 0, 1)), (100000, 352, 32, False, (128, 1, 0, 1)), (100001, 352, 288, False, (128, 1, 0, 1)),
+                                              (40003, 96, 288, True, (128, 1, 0, 1)), (19000, 128, 2400, True, (128, 1, 0, 2)), (100001, 352, 2080, False, (128, 1, 0, 2))])
+def test_streamed_raw_weights(bk, oracle, M, N, K, fused, plan):
+    assert stream_plan(bk, False, M, N, K, fused)[:4] == plan
     rng = np.random.default_rng(M + N + K)
     A, W = synth.random_bits(rng, (M, K // 8)), synth.random_bits(rng, (N, K // 8))
     thr = synth.thresholds(rng, K, N) if fused else None
