@@ -299,7 +299,7 @@ int bcnn_conv2d_b1_branches(const void *x_bits, const void *w_bits, const float 
     const int st = make_branch_problem(p, x_bits, w_bits, bn_scale, bn_shift, pad_dot, identity, prelu_slope, next_bias, y_real, y_bits, B, H, W,
                                        C_in, C_out, P, kh, kw);
     if (st != BCNN_OK) return st;
-    // on the tensor cores where the branches' accumulators and one slice of their weights fit (13 branches; bcnn_branches_plan), else on the CUDA cores
+    // on the tensor cores where the branches' accumulators (13 of them) and one part's weights of every branch fit (bcnn_branches_plan), else on the CUDA cores
     const int mod = launch_branches_tc_mod(p, static_cast<cudaStream_t>(stream));
     if (mod != BCNN_ERR_UNSUPPORTED) return mod;
     return launch_conv_branches(p, static_cast<cudaStream_t>(stream));
@@ -551,7 +551,7 @@ const char *bcnn_status_string(int status)
     case 123: return "device wait timed out: pointwise tcgen05 engine, issuer waiting for a slot's expanded rows";
     case 124: return "device wait timed out: pointwise tcgen05 engine, epilogue waiting for a chunk's accumulators";
     case 131: return "device wait timed out: streaming tcgen05 engine, producer waiting for a free ring slot";
-    case 132: return "device wait timed out: streaming tcgen05 engine, control warp waiting for a full slot or a free accumulator";
+    case 132: return "device wait timed out: streaming tcgen05 engine, issuer waiting for a full slot or a free accumulator";
     case 133: return "device wait timed out: streaming tcgen05 engine, epilogue waiting for an accumulator";
     case 134: return "device wait timed out: streaming tcgen05 engine, loader waiting for a free ring slot";
     case 125: return "device wait timed out: pointwise tcgen05 engine, producer waiting for a slot's previous MMAs";

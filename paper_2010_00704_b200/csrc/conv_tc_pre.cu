@@ -13,20 +13,21 @@
 // so there are no per-row constants, and the per-column ones are added by the epilogue from a small table.
 //
 //   warp 0        issuer: one lane waits for a stage, issues its MMAs and their commits
-//   warps 1-4     epilogue (256-wide and int32 128-wide tiles: 1-8, two teams with half of the columns each): build the
+//   warps 1-4     epilogue (256-wide tiles, and int32 128-wide ones of prepared weights: 1-8, two teams with half of the columns each): build the
 //                 column table (where the columns change), tcgen05.ld, add + sign bits (or int32), store
 //   G groups of 4 activation warps: implicit-im2col gather (cp.async), expansion, tcgen05.st into the ring in tensor memory
 //   loader warp   weight tiles by TMA into the ring in shared memory
 // Every mbarrier wait is bounded and reports through the device error word.
 //
-// 256-wide tiles have one accumulator buffer, handed over in halves of 128 columns: a tile's last two stages are multiplied half by
-// half, and so are the next one's first two, so that each half is read while the other is worked on; int32 outputs leave it as 16-bit
-// pairs (K <= 32767) and go to memory beside the next tile's MMAs.  Large products run on pairs of blocks (cta_group::2).
+// 256-wide tiles have one accumulator buffer.  Packed ones, and those of two blocks, hand it over in halves of 128 columns: a tile's last two
+// stages are multiplied half by half, and so are the next one's first two, so that each half is read while the other is worked on; int32 outputs
+// of a pair leave it as 16-bit numbers (K <= 32767) and go to memory beside the next tile's MMAs.  Int32 tiles of one block are handed over whole, and
+// each team's 128 consecutive columns go to memory one after the other.  Large products run on pairs of blocks (cta_group::2).
 //
 // RAW WEIGHTS (packed bits, new on each call): in each group as many weight warps as 32-row pieces of the CTA's weight tile expand them into
 // the ring, instead of the loader.  A pair of CTAs is what pays there, each expands half of the weight rows: 4096 x 4096 x 4608
-// packed 56 -> 37.8 us (0.48 us a stage against 0.28 of the pipe: the eight warps of a group have 250 issue slots of work per stage and its latencies),
-// 8192 x 8192 x 9216 329 -> 225, and the short set-up: 2070 x 64 x 288 4.3 -> 3.0, 34 x 3712 x 608 5.5 -> 3.5.
+// packed 56 -> 36.8 us (0.41 us a stage against 0.28 of the pipe: the eight warps of a group have 250 issue slots of work per stage and its latencies),
+// 8192 x 8192 x 9216 328 -> 220, and the short set-up: 2070 x 64 x 288 4.3 -> 3.0, 34 x 3712 x 608 5.5 -> 3.5.
 //
 // What bounds it.  Long products: power.  A 256-bit stage of a 256-wide tile takes 553 cycles of a pair (512 of the pipe), at a clock
 // that falls from 1965 to 1600 .. 1750 MHz.  Narrow tiles: the issuer - a stage of four instructions with its wait and its commit costs it 300
