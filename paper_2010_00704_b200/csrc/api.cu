@@ -119,10 +119,12 @@ int auto_engine(const ConvProblem &p)
     }
     // Weight-stationary or streaming, by their estimates, which err by a tenth: the streaming one where it is 7 % ahead.  (us, weight-stationary and
     // streaming: 3x3 128 -> 128 at M = 784 7.6 and 4.3, 64 -> 384 at 85116 19.0 and 26.6, 224 -> 608 at 82000 53 and 73, int32 160 -> 2639 at 29592 109 and
-    // 179, 64 -> 770 5x5 at 23814 33 and 50; 1x1 320 -> 256 at 200704 22.9 and 25.1, 256 -> 96 at 117120 10.5 and 15.9.)
+    // 179, 64 -> 770 5x5 at 23814 33 and 50; 1x1 320 -> 256 at 200704 22.9 and 25.1, 256 -> 96 at 117120 10.5 and 15.9.)  In slices of 64 channels, where
+    // it is the streaming estimate that comes out high, as soon as it is ahead (packed 16638 x 3584 x 4192 358 and 163, 5662 x 896 x 4704 44 and 31; int32
+    // 4096 x 4096 x 4608 71 and 54, 17903 x 512 x 3584 33.0 and 28.2).
     const bool ws = conv_tc_ws_supports(p);
     if (ws && (p.K >= 64 || p.C_out > (packed ? 64 : 32))) {
-        if (stream_raw && 107 * conv_tc_stream_estimate(p, true) < 100 * conv_tc_ws_estimate(p)) return BCNN_ENGINE_TC_I8;
+        if (stream_raw && (conv_tc_ws_narrow_slices(p) ? 100 : 107) * conv_tc_stream_estimate(p, true) < 100 * conv_tc_ws_estimate(p)) return BCNN_ENGINE_TC_I8;
         return BCNN_ENGINE_TC_WS;
     }
     // K = 32, strided, or int32 with few channels (us, warp-level int8 and streaming: packed 32 -> 64 /2 at M = 1360 4.5 and 2.9, 19656 4.8 and 4.2, 43560 5.0

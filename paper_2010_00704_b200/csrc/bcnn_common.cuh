@@ -99,6 +99,7 @@ constexpr int MAX_RAW_KTAB = 1920;       // units of the gather's table that eve
 void conv_tc_stream_plan(const ConvProblem &p, bool raw, int (&plan)[6]);
 long conv_tc_stream_estimate(const ConvProblem &p, bool raw);            // expected time, ns, on raw or prepared weights
 long conv_tc_ws_estimate(const ConvProblem &p);                          // ... of the weight-stationary engine, packed and int32 outputs
+bool conv_tc_ws_narrow_slices(const ConvProblem &p);
 // weights expanded once per layer by launch_prepare_weights (conv_tc_pre.cu): [n_pad][k_pad] signed 4-bit codes, then
 // K - 2 popc(W_n) per row
 struct PreparedWeights {

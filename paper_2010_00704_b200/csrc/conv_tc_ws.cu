@@ -546,19 +546,27 @@ bool conv_tc_ws_supports(const ConvProblem &p)
     return p.C_out > 128 && p.C_out <= 64 * 64 && fits<64, 4, false>(p);
 }
 
+// A wide layer whose K is too long for slices of 128 channels runs in slices of 64.
+bool conv_tc_ws_narrow_slices(const ConvProblem &p)
+{
+    return p.C_out > 128 && !fits<128, 4, false, 2>(p) && !fits<128, 2, true>(p) && !fits<128, 2, false>(p);
+}
+
 // Expected time, ns: a start, the expansion of a slice's weights by K, and per row tile of the longest CTA a term and one per 256-bit stage by how
-// the gather goes; int32 outputs by their number.  Fitted to 3530 drawn layers and products within 5 to 11 % (one standard deviation).
+// the gather goes; int32 outputs by their number.  Fitted to 3530 drawn layers and products within 5 to 11 % (one standard deviation); slices of 64, which
+// expand every row tile twice as often, to 94 products within 5 % (with the rates of 128 the estimate was 0.79 to 0.89 of their time).
 long conv_tc_ws_estimate(const ConvProblem &p)
 {
     struct Rates {
         long start, weights, tile, stage[3], out;
     };
-    // up to 64 channels, up to 128, slices of 128; packed, int32
-    static constexpr Rates RATES[2][3] = {
-        {{4140, 210, 180, {154, 166, 215}, 0}, {4400, 500, 560, {135, 147, 173}, 0}, {4730, 346, 490, {195, 189, 230}, 0}},
-        {{4450, 190, 141, {145, 161, 205}, 782}, {5670, 455, 543, {102, 131, 172}, 600}, {5100, 317, 1508, {173, 158, 205}, 268}}};
-    const Rates &r = RATES[p.mode == 1 ? 0 : 1][p.C_out <= 64 ? 0 : p.C_out <= 128 ? 1 : 2];
-    const long slices = ((long)p.C_out + 127) / 128, ctas = sm_count() / slices > 0 ? sm_count() / slices : 1, kt = (p.kwords + 7) / 8;
+    // up to 64 channels, up to 128, slices of 128, slices of 64; packed, int32
+    static constexpr Rates RATES[2][4] = {
+        {{4140, 210, 180, {154, 166, 215}, 0}, {4400, 500, 560, {135, 147, 173}, 0}, {4730, 346, 490, {195, 189, 230}, 0}, {4870, 276, 270, {161, 211, 299}, 0}},
+        {{4450, 190, 141, {145, 161, 205}, 782}, {5670, 455, 543, {102, 131, 172}, 600}, {5100, 317, 1508, {173, 158, 205}, 268}, {5705, 273, 157, {186, 192, 330}, 173}}};
+    const bool halved = conv_tc_ws_narrow_slices(p);
+    const Rates &r = RATES[p.mode == 1 ? 0 : 1][p.C_out <= 64 ? 0 : p.C_out <= 128 ? 1 : halved ? 3 : 2];
+    const long width = halved ? 64 : 128, slices = (p.C_out + width - 1) / width, ctas = sm_count() / slices > 0 ? sm_count() / slices : 1, kt = (p.kwords + 7) / 8;
     const long tiles = (((long)p.M + BM - 1) / BM + ctas - 1) / ctas;
     const int gw = gather_width(p.cw);
     return r.start + kt * r.weights + tiles * (r.tile + kt * r.stage[gw == 4 ? 0 : gw == 2 ? 1 : 2]) + (long)p.M * p.C_out / 1000 * r.out / 1000;

@@ -133,6 +133,16 @@ def test_module_engine_takes_wide_branch_modules():
     assert binding.bcnn_branches_plan(64, 28, 28, 128, 128, 9, 3, 3)[:2] == (32, 4)
 
 
+def test_long_products_stream_where_slices_are_narrow():
+    # wide products too long for resident slices of 128 channels: in slices of 64 the weight-stationary engine takes 1.3 to 2.2 times as long
+    from paper_2010_00704_b200 import build, binding
+    build.build()
+    for M, N, K, fused in ((16638, 3584, 4192, True), (17902, 1120, 5632, True), (4096, 4096, 4608, False), (8170, 1008, 4832, False)):
+        assert binding.bcnn_auto_engine(1, M, 1, K, N, 1, 1, 1, 0, fused=fused) == "tc_i8", (M, N, K)
+    for M, N, K in ((4096, 4096, 2304), (50176, 512, 2304)):
+        assert binding.bcnn_auto_engine(1, M, 1, K, N, 1, 1, 1, 0, fused=False) == "tc_ws", (M, N, K)
+
+
 def test_every_wait_code_has_a_name():
     # the codes as the kernels define them, each in one place
     from paper_2010_00704_b200 import build, binding
