@@ -2,7 +2,7 @@
 // branches, the paper's stand-in for a binary F x F convolution (last paragraph of Section 4.2.1).
 //
 // This is the CUDA-core path, for more branches than the module engine's accumulators hold (conv_tc_mod.cu: up to 13, nine
-// included: 256 channels at 28 x 28, batch 64, two branches 80 us here against 23.5) and for a K beyond its constants.  Every branch adds C_in / 32 xor +
+// included: 256 channels at 28 x 28, batch 64, two branches 80 us here against 18.6) and for a K beyond its constants.  Every branch adds C_in / 32 xor +
 // popcount word operations per output and the module arithmetic follows in the same thread, with no intermediate in global
 // memory; beyond a few hundred word operations per output the population counts bound it.
 //

@@ -26,7 +26,7 @@
 // wait would pass on the barrier's empty history).
 // What a launch does once - weights, parameters, constants - is written as small rolled loops with its divisions prepared on the host: an
 // instruction that runs for the first time costs some ten cycles, and unrolled eight times this set-up took 5 us.  In microseconds,
-// before and after: P = 2, 256 channels, M = 50176: 22.0, 17.7; P = 3, 160 channels, M = 96228: 47.7, 31.8; P = 3, 96 channels, M = 10496: 10.1, 7.6;
+// before and after: P = 2, 256 channels, M = 50176: 23.6, 18.6; P = 3, 160 channels, M = 96228: 47.7, 31.8; P = 3, 96 channels, M = 10496: 10.1, 7.6;
 // nine taps, 128 channels, M = 12544: 31.1, 19.9; P = 1, 128 channels: M = 1782 4.9, 3.9, M = 153064 18.8, 15.9 (12.3 of the maps' traffic).
 // Every mbarrier wait is bounded and reports through the device error word.
 #include "tc_slot.cuh"
